@@ -170,7 +170,7 @@ static stream_status build_mask_impl(const stream_problem *p, const void *q, con
     if (workspace_bytes >= sizeof(WorkspaceHeader) + n_rows * sizeof(unsigned int)) g.row_tiles = (unsigned int *)(ws + 1);
     if (tc_ok && p->impl != STREAM_IMPL_GENERIC) return launch_mask_tc(g, q, k, mask_out, score_out, ws, st);
     if (tok_ok && p->impl != STREAM_IMPL_GENERIC) return launch_mask_tok(g, q, k, mask_out, score_out, ws, st);
-    return launch_mask_generic(g, p->dtype, q, k, mask_out, score_out, ws, st);
+    return launch_mask_generic(g, p->dtype, p->impl == STREAM_IMPL_AUTO, q, k, mask_out, score_out, ws, st);
 }
 
 size_t stream_workspace_bytes_multi(const stream_problem *p, int32_t n_k) {
@@ -228,7 +228,7 @@ stream_status stream_build_mask_multi(const stream_problem *p, const void *q, co
     cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(WorkspaceHeader), st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(workspace)");
     if (!(tc_ok && p->impl != STREAM_IMPL_GENERIC))
-        return launch_mask_generic_multi(g, mk, p->dtype, q, k, mask_out, score_out, ws, st);
+        return launch_mask_generic_multi(g, mk, p->dtype, p->impl == STREAM_IMPL_AUTO, q, k, mask_out, score_out, ws, st);
     // tensor-core kernel, workspace large enough for its score memory: one launch walks every k of
     // a group before it moves on, and scores each (row, block) tile once
     const size_t score_bytes = mask_tc_score_memory_bytes(g);

@@ -50,10 +50,11 @@ void set_error(const char *fmt, ...);
 stream_status cuda_fail(cudaError_t e, const char *what);
 
 // Launchers (each validates what only it can support and returns UNSUPPORTED otherwise).
-stream_status launch_mask_generic(const Geom &g, int dtype, const void *q, const void *k, int32_t *mask,
+// allow_mma: bf16 may go through mma.sync where it fits (false: fp32 FMA whatever the dtype).
+stream_status launch_mask_generic(const Geom &g, int dtype, bool allow_mma, const void *q, const void *k, int32_t *mask,
                                   float *score, WorkspaceHeader *ws, cudaStream_t st);
 // mask / score: [mk.n][rows][k_top]; a row's tiles are scored once for all k where the cache fits.
-stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dtype, const void *q, const void *k,
+stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dtype, bool allow_mma, const void *q, const void *k,
                                         int32_t *mask, float *score, WorkspaceHeader *ws, cudaStream_t st);
 stream_status launch_attn_generic(const Geom &g, int dtype, const void *q, const void *k, const void *v,
                                   const int32_t *mask, float scale, void *out, cudaStream_t st);

@@ -1,194 +1,433 @@
-// Generic Stream mask kernel: one CTA per (batch, head, query block), fp32 FMA scoring.
-// Covers every dtype / block size / head dim the ABI accepts; the tensor-core kernel takes the
-// bf16, d = 128, 64x64 case. Follows Algorithm 2 with two exact shortcuts: only branches that
-// contain an allowed block are kept in the candidate list (the others score -inf and can never
-// displace a finite score), and a left branch inherits its parent's score (same representative).
-#include <math_constants.h>
-
-#include "common.cuh"
+// Stream mask kernel for every shape the tcgen05 kernels do not take (Algorithm 2): one CTA per
+// (batch, head, query block), its warps taking the candidate tiles of a level in turn.
+//
+// Two ways to score a tile, behind one controller:
+//   MmaScore   bf16, d = 64 / 128 / 256, 16-byte aligned rows: mma.sync m16n8k16, exact products,
+//              fp32 accumulation. A warp holds 32 keys x all queries of the row. Key fragments come
+//              straight from global memory (L2) in 16-byte loads: the contraction does not care in
+//              which order its channels are taken, so lane t of a quad reads 8 consecutive channels
+//              and both operands use that order. Query fragments come from shared memory.
+//   FmaScore   everything else (fp32; any d, alignment; bf16 when the fp32-FMA kernels are asked
+//              for): fp32 FMA, one warp per 32-key x up to 32-query part of a tile, the key rows
+//              staged in shared memory 32 channels at a time, one chunk ahead. Channels are added in
+//              ascending order, one accumulator per (query, key).
+// Bound: the L2 round trip and the barriers of a row's few small levels (issue slots 39 % busy, mma
+// pipe 22 % in the MMA form; 59 % in the FMA form), which is why a row gets only four warps and an
+// SM several rows: the 7 to 16 tiles of a level leave eight warps unequal work (12 heads,
+// T = 10007, blocks of 32, d = 128, bf16, k = 8: 310 us with eight warps a row, 222 with four; 8
+// heads, T = 5003, blocks of 32, d = 64, fp32: 246 and 216). The kernel this one replaced put 256
+// threads on one padded 64 x 64 tile at a time, with scalar loads and four barriers per tile: 5294
+// and 812 us for the same two, 4255 -> 410 us for 16 heads, T = 8192, d = 64, k = 40, not causal.
+//
+// Follows Algorithm 2 with two exact shortcuts: branches without an allowed block are dropped (they
+// score -inf and can never displace a finite score), and a left branch inherits its parent's score
+// (same representative).
+#include "warp_common.cuh"
 
 namespace stream {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kTile = 64;  // smem tiles hold up to 64 rows
+using namespace wp;
 
-// Masked maximum dot product (Eq. 4 under C) between the resident query tile and key block r.
-// All threads must call; all get the result.
-template <typename T, int D>
-__device__ float tile_score(const Geom &g, const float *Qs, float *Ks, float *red, const T *kp, int qb, int r) {
-    const int tid = threadIdx.x;
-    __syncthreads();  // previous users of Ks / red are done
-    for (int idx = tid; idx < kTile * D; idx += kThreads) {
-        int n = idx / D, c = idx % D;
-        long long tk = (long long)r * g.bk + n;
-        Ks[n * (D + 1) + c] = (n < g.bk && tk < g.T) ? to_float(kp[tk * g.ks_t + c]) : 0.f;
+constexpr int kMaxBlock = 64;
+constexpr int kWideWarps = 16;    // warps of a row when there are no more rows than SMs
+constexpr int kKeysPerUnit = 32;  // keys of a tile one warp scores at a time
+
+// Which (query m, key n) pairs of query block qb and key block r are allowed, counted from the
+// blocks' first tokens: m < n_q, n < n_k and n - m <= diag.
+struct Allowed {
+    int n_q, n_k, diag;
+    __device__ Allowed(const Geom &g, int qb, int r) {
+        const long long tq0 = (long long)qb * g.bq, tk0 = (long long)r * g.bk;
+        n_q = (int)min((long long)g.bq, g.T - tq0);
+        n_k = (int)min((long long)g.bk, g.T - tk0);
+        diag = g.causal ? (int)max(-64ll, min(64ll, tq0 - tk0)) : 64;
     }
-    __syncthreads();
-    const int tx = tid % 16, ty = tid / 16;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < D; ++c) {
-        float a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = Qs[(ty + 16 * i) * D + c];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Ks[(tx + 16 * j) * (D + 1) + c];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    __device__ bool all(int q_rows, int k_end) const { return q_rows <= n_q && k_end <= n_k && k_end - 1 <= diag; }
+    __device__ bool operator()(int m, int n) const { return m < n_q && n < n_k && n - m <= diag; }
+};
+
+// ----------------------------------------------------------------------------------------------
+// fp32 FMA
+// ----------------------------------------------------------------------------------------------
+// Lane (kq = lane / 4, kk = lane % 4) holds queries kq + 8 i (i < RQ) x keys kk + 4 j (j < 8): per
+// four channels RQ + 8 16-byte shared loads (conflict-free, broadcast over the lanes) feed 32 RQ FMA.
+template <typename T, int D, int RQ, bool kAsync>
+struct FmaScore {
+    using Elem = T;
+    static constexpr int kSQ = 8 * RQ, kCh = D < 32 ? D : 32, kChunks = D / kCh;
+    static constexpr int kRowBytes = kCh * 4, kBufBytes = kKeysPerUnit * kRowBytes, kRing = 2;
+    static constexpr int kSwz = kCh / 4 - 1;
+    static constexpr int kWarps = 4, kCtas = 4;  // warps of a row, CTAs an SM should hold
+
+    static int q_parts(const Geom &g) { return (g.bq + kSQ - 1) / kSQ; }
+    static size_t smem_bytes(const Geom &g, int warps) {
+        return (size_t)q_parts(g) * kSQ * D * 4 + (size_t)warps * kRing * kBufBytes;
     }
-    float best = -CUDART_INF_F;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int m = ty + 16 * i, n = tx + 16 * j;
-            long long tq = (long long)qb * g.bq + m, tk = (long long)r * g.bk + n;
-            bool ok = m < g.bq && n < g.bk && tq < g.T && tk < g.T && (!g.causal || tk <= tq);
-            if (ok) best = fmaxf(best, acc[i][j]);
+
+    static __device__ void load_q(const Geom &g, unsigned char *smem, const T *qp, int qb) {
+        float *Qs = (float *)smem;
+        const int rows = (g.bq + kSQ - 1) / kSQ * kSQ;
+        for (int idx = threadIdx.x; idx < rows * D; idx += blockDim.x) {
+            const int m = idx / D, c = idx % D;
+            const long long tq = (long long)qb * g.bq + m;
+            const float x = (m < g.bq && tq < g.T) ? to_float(qp[tq * g.qs_t + c]) : 0.f;
+            Qs[m * D + ((((c >> 2) ^ (m & kSwz)) << 2) | (c & 3))] = x;
         }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if ((tid & 31) == 0) red[tid >> 5] = best;
-    __syncthreads();
-    float out = red[0];
-#pragma unroll
-    for (int w = 1; w < kThreads / 32; ++w) out = fmaxf(out, red[w]);
-    return out;
-}
+    }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) mask_generic_kernel(Geom g, MultiK mk, const T *__restrict__ q,
-                                                                const T *__restrict__ k, int32_t *__restrict__ mask,
-                                                                float *__restrict__ score, WorkspaceHeader *ws) {
-    extern __shared__ float smem[];
-    float *Qs = smem;                    // [64][D]
-    float *Ks = Qs + kTile * D;          // [64][D + 1]
-    float *node_s = Ks + kTile * (D + 1);  // [k]
-    float *cand_s = node_s + g.k_top;    // [2k]
-    int *node_f = (int *)(cand_s + 2 * g.k_top);  // [k]
-    int *node_l = node_f + g.k_top;      // [k]
-    int *cand_f = node_l + g.k_top;      // [2k]
-    int *cand_l = cand_f + 2 * g.k_top;  // [2k]
-    int *keep = cand_l + 2 * g.k_top;    // [2k]
+    // Scores list[0 .. n_list) (slots of `f`) and raises their keys.
+    static __device__ void score(const Geom &g, unsigned char *smem, const T *kp, int qb, const int *list, int n_list,
+                                 const int *f, unsigned *key) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+        const int nq = (g.bq + kSQ - 1) / kSQ, nk = (g.bk + kKeysPerUnit - 1) / kKeysPerUnit, per = nq * nk;
+        const int n_units = n_list * per;
+        const int mine = n_units > warp ? (n_units - warp + warps - 1) / warps : 0;
+        const int n_chunks = mine * kChunks;
+        const float *Qs = (const float *)smem;
+        unsigned char *buf = smem + (size_t)nq * kSQ * D * 4 + (size_t)warp * kRing * kBufBytes;
+        const unsigned buf_s = smem_addr(buf);
+        const int kq = lane >> 2, kk = lane & 3;
+
+        auto issue = [&](int q) {
+            const int u = warp + (q / kChunks) * warps, cc = q % kChunks;
+            const int r = f[list[u / per]], ks = (u % per) % nk;
+            const int n0 = ks * kKeysPerUnit;
+            constexpr int per_key = kCh / 4;
+#pragma unroll
+            for (int i = 0; i < kKeysPerUnit * per_key / 32; ++i) {
+                const int idx = i * 32 + lane, n = idx / per_key, c4 = idx % per_key;
+                const int dst = (q & 1) * kBufBytes + n * kRowBytes + ((c4 ^ (n & kSwz)) << 4);
+                if (n0 + n < g.bk) {  // (keys beyond the block are never looked at)
+                    const long long tk = min((long long)r * g.bk + n0 + n, g.T - 1);
+                    const T *src = kp + tk * g.ks_t + cc * kCh + c4 * 4;
+                    if (kAsync) {
+                        cp_async16(buf_s + dst, src, 16);
+                    } else {
+                        *(float4 *)(buf + dst) = make_float4(to_float(src[0]), to_float(src[1]), to_float(src[2]), to_float(src[3]));
+                    }
+                }
+            }
+            if (kAsync) cp_async_commit();
+        };
+
+        if (n_chunks > 0) issue(0);
+        float acc[RQ][8];
+        for (int q = 0; q < n_chunks; ++q) {
+            if (q + 1 < n_chunks) {
+                __syncwarp();  // every lane is done with the buffer's previous chunk
+                issue(q + 1);
+                if (kAsync) cp_async_wait<1>();
+            } else if (kAsync) {
+                cp_async_wait<0>();
+            }
+            __syncwarp();
+            const int u = warp + (q / kChunks) * warps, cc = q % kChunks;
+            const int sub = u % per, qs = sub / nk, ks = sub % nk;
+            if (cc == 0) {
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+            }
+            const unsigned char *kb = buf + (q & 1) * kBufBytes;
+            const float *qrow = Qs + (size_t)qs * kSQ * D;
+#pragma unroll 2
+            for (int c4 = 0; c4 < kCh / 4; ++c4) {
+                float4 a[RQ], b[8];
+#pragma unroll
+                for (int i = 0; i < RQ; ++i) {
+                    const int m = kq + 8 * i;
+                    a[i] = *(const float4 *)(qrow + m * D + (((cc * (kCh / 4) + c4) ^ (m & kSwz)) << 2));
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int n = kk + 4 * j;
+                    b[j] = *(const float4 *)(kb + n * kRowBytes + ((c4 ^ (n & kSwz)) << 4));
+                }
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                        acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                        acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                        acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+                    }
+            }
+            if (cc == kChunks - 1) {
+                const int slot = list[u / per], r = f[slot];
+                float best = -CUDART_INF_F;
+                const Allowed ok(g, qb, r);
+                const bool full = ok.all((qs + 1) * kSQ, (ks + 1) * kKeysPerUnit);
+#pragma unroll
+                for (int i = 0; i < RQ; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (full || ok(qs * kSQ + kq + 8 * i, ks * kKeysPerUnit + kk + 4 * j)) best = fmaxf(best, acc[i][j]);
+                best = warp_max(best);
+                if (lane == 0 && best > -CUDART_INF_F) atomicMax(&key[slot], key_of(best));
+            }
+        }
+    }
+};
+
+// ----------------------------------------------------------------------------------------------
+// mma.sync
+// ----------------------------------------------------------------------------------------------
+template <int D, int MT>  // MT: m16 tiles of the query block
+struct MmaScore {
+    using Elem = __nv_bfloat16;
+    static constexpr int kGroups = D / 32;  // 32-channel groups: two k16 steps, one 16-byte load per lane and key
+    // 32-channel groups whose key fragments are in registers or on their way (L2 takes some 700 clocks,
+    // a group's 8 MT products 64 MT of one scheduler): what fits beside 16 MT accumulators
+    static constexpr int kFit = MT == 4 ? 2 : (MT == 2 ? 3 : 4), kAhead = kGroups < kFit ? kGroups : kFit;
+    static constexpr int kWarps = 4, kCtas = MT == 4 ? 3 : 4;
+
+    static size_t smem_bytes(const Geom &, int) { return (size_t)MT * 16 * D * 2; }
+
+    static __device__ void load_q(const Geom &g, unsigned char *smem, const __nv_bfloat16 *qp, int qb) {
+        for (int idx = threadIdx.x; idx < MT * 16 * (D / 8); idx += blockDim.x) {
+            const int m = idx / (D / 8), c = idx % (D / 8);
+            const long long tq = (long long)qb * g.bq + m;
+            uint4 x = make_uint4(0, 0, 0, 0);
+            if (m < g.bq && tq < g.T) x = *(const uint4 *)(qp + tq * g.qs_t + c * 8);
+            *(uint4 *)(smem + m * D * 2 + ((c ^ swz_rows(m)) << 4)) = x;
+        }
+    }
+
+    static __device__ void score(const Geom &g, unsigned char *smem, const __nv_bfloat16 *kp, int qb, const int *list, int n_list,
+                                 const int *f, unsigned *key) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+        const int gr = lane >> 2, t = lane & 3;
+        const int nk = (g.bk + kKeysPerUnit - 1) / kKeysPerUnit;
+        for (int u = warp; u < n_list * nk; u += warps) {
+            const int slot = list[u / nk], r = f[slot], ks = u % nk;
+            const int n_left = g.bk - ks * kKeysPerUnit;  // keys of the block from here on
+            const long long tk0 = min((long long)r * g.bk + ks * kKeysPerUnit + gr, g.T - 1);
+            const int beyond = (int)min(g.T - 1 - tk0, 24ll);  // (keys beyond T are read as the last one and never looked at)
+            const __nv_bfloat16 *row0 = kp + tk0 * g.ks_t + 8 * t;
+            int row[4];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) row[n] = min(n * 8, beyond) * (int)g.ks_t;
+            float acc[MT][4][4];
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[m][n][i] = 0.f;
+            uint4 b[kAhead][4];
+#pragma unroll
+            for (int c = 0; c < kAhead; ++c)
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+                    if (n * 8 < n_left) b[c][n] = __ldg((const uint4 *)(row0 + row[n] + 32 * c));
+#pragma unroll
+            for (int c = 0; c < kGroups; ++c) {
+                uint4 (&x)[4] = b[c % kAhead];
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    const int m0 = m * 16 + gr, ch = 4 * c + t;
+                    const uint4 qa = *(const uint4 *)(smem + m0 * D * 2 + ((ch ^ swz_rows(m0)) << 4));
+                    const uint4 qc = *(const uint4 *)(smem + (m0 + 8) * D * 2 + ((ch ^ swz_rows(m0 + 8)) << 4));
+                    // (two products of one accumulator never back to back: the second would wait for the first)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+                        if (n * 8 < n_left) mma_bf16(acc[m][n], qa.x, qc.x, qa.y, qc.y, x[n].x, x[n].y);
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+                        if (n * 8 < n_left) mma_bf16(acc[m][n], qa.z, qc.z, qa.w, qc.w, x[n].z, x[n].w);
+                }
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+                    if (c + kAhead < kGroups && n * 8 < n_left) x[n] = __ldg((const uint4 *)(row0 + row[n] + 32 * (c + kAhead)));
+            }
+            float best = -CUDART_INF_F;
+            const Allowed ok(g, qb, r);
+            if (ok.all(MT * 16, (ks + 1) * kKeysPerUnit)) {
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) best = fmaxf(best, acc[m][n][i]);
+            } else {
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (ok(m * 16 + gr + 8 * (i >> 1), ks * kKeysPerUnit + n * 8 + 2 * t + (i & 1))) best = fmaxf(best, acc[m][n][i]);
+            }
+            best = warp_max(best);
+            if (lane == 0 && best > -CUDART_INF_F) atomicMax(&key[slot], key_of(best));
+        }
+    }
+};
+
+// ----------------------------------------------------------------------------------------------
+// The row
+// ----------------------------------------------------------------------------------------------
+// A level's candidates live in slots: node i's left half in slot 2 i, its right half in 2 i + 1
+// (last < first: no such candidate), each with the key of its score (0: not known yet). Slots are
+// in block order, so the tie rule (lower block index) is the lower slot, and no compaction is
+// needed between scoring and ranking.
+struct Slots {
+    int *at;  // first [n] | last [n] | key [n]
+    int n;
+    __device__ int *first() const { return at; }
+    __device__ int *last() const { return at + n; }
+    __device__ unsigned *key() const { return (unsigned *)at + 2 * n; }
+};
+
+template <class P, int W>
+__global__ void __launch_bounds__(W * 32, W == kWideWarps ? 1 : P::kCtas)
+mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P::Elem *__restrict__ q,
+                 const typename P::Elem *__restrict__ k, int32_t *__restrict__ mask, float *__restrict__ score, WorkspaceHeader *ws) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    int *words = (int *)(smem + score_bytes);  // n_max: slots, a multiple of 32
+    int par = 0;                               // the present level's slots: the first or the second set
+    int *list = words + 6 * n_max;             // slots still without a score
+    unsigned *keep = (unsigned *)words + 7 * n_max;  // a bit per slot
     // several k: scores of this row by key block, NaN = not scored yet (a score does not depend on k)
-    float *cache = mk.use_cache ? (float *)(keep + 2 * g.k_top) : nullptr;  // [N_k]
-    __shared__ float red[kThreads / 32];
-    __shared__ int s_nodes, s_cands;
+    float *cache = mk.use_cache ? (float *)(keep + n_max / 32) : nullptr;
+    __shared__ int s_list, s_valid;
 
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, n_thr = blockDim.x;
     // heaviest rows (late query blocks) first
     const long long row_rev = blockIdx.x;
     const int qb = g.n_qb - 1 - (int)(row_rev / ((long long)g.batch * g.H));
     const int bh = (int)(row_rev % ((long long)g.batch * g.H));
     const int b = bh / g.H, h = bh % g.H, kvh = h / g.hpg;
     const long long row = ((long long)b * g.H + h) * g.n_qb + qb;
-    const T *qp = q + b * g.qs_b + h * g.qs_h;
-    const T *kp = k + b * g.ks_b + kvh * g.ks_h;
-    const int q_lim = last_valid_block(g, qb);
     const long long rows_total = (long long)g.batch * g.H * g.n_qb;
+    const typename P::Elem *kp = k + b * g.ks_b + kvh * g.ks_h;
+    const int q_lim = last_valid_block(g, qb);
 
+    P::load_q(g, smem, q + b * g.qs_b + h * g.qs_h, qb);
     if (cache != nullptr)
-        for (int r = tid; r < g.N_k; r += kThreads) cache[r] = CUDART_NAN_F;
-    for (int idx = tid; idx < kTile * D; idx += kThreads) {
-        int m = idx / D, c = idx % D;
-        long long tq = (long long)qb * g.bq + m;
-        Qs[idx] = (m < g.bq && tq < g.T) ? to_float(qp[tq * g.qs_t + c]) : 0.f;
-    }
+        for (int r = tid; r < g.N_k; r += n_thr) cache[r] = CUDART_NAN_F;
     unsigned tiles = 0;
+
+    // Candidate (fst, lst) into slot c; known = key of its score or 0 (then it goes on the list,
+    // unless `cache` knows it).
+    auto put = [&](const Slots &s, int c, bool ok, int fst, int lst, unsigned known, bool want) {
+        if (ok && known == 0u && want) {
+            if (cache != nullptr && !isnan(cache[fst])) known = key_of(cache[fst]);
+            else list[atomicAdd(&s_list, 1)] = c;
+        }
+        s.first()[c] = fst;
+        s.last()[c] = ok ? lst : fst - 1;
+        s.key()[c] = ok ? known : 0u;
+        if (ok) atomicAdd(&s_valid, 1);
+    };
+    // Node i = blocks (fst : lst) into its two slots: (fst : m) keeps the node's score, (m + 1 : lst)
+    // needs one if it holds an allowed block.
+    auto split = [&](const Slots &s, int i, bool ok, int fst, int lst, unsigned known) {
+        const int m = (fst + lst) / 2;
+        put(s, 2 * i, ok, fst, m, known, true);
+        put(s, 2 * i + 1, ok && m + 1 <= lst && m + 1 <= q_lim, m + 1, lst, 0u, true);
+    };
+    auto pad = [&](const Slots &s, int n) {  // up to a multiple of 32: absent candidates
+        const int c = n + tid;
+        if (c < ((n + 31) & ~31)) { s.first()[c] = 0; s.last()[c] = -1; s.key()[c] = 0u; }
+    };
+
     const int n_pass = mk.n > 0 ? mk.n : 1;
     for (int pass = 0; pass < n_pass; ++pass) {
-    const int kq = mk.n > 0 ? mk.k[pass] : row_k(g, qb);  // this pass's k (= k_top unless told otherwise)
-    const int levels = row_levels(g, kq);
-    __syncthreads();  // the previous pass is done with the node arrays
-    if (tid == 0) {  // initial nodes tiling [0, N_k); keep those that hold an allowed block
-        int n = 0;
-        for (int j = 0; j < kq; ++j) {
-            int f = (int)(((long long)j * g.N_k) / kq);
-            int l = (int)(((long long)(j + 1) * g.N_k) / kq) - 1;
-            if (f <= l && f <= q_lim) { node_f[n] = f; node_l[n] = l; node_s[n] = CUDART_NAN_F; ++n; }
+        const int kq = mk.n > 0 ? mk.k[pass] : row_k(g, qb);  // this pass's k (= k_top unless told otherwise)
+        const int levels = row_levels(g, kq);
+        __syncthreads();  // the previous pass is done with the slots
+        if (tid == 0) { s_list = 0; s_valid = 0; }
+        __syncthreads();
+        // initial nodes tiling [0, N_k); those without an allowed block are absent. With no level to
+        // go through (one key block) they are the result, and need a score only if it is asked for.
+        int n_slots = levels > 0 ? 2 * kq : kq;
+        par = 0;
+        const Slots start = {words, n_max};
+        for (int i = tid; i < kq; i += n_thr) {
+            const int fst = (int)(((long long)i * g.N_k) / kq), lst = (int)(((long long)(i + 1) * g.N_k) / kq) - 1;
+            const bool ok = fst <= lst && fst <= q_lim;
+            if (levels > 0) split(start, i, ok, fst, lst, 0u);
+            else put(start, i, ok, fst, lst, 0u, score != nullptr);
         }
-        s_nodes = n;
-    }
-    __syncthreads();
+        pad(start, n_slots);
+        __syncthreads();
 
-    for (int level = 0; level < levels; ++level) {
-        if (tid == 0) {
-            int n = 0;
-            for (int i = 0; i < s_nodes; ++i) {
-                int f = node_f[i], l = node_l[i], m = (f + l) / 2;
-                cand_f[n] = f; cand_l[n] = m; cand_s[n] = node_s[i]; ++n;
-                if (m + 1 <= l && m + 1 <= q_lim) { cand_f[n] = m + 1; cand_l[n] = l; cand_s[n] = CUDART_NAN_F; ++n; }
-            }
-            s_cands = n;
-        }
-        __syncthreads();
-        const int n_cand = s_cands;
-        for (int c = 0; c < n_cand; ++c) {
-            if (isnan(cand_s[c])) {  // uniform: shared value
-                const int r = cand_f[c];
-                float s = cache != nullptr ? cache[r] : CUDART_NAN_F;  // (uniform too)
-                if (isnan(s)) {
-                    s = tile_score<T, D>(g, Qs, Ks, red, kp, qb, r);
-                    ++tiles;
+        for (int level = 0;; ++level) {
+            const Slots cur = {words + par * 3 * n_max, n_max}, nxt = {words + (par ^ 1) * 3 * n_max, n_max};
+            const int n_list = s_list, n_valid = s_valid, n_words = (n_slots + 31) >> 5;
+            P::score(g, smem, kp, qb, list, n_list, cur.first(), cur.key());
+            if (level < levels) tiles += (unsigned)n_list;
+            __syncthreads();  // every key of the level is in place
+            if (tid == 0) { s_list = 0; s_valid = 0; }
+            if (cache != nullptr)
+                for (int i = tid; i < n_list; i += n_thr) cache[cur.first()[list[i]]] = score_of(cur.key()[list[i]]);
+            // Top-k by rank: a candidate is beaten by a higher score, or an equal one in a lower slot.
+            // (Absent candidates have key 0 and beat nobody.) A warp's 32 slots are consecutive: the
+            // words before its own compare with >=, those behind it with >.
+            for (int w = tid >> 5; w < n_words; w += n_thr >> 5) {
+                const int c = w * 32 + (tid & 31);
+                const unsigned mine = cur.key()[c];
+                const bool valid = cur.last()[c] >= cur.first()[c];
+                bool kept = valid;
+                if (n_valid > kq) {
+                    int rank = 0;
+                    for (int u = 0; u < n_words; ++u) {
+                        const uint4 *x = (const uint4 *)(cur.key() + u * 32);
+                        if (u == w) {
+#pragma unroll
+                            for (int v = 0; v < 32; ++v) {
+                                const unsigned y = cur.key()[u * 32 + v];
+                                rank += (y > mine) || (y == mine && v < (tid & 31));
+                            }
+                        } else {
+                            const unsigned thr = u < w && mine != 0u ? mine - 1u : mine;
+#pragma unroll
+                            for (int v = 0; v < 8; ++v) {
+                                const uint4 y = x[v];
+                                rank += (int)(y.x > thr) + (int)(y.y > thr) + (int)(y.z > thr) + (int)(y.w > thr);
+                            }
+                        }
+                    }
+                    kept = valid && rank < kq;
                 }
-                __syncthreads();
-                if (tid == 0) {
-                    cand_s[c] = s;
-                    if (cache != nullptr) cache[r] = s;
+                const unsigned bal = __ballot_sync(0xffffffffu, kept);
+                if ((tid & 31) == 0) keep[w] = bal;
+            }
+            __syncthreads();
+            // survivors stay in ascending block order: a kept slot becomes the node of its rank in the bits
+            const bool last = level + 1 >= levels;
+            int n_kept = 0;
+            for (int u = 0; u < n_words; ++u) n_kept += __popc(keep[u]);
+            const long long o = (pass * rows_total + row) * g.k_top;
+            for (int c = tid; c < n_words * 32; c += n_thr) {
+                const int w = c >> 5;
+                if (!((keep[w] >> (c & 31)) & 1u)) continue;
+                int pos = __popc(keep[w] & ((1u << (c & 31)) - 1u));
+                for (int u = 0; u < w; ++u) pos += __popc(keep[u]);
+                if (last) {
+                    mask[o + pos] = cur.first()[c];
+                    if (score != nullptr) score[o + pos] = score_of(cur.key()[c]);
+                } else {
+                    split(nxt, pos, true, cur.first()[c], cur.last()[c], cur.key()[c]);
                 }
             }
-        }
-        __syncthreads();
-        // top-k by rank: a candidate is beaten by a higher score, or an equal score at a lower index
-        for (int c = tid; c < n_cand; c += kThreads) {
-            int rank = 0;
-            if (n_cand > kq) {
-                float s = cand_s[c];
-                for (int u = 0; u < n_cand; ++u) {
-                    float su = cand_s[u];
-                    rank += (su > s) || (su == s && u < c);
+            if (last) {
+                for (int j = n_kept + tid; j < g.k_top; j += n_thr) {
+                    mask[o + j] = -1;
+                    if (score != nullptr) score[o + j] = -CUDART_INF_F;
                 }
+                break;
             }
-            keep[c] = rank < kq;
+            n_slots = 2 * n_kept;
+            pad(nxt, n_slots);
+            par ^= 1;
+            __syncthreads();
         }
-        __syncthreads();
-        if (tid == 0) {  // survivors stay in ascending block order
-            int n = 0;
-            for (int c = 0; c < n_cand; ++c)
-                if (keep[c]) { node_f[n] = cand_f[c]; node_l[n] = cand_l[c]; node_s[n] = cand_s[c]; ++n; }
-            s_nodes = n;
-        }
-        __syncthreads();
     }
-    const int n_nodes = s_nodes;
-    if (score != nullptr) {  // only reachable with zero levels: scores were never needed
-        for (int i = 0; i < n_nodes; ++i) {
-            if (isnan(node_s[i])) {
-                const int r = node_f[i];
-                float s = cache != nullptr ? cache[r] : CUDART_NAN_F;
-                if (isnan(s)) s = tile_score<T, D>(g, Qs, Ks, red, kp, qb, r);
-                __syncthreads();
-                if (tid == 0) {
-                    node_s[i] = s;
-                    if (cache != nullptr) cache[r] = s;
-                }
-            }
-        }
-        __syncthreads();
-    }
-    const long long o = (pass * rows_total + row) * g.k_top;
-    for (int j = tid; j < g.k_top; j += kThreads) {
-        mask[o + j] = j < n_nodes ? node_f[j] : -1;
-        if (score != nullptr) score[o + j] = j < n_nodes ? node_s[j] : -CUDART_INF_F;
-    }
-    }  // pass
     if (tid == 0) {
         atomicAdd(&ws->tiles_scored, (unsigned long long)tiles);
         atomicAdd(&ws->rows, 1ull);
@@ -198,53 +437,94 @@ __global__ void __launch_bounds__(kThreads) mask_generic_kernel(Geom g, MultiK m
 
 constexpr size_t kMaxDynamicSmem = 227 * 1024 - 1024;  // (the kernel has a few static words too)
 
-template <typename T, int D>
-stream_status launch(const Geom &g, MultiK mk, const T *q, const T *k, int32_t *mask, float *score, WorkspaceHeader *ws,
-                     cudaStream_t st) {
-    size_t smem = sizeof(float) * (kTile * D + kTile * (D + 1) + 3 * (size_t)g.k_top) + sizeof(int) * 8 * (size_t)g.k_top;
+template <class P, int W>
+stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, int32_t *mask, float *score, WorkspaceHeader *ws,
+                       cudaStream_t st) {
+    const long long rows = (long long)g.batch * g.H * g.n_qb;
+    const int n_max = (2 * g.k_top + 31) & ~31;
+    const size_t score_bytes = P::smem_bytes(g, W);
+    size_t smem = score_bytes + (size_t)(7 * n_max + n_max / 32) * 4;
     mk.use_cache = mk.n > 1 && smem + sizeof(float) * (size_t)g.N_k <= kMaxDynamicSmem;
     if (mk.use_cache) smem += sizeof(float) * (size_t)g.N_k;
-    auto kern = mask_generic_kernel<T, D>;
+    auto kern = mask_rows_kernel<P, W>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_generic)");
-    long long rows = (long long)g.batch * g.H * g.n_qb;
-    kern<<<(unsigned)rows, kThreads, smem, st>>>(g, mk, q, k, mask, score, ws);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_rows)");
+    kern<<<(unsigned)rows, W * 32, smem, st>>>(g, mk, (int)score_bytes, n_max, (const typename P::Elem *)q,
+                                               (const typename P::Elem *)k, mask, score, ws);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "mask_generic launch");
+    if (e != cudaSuccess) return cuda_fail(e, "mask_rows launch");
     return STREAM_OK;
 }
 
-template <typename T>
-stream_status dispatch_d(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score,
-                         WorkspaceHeader *ws, cudaStream_t st) {
-    const T *qq = (const T *)q, *kk = (const T *)k;
+template <class P>
+stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score, WorkspaceHeader *ws,
+                     cudaStream_t st) {
+    const long long rows = (long long)g.batch * g.H * g.n_qb;
+    // Sixteen warps when every row has an SM to itself anyway: a level's tiles then spread over more
+    // warps (64 rows, fp32, d = 64, blocks of 32, k = 8: 34.9 us with eight, 32.9 with sixteen).
+    if (rows <= sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
+    return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
+}
+
+template <typename T, int RQ, bool kAsync>
+stream_status fma_d(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score,
+                    WorkspaceHeader *ws, cudaStream_t st) {
     switch (g.d) {
-        case 16: return launch<T, 16>(g, mk, qq, kk, mask, score, ws, st);
-        case 32: return launch<T, 32>(g, mk, qq, kk, mask, score, ws, st);
-        case 64: return launch<T, 64>(g, mk, qq, kk, mask, score, ws, st);
-        case 128: return launch<T, 128>(g, mk, qq, kk, mask, score, ws, st);
-        case 256: return launch<T, 256>(g, mk, qq, kk, mask, score, ws, st);
+        case 16: return launch<FmaScore<T, 16, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
+        case 32: return launch<FmaScore<T, 32, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
+        case 64: return launch<FmaScore<T, 64, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
+        case 128: return launch<FmaScore<T, 128, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
+        case 256: return launch<FmaScore<T, 256, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
     }
     set_error("generic mask kernel: head dim %d not in {16, 32, 64, 128, 256}", g.d);
     return STREAM_ERR_UNSUPPORTED;
 }
 
-}  // namespace
-
-stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dtype, const void *q, const void *k,
-                                        int32_t *mask, float *score, WorkspaceHeader *ws, cudaStream_t st) {
-    if (g.bq > kTile || g.bk > kTile) {
-        set_error("generic mask kernel: block sizes up to %d (got %d, %d)", kTile, g.bq, g.bk);
-        return STREAM_ERR_UNSUPPORTED;
-    }
-    if (dtype == STREAM_F32) return dispatch_d<float>(g, mk, q, k, mask, score, ws, st);
-    return dispatch_d<__nv_bfloat16>(g, mk, q, k, mask, score, ws, st);
+template <typename T, bool kAsync>
+stream_status fma_rq(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score,
+                     WorkspaceHeader *ws, cudaStream_t st) {
+    if (g.bq <= 16) return fma_d<T, 2, kAsync>(g, mk, q, k, mask, score, ws, st);  // 16 queries per warp instead of 32
+    return fma_d<T, 4, kAsync>(g, mk, q, k, mask, score, ws, st);
 }
 
-stream_status launch_mask_generic(const Geom &g, int dtype, const void *q, const void *k, int32_t *mask,
+template <int MT>
+stream_status mma_d(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score,
+                    WorkspaceHeader *ws, cudaStream_t st) {
+    switch (g.d) {
+        case 64: return launch<MmaScore<64, MT>>(g, mk, q, k, mask, score, ws, st);
+        case 128: return launch<MmaScore<128, MT>>(g, mk, q, k, mask, score, ws, st);
+        default: return launch<MmaScore<256, MT>>(g, mk, q, k, mask, score, ws, st);
+    }
+}
+
+}  // namespace
+
+stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dtype, bool allow_mma, const void *q, const void *k,
+                                        int32_t *mask, float *score, WorkspaceHeader *ws, cudaStream_t st) {
+    if (g.bq > kMaxBlock || g.bk > kMaxBlock) {
+        set_error("generic mask kernel: block sizes up to %d (got %d, %d)", kMaxBlock, g.bq, g.bk);
+        return STREAM_ERR_UNSUPPORTED;
+    }
+    const int e = dtype == STREAM_F32 ? 4 : 2;
+    const bool k_aligned = rows_16_byte_aligned(k, g.ks_t, g.ks_h, g.ks_b, e);
+    if (dtype == STREAM_F32) {
+        if (k_aligned) return fma_rq<float, true>(g, mk, q, k, mask, score, ws, st);
+        return fma_rq<float, false>(g, mk, q, k, mask, score, ws, st);
+    }
+    // d = 16 and 32 would leave most of an mma's channels or lanes unused: they stay on the FMA form
+    if (allow_mma && (g.d == 64 || g.d == 128 || g.d == 256) && k_aligned && g.ks_t < (1 << 24) &&
+        rows_16_byte_aligned(q, g.qs_t, g.qs_h, g.qs_b, 2)) {
+        if (g.bq <= 16) return mma_d<1>(g, mk, q, k, mask, score, ws, st);
+        if (g.bq <= 32) return mma_d<2>(g, mk, q, k, mask, score, ws, st);
+        return mma_d<4>(g, mk, q, k, mask, score, ws, st);
+    }
+    return fma_rq<__nv_bfloat16, false>(g, mk, q, k, mask, score, ws, st);
+}
+
+stream_status launch_mask_generic(const Geom &g, int dtype, bool allow_mma, const void *q, const void *k, int32_t *mask,
                                   float *score, WorkspaceHeader *ws, cudaStream_t st) {
     MultiK single = {};
-    return launch_mask_generic_multi(g, single, dtype, q, k, mask, score, ws, st);
+    return launch_mask_generic_multi(g, single, dtype, allow_mma, q, k, mask, score, ws, st);
 }
 
 }  // namespace stream

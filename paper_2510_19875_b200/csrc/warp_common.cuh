@@ -1,0 +1,73 @@
+// Helpers shared by the kernels that run on warp-level instructions (mma.sync, fp32 FMA, cp.async).
+#pragma once
+#include <math_constants.h>
+
+#include "common.cuh"
+
+namespace stream {
+namespace wp {
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// 16 bytes global -> shared without a register; bytes = 0 writes zeros and reads nothing.
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// D += A B, m16n8k16, bf16 operands (exact products), fp32 accumulation.
+__device__ __forceinline__ void mma_bf16(float *c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ float warp_max(float x) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// 2^x by the special-function unit (relative error about 2^-22; -inf gives 0).
+__device__ __forceinline__ float fast_exp2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Barrier of a group of warps (one warp needs no more than reconvergence). Ids 1.. are the caller's.
+__device__ __forceinline__ void group_sync(int id, int threads) {
+    if (threads == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Which of the 8 16-byte columns of a 128-byte line a bf16 row keeps chunk c of that line in: c ^
+// swz_rows(row). Read as mma operands, 8 lanes (two rows r, r + 1, four consecutive chunks each)
+// then meet 8 different columns.
+__device__ __forceinline__ int swz_rows(int row) { return ((row & 1) << 2) | ((row >> 1) & 3); }
+
+// fp32 score <-> unsigned key of the same order (-0 first brought to +0; 0 is below every score).
+__device__ __forceinline__ unsigned key_of(float s) {
+    const unsigned b = __float_as_uint(s + 0.f);
+    return b ^ ((b & 0x80000000u) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ float score_of(unsigned key) {
+    return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+}
+
+inline bool rows_16_byte_aligned(const void *base, long long s_t, long long s_h, long long s_b, int elem) {
+    const long long per = 16 / elem;
+    return ((uintptr_t)base & 15) == 0 && s_t % per == 0 && s_h % per == 0 && s_b % per == 0;
+}
+
+// SMs of the current device (148 if it cannot be asked): only used to choose launch shapes.
+inline int sm_count_or_default() {
+    int dev = 0, n = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 148;
+    return n;
+}
+
+}  // namespace wp
+}  // namespace stream
