@@ -1,155 +1,308 @@
-// Generic block-sparse attention (Eq. 2 on a Stream mask): one CTA per (batch, head, query
-// block), fp32 FMA, online softmax over the kept key blocks. Covers every dtype / block size /
-// head dim the ABI accepts.
-#include <math_constants.h>
-
-#include "common.cuh"
+// Block-sparse attention (Eq. 2 on a Stream mask) in fp32 FMA: every dtype, head dimension, block
+// size and alignment the ABI accepts (fp32 above all).
+//
+// One CTA per (batch, head, query block). A warp owns QW query tokens (32, or 16 where the output
+// accumulators would not fit) against 32 keys at a time; ceil(block_q / QW) warps make a group that
+// walks a sequence of key tiles, and the groups of a CTA take the row's tiles in turn, each with
+// softmax statistics and accumulators of its own, added up at the end. One K and one V buffer
+// per group, filled by cp.async: the next K tile arrives behind softmax and P V, the next V tile
+// behind the next Q K^T. Inner loops read shared memory 16 bytes at a time, conflict-free:
+//   Q K^T   lane (kq, kk): queries kq + 8 i x keys kk + 4 j; QW / 8 + 8 loads per 4 QW FMA
+//   P V     lane (ro, co): QW / 4 consecutive queries x channels 4 co + 32 i, P kept key-major
+// Bound: FMA issue and its latency at 8 warps per SM (issue slots 53 % busy; a bare FMA loop measures
+// 66 of the 74.5 TFLOP/s). The kernel this one replaced padded every tile to 64 x 64 and loaded
+// scalars: 8 heads, T = 5003, blocks of 32, d = 64, k = 8: 599 -> 150 us; one head, T = 2048: 82 -> 25 us.
+#include "warp_common.cuh"
 
 namespace stream {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kTile = 64;
+using namespace wp;
+
+constexpr int kMaxBlock = 64;
+constexpr int kKeys = 32;  // keys of a tile
 
 template <typename T>
-__device__ __forceinline__ T from_float(float x);
+__device__ __forceinline__ void store4(T *dst, float4 x);
 template <>
-__device__ __forceinline__ float from_float<float>(float x) { return x; }
+__device__ __forceinline__ void store4<float>(float *dst, float4 x) {
+    dst[0] = x.x; dst[1] = x.y; dst[2] = x.z; dst[3] = x.w;
+}
 template <>
-__device__ __forceinline__ __nv_bfloat16 from_float<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
+__device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16 *dst, float4 x) {
+    dst[0] = __float2bfloat16_rn(x.x); dst[1] = __float2bfloat16_rn(x.y);
+    dst[2] = __float2bfloat16_rn(x.z); dst[3] = __float2bfloat16_rn(x.w);
+}
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) attn_generic_kernel(Geom g, const T *__restrict__ q,
-                                                                const T *__restrict__ k, const T *__restrict__ v,
-                                                                const int32_t *__restrict__ mask, float scale,
-                                                                T *__restrict__ out) {
-    extern __shared__ float smem[];
-    float *Qs = smem;                     // [64][D]
-    float *Ks = Qs + kTile * D;           // [64][D + 1]
-    float *Vs = Ks + kTile * (D + 1);     // [64][D]
-    float *Ps = Vs + kTile * D;           // [64][65]
+template <int D, int QW>
+struct Shape {
+    static constexpr int kTileBytes = kKeys * D * 4, kPPitch = QW + 8, kPBytes = kKeys * kPPitch * 4;
+    static constexpr int kSwz = (D / 4 - 1) & 7;  // 16-byte columns are permuted within a row by row & kSwz
+    static constexpr int kPart = QW * D + 2 * QW;  // floats a warp leaves behind for the final sum
+};
 
-    const int tid = threadIdx.x;
-    const long long row = blockIdx.x;
-    const int qb = (int)(row % g.n_qb);
-    const int bh = (int)(row / g.n_qb);
+// A [32][D] fp32 tile: keys n0 .. n0 + 31 of block r.
+template <typename T, int D, bool kAsync, bool kIsK>
+__device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T *base, int r, int n0, int thr, int n_thr) {
+    constexpr int per_row = D / 4;
+    for (int idx = thr; idx < kKeys * per_row; idx += n_thr) {
+        const int n = idx / per_row, c = idx % per_row;
+        const long long tk = (long long)r * g.bk + n0 + n;
+        const bool in = n0 + n < g.bk && tk < g.T;  // the rest become zeros
+        unsigned char *to = dst + n * D * 4 + ((kIsK ? c ^ (n & Shape<D, 32>::kSwz) : c) << 4);
+        const T *src = base + (in ? tk : 0) * g.ks_t + c * 4;
+        if (kAsync) {
+            cp_async16(smem_addr(to), src, in ? 16 : 0);
+        } else {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in) x = make_float4(to_float(src[0]), to_float(src[1]), to_float(src[2]), to_float(src[3]));
+            *(float4 *)to = x;
+        }
+    }
+    if (kAsync) cp_async_commit();
+}
+
+template <typename T, int D, int QW, bool kAsync>
+__global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, int splits, const T *__restrict__ q,
+                                                           const T *__restrict__ k, const T *__restrict__ v,
+                                                           const int32_t *__restrict__ mask, float scale, T *__restrict__ out) {
+    using Sh = Shape<D, QW>;
+    constexpr int RQ = QW / 8, RO = QW / 4, CO = D < 32 ? 1 : D / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_n;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int grp = warp / m_warps, mw = warp % m_warps, g_thr = m_warps * 32, g_tid = tid - grp * g_thr;
+    const int kq = lane >> 2, kk = lane & 3;   // Q K^T
+    const int ro = lane >> 3, co = lane & 7;   // P V
+    // late (longer) rows first
+    const int bh = blockIdx.x / g.n_qb, qb = g.n_qb - 1 - (int)(blockIdx.x % g.n_qb);
     const int b = bh / g.H, h = bh % g.H, kvh = h / g.hpg;
     const T *qp = q + b * g.qs_b + h * g.qs_h;
-    const T *kp = k + b * g.ks_b + kvh * g.ks_h;
-    const T *vp = v + b * g.ks_b + kvh * g.ks_h;
-    const int32_t *mrow = mask + row * g.k_top;
+    const T *kp = k + b * g.ks_b + kvh * g.ks_h, *vp = v + b * g.ks_b + kvh * g.ks_h;
+    const int32_t *mrow = mask + ((long long)bh * g.n_qb + qb) * g.k_top;
 
-    for (int idx = tid; idx < kTile * D; idx += kThreads) {
-        int m = idx / D, c = idx % D;
-        long long tq = (long long)qb * g.bq + m;
-        Qs[idx] = (m < g.bq && tq < g.T) ? to_float(qp[tq * g.qs_t + c]) : 0.f;
+    // Q | per group K, V | per warp P | per warp row factors | kept blocks
+    float *Qs = (float *)smem;
+    unsigned char *ks = smem + (size_t)m_warps * QW * D * 4 + (size_t)grp * 2 * Sh::kTileBytes, *vs = ks + Sh::kTileBytes;
+    unsigned char *pw = smem + (size_t)m_warps * QW * D * 4 + (size_t)splits * 2 * Sh::kTileBytes;
+    float *Ps = (float *)(pw + (size_t)warp * Sh::kPBytes);
+    pw += (size_t)m_warps * splits * Sh::kPBytes;
+    float *factor = (float *)pw + warp * QW;
+    int *list = (int *)((float *)pw + m_warps * splits * QW);
+
+    for (int idx = tid; idx < m_warps * QW * D; idx += blockDim.x) {
+        const int m = idx / D, c = idx % D;
+        const long long tq = (long long)qb * g.bq + m;
+        const float x = (m < g.bq && tq < g.T) ? to_float(qp[tq * g.qs_t + c]) : 0.f;
+        Qs[m * D + ((((c >> 2) ^ (m & Sh::kSwz)) << 2) | (c & 3))] = x;
     }
-    const int tx = tid % 16, ty = tid / 16;  // logits: rows ty + 16 i, keys tx + 16 j
-    const int om = tid / 4, og = tid % 4;    // output: row om, channels og + 4 i
-    float o[D / 4];
-#pragma unroll
-    for (int i = 0; i < D / 4; ++i) o[i] = 0.f;
-    float run_max = -CUDART_INF_F, run_sum = 0.f;
+    if (warp == 0) {  // the row's kept blocks, in order
+        int n = 0;
+        for (int j = 0; j < g.k_top; j += 32) {
+            const int r = j + lane < g.k_top ? mrow[j + lane] : -1;
+            const unsigned bal = __ballot_sync(0xffffffffu, r >= 0);
+            if (r >= 0) list[n + __popc(bal & ((1u << lane) - 1u))] = r;
+            n += __popc(bal);
+        }
+        if (lane == 0) s_n = n;
+    }
+    __syncthreads();
 
-    for (int j = 0; j < g.k_top; ++j) {
-        const int r = mrow[j];
-        if (r < 0) continue;  // uniform: same value for the whole CTA
-        __syncthreads();
-        for (int idx = tid; idx < kTile * D; idx += kThreads) {
-            int n = idx / D, c = idx % D;
-            long long tk = (long long)r * g.bk + n;
-            bool in = n < g.bk && tk < g.T;
-            Ks[n * (D + 1) + c] = in ? to_float(kp[tk * g.ks_t + c]) : 0.f;
-            Vs[idx] = in ? to_float(vp[tk * g.ks_t + c]) : 0.f;
-        }
-        __syncthreads();
-        float acc[4][4];
+    float o[RO][CO * 4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RO; ++i)
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) acc[i][jj] = 0.f;
-#pragma unroll 4
-        for (int c = 0; c < D; ++c) {
-            float a[4], bb[4];
+        for (int j = 0; j < CO * 4; ++j) o[i][j] = 0.f;
+    float m_run[RQ], l_run[RQ];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = Qs[(ty + 16 * i) * D + c];
+    for (int i = 0; i < RQ; ++i) { m_run[i] = -CUDART_INF_F; l_run[i] = 0.f; }
+    const float *qw = Qs + (size_t)mw * QW * D;
+
+    const int n_sub = (g.bk + kKeys - 1) / kKeys, n_tiles = s_n * n_sub;
+    if (grp < n_tiles) {
+        fetch<T, D, kAsync, true>(g, ks, kp, list[grp / n_sub], grp % n_sub * kKeys, g_tid, g_thr);
+        fetch<T, D, kAsync, false>(g, vs, vp, list[grp / n_sub], grp % n_sub * kKeys, g_tid, g_thr);
+    }
+    for (int i0 = grp; i0 < n_tiles; i0 += splits) {
+        const int r = list[i0 / n_sub], n0 = i0 % n_sub * kKeys, nxt = i0 + splits;
+        const long long k0 = (long long)r * g.bk + n0;
+        const int n_keys = (int)max(0ll, min((long long)min(g.bk - n0, kKeys), g.T - k0));
+        if (kAsync) cp_async_wait<1>();
+        group_sync(1 + grp, g_thr);  // the K tile is there
+        float s[RQ][8];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) bb[jj] = Ks[(tx + 16 * jj) * (D + 1) + c];
+        for (int i = 0; i < RQ; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 8; ++j) s[i][j] = 0.f;
+#pragma unroll 2
+        for (int c4 = 0; c4 < D / 4; ++c4) {
+            float4 a[RQ], x[8];
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(a[i], bb[jj], acc[i][jj]);
-        }
+            for (int i = 0; i < RQ; ++i) a[i] = *(const float4 *)(qw + (kq + 8 * i) * D + ((c4 ^ (kq & Sh::kSwz)) << 2));
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                int m = ty + 16 * i, n = tx + 16 * jj;
-                long long tq = (long long)qb * g.bq + m, tk = (long long)r * g.bk + n;
-                bool ok = m < g.bq && n < g.bk && tq < g.T && tk < g.T && (!g.causal || tk <= tq);
-                Ps[m * (kTile + 1) + n] = ok ? scale * acc[i][jj] : -CUDART_INF_F;
+            for (int j = 0; j < 8; ++j) {
+                const int n = kk + 4 * j;
+                x[j] = *(const float4 *)(ks + n * D * 4 + ((c4 ^ (n & Sh::kSwz)) << 4));
             }
-        __syncthreads();
-        // online softmax: the four threads of a row split its keys
-        float mx = -CUDART_INF_F;
-        for (int n = og; n < kTile; n += 4) mx = fmaxf(mx, Ps[om * (kTile + 1) + n]);
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float new_max = fmaxf(run_max, mx);
-        const float alpha = (new_max == -CUDART_INF_F) ? 1.f : expf(run_max - new_max);
-        float part = 0.f;
-        for (int n = og; n < kTile; n += 4) {
-            float s = Ps[om * (kTile + 1) + n];
-            float p = (s == -CUDART_INF_F) ? 0.f : expf(s - new_max);
-            Ps[om * (kTile + 1) + n] = p;
-            part += p;
-        }
-        part += __shfl_xor_sync(0xffffffffu, part, 1);
-        part += __shfl_xor_sync(0xffffffffu, part, 2);
-        run_sum = run_sum * alpha + part;
-        run_max = new_max;
-        __syncwarp();
 #pragma unroll
-        for (int i = 0; i < D / 4; ++i) o[i] *= alpha;
-        for (int n = 0; n < kTile; ++n) {
-            float p = Ps[om * (kTile + 1) + n];
+            for (int i = 0; i < RQ; ++i)
 #pragma unroll
-            for (int i = 0; i < D / 4; ++i) o[i] = fmaf(p, Vs[n * D + og + 4 * i], o[i]);
+                for (int j = 0; j < 8; ++j) {
+                    s[i][j] = fmaf(a[i].x, x[j].x, s[i][j]);
+                    s[i][j] = fmaf(a[i].y, x[j].y, s[i][j]);
+                    s[i][j] = fmaf(a[i].z, x[j].z, s[i][j]);
+                    s[i][j] = fmaf(a[i].w, x[j].w, s[i][j]);
+                }
         }
+        group_sync(1 + grp, g_thr);  // everybody is done with the K tile
+        if (nxt < n_tiles) fetch<T, D, kAsync, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
+        else if (kAsync) cp_async_commit();
+        // online softmax; the four lanes of a query share its keys
+        bool moved = false;
+#pragma unroll
+        for (int i = 0; i < RQ; ++i) {
+            const int m = mw * QW + kq + 8 * i;
+            const long long tq = (long long)qb * g.bq + m;
+            int lim = m < g.bq && tq < g.T ? n_keys : 0;
+            if (g.causal) lim = (int)max(0ll, min((long long)lim, tq - k0 + 1));
+            float mx = m_run[i];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                s[i][j] = kk + 4 * j < lim ? scale * s[i][j] : -CUDART_INF_F;
+                mx = fmaxf(mx, s[i][j]);
+            }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            const float ref = mx == -CUDART_INF_F ? 0.f : mx;
+            const float alpha = m_run[i] == -CUDART_INF_F ? 0.f : expf(m_run[i] - ref);
+            float sum = 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float p = s[i][j] == -CUDART_INF_F ? 0.f : expf(s[i][j] - ref);
+                sum += p;
+                Ps[(kk + 4 * j) * Sh::kPPitch + kq + 8 * i] = p;
+            }
+            l_run[i] = l_run[i] * alpha + sum;  // (each lane its own keys' part; they meet at the end)
+            m_run[i] = mx;
+            if (kk == 0) factor[kq + 8 * i] = alpha;
+            moved |= alpha != 1.f;
+        }
+        moved = __any_sync(0xffffffffu, moved);
+        if (kAsync) cp_async_wait<1>();
+        group_sync(1 + grp, g_thr);  // the V tile and this warp's P are there
+        if (moved) {
+#pragma unroll
+            for (int i = 0; i < RO; ++i) {
+                const float f = factor[ro * RO + i];
+#pragma unroll
+                for (int j = 0; j < CO * 4; ++j) o[i][j] *= f;
+            }
+        }
+        if (D >= 32 || co * 4 < D) {
+#pragma unroll 4
+            for (int n = 0; n < n_keys; ++n) {
+                float p[RO];
+#pragma unroll
+                for (int i = 0; i < RO; i += 4) *(float4 *)(p + i) = *(const float4 *)(Ps + n * Sh::kPPitch + ro * RO + i);
+#pragma unroll
+                for (int j = 0; j < CO; ++j) {
+                    const float4 x = *(const float4 *)(vs + n * D * 4 + (co + 8 * j) * 16);
+#pragma unroll
+                    for (int i = 0; i < RO; ++i) {
+                        o[i][4 * j] = fmaf(p[i], x.x, o[i][4 * j]);
+                        o[i][4 * j + 1] = fmaf(p[i], x.y, o[i][4 * j + 1]);
+                        o[i][4 * j + 2] = fmaf(p[i], x.z, o[i][4 * j + 2]);
+                        o[i][4 * j + 3] = fmaf(p[i], x.w, o[i][4 * j + 3]);
+                    }
+                }
+            }
+        }
+        group_sync(1 + grp, g_thr);  // done with the V tile and with P
+        if (nxt < n_tiles) fetch<T, D, kAsync, false>(g, vs, vp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
     }
-    const long long tq = (long long)qb * g.bq + om;
-    if (om < g.bq && tq < g.T) {
-        const float inv = run_sum > 0.f ? 1.f / run_sum : 0.f;
-        T *op = out + (((long long)b * g.H + h) * g.T + tq) * D;
+    if (kAsync) cp_async_wait<0>();
+
+    // Sum over the groups through shared memory (all tiles are done with): per warp its rows' maxima
+    // and sums, then its accumulators.
+    __syncthreads();
+    float *part = (float *)smem + (size_t)warp * Sh::kPart;
 #pragma unroll
-        for (int i = 0; i < D / 4; ++i) op[og + 4 * i] = from_float<T>(o[i] * inv);
+    for (int i = 0; i < RQ; ++i) {
+        float l = l_run[i];
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        l += __shfl_xor_sync(0xffffffffu, l, 2);
+        if (kk == 0) { part[kq + 8 * i] = m_run[i]; part[QW + kq + 8 * i] = l; }
+    }
+    if (grp > 0) {
+#pragma unroll
+        for (int i = 0; i < RO; ++i)
+#pragma unroll
+            for (int j = 0; j < CO * 4; ++j) part[2 * QW + (i * CO * 4 + j) * 32 + lane] = o[i][j];
+    }
+    __syncthreads();
+    if (grp > 0) return;
+    if (D < 32 && co * 4 >= D) return;
+#pragma unroll
+    for (int i = 0; i < RO; ++i) {
+        const int mr = ro * RO + i, m = mw * QW + mr;
+        const long long tq = (long long)qb * g.bq + m;
+        float top = -CUDART_INF_F;
+        for (int s = 0; s < splits; ++s) top = fmaxf(top, ((float *)smem)[(size_t)(s * m_warps + mw) * Sh::kPart + mr]);
+        const float ref = top == -CUDART_INF_F ? 0.f : top;
+        float total = 0.f, x[CO * 4];
+#pragma unroll
+        for (int j = 0; j < CO * 4; ++j) x[j] = 0.f;
+        for (int s = 0; s < splits; ++s) {
+            const float *ps = (float *)smem + (size_t)(s * m_warps + mw) * Sh::kPart;
+            const float f = ps[mr] == -CUDART_INF_F ? 0.f : expf(ps[mr] - ref);
+            total += f * ps[QW + mr];
+#pragma unroll
+            for (int j = 0; j < CO * 4; ++j) x[j] = fmaf(f, s == 0 ? o[i][j] : ps[2 * QW + (i * CO * 4 + j) * 32 + lane], x[j]);
+        }
+        const float inv = total > 0.f ? 1.f / total : 0.f;
+        if (m >= g.bq || tq >= g.T) continue;
+        T *dst = out + ((long long)bh * g.T + tq) * D;
+#pragma unroll
+        for (int j = 0; j < CO; ++j)
+            store4(dst + 4 * co + 32 * j, make_float4(x[4 * j] * inv, x[4 * j + 1] * inv, x[4 * j + 2] * inv, x[4 * j + 3] * inv));
     }
 }
 
-template <typename T, int D>
-stream_status launch(const Geom &g, const T *q, const T *k, const T *v, const int32_t *mask, float scale, T *out,
+template <typename T, int D, bool kAsync>
+stream_status launch(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
                      cudaStream_t st) {
-    size_t smem = sizeof(float) * (kTile * D * 2 + kTile * (D + 1) + kTile * (kTile + 1));
-    auto kern = attn_generic_kernel<T, D>;
+    constexpr int QW = D <= 64 ? 32 : 16;  // 64 (d = 256: 128) accumulators a lane
+    using Sh = Shape<D, QW>;
+    const int m_warps = (g.bq + QW - 1) / QW;
+    const long long rows = (long long)g.batch * g.H * g.n_qb;
+    // Four warps a CTA, so that several CTAs share an SM; eight when every row has an SM to itself
+    // anyway (64 rows of 8 blocks of 32, d = 64: 26.8 us with four, 25.3 with eight).
+    int splits = (rows <= sm_count_or_default() ? 8 : 4) / m_warps;
+    auto bytes = [&](int s) {
+        const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * (Sh::kPBytes + QW * 4) + (size_t)g.k_top * 4;
+        const size_t sum = (size_t)m_warps * s * Sh::kPart * 4;
+        return walk > sum ? walk : sum;
+    };
+    while (splits > 1 && bytes(splits) > 220 * 1024) splits /= 2;
+    const size_t smem = bytes(splits);
+    auto kern = attn_generic_kernel<T, D, QW, kAsync>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
-    long long rows = (long long)g.batch * g.H * g.n_qb;
-    kern<<<(unsigned)rows, kThreads, smem, st>>>(g, q, k, v, mask, scale, out);
+    kern<<<(unsigned)rows, m_warps * splits * 32, smem, st>>>(g, m_warps, splits, (const T *)q, (const T *)k, (const T *)v, mask, scale, (T *)out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "attn_generic launch");
     return STREAM_OK;
 }
 
-template <typename T>
-stream_status dispatch_d(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask,
-                         float scale, void *out, cudaStream_t st) {
-    const T *qq = (const T *)q, *kk = (const T *)k, *vv = (const T *)v;
+template <typename T, bool kAsync>
+stream_status dispatch_d(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
+                         cudaStream_t st) {
     switch (g.d) {
-        case 16: return launch<T, 16>(g, qq, kk, vv, mask, scale, (T *)out, st);
-        case 32: return launch<T, 32>(g, qq, kk, vv, mask, scale, (T *)out, st);
-        case 64: return launch<T, 64>(g, qq, kk, vv, mask, scale, (T *)out, st);
-        case 128: return launch<T, 128>(g, qq, kk, vv, mask, scale, (T *)out, st);
-        case 256: return launch<T, 256>(g, qq, kk, vv, mask, scale, (T *)out, st);
+        case 16: return launch<T, 16, kAsync>(g, q, k, v, mask, scale, out, st);
+        case 32: return launch<T, 32, kAsync>(g, q, k, v, mask, scale, out, st);
+        case 64: return launch<T, 64, kAsync>(g, q, k, v, mask, scale, out, st);
+        case 128: return launch<T, 128, kAsync>(g, q, k, v, mask, scale, out, st);
+        case 256: return launch<T, 256, kAsync>(g, q, k, v, mask, scale, out, st);
     }
     set_error("generic attention kernel: head dim %d not in {16, 32, 64, 128, 256}", g.d);
     return STREAM_ERR_UNSUPPORTED;
@@ -159,12 +312,14 @@ stream_status dispatch_d(const Geom &g, const void *q, const void *k, const void
 
 stream_status launch_attn_generic(const Geom &g, int dtype, const void *q, const void *k, const void *v,
                                   const int32_t *mask, float scale, void *out, cudaStream_t st) {
-    if (g.bq > kTile || g.bk > kTile) {
-        set_error("generic attention kernel: block sizes up to %d (got %d, %d)", kTile, g.bq, g.bk);
+    if (g.bq > kMaxBlock || g.bk > kMaxBlock) {
+        set_error("generic attention kernel: block sizes up to %d (got %d, %d)", kMaxBlock, g.bq, g.bk);
         return STREAM_ERR_UNSUPPORTED;
     }
-    if (dtype == STREAM_F32) return dispatch_d<float>(g, q, k, v, mask, scale, out, st);
-    return dispatch_d<__nv_bfloat16>(g, q, k, v, mask, scale, out, st);
+    if (dtype != STREAM_F32) return dispatch_d<__nv_bfloat16, false>(g, q, k, v, mask, scale, out, st);
+    const bool aligned = rows_16_byte_aligned(k, g.ks_t, g.ks_h, g.ks_b, 4) && ((uintptr_t)v & 15) == 0;
+    if (aligned) return dispatch_d<float, true>(g, q, k, v, mask, scale, out, st);
+    return dispatch_d<float, false>(g, q, k, v, mask, scale, out, st);
 }
 
 }  // namespace stream
