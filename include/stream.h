@@ -46,7 +46,8 @@ typedef enum {
 typedef enum { STREAM_F32 = 0, STREAM_BF16 = 1 } stream_dtype;
 
 typedef enum {
-    STREAM_IMPL_AUTO = 0,    /* tensor-core kernels when the shape allows, else the generic ones */
+    STREAM_IMPL_AUTO = 0,    /* tcgen05 kernels when the shape allows, else mma.sync for bf16 with d in
+                                {64, 128, 256} and 16-byte aligned rows, else the generic ones */
     STREAM_IMPL_GENERIC = 1, /* fp32-FMA kernels: any dtype, d in {16,32,64,128,256}, blocks 1..64 */
     STREAM_IMPL_TENSOR = 2   /* tcgen05 kernels only: bf16, d = 128, block_q = block_k = 64, strides
                                 that are multiples of 8 elements, 16-byte aligned pointers (and

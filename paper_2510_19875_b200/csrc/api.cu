@@ -294,6 +294,7 @@ stream_status stream_sparse_attention(const stream_problem *p, const void *q, co
         return STREAM_ERR_UNSUPPORTED;
     }
     if (tc_ok && p->impl != STREAM_IMPL_GENERIC) return launch_attn_tc(g, q, k, v, mask, scale, out, st);
+    if (p->impl == STREAM_IMPL_AUTO && attn_mma_supported(g, p->dtype, q, k, v, out)) return launch_attn_mma(g, q, k, v, mask, scale, out, st);
     return launch_attn_generic(g, p->dtype, q, k, v, mask, scale, out, st);
 }
 

@@ -58,6 +58,10 @@ stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dty
                                         int32_t *mask, float *score, WorkspaceHeader *ws, cudaStream_t st);
 stream_status launch_attn_generic(const Geom &g, int dtype, const void *q, const void *k, const void *v,
                                   const int32_t *mask, float scale, void *out, cudaStream_t st);
+// bf16 attention on mma.sync (whatever the tcgen05 kernel does not take, with 16-byte aligned rows).
+bool attn_mma_supported(const Geom &g, int dtype, const void *q, const void *k, const void *v, const void *out);
+stream_status launch_attn_mma(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale,
+                              void *out, cudaStream_t st);
 bool mask_tc_supported(const Geom &g, int dtype);
 stream_status launch_mask_tc(const Geom &g, const void *q, const void *k, int32_t *mask, float *score,
                              WorkspaceHeader *ws, cudaStream_t st);
