@@ -38,7 +38,7 @@ template <int D, int QW>
 struct Shape {
     static constexpr int kTileBytes = kKeys * D * 4, kPPitch = QW + 8, kPBytes = kKeys * kPPitch * 4;
     static constexpr int kSwz = (D / 4 - 1) & 7;  // 16-byte columns are permuted within a row by row & kSwz
-    static constexpr int kPart = QW * D + 2 * QW;  // floats a warp leaves behind for the final sum
+    static constexpr int kPart = QW * (D < 32 ? 32 : D) + 2 * QW;  // floats a warp leaves behind for the final sum (d = 16: idle lanes too)
 };
 
 // A [32][D] fp32 tile: keys n0 .. n0 + 31 of block r.
