@@ -1,29 +1,37 @@
 // Tensor-core block-sparse attention for sm_100a (Eq. 2 on a Stream mask): bf16, d = 128,
 // 64 x 64 blocks.
 //
-// One persistent CTA per SM works through "pairs": two query heads of one kv head at one query
-// block. Their Q tiles are stacked into one 128-row A operand. For every mask entry e the two
-// rows name one key block each (K_a, K_b, usually different); the tiles arrive by TMA (128-byte
-// swizzle), stacked too, and
+// One persistent CTA per SM works through "pairs": two rows (query blocks) of one kv head - two query
+// heads at one query block, or, where the number of heads per kv head is odd, two neighbouring
+// query blocks of the last head. Their Q tiles are stacked into one 128-row A operand. For every mask
+// entry e the two rows name one key block each (K_a, K_b, usually different); the tiles arrive by
+// TMA (128-byte swizzle), stacked too, and
 //     S = [Q_0; Q_1] [K_a; K_b]^T      (128 x 128, fp32 in TMEM)
 // holds row 0's logits in its upper-left quadrant and row 1's in its lower-right one.
 //
 // Two softmax groups of four warps take a pair's entries in turn (its n-th kept entry belongs to
 // group n % 2, so that a pair's arithmetic does not depend on what the CTA did before), so
-// that one group's chain of waits, TMEM loads, exponentials and fences runs beside the other's.
-// A thread owns one query token (TMEM lane) of its group's entries: it reads the token's 64
-// logits, applies the element-level mask C, and writes P = exp2(scale (s - ref)) as bf16 into
-// its row of the group's 128 x 64 A operand in shared memory. Then two chains with an
-// output-lane mask,
-//     O_g[lanes 0..63]   += P[rows 0..63]   V_a,      O_g[lanes 64..127] += P[rows 64..127] V_b
-// (128 x 128, fp32, accumulated in TMEM per group g; V tiles MN-major), add each row's
-// contribution and leave the other row's lanes alone. `ref` is a per-token reference the group keeps
-// instead of the exact running maximum (bf16 P and fp32 sums keep their relative precision
-// whatever the reference, as long as nothing overflows): the maximum of the token's first allowed
-// logits, moved (with the token's O_g lane and sum rescaled in place) only when a logit has
-// outgrown it by about 2^30 in exp2's argument, which the entry's sum of P shows. At the end of a
-// pair the two groups exchange (ref, sum) per token, bring O_0 and O_1 to the common reference,
-// add, normalise and store.
+// that one group's chain of waits, TMEM loads and exponentials runs beside the other's. A thread
+// owns one query token (TMEM lane) of its group's entries: it reads the token's 64 logits, applies
+// the element-level mask C, and writes P = exp2(scale (s - ref)) as bf16 back over the logits, where
+// the P V product takes it as its A operand from TMEM. Two chains with an output-lane mask,
+//     O[lanes 0..63]   += P[rows 0..63]   V_a,      O[lanes 64..127] += P[rows 64..127] V_b
+// (128 x 128, fp32, in TMEM; V tiles MN-major), add each row's contribution and leave the other
+// row's lanes alone. Three logit buffers and one O fill the 512 TMEM columns.
+//
+// `ref` is a per-token reference kept instead of the exact running maximum (bf16 P and fp32 sums
+// keep their relative precision whatever the reference, as long as nothing overflows): the
+// maximum of the token's first allowed logits, moved (with the token's O lane and sums rescaled)
+// only when a logit has outgrown it by about 2^30 in exp2's argument, which the entry's sum of P
+// shows. The groups share O, so they share the reference: it lives in shared memory, entry 0's
+// group sets it before it computes its P, and entry n's warp looks at it again after entry n - 1's
+// warp of the same lanes has published (`turn`), so that a reference that moved meanwhile is seen
+// and P computed again. At the end of a pair the groups exchange their sums, normalise and store
+// half of the channels each.
+//
+// What this form replaces kept P in shared memory (64 KB of stores and proxy fences, and a group's
+// buffer held until its product was complete) and one O per group: an entry took 1560 clocks, the
+// two chains of an entry keep the tensor pipe busy for 1024 (ATTN_V2).
 //
 // Roles (384 threads): warp 0 TMA producer (converged, one elected lane issues; two independent
 // non-blocking load streams, K with Q and V); warp 1 issues the Q K^T chains and owns TMEM; warp 3
@@ -52,31 +60,35 @@ constexpr int kBlk = 64, kD = 128;
 constexpr int kHalfTile = kBlk * 128;       // 64 rows x 128 bytes
 constexpr int kTile = 2 * kHalfTile;        // one 64 x 128 tile
 constexpr int kOperand = 2 * kTile;         // two tiles (K_a, K_b or V_a, V_b), or the 128-row Q operand
-constexpr int kPBytes = 2 * kHalfTile;      // one group's P: 128 rows x 64 keys
-// Stages of the two rings, out of the five operand buffers shared memory has room for beside Q
-// and P (four when the mask rows are long): a V stage is held from its load until the product of
-// its entry is complete, a whole softmax later, so V gets three when there are five, K two.
+// Stages of the two rings, out of the operand buffers shared memory has room for beside Q: six when
+// the mask rows are short (three each), else five (a V stage is held from its load until the
+// product of its entry is complete, a whole softmax later: V three, K two) or four.
 constexpr int kMaxKStages = 3, kMaxVStages = 3;
+constexpr int kSBufs = 3;                   // logit buffers: entry n of the kernel's sequence uses buffer n % 3
 constexpr int kMaskSlots = 2;               // pairs whose mask rows are resident
 constexpr int kMaxKTopTc = 1024;
+constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while pairs of several heads are walked
 constexpr float kLazySum = 68719476736.f;   // 2^36 = 64 * 2^30: the 64 P of an entry add up to more only if one of them exceeds 2^30 (its logit has outgrown the reference by 30 in log2 units)
 
-// TMEM columns: S of group g at 128 g, O of group g at 256 + 128 g.
+// TMEM columns: S / P buffer b at 128 b (P: its first 32), O at 384.
+constexpr int kOCol = kSBufs * 128;
 struct Tail {
     unsigned long long q_full, q_empty;
     unsigned long long k_full[kMaxKStages], k_empty[kMaxKStages], v_full[kMaxVStages], v_empty[kMaxVStages];
-    // Per group g (a pair's kept entries n with n % 2 == g): logits ready / read, P published, product added.
-    // o_full[g] also tells the group that its P buffer is free again.
-    unsigned long long s_full[2], s_empty[2], p_full[2], o_full[2];
+    unsigned long long s_full[kSBufs], p_full[kSBufs], s_free[kSBufs];  // logits ready, P in their place, product added
+    unsigned long long o_done, o_free;     // a pair's last product is complete; its O has been read (8 warps)
+    // Between the two softmax warps of a lane quarter (one per group): the pair's first references
+    // are set; group g has published an entry; both have left their sums.
+    unsigned long long ref_set[4], turn[4][2], sums_there[4];
     unsigned long long m_full[kMaskSlots], m_empty[kMaskSlots];
-    unsigned long long x_bar[4];  // the two softmax warps of a lane quarter (one per group) meet here
     unsigned int tmem_base;
     int abort_flag;
     int m_count[kMaskSlots];  // kept entries of the pair in each mask slot
+    float ref[128], sum[2][128];
 };
-// Dynamic shared memory: Q | P of group 0, P of group 1 | V stages | K stages | Tail | mask rows
-// [kMaskSlots][2][row_stride] (-1 where a row has nothing), the operands 1024-byte aligned.
-constexpr int kFixedOperands = 2;  // Q, the two P together; behind them the V stages, then the K stages
+// Dynamic shared memory: Q | V stages | K stages | Tail | mask rows [kMaskSlots][2][row_stride] (-1
+// where a row has nothing), the operands 1024-byte aligned.
+constexpr int kFixedOperands = 1;  // Q; behind it the V stages, then the K stages
 constexpr int kMaxSmemPerCta = 232448;
 
 constexpr unsigned kIdescQK = idesc_bf16(128, 128, false);  // B = stacked K tiles, K-major
@@ -85,7 +97,8 @@ constexpr unsigned kHiK = desc_hi_sw128(1024);              // every operand: 8-
 
 struct Params {
     Geom g;
-    int n_items, n_pairs;  // pairs per kv head: ceil(hpg / 2)
+    int n_items;           // pairs
+    int group_heads;       // kv heads (of the batch * G) whose pairs are walked together
     int row_stride;        // ints per resident mask row (k_top rounded up to a multiple of 4)
     int smem_bytes;        // dynamic shared memory of the launch
     int n_k_stages, n_v_stages;  // set by the kernel from what fits behind its aligned base
@@ -108,26 +121,46 @@ __device__ __forceinline__ int *mask_rows(Tail *tl, const Params &P, int slot) {
     return reinterpret_cast<int *>(tl + 1) + slot * 2 * P.row_stride;
 }
 
-// The pair a CTA works on in its n-th round.
+// The pair a CTA works on. h[r], qb[r]: head and query block of row r < R (R = 0: a place of the
+// order without a pair).
 struct Item {
-    int b, kvh, qb, h0, R;
+    int b, kvh, R;
+    int h[2], qb[2];
 };
 
+// A CTA's n-th place in the order of pairs. Every second round runs backwards, so that with pairs in
+// order of falling length every CTA gets about the same sum.
+__device__ __forceinline__ int nth_item(const Params &P, int n) {
+    return n * (int)gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+}
+
+// The order: `group_heads` kv heads at a time, as many as have K and V in L2 together, and within
+// them late query blocks (most kept blocks under a causal mask) first. One kv head after the other,
+// every head's short pairs in between, left the CTAs 11 % apart at T = 4096 (32 / 8 heads, k = 32;
+// 4 % at T = 16384), this order with the turn of nth_item 1 %. Two query blocks make a level: their
+// pairs of heads, and the odd last head's pair of its own two query blocks.
 __device__ __forceinline__ Item decode_item(const Params &P, int id) {
     const Geom &g = P.g;
     Item it;
-    // kv head by kv head, so that the K and V tiles in flight belong to one head at a time (64 MiB
-    // at T = 131072: they stay in L2); within a head late query blocks (most kept blocks under a
-    // causal mask) first
-    const int per_head = g.n_qb * P.n_pairs;
-    const int bh = id / per_head;
-    const int rem = id % per_head;
-    it.qb = g.n_qb - 1 - rem / P.n_pairs;
-    const int pair = rem % P.n_pairs;
+    const int pairs = g.hpg >> 1, per_level = 2 * pairs + (g.hpg & 1), levels = (g.n_qb + 1) >> 1;
+    const int per_head = levels * per_level, per_group = P.group_heads * per_head;
+    const int grp = id / per_group, rem = id - grp * per_group;
+    const int heads = min(P.group_heads, g.batch * g.G - grp * P.group_heads);
+    const int level = rem / (heads * per_level), in_level = rem - level * heads * per_level;
+    const int head = in_level / per_level, slot = in_level - head * per_level;
+    const int bh = grp * P.group_heads + head, j = levels - 1 - level;
     it.kvh = bh % g.G;
     it.b = bh / g.G;
-    it.h0 = it.kvh * g.hpg + pair * 2;
-    it.R = min(2, g.hpg - pair * 2);
+    if (slot < 2 * pairs) {
+        const int qb = 2 * j + 1 - slot / pairs, h0 = it.kvh * g.hpg + slot % pairs * 2;
+        it.R = qb < g.n_qb ? 2 : 0;
+        it.h[0] = h0; it.h[1] = h0 + 1;
+        it.qb[0] = it.qb[1] = min(qb, g.n_qb - 1);
+    } else {
+        it.R = 2 * j + 1 < g.n_qb ? 2 : 1;
+        it.h[0] = it.h[1] = it.kvh * g.hpg + g.hpg - 1;
+        it.qb[0] = 2 * j; it.qb[1] = min(2 * j + 1, g.n_qb - 1);
+    }
     return it;
 }
 
@@ -150,11 +183,11 @@ __device__ __forceinline__ Entry entry_at(const int *rows, int stride, int n) {
 __device__ void mask_loader_role(const Params &P, Tail *tl, int lane) {
     const Geom &g = P.g;
     Ring ms;
-    for (int id = blockIdx.x; id < P.n_items; id += gridDim.x) {
+    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         const Item it = decode_item(P, id);
         if (!wait(smem_u32(&tl->m_empty[ms.idx]), ms.phase ^ 1, tl, 401)) return;
-        const int32_t *m0 = P.mask + (((long long)it.b * g.H + it.h0) * g.n_qb + it.qb) * g.k_top;
-        const int32_t *m1 = m0 + (long long)g.n_qb * g.k_top;
+        const int32_t *m0 = P.mask + (((long long)it.b * g.H + it.h[0]) * g.n_qb + it.qb[0]) * g.k_top;
+        const int32_t *m1 = P.mask + (((long long)it.b * g.H + it.h[1]) * g.n_qb + it.qb[1]) * g.k_top;
         int *dst = mask_rows(tl, P, ms.idx);
         // an entry is kept if either row has a block there; the kept ones move to the front, so that
         // the other roles index them instead of searching (their serial code is the kernel's pace)
@@ -163,7 +196,7 @@ __device__ void mask_loader_role(const Params &P, Tail *tl, int lane) {
             const int e = base + lane;
             int a = -1, b = -1;
             if (e < g.k_top) {
-                a = __ldg(m0 + e);
+                if (it.R >= 1) a = __ldg(m0 + e);
                 if (it.R == 2) b = __ldg(m1 + e);
             }
             const bool kept = a >= 0 || b >= 0;
@@ -189,7 +222,7 @@ __device__ void mask_loader_role(const Params &P, Tail *tl, int lane) {
 // while the other could move: every step probes its barrier without waiting. The warp runs
 // converged (lane 0's probe result is broadcast) and one elected lane issues.
 struct LoadStream {
-    int id;            // pair being walked
+    int round, id;     // pair being walked
     int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
     int n;             // kept entries of the pair
     int n_issued;      // loads issued for this pair
@@ -207,7 +240,8 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
                               Tail *tl, unsigned q_smem, unsigned k_smem, unsigned v_smem) {
     unsigned q_par = 0;
     LoadStream K, V;
-    K.id = V.id = blockIdx.x;
+    K.round = V.round = 0;
+    K.id = V.id = nth_item(P, 0);
     K.e = V.e = -2;
     K.q_due = V.q_due = false;
     // a row without a block at an entry gets block 0; its logits are masked out entirely
@@ -244,7 +278,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
             if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
             __syncwarp();
             S.ms.advance(kMaskSlots);
-            S.id += gridDim.x;
+            S.id = nth_item(P, ++S.round);
             S.e = -2;
             return true;
         }
@@ -265,7 +299,14 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
             if (elect_one()) {
                 const unsigned bar = smem_u32(&tl->q_full);
                 mbar_arrive_expect_tx(bar, (unsigned)kOperand);
-                tma_load_5d(q_smem, tq, bar, 0, S.it.qb * kBlk, S.it.h0, 0, S.it.b);  // heads h0 and h0 + 1
+#pragma unroll
+                for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const bool second = r == 1 && S.it.R == 2;
+                        tma_load_4d(q_smem + (2 * c + r) * kHalfTile, tq, bar, c * 64, (second ? S.it.qb[1] : S.it.qb[0]) * kBlk,
+                                    second ? S.it.h[1] : S.it.h[0], S.it.b);
+                    }
             }
             __syncwarp();
             S.q_due = false;
@@ -304,13 +345,12 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
 // The two issuing roles are run by all 32 lanes of their warps, converged: the waits are
 // warp-wide, one elected lane issues.
 
-// S_g = [Q_0; Q_1] [K_a; K_b]^T for every kept entry (g = the entry's number within its pair % 2).
+// S = [Q_0; Q_1] [K_a; K_b]^T for every kept entry.
 __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base) {
-    Ring ks, ms;
-    unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
+    Ring ks, ms, sb;
     unsigned q_par = 0;
     const unsigned q_lo = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
-    for (int id = blockIdx.x; id < P.n_items; id += gridDim.x) {
+    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
         const int n_entries = tl->m_count[ms.idx];  // the issuers need no more than the count
         if (n_entries > 0) {
@@ -319,10 +359,9 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
         }
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, tl, 202)) return;
-            const unsigned gi = (unsigned)(i & 1), use = cnt[gi]++;  // entry i of a pair belongs to group i % 2
-            if (!wait_w(smem_u32(&tl->s_empty[gi]), (use & 1u) ^ 1u, tl, 203)) return;
+            if (!wait_w(smem_u32(&tl->s_free[sb.idx]), sb.phase ^ 1u, tl, 203)) return;  // the buffer's last P has been used
             tc_fence_after();
-            const unsigned d_tmem = tmem_base + gi * 128;
+            const unsigned d_tmem = tmem_base + sb.idx * 128;
             const unsigned b_lo = k_lo + ks.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
@@ -331,12 +370,13 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
                     for (int k4 = 0; k4 < 4; ++k4)
                         tc_mma_bf16_split(d_tmem, q_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK,
                                           b_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
-                tc_commit(smem_u32(&tl->s_full[gi]));
+                tc_commit(smem_u32(&tl->s_full[sb.idx]));
                 tc_commit(smem_u32(&tl->k_empty[ks.idx]));
                 if (i + 1 == n_entries) tc_commit(smem_u32(&tl->q_empty));  // that was the pair's last use of Q
             }
             __syncwarp();
             ks.advance(P.n_k_stages);
+            sb.advance(kSBufs);
         }
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
@@ -344,39 +384,40 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
     }
 }
 
-// O_g (+)= P_g [V_a; V_b] for every kept entry; a group's first entry of a pair starts its O afresh.
-__device__ void pv_role(const Params &P, Tail *tl, unsigned p_smem, unsigned v_smem, unsigned tmem_base) {
-    Ring vs, ms;  // vs: the entry's V stage
-    unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
+// O (+)= P [V_a; V_b] for every kept entry; a pair's first entry starts O afresh.
+__device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tmem_base) {
+    Ring vs, ms, sb;  // vs: the entry's V stage
+    unsigned free_par = 1;  // (the first wait passes at once)
     // the MN-major V tiles have their two 64-channel halves kHalfTile apart
-    const unsigned p_lo = desc_lo_sw128(p_smem, 16), v_lo = desc_lo_sw128(v_smem, kHalfTile);
-    for (int id = blockIdx.x; id < P.n_items; id += gridDim.x) {
+    const unsigned v_lo = desc_lo_sw128(v_smem, kHalfTile), d_tmem = tmem_base + kOCol;
+    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
         const int n_entries = tl->m_count[ms.idx];
-        unsigned fresh = 3u;  // bit g: group g has not added anything for this pair yet
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->v_full[vs.idx]), vs.phase, tl, 205)) return;
-            const unsigned gi = (unsigned)(i & 1), use = cnt[gi]++;  // group = O buffer of the entry
-            if (!wait_w(smem_u32(&tl->p_full[gi]), use & 1u, tl, 204)) return;  // also: O_g rescaled if it had to be
+            if (!wait_w(smem_u32(&tl->p_full[sb.idx]), sb.phase, tl, 204)) return;  // also: O rescaled if it had to be
+            if (i == 0) {
+                if (!wait_w(smem_u32(&tl->o_free), free_par, tl, 206)) return;  // the previous pair's O has been read
+                free_par ^= 1;
+            }
             tc_fence_after();
-            const unsigned d_tmem = tmem_base + 256 + gi * 128;
-            const unsigned a_lo = p_lo + gi * (kPBytes >> 4), b_lo = v_lo + vs.idx * (kOperand >> 4);
-            const unsigned keep = ((fresh >> gi) & 1u) ^ 1u;
-            fresh &= ~(1u << gi);
+            const unsigned a_tmem = tmem_base + sb.idx * 128, b_lo = v_lo + vs.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
                 for (int tile = 0; tile < 2; ++tile) {  // row `tile` of the pair: its P rows, its V tile, its lanes
                     const unsigned lo_off = tile ? 0xFFFFFFFFu : 0u, hi_off = tile ? 0u : 0xFFFFFFFFu;
 #pragma unroll
-                    for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step
-                        tc_mma_bf16_split_masked(d_tmem, a_lo + ((s4 * 32) >> 4), kHiK, b_lo + ((tile * kTile + s4 * 2048) >> 4),
-                                                 kHiK, kIdescPV, s4 != 0 ? 1u : keep, lo_off, lo_off, hi_off, hi_off);
+                    for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step: 8 columns of packed bf16
+                        tc_mma_bf16_ta_masked(d_tmem, a_tmem + s4 * 8, b_lo + ((tile * kTile + s4 * 2048) >> 4), kHiK, kIdescPV,
+                                              (i | s4) != 0, lo_off, lo_off, hi_off, hi_off);
                 }
-                tc_commit(smem_u32(&tl->o_full[gi]));  // product added: the group's P buffer is free
+                tc_commit(smem_u32(&tl->s_free[sb.idx]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
+                if (i + 1 == n_entries) tc_commit(smem_u32(&tl->o_done));
             }
             __syncwarp();
             vs.advance(P.n_v_stages);
+            sb.advance(kSBufs);
         }
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
@@ -410,47 +451,31 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 // entries n with n % 2 == grp (n numbers the kept entries of each pair, as in every role).
 // The waits are warp-wide (same answer in every lane), so the warp stays converged for the
 // warp-collective TMEM loads and stores and leaves together if the CTA aborts.
-__device__ void softmax_role(const Params &P, Tail *tl, unsigned char *p_ptr, unsigned tmem_base, int t) {
+//
+// A parity wait needs the phase before it complete in the eyes of the waiting thread. Within a pair a
+// warp that comes to entry n has published n - 2 after it saw n - 3 published (`turn`), so
+// buffer n % 3's previous use is complete; everything of earlier pairs is, after o_done.
+__device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int t) {
     const Geom &g = P.g;
     const int lane = t & 31, row = t & 127, grp = t >> 7, half = row >> 6, mq = row & 63, wq = row >> 5;
-    const unsigned lane_off = (unsigned)(row & ~31) << 16;
-    // this thread's row of its group's P operand, and the same row in the other group's: the two
-    // exchange a few bytes there at the end of a pair
-    const int row_off = (row >> 3) * 1024 + (row & 7) * 128;
-    unsigned char *p_row = p_ptr + grp * kPBytes + row_off;
-    const unsigned char *p_row_other = p_ptr + (grp ^ 1) * kPBytes + row_off;
-    const int sw = row & 7;
-    const unsigned s_full = smem_u32(&tl->s_full[grp]), s_empty = smem_u32(&tl->s_empty[grp]),
-                   p_full = smem_u32(&tl->p_full[grp]), o_full = smem_u32(&tl->o_full[grp]), x_bar = smem_u32(&tl->x_bar[wq]);
-    const unsigned s_addr = tmem_base + grp * 128 + half * 64 + lane_off;
-    const unsigned o_own = tmem_base + 256 + grp * 128 + lane_off, o_other = tmem_base + 256 + (grp ^ 1) * 128 + lane_off;
-    unsigned s_par = 0, o_par = 0, x_par = 0;
+    const unsigned lanes = tmem_base + ((unsigned)(row & ~31) << 16);
+    const unsigned turn_own = smem_u32(&tl->turn[wq][grp]), turn_other = smem_u32(&tl->turn[wq][grp ^ 1]);
+    unsigned seq = 0;         // entries before this pair, over the whole kernel
+    unsigned n_other = 0;     // how many of them were the other group's
+    unsigned pair_par = 0;    // phase of the barriers that complete once per pair
     Ring ms;
-    for (int id = blockIdx.x; id < P.n_items; id += gridDim.x) {
+    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         const Item it = decode_item(P, id);
-        const long long tq = (long long)it.qb * kBlk + mq;
+        const long long tq = (long long)(half ? it.qb[1] : it.qb[0]) * kBlk + mq;
         const bool row_active = half < it.R && tq < g.T;
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 305)) return;
-        const int *rows = mask_rows(tl, P, ms.idx);
-        float ref = -CUDART_INF_F, l = 0.f;
-        bool ref_open = true;  // some token of this warp has no reference yet (the same in every lane)
-        bool pending = false;  // a P V chain of this group and pair may still be running
         const int n_entries = tl->m_count[ms.idx];
-        const int *my_row = rows + half * P.row_stride;  // this token's row of the pair
+        const int *my_row = mask_rows(tl, P, ms.idx) + half * P.row_stride;  // this token's row of the pair
+        float ref = -CUDART_INF_F, l = 0.f;
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
-            // the token's 64 logits against its row's key block
-            if (!wait_w(s_full, s_par, tl, 301)) return;
-            s_par ^= 1;
-            tc_fence_after();
-            unsigned sr[64];
-            tmem_ld_32x32_issue(s_addr, sr);
-            tmem_ld_32x32_issue(s_addr + 32, sr + 32);
-            tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(s_empty);
-            // keys of the block this token may attend: a prefix of n_hi keys (inside T, not after it if causal)
+            const unsigned use = (seq + (unsigned)n) / kSBufs, buf = seq + (unsigned)n - use * kSBufs;
             const int blk = my_row[n];
+            // keys of the block this token may attend: a prefix of n_hi keys (inside T, not after it if causal)
             int n_hi = 0;
             if (blk >= 0 && row_active) {
                 const long long k0 = (long long)blk * kBlk;
@@ -458,137 +483,130 @@ __device__ void softmax_role(const Params &P, Tail *tl, unsigned char *p_ptr, un
                 if (g.causal) lim = min(lim, tq - k0 + 1);
                 n_hi = (int)max(0ll, min(lim, (long long)kBlk));
             }
-            const bool all_keys = n_hi == kBlk;  // every block but the diagonal one and the one across T
-            // P = exp2(scale (s - ref)) under the token's current reference, their sum, the packed row.
-            // No reference yet (+inf shift: any allowed logit then gives +inf) or a logit that has
-            // outgrown the reference by more than kLazyLog2 both show in the sum of the 64 P, which
-            // is needed anyway: the maximum itself is only taken when that happens.
+            // the token's 64 logits against its row's key block
+            if (!wait_w(smem_u32(&tl->s_full[buf]), use & 1u, tl, 301)) return;
+            tc_fence_after();
+            unsigned sr[64];
+            tmem_ld_32x32_issue(lanes + buf * 128 + half * 64, sr);
+            tmem_ld_32x32_issue(lanes + buf * 128 + half * 64 + 32, sr + 32);
+            tmem_ld_wait();
+            if (__any_sync(0xffffffffu, n_hi != kBlk)) {  // the diagonal block, one across T, a row without one
+#pragma unroll
+                for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
+            }
+            // the pair's first entry sets the references of the tokens it has keys for
+            if (n == 0) {
+                ref = max_of_64(reinterpret_cast<const float *>(sr));
+                tl->ref[row] = ref;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&tl->ref_set[wq]));
+            } else if (n == 1) {
+                if (!wait_w(smem_u32(&tl->ref_set[wq]), pair_par, tl, 307)) return;
+                ref = tl->ref[row];
+            }
+            // P under the present reference, their sum, the packed row. A token without a reference, or
+            // with a logit that has outgrown it, shows in the sum, and a reference the other group has
+            // moved meanwhile in shared memory: then once more.
             unsigned packed[32];
             float esum;
-            auto make_p = [&](float shift) {
-                float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-                if (all_keys) {
+            for (int attempt = 0;; ++attempt) {
+                const float shift = ref == -CUDART_INF_F ? 0.f : -ref * P.scale_log2;
+                const unsigned long long scale2 = pack_f32x2(P.scale_log2, P.scale_log2), shift2 = pack_f32x2(shift, shift);
+                unsigned long long sum2[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-                    for (int i = 0; i < 64; i += 2) {
-                        const float p0 = fast_exp2(fmaf(__uint_as_float(sr[i]), P.scale_log2, shift));
-                        const float p1 = fast_exp2(fmaf(__uint_as_float(sr[i + 1]), P.scale_log2, shift));
-                        sum4[(i >> 1) & 3] += p0 + p1;
-                        __nv_bfloat162 pk = __floats2bfloat162_rn(p0, p1);
-                        packed[i >> 1] = *reinterpret_cast<unsigned *>(&pk);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 64; i += 2) {
-                        float p0 = fast_exp2(fmaf(__uint_as_float(sr[i]), P.scale_log2, shift));
-                        float p1 = fast_exp2(fmaf(__uint_as_float(sr[i + 1]), P.scale_log2, shift));
-                        p0 = i < n_hi ? p0 : 0.f;
-                        p1 = i + 1 < n_hi ? p1 : 0.f;
-                        sum4[(i >> 1) & 3] += p0 + p1;
-                        __nv_bfloat162 pk = __floats2bfloat162_rn(p0, p1);
-                        packed[i >> 1] = *reinterpret_cast<unsigned *>(&pk);
-                    }
+                for (int i = 0; i < 64; i += 2) {
+                    float x0, x1;
+                    unpack_f32x2(fma_f32x2(pack_u32x2(sr[i], sr[i + 1]), scale2, shift2), x0, x1);
+                    const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                    sum2[(i >> 1) & 3] = add_f32x2(sum2[(i >> 1) & 3], pack_f32x2(p0, p1));
+                    const __nv_bfloat162 pk = __floats2bfloat162_rn(p0, p1);
+                    packed[i >> 1] = *reinterpret_cast<const unsigned *>(&pk);
                 }
-                esum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-            };
-            auto masked_max = [&]() {
-                float x[64];
-#pragma unroll
-                for (int i = 0; i < 64; ++i) x[i] = i < n_hi ? __uint_as_float(sr[i]) : -CUDART_INF_F;
-                return max_of_64(x);
-            };
-            // the token's first allowed logits set its reference (once per pair)
-            if (ref_open && __any_sync(0xffffffffu, ref == -CUDART_INF_F && n_hi > 0)) {
-                const float mx = masked_max();
-                if (ref == -CUDART_INF_F) ref = mx;
-                ref_open = __any_sync(0xffffffffu, ref == -CUDART_INF_F);
-            }
-            make_p(ref == -CUDART_INF_F ? 0.f : -ref * P.scale_log2);
-            const bool redo = !(esum <= kLazySum);
-            // this group's previous chain of the pair must be done before its P buffer is rewritten
-            // or its O lane rescaled
-            if (pending) {
-                if (!wait_w(o_full, o_par, tl, 302)) return;
-                o_par ^= 1;
-                tc_fence_after();
-            }
-            if (__any_sync(0xffffffffu, redo)) {  // rare: a logit has outgrown the token's reference
-                const float mx = masked_max();
-                float f = 1.f;
-                if (redo) {
-                    f = fast_exp2((ref - mx) * P.scale_log2);
-                    ref = mx;
+                float e0, e1;
+                unpack_f32x2(add_f32x2(add_f32x2(sum2[0], sum2[1]), add_f32x2(sum2[2], sum2[3])), e0, e1);
+                esum = e0 + e1;
+                if (n > 0 && attempt == 0) {  // entry n - 1 of this lane quarter is published
+                    if (!wait_w(turn_other, (n_other + (unsigned)((n - 1) >> 1)) & 1u, tl, 308)) return;
                 }
-                // what the group has accumulated for this token is brought to the new reference
-                rescale_lane(o_own, f);
-                l *= f;
-                if (redo) make_p(-ref * P.scale_log2);
+                const float now = n > 0 ? tl->ref[row] : ref;
+                const bool moved = __float_as_uint(now) != __float_as_uint(ref);
+                const bool outgrown = (ref == -CUDART_INF_F && n_hi > 0) || !(esum <= kLazySum);
+                // (no attempt beyond the third: a reference moves at most once under each group's hands)
+                if (attempt == 2 || !__any_sync(0xffffffffu, moved || outgrown)) break;
+                if (moved) {
+                    if (ref != -CUDART_INF_F) l *= fast_exp2((ref - now) * P.scale_log2);
+                    ref = now;
+                }
+                const bool move = outgrown && !moved;
+                if (__any_sync(0xffffffffu, move)) {
+                    float f = 1.f;
+                    if (move) {
+                        const float mx = max_of_64(reinterpret_cast<const float *>(sr));
+                        if (ref != -CUDART_INF_F) f = fast_exp2((ref - mx) * P.scale_log2);
+                        ref = mx;
+                        tl->ref[row] = ref;
+                    }
+                    if (n > 0) {  // what has been added up so far is brought to the new reference
+                        const unsigned pu = (seq + (unsigned)n - 1u) / kSBufs, pb = seq + (unsigned)n - 1u - pu * kSBufs;
+                        if (!wait_w(smem_u32(&tl->s_free[pb]), pu & 1u, tl, 302)) return;
+                        tc_fence_after();
+                        rescale_lane(lanes + kOCol, f);
+                    }
+                    l *= f;
+                }
             }
             l += esum;
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                *reinterpret_cast<uint4 *>(p_row + ((c ^ sw) << 4)) =
-                    make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
-            fence_async_smem();
-            tc_fence_before();  // the rescaled O lane, if any, is in place
+            tmem_st_32x32_issue(lanes + buf * 128, packed);
+            tmem_st_wait();
+            tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(p_full);
-            pending = true;
+            if (lane == 0) {
+                mbar_arrive(turn_own);
+                mbar_arrive(smem_u32(&tl->p_full[buf]));
+            }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         ms.advance(kMaskSlots);
-        // End of the pair: bring the two groups' sums to a common reference and store.
-        if (pending) {
-            if (!wait_w(o_full, o_par, tl, 303)) return;
-            o_par ^= 1;
-            tc_fence_after();
-        }
-        *reinterpret_cast<float2 *>(p_row) = make_float2(ref, l);  // the P row is free: use it as mailbox
-        __syncwarp();
-        if (lane == 0) mbar_arrive(x_bar);
-        if (!wait_w(x_bar, x_par, tl, 304)) return;
-        x_par ^= 1;
-        tc_fence_after();  // the other group's last chain is complete too
-        const float2 oth = *reinterpret_cast<const float2 *>(p_row_other);
-        const float top = fmaxf(ref, oth.x);
-        const float f_own = ref == -CUDART_INF_F ? 0.f : fast_exp2((ref - top) * P.scale_log2);
-        const float f_oth = oth.x == -CUDART_INF_F ? 0.f : fast_exp2((oth.x - top) * P.scale_log2);
-        const float total = l * f_own + oth.y * f_oth;
-        const float inv = total > 0.f ? 1.f / total : 0.f;
-        const float w_own = f_own * inv, w_oth = f_oth * inv;
-        // this group stores channels 64 grp .. 64 grp + 63 of every token
         uint4 out_words[8];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            unsigned ra[32], rb[32];
-            tmem_ld_32x32_issue(o_own + grp * 64 + c * 32, ra);
-            tmem_ld_32x32_issue(o_other + grp * 64 + c * 32, rb);
+        if (n_entries > 0) {
+            if (!wait_w(smem_u32(&tl->o_done), pair_par, tl, 303)) return;
+            tc_fence_after();
+            // both groups' sums, under the pair's last reference
+            const float now = tl->ref[row];
+            if (ref != -CUDART_INF_F && now != ref) l *= fast_exp2((ref - now) * P.scale_log2);
+            tl->sum[grp][row] = l;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tl->sums_there[wq]));
+            unsigned ra[64];  // this group stores channels 64 grp .. 64 grp + 63 of every token
+            tmem_ld_32x32_issue(lanes + kOCol + grp * 64, ra);
+            tmem_ld_32x32_issue(lanes + kOCol + grp * 64 + 32, ra + 32);
             tmem_ld_wait();
+            tc_fence_before();
+            if (!wait_w(smem_u32(&tl->sums_there[wq]), pair_par, tl, 304)) return;
+            const float total = l + tl->sum[grp ^ 1][row];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tl->o_free));
+            const float inv = total > 0.f ? 1.f / total : 0.f;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int c = 0; c < 8; ++c) {
                 unsigned w[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int i = 8 * j + 2 * u;
-                    // a group without entries in this pair holds stale numbers: weight 0 means "leave out"
-                    const float a0 = w_own != 0.f ? __uint_as_float(ra[i]) * w_own : 0.f;
-                    const float a1 = w_own != 0.f ? __uint_as_float(ra[i + 1]) * w_own : 0.f;
-                    const float v0 = w_oth != 0.f ? fmaf(__uint_as_float(rb[i]), w_oth, a0) : a0;
-                    const float v1 = w_oth != 0.f ? fmaf(__uint_as_float(rb[i + 1]), w_oth, a1) : a1;
-                    __nv_bfloat162 pk = __floats2bfloat162_rn(v0, v1);
-                    w[u] = *reinterpret_cast<unsigned *>(&pk);
+                    const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(ra[8 * c + 2 * u]) * inv, __uint_as_float(ra[8 * c + 2 * u + 1]) * inv);
+                    w[u] = *reinterpret_cast<const unsigned *>(&pk);
                 }
-                out_words[c * 4 + j] = make_uint4(w[0], w[1], w[2], w[3]);
+                out_words[c] = make_uint4(w[0], w[1], w[2], w[3]);
             }
+            pair_par ^= 1;
+            seq += (unsigned)n_entries;
+            n_other += (unsigned)(grp == 0 ? n_entries >> 1 : (n_entries + 1) >> 1);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) out_words[c] = make_uint4(0, 0, 0, 0);
         }
-        // second meeting: both groups have read both O buffers and both mailboxes
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(x_bar);
-        if (!wait_w(x_bar, x_par, tl, 306)) return;
-        x_par ^= 1;
         if (row_active) {
-            uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)it.b * g.H + it.h0 + half) * g.T + tq) * kD + grp * 64);
+            uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)it.b * g.H + (half ? it.h[1] : it.h[0])) * g.T + tq) * kD + grp * 64);
 #pragma unroll
             for (int c = 0; c < 8; ++c) dst[c] = out_words[c];
         }
@@ -602,11 +620,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     // what is left behind the aligned base decides the number of V and K stages (the same in every thread)
     const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
-    const int n_rings = (P.smem_bytes - fixed_bytes) / kOperand - kFixedOperands;  // buffers for the two rings: 4 or 5
+    const int n_rings = (P.smem_bytes - fixed_bytes) / kOperand - kFixedOperands;  // buffers for the two rings: 4 to 6
     P.n_v_stages = n_rings >= 5 ? 3 : 2;
     P.n_k_stages = min(kMaxKStages, n_rings - P.n_v_stages);
-    const unsigned q_smem = smem_u32(smem), p_smem = q_smem + kOperand, v_smem = p_smem + 2 * kPBytes,
-                   k_smem = v_smem + P.n_v_stages * kOperand;
+    const unsigned q_smem = smem_u32(smem), v_smem = q_smem + kOperand, k_smem = v_smem + P.n_v_stages * kOperand;
     Tail *tl = (Tail *)(smem + (kFixedOperands + P.n_v_stages + P.n_k_stages) * kOperand);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -615,11 +632,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         mbar_init(smem_u32(&tl->q_empty), 1);
         for (int i = 0; i < kMaxKStages; ++i) { mbar_init(smem_u32(&tl->k_full[i]), 1); mbar_init(smem_u32(&tl->k_empty[i]), 1); }
         for (int i = 0; i < kMaxVStages; ++i) { mbar_init(smem_u32(&tl->v_full[i]), 1); mbar_init(smem_u32(&tl->v_empty[i]), 1); }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(smem_u32(&tl->s_full[i]), 1); mbar_init(smem_u32(&tl->s_empty[i]), 4);
-            mbar_init(smem_u32(&tl->p_full[i]), 4); mbar_init(smem_u32(&tl->o_full[i]), 1);
+        for (int i = 0; i < kSBufs; ++i) {
+            mbar_init(smem_u32(&tl->s_full[i]), 1);
+            mbar_init(smem_u32(&tl->p_full[i]), 4);
+            mbar_init(smem_u32(&tl->s_free[i]), 1);
         }
-        for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&tl->x_bar[i]), 2);
+        mbar_init(smem_u32(&tl->o_done), 1);
+        mbar_init(smem_u32(&tl->o_free), 8);
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(smem_u32(&tl->ref_set[i]), 1);
+            mbar_init(smem_u32(&tl->turn[i][0]), 1);
+            mbar_init(smem_u32(&tl->turn[i][1]), 1);
+            mbar_init(smem_u32(&tl->sums_there[i]), 2);
+        }
         for (int i = 0; i < kMaskSlots; ++i) { mbar_init(smem_u32(&tl->m_full[i]), 1); mbar_init(smem_u32(&tl->m_empty[i]), 12); }
         tl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -637,9 +662,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     } else if (warp == 2) {
         mask_loader_role(P, tl, lane);
     } else if (warp == 3) {
-        pv_role(P, tl, p_smem, v_smem, tmem_base);
+        pv_role(P, tl, v_smem, tmem_base);
     } else {
-        softmax_role(P, tl, smem + kOperand, tmem_base, (int)threadIdx.x - 128);
+        softmax_role(P, tl, tmem_base, (int)threadIdx.x - 128);
     }
     __syncwarp();
 
@@ -670,27 +695,30 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
         return STREAM_ERR_UNSUPPORTED;
     }
     CUtensorMap tq, tk, tv;
-    stream_status rc = make_map5_bf16_d128(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, 2, "q");
+    stream_status rc = make_map_bf16_d128(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q");  // 4-D: 64 x 64 half tiles
     if (rc != STREAM_OK) return rc;
-    rc = make_map_bf16_d128(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k");  // 4-D: 64 x 64 half tiles
+    rc = make_map_bf16_d128(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k");
     if (rc != STREAM_OK) return rc;
-    rc = make_map5_bf16_d128(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, 1, "v");
+    rc = make_map5_bf16_d128(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v");
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;
-    P.n_pairs = (g.hpg + 1) / 2;
-    const long long n_items = (long long)g.batch * g.G * g.n_qb * P.n_pairs;
+    const long long kv_bytes = 2ll * g.T * kD * 2;  // K and V of one kv head
+    const long long fit = kL2KvBytes / kv_bytes, all = (long long)g.batch * g.G;
+    P.group_heads = (int)(fit < 1 ? 1 : (fit > all ? all : fit));
+    const long long n_items = all * ((g.n_qb + 1) / 2) * (2 * (g.hpg / 2) + g.hpg % 2);
+    if (n_items > 0x7fffffffLL - (1 << 20)) { set_error("too many rows for 32-bit indexing"); return STREAM_ERR_UNSUPPORTED; }
     P.n_items = (int)n_items;
     P.mask = mask;
     P.out = (__nv_bfloat16 *)out;
     P.scale_log2 = scale * 1.4426950408889634f;
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    // room for five ring buffers (three V, two K) if the mask rows are short enough, else four; 1 KB of slack for the
-    // alignment of the base (the kernel counts its stages from what it really gets)
+    // room for up to six ring buffers, as many as the mask rows leave; 1 KB of slack for the alignment
+    // of the base (the kernel counts its stages from what it really gets)
     P.row_stride = (g.k_top + 3) & ~3;
     const int tail_bytes = (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
-    int smem_bytes = (kFixedOperands + 5) * kOperand + tail_bytes + 1024;
+    int smem_bytes = (kFixedOperands + 6) * kOperand + tail_bytes + 1024;
     if (smem_bytes > kMaxSmemPerCta) smem_bytes = kMaxSmemPerCta;
     if (smem_bytes < (kFixedOperands + 4) * kOperand + tail_bytes + 1024) {
         set_error("tensor-core attention kernel: k_top = %d needs more shared memory than one CTA has", g.k_top);

@@ -137,17 +137,37 @@ __device__ __forceinline__ void tc_mma_bf16_split(unsigned d_tmem, unsigned a_lo
         : "memory");
 }
 
-// The same with an output-lane mask: bit i of the 128-bit vector {m0 (lanes 0..31), m1, m2, m3}
-// set = accumulator lane i is left untouched by this instruction.
-__device__ __forceinline__ void tc_mma_bf16_split_masked(unsigned d_tmem, unsigned a_lo, unsigned a_hi, unsigned b_lo,
-                                                         unsigned b_hi, unsigned idesc, unsigned accumulate, unsigned m0,
-                                                         unsigned m1, unsigned m2, unsigned m3) {
+// The same with A from TMEM (lane = row, two bf16 per column) and an output-lane mask: bit i of the
+// 128-bit vector {m0 (lanes 0..31), m1, m2, m3} set = accumulator lane i is left untouched.
+__device__ __forceinline__ void tc_mma_bf16_ta_masked(unsigned d_tmem, unsigned a_tmem, unsigned b_lo, unsigned b_hi,
+                                                      unsigned idesc, unsigned accumulate, unsigned m0, unsigned m1,
+                                                      unsigned m2, unsigned m3) {
     asm volatile(
-        "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\nsetp.ne.b32 p, %6, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, {%7, %8, %9, %10}, p;\n}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(m0), "r"(m1), "r"(m2),
-          "r"(m3)
+        "{\n.reg .pred p;\n.reg .b64 db;\nmov.b64 db, {%2, %3};\nsetp.ne.b32 p, %5, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, {%6, %7, %8, %9}, p;\n}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(m0), "r"(m1), "r"(m2), "r"(m3)
         : "memory");
+}
+
+// Two fp32 in a register pair: one instruction for both.
+__device__ __forceinline__ unsigned long long pack_u32x2(unsigned a, unsigned b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long pack_f32x2(float a, float b) { return pack_u32x2(__float_as_uint(a), __float_as_uint(b)); }
+__device__ __forceinline__ void unpack_f32x2(unsigned long long x, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
+}
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 __device__ __forceinline__ void tmem_alloc_512(unsigned smem_dst) {
@@ -338,18 +358,17 @@ inline stream_status make_map_bf16_d128(CUtensorMap *map, const void *base, long
 
 // The same tensor seen as [batch, heads, 2 channel halves, T, 64]: one box brings a whole
 // 64-token x 128-channel tile (16 KB) as [half][64 rows][128 B], the layout of a 128-byte-swizzled
-// K-major (or, read along the rows, MN-major) tcgen05 operand. With heads_in_box = 2 the two
-// heads h, h + 1 land as [half][head][64 rows][128 B]: a 128-row operand per half.
+// K-major (or, read along the rows, MN-major) tcgen05 operand.
 // Coordinates: (0, token, head, 0, batch) with the half as dimension 3.
 inline stream_status make_map5_bf16_d128(CUtensorMap *map, const void *base, long long T, int heads, int batch,
-                                         long long s_t, long long s_h, long long s_b, int heads_in_box, const char *what) {
+                                         long long s_t, long long s_h, long long s_b, const char *what) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return STREAM_ERR_CUDA; }
     if (heads == 1) s_h = s_t * T;
     if (batch == 1) s_b = s_h * heads;
     cuuint64_t dims[5] = {64, (cuuint64_t)T, (cuuint64_t)heads, 2, (cuuint64_t)batch};
     cuuint64_t strides[4] = {(cuuint64_t)s_t * 2, (cuuint64_t)s_h * 2, 128, (cuuint64_t)s_b * 2};
-    cuuint32_t box[5] = {64, 64, (cuuint32_t)heads_in_box, 2, 1}, estr[5] = {1, 1, 1, 1, 1};
+    cuuint32_t box[5] = {64, 64, 1, 2, 1}, estr[5] = {1, 1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
