@@ -60,20 +60,27 @@ constexpr int kBlk = 64, kD = 128;
 constexpr int kHalfTile = kBlk * 128;       // 64 rows x 128 bytes
 constexpr int kTile = 2 * kHalfTile;        // one 64 x 128 tile
 constexpr int kOperand = 2 * kTile;         // two tiles (K_a, K_b or V_a, V_b), or the 128-row Q operand
-// Stages of the two rings, out of the operand buffers shared memory has room for beside Q: six when
-// the mask rows are short (three each), else five (a V stage is held from its load until the
-// product of its entry is complete, a whole softmax later: V three, K two) or four.
-constexpr int kMaxKStages = 3, kMaxVStages = 3;
+// Stages of the two rings, out of the operand buffers shared memory has room for beside Q: five (a V
+// stage is held from its load until the product of its entry is complete, a whole softmax later:
+// V three, K two), or four when the mask rows are long.
+constexpr int kMaxKStages = 2, kMaxVStages = 3;
 constexpr int kSBufs = 3;                   // logit buffers: entry n of the kernel's sequence uses buffer n % 3
 constexpr int kMaskSlots = 2;               // pairs whose mask rows are resident
 constexpr int kMaxKTopTc = 1024;
 constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while pairs of several heads are walked
 constexpr float kLazySum = 68719476736.f;   // 2^36 = 64 * 2^30: the 64 P of an entry add up to more only if one of them exceeds 2^30 (its logit has outgrown the reference by 30 in log2 units)
 
+// The pair a CTA works on. h[r], qb[r]: head and query block of row r < R (R = 0: a place of the
+// order without a pair).
+struct Item {
+    int b, kvh, R;
+    int h[2], qb[2];
+};
+
 // TMEM columns: S / P buffer b at 128 b (P: its first 32), O at 384.
 constexpr int kOCol = kSBufs * 128;
 struct Tail {
-    unsigned long long q_full, q_empty;
+    unsigned long long q_full[2], q_free[2];  // q_free: the output staged over the pair's Q has left (8 warps)
     unsigned long long k_full[kMaxKStages], k_empty[kMaxKStages], v_full[kMaxVStages], v_empty[kMaxVStages];
     unsigned long long s_full[kSBufs], p_full[kSBufs], s_free[kSBufs];  // logits ready, P in their place, product added
     unsigned long long o_done, o_free;     // a pair's last product is complete; its O has been read (8 warps)
@@ -84,11 +91,13 @@ struct Tail {
     unsigned int tmem_base;
     int abort_flag;
     int m_count[kMaskSlots];  // kept entries of the pair in each mask slot
+    Item m_item[kMaskSlots];  // and the pair itself
     float ref[128], sum[2][128];
 };
-// Dynamic shared memory: Q | V stages | K stages | Tail | mask rows [kMaskSlots][2][row_stride] (-1
-// where a row has nothing), the operands 1024-byte aligned.
-constexpr int kFixedOperands = 1;  // Q; behind it the V stages, then the K stages
+// Dynamic shared memory: Q (two buffers; a pair's output is staged over its Q) | V stages | K stages |
+// Tail | mask rows [kMaskSlots][2][row_stride] (-1 where a row has nothing), the operands 1024-byte
+// aligned.
+constexpr int kFixedOperands = 2;  // Q; behind it the V stages, then the K stages
 constexpr int kMaxSmemPerCta = 232448;
 
 constexpr unsigned kIdescQK = idesc_bf16(128, 128, false);  // B = stacked K tiles, K-major
@@ -120,13 +129,6 @@ __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail *tl, 
 __device__ __forceinline__ int *mask_rows(Tail *tl, const Params &P, int slot) {
     return reinterpret_cast<int *>(tl + 1) + slot * 2 * P.row_stride;
 }
-
-// The pair a CTA works on. h[r], qb[r]: head and query block of row r < R (R = 0: a place of the
-// order without a pair).
-struct Item {
-    int b, kvh, R;
-    int h[2], qb[2];
-};
 
 // A CTA's n-th place in the order of pairs. Every second round runs backwards, so that with pairs in
 // order of falling length every CTA gets about the same sum.
@@ -211,6 +213,7 @@ __device__ void mask_loader_role(const Params &P, Tail *tl, int lane) {
         __syncwarp();
         if (lane == 0) {
             tl->m_count[ms.idx] = cnt;
+            tl->m_item[ms.idx] = it;
             mbar_arrive(smem_u32(&tl->m_full[ms.idx]));
         }
         ms.advance(kMaskSlots);
@@ -238,7 +241,7 @@ __device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
 
 __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, const CUtensorMap *tv,
                               Tail *tl, unsigned q_smem, unsigned k_smem, unsigned v_smem) {
-    unsigned q_par = 0;
+    Ring qs;
     LoadStream K, V;
     K.round = V.round = 0;
     K.id = V.id = nth_item(P, 0);
@@ -266,7 +269,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
         const int *rows = mask_rows(tl, P, S.ms.idx);
         if (S.e == -2) {  // open the pair: its mask rows must be resident
             if (!probe_w(smem_u32(&tl->m_full[S.ms.idx]), S.ms.phase)) return false;
-            S.it = decode_item(P, S.id);
+            S.it = tl->m_item[S.ms.idx];
             S.n = tl->m_count[S.ms.idx];
             S.e = 0;
             if (S.n > 0) S.cur = entry_at(rows, P.row_stride, 0);
@@ -294,22 +297,22 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
                 return true;
             }
             // Q goes behind the pair's first K tiles, which do not depend on the Q buffer
-            if (!probe_w(smem_u32(&tl->q_empty), q_par ^ 1)) return false;
-            q_par ^= 1;
+            if (!probe_w(smem_u32(&tl->q_free[qs.idx]), qs.phase ^ 1)) return false;
             if (elect_one()) {
-                const unsigned bar = smem_u32(&tl->q_full);
+                const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
                 mbar_arrive_expect_tx(bar, (unsigned)kOperand);
 #pragma unroll
                 for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         const bool second = r == 1 && S.it.R == 2;
-                        tma_load_4d(q_smem + (2 * c + r) * kHalfTile, tq, bar, c * 64, (second ? S.it.qb[1] : S.it.qb[0]) * kBlk,
+                        tma_load_4d(q_smem + qs.idx * kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64, (second ? S.it.qb[1] : S.it.qb[0]) * kBlk,
                                     second ? S.it.h[1] : S.it.h[0], S.it.b);
                     }
             }
             __syncwarp();
             S.q_due = false;
+            qs.advance(2);
             return true;
         }
         // a V stage is free once the product computed from it is complete
@@ -337,7 +340,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
                 }
             }
             if (__shfl_sync(0xffffffffu, stop, 0)) return;
-            __nanosleep(200);  // leave the issue slots to the softmax warps of this scheduler
+            __nanosleep(40);  // leave the issue slots to the softmax warps of this scheduler
         }
     }
 }
@@ -347,15 +350,15 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
 
 // S = [Q_0; Q_1] [K_a; K_b]^T for every kept entry.
 __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base) {
-    Ring ks, ms, sb;
-    unsigned q_par = 0;
-    const unsigned q_lo = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
+    Ring ks, ms, sb, qs;
+    const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
     for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
         const int n_entries = tl->m_count[ms.idx];  // the issuers need no more than the count
+        const unsigned q_lo = q_lo0 + qs.idx * (kOperand >> 4);
         if (n_entries > 0) {
-            if (!wait_w(smem_u32(&tl->q_full), q_par, tl, 201)) return;
-            q_par ^= 1;
+            if (!wait_w(smem_u32(&tl->q_full[qs.idx]), qs.phase, tl, 201)) return;
+            qs.advance(2);
         }
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, tl, 202)) return;
@@ -372,7 +375,6 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
                                           b_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
                 tc_commit(smem_u32(&tl->s_full[sb.idx]));
                 tc_commit(smem_u32(&tl->k_empty[ks.idx]));
-                if (i + 1 == n_entries) tc_commit(smem_u32(&tl->q_empty));  // that was the pair's last use of Q
             }
             __syncwarp();
             ks.advance(P.n_k_stages);
@@ -455,42 +457,52 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 // A parity wait needs the phase before it complete in the eyes of the waiting thread. Within a pair a
 // warp that comes to entry n has published n - 2 after it saw n - 3 published (`turn`), so
 // buffer n % 3's previous use is complete; everything of earlier pairs is, after o_done.
-__device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int t) {
+__device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
     const Geom &g = P.g;
     const int lane = t & 31, row = t & 127, grp = t >> 7, half = row >> 6, mq = row & 63, wq = row >> 5;
     const unsigned lanes = tmem_base + ((unsigned)(row & ~31) << 16);
     const unsigned turn_own = smem_u32(&tl->turn[wq][grp]), turn_other = smem_u32(&tl->turn[wq][grp ^ 1]);
-    unsigned seq = 0;         // entries before this pair, over the whole kernel
-    unsigned n_other = 0;     // how many of them were the other group's
-    unsigned pair_par = 0;    // phase of the barriers that complete once per pair
-    Ring ms;
-    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
-        const Item it = decode_item(P, id);
-        const long long tq = (long long)(half ? it.qb[1] : it.qb[0]) * kBlk + mq;
-        const bool row_active = half < it.R && tq < g.T;
+    unsigned char *const stage = q_ptr + (grp * 4 + wq) * 4096;  // this warp's 32 tokens x 64 channels in a Q buffer
+    unsigned n_other = 0;     // entries of the other group before this pair, over the whole kernel
+    unsigned pair_par = 0;    // phase of the barriers that complete once per pair with entries
+    int staged = -1;          // Q buffer whose staged output may still be on its way out
+    Ring ms, sb, qs;          // sb: buffer of the pair's first entry
+    auto release_stage = [&]() {
+        if (staged < 0) return;
+        if (lane == 0) {
+            tma_store_wait_read();
+            mbar_arrive(smem_u32(&tl->q_free[staged]));
+        }
+        __syncwarp();
+        staged = -1;
+    };
+    for (int round = 0; nth_item(P, round) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 305)) return;
+        const Item &it = tl->m_item[ms.idx];
+        const int h = half ? it.h[1] : it.h[0], qb = half ? it.qb[1] : it.qb[0], b = it.b;
+        const int tq0 = qb * kBlk;  // (token numbers fit 32 bits: TMA coordinates)
+        const bool row_active = half < it.R && tq0 + mq < g.T;
+        const int key_end = row_active ? (g.causal ? tq0 + mq + 1 : (int)g.T) : 0;  // keys this token may attend: those before
         const int n_entries = tl->m_count[ms.idx];
         const int *my_row = mask_rows(tl, P, ms.idx) + half * P.row_stride;  // this token's row of the pair
         float ref = -CUDART_INF_F, l = 0.f;
+        Ring eb = sb;  // buffer of entry n, with the phase of its use
+        if (grp) eb.advance(kSBufs);
+        int blk = grp < n_entries ? my_row[grp] : -1;
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
-            const unsigned use = (seq + (unsigned)n) / kSBufs, buf = seq + (unsigned)n - use * kSBufs;
-            const int blk = my_row[n];
-            // keys of the block this token may attend: a prefix of n_hi keys (inside T, not after it if causal)
-            int n_hi = 0;
-            if (blk >= 0 && row_active) {
-                const long long k0 = (long long)blk * kBlk;
-                long long lim = g.T - k0;
-                if (g.causal) lim = min(lim, tq - k0 + 1);
-                n_hi = (int)max(0ll, min(lim, (long long)kBlk));
-            }
+            const unsigned buf = (unsigned)eb.idx;
+            // keys of the block this token may attend: a prefix of n_hi
+            const int n_hi = blk >= 0 ? max(0, min(key_end - blk * kBlk, kBlk)) : 0;
+            const bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
+            blk = n + 2 < n_entries ? my_row[n + 2] : -1;
             // the token's 64 logits against its row's key block
-            if (!wait_w(smem_u32(&tl->s_full[buf]), use & 1u, tl, 301)) return;
+            if (!wait_w(smem_u32(&tl->s_full[buf]), eb.phase, tl, 301)) return;
             tc_fence_after();
             unsigned sr[64];
             tmem_ld_32x32_issue(lanes + buf * 128 + half * 64, sr);
             tmem_ld_32x32_issue(lanes + buf * 128 + half * 64 + 32, sr + 32);
             tmem_ld_wait();
-            if (__any_sync(0xffffffffu, n_hi != kBlk)) {  // the diagonal block, one across T, a row without one
+            if (masked) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
             }
@@ -506,32 +518,46 @@ __device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int 
             }
             // P under the present reference, their sum, the packed row. A token without a reference, or
             // with a logit that has outgrown it, shows in the sum, and a reference the other group has
-            // moved meanwhile in shared memory: then once more.
+            // moved meanwhile in shared memory: then once more. Whether entry n - 1 of this lane
+            // quarter is published is looked up halfway through, so that its latency is hidden.
+            const unsigned turn_par = (n_other + (unsigned)((n - 1) >> 1)) & 1u;
             unsigned packed[32];
             float esum;
             for (int attempt = 0;; ++attempt) {
                 const float shift = ref == -CUDART_INF_F ? 0.f : -ref * P.scale_log2;
                 const unsigned long long scale2 = pack_f32x2(P.scale_log2, P.scale_log2), shift2 = pack_f32x2(shift, shift);
                 unsigned long long sum2[4] = {0ull, 0ull, 0ull, 0ull};
+                auto weights = [&](int i0) {
 #pragma unroll
-                for (int i = 0; i < 64; i += 2) {
-                    float x0, x1;
-                    unpack_f32x2(fma_f32x2(pack_u32x2(sr[i], sr[i + 1]), scale2, shift2), x0, x1);
-                    const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-                    sum2[(i >> 1) & 3] = add_f32x2(sum2[(i >> 1) & 3], pack_f32x2(p0, p1));
-                    const __nv_bfloat162 pk = __floats2bfloat162_rn(p0, p1);
-                    packed[i >> 1] = *reinterpret_cast<const unsigned *>(&pk);
+                    for (int i = i0; i < i0 + 32; i += 2) {
+                        float x0, x1;
+                        unpack_f32x2(fma_f32x2(pack_u32x2(sr[i], sr[i + 1]), scale2, shift2), x0, x1);
+                        const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                        sum2[(i >> 1) & 3] = add_f32x2(sum2[(i >> 1) & 3], pack_f32x2(p0, p1));
+                        const __nv_bfloat162 pk = __floats2bfloat162_rn(p0, p1);
+                        packed[i >> 1] = *reinterpret_cast<const unsigned *>(&pk);
+                    }
+                };
+                weights(0);
+                bool seen = true;
+                float now = ref;
+                if (n > 0) {
+                    seen = mbar_test_wait(turn_other, turn_par);
+                    now = *(volatile float *)&tl->ref[row];
                 }
+                weights(32);
                 float e0, e1;
                 unpack_f32x2(add_f32x2(add_f32x2(sum2[0], sum2[1]), add_f32x2(sum2[2], sum2[3])), e0, e1);
                 esum = e0 + e1;
-                if (n > 0 && attempt == 0) {  // entry n - 1 of this lane quarter is published
-                    if (!wait_w(turn_other, (n_other + (unsigned)((n - 1) >> 1)) & 1u, tl, 308)) return;
-                }
-                const float now = n > 0 ? tl->ref[row] : ref;
-                const bool moved = __float_as_uint(now) != __float_as_uint(ref);
+                bool moved = __float_as_uint(now) != __float_as_uint(ref);
                 const bool outgrown = (ref == -CUDART_INF_F && n_hi > 0) || !(esum <= kLazySum);
                 // (no attempt beyond the third: a reference moves at most once under each group's hands)
+                if (!__any_sync(0xffffffffu, !seen || moved || outgrown)) break;
+                if (n > 0) {
+                    if (!wait_w(turn_other, turn_par, tl, 308)) return;
+                    now = *(volatile float *)&tl->ref[row];
+                    moved = __float_as_uint(now) != __float_as_uint(ref);
+                }
                 if (attempt == 2 || !__any_sync(0xffffffffu, moved || outgrown)) break;
                 if (moved) {
                     if (ref != -CUDART_INF_F) l *= fast_exp2((ref - now) * P.scale_log2);
@@ -547,8 +573,9 @@ __device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int 
                         tl->ref[row] = ref;
                     }
                     if (n > 0) {  // what has been added up so far is brought to the new reference
-                        const unsigned pu = (seq + (unsigned)n - 1u) / kSBufs, pb = seq + (unsigned)n - 1u - pu * kSBufs;
-                        if (!wait_w(smem_u32(&tl->s_free[pb]), pu & 1u, tl, 302)) return;
+                        Ring pb = eb;  // entry n - 1's buffer
+                        pb.retreat(kSBufs);
+                        if (!wait_w(smem_u32(&tl->s_free[pb.idx]), pb.phase, tl, 302)) return;
                         tc_fence_after();
                         rescale_lane(lanes + kOCol, f);
                     }
@@ -564,12 +591,15 @@ __device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int 
                 mbar_arrive(turn_own);
                 mbar_arrive(smem_u32(&tl->p_full[buf]));
             }
+            eb.advance(kSBufs);
+            eb.advance(kSBufs);
+            release_stage();  // the previous pair's output has long been read
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
+        if (lane == 0) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));  // (nothing of the slot is read below)
         ms.advance(kMaskSlots);
-        uint4 out_words[8];
         if (n_entries > 0) {
+            release_stage();
             if (!wait_w(smem_u32(&tl->o_done), pair_par, tl, 303)) return;
             tc_fence_after();
             // both groups' sums, under the pair's last reference
@@ -588,6 +618,10 @@ __device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int 
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tl->o_free));
             const float inv = total > 0.f ? 1.f / total : 0.f;
+            // The warp's 32 x 64 part goes to the pair's Q buffer, whose last product is complete, and
+            // from there to global memory as one TMA store (rows beyond T are left out): a lane's
+            // own 128 bytes stored directly would touch 32 lines with every instruction.
+            unsigned char *const dst = stage + qs.idx * kOperand + lane * 128;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 unsigned w[4];
@@ -596,40 +630,46 @@ __device__ void softmax_role(const Params &P, Tail *tl, unsigned tmem_base, int 
                     const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(ra[8 * c + 2 * u]) * inv, __uint_as_float(ra[8 * c + 2 * u + 1]) * inv);
                     w[u] = *reinterpret_cast<const unsigned *>(&pk);
                 }
-                out_words[c] = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4 *>(dst + ((c ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
             }
+            fence_async_smem();
+            __syncwarp();
+            const int tok = tq0 + (wq & 1) * 32;
+            if (lane == 0 && row_active) {  // lane 0 holds the first of the 32 tokens
+                tma_store_4d(to, smem_u32(stage + qs.idx * kOperand), grp * 64, tok, h, b);
+                tma_store_commit();
+            }
+            staged = qs.idx;
+            qs.advance(2);
             pair_par ^= 1;
-            seq += (unsigned)n_entries;
+            for (int i = n_entries % (2 * kSBufs); i > 0; --i) sb.advance(kSBufs);
             n_other += (unsigned)(grp == 0 ? n_entries >> 1 : (n_entries + 1) >> 1);
-        } else {
+        } else if (row_active) {
+            uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)b * g.H + h) * g.T + tq0 + mq) * kD + grp * 64);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) out_words[c] = make_uint4(0, 0, 0, 0);
-        }
-        if (row_active) {
-            uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)it.b * g.H + (half ? it.h[1] : it.h[0])) * g.T + tq) * kD + grp * 64);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) dst[c] = out_words[c];
+            for (int c = 0; c < 8; ++c) dst[c] = make_uint4(0, 0, 0, 0);
         }
     }
+    if (lane == 0) tma_store_wait_read();  // shared memory is given back when the CTA leaves
+    __syncwarp();
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
-               const __grid_constant__ CUtensorMap tmap_v, Params P) {  // P by value: n_k_stages is filled in here
+               const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_out, Params P) {  // P by value: n_k_stages is filled in here
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     // what is left behind the aligned base decides the number of V and K stages (the same in every thread)
     const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
-    const int n_rings = (P.smem_bytes - fixed_bytes) / kOperand - kFixedOperands;  // buffers for the two rings: 4 to 6
+    const int n_rings = (P.smem_bytes - fixed_bytes) / kOperand - kFixedOperands;  // buffers for the two rings: 4 or 5
     P.n_v_stages = n_rings >= 5 ? 3 : 2;
     P.n_k_stages = min(kMaxKStages, n_rings - P.n_v_stages);
-    const unsigned q_smem = smem_u32(smem), v_smem = q_smem + kOperand, k_smem = v_smem + P.n_v_stages * kOperand;
+    const unsigned q_smem = smem_u32(smem), v_smem = q_smem + kFixedOperands * kOperand, k_smem = v_smem + P.n_v_stages * kOperand;
     Tail *tl = (Tail *)(smem + (kFixedOperands + P.n_v_stages + P.n_k_stages) * kOperand);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        mbar_init(smem_u32(&tl->q_full), 1);
-        mbar_init(smem_u32(&tl->q_empty), 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), 8); }
         for (int i = 0; i < kMaxKStages; ++i) { mbar_init(smem_u32(&tl->k_full[i]), 1); mbar_init(smem_u32(&tl->k_empty[i]), 1); }
         for (int i = 0; i < kMaxVStages; ++i) { mbar_init(smem_u32(&tl->v_full[i]), 1); mbar_init(smem_u32(&tl->v_empty[i]), 1); }
         for (int i = 0; i < kSBufs; ++i) {
@@ -664,7 +704,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     } else if (warp == 3) {
         pv_role(P, tl, v_smem, tmem_base);
     } else {
-        softmax_role(P, tl, tmem_base, (int)threadIdx.x - 128);
+        softmax_role(P, &tmap_out, tl, smem, tmem_base, (int)threadIdx.x - 128);
     }
     __syncwarp();
 
@@ -694,12 +734,14 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
         set_error("tensor-core attention kernel needs 16-byte aligned q, k, v and out");
         return STREAM_ERR_UNSUPPORTED;
     }
-    CUtensorMap tq, tk, tv;
+    CUtensorMap tq, tk, tv, to;
     stream_status rc = make_map_bf16_d128(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q");  // 4-D: 64 x 64 half tiles
     if (rc != STREAM_OK) return rc;
     rc = make_map_bf16_d128(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k");
     if (rc != STREAM_OK) return rc;
     rc = make_map5_bf16_d128(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v");
+    if (rc != STREAM_OK) return rc;
+    rc = make_map_bf16_d128(&to, out, g.T, g.H, g.batch, kD, g.T * kD, (long long)g.H * g.T * kD, "out", 32);
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;
@@ -714,11 +756,11 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
     P.scale_log2 = scale * 1.4426950408889634f;
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    // room for up to six ring buffers, as many as the mask rows leave; 1 KB of slack for the alignment
+    // room for five ring buffers if the mask rows are short enough, else four; 1 KB of slack for the alignment
     // of the base (the kernel counts its stages from what it really gets)
     P.row_stride = (g.k_top + 3) & ~3;
     const int tail_bytes = (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
-    int smem_bytes = (kFixedOperands + 6) * kOperand + tail_bytes + 1024;
+    int smem_bytes = (kFixedOperands + 5) * kOperand + tail_bytes + 1024;
     if (smem_bytes > kMaxSmemPerCta) smem_bytes = kMaxSmemPerCta;
     if (smem_bytes < (kFixedOperands + 4) * kOperand + tail_bytes + 1024) {
         set_error("tensor-core attention kernel: k_top = %d needs more shared memory than one CTA has", g.k_top);
@@ -729,7 +771,7 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
     cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemPerCta);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_tc)");
     const int grid = (int)(n_items < n_sm ? n_items : n_sm);
-    attn_tc_kernel<<<grid, kThreads, smem_bytes, st>>>(tq, tk, tv, P);
+    attn_tc_kernel<<<grid, kThreads, smem_bytes, st>>>(tq, tk, tv, to, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "attn_tc launch");
     return STREAM_OK;

@@ -115,6 +115,16 @@ __device__ __forceinline__ void tma_load_5d(unsigned dst, const CUtensorMap *map
         : "memory");
 }
 
+// A box from shared to global memory (rows beyond the tensor are left out), in a bulk group.
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, unsigned src, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+                 ::"l"((unsigned long long)map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// Every box this thread has stored has been read from shared memory.
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // Makes this thread's shared-memory writes visible to the async proxy (TMA, tcgen05.mma operands).
@@ -315,6 +325,9 @@ struct Ring {  // position in a ring of barriers with phase tracking
     unsigned phase = 0;
     __device__ void advance(int n) {
         if (++idx == n) { idx = 0; phase ^= 1; }
+    }
+    __device__ void retreat(int n) {
+        if (--idx < 0) { idx = n - 1; phase ^= 1; }
     }
 };
 
