@@ -13,11 +13,14 @@
 // group n % 2, so that a pair's arithmetic does not depend on what the CTA did before), so
 // that one group's chain of waits, TMEM loads and exponentials runs beside the other's. A thread
 // owns one query token (TMEM lane) of its group's entries: it reads the token's 64 logits, applies
-// the element-level mask C, and writes P = exp2(scale (s - ref)) as bf16 back over the logits, where
-// the P V product takes it as its A operand from TMEM. Two chains with an output-lane mask,
+// the element-level mask C, and writes P = exp2(scale (s - ref)) as bf16 to TMEM, where the P V
+// product takes it as its A operand. Two chains with an output-lane mask,
 //     O[lanes 0..63]   += P[rows 0..63]   V_a,      O[lanes 64..127] += P[rows 64..127] V_b
 // (128 x 128, fp32, in TMEM; V tiles MN-major), add each row's contribution and leave the other
-// row's lanes alone. Three logit buffers and one O fill the 512 TMEM columns.
+// row's lanes alone. One logit buffer and two P buffers per group and one O fill the 512 TMEM
+// columns: the logits are given back as soon as they are in registers, and P need not wait for the
+// product before. (Three logit buffers with P in their place instead hold a buffer through Q K^T,
+// softmax and P V: 1470 clocks an entry, this split V3_CLK.)
 //
 // `ref` is a per-token reference kept instead of the exact running maximum (bf16 P and fp32 sums
 // keep their relative precision whatever the reference, as long as nothing overflows): the
@@ -33,11 +36,10 @@
 // buffer held until its product was complete) and one O per group: an entry took 1560 clocks, the
 // two chains of an entry keep the tensor pipe busy for 1024 (ATTN_V2).
 //
-// Roles (384 threads): warp 0 TMA producer (converged, one elected lane issues; two independent
-// non-blocking load streams, K with Q and V); warp 1 issues the Q K^T chains and owns TMEM; warp 3
-// issues the P V chains (separate issuing warps, because the thread that issues a chain is held
-// until the tensor core has taken it); warp 2 copies the pairs' mask rows from global to shared
-// memory ahead of everyone else; warps 4..7 and 8..11 are the two softmax groups. Every role
+// Roles (384 threads): warp 0 brings the K and Q tiles by TMA, warp 2 the V tiles and, ahead of
+// everyone else, the pairs' mask rows; warp 1 issues the Q K^T chains and owns TMEM; warp 3 issues
+// the P V chains (separate issuing warps, because the thread that issues a chain is held until the
+// tensor core has taken it); warps 4..7 and 8..11 are the two softmax groups. Every role
 // walks the same sequence of (pair, entry), read from the shared copy of the mask rows; they meet
 // only on mbarriers. Every wait is bounded: on a timeout the CTA records a code in a device
 // status word, raises a shared abort flag, lets its copies drain and leaves.
@@ -64,7 +66,6 @@ constexpr int kOperand = 2 * kTile;         // two tiles (K_a, K_b or V_a, V_b),
 // stage is held from its load until the product of its entry is complete, a whole softmax later:
 // V three, K two), or four when the mask rows are long.
 constexpr int kMaxKStages = 2, kMaxVStages = 3;
-constexpr int kSBufs = 3;                   // logit buffers: entry n of the kernel's sequence uses buffer n % 3
 constexpr int kMaskSlots = 2;               // pairs whose mask rows are resident
 constexpr int kMaxKTopTc = 1024;
 constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while pairs of several heads are walked
@@ -77,12 +78,13 @@ struct Item {
     int h[2], qb[2];
 };
 
-// TMEM columns: S / P buffer b at 128 b (P: its first 32), O at 384.
-constexpr int kOCol = kSBufs * 128;
+// TMEM columns: logits of group g at 128 g, its two P buffers at 256 + 64 g and 32 behind, O at 384.
+constexpr int kPCol = 256, kOCol = 384;
 struct Tail {
     unsigned long long q_full[2], q_free[2];  // q_free: the output staged over the pair's Q has left (8 warps)
     unsigned long long k_full[kMaxKStages], k_empty[kMaxKStages], v_full[kMaxVStages], v_empty[kMaxVStages];
-    unsigned long long s_full[kSBufs], p_full[kSBufs], s_free[kSBufs];  // logits ready, P in their place, product added
+    unsigned long long s_full[2], s_free[2];              // per group: logits ready / read
+    unsigned long long p_full[2][2], p_free[2][2];        // per group and P buffer: published / product added
     unsigned long long o_done, o_free;     // a pair's last product is complete; its O has been read (8 warps)
     // Between the two softmax warps of a lane quarter (one per group): the pair's first references
     // are set; group g has published an entry; both have left their sums.
@@ -182,25 +184,160 @@ __device__ __forceinline__ Entry entry_at(const int *rows, int stride, int n) {
 // Roles. All walk the kept entries x_0 .. x_{n-1} of a pair in "rounds": round r handles the
 // logits of x_r and the P V product of x_{r-1}.
 // ----------------------------------------------------------------------------------------------
-__device__ void mask_loader_role(const Params &P, Tail *tl, int lane) {
+// Two warps feed the operand buffers, one the K tiles (with each pair's Q tiles), the other the V tiles
+// and the mask rows: the copies one warp issues stream at 47 bytes per clock, and an entry's 64 KB
+// would take 1400 clocks that way, more than its two chains. Neither blocks on one thing while another could
+// move: every step probes its barrier without waiting. The warps run converged (lane 0's probe
+// result is broadcast) and one elected lane issues.
+struct LoadStream {
+    int round, id;     // pair being walked
+    int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
+    int n;             // kept entries of the pair
+    Entry cur;
+    int b, kvh;
+    Ring ring, ms;
+};
+
+__device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
+    return __shfl_sync(0xffffffffu, (int)mbar_test_wait(bar, parity), 0) != 0;
+}
+
+// Opens the stream's pair (its mask rows must be resident) or closes it; true if it did.
+__device__ __forceinline__ bool open_pair(const Params &P, Tail *tl, LoadStream &S) {
+    if (!probe_w(smem_u32(&tl->m_full[S.ms.idx]), S.ms.phase)) return false;
+    S.b = tl->m_item[S.ms.idx].b;
+    S.kvh = tl->m_item[S.ms.idx].kvh;
+    S.n = tl->m_count[S.ms.idx];
+    S.e = 0;
+    if (S.n > 0) S.cur = entry_at(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
+    return true;
+}
+__device__ __forceinline__ void close_pair(const Params &P, Tail *tl, LoadStream &S) {
+    if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
+    __syncwarp();
+    S.ms.advance(kMaskSlots);
+    S.id = nth_item(P, ++S.round);
+    S.e = -2;
+}
+__device__ __forceinline__ void next_entry(const Params &P, Tail *tl, LoadStream &S) {
+    if (++S.e < S.n) S.cur = entry_at(mask_rows(tl, P, S.ms.idx), P.row_stride, S.e);
+}
+
+// After a step that could not move: false if the CTA is aborting or nothing has moved for too long.
+__device__ __forceinline__ bool idle_ok(Tail *tl, long long t_last, unsigned code) {
+    int stop = 0;
+    if ((threadIdx.x & 31) == 0) {  // lane 0 decides for the warp
+        if (*(volatile int *)&tl->abort_flag) stop = 1;
+        else if (clock64() - t_last > kWaitCycles) {
+            *(volatile int *)&tl->abort_flag = 1;
+            if (atomicCAS(&g_attn_status[0], 0u, code) == 0u) g_attn_status[1] = blockIdx.x;
+            stop = 1;
+        }
+    }
+    if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+    __nanosleep(40);  // leave the issue slots to the softmax warps of this scheduler
+    return true;
+}
+
+__device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, Tail *tl, unsigned q_smem,
+                                unsigned k_smem) {
+    Ring qs;
+    LoadStream S;
+    S.round = 0;
+    S.id = nth_item(P, 0);
+    S.e = -2;
+    bool q_due = false;  // the pair's Q tiles still have to be requested
+    auto step = [&]() -> bool {
+        if (S.e == -2) {
+            if (!open_pair(P, tl, S)) return false;
+            q_due = S.n > 0;
+            return true;
+        }
+        if (S.e >= S.n && !q_due) { close_pair(P, tl, S); return true; }
+        if (S.e == 0 || !q_due) {
+            // a K stage is free once the logits computed from it are complete
+            if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
+            if (elect_one()) {
+                // [half][tile][64 rows][128 B]; a row without a block at an entry gets block 0, its logits are masked out
+                const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * kOperand;
+                const int ba = max(S.cur.a, 0), bb = max(S.cur.b, 0);
+                mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, ba * kBlk, S.kvh, S.b);
+                    tma_load_4d(dst + c * 2 * kHalfTile + kHalfTile, tk, bar, c * 64, bb * kBlk, S.kvh, S.b);
+                }
+            }
+            __syncwarp();
+            S.ring.advance(P.n_k_stages);
+            next_entry(P, tl, S);
+            return true;
+        }
+        // Q goes behind the pair's first K tiles, which do not depend on the Q buffer
+        if (!probe_w(smem_u32(&tl->q_free[qs.idx]), qs.phase ^ 1)) return false;
+        if (elect_one()) {
+            const Item &it = tl->m_item[S.ms.idx];
+            const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
+            mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+#pragma unroll
+            for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const bool second = r == 1 && it.R == 2;
+                    tma_load_4d(q_smem + qs.idx * kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64,
+                                (second ? it.qb[1] : it.qb[0]) * kBlk, second ? it.h[1] : it.h[0], S.b);
+                }
+        }
+        __syncwarp();
+        q_due = false;
+        qs.advance(2);
+        return true;
+    };
+    long long t_last = clock64();
+    while (S.id < P.n_items) {
+        if (step()) t_last = clock64();
+        else if (!idle_ok(tl, t_last, 101)) return;
+    }
+}
+
+// The V tiles, and the pairs' mask rows up to two pairs ahead of everyone else: only the kept entries
+// of a pair (an entry is kept if either row has a block there) go to shared memory, in order, with
+// their number, so that the other roles index them instead of searching.
+__device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail *tl, unsigned v_smem, int lane) {
     const Geom &g = P.g;
-    Ring ms;
-    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
-        const Item it = decode_item(P, id);
-        if (!wait(smem_u32(&tl->m_empty[ms.idx]), ms.phase ^ 1, tl, 401)) return;
-        const int32_t *m0 = P.mask + (((long long)it.b * g.H + it.h[0]) * g.n_qb + it.qb[0]) * g.k_top;
-        const int32_t *m1 = P.mask + (((long long)it.b * g.H + it.h[1]) * g.n_qb + it.qb[1]) * g.k_top;
-        int *dst = mask_rows(tl, P, ms.idx);
-        // an entry is kept if either row has a block there; the kept ones move to the front, so that
-        // the other roles index them instead of searching (their serial code is the kernel's pace)
+    LoadStream S;
+    S.round = 0;
+    S.id = nth_item(P, 0);
+    S.e = -2;
+    int m_round = 0, m_id = nth_item(P, 0);  // the next pair whose mask rows are due
+    bool asked = false;                      // its first 32 entries are on their way to registers
+    Item it;
+    int a0 = -1, b0 = -1;
+    const int32_t *m0 = nullptr, *m1 = nullptr;
+    Ring mw;
+    auto fetch = [&](int e, int &a, int &b) {
+        a = b = -1;
+        if (e < g.k_top) {
+            if (it.R >= 1) a = __ldg(m0 + e);
+            if (it.R == 2) b = __ldg(m1 + e);
+        }
+    };
+    auto mask_step = [&]() -> bool {
+        if (m_id >= P.n_items) return false;
+        if (!asked) {
+            it = decode_item(P, m_id);
+            m0 = P.mask + (((long long)it.b * g.H + it.h[0]) * g.n_qb + it.qb[0]) * g.k_top;
+            m1 = P.mask + (((long long)it.b * g.H + it.h[1]) * g.n_qb + it.qb[1]) * g.k_top;
+            fetch(lane, a0, b0);
+            asked = true;
+            return true;
+        }
+        if (!probe_w(smem_u32(&tl->m_empty[mw.idx]), mw.phase ^ 1)) return false;
+        int *dst = mask_rows(tl, P, mw.idx);
         int cnt = 0;
         for (int base = 0; base < g.k_top; base += 32) {
-            const int e = base + lane;
-            int a = -1, b = -1;
-            if (e < g.k_top) {
-                if (it.R >= 1) a = __ldg(m0 + e);
-                if (it.R == 2) b = __ldg(m1 + e);
-            }
+            int a = a0, b = b0;
+            if (base > 0) fetch(base + lane, a, b);
             const bool kept = a >= 0 || b >= 0;
             const unsigned bal = __ballot_sync(0xffffffffu, kept);
             if (kept) {
@@ -212,136 +349,36 @@ __device__ void mask_loader_role(const Params &P, Tail *tl, int lane) {
         }
         __syncwarp();
         if (lane == 0) {
-            tl->m_count[ms.idx] = cnt;
-            tl->m_item[ms.idx] = it;
-            mbar_arrive(smem_u32(&tl->m_full[ms.idx]));
+            tl->m_count[mw.idx] = cnt;
+            tl->m_item[mw.idx] = it;
+            mbar_arrive(smem_u32(&tl->m_full[mw.idx]));
         }
-        ms.advance(kMaskSlots);
-    }
-}
-
-// One warp feeds two independent streams of TMA loads, the K tiles (with each pair's Q tiles)
-// and the V tiles, each as far ahead as its ring of stages allows. It never blocks on one stream
-// while the other could move: every step probes its barrier without waiting. The warp runs
-// converged (lane 0's probe result is broadcast) and one elected lane issues.
-struct LoadStream {
-    int round, id;     // pair being walked
-    int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
-    int n;             // kept entries of the pair
-    int n_issued;      // loads issued for this pair
-    Entry cur;
-    Item it;
-    Ring ring, ms;
-    bool q_due;        // (K stream) the pair's Q tiles still have to be requested
-};
-
-__device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
-    return __shfl_sync(0xffffffffu, (int)mbar_test_wait(bar, parity), 0) != 0;
-}
-
-__device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, const CUtensorMap *tv,
-                              Tail *tl, unsigned q_smem, unsigned k_smem, unsigned v_smem) {
-    Ring qs;
-    LoadStream K, V;
-    K.round = V.round = 0;
-    K.id = V.id = nth_item(P, 0);
-    K.e = V.e = -2;
-    K.q_due = V.q_due = false;
-    // a row without a block at an entry gets block 0; its logits are masked out entirely
-    auto load_k_pair = [&](unsigned dst, unsigned bar, const Item &it, Entry x) {  // [half][tile][64 rows][128 B]
-        const int ba = x.a >= 0 ? x.a : 0, bb = x.b >= 0 ? x.b : 0;
-        mbar_arrive_expect_tx(bar, (unsigned)kOperand);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, ba * kBlk, it.kvh, it.b);
-            tma_load_4d(dst + c * 2 * kHalfTile + kHalfTile, tk, bar, c * 64, bb * kBlk, it.kvh, it.b);
-        }
+        __syncwarp();
+        mw.advance(kMaskSlots);
+        m_id = nth_item(P, ++m_round);
+        asked = false;
+        return true;
     };
-    auto load_v_pair = [&](unsigned dst, unsigned bar, const Item &it, Entry x) {  // [tile][half][64 rows][128 B]
-        const int ba = x.a >= 0 ? x.a : 0, bb = x.b >= 0 ? x.b : 0;
-        mbar_arrive_expect_tx(bar, (unsigned)kOperand);
-        tma_load_5d(dst, tv, bar, 0, ba * kBlk, it.kvh, 0, it.b);
-        tma_load_5d(dst + kTile, tv, bar, 0, bb * kBlk, it.kvh, 0, it.b);
-    };
-    // One step of a stream; true if it did something. is_k selects the K (+ Q) or the V stream.
-    auto step = [&](LoadStream &S, bool is_k) -> bool {
-        if (S.id >= P.n_items) return false;
-        const int *rows = mask_rows(tl, P, S.ms.idx);
-        if (S.e == -2) {  // open the pair: its mask rows must be resident
-            if (!probe_w(smem_u32(&tl->m_full[S.ms.idx]), S.ms.phase)) return false;
-            S.it = tl->m_item[S.ms.idx];
-            S.n = tl->m_count[S.ms.idx];
-            S.e = 0;
-            if (S.n > 0) S.cur = entry_at(rows, P.row_stride, 0);
-            S.q_due = is_k && S.n > 0;  // (a pair with nothing kept: only the softmax warps act)
-            S.n_issued = 0;
-            return true;
-        }
-        if (S.e >= S.n && !S.q_due) {  // pair exhausted: give its mask rows back, go to the next one
-            if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
-            __syncwarp();
-            S.ms.advance(kMaskSlots);
-            S.id = nth_item(P, ++S.round);
-            S.e = -2;
-            return true;
-        }
-        if (is_k) {
-            if (S.e < S.n && !(S.q_due && S.n_issued > 0)) {
-                // a K stage is free once the logits computed from it are complete
-                if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
-                if (elect_one()) load_k_pair(k_smem + S.ring.idx * kOperand, smem_u32(&tl->k_full[S.ring.idx]), S.it, S.cur);
-                __syncwarp();
-                S.ring.advance(P.n_k_stages);
-                if (++S.e < S.n) S.cur = entry_at(rows, P.row_stride, S.e);
-                ++S.n_issued;
-                return true;
-            }
-            // Q goes behind the pair's first K tiles, which do not depend on the Q buffer
-            if (!probe_w(smem_u32(&tl->q_free[qs.idx]), qs.phase ^ 1)) return false;
-            if (elect_one()) {
-                const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
-                mbar_arrive_expect_tx(bar, (unsigned)kOperand);
-#pragma unroll
-                for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const bool second = r == 1 && S.it.R == 2;
-                        tma_load_4d(q_smem + qs.idx * kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64, (second ? S.it.qb[1] : S.it.qb[0]) * kBlk,
-                                    second ? S.it.h[1] : S.it.h[0], S.it.b);
-                    }
-            }
-            __syncwarp();
-            S.q_due = false;
-            qs.advance(2);
-            return true;
-        }
+    auto step = [&]() -> bool {
+        if (S.e == -2) return open_pair(P, tl, S);
+        if (S.e >= S.n) { close_pair(P, tl, S); return true; }
         // a V stage is free once the product computed from it is complete
         if (!probe_w(smem_u32(&tl->v_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
-        if (elect_one()) load_v_pair(v_smem + S.ring.idx * kOperand, smem_u32(&tl->v_full[S.ring.idx]), S.it, S.cur);
+        if (elect_one()) {  // [tile][half][64 rows][128 B]
+            const unsigned bar = smem_u32(&tl->v_full[S.ring.idx]), dst = v_smem + S.ring.idx * kOperand;
+            mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+            tma_load_5d(dst, tv, bar, 0, max(S.cur.a, 0) * kBlk, S.kvh, 0, S.b);
+            tma_load_5d(dst + kTile, tv, bar, 0, max(S.cur.b, 0) * kBlk, S.kvh, 0, S.b);
+        }
         __syncwarp();
         S.ring.advance(P.n_v_stages);
-        if (++S.e < S.n) S.cur = entry_at(rows, P.row_stride, S.e);
+        next_entry(P, tl, S);
         return true;
     };
     long long t_last = clock64();
-    while (K.id < P.n_items || V.id < P.n_items) {
-        const bool moved_k = step(K, true), moved_v = step(V, false);
-        if (moved_k || moved_v) {
-            t_last = clock64();
-        } else {
-            // nothing to do right now: lane 0 decides for the warp whether to go on
-            int stop = 0;
-            if ((threadIdx.x & 31) == 0) {
-                if (*(volatile int *)&tl->abort_flag) stop = 1;
-                else if (clock64() - t_last > kWaitCycles) {
-                    *(volatile int *)&tl->abort_flag = 1;
-                    if (atomicCAS(&g_attn_status[0], 0u, 101u) == 0u) g_attn_status[1] = blockIdx.x;
-                    stop = 1;
-                }
-            }
-            if (__shfl_sync(0xffffffffu, stop, 0)) return;
-            __nanosleep(40);  // leave the issue slots to the softmax warps of this scheduler
-        }
+    while (S.id < P.n_items) {
+        if (step() || mask_step()) t_last = clock64();
+        else if (!idle_ok(tl, t_last, 102)) return;
     }
 }
 
@@ -350,7 +387,8 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
 
 // S = [Q_0; Q_1] [K_a; K_b]^T for every kept entry.
 __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base) {
-    Ring ks, ms, sb, qs;
+    Ring ks, ms, qs;
+    unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
     const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
     for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
@@ -362,9 +400,10 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
         }
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, tl, 202)) return;
-            if (!wait_w(smem_u32(&tl->s_free[sb.idx]), sb.phase ^ 1u, tl, 203)) return;  // the buffer's last P has been used
+            const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++;  // entry i of a pair belongs to group i % 2
+            if (!wait_w(smem_u32(&tl->s_free[gi]), (use & 1u) ^ 1u, tl, 203)) return;
             tc_fence_after();
-            const unsigned d_tmem = tmem_base + sb.idx * 128;
+            const unsigned d_tmem = tmem_base + gi * 128;
             const unsigned b_lo = k_lo + ks.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
@@ -373,12 +412,11 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
                     for (int k4 = 0; k4 < 4; ++k4)
                         tc_mma_bf16_split(d_tmem, q_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK,
                                           b_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
-                tc_commit(smem_u32(&tl->s_full[sb.idx]));
+                tc_commit(smem_u32(&tl->s_full[gi]));
                 tc_commit(smem_u32(&tl->k_empty[ks.idx]));
             }
             __syncwarp();
             ks.advance(P.n_k_stages);
-            sb.advance(kSBufs);
         }
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
@@ -388,7 +426,8 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
 
 // O (+)= P [V_a; V_b] for every kept entry; a pair's first entry starts O afresh.
 __device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tmem_base) {
-    Ring vs, ms, sb;  // vs: the entry's V stage
+    Ring vs, ms;  // vs: the entry's V stage
+    unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
     unsigned free_par = 1;  // (the first wait passes at once)
     // the MN-major V tiles have their two 64-channel halves kHalfTile apart
     const unsigned v_lo = desc_lo_sw128(v_smem, kHalfTile), d_tmem = tmem_base + kOCol;
@@ -397,13 +436,14 @@ __device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tme
         const int n_entries = tl->m_count[ms.idx];
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->v_full[vs.idx]), vs.phase, tl, 205)) return;
-            if (!wait_w(smem_u32(&tl->p_full[sb.idx]), sb.phase, tl, 204)) return;  // also: O rescaled if it had to be
+            const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use & 1u;
+            if (!wait_w(smem_u32(&tl->p_full[gi][pb]), (use >> 1) & 1u, tl, 204)) return;  // also: O rescaled if it had to be
             if (i == 0) {
                 if (!wait_w(smem_u32(&tl->o_free), free_par, tl, 206)) return;  // the previous pair's O has been read
                 free_par ^= 1;
             }
             tc_fence_after();
-            const unsigned a_tmem = tmem_base + sb.idx * 128, b_lo = v_lo + vs.idx * (kOperand >> 4);
+            const unsigned a_tmem = tmem_base + kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
                 for (int tile = 0; tile < 2; ++tile) {  // row `tile` of the pair: its P rows, its V tile, its lanes
@@ -413,13 +453,12 @@ __device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tme
                         tc_mma_bf16_ta_masked(d_tmem, a_tmem + s4 * 8, b_lo + ((tile * kTile + s4 * 2048) >> 4), kHiK, kIdescPV,
                                               (i | s4) != 0, lo_off, lo_off, hi_off, hi_off);
                 }
-                tc_commit(smem_u32(&tl->s_free[sb.idx]));
+                tc_commit(smem_u32(&tl->p_free[gi][pb]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
                 if (i + 1 == n_entries) tc_commit(smem_u32(&tl->o_done));
             }
             __syncwarp();
             vs.advance(P.n_v_stages);
-            sb.advance(kSBufs);
         }
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
@@ -454,9 +493,10 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 // The waits are warp-wide (same answer in every lane), so the warp stays converged for the
 // warp-collective TMEM loads and stores and leaves together if the CTA aborts.
 //
-// A parity wait needs the phase before it complete in the eyes of the waiting thread. Within a pair a
-// warp that comes to entry n has published n - 2 after it saw n - 3 published (`turn`), so
-// buffer n % 3's previous use is complete; everything of earlier pairs is, after o_done.
+// A parity wait needs the phase before it complete in the eyes of the waiting thread: a group sees
+// every phase of its own logit and P buffers; what it waits for of the other group's (`turn`) it
+// has followed entry by entry within the pair, and everything of earlier pairs is complete after
+// o_done.
 __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
     const Geom &g = P.g;
     const int lane = t & 31, row = t & 127, grp = t >> 7, half = row >> 6, mq = row & 63, wq = row >> 5;
@@ -464,9 +504,11 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
     const unsigned turn_own = smem_u32(&tl->turn[wq][grp]), turn_other = smem_u32(&tl->turn[wq][grp ^ 1]);
     unsigned char *const stage = q_ptr + (grp * 4 + wq) * 4096;  // this warp's 32 tokens x 64 channels in a Q buffer
     unsigned n_other = 0;     // entries of the other group before this pair, over the whole kernel
+    unsigned n_own = 0;       // entries of this group so far
+    const unsigned s_full = smem_u32(&tl->s_full[grp]), s_free = smem_u32(&tl->s_free[grp]), s_addr = lanes + grp * 128 + half * 64;
     unsigned pair_par = 0;    // phase of the barriers that complete once per pair with entries
     int staged = -1;          // Q buffer whose staged output may still be on its way out
-    Ring ms, sb, qs;          // sb: buffer of the pair's first entry
+    Ring ms, qs;
     auto release_stage = [&]() {
         if (staged < 0) return;
         if (lane == 0) {
@@ -486,22 +528,22 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
         const int n_entries = tl->m_count[ms.idx];
         const int *my_row = mask_rows(tl, P, ms.idx) + half * P.row_stride;  // this token's row of the pair
         float ref = -CUDART_INF_F, l = 0.f;
-        Ring eb = sb;  // buffer of entry n, with the phase of its use
-        if (grp) eb.advance(kSBufs);
         int blk = grp < n_entries ? my_row[grp] : -1;
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
-            const unsigned buf = (unsigned)eb.idx;
             // keys of the block this token may attend: a prefix of n_hi
             const int n_hi = blk >= 0 ? max(0, min(key_end - blk * kBlk, kBlk)) : 0;
             const bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
             blk = n + 2 < n_entries ? my_row[n + 2] : -1;
             // the token's 64 logits against its row's key block
-            if (!wait_w(smem_u32(&tl->s_full[buf]), eb.phase, tl, 301)) return;
+            if (!wait_w(s_full, n_own & 1u, tl, 301)) return;
             tc_fence_after();
             unsigned sr[64];
-            tmem_ld_32x32_issue(lanes + buf * 128 + half * 64, sr);
-            tmem_ld_32x32_issue(lanes + buf * 128 + half * 64 + 32, sr + 32);
+            tmem_ld_32x32_issue(s_addr, sr);
+            tmem_ld_32x32_issue(s_addr + 32, sr + 32);
             tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_free);
             if (masked) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
@@ -519,8 +561,10 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             // P under the present reference, their sum, the packed row. A token without a reference, or
             // with a logit that has outgrown it, shows in the sum, and a reference the other group has
             // moved meanwhile in shared memory: then once more. Whether entry n - 1 of this lane
-            // quarter is published is looked up halfway through, so that its latency is hidden.
-            const unsigned turn_par = (n_other + (unsigned)((n - 1) >> 1)) & 1u;
+            // quarter is published, and the P buffer's last product added, is looked up halfway
+            // through, so that the latency of it is hidden.
+            const unsigned other = n_other + (unsigned)((n - 1) >> 1), turn_par = other & 1u;  // entry n - 1 is the other group's `other`-th
+            const unsigned pb = n_own & 1u, p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own >> 1) & 1u) ^ 1u;
             unsigned packed[32];
             float esum;
             for (int attempt = 0;; ++attempt) {
@@ -539,10 +583,10 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                     }
                 };
                 weights(0);
-                bool seen = true;
+                bool seen = mbar_test_wait(p_free, p_par);
                 float now = ref;
                 if (n > 0) {
-                    seen = mbar_test_wait(turn_other, turn_par);
+                    seen = mbar_test_wait(turn_other, turn_par) && seen;
                     now = *(volatile float *)&tl->ref[row];
                 }
                 weights(32);
@@ -553,6 +597,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                 const bool outgrown = (ref == -CUDART_INF_F && n_hi > 0) || !(esum <= kLazySum);
                 // (no attempt beyond the third: a reference moves at most once under each group's hands)
                 if (!__any_sync(0xffffffffu, !seen || moved || outgrown)) break;
+                if (!wait_w(p_free, p_par, tl, 309)) return;
                 if (n > 0) {
                     if (!wait_w(turn_other, turn_par, tl, 308)) return;
                     now = *(volatile float *)&tl->ref[row];
@@ -573,9 +618,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                         tl->ref[row] = ref;
                     }
                     if (n > 0) {  // what has been added up so far is brought to the new reference
-                        Ring pb = eb;  // entry n - 1's buffer
-                        pb.retreat(kSBufs);
-                        if (!wait_w(smem_u32(&tl->s_free[pb.idx]), pb.phase, tl, 302)) return;
+                        if (!wait_w(smem_u32(&tl->p_free[grp ^ 1][other & 1u]), (other >> 1) & 1u, tl, 302)) return;
                         tc_fence_after();
                         rescale_lane(lanes + kOCol, f);
                     }
@@ -583,16 +626,15 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                 }
             }
             l += esum;
-            tmem_st_32x32_issue(lanes + buf * 128, packed);
+            tmem_st_32x32_issue(lanes + kPCol + grp * 64 + pb * 32, packed);
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(turn_own);
-                mbar_arrive(smem_u32(&tl->p_full[buf]));
+                mbar_arrive(smem_u32(&tl->p_full[grp][pb]));
             }
-            eb.advance(kSBufs);
-            eb.advance(kSBufs);
+            ++n_own;
             release_stage();  // the previous pair's output has long been read
         }
         __syncwarp();
@@ -642,7 +684,6 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             staged = qs.idx;
             qs.advance(2);
             pair_par ^= 1;
-            for (int i = n_entries % (2 * kSBufs); i > 0; --i) sb.advance(kSBufs);
             n_other += (unsigned)(grp == 0 ? n_entries >> 1 : (n_entries + 1) >> 1);
         } else if (row_active) {
             uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)b * g.H + h) * g.T + tq0 + mq) * kD + grp * 64);
@@ -672,10 +713,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), 8); }
         for (int i = 0; i < kMaxKStages; ++i) { mbar_init(smem_u32(&tl->k_full[i]), 1); mbar_init(smem_u32(&tl->k_empty[i]), 1); }
         for (int i = 0; i < kMaxVStages; ++i) { mbar_init(smem_u32(&tl->v_full[i]), 1); mbar_init(smem_u32(&tl->v_empty[i]), 1); }
-        for (int i = 0; i < kSBufs; ++i) {
+        for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&tl->s_full[i]), 1);
-            mbar_init(smem_u32(&tl->p_full[i]), 4);
-            mbar_init(smem_u32(&tl->s_free[i]), 1);
+            mbar_init(smem_u32(&tl->s_free[i]), 4);
+            for (int j = 0; j < 2; ++j) { mbar_init(smem_u32(&tl->p_full[i][j]), 4); mbar_init(smem_u32(&tl->p_free[i][j]), 1); }
         }
         mbar_init(smem_u32(&tl->o_done), 1);
         mbar_init(smem_u32(&tl->o_free), 8);
@@ -696,11 +737,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     const unsigned tmem_base = tl->tmem_base;
 
     if (warp == 0) {
-        producer_role(P, &tmap_q, &tmap_k, &tmap_v, tl, q_smem, k_smem, v_smem);
+        k_producer_role(P, &tmap_q, &tmap_k, tl, q_smem, k_smem);
     } else if (warp == 1) {
         qk_role(P, tl, q_smem, k_smem, tmem_base);
     } else if (warp == 2) {
-        mask_loader_role(P, tl, lane);
+        v_producer_role(P, &tmap_v, tl, v_smem, lane);
     } else if (warp == 3) {
         pv_role(P, tl, v_smem, tmem_base);
     } else {

@@ -326,9 +326,6 @@ struct Ring {  // position in a ring of barriers with phase tracking
     __device__ void advance(int n) {
         if (++idx == n) { idx = 0; phase ^= 1; }
     }
-    __device__ void retreat(int n) {
-        if (--idx < 0) { idx = n - 1; phase ^= 1; }
-    }
 };
 
 // ----------------------------------------------------------------------------------------------
