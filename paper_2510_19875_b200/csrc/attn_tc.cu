@@ -525,15 +525,14 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
         const int tq0 = qb * kBlk;  // (token numbers fit 32 bits: TMA coordinates)
         const bool row_active = half < it.R && tq0 + mq < g.T;
         const int key_end = row_active ? (g.causal ? tq0 + mq + 1 : (int)g.T) : 0;  // keys this token may attend: those before
-        const int n_entries = tl->m_count[ms.idx];
+        const int n_entries = tl->m_count[ms.idx], last_entry = max(n_entries - 1, 0);
         const int *my_row = mask_rows(tl, P, ms.idx) + half * P.row_stride;  // this token's row of the pair
         float ref = -CUDART_INF_F, l = 0.f;
-        int blk = grp < n_entries ? my_row[grp] : -1;
+        // the entry's key block of this token's row; the keys of it the token may attend, a prefix of n_hi
+        auto allowed_keys = [&](int blk) { return blk >= 0 ? max(0, min(key_end - blk * kBlk, kBlk)) : 0; };
+        int n_hi = allowed_keys(grp < n_entries ? my_row[grp] : -1);
+        bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
-            // keys of the block this token may attend: a prefix of n_hi
-            const int n_hi = blk >= 0 ? max(0, min(key_end - blk * kBlk, kBlk)) : 0;
-            const bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
-            blk = n + 2 < n_entries ? my_row[n + 2] : -1;
             // the token's 64 logits against its row's key block
             if (!wait_w(s_full, n_own & 1u, tl, 301)) return;
             tc_fence_after();
@@ -542,8 +541,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             tmem_ld_32x32_issue(s_addr + 32, sr + 32);
             tmem_ld_wait();
             tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(s_free);
+            mbar_arrive_if(s_free, lane == 0);
             if (masked) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
@@ -564,6 +562,8 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             // quarter is published, and the P buffer's last product added, is looked up halfway
             // through, so that the latency of it is hidden.
             const unsigned other = n_other + (unsigned)((n - 1) >> 1), turn_par = other & 1u;  // entry n - 1 is the other group's `other`-th
+            const int next_blk = my_row[min(n + 2, last_entry)];  // (of no meaning behind the last)
+            int next_hi = 0;
             const unsigned pb = n_own & 1u, p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own >> 1) & 1u) ^ 1u;
             unsigned packed[32];
             float esum;
@@ -589,6 +589,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                     seen = mbar_test_wait(turn_other, turn_par) && seen;
                     now = *(volatile float *)&tl->ref[row];
                 }
+                next_hi = allowed_keys(next_blk);
                 weights(32);
                 float e0, e1;
                 unpack_f32x2(add_f32x2(add_f32x2(sum2[0], sum2[1]), add_f32x2(sum2[2], sum2[3])), e0, e1);
@@ -629,12 +630,11 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             tmem_st_32x32_issue(lanes + kPCol + grp * 64 + pb * 32, packed);
             tmem_st_wait();
             tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(turn_own);
-                mbar_arrive(smem_u32(&tl->p_full[grp][pb]));
-            }
+            mbar_arrive_if(turn_own, lane == 0);
+            mbar_arrive_if(smem_u32(&tl->p_full[grp][pb]), lane == 0);
             ++n_own;
+            n_hi = next_hi;
+            masked = __any_sync(0xffffffffu, n_hi != kBlk);
             release_stage();  // the previous pair's output has long been read
         }
         __syncwarp();

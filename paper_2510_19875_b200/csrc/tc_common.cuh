@@ -95,8 +95,16 @@ __device__ __forceinline__ bool elect_one() {
 // stays converged for the elect_one() that follows.
 __device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, int *abort_flag, unsigned *err_code,
                                                unsigned *err_info, unsigned code, long long limit = kWaitCycles) {
-    const bool ok = mbar_wait_bounded(bar, parity, abort_flag, err_code, err_info, code, limit);
-    return __all_sync(0xffffffffu, ok);
+    // (one vote on the first look and no divergence on the way: this is what the warps' serial code
+    // does most, and a look per lane with a branch of its own costs twice the clocks)
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, err_code, err_info, code, limit));
+}
+
+// Arrival of the lanes that say so (one of a warp, as a rule), without a branch.
+__device__ __forceinline__ void mbar_arrive_if(unsigned bar, bool mine) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %1, 0;\n@p mbarrier.arrive.shared::cta.b64 _, [%0];\n}" ::"r"(bar), "r"((unsigned)mine)
+                 : "memory");
 }
 
 __device__ __forceinline__ void tma_load_4d(unsigned dst, const CUtensorMap *map, unsigned bar, int c0, int c1, int c2,
