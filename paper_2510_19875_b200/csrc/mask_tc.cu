@@ -7,18 +7,26 @@
 // into a 64-column TMEM slot; four epilogue warps reduce the slot to the two masked tile maxima
 // (Eq. 4 under C). There are two such groups of four, each serving one of every issuing warp's
 // two slots: the fixed cost of a hand-over (wait, fences, arrive) is larger than the reduction
-// itself, and one group alone would be the longest stage of the pipeline. A controller warp keeps
-// each row's nodes in registers, ranks the 2k branch scores (higher score, then lower block
+// itself, and one group alone would be the longest stage of the pipeline. A controller warp per
+// row keeps the row's nodes in registers, ranks the 2k branch scores (higher score, then lower block
 // index), compacts the survivors with ballots and publishes the next level's fetch list. The
 // first level's representatives are the same for every row of a group, so one fetched stage
 // serves all its rows; from the second level on a left branch inherits its parent's score and
 // only right branches are fetched. With several k per call a group runs the hierarchy once per
 // k on the same Q tiles and fetches only blocks whose score it does not have yet.
 //
-// Roles (512 threads, the last warp idle): warps 0 and 14 TMA producers (even and odd stage
-// buffers; warp 0 also brings the Q tiles), warps 1, 3, 12, 13 MMA issuers (warp 1 owns TMEM),
-// warp 2 controller, warps 4..7 and 8..11 the two epilogue groups (TMEM lane quarter = warp % 4). All roles walk the same fixed unit order (level 1: stage-major,
-// row-minor; later levels: row-major), synchronised by mbarriers only. Every wait is bounded: on
+// Nothing of a group's beginning waits for the end of the group before: a dispatcher warp has the next
+// group's number before it is needed, publishes its first list while the last one's later levels
+// run (the level depends on the query block alone), and replaces a row's Q tile as soon as the row's
+// last products are complete, so that the first tiles of the next group arrive behind the last
+// products of this one. (One warp doing all of it, and ranking all four rows, kept the issuing
+// warps waiting for a group or a list for 17 % (T = 16384, k = 16) to 29 % (several k) of the time.)
+//
+// Roles (608 threads): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
+// 3, 13, 17 MMA issuers (warp 1 owns TMEM), warp 18 dispatcher (groups, first lists, Q tiles), warps 0,
+// 12, 16, 15 the controllers of rows 0..3, warps 4..7 and 8..11 the two epilogue groups (TMEM lane
+// quarter = warp % 4). All roles walk the same fixed unit order (level 1: stage-major, row-minor;
+// later levels: row-major), synchronised by mbarriers only. Every wait is bounded: on
 // a timeout the CTA records an error code in the workspace header, raises a shared abort flag,
 // drains its own copies and leaves.
 #include <math_constants.h>
@@ -30,9 +38,9 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 608;
 constexpr int kEpiGroups = 2;  // group g reduces the chains that land in slot g of their issuing warp
-constexpr int kMmaWarps = 4;   // warps 1, 3, 12, 13 take the stages in turn
+constexpr int kMmaWarps = 4;   // they take the stages in turn
 constexpr int kR = 4;          // rows (query heads) per group
 constexpr int kStages = 4;     // K-pair stages
 constexpr int kSlots = 8;      // TMEM accumulator slots of 64 fp32 columns
@@ -41,8 +49,9 @@ constexpr int kHalfTile = kBlk * 128;          // 64 rows x 128 bytes (one 64-ch
 constexpr int kStageBytes = 4 * kHalfTile;     // [2 channel halves][2 tiles]
 constexpr int kQBytes = 2 * kR * kHalfTile;    // [2 channel halves][kR rows]
 constexpr int kMaxJobs = 64;
-constexpr int kProducers = 2;     // warps 0 and 14: producer p fills the stage buffers b with b % 2 == p
-constexpr int kListReaders = kProducers + kMmaWarps + 4 * kEpiGroups;  // producer, MMA and epilogue warps
+constexpr int kProducers = 2;     // producer p fills the stage buffers b with b % 2 == p
+constexpr int kListReaders = kProducers + kMmaWarps + 4 * kEpiGroups;  // producer, MMA and epilogue warps; of a first list and the group record also the controllers
+constexpr int kMaxRowJobs = 32;   // a row's list on a later level: at most one tile per node
 // A parity wait only means something to a thread that saw the phase before it complete, and an
 // arrival only if it cannot come a phase early. So every stage buffer and every TMEM slot
 // belongs to one issuing warp: stage s of the kernel's whole sequence goes, with all its chains,
@@ -53,32 +62,39 @@ static_assert(kSlots == 2 * kMmaWarps, "two private TMEM slots per issuing warp"
 
 struct Tail {
     unsigned long long full[kStages], empty[kStages], tmem_full[kSlots], tmem_empty[kSlots];
-    unsigned long long q_full, jobs_ready[kR + 1], scores_done[kR];
-    // jobs_ack[i]: every reader of list i (the producer, the MMA warps, the epilogue warps) has
-    // taken what it needs from n_jobs[i], jobs_blk[i] and, for i = kR, the group record; the
-    // controller waits for it before it writes them again. Without it a warp with nothing to do
-    // in a short list could still be about to read it when the next one is written, or fall two
-    // phases behind jobs_ready[i].
+    // Per row: its Q tile is there; the last products of a group with it are complete (one commit of
+    // every issuing warp).
+    unsigned long long q_full[kR], q_free[kR];
+    // Lists 0..kR-1: the rows' lists of the later levels; list kR: the first level's, with the group
+    // record. The scores of the two kinds are kept and reported apart, those of the first level twice
+    // (by the parity of the record): the next record's first level may be scored before a row's
+    // controller has looked at this one's last, but the one after that is only published when
+    // the controllers have read the next record, and are done with this one.
+    unsigned long long jobs_ready[kR + 1], first_done[2][kR], scores_done[kR];
+    // jobs_ack[i]: every reader of list i has taken what it needs from n_jobs[i], its blocks and, for
+    // i = kR, the group record; who publishes the list waits for it before it writes them again.
+    // Without it a warp with nothing to do in a short list could still be about to read it when the
+    // next one is written, or fall two phases behind jobs_ready[i].
     unsigned long long jobs_ack[kR + 1];
+    unsigned long long pass_done;  // several k: every row's controller has finished the pass
     unsigned int tmem_base;
     int abort_flag;
     int grp_id, grp_b, grp_kvh, grp_qb, grp_h0, grp_R;
     int grp_levels;  // levels of this group's rows (they share the query block, hence k)
+    int grp_k, grp_pass;
+    unsigned grp_left, grp_right;  // bit i: the left / right candidate of initial node i is on the first list
     int grp_new_q;   // 0: another pass over the same rows (several k), the Q tiles are already there
+    int grp_last;    // the last pass over these rows: the Q tiles are given back
     int n_jobs[kR + 1];
-    int jobs_blk[kR + 1][kMaxJobs];
-    float part[kR][kMaxJobs][2];
-    int node_f[32], node_l[32];
-    float node_s[32];
+    int first_blk[kMaxJobs], jobs_blk[kR][kMaxRowJobs];
+    float first_part[2][kR][kMaxJobs][2], part[kR][kMaxRowJobs][2];
+    int node_f[kR][32], node_l[kR][32];
+    float node_s[kR][32];
 };
 constexpr int kSmemBytes = kQBytes + kStages * kStageBytes + (int)sizeof(Tail) + 1024;
 
-// Bounded wait that reports into the workspace header; false means the CTA is aborting.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, Tail *tl, WorkspaceHeader *ws, unsigned code) {
-    return mbar_wait_bounded(bar, parity, &tl->abort_flag, &ws->error, &ws->error_info, code);
-}
-
-// The same for a whole converged warp (all lanes get the same answer).
+// Bounded wait of a whole converged warp (all lanes get the same answer) that reports into the
+// workspace header; false means the CTA is aborting.
 __device__ __forceinline__ bool mbar_wait_w(unsigned bar, unsigned parity, Tail *tl, WorkspaceHeader *ws, unsigned code) {
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &ws->error, &ws->error_info, code);
 }
@@ -115,8 +131,7 @@ __device__ __forceinline__ unsigned long long cache_pack(unsigned tag, float s) 
 // single diverged lane issues TMA copies several times more slowly. Two producers share the
 // stages by buffer parity: one alone is busy more than half of the time with the four copies and
 // the barrier arm of a stage, and the issuing warps then wait for data.
-__device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, Tail *tl, unsigned q_smem,
-                              unsigned k_smem, int which) {
+__device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail *tl, unsigned k_smem, int which) {
     Ring st;
     unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
     unsigned long long fetched = 0;  // tiles this warp has asked TMA for
@@ -127,17 +142,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
             if (elect_one()) atomicAdd(&P.ws->tiles_fetched, fetched);
             return;
         }
-        const int b = tl->grp_b, kvh = tl->grp_kvh, qb = tl->grp_qb, h0 = tl->grp_h0, R = tl->grp_R;
-        const int levels = tl->grp_levels;
-        // Q tiles of the group's rows (previous group's MMAs are all complete by now)
-        if (which == 0 && tl->grp_new_q && elect_one()) {
-            mbar_arrive_expect_tx(smem_u32(&tl->q_full), (unsigned)(R * 2 * kHalfTile));
-            for (int r = 0; r < R; ++r)
-                for (int c = 0; c < 2; ++c)
-                    tma_load_4d(q_smem + (c * kR + r) * kHalfTile, tq, smem_u32(&tl->q_full), c * 64, qb * kBlk, h0 + r, b);
-        }
-        if (which == 0 && tl->grp_new_q) fetched += (unsigned)R;
-        __syncwarp();
+        const int b = tl->grp_b, kvh = tl->grp_kvh, R = tl->grp_R, levels = tl->grp_levels;
         for (int level = 0; level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
@@ -147,12 +152,13 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
                     jr_par[x] ^= 1;
                 }
                 const int n = tl->n_jobs[li];
+                const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
                 for (int j = 0; j < n; j += 2) {
                     if ((st.idx & (kProducers - 1)) != which) { st.advance(kStages); continue; }  // the other producer's buffer
                     if (!mbar_wait_w(smem_u32(&tl->empty[st.idx]), st.phase ^ 1, tl, P.ws, 103)) return;
                     const int two = (j + 1 < n);
                     fetched += 1u + (unsigned)two;
-                    const int blk0 = tl->jobs_blk[li][j], blk1 = two ? tl->jobs_blk[li][j + 1] : 0;
+                    const int blk0 = list[j], blk1 = two ? list[j + 1] : 0;
                     if (elect_one()) {
                         const unsigned bar = smem_u32(&tl->full[st.idx]);
                         const unsigned dst = k_smem + st.idx * kStageBytes;
@@ -189,7 +195,8 @@ __device__ __forceinline__ int chain_slot(int level, int r, unsigned stage) {
 }
 
 __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base, int which) {
-    unsigned grp_par = 0, q_par = 0, jr_par[kR] = {0, 0, 0, 0};
+    unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
+    unsigned q_par = 0;       // bit r: phase of row r's next Q tile
     unsigned stage_seq = 0;   // stages so far, over the whole kernel (the same in every role)
     unsigned slot_par = 0;    // bit i: phase of the next use of this warp's slot i
     const unsigned q_lo = desc_lo_sw128(q_smem, 16);
@@ -200,10 +207,8 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
         grp_par ^= 1;
         if (tl->grp_id < 0) return;
         const int R = tl->grp_R, levels = tl->grp_levels;
-        if (tl->grp_new_q) {
-            if (!mbar_wait_w(smem_u32(&tl->q_full), q_par, tl, P.ws, 202)) return;
-            q_par ^= 1;
-        }
+        const bool give_back = tl->grp_last != 0;
+        unsigned q_due = tl->grp_new_q ? (1u << R) - 1u : 0u;  // rows whose Q tile this warp has yet to see arrive
         for (int level = 0; level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
@@ -224,6 +229,11 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                     for (int r = r0; r < r1; ++r) {
                         const int sl = chain_slot(level, r, s);
                         const int slot = 2 * which + sl;
+                        if ((q_due >> r) & 1u) {
+                            if (!mbar_wait_w(smem_u32(&tl->q_full[r]), (q_par >> r) & 1u, tl, P.ws, 202)) return;
+                            q_par ^= 1u << r;
+                            q_due &= ~(1u << r);
+                        }
                         if (!mbar_wait_w(smem_u32(&tl->tmem_empty[slot]), ((slot_par >> sl) & 1u) ^ 1u, tl, P.ws, 205)) return;
                         slot_par ^= 1u << sl;
                         tc_fence_after();
@@ -245,6 +255,18 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                     }
                 }
                 stage_seq = s_end;
+                if (level == 0)  // (a warp without a stage in this list)
+                    for (int r = 0; r < R; ++r)
+                        if ((q_due >> r) & 1u) {
+                            if (!mbar_wait_w(smem_u32(&tl->q_full[r]), (q_par >> r) & 1u, tl, P.ws, 206)) return;
+                            q_par ^= 1u << r;
+                            q_due &= ~(1u << r);
+                        }
+                if (give_back && level + 1 == levels) {  // the rows' last products with these Q tiles
+                    if (elect_one())
+                        for (int r = r0; r < r1; ++r) tc_commit(smem_u32(&tl->q_free[r]));
+                    __syncwarp();
+                }
             }
         }
     }
@@ -264,40 +286,50 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
     const int key = (wq & 1) * 32 + lane;    // key index inside the tile
     const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16) + grp * 64;
     for (;;) {
-        if (!mbar_wait(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 301)) return;
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 301)) return;
+        const unsigned set = grp_par;
         grp_par ^= 1;
         if (tl->grp_id < 0) return;
         const int R = tl->grp_R, qb = tl->grp_qb, levels = tl->grp_levels;
         const long long rem_q = g.T - (long long)qb * kBlk;
         const int m_lim = rem_q < kBlk ? (int)rem_q : kBlk;  // query tokens of this block inside T
-        // One chain of this group: stage s, row r, this warp's tile at position c of list li.
-        auto reduce = [&](unsigned s, int r, int li, int c, int n) -> bool {
+        // One chain of this group: stage s, this warp's tile of it, where its maximum goes.
+        auto reduce = [&](unsigned s, int blk_of, float *to) -> bool {  // blk_of < 0: no tile at this place
             const unsigned owner = s & (kMmaWarps - 1);
             const unsigned slot = 2 * owner + grp;
-            if (!mbar_wait(smem_u32(&tl->tmem_full[slot]), (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
+            if (!mbar_wait_w(smem_u32(&tl->tmem_full[slot]), (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
             full_par ^= 1u << owner;
             tc_fence_after();
-            if (c < n) {
-                const int blk = tl->jobs_blk[li][c];
-                float v[64];
+            if (blk_of >= 0) {
+                const int blk = blk_of;
                 const unsigned taddr = t_lane + owner * 128;
-                tmem_ld_32x32(taddr, v);
-                tmem_ld_32x32(taddr + 32, v + 32);
+                float best;
                 // allowed queries for this key: inside T, and not before the key if causal
                 const long long rem_k = g.T - (long long)blk * kBlk;
                 int lo = (g.causal && blk == qb) ? key : 0;
                 if (key >= rem_k) lo = kBlk;  // key beyond T
-                if (lo != 0 || m_lim != kBlk) {  // the diagonal block, or a block across T
+                if (!__any_sync(0xffffffffu, lo != 0 || m_lim != kBlk)) {
+                    float v[64];
+                    tmem_ld_32x32(taddr, v);
+                    tmem_ld_32x32(taddr + 32, v + 32);
+                    best = max_of_64(v);
+                } else {  // the diagonal block, or a block across T: rare, so little code rather than little time
+                    best = -CUDART_INF_F;
+#pragma unroll 1
+                    for (int i0 = 0; i0 < 64; i0 += 8) {
+                        unsigned v[8];
+                        tmem_ld_32x8_issue(taddr + i0, v);
+                        tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 64; ++i) v[i] = (i >= lo && i < m_lim) ? v[i] : -CUDART_INF_F;
+                        for (int i = 0; i < 8; ++i)
+                            if (i0 + i >= lo && i0 + i < m_lim) best = fmaxf(best, __uint_as_float(v[i]));
+                    }
                 }
-                float best = max_of_64(v);
                 best = warp_max(best);
-                if (lane == 0) tl->part[r][c][wq & 1] = best;
+                if (lane == 0) to[wq & 1] = best;
             }
             tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tl->tmem_empty[slot]));
+            mbar_arrive_if(smem_u32(&tl->tmem_empty[slot]), lane == 0);
             return true;
         };
         for (int level = 0; level < levels; ++level) {
@@ -305,32 +337,35 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
             for (int x = 0; x < lists; ++x) {
                 const int li = level == 0 ? kR : x;
                 if (level > 0) {
-                    if (!mbar_wait(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 302)) return;
+                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 302)) return;
                     jr_par[x] ^= 1;
                 }
                 const int n = tl->n_jobs[li];
                 const unsigned s_end = stage_seq + ((unsigned)(n + 1) >> 1);
-                if (level == 0) {
-                    // every stage serves all rows; rows grp, grp + 2 are this group's
-                    for (unsigned s = stage_seq; s < s_end; ++s) {
-                        const int c = 2 * (int)(s - stage_seq) + tile;
-                        for (int r = grp; r < R; r += 2)
-                            if (!reduce(s, r, li, c, n)) return;
-                    }
-                } else {
-                    // one chain per stage; this group's are the stages with (s / kMmaWarps) % 2 == grp
-                    unsigned s = stage_seq;
-                    while (s < s_end) {
-                        if ((int)((s / kMmaWarps) & 1u) != grp) { s = (s | (kMmaWarps - 1)) + 1; continue; }
-                        if (!reduce(s, x, li, 2 * (int)(s - stage_seq) + tile, n)) return;
-                        ++s;
-                    }
+                // First level: every stage serves all rows, rows grp, grp + 2 are this group's, and each
+                // issuing warp needs its slot back from the first before it can issue the second: so
+                // the first rows of kMmaWarps stages, then the second ones (stage by stage the group
+                // waited for that round trip with other warps' chains ready: 115 -> 99 us at
+                // T = 4096, 32 / 8 heads, k = 32). Later one chain per stage, this group's are the
+                // stages with (s / kMmaWarps) % 2 == grp.
+                const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
+                const int r0 = level == 0 ? grp : x, r1 = level == 0 ? R : x + 1;
+                float(*const part)[2] = level == 0 ? tl->first_part[set][0] : tl->part[x];
+                const int row_step = level == 0 ? kMaxJobs : 0;
+                for (unsigned base = level == 0 ? stage_seq : stage_seq & ~(unsigned)(kMmaWarps - 1); base < s_end; base += kMmaWarps) {
+                    if (level > 0 && (int)((base / kMmaWarps) & 1u) != grp) continue;
+                    const unsigned lo = max(base, stage_seq), hi = min(base + kMmaWarps, s_end);
+                    for (int r = r0; r < r1; r += 2)
+                        for (unsigned s = lo; s < hi; ++s) {
+                            const int c = 2 * (int)(s - stage_seq) + tile;
+                            if (!reduce(s, c < n ? list[c] : -1, part[r * row_step + c])) return;
+                        }
                 }
                 stage_seq = s_end;
-                // this list is done for rows r0..r1: tell the controller
+                // this list is done for rows r0..r1: tell their controllers
+                __syncwarp();
                 if (lane == 0) {
-                    const int r0 = level == 0 ? 0 : x, r1 = level == 0 ? R : x + 1;
-                    for (int r = r0; r < r1; ++r) mbar_arrive(smem_u32(&tl->scores_done[r]));
+                    for (int r = level == 0 ? 0 : x; r < r1; ++r) mbar_arrive(smem_u32(level == 0 ? &tl->first_done[set][r] : &tl->scores_done[r]));
                     mbar_arrive(smem_u32(&tl->jobs_ack[li]));  // done reading this list
                 }
             }
@@ -338,22 +373,39 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
     }
 }
 
-// Controller ----------------------------------------------------------------------------------------
-// kMulti: several k per group with the score memory; false compiles the plain single-pass
-// controller (its ranking step is on every group's critical path, so it carries nothing extra).
+// Dispatcher and controllers ------------------------------------------------------------------------
+// kMulti: several k per group with the score memory; false compiles the plain single-pass form.
+
+// The two candidates of initial node `lane` (the same for every row of a group).
+struct FirstNodes {
+    int f, l, m;
+    bool vl, vr;
+    __device__ FirstNodes(const Geom &g, int kq, int q_lim, int lane) {
+        f = (int)(((long long)lane * g.N_k) / kq);
+        l = (int)(((long long)(lane + 1) * g.N_k) / kq) - 1;
+        m = (f + l) / 2;
+        vl = lane < kq && f <= l && f <= q_lim;
+        vr = vl && m + 1 <= l && m + 1 <= q_lim;
+    }
+};
+
 template <bool kMulti>
-__device__ void controller_role(const Params &P, Tail *tl, int lane) {
+__device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl, unsigned q_smem, int lane) {
     const Geom &g = P.g;
     const unsigned lt = (1u << lane) - 1u;
-    unsigned sd_par[kR] = {0, 0, 0, 0};
-    unsigned ack_par[kR + 1] = {0, 0, 0, 0, 0};  // phase of the next acknowledgement of each list
-    // this CTA's score memory for the rows of its current group (several k only)
-    unsigned long long *const cache = kMulti ? P.cache + (size_t)blockIdx.x * kR * g.N_k : nullptr;
+    unsigned ack_par = 1, q_par = (1u << kR) - 1u, pass_par = 0;  // (the first waits pass at once)
+    unsigned long long fetched = 0;  // Q tiles asked of TMA
+    const unsigned long long *const cache = kMulti ? P.cache + (size_t)blockIdx.x * kR * g.N_k : nullptr;
+    int next = -1;  // (lane 0) the next group's number, if it has been fetched
     for (;;) {
-        int id = 0;
-        if (lane == 0) id = (int)atomicAdd(&P.ws->work_counter, 1u);
-        id = __shfl_sync(0xffffffffu, id, 0);
+        // the previous list and record have been read by everybody
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ack[kR]), ack_par, tl, P.ws, 402)) return;
+        if (lane == 0 && next < 0) next = (int)atomicAdd(&P.ws->work_counter, 1u);
+        const int id = __shfl_sync(0xffffffffu, next, 0);
         const bool done = id >= P.n_groups || *(volatile int *)&tl->abort_flag;
+        // the one after it a group ahead, unless that could leave another CTA without work
+        next = -1;
+        if (lane == 0 && id + 2 * (int)gridDim.x < P.n_groups) next = (int)atomicAdd(&P.ws->work_counter, 1u);
         int b = 0, kvh = 0, qb = 0, h0 = 0, R = 0;
         if (!done) {
             const int per = g.n_qb * P.n_chunks;
@@ -365,139 +417,187 @@ __device__ void controller_role(const Params &P, Tail *tl, int lane) {
             R = min(kR, g.hpg - chunk * kR);
         }
         const int q_lim = last_valid_block(g, qb);
-        const unsigned tag = (unsigned)id + 1u;  // marks this group's entries of the score memory (0 = never written)
+        const unsigned tag = (unsigned)id + 1u;
         const int n_pass = (!kMulti || done) ? 1 : P.mk.n;
         for (int pass = 0; pass < n_pass; ++pass) {
-            // the group's k: all its rows are the same query block
             const int kq = done ? g.k_top : (kMulti ? P.mk.k[pass] : row_k(g, qb));
-            const int levels = row_levels(g, kq);
-            // initial nodes: lane i holds node i (the same for every row of the group)
-            int f0 = (int)(((long long)lane * g.N_k) / kq), l0 = (int)(((long long)(lane + 1) * g.N_k) / kq) - 1;
-            const bool v0 = !done && lane < kq && f0 <= l0 && f0 <= q_lim;
-            const int m0 = (f0 + l0) / 2;
-            const bool vl1 = v0, vr1 = v0 && m0 + 1 <= l0 && m0 + 1 <= q_lim;
-            // Which of the two candidates does some row still lack a score for? (Without a score
-            // memory: all of them.) A block on the first level's list is scored for every row.
-            unsigned miss_l = vl1 ? (1u << R) - 1u : 0u, miss_r = vr1 ? (1u << R) - 1u : 0u;  // bit r: row r lacks it
-            float cl[kR], cr[kR];
-            if (kMulti && !done) {
-#pragma unroll
-                for (int r = 0; r < kR; ++r) {
-                    cl[r] = cr[r] = -CUDART_INF_F;
-                    if (r >= R) continue;
-                    if (vl1) {
-                        const unsigned long long e = __ldcg(cache + (size_t)r * g.N_k + f0);
-                        if ((unsigned)(e >> 32) == tag) { cl[r] = __uint_as_float((unsigned)e); miss_l &= ~(1u << r); }
-                    }
-                    if (vr1) {
-                        const unsigned long long e = __ldcg(cache + (size_t)r * g.N_k + m0 + 1);
-                        if ((unsigned)(e >> 32) == tag) { cr[r] = __uint_as_float((unsigned)e); miss_r &= ~(1u << r); }
-                    }
+            const FirstNodes fn(g, kq, q_lim, lane);
+            bool on_l = fn.vl && !done, on_r = fn.vr && !done;  // goes on the list
+            if (kMulti && pass > 0) {  // only what some row still lacks a score for; the rows' passes before must be over
+                if (!mbar_wait_w(smem_u32(&tl->pass_done), pass_par, tl, P.ws, 404)) return;
+                pass_par ^= 1;
+                bool need_l = false, need_r = false;
+                for (int r = 0; r < R; ++r) {
+                    if (on_l) need_l |= (unsigned)(__ldcg(cache + (size_t)r * g.N_k + fn.f) >> 32) != tag;
+                    if (on_r) need_r |= (unsigned)(__ldcg(cache + (size_t)r * g.N_k + fn.m + 1) >> 32) != tag;
                 }
+                on_l = need_l;
+                on_r = need_r;
             }
-            const bool fl1 = miss_l != 0u, fr1 = miss_r != 0u;  // goes on the list
-            const unsigned bl = __ballot_sync(0xffffffffu, fl1), br = __ballot_sync(0xffffffffu, fr1);
-            const int c_l1 = __popc(bl & lt) + __popc(br & lt), c_r1 = c_l1 + (fl1 ? 1 : 0);
-            // the previous list and record have been read by everybody (passes at once the first time)
-            if (!mbar_wait(smem_u32(&tl->jobs_ack[kR]), ack_par[kR] ^ 1, tl, P.ws, 402)) return;
-            ack_par[kR] ^= 1;
-            if (fl1) tl->jobs_blk[kR][c_l1] = f0;
-            if (fr1) tl->jobs_blk[kR][c_r1] = m0 + 1;
-            const int n1 = __popc(bl) + __popc(br);
+            const unsigned bl = __ballot_sync(0xffffffffu, on_l), br = __ballot_sync(0xffffffffu, on_r);
+            const int c_l = __popc(bl & lt) + __popc(br & lt), c_r = c_l + (on_l ? 1 : 0);
+            if (pass > 0 && !mbar_wait_w(smem_u32(&tl->jobs_ack[kR]), ack_par, tl, P.ws, 409)) return;
+            ack_par ^= 1;
+            if (on_l) tl->first_blk[c_l] = fn.f;
+            if (on_r) tl->first_blk[c_r] = fn.m + 1;
             if (lane == 0) {
-                tl->n_jobs[kR] = n1;
+                tl->n_jobs[kR] = __popc(bl) + __popc(br);
                 tl->grp_id = done ? -1 : id; tl->grp_b = b; tl->grp_kvh = kvh; tl->grp_qb = qb; tl->grp_h0 = h0; tl->grp_R = R;
-                tl->grp_levels = levels;
+                tl->grp_levels = row_levels(g, kq);
+                tl->grp_k = kq; tl->grp_pass = pass;
+                tl->grp_left = bl; tl->grp_right = br;
                 tl->grp_new_q = pass == 0;
+                tl->grp_last = pass + 1 == n_pass;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[kR]));
-            if (done) return;
-
-            int nf[kR], nl[kR], my_c[kR], n_nodes[kR], rb[kR];
-            float ns[kR], cs[kR];
-            bool has_r[kR], need[kR];
-            unsigned tiles = 0;  // (row, block) tiles that had no score yet
-            unsigned rt[kR];     // the same, row by row
-#pragma unroll
-            for (int r = 0; r < kR; ++r) {
-                rt[r] = 0;
-                if (r < R) rt[r] = (unsigned)(__popc(__ballot_sync(0xffffffffu, (miss_l >> r) & 1u)) + __popc(__ballot_sync(0xffffffffu, (miss_r >> r) & 1u)));
-                tiles += rt[r];
+            if (done) {
+                if (lane == 0) atomicAdd(&P.ws->tiles_fetched, fetched);
+                return;
             }
-            for (int level = 0; level < levels; ++level) {
+            if (pass > 0) continue;
+            for (int r = 0; r < R; ++r) {  // the rows' Q tiles, each once the last group is done with the one before
+                if (!mbar_wait_w(smem_u32(&tl->q_free[r]), (q_par >> r) & 1u, tl, P.ws, 405)) return;
+                q_par ^= 1u << r;
+                if (elect_one()) {
+                    const unsigned bar = smem_u32(&tl->q_full[r]);
+                    mbar_arrive_expect_tx(bar, (unsigned)(2 * kHalfTile));
 #pragma unroll
-                for (int r = 0; r < kR; ++r) {
-                    if (r >= R) continue;
-                    if (!mbar_wait(smem_u32(&tl->scores_done[r]), sd_par[r], tl, P.ws, 401)) return;
-                    sd_par[r] ^= 1;
-                    // candidates of this lane's node: left (f : m) and right (m + 1 : l)
-                    int f, l, m;
-                    bool vl, vr;
-                    float sl = -CUDART_INF_F, sr = -CUDART_INF_F;
-                    if (level == 0) {
-                        f = f0; l = l0; m = m0; vl = vl1; vr = vr1;
-                        if (vl) sl = fl1 ? fmaxf(tl->part[r][c_l1][0], tl->part[r][c_l1][1]) : cl[r];
-                        if (vr) sr = fr1 ? fmaxf(tl->part[r][c_r1][0], tl->part[r][c_r1][1]) : cr[r];
-                        if (kMulti) {
-                            if (fl1) __stcg(cache + (size_t)r * g.N_k + f0, cache_pack(tag, sl));
-                            if (fr1) __stcg(cache + (size_t)r * g.N_k + m0 + 1, cache_pack(tag, sr));
-                        }
-                    } else {
-                        f = nf[r]; l = nl[r]; m = (f + l) / 2;
-                        vl = lane < n_nodes[r]; vr = has_r[r];
-                        sl = ns[r];
-                        if (vr) sr = need[r] ? fmaxf(tl->part[r][my_c[r]][0], tl->part[r][my_c[r]][1]) : cs[r];
-                        if (kMulti && need[r]) __stcg(cache + (size_t)r * g.N_k + rb[r], cache_pack(tag, sr));
-                    }
-                    const Keep kp = select_topk(vl, sl, vr, sr, kq, lane);
-                    const unsigned kl = __ballot_sync(0xffffffffu, kp.l), kr = __ballot_sync(0xffffffffu, kp.r);
-                    const int pos_l = __popc(kl & lt) + __popc(kr & lt), pos_r = pos_l + (kp.l ? 1 : 0);
-                    __syncwarp();
-                    if (kp.l) { tl->node_f[pos_l] = f; tl->node_l[pos_l] = m; tl->node_s[pos_l] = sl; }
-                    if (kp.r) { tl->node_f[pos_r] = m + 1; tl->node_l[pos_r] = l; tl->node_s[pos_r] = sr; }
-                    __syncwarp();
-                    n_nodes[r] = __popc(kl) + __popc(kr);
-                    const bool live = lane < n_nodes[r];
-                    nf[r] = live ? tl->node_f[lane] : 0;
-                    nl[r] = live ? tl->node_l[lane] : -1;
-                    ns[r] = live ? tl->node_s[lane] : -CUDART_INF_F;
-                    if (level + 1 < levels) {
-                        // next level: only right branches need a tile; left ones keep the node's score
-                        const int mm = (nf[r] + nl[r]) / 2;
-                        has_r[r] = live && nl[r] > nf[r] && mm + 1 <= q_lim;
-                        rb[r] = mm + 1;
-                        need[r] = has_r[r];
-                        if (kMulti && has_r[r]) {  // an earlier pass (another k) may have scored it
-                            const unsigned long long e = __ldcg(cache + (size_t)r * g.N_k + rb[r]);
-                            if ((unsigned)(e >> 32) == tag) { cs[r] = __uint_as_float((unsigned)e); need[r] = false; }
-                        }
-                        const unsigned hb = __ballot_sync(0xffffffffu, need[r]);
-                        my_c[r] = __popc(hb & lt);
-                        if (!mbar_wait(smem_u32(&tl->jobs_ack[r]), ack_par[r] ^ 1, tl, P.ws, 403)) return;
-                        ack_par[r] ^= 1;
-                        if (need[r]) tl->jobs_blk[r][my_c[r]] = rb[r];
-                        if (lane == 0) tl->n_jobs[r] = __popc(hb);
-                        tiles += (unsigned)__popc(hb);
-                        rt[r] += (unsigned)__popc(hb);
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[r]));
-                    } else {
-                        // emit I[q, :]: first block of every surviving node, ascending, -1 padded
-                        const long long o = (long long)pass * P.slab + (((long long)b * g.H + (h0 + r)) * g.n_qb + qb) * g.k_top;
-                        if (lane < g.k_top) {
-                            P.mask[o + lane] = live ? nf[r] : -1;
-                            if (P.score != nullptr) P.score[o + lane] = live ? ns[r] : -CUDART_INF_F;
-                        }
-                        if (!kMulti && g.row_tiles != nullptr && lane == 0)
-                            g.row_tiles[((long long)b * g.H + (h0 + r)) * g.n_qb + qb] = rt[r];
-                    }
+                    for (int c = 0; c < 2; ++c) tma_load_4d(q_smem + (c * kR + r) * kHalfTile, tq, bar, c * 64, qb * kBlk, h0 + r, b);
                 }
+                __syncwarp();
             }
+            fetched += (unsigned)R;
+        }
+        if (kMulti) {  // (the next group may reuse the pass barrier)
+            if (!mbar_wait_w(smem_u32(&tl->pass_done), pass_par, tl, P.ws, 406)) return;
+            pass_par ^= 1;
+        }
+    }
+}
+
+// Row r of every group.
+template <bool kMulti>
+__device__ void controller_role(const Params &P, Tail *tl, int r, int lane) {
+    const Geom &g = P.g;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned grp_par = 0, first_par = 0, sd_par = 0, ack_par = 1;  // first_par: bit by bit for the two sets
+    // this CTA's score memory for the row (several k only)
+    unsigned long long *const cache = kMulti ? P.cache + ((size_t)blockIdx.x * kR + r) * g.N_k : nullptr;
+    unsigned long long tiles_all = 0, rows_all = 0;
+    for (;;) {
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 407)) return;
+        const unsigned set = grp_par;
+        grp_par ^= 1;
+        const int id = tl->grp_id, b = tl->grp_b, qb = tl->grp_qb, h = tl->grp_h0 + r, R = tl->grp_R, levels = tl->grp_levels;
+        const int kq = tl->grp_k, pass = tl->grp_pass;
+        const unsigned on_left = tl->grp_left, on_right = tl->grp_right;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ack[kR]));  // (the list itself is not needed)
+        if (id < 0) {
             if (lane == 0) {
-                atomicAdd(&P.ws->tiles_scored, (unsigned long long)tiles);
-                atomicAdd(&P.ws->rows, (unsigned long long)R);
+                atomicAdd(&P.ws->tiles_scored, tiles_all);
+                atomicAdd(&P.ws->rows, rows_all);
             }
+            return;
+        }
+        if (r >= R) {
+            if (kMulti && lane == 0) mbar_arrive(smem_u32(&tl->pass_done));
+            continue;
+        }
+        const int q_lim = last_valid_block(g, qb);
+        const unsigned tag = (unsigned)id + 1u;  // marks this group's entries of the score memory (0 = never written)
+        const FirstNodes fn(g, kq, q_lim, lane);
+        const bool fl1 = (on_left >> lane) & 1u, fr1 = (on_right >> lane) & 1u;
+        const int c_l1 = __popc(on_left & lt) + __popc(on_right & lt), c_r1 = c_l1 + (fl1 ? 1 : 0);
+        bool miss_l = fn.vl, miss_r = fn.vr;  // this row has no score for the candidate yet
+        float cl = -CUDART_INF_F, cr = -CUDART_INF_F;
+        if (kMulti) {
+            if (fn.vl) {
+                const unsigned long long e = __ldcg(cache + fn.f);
+                if ((unsigned)(e >> 32) == tag) { cl = __uint_as_float((unsigned)e); miss_l = false; }
+            }
+            if (fn.vr) {
+                const unsigned long long e = __ldcg(cache + fn.m + 1);
+                if ((unsigned)(e >> 32) == tag) { cr = __uint_as_float((unsigned)e); miss_r = false; }
+            }
+        }
+        // (row, block) tiles that had no score yet
+        unsigned tiles = (unsigned)(__popc(__ballot_sync(0xffffffffu, miss_l)) + __popc(__ballot_sync(0xffffffffu, miss_r)));
+        int nf = 0, nl = -1, my_c = 0, n_nodes = 0, rb = 0;
+        float ns = -CUDART_INF_F, cs = 0.f;
+        bool has_r = false, need = false;
+        for (int level = 0; level < levels; ++level) {
+            // candidates of this lane's node: left (f : m) and right (m + 1 : l)
+            int f, l, m;
+            bool vl, vr;
+            float sl = -CUDART_INF_F, sr = -CUDART_INF_F;
+            if (level == 0) {
+                if (!mbar_wait_w(smem_u32(&tl->first_done[set][r]), (first_par >> set) & 1u, tl, P.ws, 408)) return;
+                first_par ^= 1u << set;
+                f = fn.f; l = fn.l; m = fn.m; vl = fn.vl; vr = fn.vr;
+                if (vl) sl = fl1 ? fmaxf(tl->first_part[set][r][c_l1][0], tl->first_part[set][r][c_l1][1]) : cl;
+                if (vr) sr = fr1 ? fmaxf(tl->first_part[set][r][c_r1][0], tl->first_part[set][r][c_r1][1]) : cr;
+                if (kMulti) {
+                    if (fl1) __stcg(cache + f, cache_pack(tag, sl));
+                    if (fr1) __stcg(cache + m + 1, cache_pack(tag, sr));
+                }
+            } else {
+                if (!mbar_wait_w(smem_u32(&tl->scores_done[r]), sd_par, tl, P.ws, 401)) return;
+                sd_par ^= 1;
+                f = nf; l = nl; m = (f + l) / 2;
+                vl = lane < n_nodes; vr = has_r;
+                sl = ns;
+                if (vr) sr = need ? fmaxf(tl->part[r][my_c][0], tl->part[r][my_c][1]) : cs;
+                if (kMulti && need) __stcg(cache + rb, cache_pack(tag, sr));
+            }
+            const Keep kp = select_topk(vl, sl, vr, sr, kq, lane);
+            const unsigned kl = __ballot_sync(0xffffffffu, kp.l), kr = __ballot_sync(0xffffffffu, kp.r);
+            const int pos_l = __popc(kl & lt) + __popc(kr & lt), pos_r = pos_l + (kp.l ? 1 : 0);
+            __syncwarp();
+            if (kp.l) { tl->node_f[r][pos_l] = f; tl->node_l[r][pos_l] = m; tl->node_s[r][pos_l] = sl; }
+            if (kp.r) { tl->node_f[r][pos_r] = m + 1; tl->node_l[r][pos_r] = l; tl->node_s[r][pos_r] = sr; }
+            __syncwarp();
+            n_nodes = __popc(kl) + __popc(kr);
+            const bool live = lane < n_nodes;
+            nf = live ? tl->node_f[r][lane] : 0;
+            nl = live ? tl->node_l[r][lane] : -1;
+            ns = live ? tl->node_s[r][lane] : -CUDART_INF_F;
+            if (level + 1 < levels) {
+                // next level: only right branches need a tile; left ones keep the node's score
+                const int mm = (nf + nl) / 2;
+                has_r = live && nl > nf && mm + 1 <= q_lim;
+                rb = mm + 1;
+                need = has_r;
+                if (kMulti && has_r) {  // an earlier pass (another k) may have scored it
+                    const unsigned long long e = __ldcg(cache + rb);
+                    if ((unsigned)(e >> 32) == tag) { cs = __uint_as_float((unsigned)e); need = false; }
+                }
+                const unsigned hb = __ballot_sync(0xffffffffu, need);
+                my_c = __popc(hb & lt);
+                if (!mbar_wait_w(smem_u32(&tl->jobs_ack[r]), ack_par, tl, P.ws, 403)) return;
+                ack_par ^= 1;
+                if (need) tl->jobs_blk[r][my_c] = rb;
+                if (lane == 0) tl->n_jobs[r] = __popc(hb);
+                tiles += (unsigned)__popc(hb);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[r]));
+            } else {
+                // emit I[q, :]: first block of every surviving node, ascending, -1 padded
+                const long long row = ((long long)b * g.H + h) * g.n_qb + qb;
+                const long long o = (long long)pass * P.slab + row * g.k_top;
+                if (lane < g.k_top) {
+                    P.mask[o + lane] = live ? nf : -1;
+                    if (P.score != nullptr) P.score[o + lane] = live ? ns : -CUDART_INF_F;
+                }
+                if (!kMulti && g.row_tiles != nullptr && lane == 0) g.row_tiles[row] = tiles;
+            }
+        }
+        tiles_all += tiles;
+        ++rows_all;
+        if (kMulti) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tl->pass_done));
         }
     }
 }
@@ -514,9 +614,12 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(smem_u32(&tl->full[i]), 1); mbar_init(smem_u32(&tl->empty[i]), 1); }
         for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&tl->tmem_full[i]), 1); mbar_init(smem_u32(&tl->tmem_empty[i]), 4); }
-        mbar_init(smem_u32(&tl->q_full), 1);
-        for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), kListReaders); }
-        for (int i = 0; i < kR; ++i) mbar_init(smem_u32(&tl->scores_done[i]), 4 * kEpiGroups);
+        for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), kListReaders + (i == kR ? kR : 0)); }
+        for (int i = 0; i < kR; ++i) {
+            mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), kMmaWarps);
+            mbar_init(smem_u32(&tl->first_done[0][i]), 4 * kEpiGroups); mbar_init(smem_u32(&tl->first_done[1][i]), 4 * kEpiGroups); mbar_init(smem_u32(&tl->scores_done[i]), 4 * kEpiGroups);
+        }
+        mbar_init(smem_u32(&tl->pass_done), kR);
         tl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
@@ -529,18 +632,20 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     tc_fence_after();
     const unsigned tmem_base = tl->tmem_base;
 
-    if (warp == 0 || warp == 14) {
-        producer_role(P, &tmap_q, &tmap_k, tl, q_smem, k_smem, warp == 0 ? 0 : 1);
-    } else if (warp == 1) {
-        mma_role(P, tl, q_smem, k_smem, tmem_base, 0);
-    } else if (warp == 2) {
-        controller_role<kMulti>(P, tl, lane);
-    } else if (warp == 3) {
-        mma_role(P, tl, q_smem, k_smem, tmem_base, 1);
-    } else if (warp == 12 || warp == 13) {
-        mma_role(P, tl, q_smem, k_smem, tmem_base, warp - 10);
-    } else if (warp >= 4 && warp < 12) {
+    // One call of each role, so that its code is in the instruction cache once, and the roles dealt so
+    // that a scheduler (warp % 4) runs little beside its two epilogue warps: three copies of the
+    // issuing role and two of the controllers', spread over all schedulers, cost a quarter of the
+    // kernel's time in instruction fetches.
+    if (warp >= 4 && warp < 12) {
         epilogue_role(P, tl, tmem_base, warp & 3, (warp - 4) >> 2, lane);
+    } else if (warp == 1 || warp == 3 || warp == 13 || warp == 17) {
+        mma_role(P, tl, q_smem, k_smem, tmem_base, warp == 1 ? 0 : (warp == 3 ? 1 : (warp == 13 ? 2 : 3)));
+    } else if (warp == 2 || warp == 14) {
+        producer_role(P, &tmap_k, tl, k_smem, warp == 2 ? 0 : 1);
+    } else if (warp == 18) {
+        dispatcher_role<kMulti>(P, &tmap_q, tl, q_smem, lane);
+    } else {
+        controller_role<kMulti>(P, tl, warp == 0 ? 0 : (warp == 12 ? 1 : (warp == 16 ? 2 : 3)), lane);
     }
     __syncwarp();
 
