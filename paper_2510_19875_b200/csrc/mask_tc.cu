@@ -293,28 +293,29 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
         const int R = tl->grp_R, qb = tl->grp_qb, levels = tl->grp_levels;
         const long long rem_q = g.T - (long long)qb * kBlk;
         const int m_lim = rem_q < kBlk ? (int)rem_q : kBlk;  // query tokens of this block inside T
+        const int full_blocks = m_lim == kBlk ? (int)(g.T / kBlk) : 0, diag = g.causal ? qb : -1;  // key blocks without a mask: those before, but for the diagonal one
         // One chain of this group: stage s, this warp's tile of it, where its maximum goes.
-        auto reduce = [&](unsigned s, int blk_of, float *to) -> bool {  // blk_of < 0: no tile at this place
+        auto reduce = [&](unsigned s, int blk, float *to) -> bool {  // blk < 0: no tile at this place (its maximum is not looked at)
             const unsigned owner = s & (kMmaWarps - 1);
             const unsigned slot = 2 * owner + grp;
             if (!mbar_wait_w(smem_u32(&tl->tmem_full[slot]), (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
             full_par ^= 1u << owner;
             tc_fence_after();
-            if (blk_of >= 0) {
-                const int blk = blk_of;
-                const unsigned taddr = t_lane + owner * 128;
-                float best;
-                // allowed queries for this key: inside T, and not before the key if causal
-                const long long rem_k = g.T - (long long)blk * kBlk;
-                int lo = (g.causal && blk == qb) ? key : 0;
-                if (key >= rem_k) lo = kBlk;  // key beyond T
-                if (!__any_sync(0xffffffffu, lo != 0 || m_lim != kBlk)) {
-                    float v[64];
-                    tmem_ld_32x32(taddr, v);
-                    tmem_ld_32x32(taddr + 32, v + 32);
-                    best = max_of_64(v);
-                } else {  // the diagonal block, or a block across T: rare, so little code rather than little time
-                    best = -CUDART_INF_F;
+            float best = -CUDART_INF_F;
+            const unsigned taddr = t_lane + owner * 128;
+            if (blk >= 0 && blk < full_blocks && blk != diag) {
+                unsigned v[64];
+                tmem_ld_32x32_issue(taddr, v);
+                tmem_ld_32x32_issue(taddr + 32, v + 32);
+                tmem_ld_wait();
+                // the slot goes back as soon as it is in registers: its issuing warp waits for it
+                tc_fence_before();
+                mbar_arrive_if(smem_u32(&tl->tmem_empty[slot]), lane == 0);
+                best = max_of_64(reinterpret_cast<const float *>(v));
+            } else {
+                if (blk >= 0) {  // the diagonal block, or a block across T: rare, so little code rather than little time
+                    // allowed queries for this key: inside T, and not before the key if causal
+                    const int lo = key >= (int)g.T - blk * kBlk ? kBlk : (blk == diag ? key : 0);
 #pragma unroll 1
                     for (int i0 = 0; i0 < 64; i0 += 8) {
                         unsigned v[8];
@@ -325,11 +326,11 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
                             if (i0 + i >= lo && i0 + i < m_lim) best = fmaxf(best, __uint_as_float(v[i]));
                     }
                 }
-                best = warp_max(best);
-                if (lane == 0) to[wq & 1] = best;
+                tc_fence_before();
+                mbar_arrive_if(smem_u32(&tl->tmem_empty[slot]), lane == 0);
             }
-            tc_fence_before();
-            mbar_arrive_if(smem_u32(&tl->tmem_empty[slot]), lane == 0);
+            best = warp_max(best);
+            if (lane == 0) to[wq & 1] = best;
             return true;
         };
         for (int level = 0; level < levels; ++level) {
