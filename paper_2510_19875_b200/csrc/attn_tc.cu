@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_out, Params P) {  // P by value: n_k_stages is filled in here
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *smem = aligned_smem(smem_raw);
     // what is left behind the aligned base decides the number of V and K stages (the same in every thread)
     const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
     const int n_rings = (P.smem_bytes - fixed_bytes) / kOperand - kFixedOperands;  // buffers for the two rings: 4 or 5

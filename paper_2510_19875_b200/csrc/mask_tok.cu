@@ -85,7 +85,7 @@ __device__ __forceinline__ unsigned pack_node(int f, int len) { return (unsigned
 __global__ void __launch_bounds__(kThreads, 1)
 mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, Params P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *smem = aligned_smem(smem_raw);
     const unsigned q_smem = smem_u32(smem), k_smem = q_smem + kQBytes;
     float *scores = (float *)(smem + kQBytes + kStages * kStageBytes);
     unsigned *nodes = (unsigned *)((unsigned char *)scores + kScoresBytes);

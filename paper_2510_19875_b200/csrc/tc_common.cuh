@@ -11,6 +11,11 @@ constexpr long long kWaitCycles = 1ll << 31;  // ~1 s: far beyond any legitimate
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
+// The first 1024-byte boundary of the dynamic shared memory, as an offset from its start: an address
+// that has gone through an integer is a generic one to the compiler, and every access to it a 64-bit
+// address and a longer wait.
+__device__ __forceinline__ unsigned char *aligned_smem(unsigned char *raw) { return raw + ((0u - smem_u32(raw)) & 1023u); }
+
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
