@@ -76,7 +76,6 @@ struct Tail {
     // Without it a warp with nothing to do in a short list could still be about to read it when the
     // next one is written, or fall two phases behind jobs_ready[i].
     unsigned long long jobs_ack[kR + 1];
-    unsigned long long pass_done;  // several k: every row's controller has finished the pass
     unsigned int tmem_base;
     int abort_flag;
     int grp_id, grp_b, grp_kvh, grp_qb, grp_h0, grp_R;
@@ -390,13 +389,19 @@ struct FirstNodes {
     }
 };
 
+// Is block blk a first-level candidate of a build with k = kq?
+__device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int blk) {
+    const int i = (int)(((long long)(blk + 1) * kq - 1) / g.N_k);  // the node that holds blk: the last that begins at or before it
+    const int f = (int)(((long long)i * g.N_k) / kq), l = (int)(((long long)(i + 1) * g.N_k) / kq) - 1;
+    return blk == f || blk == (f + l) / 2 + 1;
+}
+
 template <bool kMulti>
 __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl, unsigned q_smem, int lane) {
     const Geom &g = P.g;
     const unsigned lt = (1u << lane) - 1u;
-    unsigned ack_par = 1, q_par = (1u << kR) - 1u, pass_par = 0;  // (the first waits pass at once)
+    unsigned ack_par = 1, q_par = (1u << kR) - 1u;  // (the first waits pass at once)
     unsigned long long fetched = 0;  // Q tiles asked of TMA
-    const unsigned long long *const cache = kMulti ? P.cache + (size_t)blockIdx.x * kR * g.N_k : nullptr;
     int next = -1;  // (lane 0) the next group's number, if it has been fetched
     for (;;) {
         // the previous list and record have been read by everybody
@@ -418,22 +423,16 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl
             R = min(kR, g.hpg - chunk * kR);
         }
         const int q_lim = last_valid_block(g, qb);
-        const unsigned tag = (unsigned)id + 1u;
         const int n_pass = (!kMulti || done) ? 1 : P.mk.n;
         for (int pass = 0; pass < n_pass; ++pass) {
             const int kq = done ? g.k_top : (kMulti ? P.mk.k[pass] : row_k(g, qb));
             const FirstNodes fn(g, kq, q_lim, lane);
             bool on_l = fn.vl && !done, on_r = fn.vr && !done;  // goes on the list
-            if (kMulti && pass > 0) {  // only what some row still lacks a score for; the rows' passes before must be over
-                if (!mbar_wait_w(smem_u32(&tl->pass_done), pass_par, tl, P.ws, 404)) return;
-                pass_par ^= 1;
-                bool need_l = false, need_r = false;
-                for (int r = 0; r < R; ++r) {
-                    if (on_l) need_l |= (unsigned)(__ldcg(cache + (size_t)r * g.N_k + fn.f) >> 32) != tag;
-                    if (on_r) need_r |= (unsigned)(__ldcg(cache + (size_t)r * g.N_k + fn.m + 1) >> 32) != tag;
-                }
-                on_l = need_l;
-                on_r = need_r;
+            // Not what an earlier pass has had on its first list: every row has that score. (What rows have
+            // met on later levels is for their controllers to know, which may still be at it.)
+            for (int e = 0; kMulti && e < pass; ++e) {
+                on_l = on_l && !on_first_list(g, P.mk.k[e], fn.f);
+                on_r = on_r && !on_first_list(g, P.mk.k[e], fn.m + 1);
             }
             const unsigned bl = __ballot_sync(0xffffffffu, on_l), br = __ballot_sync(0xffffffffu, on_r);
             const int c_l = __popc(bl & lt) + __popc(br & lt), c_r = c_l + (on_l ? 1 : 0);
@@ -470,10 +469,6 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl
             }
             fetched += (unsigned)R;
         }
-        if (kMulti) {  // (the next group may reuse the pass barrier)
-            if (!mbar_wait_w(smem_u32(&tl->pass_done), pass_par, tl, P.ws, 406)) return;
-            pass_par ^= 1;
-        }
     }
 }
 
@@ -502,10 +497,7 @@ __device__ void controller_role(const Params &P, Tail *tl, int r, int lane) {
             }
             return;
         }
-        if (r >= R) {
-            if (kMulti && lane == 0) mbar_arrive(smem_u32(&tl->pass_done));
-            continue;
-        }
+        if (r >= R) continue;
         const int q_lim = last_valid_block(g, qb);
         const unsigned tag = (unsigned)id + 1u;  // marks this group's entries of the score memory (0 = never written)
         const FirstNodes fn(g, kq, q_lim, lane);
@@ -596,10 +588,6 @@ __device__ void controller_role(const Params &P, Tail *tl, int r, int lane) {
         }
         tiles_all += tiles;
         ++rows_all;
-        if (kMulti) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tl->pass_done));
-        }
     }
 }
 
@@ -620,7 +608,6 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), kMmaWarps);
             mbar_init(smem_u32(&tl->first_done[0][i]), 4 * kEpiGroups); mbar_init(smem_u32(&tl->first_done[1][i]), 4 * kEpiGroups); mbar_init(smem_u32(&tl->scores_done[i]), 4 * kEpiGroups);
         }
-        mbar_init(smem_u32(&tl->pass_done), kR);
         tl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
