@@ -15,7 +15,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstream.so")
-SOURCES = ["api.cu", "mask_generic.cu", "attn_generic.cu", "attn_mma.cu", "mask_tc.cu", "attn_tc.cu", "mask_tok.cu",
+SOURCES = ["api.cu", "mask_generic.cu", "attn_generic.cu", "attn_mma.cu", "attn_tok.cu", "mask_tc.cu", "attn_tc.cu", "mask_tok.cu",
            "static_scratch.cu", "vertical.cu", "mask_diff.cu", "selftest.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -294,6 +294,7 @@ stream_status stream_sparse_attention(const stream_problem *p, const void *q, co
         return STREAM_ERR_UNSUPPORTED;
     }
     if (tc_ok && p->impl != STREAM_IMPL_GENERIC) return launch_attn_tc(g, q, k, v, mask, scale, out, st);
+    if (p->impl == STREAM_IMPL_AUTO && attn_tok_supported(g, p->dtype, q, k, v, out)) return launch_attn_tok(g, q, k, v, mask, scale, out, st);
     if (p->impl == STREAM_IMPL_AUTO && attn_mma_supported(g, p->dtype, q, k, v, out)) return launch_attn_mma(g, q, k, v, mask, scale, out, st);
     return launch_attn_generic(g, p->dtype, q, k, v, mask, scale, out, st);
 }
@@ -343,6 +344,8 @@ stream_status stream_mask_difference(int64_t n_rows, int32_t k_a, const int32_t 
 stream_status stream_check_device_status(void *cuda_stream) {
     unsigned int words[2] = {0, 0};
     stream_status rc = read_attn_status(words, (cudaStream_t)cuda_stream);
+    if (rc != STREAM_OK) return rc;
+    if (words[0] == 0) rc = read_attn_tok_status(words, (cudaStream_t)cuda_stream);
     if (rc != STREAM_OK) return rc;
     if (words[0] != 0) {
         set_error("attention kernel gave up on a bounded wait: code %u, block %u", words[0], words[1]);

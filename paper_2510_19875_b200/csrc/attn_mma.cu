@@ -20,8 +20,7 @@
 //           merged, a window of 128 key blocks at a time, into one ascending list with a bit per
 //           row: each tile is fetched once and multiplied for the warps that have a token keeping
 //           it; tokens that do not keep it are masked like keys after the token.
-//           32 heads, T = 4096, k = 16, block_q = 1: 202900 us on the fp32-FMA kernel (one CTA per
-//           token, 63 of its 64 tile rows padding) -> 1046 us.
+//           (d = 128 with blocks of 64 keys: attn_tok.cu.)
 // Bound: the latency of dependent steps at 8 to 16 warps per SM (issue slots 41 % busy, mma pipe 23
 // to 35 %); hence the register limits below (12 heads, T = 10007, blocks of 32, d = 128, k = 8: 180
 // us at two CTAs of four warps per SM, 152 at three; 3220 on the fp32-FMA kernel. 16 heads,

@@ -82,8 +82,13 @@ stream_status launch_vertical(const Geom &g, const int32_t *mask, const float *s
                               unsigned int *bad_flag, cudaStream_t st);
 stream_status launch_mask_diff(long long n_rows, int k_a, const int32_t *mask_a, const float *score_a, int k_b,
                                const int32_t *mask_b, int32_t *diff, float *diff_score, cudaStream_t st);
-// Drains `st` and copies the tensor-core attention kernel's status words (code, block) to out.
+// Attention under masks of short query blocks (block_q < 16) on the tensor cores.
+bool attn_tok_supported(const Geom &g, int dtype, const void *q, const void *k, const void *v, const void *out);
+stream_status launch_attn_tok(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale,
+                              void *out, cudaStream_t st);
+// Drain `st` and copy a tensor-core attention kernel's status words (code, block) to out.
 stream_status read_attn_status(unsigned int out[2], cudaStream_t st);
+stream_status read_attn_tok_status(unsigned int out[2], cudaStream_t st);
 
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }

@@ -1,4 +1,5 @@
-"""The warp-level kernels (mma.sync and fp32 FMA) against the CPU oracle, at the sizes where their tiles,
+"""The kernels behind the shapes other than 64 x 64 blocks at d = 128 (mma.sync, fp32 FMA, per-token
+attention on tcgen05) against the CPU oracle, at the sizes where their tiles,
 remainders and launch shapes change: masks bit for bit outside near-ties, attention within
 tolerance, also on arbitrary masks (holes, empty rows, a block twice in a row)."""
 import numpy as np
@@ -31,6 +32,11 @@ CASES = [  # spec changes, block_q, block_k (None: the spec's block), causal
     (dict(d=128, T=9000, k_top=6, block=64, n_q_heads=2, n_kv_heads=1), 8, 64, True),  # two windows of key blocks
     (dict(d=128, block=64, k_top=1, T=64), None, None, True),          # a single key block
     (dict(d=128, T=1, k_top=3), None, None, True),                     # a single token
+    (dict(d=128, T=515, k_top=7), 1, 64, True),                        # per-token attention on tcgen05: tokens beyond T
+    (dict(d=128, T=128, k_top=2), 1, 64, False),
+    (dict(d=128, T=9000, k_top=1, n_q_heads=2, n_kv_heads=1), 1, 64, True),  # (arbitrary masks) whole groups of tokens that keep nothing
+    (dict(d=128, T=700, k_top=7, n_q_heads=3, n_kv_heads=1), 5, 64, False),  # rows that straddle 128 tokens
+    (dict(d=128, T=33000, k_top=4, n_q_heads=1, n_kv_heads=1), 1, 64, True),  # two windows of 512 key blocks
     (dict(dtype="f32", T=1003, n_q_heads=8), None, None, True),
     (dict(dtype="f32", T=515, d=128, k_top=40, block=16), None, None, True),
     (dict(dtype="f32", T=300, d=256, block=64, k_top=3), None, None, False),
@@ -72,3 +78,38 @@ def test_masks_and_attention_at_tile_edges(S, kw, bq, bk, causal):
             bh, qb = divmod(int(rid), nqb)
             lo, hi = qb * BQ, min(spec.T, qb * BQ + BQ)
             assert np.abs(out[bh, lo:hi] - ref[i, : hi - lo]).max() <= TOL[spec.dtype], rid
+
+
+@pytest.mark.parametrize("bq", [64, 1])
+@pytest.mark.parametrize("shift,scale", [(0.0, 8.0), (-40.0, 1.0), (40.0, 1.0), (-40.0, 6.0)])
+def test_attention_with_logits_far_from_the_reference(S, bq, shift, scale):
+    """Logits of several hundred in size, all far below zero, or growing along the row: the tcgen05
+    attention kernels keep a reference per token instead of a running maximum, and move it."""
+    spec = wl.WorkloadSpec("far", 9, 1, 3, 1, 900, 128, 64, 6, "bf16")
+    w = wl.generate(spec)
+    q, k, v = w.torch_tensors("cpu")
+    u = torch.ones(128) / 128 ** 0.5
+    ramp = torch.linspace(0.2, 1.0, spec.T)[:, None]  # later keys lie further out
+    qf = q.float() * scale + 25 * u
+    kf = k.float() * ramp + shift * ramp * u
+    w.q = wl.to_bf16_bits(qf.numpy())
+    w.k = wl.to_bf16_bits(kf.numpy())
+    q, k, v = w.torch_tensors("cuda")
+    p = oracle_problem(spec, block_q=bq)
+    n_rows = spec.n_q_heads * so.num_query_blocks(p)
+    mask = np.random.default_rng(2).integers(0, spec.n_blocks, size=(n_rows, spec.k_top)).astype(np.int32)
+    mask[np.random.default_rng(4).random(mask.shape) < 0.2] = -1
+    out = S.sparse_attention(q, k, v, torch.from_numpy(mask.reshape(1, spec.n_q_heads, -1, spec.k_top)).cuda(), block_q=bq, block_k=64)
+    S.stream_check_device_status()
+    out = out.float().cpu().numpy().reshape(-1, spec.T, spec.d)
+    ref = so.sparse_attention_rows(p, w.q, w.k, w.v, mask, None)
+    nqb = so.num_query_blocks(p)
+    # The output's rounding to bf16 is up to 2^-8 of its size. The logits reach 500: 2^-22 of that each for
+    # their fp32 sums, their scaling and the exponential's argument make the weights, and with them an
+    # output of size up to 5, uncertain by 2e-3. Weights in bf16 (block_q = 64) add 2^-8 of a value's size.
+    few = 2e-3 if bq == 1 else 2e-3 + 5 / 256
+    for rid in range(n_rows):
+        bh, qb = divmod(rid, nqb)
+        lo, hi = qb * bq, min(spec.T, qb * bq + bq)
+        want = ref[rid, : hi - lo]
+        assert (np.abs(out[bh, lo:hi] - want) <= few + np.abs(want) / 256).all(), rid
