@@ -11,7 +11,7 @@
 //   P V     lane (ro, co): QW / 4 consecutive queries x channels 4 co + 32 i, P kept key-major
 // Bound: FMA issue and its latency at 8 warps per SM (issue slots 53 % busy; a bare FMA loop measures
 // 66 of the 74.5 TFLOP/s). The kernel this one replaced padded every tile to 64 x 64 and loaded
-// scalars: 8 heads, T = 5003, blocks of 32, d = 64, k = 8: 599 -> 150 us; one head, T = 2048: 82 -> 25 us.
+// scalars: 8 heads, T = 5003, blocks of 32, d = 64, k = 8: 599 -> 150 us; one head, T = 2048: 82 -> 18 us.
 #include "warp_common.cuh"
 
 namespace stream {
@@ -38,7 +38,8 @@ template <int D, int QW>
 struct Shape {
     static constexpr int kTileBytes = kKeys * D * 4, kPPitch = QW + 8, kPBytes = kKeys * kPPitch * 4;
     static constexpr int kSwz = (D / 4 - 1) & 7;  // 16-byte columns are permuted within a row by row & kSwz
-    static constexpr int kPart = QW * (D < 32 ? 32 : D) + 2 * QW;  // floats a warp leaves behind for the final sum (d = 16: idle lanes too)
+    static constexpr int kRowPitch = D + 4;                // (eight lanes, eight different 16-byte columns)
+    static constexpr int kPart = QW * kRowPitch + 2 * QW;  // floats a warp leaves behind for the final sum
 };
 
 // A [32][D] fp32 tile: keys n0 .. n0 + 31 of block r.
@@ -144,15 +145,10 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
                 const int n = kk + 4 * j;
                 x[j] = *(const float4 *)(ks + n * D * 4 + ((c4 ^ (n & Sh::kSwz)) << 4));
             }
-#pragma unroll
-            for (int i = 0; i < RQ; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    s[i][j] = fmaf(a[i].x, x[j].x, s[i][j]);
-                    s[i][j] = fmaf(a[i].y, x[j].y, s[i][j]);
-                    s[i][j] = fmaf(a[i].z, x[j].z, s[i][j]);
-                    s[i][j] = fmaf(a[i].w, x[j].w, s[i][j]);
-                }
+            fma_channel<RQ>(s, a, x, &float4::x);
+            fma_channel<RQ>(s, a, x, &float4::y);
+            fma_channel<RQ>(s, a, x, &float4::z);
+            fma_channel<RQ>(s, a, x, &float4::w);
         }
         group_sync(1 + grp, g_thr);  // everybody is done with the K tile
         if (nxt < n_tiles) fetch<T, D, kAsync, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
@@ -222,8 +218,10 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
     }
     if (kAsync) cp_async_wait<0>();
 
-    // Sum over the groups through shared memory (all tiles are done with): per warp its rows' maxima
-    // and sums, then its accumulators.
+    // Sum over the groups through shared memory (all tiles are done with): every warp leaves its rows'
+    // maxima and sums and its accumulators, row by row; the weights of the groups are taken once per
+    // row; then all threads add up and store four channels of a row at a time. (One warp per row
+    // group doing it alone took a third of a small call: 25.3 -> 18.5 us for 64 rows of 8 blocks.)
     __syncthreads();
     float *part = (float *)smem + (size_t)warp * Sh::kPart;
 #pragma unroll
@@ -233,50 +231,54 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
         l += __shfl_xor_sync(0xffffffffu, l, 2);
         if (kk == 0) { part[kq + 8 * i] = m_run[i]; part[QW + kq + 8 * i] = l; }
     }
-    if (grp > 0) {
+    if (D >= 32 || co * 4 < D) {
 #pragma unroll
         for (int i = 0; i < RO; ++i)
 #pragma unroll
-            for (int j = 0; j < CO * 4; ++j) part[2 * QW + (i * CO * 4 + j) * 32 + lane] = o[i][j];
+            for (int j = 0; j < CO; ++j)
+                *(float4 *)(part + 2 * QW + (ro * RO + i) * Sh::kRowPitch + 4 * co + 32 * j) =
+                    make_float4(o[i][4 * j], o[i][4 * j + 1], o[i][4 * j + 2], o[i][4 * j + 3]);
     }
     __syncthreads();
-    if (grp > 0) return;
-    if (D < 32 && co * 4 >= D) return;
-#pragma unroll
-    for (int i = 0; i < RO; ++i) {
-        const int mr = ro * RO + i, m = mw * QW + mr;
-        const long long tq = (long long)qb * g.bq + m;
-        float top = -CUDART_INF_F;
-        for (int s = 0; s < splits; ++s) top = fmaxf(top, ((float *)smem)[(size_t)(s * m_warps + mw) * Sh::kPart + mr]);
+    for (int m = tid; m < m_warps * QW; m += blockDim.x) {
+        float *first = (float *)smem + (size_t)(m / QW) * Sh::kPart + m % QW;
+        const size_t step = (size_t)m_warps * Sh::kPart;  // to the same row of the next group
+        float top = -CUDART_INF_F, total = 0.f;
+        for (int s = 0; s < splits; ++s) top = fmaxf(top, first[s * step]);
         const float ref = top == -CUDART_INF_F ? 0.f : top;
-        float total = 0.f, x[CO * 4];
-#pragma unroll
-        for (int j = 0; j < CO * 4; ++j) x[j] = 0.f;
         for (int s = 0; s < splits; ++s) {
-            const float *ps = (float *)smem + (size_t)(s * m_warps + mw) * Sh::kPart;
-            const float f = ps[mr] == -CUDART_INF_F ? 0.f : expf(ps[mr] - ref);
-            total += f * ps[QW + mr];
-#pragma unroll
-            for (int j = 0; j < CO * 4; ++j) x[j] = fmaf(f, s == 0 ? o[i][j] : ps[2 * QW + (i * CO * 4 + j) * 32 + lane], x[j]);
+            const float f = first[s * step] == -CUDART_INF_F ? 0.f : expf(first[s * step] - ref);
+            total += f * first[s * step + QW];
+            first[s * step] = f;
         }
         const float inv = total > 0.f ? 1.f / total : 0.f;
+        for (int s = 0; s < splits; ++s) first[s * step] *= inv;
+    }
+    __syncthreads();
+    for (int idx = tid; idx < m_warps * QW * (D / 4); idx += blockDim.x) {
+        const int m = idx / (D / 4), c = idx % (D / 4) * 4;
+        const long long tq = (long long)qb * g.bq + m;
         if (m >= g.bq || tq >= g.T) continue;
-        T *dst = out + ((long long)bh * g.T + tq) * D;
-#pragma unroll
-        for (int j = 0; j < CO; ++j)
-            store4(dst + 4 * co + 32 * j, make_float4(x[4 * j] * inv, x[4 * j + 1] * inv, x[4 * j + 2] * inv, x[4 * j + 3] * inv));
+        const float *first = (float *)smem + (size_t)(m / QW) * Sh::kPart;
+        const size_t step = (size_t)m_warps * Sh::kPart;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s = 0; s < splits; ++s) {
+            const float f = first[s * step + m % QW];
+            const float4 y = *(const float4 *)(first + s * step + 2 * QW + (m % QW) * Sh::kRowPitch + c);
+            x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
+        }
+        store4(out + ((long long)bh * g.T + tq) * D + c, x);
     }
 }
 
-template <typename T, int D, bool kAsync>
-stream_status launch(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
+template <typename T, int D, int QW, bool kAsync>
+stream_status launch_qw(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
                      cudaStream_t st) {
-    constexpr int QW = D <= 64 ? 32 : 16;  // 64 (d = 256: 128) accumulators a lane
     using Sh = Shape<D, QW>;
     const int m_warps = (g.bq + QW - 1) / QW;
     const long long rows = (long long)g.batch * g.H * g.n_qb;
     // Four warps a CTA, so that several CTAs share an SM; eight when every row has an SM to itself
-    // anyway (64 rows of 8 blocks of 32, d = 64: 26.8 us with four, 25.3 with eight).
+    // anyway.
     int splits = (rows <= sm_count_or_default() ? 8 : 4) / m_warps;
     auto bytes = [&](int s) {
         const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * (Sh::kPBytes + QW * 4) + (size_t)g.k_top * 4;
@@ -292,6 +294,14 @@ stream_status launch(const Geom &g, const void *q, const void *k, const void *v,
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "attn_generic launch");
     return STREAM_OK;
+}
+
+template <typename T, int D, bool kAsync>
+stream_status launch(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
+                     cudaStream_t st) {
+    // 32 tokens a warp are 64 accumulators a lane at d = 64; not where half of them would be padding
+    if (D <= 64 && g.bq > 16) return launch_qw<T, D, 32, kAsync>(g, q, k, v, mask, scale, out, st);
+    return launch_qw<T, D, 16, kAsync>(g, q, k, v, mask, scale, out, st);
 }
 
 template <typename T, bool kAsync>

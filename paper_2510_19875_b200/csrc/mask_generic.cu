@@ -145,15 +145,10 @@ struct FmaScore {
                     const int n = kk + 4 * j;
                     b[j] = *(const float4 *)(kb + n * kRowBytes + ((c4 ^ (n & kSwz)) << 4));
                 }
-#pragma unroll
-                for (int i = 0; i < RQ; ++i)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-                        acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-                        acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-                        acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-                    }
+                fma_channel<RQ>(acc, a, b, &float4::x);
+                fma_channel<RQ>(acc, a, b, &float4::y);
+                fma_channel<RQ>(acc, a, b, &float4::z);
+                fma_channel<RQ>(acc, a, b, &float4::w);
             }
             if (cc == kChunks - 1) {
                 const int slot = list[u / per], r = f[slot];

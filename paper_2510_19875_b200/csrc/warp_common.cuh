@@ -37,6 +37,16 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
+// One channel of an RQ x 8 tile: acc += a b^T. (Channel by channel, so that an accumulator's next
+// addition is 8 RQ instructions away; four in a row on one accumulator wait for each other.)
+template <int RQ>
+__device__ __forceinline__ void fma_channel(float (&acc)[RQ][8], const float4 (&a)[RQ], const float4 (&b)[8], float float4::*ch) {
+#pragma unroll
+    for (int i = 0; i < RQ; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].*ch, b[j].*ch, acc[i][j]);
+}
+
 // Barrier of a group of warps (one warp needs no more than reconvergence). Ids 1.. are the caller's.
 __device__ __forceinline__ void group_sync(int id, int threads) {
     if (threads == 32) __syncwarp();
