@@ -15,7 +15,8 @@
 // pipe 22 % in the MMA form; 59 % in the FMA form), which is why a row gets only four warps and an
 // SM several rows: the 7 to 16 tiles of a level leave eight warps unequal work (12 heads,
 // T = 10007, blocks of 32, d = 128, bf16, k = 8: 310 us with eight warps a row, 222 with four; 8
-// heads, T = 5003, blocks of 32, d = 64, fp32: 246 and 216). The kernel this one replaced put 256
+// heads, T = 5003, blocks of 32, d = 64, fp32: 246 and 216, and 181 since a unit's divisions are done
+// once and not with every chunk). The kernel this one replaced put 256
 // threads on one padded 64 x 64 tile at a time, with scalar loads and four barriers per tile: 5294
 // and 812 us for the same two, 4255 -> 410 us for 16 heads, T = 8192, d = 64, k = 40, not causal.
 //
@@ -89,18 +90,29 @@ struct FmaScore {
         const unsigned buf_s = smem_addr(buf);
         const int kq = lane >> 2, kk = lane & 3;
 
-        auto issue = [&](int q) {
-            const int u = warp + (q / kChunks) * warps, cc = q % kChunks;
-            const int r = f[list[u / per]], ks = (u % per) % nk;
-            const int n0 = ks * kKeysPerUnit;
+        // A unit: slot, its key block, which queries and keys of the tile. (Taken apart once per unit: the
+        // divisions are some hundred clocks each.)
+        struct Unit { int slot, r, qs, ks; };
+        auto unit = [&](int u) {
+            const int e = per == 1 ? u : u / per, sub = u - e * per;
+            Unit x;
+            x.slot = list[e];
+            x.r = f[x.slot];
+            x.qs = nk == 1 ? sub : sub / nk;
+            x.ks = sub - x.qs * nk;
+            return x;
+        };
+        auto issue = [&](const Unit &x, int q, int cc) {
+            const int n0 = x.ks * kKeysPerUnit;
             constexpr int per_key = kCh / 4;
+            const int last = (int)min((long long)g.bk, g.T - (long long)x.r * g.bk) - n0 - 1;  // (the tile's last key inside T stands in for those beyond)
+            const T *base = kp + ((long long)x.r * g.bk + n0) * g.ks_t + cc * kCh;
 #pragma unroll
             for (int i = 0; i < kKeysPerUnit * per_key / 32; ++i) {
                 const int idx = i * 32 + lane, n = idx / per_key, c4 = idx % per_key;
                 const int dst = (q & 1) * kBufBytes + n * kRowBytes + ((c4 ^ (n & kSwz)) << 4);
                 if (n0 + n < g.bk) {  // (keys beyond the block are never looked at)
-                    const long long tk = min((long long)r * g.bk + n0 + n, g.T - 1);
-                    const T *src = kp + tk * g.ks_t + cc * kCh + c4 * 4;
+                    const T *src = base + (long long)min(n, last) * g.ks_t + c4 * 4;
                     if (kAsync) {
                         cp_async16(buf_s + dst, src, 16);
                     } else {
@@ -111,19 +123,21 @@ struct FmaScore {
             if (kAsync) cp_async_commit();
         };
 
-        if (n_chunks > 0) issue(0);
+        Unit cur = {}, ahead = {};  // the unit being scored, the one being fetched
+        if (n_chunks > 0) { ahead = unit(warp); issue(ahead, 0, 0); }
         float acc[RQ][8];
         for (int q = 0; q < n_chunks; ++q) {
+            const int cc = q % kChunks;
+            if (cc == 0) cur = ahead;
             if (q + 1 < n_chunks) {
+                if (cc == kChunks - 1) ahead = unit(warp + (q + 1) / kChunks * warps);
                 __syncwarp();  // every lane is done with the buffer's previous chunk
-                issue(q + 1);
+                issue(ahead, q + 1, (q + 1) % kChunks);
                 if (kAsync) cp_async_wait<1>();
             } else if (kAsync) {
                 cp_async_wait<0>();
             }
             __syncwarp();
-            const int u = warp + (q / kChunks) * warps, cc = q % kChunks;
-            const int sub = u % per, qs = sub / nk, ks = sub % nk;
             if (cc == 0) {
 #pragma unroll
                 for (int i = 0; i < RQ; ++i)
@@ -131,8 +145,8 @@ struct FmaScore {
                     for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
             }
             const unsigned char *kb = buf + (q & 1) * kBufBytes;
-            const float *qrow = Qs + (size_t)qs * kSQ * D;
-#pragma unroll 2
+            const float *qrow = Qs + (size_t)cur.qs * kSQ * D;
+#pragma unroll 1
             for (int c4 = 0; c4 < kCh / 4; ++c4) {
                 float4 a[RQ], b[8];
 #pragma unroll
@@ -151,17 +165,23 @@ struct FmaScore {
                 fma_channel<RQ>(acc, a, b, &float4::w);
             }
             if (cc == kChunks - 1) {
-                const int slot = list[u / per], r = f[slot];
                 float best = -CUDART_INF_F;
-                const Allowed ok(g, qb, r);
-                const bool full = ok.all((qs + 1) * kSQ, (ks + 1) * kKeysPerUnit);
+                const Allowed ok(g, qb, cur.r);
+                if (ok.all((cur.qs + 1) * kSQ, (cur.ks + 1) * kKeysPerUnit)) {
 #pragma unroll
-                for (int i = 0; i < RQ; ++i)
+                    for (int i = 0; i < RQ; ++i)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (full || ok(qs * kSQ + kq + 8 * i, ks * kKeysPerUnit + kk + 4 * j)) best = fmaxf(best, acc[i][j]);
+                        for (int j = 0; j < 8; ++j) best = fmaxf(best, acc[i][j]);
+                } else {
+                    const int m0 = cur.qs * kSQ + kq, n0 = cur.ks * kKeysPerUnit + kk;
+#pragma unroll
+                    for (int i = 0; i < RQ; ++i)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            if (ok(m0 + 8 * i, n0 + 4 * j)) best = fmaxf(best, acc[i][j]);
+                }
                 best = warp_max(best);
-                if (lane == 0 && best > -CUDART_INF_F) atomicMax(&key[slot], key_of(best));
+                if (lane == 0 && best > -CUDART_INF_F) atomicMax(&key[cur.slot], key_of(best));
             }
         }
     }
@@ -456,7 +476,8 @@ stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void 
                      cudaStream_t st) {
     const long long rows = (long long)g.batch * g.H * g.n_qb;
     // Sixteen warps when every row has an SM to itself anyway: a level's tiles then spread over more
-    // warps (64 rows, fp32, d = 64, blocks of 32, k = 8: 34.9 us with eight, 32.9 with sixteen).
+    // warps (64 rows, fp32, d = 64, blocks of 32, k = 8: 34.9 us with eight, 32.9 with sixteen, before the
+    // divisions went; 28.9 now).
     if (rows <= sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
     return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
 }
