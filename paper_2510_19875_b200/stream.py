@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 
 import torch
@@ -34,6 +35,10 @@ class StreamProblem(ctypes.Structure):
         ("q_stride_b", ctypes.c_int64), ("q_stride_h", ctypes.c_int64), ("q_stride_t", ctypes.c_int64),
         ("kv_stride_b", ctypes.c_int64), ("kv_stride_h", ctypes.c_int64), ("kv_stride_t", ctypes.c_int64),
     ]
+
+
+_PROBLEM = struct.Struct("@iiiqiiiiiiiqqqqqq")  # StreamProblem's fields with the C compiler's padding
+assert _PROBLEM.size == ctypes.sizeof(StreamProblem)
 
 
 class StreamStats(ctypes.Structure):
@@ -121,21 +126,22 @@ def _load():
 
 
 def _addr(x):
-    if x is None:
-        return None
     if isinstance(x, torch.Tensor):
         return x.data_ptr()
-    return int(x)
+    return None if x is None else int(x)
 
 
 def _stream_handle(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current device's current stream, by its handle: a Stream object for it takes 3 us to make
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
 
 
 def _raise(status: int):
-    if status != STREAM_OK:
+    if status:
         raise StreamError(status, _load().stream_last_error().decode())
 
 
@@ -263,16 +269,18 @@ def stream_run_host_var(p: StreamProblem, q_host, k_host, v_host, k_row_host, ma
 def make_problem(q: torch.Tensor, k: torch.Tensor, *, block_q: int, block_k: int, k_top: int, causal: bool = True,
                  impl: str = "auto") -> StreamProblem:
     """Problem struct for q ``[B, H, T, d]`` and k ``[B, G, T, d]`` (any strides with unit innermost)."""
-    if q.dim() != 4 or k.dim() != 4 or q.shape[0] != k.shape[0] or q.shape[2:] != k.shape[2:]:
+    qs, ks, dtype = q.shape, k.shape, q.dtype
+    if len(qs) != 4 or len(ks) != 4 or qs[0] != ks[0] or qs[2] != ks[2] or qs[3] != ks[3]:
         raise ValueError("q must be [B, H, T, d] and k [B, G, T, d] with matching B, T, d")
-    if q.dtype != k.dtype or q.dtype not in (torch.float32, torch.bfloat16):
+    if k.dtype is not dtype or (dtype is not torch.float32 and dtype is not torch.bfloat16):
         raise ValueError("q and k must both be float32 or bfloat16")
-    if q.stride(3) != 1 or k.stride(3) != 1:
+    (q_b, q_h, q_t, q_d), (k_b, k_h, k_t, k_d) = q.stride(), k.stride()
+    if q_d != 1 or k_d != 1:
         raise ValueError("innermost stride must be 1")
-    B, H, T, d = q.shape
-    return StreamProblem(B, H, k.shape[1], T, d, block_q, block_k, k_top, int(causal),
-                         STREAM_F32 if q.dtype == torch.float32 else STREAM_BF16, IMPL[impl],
-                         q.stride(0), q.stride(1), q.stride(2), k.stride(0), k.stride(1), k.stride(2))
+    # (packed at once: field by field the struct takes three times as long)
+    return StreamProblem.from_buffer_copy(_PROBLEM.pack(
+        qs[0], qs[1], ks[1], qs[2], qs[3], block_q, block_k, k_top, int(causal),
+        STREAM_F32 if dtype is torch.float32 else STREAM_BF16, IMPL[impl], q_b, q_h, q_t, k_b, k_h, k_t))
 
 
 def n_query_blocks(p: StreamProblem) -> int:
@@ -297,11 +305,25 @@ class MaskResult:
         return self.workspace[self.header_bytes:self.header_bytes + 4 * rows].view(torch.int32).view(self.mask.shape[:3])
 
 
-def new_workspace(p: StreamProblem, device, row_tiles: bool = False) -> torch.Tensor:
-    """Workspace of the size the library asks for; with ``row_tiles`` also room for one counter per row."""
-    n = stream_workspace_bytes(p)
+def _empty(shape, dtype, device) -> torch.Tensor:
+    """Contiguous new tensor (with its strides given, it costs a third less of the host's time)."""
+    strides, n = [1] * len(shape), 1
+    for i in range(len(shape) - 1, -1, -1):
+        strides[i] = n
+        n *= max(1, shape[i])
+    return torch.empty_strided(shape, strides, dtype=dtype, device=device)
+
+
+def _header_bytes(p: StreamProblem) -> int:
+    n = (_lib or _load()).stream_workspace_bytes(ctypes.byref(p))
     if n == 0:
         raise StreamError(STREAM_ERR_INVALID_ARG, stream_last_error())
+    return n
+
+
+def new_workspace(p: StreamProblem, device, row_tiles: bool = False) -> torch.Tensor:
+    """Workspace of the size the library asks for; with ``row_tiles`` also room for one counter per row."""
+    n = _header_bytes(p)
     if row_tiles:
         n += 4 * p.batch * p.n_q_heads * n_query_blocks(p)
     return torch.empty(n, dtype=torch.uint8, device=device)
@@ -317,17 +339,19 @@ def build_mask(q: torch.Tensor, k: torch.Tensor, *, block_q: int, block_k: int, 
     if not q.is_cuda or not k.is_cuda:
         raise ValueError("q and k must be CUDA tensors (there is no CPU path)")
     p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=k_top, causal=causal, impl=impl)
-    shape = (p.batch, p.n_q_heads, n_query_blocks(p), k_top)
-    mask = mask_out if mask_out is not None else torch.empty(shape, dtype=torch.int32, device=q.device)
-    scores = torch.empty(shape, dtype=torch.float32, device=q.device) if want_scores else None
-    ws = workspace if workspace is not None else new_workspace(p, q.device, row_tiles)
+    header = _header_bytes(p)
+    device, shape = q.device, (p.batch, p.n_q_heads, n_query_blocks(p), k_top)
+    mask = mask_out if mask_out is not None else _empty(shape, torch.int32, device)
+    scores = _empty(shape, torch.float32, device) if want_scores else None
+    if workspace is None:
+        workspace = _empty((header + (4 * shape[0] * shape[1] * shape[2] if row_tiles else 0),), torch.uint8, device)
     if k_row is None:
-        stream_build_mask(p, q, k, mask, scores, ws, ws.numel(), stream)
+        stream_build_mask(p, q, k, mask, scores, workspace, workspace.numel(), stream)
     else:
         if not k_row.is_cuda or k_row.dtype != torch.int32 or not k_row.is_contiguous() or tuple(k_row.shape) != (shape[2],):
             raise ValueError(f"k_row must be a contiguous int32 CUDA tensor of shape ({shape[2]},)")
-        stream_build_mask_var(p, q, k, k_row, mask, scores, ws, ws.numel(), stream)
-    return MaskResult(mask, scores, ws, stream_workspace_bytes(p))
+        stream_build_mask_var(p, q, k, k_row, mask, scores, workspace, workspace.numel(), stream)
+    return MaskResult(mask, scores, workspace, header)
 
 
 def build_masks(q: torch.Tensor, k: torch.Tensor, k_list, *, block_q: int, block_k: int, causal: bool = True,
@@ -337,16 +361,17 @@ def build_masks(q: torch.Tensor, k: torch.Tensor, k_list, *, block_q: int, block
     once per k and does not reuse tile scores between them)."""
     if not q.is_cuda or not k.is_cuda:
         raise ValueError("q and k must be CUDA tensors (there is no CPU path)")
-    ks = torch.tensor(list(k_list), dtype=torch.int32)
-    p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=int(ks.max()), causal=causal, impl=impl)
+    ks = [int(x) for x in k_list]
+    p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=max(ks), causal=causal, impl=impl)
     shape = (len(ks), p.batch, p.n_q_heads, n_query_blocks(p), p.k_top)
-    mask = torch.empty(shape, dtype=torch.int32, device=q.device)
-    scores = torch.empty(shape, dtype=torch.float32, device=q.device) if want_scores else None
+    mask = _empty(shape, torch.int32, q.device)
+    scores = _empty(shape, torch.float32, q.device) if want_scores else None
     n_ws = stream_workspace_bytes_multi(p, len(ks)) if share else stream_workspace_bytes(p)
     if n_ws == 0:
         raise StreamError(STREAM_ERR_INVALID_ARG, stream_last_error())
-    ws = torch.empty(n_ws, dtype=torch.uint8, device=q.device)
-    stream_build_mask_multi(p, q, k, len(ks), ks.data_ptr(), mask, scores, ws, ws.numel(), stream)
+    ws = _empty((n_ws,), torch.uint8, q.device)
+    k_host = (ctypes.c_int32 * len(ks))(*ks)
+    stream_build_mask_multi(p, q, k, len(ks), ctypes.addressof(k_host), mask, scores, ws, n_ws, stream)
     return MaskResult(mask, scores, ws)
 
 
@@ -368,11 +393,13 @@ def sparse_attention(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, mask: to
         raise ValueError("v must have k's shape, strides and dtype")
     if mask.dtype != torch.int32 or not mask.is_contiguous():
         raise ValueError("mask must be a contiguous int32 tensor")
-    p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=mask.shape[-1], causal=causal, impl=impl)
-    if tuple(mask.shape) != (p.batch, p.n_q_heads, n_query_blocks(p), mask.shape[-1]):
+    m_shape = tuple(mask.shape)
+    p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=m_shape[-1], causal=causal, impl=impl)
+    B, H, T, d = q.shape
+    if m_shape != (B, H, -(-T // block_q), m_shape[-1]):
         raise ValueError("mask must be [B, H, ceil(T / block_q), k_top]")
     if out is None:
-        out = torch.empty((p.batch, p.n_q_heads, p.T, p.d), dtype=q.dtype, device=q.device)
+        out = _empty((B, H, T, d), q.dtype, q.device)
     stream_sparse_attention(p, q, k, v, mask, scale, out, stream)
     return out
 
@@ -400,8 +427,8 @@ def vertical_scores(p: StreamProblem, mask: torch.Tensor, scores: torch.Tensor |
     if scores is not None and (scores.shape != mask.shape or scores.dtype != torch.float32 or not scores.is_contiguous()):
         raise ValueError("scores must be a contiguous float32 tensor of the mask's shape")
     n_kb = -(-p.T // p.block_k)
-    vert = torch.empty((p.batch, p.n_q_heads, n_kb), dtype=torch.float32, device=mask.device)
-    kurt = torch.empty((p.batch, p.n_q_heads), dtype=torch.float32, device=mask.device)
+    vert = _empty((p.batch, p.n_q_heads, n_kb), torch.float32, mask.device)
+    kurt = _empty((p.batch, p.n_q_heads), torch.float32, mask.device)
     ws = new_workspace(p, mask.device)
     stream_vertical_scores(p, mask, scores, vert, kurt, ws, ws.numel(), stream)
     stream_read_stats(ws, stream)
