@@ -102,7 +102,7 @@ __device__ __forceinline__ bool mbar_wait_w(unsigned bar, unsigned parity, Tail 
 constexpr unsigned kDescHi = desc_hi_sw128(1024);
 
 // D fp32, A and B bf16, both K-major, M = 128, N = 64.
-constexpr unsigned kIdesc = idesc_bf16(128, 64, false);
+constexpr unsigned kIdesc = idesc_bf16(128, 64, false), kIdescTwo = idesc_bf16(128, 128, false);
 
 struct Params {
     Geom g;
@@ -225,30 +225,37 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                 // this warp's stages of the list: s = which (mod kMmaWarps)
                 for (unsigned s = stage_seq + (((unsigned)which - stage_seq) & (kMmaWarps - 1)); s < s_end; s += kMmaWarps) {
                     if (!mbar_wait_w(smem_u32(&tl->full[sidx]), (s / kStages) & 1u, tl, P.ws, 204)) return;
-                    for (int r = r0; r < r1; ++r) {
+                    for (int r = r0; r < r1; r += 2) {
+                        // first level: rows r and r + 1 in one chain, each in its slot
+                        const bool two = level == 0 && r + 1 < r1;
                         const int sl = chain_slot(level, r, s);
                         const int slot = 2 * which + sl;
-                        if ((q_due >> r) & 1u) {
-                            if (!mbar_wait_w(smem_u32(&tl->q_full[r]), (q_par >> r) & 1u, tl, P.ws, 202)) return;
-                            q_par ^= 1u << r;
-                            q_due &= ~(1u << r);
+                        const unsigned rows = two ? 3u << r : 1u << r;
+                        for (int i = r; (q_due & rows) != 0; ++i) {
+                            if (!((q_due >> i) & 1u)) continue;
+                            if (!mbar_wait_w(smem_u32(&tl->q_full[i]), (q_par >> i) & 1u, tl, P.ws, 202)) return;
+                            q_par ^= 1u << i;
+                            q_due &= ~(1u << i);
                         }
                         if (!mbar_wait_w(smem_u32(&tl->tmem_empty[slot]), ((slot_par >> sl) & 1u) ^ 1u, tl, P.ws, 205)) return;
-                        slot_par ^= 1u << sl;
+                        if (two && !mbar_wait_w(smem_u32(&tl->tmem_empty[slot + 1]), ((slot_par >> 1) & 1u) ^ 1u, tl, P.ws, 205)) return;
+                        slot_par ^= two ? 3u : 1u << sl;
                         tc_fence_after();
                         const unsigned d_tmem = tmem_base + slot * 64;
                         const unsigned b_lo = q_lo + r * (kHalfTile >> 4);
+                        const unsigned idesc = two ? kIdescTwo : kIdesc;
                         if (elect_one()) {
 #pragma unroll
                             for (int c = 0; c < 2; ++c)
 #pragma unroll
                                 for (int k4 = 0; k4 < 4; ++k4)
                                     tc_mma_bf16_split(d_tmem, a_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kDescHi,
-                                                      b_lo + ((c * kR * kHalfTile + k4 * 32) >> 4), kDescHi, kIdesc, (c | k4) != 0);
+                                                      b_lo + ((c * kR * kHalfTile + k4 * 32) >> 4), kDescHi, idesc, (c | k4) != 0);
                             tc_commit(smem_u32(&tl->tmem_full[slot]));
+                            if (two) tc_commit(smem_u32(&tl->tmem_full[slot + 1]));
                             // the stage is free once its last chain has read it (a commit covers all
                             // earlier instructions of this thread)
-                            if (r + 1 == r1) tc_commit(smem_u32(&tl->empty[sidx]));
+                            if (r + 2 >= r1) tc_commit(smem_u32(&tl->empty[sidx]));
                         }
                         __syncwarp();
                     }
