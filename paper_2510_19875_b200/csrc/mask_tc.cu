@@ -61,7 +61,8 @@ static_assert(kStages == kMmaWarps, "a stage buffer must always meet the same is
 static_assert(kSlots == 2 * kMmaWarps, "two private TMEM slots per issuing warp");
 
 struct Tail {
-    unsigned long long full[kStages], empty[kStages], tmem_full[kSlots], tmem_empty[kSlots];
+    unsigned long long full[2][kStages];  // by channel half
+    unsigned long long empty[kStages], tmem_full[kSlots], tmem_empty[kSlots];
     // Per row: its Q tile is there; the last products of a group with it are complete (one commit of
     // every issuing warp).
     unsigned long long q_full[kR], q_free[kR];
@@ -87,6 +88,7 @@ struct Tail {
     int n_jobs[kR + 1];
     int first_blk[kMaxJobs], jobs_blk[kR][kMaxRowJobs];
     float first_part[2][kR][kMaxJobs][2], part[kR][kMaxRowJobs][2];
+    float no_part;   // (written before a list's first tile, not read)
     int node_f[kR][32], node_l[kR][32];
     float node_s[kR][32];
 };
@@ -154,18 +156,23 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail *tl, 
                 const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
                 for (int j = 0; j < n; j += 2) {
                     if ((st.idx & (kProducers - 1)) != which) { st.advance(kStages); continue; }  // the other producer's buffer
-                    if (!mbar_wait_w(smem_u32(&tl->empty[st.idx]), st.phase ^ 1, tl, P.ws, 103)) return;
                     const int two = (j + 1 < n);
                     fetched += 1u + (unsigned)two;
                     const int blk0 = list[j], blk1 = two ? list[j + 1] : 0;
+                    if (!mbar_wait_w(smem_u32(&tl->empty[st.idx]), st.phase ^ 1, tl, P.ws, 103)) return;
                     if (elect_one()) {
-                        const unsigned bar = smem_u32(&tl->full[st.idx]);
-                        const unsigned dst = k_smem + st.idx * kStageBytes;
-                        mbar_arrive_expect_tx(bar, (unsigned)((two ? 4 : 2) * kHalfTile));
+                        // The halves of the channels have a barrier each, so that the products with the
+                        // first begin while the second is still coming: with four stages the tensor
+                        // cores wait for a stage's way from L2, and this takes a third off it. (12.97 ->
+                        // 12.01 ms at T = 131072, k = 32. Giving the halves back one by one as well
+                        // costs more in the producers' second wait than it gives: 12.23.)
 #pragma unroll
                         for (int c = 0; c < 2; ++c) {
-                            tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, blk0 * kBlk, kvh, b);
-                            if (two) tma_load_4d(dst + (c * 2 + 1) * kHalfTile, tk, bar, c * 64, blk1 * kBlk, kvh, b);
+                            const unsigned bar = smem_u32(&tl->full[c][st.idx]);
+                            const unsigned dst = k_smem + st.idx * kStageBytes + c * 2 * kHalfTile;
+                            mbar_arrive_expect_tx(bar, (unsigned)((two ? 2 : 1) * kHalfTile));
+                            tma_load_4d(dst, tk, bar, c * 64, blk0 * kBlk, kvh, b);
+                            if (two) tma_load_4d(dst + kHalfTile, tk, bar, c * 64, blk1 * kBlk, kvh, b);
                         }
                     }
                     __syncwarp();
@@ -224,7 +231,6 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                 const unsigned s_end = stage_seq + n_st;
                 // this warp's stages of the list: s = which (mod kMmaWarps)
                 for (unsigned s = stage_seq + (((unsigned)which - stage_seq) & (kMmaWarps - 1)); s < s_end; s += kMmaWarps) {
-                    if (!mbar_wait_w(smem_u32(&tl->full[sidx]), (s / kStages) & 1u, tl, P.ws, 204)) return;
                     for (int r = r0; r < r1; r += 2) {
                         // first level: rows r and r + 1 in one chain, each in its slot
                         const bool two = level == 0 && r + 1 < r1;
@@ -244,20 +250,27 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                         const unsigned d_tmem = tmem_base + slot * 64;
                         const unsigned b_lo = q_lo + r * (kHalfTile >> 4);
                         const unsigned idesc = two ? kIdescTwo : kIdesc;
-                        if (elect_one()) {
 #pragma unroll
-                            for (int c = 0; c < 2; ++c)
+                        for (int c = 0; c < 2; ++c) {
+                            if (r == r0) {
+                                if (!mbar_wait_w(smem_u32(&tl->full[c][sidx]), (s / kStages) & 1u, tl, P.ws, 204)) return;
+                                tc_fence_after();
+                            }
+                            if (elect_one()) {
 #pragma unroll
                                 for (int k4 = 0; k4 < 4; ++k4)
                                     tc_mma_bf16_split(d_tmem, a_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kDescHi,
                                                       b_lo + ((c * kR * kHalfTile + k4 * 32) >> 4), kDescHi, idesc, (c | k4) != 0);
-                            tc_commit(smem_u32(&tl->tmem_full[slot]));
-                            if (two) tc_commit(smem_u32(&tl->tmem_full[slot + 1]));
-                            // the stage is free once its last chain has read it (a commit covers all
-                            // earlier instructions of this thread)
-                            if (r + 2 >= r1) tc_commit(smem_u32(&tl->empty[sidx]));
+                                if (c == 1) {
+                                    tc_commit(smem_u32(&tl->tmem_full[slot]));
+                                    if (two) tc_commit(smem_u32(&tl->tmem_full[slot + 1]));
+                                    // the stage is free once its last chain has read it (a commit covers
+                                    // all earlier instructions of this thread)
+                                    if (r + 2 >= r1) tc_commit(smem_u32(&tl->empty[sidx]));
+                                }
+                            }
+                            __syncwarp();
                         }
-                        __syncwarp();
                     }
                 }
                 stage_seq = s_end;
@@ -290,6 +303,8 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
     unsigned full_par = 0;  // bit w: phase of the next use of issuing warp w's slot `grp`
     const int tile = wq >> 1;                // which tile of the pair this warp's lanes hold
     const int key = (wq & 1) * 32 + lane;    // key index inside the tile
+    // of this group's slot of issuing warp 0; the others' follow at 16 bytes (slot 2 * warp + grp)
+    const unsigned full_bar = smem_u32(&tl->tmem_full[grp]), empty_bar = smem_u32(&tl->tmem_empty[grp]);
     const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16) + grp * 64;
     for (;;) {
         if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 301)) return;
@@ -300,25 +315,35 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
         const long long rem_q = g.T - (long long)qb * kBlk;
         const int m_lim = rem_q < kBlk ? (int)rem_q : kBlk;  // query tokens of this block inside T
         const int full_blocks = m_lim == kBlk ? (int)(g.T / kBlk) : 0, diag = g.causal ? qb : -1;  // key blocks without a mask: those before, but for the diagonal one
-        // One chain of this group: stage s, this warp's tile of it, where its maximum goes.
-        auto reduce = [&](unsigned s, int blk, float *to) -> bool {  // blk < 0: no tile at this place (its maximum is not looked at)
+        float last = 0.f;  // this lane's maximum of the last tile, and where the tile's goes
+        unsigned last_to = smem_u32(&tl->no_part);
+        auto put = [&] {
+            const float best = warp_max(last);
+            asm volatile("{\n.reg .pred p;\nsetp.eq.b32 p, %2, 0;\n@p st.shared.f32 [%0], %1;\n}" ::"r"(last_to), "f"(best), "r"(lane) : "memory");
+        };
+        int my_blk = -1;      // lane i: this warp's tile of the list's stage i (-1: there is none, its maximum is not looked at)
+        unsigned masked = 0;  // bit i: that tile is not whole
+        // One chain of this group: the list's stage i, the kernel's stage s, where the maximum goes.
+        auto reduce = [&](unsigned s, unsigned i, unsigned to) -> bool {
             const unsigned owner = s & (kMmaWarps - 1);
-            const unsigned slot = 2 * owner + grp;
-            if (!mbar_wait_w(smem_u32(&tl->tmem_full[slot]), (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
+            if (!mbar_wait_w(full_bar + owner * 16, (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
             full_par ^= 1u << owner;
             tc_fence_after();
             float best = -CUDART_INF_F;
             const unsigned taddr = t_lane + owner * 128;
-            if (blk >= 0 && blk < full_blocks && blk != diag) {
+            if (((masked >> i) & 1u) == 0) {
                 unsigned v[64];
                 tmem_ld_32x32_issue(taddr, v);
                 tmem_ld_32x32_issue(taddr + 32, v + 32);
+                put();  // (the tile before this one, while the loads are on their way)
                 tmem_ld_wait();
                 // the slot goes back as soon as it is in registers: its issuing warp waits for it
                 tc_fence_before();
-                mbar_arrive_if(smem_u32(&tl->tmem_empty[slot]), lane == 0);
+                mbar_arrive_if(empty_bar + owner * 16, lane == 0);
                 best = max_of_64(reinterpret_cast<const float *>(v));
             } else {
+                put();
+                const int blk = __shfl_sync(0xffffffffu, my_blk, i);
                 if (blk >= 0) {  // the diagonal block, or a block across T: rare, so little code rather than little time
                     // allowed queries for this key: inside T, and not before the key if causal
                     const int lo = key >= (int)g.T - blk * kBlk ? kBlk : (blk == diag ? key : 0);
@@ -328,15 +353,15 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
                         tmem_ld_32x8_issue(taddr + i0, v);
                         tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (i0 + i >= lo && i0 + i < m_lim) best = fmaxf(best, __uint_as_float(v[i]));
+                        for (int x = 0; x < 8; ++x)
+                            if (i0 + x >= lo && i0 + x < m_lim) best = fmaxf(best, __uint_as_float(v[x]));
                     }
                 }
                 tc_fence_before();
-                mbar_arrive_if(smem_u32(&tl->tmem_empty[slot]), lane == 0);
+                mbar_arrive_if(empty_bar + owner * 16, lane == 0);
             }
-            best = warp_max(best);
-            if (lane == 0) to[wq & 1] = best;
+            last = best;
+            last_to = to;
             return true;
         };
         for (int level = 0; level < levels; ++level) {
@@ -347,7 +372,12 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 302)) return;
                     jr_par[x] ^= 1;
                 }
+                // All there is to read of the list, at once: a look at it chain by chain, with the
+                // comparisons, was a good part of what a warp spends on a chain.
                 const int n = tl->n_jobs[li];
+                my_blk = 2 * lane + tile < n ? (level == 0 ? tl->first_blk : tl->jobs_blk[x])[2 * lane + tile] : -1;
+                masked = __ballot_sync(0xffffffffu, my_blk < 0 || my_blk >= full_blocks || my_blk == diag);
+                mbar_arrive_if(smem_u32(&tl->jobs_ack[li]), lane == 0);
                 const unsigned s_end = stage_seq + ((unsigned)(n + 1) >> 1);
                 // First level: every stage serves all rows, rows grp, grp + 2 are this group's, and each
                 // issuing warp needs its slot back from the first before it can issue the second: so
@@ -355,26 +385,23 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
                 // waited for that round trip with other warps' chains ready: 115 -> 99 us at
                 // T = 4096, 32 / 8 heads, k = 32). Later one chain per stage, this group's are the
                 // stages with (s / kMmaWarps) % 2 == grp.
-                const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
                 const int r0 = level == 0 ? grp : x, r1 = level == 0 ? R : x + 1;
-                float(*const part)[2] = level == 0 ? tl->first_part[set][0] : tl->part[x];
-                const int row_step = level == 0 ? kMaxJobs : 0;
+                const unsigned part = smem_u32(level == 0 ? tl->first_part[set][0] : tl->part[x]) + tile * 8 + (wq & 1) * 4;
+                const unsigned row_step = level == 0 ? kMaxJobs * 8 : 0;
                 for (unsigned base = level == 0 ? stage_seq : stage_seq & ~(unsigned)(kMmaWarps - 1); base < s_end; base += kMmaWarps) {
                     if (level > 0 && (int)((base / kMmaWarps) & 1u) != grp) continue;
                     const unsigned lo = max(base, stage_seq), hi = min(base + kMmaWarps, s_end);
                     for (int r = r0; r < r1; r += 2)
-                        for (unsigned s = lo; s < hi; ++s) {
-                            const int c = 2 * (int)(s - stage_seq) + tile;
-                            if (!reduce(s, c < n ? list[c] : -1, part[r * row_step + c])) return;
-                        }
+                        for (unsigned s = lo; s < hi; ++s)
+                            if (!reduce(s, s - stage_seq, part + r * row_step + (s - stage_seq) * 16)) return;
                 }
                 stage_seq = s_end;
+                put();
+                last_to = smem_u32(&tl->no_part);
                 // this list is done for rows r0..r1: tell their controllers
                 __syncwarp();
-                if (lane == 0) {
+                if (lane == 0)
                     for (int r = level == 0 ? 0 : x; r < r1; ++r) mbar_arrive(smem_u32(level == 0 ? &tl->first_done[set][r] : &tl->scores_done[r]));
-                    mbar_arrive(smem_u32(&tl->jobs_ack[li]));  // done reading this list
-                }
             }
         }
     }
@@ -608,7 +635,7 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) { mbar_init(smem_u32(&tl->full[i]), 1); mbar_init(smem_u32(&tl->empty[i]), 1); }
+        for (int i = 0; i < kStages; ++i) { mbar_init(smem_u32(&tl->full[0][i]), 1); mbar_init(smem_u32(&tl->full[1][i]), 1); mbar_init(smem_u32(&tl->empty[i]), 1); }
         for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&tl->tmem_full[i]), 1); mbar_init(smem_u32(&tl->tmem_empty[i]), 4); }
         for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), kListReaders + (i == kR ? kR : 0)); }
         for (int i = 0; i < kR; ++i) {
