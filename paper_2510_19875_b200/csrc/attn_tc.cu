@@ -3,24 +3,25 @@
 //
 // One persistent CTA per SM works through "pairs": two rows (query blocks) of one kv head - two query
 // heads at one query block, or, where the number of heads per kv head is odd, two neighbouring
-// query blocks of the last head. Their Q tiles are stacked into one 128-row A operand. For every mask
-// entry e the two rows name one key block each (K_a, K_b, usually different); the tiles arrive by
-// TMA (128-byte swizzle), stacked too, and
-//     S = [Q_0; Q_1] [K_a; K_b]^T      (128 x 128, fp32 in TMEM)
-// holds row 0's logits in its upper-left quadrant and row 1's in its lower-right one.
+// query blocks of the last head. For every mask entry e the two rows name one key block each (K_0, K_1,
+// usually different); the tiles arrive by TMA (128-byte swizzle), and each row r has its own products,
+//     S_r = Q_r K_r^T  (64 x 64),     O_r += P_r V_r  (64 x 128),
+// with M = 64: a row's 64 tokens take 16 of every 32 TMEM lanes (token 16 w + i in lane 32 w + 16 r + i),
+// so the two rows share the columns of an accumulator and of P. A 64-row product takes the tensor
+// cores as long as one of both rows together would (128 x 128 with half of S thrown away, 128 x 128
+// under an output-lane mask for O), but less energy, and the chip is at its power limit here:
+// 1475 -> 1660 MHz in a long run, 128k tokens (32 / 8 heads, k = 32) 6560 -> 6330 us, four layers of
+// 9999 (k = 16) 935 -> 883, 4096 (k = 32) 166 -> 158.
 //
 // Two softmax groups of four warps take a pair's entries in turn (its n-th kept entry belongs to
 // group n % 2, so that a pair's arithmetic does not depend on what the CTA did before), so
 // that one group's chain of waits, TMEM loads and exponentials runs beside the other's. A thread
 // owns one query token (TMEM lane) of its group's entries: it reads the token's 64 logits, applies
 // the element-level mask C, and writes P = exp2(scale (s - ref)) as bf16 to TMEM, where the P V
-// product takes it as its A operand. Two chains with an output-lane mask,
-//     O[lanes 0..63]   += P[rows 0..63]   V_a,      O[lanes 64..127] += P[rows 64..127] V_b
-// (128 x 128, fp32, in TMEM; V tiles MN-major), add each row's contribution and leave the other
-// row's lanes alone. One logit buffer and two P buffers per group and one O fill the 512 TMEM
-// columns: the logits are given back as soon as they are in registers, and P need not wait for the
-// product before. (Three logit buffers with P in their place instead hold a buffer through Q K^T,
-// softmax and P V: 1470 clocks an entry, this split V3_CLK.)
+// product takes it as its A operand. The logits are given back as soon as they are in registers, and
+// P, with two buffers per group, need not wait for the product before. (Three logit buffers with P in
+// their place instead hold a buffer through Q K^T, softmax and P V: 1470 clocks an entry, this
+// split 1330.)
 //
 // `ref` is a per-token reference kept instead of the exact running maximum (bf16 P and fp32 sums
 // keep their relative precision whatever the reference, as long as nothing overflows): the
@@ -32,9 +33,10 @@
 // and P computed again. At the end of a pair the groups exchange their sums, normalise and store
 // half of the channels each.
 //
-// What this form replaces kept P in shared memory (64 KB of stores and proxy fences, and a group's
-// buffer held until its product was complete) and one O per group: an entry took 1560 clocks, the
-// two chains of an entry keep the tensor pipe busy for 1024 (ATTN_V2).
+// What bounds it: an entry's products keep the tensor cores busy for 1050 clocks, its softmax work is
+// about 2000 of one group's, and the chip runs at its power limit; an entry takes 1500 clocks at
+// 1660 MHz. (With P in shared memory, 64 KB of stores and proxy fences, and one O per group: 1560 at
+// the lower clock.)
 //
 // Roles (384 threads): warp 0 brings the K and Q tiles by TMA, warp 2 the V tiles and, ahead of
 // everyone else, the pairs' mask rows; warp 1 issues the Q K^T chains and owns TMEM; warp 3 issues
@@ -61,7 +63,7 @@ constexpr int kThreads = 384;
 constexpr int kBlk = 64, kD = 128;
 constexpr int kHalfTile = kBlk * 128;       // 64 rows x 128 bytes
 constexpr int kTile = 2 * kHalfTile;        // one 64 x 128 tile
-constexpr int kOperand = 2 * kTile;         // two tiles (K_a, K_b or V_a, V_b), or the 128-row Q operand
+constexpr int kOperand = 2 * kTile;         // two tiles: an entry's K or V, or the Q of a pair
 // Stages of the two rings, out of the operand buffers shared memory has room for beside Q: five (a V
 // stage is held from its load until the product of its entry is complete, a whole softmax later:
 // V three, K two), or four when the mask rows are long.
@@ -78,8 +80,8 @@ struct Item {
     int h[2], qb[2];
 };
 
-// TMEM columns: logits of group g at 128 g, its two P buffers at 256 + 64 g and 32 behind, O at 384.
-constexpr int kPCol = 256, kOCol = 384;
+// TMEM columns: logits of group g at 64 g, its two P buffers at 128 + 64 g and 32 behind, O at 256.
+constexpr int kPCol = 128, kOCol = 256;
 struct Tail {
     unsigned long long q_full[2], q_free[2];  // q_free: the output staged over the pair's Q has left (8 warps)
     unsigned long long k_full[kMaxKStages], k_empty[kMaxKStages], v_full[kMaxVStages], v_empty[kMaxVStages];
@@ -102,8 +104,9 @@ struct Tail {
 constexpr int kFixedOperands = 2;  // Q; behind it the V stages, then the K stages
 constexpr int kMaxSmemPerCta = 232448;
 
-constexpr unsigned kIdescQK = idesc_bf16(128, 128, false);  // B = stacked K tiles, K-major
-constexpr unsigned kIdescPV = idesc_bf16(128, 128, true);   // B = stacked V tiles, MN-major
+constexpr unsigned kIdescQK = idesc_bf16(64, 64, false);  // B = a K tile, K-major
+constexpr unsigned kIdescPV = idesc_bf16(64, 128, true);  // B = a V tile, MN-major
+constexpr unsigned kRowLanes = 16u << 16;  // row 1's accumulator and P: the upper half of every 32 lanes
 constexpr unsigned kHiK = desc_hi_sw128(1024);              // every operand: 8-row (8-key) groups 1024 bytes apart
 
 struct Params {
@@ -385,7 +388,7 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail *tl
 // The two issuing roles are run by all 32 lanes of their warps, converged: the waits are
 // warp-wide, one elected lane issues.
 
-// S = [Q_0; Q_1] [K_a; K_b]^T for every kept entry.
+// S_r = Q_r K_r^T of both rows for every kept entry.
 __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base) {
     Ring ks, ms, qs;
     unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
@@ -403,15 +406,17 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++;  // entry i of a pair belongs to group i % 2
             if (!wait_w(smem_u32(&tl->s_free[gi]), (use & 1u) ^ 1u, tl, 203)) return;
             tc_fence_after();
-            const unsigned d_tmem = tmem_base + gi * 128;
+            const unsigned d_tmem = tmem_base + gi * 64;
             const unsigned b_lo = k_lo + ks.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
+                for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int k4 = 0; k4 < 4; ++k4)
-                        tc_mma_bf16_split(d_tmem, q_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK,
-                                          b_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int k4 = 0; k4 < 4; ++k4)
+                            tc_mma_bf16_split(d_tmem + r * kRowLanes, q_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK,
+                                              b_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
                 tc_commit(smem_u32(&tl->s_full[gi]));
                 tc_commit(smem_u32(&tl->k_empty[ks.idx]));
             }
@@ -424,7 +429,7 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
     }
 }
 
-// O (+)= P [V_a; V_b] for every kept entry; a pair's first entry starts O afresh.
+// O_r (+)= P_r V_r of both rows for every kept entry; a pair's first entry starts O afresh.
 __device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tmem_base) {
     Ring vs, ms;  // vs: the entry's V stage
     unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
@@ -446,13 +451,11 @@ __device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tme
             const unsigned a_tmem = tmem_base + kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
-                for (int tile = 0; tile < 2; ++tile) {  // row `tile` of the pair: its P rows, its V tile, its lanes
-                    const unsigned lo_off = tile ? 0xFFFFFFFFu : 0u, hi_off = tile ? 0u : 0xFFFFFFFFu;
+                for (int r = 0; r < 2; ++r)  // row r of the pair: its P, its V tile
 #pragma unroll
                     for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step: 8 columns of packed bf16
-                        tc_mma_bf16_ta_masked(d_tmem, a_tmem + s4 * 8, b_lo + ((tile * kTile + s4 * 2048) >> 4), kHiK, kIdescPV,
-                                              (i | s4) != 0, lo_off, lo_off, hi_off, hi_off);
-                }
+                        tc_mma_bf16_ta(d_tmem + r * kRowLanes, a_tmem + r * kRowLanes + s4 * 8, b_lo + ((r * kTile + s4 * 2048) >> 4), kHiK,
+                                       kIdescPV, (i | s4) != 0);
                 tc_commit(smem_u32(&tl->p_free[gi][pb]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
                 if (i + 1 == n_entries) tc_commit(smem_u32(&tl->o_done));
@@ -488,7 +491,7 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
     tmem_st_wait();
 }
 
-// One softmax group: four warps, thread = query token (TMEM lane) `row` of the pair, for the
+// One softmax group: four warps, thread = TMEM lane `row`, token `mq` of the pair's row `half`, for the
 // entries n with n % 2 == grp (n numbers the kept entries of each pair, as in every role).
 // The waits are warp-wide (same answer in every lane), so the warp stays converged for the
 // warp-collective TMEM loads and stores and leaves together if the CTA aborts.
@@ -499,13 +502,13 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 // o_done.
 __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
     const Geom &g = P.g;
-    const int lane = t & 31, row = t & 127, grp = t >> 7, half = row >> 6, mq = row & 63, wq = row >> 5;
+    const int lane = t & 31, row = t & 127, grp = t >> 7, wq = row >> 5, half = lane >> 4, mq = wq * 16 + (lane & 15);
     const unsigned lanes = tmem_base + ((unsigned)(row & ~31) << 16);
     const unsigned turn_own = smem_u32(&tl->turn[wq][grp]), turn_other = smem_u32(&tl->turn[wq][grp ^ 1]);
     unsigned char *const stage = q_ptr + (grp * 4 + wq) * 4096;  // this warp's 32 tokens x 64 channels in a Q buffer
     unsigned n_other = 0;     // entries of the other group before this pair, over the whole kernel
     unsigned n_own = 0;       // entries of this group so far
-    const unsigned s_full = smem_u32(&tl->s_full[grp]), s_free = smem_u32(&tl->s_free[grp]), s_addr = lanes + grp * 128 + half * 64;
+    const unsigned s_full = smem_u32(&tl->s_full[grp]), s_free = smem_u32(&tl->s_free[grp]), s_addr = lanes + grp * 64;
     unsigned pair_par = 0;    // phase of the barriers that complete once per pair with entries
     int staged = -1;          // Q buffer whose staged output may still be on its way out
     Ring ms, qs;
@@ -676,9 +679,12 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             }
             fence_async_smem();
             __syncwarp();
-            const int tok = tq0 + (wq & 1) * 32;
-            if (lane == 0 && row_active) {  // lane 0 holds the first of the 32 tokens
-                tma_store_4d(to, smem_u32(stage + qs.idx * kOperand), grp * 64, tok, h, b);
+            const int h_1 = __shfl_sync(0xffffffffu, h, 16), tok_1 = __shfl_sync(0xffffffffu, tq0, 16) + wq * 16;
+            const bool there_1 = __shfl_sync(0xffffffffu, (int)row_active, 16) != 0;
+            if (lane == 0) {  // lanes 0 and 16 hold the first of the 16 tokens of a row
+                const unsigned src = smem_u32(stage + qs.idx * kOperand);
+                if (row_active) tma_store_4d(to, src, grp * 64, tq0 + wq * 16, h, b);
+                if (there_1) tma_store_4d(to, src + 16 * 128, grp * 64, tok_1, h_1, b);
                 tma_store_commit();
             }
             staged = qs.idx;
@@ -782,7 +788,7 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
     if (rc != STREAM_OK) return rc;
     rc = make_map5_bf16_d128(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v");
     if (rc != STREAM_OK) return rc;
-    rc = make_map_bf16_d128(&to, out, g.T, g.H, g.batch, kD, g.T * kD, (long long)g.H * g.T * kD, "out", 32);
+    rc = make_map_bf16_d128(&to, out, g.T, g.H, g.batch, kD, g.T * kD, (long long)g.H * g.T * kD, "out", 16);
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;

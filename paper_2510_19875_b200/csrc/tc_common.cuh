@@ -160,7 +160,19 @@ __device__ __forceinline__ void tc_mma_bf16_split(unsigned d_tmem, unsigned a_lo
         : "memory");
 }
 
-// The same with A from TMEM (lane = row, two bf16 per column) and an output-lane mask: bit i of the
+// The same with A from TMEM (two bf16 per column). M = 128: lane = row. M = 64: row r of A and of the
+// accumulator in lane (r / 16) * 32 + r % 16, or, with 16 added to both lane addresses, 16 lanes behind:
+// two such products share their columns.
+__device__ __forceinline__ void tc_mma_bf16_ta(unsigned d_tmem, unsigned a_tmem, unsigned b_lo, unsigned b_hi, unsigned idesc,
+                                               unsigned accumulate) {
+    asm volatile(
+        "{\n.reg .pred p;\n.reg .b64 db;\nmov.b64 db, {%2, %3};\nsetp.ne.b32 p, %5, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// With A from TMEM, M = 128 and an output-lane mask: bit i of the
 // 128-bit vector {m0 (lanes 0..31), m1, m2, m3} set = accumulator lane i is left untouched.
 __device__ __forceinline__ void tc_mma_bf16_ta_masked(unsigned d_tmem, unsigned a_tmem, unsigned b_lo, unsigned b_hi,
                                                       unsigned idesc, unsigned accumulate, unsigned m0, unsigned m1,
