@@ -18,8 +18,9 @@
 // that one group's chain of waits, TMEM loads and exponentials runs beside the other's. A thread
 // owns one query token (TMEM lane) of its group's entries: it reads the token's 64 logits, applies
 // the element-level mask C, and writes P = exp2(scale (s - ref)) as bf16 to TMEM, where the P V
-// product takes it as its A operand. The logits are given back as soon as they are in registers, and
-// P, with two buffers per group, need not wait for the product before. (Three logit buffers with P in
+// product takes it as its A operand. The logits are given back as soon as they are in registers.
+// A group has two buffers of logits and two of P: its next logits are there when it comes for them
+// (with one buffer 421 against 411 us at T = 16384), and P need not wait for the product before. (Three logit buffers with P in
 // their place instead hold a buffer through Q K^T, softmax and P V: 1470 clocks an entry, this
 // split 1330.)
 //
@@ -80,12 +81,13 @@ struct Item {
     int h[2], qb[2];
 };
 
-// TMEM columns: logits of group g at 64 g, its two P buffers at 128 + 64 g and 32 behind, O at 256.
-constexpr int kPCol = 128, kOCol = 256;
+// TMEM columns: the two logit buffers of group g at 128 g and 64 behind, its two P buffers at 256 + 64 g
+// and 32 behind, O at 384.
+constexpr int kPCol = 256, kOCol = 384;
 struct Tail {
     unsigned long long q_full[2], q_free[2];  // q_free: the output staged over the pair's Q has left (8 warps)
     unsigned long long k_full[kMaxKStages], k_empty[kMaxKStages], v_full[kMaxVStages], v_empty[kMaxVStages];
-    unsigned long long s_full[2], s_free[2];              // per group: logits ready / read
+    unsigned long long s_full[2][2], s_free[2][2];        // per group and logit buffer: ready / read
     unsigned long long p_full[2][2], p_free[2][2];        // per group and P buffer: published / product added
     unsigned long long o_done, o_free;     // a pair's last product is complete; its O has been read (8 warps)
     // Between the two softmax warps of a lane quarter (one per group): the pair's first references
@@ -244,61 +246,64 @@ __device__ __forceinline__ bool idle_ok(Tail *tl, long long t_last, unsigned cod
 
 __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, Tail *tl, unsigned q_smem,
                                 unsigned k_smem) {
-    Ring qs;
     LoadStream S;
     S.round = 0;
     S.id = nth_item(P, 0);
     S.e = -2;
-    bool q_due = false;  // the pair's Q tiles still have to be requested
     auto step = [&]() -> bool {
-        if (S.e == -2) {
-            if (!open_pair(P, tl, S)) return false;
-            q_due = S.n > 0;
-            return true;
-        }
-        if (S.e >= S.n && !q_due) { close_pair(P, tl, S); return true; }
-        if (S.e == 0 || !q_due) {
-            // a K stage is free once the logits computed from it are complete
-            if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
-            if (elect_one()) {
-                // [half][tile][64 rows][128 B]; a row without a block at an entry gets block 0, its logits are masked out
-                const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * kOperand;
-                const int ba = max(S.cur.a, 0), bb = max(S.cur.b, 0);
-                mbar_arrive_expect_tx(bar, (unsigned)kOperand);
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, ba * kBlk, S.kvh, S.b);
-                    tma_load_4d(dst + c * 2 * kHalfTile + kHalfTile, tk, bar, c * 64, bb * kBlk, S.kvh, S.b);
-                }
-            }
-            __syncwarp();
-            S.ring.advance(P.n_k_stages);
-            next_entry(P, tl, S);
-            return true;
-        }
-        // Q goes behind the pair's first K tiles, which do not depend on the Q buffer
-        if (!probe_w(smem_u32(&tl->q_free[qs.idx]), qs.phase ^ 1)) return false;
+        if (S.e == -2) return open_pair(P, tl, S);
+        if (S.e >= S.n) { close_pair(P, tl, S); return true; }
+        // a K stage is free once the logits computed from it are complete
+        if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
         if (elect_one()) {
-            const Item &it = tl->m_item[S.ms.idx];
-            const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
+            // [half][tile][64 rows][128 B]; a row without a block at an entry gets block 0, its logits are masked out
+            const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * kOperand;
+            const int ba = max(S.cur.a, 0), bb = max(S.cur.b, 0);
             mbar_arrive_expect_tx(bar, (unsigned)kOperand);
 #pragma unroll
-            for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const bool second = r == 1 && it.R == 2;
-                    tma_load_4d(q_smem + qs.idx * kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64,
-                                (second ? it.qb[1] : it.qb[0]) * kBlk, second ? it.h[1] : it.h[0], S.b);
-                }
+            for (int c = 0; c < 2; ++c) {
+                tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, ba * kBlk, S.kvh, S.b);
+                tma_load_4d(dst + c * 2 * kHalfTile + kHalfTile, tk, bar, c * 64, bb * kBlk, S.kvh, S.b);
+            }
         }
         __syncwarp();
-        q_due = false;
-        qs.advance(2);
+        S.ring.advance(P.n_k_stages);
+        next_entry(P, tl, S);
+        return true;
+    };
+    // The pairs' Q tiles, as early as a buffer and the pair's mask rows allow, a pair ahead of its K tiles
+    // as a rule: asked for behind the pair's first K tiles they came 1200 clocks late. (A pair's mask
+    // slot stays until this warp has closed the pair on the K side, which a pair's Q precedes.)
+    Ring qs, qm;
+    int q_round = 0, q_id = nth_item(P, 0);
+    auto q_step = [&]() -> bool {
+        if (q_id >= P.n_items || !probe_w(smem_u32(&tl->m_full[qm.idx]), qm.phase)) return false;
+        if (tl->m_count[qm.idx] > 0) {
+            if (!probe_w(smem_u32(&tl->q_free[qs.idx]), qs.phase ^ 1)) return false;
+            if (elect_one()) {
+                const Item &it = tl->m_item[qm.idx];
+                const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
+                mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+#pragma unroll
+                for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const bool second = r == 1 && it.R == 2;
+                        tma_load_4d(q_smem + qs.idx * kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64,
+                                    (second ? it.qb[1] : it.qb[0]) * kBlk, second ? it.h[1] : it.h[0], it.b);
+                    }
+            }
+            __syncwarp();
+            qs.advance(2);
+        }
+        qm.advance(kMaskSlots);
+        q_id = nth_item(P, ++q_round);
         return true;
     };
     long long t_last = clock64();
     while (S.id < P.n_items) {
-        if (step()) t_last = clock64();
+        // (a pair is closed only when its Q has been asked for: its mask slot is then given back)
+        if (((S.e < S.n || S.round < q_round) && step()) || q_step()) t_last = clock64();
         else if (!idle_ok(tl, t_last, 101)) return;
     }
 }
@@ -404,9 +409,9 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, tl, 202)) return;
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++;  // entry i of a pair belongs to group i % 2
-            if (!wait_w(smem_u32(&tl->s_free[gi]), (use & 1u) ^ 1u, tl, 203)) return;
+            if (!wait_w(smem_u32(&tl->s_free[gi][use & 1u]), ((use >> 1) & 1u) ^ 1u, tl, 203)) return;
             tc_fence_after();
-            const unsigned d_tmem = tmem_base + gi * 64;
+            const unsigned d_tmem = tmem_base + gi * 128 + (use & 1u) * 64;
             const unsigned b_lo = k_lo + ks.idx * (kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
@@ -417,7 +422,7 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
                         for (int k4 = 0; k4 < 4; ++k4)
                             tc_mma_bf16_split(d_tmem + r * kRowLanes, q_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK,
                                               b_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
-                tc_commit(smem_u32(&tl->s_full[gi]));
+                tc_commit(smem_u32(&tl->s_full[gi][use & 1u]));
                 tc_commit(smem_u32(&tl->k_empty[ks.idx]));
             }
             __syncwarp();
@@ -508,7 +513,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
     unsigned char *const stage = q_ptr + (grp * 4 + wq) * 4096;  // this warp's 32 tokens x 64 channels in a Q buffer
     unsigned n_other = 0;     // entries of the other group before this pair, over the whole kernel
     unsigned n_own = 0;       // entries of this group so far
-    const unsigned s_full = smem_u32(&tl->s_full[grp]), s_free = smem_u32(&tl->s_free[grp]), s_addr = lanes + grp * 64;
+    const unsigned s_full = smem_u32(&tl->s_full[grp][0]), s_free = smem_u32(&tl->s_free[grp][0]), s_addr = lanes + grp * 128;
     unsigned pair_par = 0;    // phase of the barriers that complete once per pair with entries
     int staged = -1;          // Q buffer whose staged output may still be on its way out
     Ring ms, qs;
@@ -537,14 +542,15 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
         bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
             // the token's 64 logits against its row's key block
-            if (!wait_w(s_full, n_own & 1u, tl, 301)) return;
+            const unsigned pb = n_own & 1u;  // the entry's logit and P buffer
+            if (!wait_w(s_full + pb * 8, (n_own >> 1) & 1u, tl, 301)) return;
             tc_fence_after();
             unsigned sr[64];
-            tmem_ld_32x32_issue(s_addr, sr);
-            tmem_ld_32x32_issue(s_addr + 32, sr + 32);
+            tmem_ld_32x32_issue(s_addr + pb * 64, sr);
+            tmem_ld_32x32_issue(s_addr + pb * 64 + 32, sr + 32);
             tmem_ld_wait();
             tc_fence_before();
-            mbar_arrive_if(s_free, lane == 0);
+            mbar_arrive_if(s_free + pb * 8, lane == 0);
             if (masked) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
@@ -567,7 +573,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             const unsigned other = n_other + (unsigned)((n - 1) >> 1), turn_par = other & 1u;  // entry n - 1 is the other group's `other`-th
             const int next_blk = my_row[min(n + 2, last_entry)];  // (of no meaning behind the last)
             int next_hi = 0;
-            const unsigned pb = n_own & 1u, p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own >> 1) & 1u) ^ 1u;
+            const unsigned p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own >> 1) & 1u) ^ 1u;
             unsigned packed[32];
             float esum;
             for (int attempt = 0;; ++attempt) {
@@ -720,9 +726,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         for (int i = 0; i < kMaxKStages; ++i) { mbar_init(smem_u32(&tl->k_full[i]), 1); mbar_init(smem_u32(&tl->k_empty[i]), 1); }
         for (int i = 0; i < kMaxVStages; ++i) { mbar_init(smem_u32(&tl->v_full[i]), 1); mbar_init(smem_u32(&tl->v_empty[i]), 1); }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(smem_u32(&tl->s_full[i]), 1);
-            mbar_init(smem_u32(&tl->s_free[i]), 4);
-            for (int j = 0; j < 2; ++j) { mbar_init(smem_u32(&tl->p_full[i][j]), 4); mbar_init(smem_u32(&tl->p_free[i][j]), 1); }
+            for (int j = 0; j < 2; ++j) { mbar_init(smem_u32(&tl->s_full[i][j]), 1); mbar_init(smem_u32(&tl->s_free[i][j]), 4); mbar_init(smem_u32(&tl->p_full[i][j]), 4); mbar_init(smem_u32(&tl->p_free[i][j]), 1); }
         }
         mbar_init(smem_u32(&tl->o_done), 1);
         mbar_init(smem_u32(&tl->o_free), 8);
