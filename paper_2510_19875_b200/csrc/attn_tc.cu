@@ -197,7 +197,7 @@ __device__ __forceinline__ Entry entry_at(const int *rows, int stride, int n) {
 struct LoadStream {
     int round, id;     // pair being walked
     int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
-    int n;             // kept entries of the pair
+    int n = 0;         // kept entries of the pair
     Entry cur;
     int b, kvh;
     Ring ring, ms;
