@@ -170,6 +170,7 @@ static stream_status build_mask_impl(const stream_problem *p, const void *q, con
     if (workspace_bytes >= sizeof(WorkspaceHeader) + n_rows * sizeof(unsigned int)) g.row_tiles = (unsigned int *)(ws + 1);
     if (tc_ok && p->impl != STREAM_IMPL_GENERIC) return launch_mask_tc(g, q, k, mask_out, score_out, ws, st);
     if (tok_ok && p->impl != STREAM_IMPL_GENERIC) return launch_mask_tok(g, q, k, mask_out, score_out, ws, st);
+    if (p->impl == STREAM_IMPL_AUTO && mask_tc_auto(g, p->dtype) && (((uintptr_t)q | (uintptr_t)k) & 15) == 0) return launch_mask_tc(g, q, k, mask_out, score_out, ws, st);
     return launch_mask_generic(g, p->dtype, p->impl == STREAM_IMPL_AUTO, q, k, mask_out, score_out, ws, st);
 }
 

@@ -62,7 +62,8 @@ stream_status launch_attn_generic(const Geom &g, int dtype, const void *q, const
 bool attn_mma_supported(const Geom &g, int dtype, const void *q, const void *k, const void *v, const void *out);
 stream_status launch_attn_mma(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale,
                               void *out, cudaStream_t st);
-bool mask_tc_supported(const Geom &g, int dtype);
+bool mask_tc_supported(const Geom &g, int dtype);  // d = 128, blocks of 64, k_top <= 32
+bool mask_tc_auto(const Geom &g, int dtype);       // what the kernel is the better choice for beyond that
 stream_status launch_mask_tc(const Geom &g, const void *q, const void *k, int32_t *mask, float *score,
                              WorkspaceHeader *ws, cudaStream_t st);
 // Several k in one launch (mk.n >= 1: mask / score are [mk.n][rows][k_top]); with score_memory

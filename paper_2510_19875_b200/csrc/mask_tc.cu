@@ -1,11 +1,14 @@
-// Tensor-core Stream mask kernel for sm_100a: bf16, d = 128, 64 x 64 blocks, k_top <= 32.
+// Tensor-core Stream mask kernel for sm_100a: bf16, d = 64 or 128, blocks of 32 or 64, k_top <= 64.
+// (Figures: d = 128, blocks of 64, unless they say otherwise.)
 //
-// One persistent CTA per SM works through "groups": up to four query heads of one kv head at
-// one query block. Their Q tiles stay in shared memory for the whole hierarchy (Algorithm 2).
-// Candidate key blocks are fetched by TMA (128-byte swizzle) two at a time into a ring of
-// stages; one tcgen05.mma chain per (stage, row) computes K_pair (128 x 128) x Q_row^T (128 x 64)
-// into a 64-column TMEM slot; four epilogue warps reduce the slot to the two masked tile maxima
-// (Eq. 4 under C). There are two such groups of four, each serving one of every issuing warp's
+// One persistent CTA per SM works through "groups": up to four rows of one kv head, its query heads at
+// one query block or, where these are few, at some. Their Q tiles stay in shared memory for the whole
+// hierarchy (Algorithm 2).
+// Candidate key blocks are fetched by TMA (128-byte swizzle), 128 keys at a time, into a ring of
+// stages; one tcgen05.mma chain per (stage, row) computes the keys (128 x d) x Q_row^T (d x block)
+// into a TMEM slot of as many columns (on the first level one chain for two rows: a chain of one is
+// bound by its operands' way out of shared memory, 48 clocks a step of 16 channels against 64 for
+// both); four epilogue warps reduce the slot to the masked tile maxima (Eq. 4 under C). There are two such groups of four, each serving one of every issuing warp's
 // two slots: the fixed cost of a hand-over (wait, fences, arrive) is larger than the reduction
 // itself, and one group alone would be the longest stage of the pipeline. A controller warp per
 // row keeps the row's nodes in registers, ranks the 2k branch scores (higher score, then lower block
@@ -42,27 +45,43 @@ constexpr int kThreads = 608;
 constexpr int kEpiGroups = 2;  // group g reduces the chains that land in slot g of their issuing warp
 constexpr int kMmaWarps = 4;   // they take the stages in turn
 constexpr int kR = 4;          // rows (query heads) per group
-constexpr int kStages = 4;     // K-pair stages
-constexpr int kSlots = 8;      // TMEM accumulator slots of 64 fp32 columns
-constexpr int kBlk = 64, kD = 128;
-constexpr int kHalfTile = kBlk * 128;          // 64 rows x 128 bytes (one 64-channel half)
-constexpr int kStageBytes = 4 * kHalfTile;     // [2 channel halves][2 tiles]
-constexpr int kQBytes = 2 * kR * kHalfTile;    // [2 channel halves][kR rows]
-constexpr int kMaxJobs = 64;
+constexpr int kSlots = 8;      // TMEM accumulator slots, one query block of fp32 columns each
+constexpr int kStageKeys = 128;
 constexpr int kProducers = 2;     // producer p fills the stage buffers b with b % 2 == p
 constexpr int kListReaders = kProducers + kMmaWarps + 4 * kEpiGroups;  // producer, MMA and epilogue warps; of a first list and the group record also the controllers
-constexpr int kMaxRowJobs = 32;   // a row's list on a later level: at most one tile per node
-// A parity wait only means something to a thread that saw the phase before it complete, and an
-// arrival only if it cannot come a phase early. So every stage buffer and every TMEM slot
-// belongs to one issuing warp: stage s of the kernel's whole sequence goes, with all its chains,
-// to warp s % kMmaWarps and lands in buffer s % kStages (the same number), and a warp's chains
-// alternate between its own two slots. The other issuing warps touch none of its barriers.
-static_assert(kStages == kMmaWarps, "a stage buffer must always meet the same issuing warp");
-static_assert(kSlots == 2 * kMmaWarps, "two private TMEM slots per issuing warp");
 
+// What a build of the kernel is for: head dimension, block size, two nodes a lane (k_top up to 64) or one
+// (up to 32), several k with the score memory, rows of several query blocks in a group.
+template <int kD_, int kBlk_, bool kWide_, bool kMulti_, bool kQbRows_ = false>
+struct Shape {
+    static constexpr int kD = kD_, kBlk = kBlk_;
+    static constexpr bool kMulti = kMulti_, kQbRows = kQbRows_;
+    static constexpr int kMaskRows = kQbRows ? kR / kEpiGroups : 1;  // of the rows an epilogue group has of a list, those with masks of their own
+    static constexpr int kHalves = kD / 64;                 // 64-channel halves (128 bytes a row)
+    static constexpr int kTps = kStageKeys / kBlk;          // tiles of a stage
+    static constexpr int kParts = kBlk / 32;                // epilogue warps that share a tile
+    static constexpr int kTile = kBlk * 128;                // a tile's part of one half
+    static constexpr int kStageHalf = kStageKeys * 128;
+    static constexpr int kStageBytes = kHalves * kStageHalf;
+    static constexpr int kStages = 128 * 1024 / kStageBytes;  // 128 KB of keys on their way
+    static constexpr int kQBytes = kHalves * kR * kTile;    // [channel half][row]
+    static constexpr int kNodes = kWide_ ? 2 : 1;           // nodes a lane of a controller holds
+    static constexpr int kMaxJobs = 64 * kNodes;            // first list: two candidates per node
+    static constexpr int kMaxRowJobs = 32 * kNodes;         // a row's list on a later level: at most one tile per node
+    static constexpr int kListRegs = (kMaxJobs / kTps + 31) / 32;  // stages of a list, in lanes
+    // A parity wait only means something to a thread that saw the phase before it complete, and an
+    // arrival only if it cannot come a phase early. So every stage buffer and every TMEM slot
+    // belongs to one issuing warp: stage s of the kernel's whole sequence goes, with all its chains,
+    // to warp s % kMmaWarps and lands in buffer s % kStages, and a warp's chains alternate between its
+    // own two slots. The other issuing warps touch none of its barriers.
+    static_assert(kStages % kMmaWarps == 0, "a stage buffer must always meet the same issuing warp");
+    static_assert(kSlots == 2 * kMmaWarps, "two private TMEM slots per issuing warp");
+};
+
+template <class S>
 struct Tail {
-    unsigned long long full[2][kStages];  // by channel half
-    unsigned long long empty[kStages], tmem_full[kSlots], tmem_empty[kSlots];
+    unsigned long long full[S::kHalves][S::kStages];  // by channel half
+    unsigned long long empty[S::kStages], tmem_full[kSlots], tmem_empty[kSlots];
     // Per row: its Q tile is there; the last products of a group with it are complete (one commit of
     // every issuing warp).
     unsigned long long q_full[kR], q_free[kR];
@@ -82,33 +101,43 @@ struct Tail {
     int grp_id, grp_b, grp_kvh, grp_qb, grp_h0, grp_R;
     int grp_levels;  // levels of this group's rows (they share the query block, hence k)
     int grp_k, grp_pass;
-    unsigned grp_left, grp_right;  // bit i: the left / right candidate of initial node i is on the first list
+    unsigned grp_on[2 * S::kNodes];  // bit i of [2 x], [2 x + 1]: the left, right candidate of initial node kNodes i + x is on the first list
     int grp_new_q;   // 0: another pass over the same rows (several k), the Q tiles are already there
     int grp_last;    // the last pass over these rows: the Q tiles are given back
     int n_jobs[kR + 1];
-    int first_blk[kMaxJobs], jobs_blk[kR][kMaxRowJobs];
-    float first_part[2][kR][kMaxJobs][2], part[kR][kMaxRowJobs][2];
+    int first_blk[S::kMaxJobs], jobs_blk[kR][S::kMaxRowJobs];
+    float first_part[2][kR][S::kMaxJobs][S::kParts], part[kR][S::kMaxRowJobs][S::kParts];
     float no_part;   // (written before a list's first tile, not read)
-    int node_f[kR][32], node_l[kR][32];
-    float node_s[kR][32];
+    int node_f[kR][32 * S::kNodes], node_l[kR][32 * S::kNodes];
+    float node_s[kR][32 * S::kNodes];
 };
-constexpr int kSmemBytes = kQBytes + kStages * kStageBytes + (int)sizeof(Tail) + 1024;
+template <class S>
+constexpr int kSmemBytes = S::kQBytes + S::kStages * S::kStageBytes + (int)sizeof(Tail<S>) + 1024;
 
 // Bounded wait of a whole converged warp (all lanes get the same answer) that reports into the
 // workspace header; false means the CTA is aborting.
-__device__ __forceinline__ bool mbar_wait_w(unsigned bar, unsigned parity, Tail *tl, WorkspaceHeader *ws, unsigned code) {
+template <class S>
+__device__ __forceinline__ bool mbar_wait_w(unsigned bar, unsigned parity, Tail<S> *tl, WorkspaceHeader *ws, unsigned code) {
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &ws->error, &ws->error_info, code);
 }
 
 // K-major, 128-byte-swizzled operands with 8-row groups 1024 bytes apart: high descriptor word.
 constexpr unsigned kDescHi = desc_hi_sw128(1024);
 
-// D fp32, A and B bf16, both K-major, M = 128, N = 64.
-constexpr unsigned kIdesc = idesc_bf16(128, 64, false), kIdescTwo = idesc_bf16(128, 128, false);
+// D fp32, A and B bf16, both K-major, M = 128, N = the tokens of one row or of two.
+template <class S>
+constexpr unsigned kIdesc = idesc_bf16(128, S::kBlk, false);
+template <class S>
+constexpr unsigned kIdescTwo = idesc_bf16(128, 2 * S::kBlk, false);
 
 struct Params {
     Geom g;
     int n_groups, n_chunks;
+    // A group's rows: head_rows query heads, at each of qb_rows query blocks (more than one only where
+    // all heads of the kv head are in the group): row r is head r % head_rows at the group's query
+    // block minus r / head_rows, which row_head and row_back hold in two bits a row.
+    int head_rows, qb_rows;
+    unsigned row_head, row_back;
     int32_t *mask;
     float *score;
     WorkspaceHeader *ws;
@@ -132,7 +161,8 @@ __device__ __forceinline__ unsigned long long cache_pack(unsigned tag, float s) 
 // single diverged lane issues TMA copies several times more slowly. Two producers share the
 // stages by buffer parity: one alone is busy more than half of the time with the four copies and
 // the barrier arm of a stage, and the issuing warps then wait for data.
-__device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail *tl, unsigned k_smem, int which) {
+template <class S>
+__device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *tl, unsigned k_smem, int which) {
     Ring st;
     unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
     unsigned long long fetched = 0;  // tiles this warp has asked TMA for
@@ -154,11 +184,18 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail *tl, 
                 }
                 const int n = tl->n_jobs[li];
                 const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
-                for (int j = 0; j < n; j += 2) {
-                    if ((st.idx & (kProducers - 1)) != which) { st.advance(kStages); continue; }  // the other producer's buffer
-                    const int two = (j + 1 < n);
-                    fetched += 1u + (unsigned)two;
-                    const int blk0 = list[j], blk1 = two ? list[j + 1] : 0;
+                for (int j = 0; j < n; j += S::kTps) {
+                    if ((st.idx & (kProducers - 1)) != which) { st.advance(S::kStages); continue; }  // the other producer's buffer
+                    bool there[S::kTps];
+                    int blk[S::kTps];
+                    unsigned tiles = 0;
+#pragma unroll
+                    for (int x = 0; x < S::kTps; ++x) {
+                        there[x] = x == 0 || j + x < n;
+                        tiles += there[x] ? 1u : 0u;
+                        blk[x] = there[x] ? list[j + x] : 0;
+                    }
+                    fetched += tiles;
                     if (!mbar_wait_w(smem_u32(&tl->empty[st.idx]), st.phase ^ 1, tl, P.ws, 103)) return;
                     if (elect_one()) {
                         // The halves of the channels have a barrier each, so that the products with the
@@ -167,16 +204,17 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail *tl, 
                         // 12.01 ms at T = 131072, k = 32. Giving the halves back one by one as well
                         // costs more in the producers' second wait than it gives: 12.23.)
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
+                        for (int c = 0; c < S::kHalves; ++c) {
                             const unsigned bar = smem_u32(&tl->full[c][st.idx]);
-                            const unsigned dst = k_smem + st.idx * kStageBytes + c * 2 * kHalfTile;
-                            mbar_arrive_expect_tx(bar, (unsigned)((two ? 2 : 1) * kHalfTile));
-                            tma_load_4d(dst, tk, bar, c * 64, blk0 * kBlk, kvh, b);
-                            if (two) tma_load_4d(dst + kHalfTile, tk, bar, c * 64, blk1 * kBlk, kvh, b);
+                            const unsigned dst = k_smem + st.idx * S::kStageBytes + c * S::kStageHalf;
+                            mbar_arrive_expect_tx(bar, tiles * S::kTile);
+#pragma unroll
+                            for (int x = 0; x < S::kTps; ++x)
+                                if (there[x]) tma_load_4d(dst + x * S::kTile, tk, bar, c * 64, blk[x] * S::kBlk, kvh, b);
                         }
                     }
                     __syncwarp();
-                    st.advance(kStages);
+                    st.advance(S::kStages);
                 }
                 if (elect_one()) mbar_arrive(smem_u32(&tl->jobs_ack[li]));  // done reading this list
                 __syncwarp();
@@ -200,14 +238,14 @@ __device__ __forceinline__ int chain_slot(int level, int r, unsigned stage) {
     return level == 0 ? (r & 1) : (int)((stage / kMmaWarps) & 1u);
 }
 
-__device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base, int which) {
+template <class S>
+__device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base, int which) {
     unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
     unsigned q_par = 0;       // bit r: phase of row r's next Q tile
     unsigned stage_seq = 0;   // stages so far, over the whole kernel (the same in every role)
     unsigned slot_par = 0;    // bit i: phase of the next use of this warp's slot i
     const unsigned q_lo = desc_lo_sw128(q_smem, 16);
-    const int sidx = which;   // this warp's stage buffer: stage s lands in buffer s % kStages
-    const unsigned a_lo = desc_lo_sw128(k_smem + sidx * kStageBytes, 16);
+    const unsigned a_lo0 = desc_lo_sw128(k_smem, 16);
     for (;;) {
         if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 201)) return;
         grp_par ^= 1;
@@ -223,7 +261,7 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 203)) return;
                     jr_par[x] ^= 1;
                 }
-                const unsigned n_st = (unsigned)(tl->n_jobs[li] + 1) >> 1;  // stages of this list
+                const unsigned n_st = (unsigned)(tl->n_jobs[li] + S::kTps - 1) / S::kTps;  // stages of this list
                 __syncwarp();
                 if (elect_one()) mbar_arrive(smem_u32(&tl->jobs_ack[li]));  // the count is all this role reads
                 __syncwarp();
@@ -231,6 +269,7 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                 const unsigned s_end = stage_seq + n_st;
                 // this warp's stages of the list: s = which (mod kMmaWarps)
                 for (unsigned s = stage_seq + (((unsigned)which - stage_seq) & (kMmaWarps - 1)); s < s_end; s += kMmaWarps) {
+                    const unsigned sidx = S::kStages == kMmaWarps ? (unsigned)which : s % S::kStages, a_lo = a_lo0 + sidx * (S::kStageBytes >> 4);
                     for (int r = r0; r < r1; r += 2) {
                         // first level: rows r and r + 1 in one chain, each in its slot
                         const bool two = level == 0 && r + 1 < r1;
@@ -247,21 +286,21 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
                         if (two && !mbar_wait_w(smem_u32(&tl->tmem_empty[slot + 1]), ((slot_par >> 1) & 1u) ^ 1u, tl, P.ws, 205)) return;
                         slot_par ^= two ? 3u : 1u << sl;
                         tc_fence_after();
-                        const unsigned d_tmem = tmem_base + slot * 64;
-                        const unsigned b_lo = q_lo + r * (kHalfTile >> 4);
-                        const unsigned idesc = two ? kIdescTwo : kIdesc;
+                        const unsigned d_tmem = tmem_base + slot * S::kBlk;
+                        const unsigned b_lo = q_lo + r * (S::kTile >> 4);
+                        const unsigned idesc = two ? kIdescTwo<S> : kIdesc<S>;
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
+                        for (int c = 0; c < S::kHalves; ++c) {
                             if (r == r0) {
-                                if (!mbar_wait_w(smem_u32(&tl->full[c][sidx]), (s / kStages) & 1u, tl, P.ws, 204)) return;
+                                if (!mbar_wait_w(smem_u32(&tl->full[c][sidx]), (s / S::kStages) & 1u, tl, P.ws, 204)) return;
                                 tc_fence_after();
                             }
                             if (elect_one()) {
 #pragma unroll
                                 for (int k4 = 0; k4 < 4; ++k4)
-                                    tc_mma_bf16_split(d_tmem, a_lo + ((c * 2 * kHalfTile + k4 * 32) >> 4), kDescHi,
-                                                      b_lo + ((c * kR * kHalfTile + k4 * 32) >> 4), kDescHi, idesc, (c | k4) != 0);
-                                if (c == 1) {
+                                    tc_mma_bf16_split(d_tmem, a_lo + ((c * S::kStageHalf + k4 * 32) >> 4), kDescHi,
+                                                      b_lo + ((c * kR * S::kTile + k4 * 32) >> 4), kDescHi, idesc, (c | k4) != 0);
+                                if (c + 1 == S::kHalves) {
                                     tc_commit(smem_u32(&tl->tmem_full[slot]));
                                     if (two) tc_commit(smem_u32(&tl->tmem_full[slot + 1]));
                                     // the stage is free once its last chain has read it (a commit covers
@@ -296,59 +335,66 @@ __device__ void mma_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_
 // then used by one group only, which sees every phase of them. It steps over the other group's
 // chains without looking at them: the bookkeeping of a warp is serial code, and what it spends
 // there it cannot spend reducing.
-__device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int wq, int grp, int lane) {
+template <class S>
+__device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, int wq, int grp, int lane) {
     const Geom &g = P.g;
     unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
     unsigned stage_seq = 0;
     unsigned full_par = 0;  // bit w: phase of the next use of issuing warp w's slot `grp`
-    const int tile = wq >> 1;                // which tile of the pair this warp's lanes hold
-    const int key = (wq & 1) * 32 + lane;    // key index inside the tile
+    constexpr int kBlk = S::kBlk;
+    const int tile = wq / S::kParts;                       // which tile of the stage this warp's lanes hold
+    const int key = (wq % S::kParts) * 32 + lane;          // key index inside the tile
     // of this group's slot of issuing warp 0; the others' follow at 16 bytes (slot 2 * warp + grp)
     const unsigned full_bar = smem_u32(&tl->tmem_full[grp]), empty_bar = smem_u32(&tl->tmem_empty[grp]);
-    const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16) + grp * 64;
+    const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16) + grp * kBlk;
+    const int whole_blocks = (int)(g.T / kBlk);
     for (;;) {
         if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 301)) return;
         const unsigned set = grp_par;
         grp_par ^= 1;
         if (tl->grp_id < 0) return;
-        const int R = tl->grp_R, qb = tl->grp_qb, levels = tl->grp_levels;
-        const long long rem_q = g.T - (long long)qb * kBlk;
-        const int m_lim = rem_q < kBlk ? (int)rem_q : kBlk;  // query tokens of this block inside T
-        const int full_blocks = m_lim == kBlk ? (int)(g.T / kBlk) : 0, diag = g.causal ? qb : -1;  // key blocks without a mask: those before, but for the diagonal one
+        const int R = tl->grp_R, grp_qb = tl->grp_qb, levels = tl->grp_levels;
+        auto qb_of = [&](int r) { return S::kQbRows ? grp_qb - (int)((P.row_back >> (2 * r)) & 3u) : grp_qb; };
         float last = 0.f;  // this lane's maximum of the last tile, and where the tile's goes
         unsigned last_to = smem_u32(&tl->no_part);
         auto put = [&] {
             const float best = warp_max(last);
             asm volatile("{\n.reg .pred p;\nsetp.eq.b32 p, %2, 0;\n@p st.shared.f32 [%0], %1;\n}" ::"r"(last_to), "f"(best), "r"(lane) : "memory");
         };
-        int my_blk = -1;      // lane i: this warp's tile of the list's stage i (-1: there is none, its maximum is not looked at)
-        unsigned masked = 0;  // bit i: that tile is not whole
-        // One chain of this group: the list's stage i, the kernel's stage s, where the maximum goes.
-        auto reduce = [&](unsigned s, unsigned i, unsigned to) -> bool {
+        // Register x of lane i: this warp's tile of the list's stage 32 x + i (-1: there is none, its
+        // maximum is not looked at); bit i of masked[y][x]: that tile is not whole for the y-th of
+        // this group's rows that the list serves.
+        int my_blk[S::kListRegs];
+        unsigned masked[S::kMaskRows][S::kListRegs];
+        // One chain of this group: the list's stage i, the kernel's stage s, row r, the y-th, where the maximum goes.
+        auto reduce = [&](unsigned s, unsigned i, int r, int y, unsigned to) -> bool {
             const unsigned owner = s & (kMmaWarps - 1);
             if (!mbar_wait_w(full_bar + owner * 16, (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
             full_par ^= 1u << owner;
             tc_fence_after();
             float best = -CUDART_INF_F;
-            const unsigned taddr = t_lane + owner * 128;
-            if (((masked >> i) & 1u) == 0) {
-                unsigned v[64];
-                tmem_ld_32x32_issue(taddr, v);
-                tmem_ld_32x32_issue(taddr + 32, v + 32);
+            const unsigned taddr = t_lane + owner * (2 * kBlk);
+            const unsigned m0 = y ? masked[S::kMaskRows - 1][0] : masked[0][0], m1 = y ? masked[S::kMaskRows - 1][S::kListRegs - 1] : masked[0][S::kListRegs - 1];
+            const bool whole = (((S::kListRegs > 1 && i >= 32 ? m1 : m0) >> (i & 31)) & 1u) == 0;
+            if (whole) {
+                unsigned v[kBlk];
+#pragma unroll
+                for (int x = 0; x < S::kParts; ++x) tmem_ld_32x32_issue(taddr + 32 * x, v + 32 * x);
                 put();  // (the tile before this one, while the loads are on their way)
                 tmem_ld_wait();
                 // the slot goes back as soon as it is in registers: its issuing warp waits for it
                 tc_fence_before();
                 mbar_arrive_if(empty_bar + owner * 16, lane == 0);
-                best = max_of_64(reinterpret_cast<const float *>(v));
+                best = max_of<kBlk>(reinterpret_cast<const float *>(v));
             } else {
                 put();
-                const int blk = __shfl_sync(0xffffffffu, my_blk, i);
+                const int blk = __shfl_sync(0xffffffffu, S::kListRegs > 1 && i >= 32 ? my_blk[S::kListRegs - 1] : my_blk[0], i & 31);
                 if (blk >= 0) {  // the diagonal block, or a block across T: rare, so little code rather than little time
                     // allowed queries for this key: inside T, and not before the key if causal
-                    const int lo = key >= (int)g.T - blk * kBlk ? kBlk : (blk == diag ? key : 0);
+                    const int qb = qb_of(r), m_lim = min(kBlk, (int)g.T - qb * kBlk);
+                    const int lo = key >= (int)g.T - blk * kBlk ? kBlk : (g.causal && blk == qb ? key : 0);
 #pragma unroll 1
-                    for (int i0 = 0; i0 < 64; i0 += 8) {
+                    for (int i0 = 0; i0 < kBlk; i0 += 8) {
                         unsigned v[8];
                         tmem_ld_32x8_issue(taddr + i0, v);
                         tmem_ld_wait();
@@ -375,25 +421,38 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
                 // All there is to read of the list, at once: a look at it chain by chain, with the
                 // comparisons, was a good part of what a warp spends on a chain.
                 const int n = tl->n_jobs[li];
-                my_blk = 2 * lane + tile < n ? (level == 0 ? tl->first_blk : tl->jobs_blk[x])[2 * lane + tile] : -1;
-                masked = __ballot_sync(0xffffffffu, my_blk < 0 || my_blk >= full_blocks || my_blk == diag);
+                const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
+#pragma unroll
+                for (int y = 0; y < S::kListRegs; ++y) {
+                    const int at = S::kTps * (32 * y + lane) + tile;
+                    my_blk[y] = at < n ? list[at] : -1;
+                }
+                const int r0 = level == 0 ? grp : x, r1 = level == 0 ? R : x + 1;
+#pragma unroll
+                for (int z = 0; z < S::kMaskRows; ++z) {
+                    if (z > 0 && level > 0) continue;
+                    // key blocks without a mask: those before `whole`, but for the diagonal one
+                    const int qb = qb_of(r0 + 2 * z), whole = qb < whole_blocks ? whole_blocks : 0, diag = g.causal ? qb : -1;
+#pragma unroll
+                    for (int y = 0; y < S::kListRegs; ++y)
+                        masked[z][y] = __ballot_sync(0xffffffffu, my_blk[y] < 0 || my_blk[y] >= whole || my_blk[y] == diag);
+                }
                 mbar_arrive_if(smem_u32(&tl->jobs_ack[li]), lane == 0);
-                const unsigned s_end = stage_seq + ((unsigned)(n + 1) >> 1);
+                const unsigned s_end = stage_seq + (unsigned)(n + S::kTps - 1) / S::kTps;
                 // First level: every stage serves all rows, rows grp, grp + 2 are this group's, and each
                 // issuing warp needs its slot back from the first before it can issue the second: so
                 // the first rows of kMmaWarps stages, then the second ones (stage by stage the group
                 // waited for that round trip with other warps' chains ready: 115 -> 99 us at
                 // T = 4096, 32 / 8 heads, k = 32). Later one chain per stage, this group's are the
                 // stages with (s / kMmaWarps) % 2 == grp.
-                const int r0 = level == 0 ? grp : x, r1 = level == 0 ? R : x + 1;
-                const unsigned part = smem_u32(level == 0 ? tl->first_part[set][0] : tl->part[x]) + tile * 8 + (wq & 1) * 4;
-                const unsigned row_step = level == 0 ? kMaxJobs * 8 : 0;
+                const unsigned part = smem_u32(level == 0 ? tl->first_part[set][0] : tl->part[x]) + wq * 4;  // (four warps: the kTps * kParts parts of a stage in order)
+                const unsigned row_step = level == 0 ? S::kMaxJobs * S::kParts * 4 : 0;
                 for (unsigned base = level == 0 ? stage_seq : stage_seq & ~(unsigned)(kMmaWarps - 1); base < s_end; base += kMmaWarps) {
                     if (level > 0 && (int)((base / kMmaWarps) & 1u) != grp) continue;
                     const unsigned lo = max(base, stage_seq), hi = min(base + kMmaWarps, s_end);
                     for (int r = r0; r < r1; r += 2)
                         for (unsigned s = lo; s < hi; ++s)
-                            if (!reduce(s, s - stage_seq, part + r * row_step + (s - stage_seq) * 16)) return;
+                            if (!reduce(s, s - stage_seq, r, S::kQbRows && r > r0, part + r * row_step + (s - stage_seq) * 16)) return;
                 }
                 stage_seq = s_end;
                 put();
@@ -410,18 +469,29 @@ __device__ void epilogue_role(const Params &P, Tail *tl, unsigned tmem_base, int
 // Dispatcher and controllers ------------------------------------------------------------------------
 // kMulti: several k per group with the score memory; false compiles the plain single-pass form.
 
-// The two candidates of initial node `lane` (the same for every row of a group).
-struct FirstNodes {
+// The two candidates of an initial node (the same for every row of a group).
+struct FirstNode {
     int f, l, m;
     bool vl, vr;
-    __device__ FirstNodes(const Geom &g, int kq, int q_lim, int lane) {
-        f = (int)(((long long)lane * g.N_k) / kq);
-        l = (int)(((long long)(lane + 1) * g.N_k) / kq) - 1;
+    __device__ FirstNode(const Geom &g, int kq, int q_lim, int i) {
+        f = (int)(((long long)i * g.N_k) / kq);
+        l = (int)(((long long)(i + 1) * g.N_k) / kq) - 1;
         m = (f + l) / 2;
-        vl = lane < kq && f <= l && f <= q_lim;
+        vl = i < kq && f <= l && f <= q_lim;
         vr = vl && m + 1 <= l && m + 1 <= q_lim;
     }
 };
+
+// Places of a warp's flags, n of them a lane, in lane order: those before this lane's; all of them.
+template <int n>
+__device__ __forceinline__ int flags_before(const unsigned (&ballots)[n], unsigned lt) {
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) c += __popc(ballots[i] & lt);
+    return c;
+}
+template <int n>
+__device__ __forceinline__ int flags_all(const unsigned (&ballots)[n]) { return flags_before(ballots, 0xffffffffu); }
 
 // Is block blk a first-level candidate of a build with k = kq?
 __device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int blk) {
@@ -430,9 +500,11 @@ __device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int blk) {
     return blk == f || blk == (f + l) / 2 + 1;
 }
 
-template <bool kMulti>
-__device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl, unsigned q_smem, int lane) {
+template <class S>
+__device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> *tl, unsigned q_smem, int lane) {
     const Geom &g = P.g;
+    constexpr bool kMulti = S::kMulti;
+    constexpr int kNodes = S::kNodes;
     const unsigned lt = (1u << lane) - 1u;
     unsigned ack_par = 1, q_par = (1u << kR) - 1u;  // (the first waits pass at once)
     unsigned long long fetched = 0;  // Q tiles asked of TMA
@@ -448,38 +520,47 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl
         if (lane == 0 && id + 2 * (int)gridDim.x < P.n_groups) next = (int)atomicAdd(&P.ws->work_counter, 1u);
         int b = 0, kvh = 0, qb = 0, h0 = 0, R = 0;
         if (!done) {
-            const int per = g.n_qb * P.n_chunks;
+            const int per = (g.n_qb + P.qb_rows - 1) / P.qb_rows * P.n_chunks;
             const int bkv = id / per, rem = id % per;
             b = bkv / g.G; kvh = bkv % g.G;
-            qb = g.n_qb - 1 - rem / P.n_chunks;  // late (expensive) query blocks first
+            qb = g.n_qb - 1 - rem / P.n_chunks * P.qb_rows;  // late (expensive) query blocks first
             const int chunk = rem % P.n_chunks;
-            h0 = kvh * g.hpg + chunk * kR;
-            R = min(kR, g.hpg - chunk * kR);
+            h0 = kvh * g.hpg + chunk * P.head_rows;
+            R = min(P.head_rows, g.hpg - chunk * P.head_rows) * min(P.qb_rows, qb + 1);
         }
         const int q_lim = last_valid_block(g, qb);
         const int n_pass = (!kMulti || done) ? 1 : P.mk.n;
         for (int pass = 0; pass < n_pass; ++pass) {
             const int kq = done ? g.k_top : (kMulti ? P.mk.k[pass] : row_k(g, qb));
-            const FirstNodes fn(g, kq, q_lim, lane);
-            bool on_l = fn.vl && !done, on_r = fn.vr && !done;  // goes on the list
+            bool on[2 * kNodes];  // goes on the list
+            int cand[2 * kNodes];
+            unsigned ballots[2 * kNodes];
+#pragma unroll
+            for (int x = 0; x < kNodes; ++x) {
+                const FirstNode fn(g, kq, q_lim, kNodes * lane + x);
+                cand[2 * x] = fn.f; cand[2 * x + 1] = fn.m + 1;
+                on[2 * x] = fn.vl && !done; on[2 * x + 1] = fn.vr && !done;
+            }
             // Not what an earlier pass has had on its first list: every row has that score. (What rows have
             // met on later levels is for their controllers to know, which may still be at it.)
-            for (int e = 0; kMulti && e < pass; ++e) {
-                on_l = on_l && !on_first_list(g, P.mk.k[e], fn.f);
-                on_r = on_r && !on_first_list(g, P.mk.k[e], fn.m + 1);
-            }
-            const unsigned bl = __ballot_sync(0xffffffffu, on_l), br = __ballot_sync(0xffffffffu, on_r);
-            const int c_l = __popc(bl & lt) + __popc(br & lt), c_r = c_l + (on_l ? 1 : 0);
+            for (int e = 0; kMulti && e < pass; ++e)
+#pragma unroll
+                for (int x = 0; x < 2 * kNodes; ++x) on[x] = on[x] && !on_first_list(g, P.mk.k[e], cand[x]);
+#pragma unroll
+            for (int x = 0; x < 2 * kNodes; ++x) ballots[x] = __ballot_sync(0xffffffffu, on[x]);
+            int place = flags_before(ballots, lt);
             if (pass > 0 && !mbar_wait_w(smem_u32(&tl->jobs_ack[kR]), ack_par, tl, P.ws, 409)) return;
             ack_par ^= 1;
-            if (on_l) tl->first_blk[c_l] = fn.f;
-            if (on_r) tl->first_blk[c_r] = fn.m + 1;
+#pragma unroll
+            for (int x = 0; x < 2 * kNodes; ++x)
+                if (on[x]) tl->first_blk[place++] = cand[x];
             if (lane == 0) {
-                tl->n_jobs[kR] = __popc(bl) + __popc(br);
+                tl->n_jobs[kR] = flags_all(ballots);
                 tl->grp_id = done ? -1 : id; tl->grp_b = b; tl->grp_kvh = kvh; tl->grp_qb = qb; tl->grp_h0 = h0; tl->grp_R = R;
                 tl->grp_levels = row_levels(g, kq);
                 tl->grp_k = kq; tl->grp_pass = pass;
-                tl->grp_left = bl; tl->grp_right = br;
+#pragma unroll
+                for (int x = 0; x < 2 * kNodes; ++x) tl->grp_on[x] = ballots[x];
                 tl->grp_new_q = pass == 0;
                 tl->grp_last = pass + 1 == n_pass;
             }
@@ -495,9 +576,9 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl
                 q_par ^= 1u << r;
                 if (elect_one()) {
                     const unsigned bar = smem_u32(&tl->q_full[r]);
-                    mbar_arrive_expect_tx(bar, (unsigned)(2 * kHalfTile));
+                    mbar_arrive_expect_tx(bar, (unsigned)(S::kHalves * S::kTile));
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) tma_load_4d(q_smem + (c * kR + r) * kHalfTile, tq, bar, c * 64, qb * kBlk, h0 + r, b);
+                    for (int c = 0; c < S::kHalves; ++c) tma_load_4d(q_smem + (c * kR + r) * S::kTile, tq, bar, c * 64, (S::kQbRows ? qb - (int)((P.row_back >> (2 * r)) & 3u) : qb) * S::kBlk, h0 + (S::kQbRows ? (int)((P.row_head >> (2 * r)) & 3u) : r), b);
                 }
                 __syncwarp();
             }
@@ -506,22 +587,33 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail *tl
     }
 }
 
-// Row r of every group.
-template <bool kMulti>
-__device__ void controller_role(const Params &P, Tail *tl, int r, int lane) {
+// Row r of every group. Lane i holds nodes kNodes i .. kNodes i + kNodes - 1 of the row.
+template <class S>
+__device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
     const Geom &g = P.g;
+    constexpr bool kMulti = S::kMulti;
+    constexpr int kNodes = S::kNodes;
     const unsigned lt = (1u << lane) - 1u;
     unsigned grp_par = 0, first_par = 0, sd_par = 0, ack_par = 1;  // first_par: bit by bit for the two sets
     // this CTA's score memory for the row (several k only)
     unsigned long long *const cache = kMulti ? P.cache + ((size_t)blockIdx.x * kR + r) * g.N_k : nullptr;
+    auto remembered = [&](int blk, unsigned tag, float &score) {
+        const unsigned long long e = __ldcg(cache + blk);
+        if ((unsigned)(e >> 32) != tag) return false;
+        score = __uint_as_float((unsigned)e);
+        return true;
+    };
+    auto tile_max = [](const float (&parts)[S::kParts]) { return S::kParts == 2 ? fmaxf(parts[0], parts[S::kParts - 1]) : parts[0]; };
     unsigned long long tiles_all = 0, rows_all = 0;
     for (;;) {
         if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 407)) return;
         const unsigned set = grp_par;
         grp_par ^= 1;
-        const int id = tl->grp_id, b = tl->grp_b, qb = tl->grp_qb, h = tl->grp_h0 + r, R = tl->grp_R, levels = tl->grp_levels;
+        const int id = tl->grp_id, b = tl->grp_b, qb = S::kQbRows ? tl->grp_qb - (int)((P.row_back >> (2 * r)) & 3u) : tl->grp_qb, h = tl->grp_h0 + (S::kQbRows ? (int)((P.row_head >> (2 * r)) & 3u) : r), R = tl->grp_R, levels = tl->grp_levels;
         const int kq = tl->grp_k, pass = tl->grp_pass;
-        const unsigned on_left = tl->grp_left, on_right = tl->grp_right;
+        unsigned on[2 * kNodes];
+#pragma unroll
+        for (int x = 0; x < 2 * kNodes; ++x) on[x] = tl->grp_on[x];
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ack[kR]));  // (the list itself is not needed)
         if (id < 0) {
@@ -534,88 +626,117 @@ __device__ void controller_role(const Params &P, Tail *tl, int r, int lane) {
         if (r >= R) continue;
         const int q_lim = last_valid_block(g, qb);
         const unsigned tag = (unsigned)id + 1u;  // marks this group's entries of the score memory (0 = never written)
-        const FirstNodes fn(g, kq, q_lim, lane);
-        const bool fl1 = (on_left >> lane) & 1u, fr1 = (on_right >> lane) & 1u;
-        const int c_l1 = __popc(on_left & lt) + __popc(on_right & lt), c_r1 = c_l1 + (fl1 ? 1 : 0);
-        bool miss_l = fn.vl, miss_r = fn.vr;  // this row has no score for the candidate yet
-        float cl = -CUDART_INF_F, cr = -CUDART_INF_F;
-        if (kMulti) {
-            if (fn.vl) {
-                const unsigned long long e = __ldcg(cache + fn.f);
-                if ((unsigned)(e >> 32) == tag) { cl = __uint_as_float((unsigned)e); miss_l = false; }
+        // A level's candidates, in ascending order: left and right of every node. cand: what they keep if
+        // they survive (first and last block, score); have: it is there.
+        int nf[kNodes], nl[kNodes];       // this lane's nodes
+        float ns[kNodes];
+        bool has[2 * kNodes];
+        float sc[2 * kNodes];
+        unsigned tiles = 0;               // (row, block) tiles that had no score yet
+#pragma unroll
+        for (int x = 0; x < kNodes; ++x) {
+            const FirstNode fn(g, kq, q_lim, kNodes * lane + x);
+            nf[x] = fn.f; nl[x] = fn.l;
+            has[2 * x] = fn.vl; has[2 * x + 1] = fn.vr;
+            bool miss_l = fn.vl, miss_r = fn.vr;
+            sc[2 * x] = sc[2 * x + 1] = -CUDART_INF_F;
+            if (kMulti) {
+                if (fn.vl && remembered(fn.f, tag, sc[2 * x])) miss_l = false;
+                if (fn.vr && remembered(fn.m + 1, tag, sc[2 * x + 1])) miss_r = false;
             }
-            if (fn.vr) {
-                const unsigned long long e = __ldcg(cache + fn.m + 1);
-                if ((unsigned)(e >> 32) == tag) { cr = __uint_as_float((unsigned)e); miss_r = false; }
-            }
+            tiles += (unsigned)(__popc(__ballot_sync(0xffffffffu, miss_l)) + __popc(__ballot_sync(0xffffffffu, miss_r)));
         }
-        // (row, block) tiles that had no score yet
-        unsigned tiles = (unsigned)(__popc(__ballot_sync(0xffffffffu, miss_l)) + __popc(__ballot_sync(0xffffffffu, miss_r)));
-        int nf = 0, nl = -1, my_c = 0, n_nodes = 0, rb = 0;
-        float ns = -CUDART_INF_F, cs = 0.f;
-        bool has_r = false, need = false;
+        bool need[kNodes];                // the right candidate's score comes from the list
+        int my_c[kNodes], n_nodes = 0;
         for (int level = 0; level < levels; ++level) {
-            // candidates of this lane's node: left (f : m) and right (m + 1 : l)
-            int f, l, m;
-            bool vl, vr;
-            float sl = -CUDART_INF_F, sr = -CUDART_INF_F;
             if (level == 0) {
                 if (!mbar_wait_w(smem_u32(&tl->first_done[set][r]), (first_par >> set) & 1u, tl, P.ws, 408)) return;
                 first_par ^= 1u << set;
-                f = fn.f; l = fn.l; m = fn.m; vl = fn.vl; vr = fn.vr;
-                if (vl) sl = fl1 ? fmaxf(tl->first_part[set][r][c_l1][0], tl->first_part[set][r][c_l1][1]) : cl;
-                if (vr) sr = fr1 ? fmaxf(tl->first_part[set][r][c_r1][0], tl->first_part[set][r][c_r1][1]) : cr;
-                if (kMulti) {
-                    if (fl1) __stcg(cache + f, cache_pack(tag, sl));
-                    if (fr1) __stcg(cache + m + 1, cache_pack(tag, sr));
+                int place = flags_before(on, lt);
+#pragma unroll
+                for (int x = 0; x < 2 * kNodes; ++x) {
+                    if (!((on[x] >> lane) & 1u)) continue;
+                    sc[x] = tile_max(tl->first_part[set][r][place++]);
+                    if (kMulti) __stcg(cache + ((x & 1) ? (nf[x >> 1] + nl[x >> 1]) / 2 + 1 : nf[x >> 1]), cache_pack(tag, sc[x]));
                 }
             } else {
                 if (!mbar_wait_w(smem_u32(&tl->scores_done[r]), sd_par, tl, P.ws, 401)) return;
                 sd_par ^= 1;
-                f = nf; l = nl; m = (f + l) / 2;
-                vl = lane < n_nodes; vr = has_r;
-                sl = ns;
-                if (vr) sr = need ? fmaxf(tl->part[r][my_c][0], tl->part[r][my_c][1]) : cs;
-                if (kMulti && need) __stcg(cache + rb, cache_pack(tag, sr));
+#pragma unroll
+                for (int x = 0; x < kNodes; ++x) {
+                    has[2 * x] = kNodes * lane + x < n_nodes;
+                    sc[2 * x] = ns[x];
+                    if (need[x]) {
+                        sc[2 * x + 1] = tile_max(tl->part[r][my_c[x]]);
+                        if (kMulti) __stcg(cache + (nf[x] + nl[x]) / 2 + 1, cache_pack(tag, sc[2 * x + 1]));
+                    }
+                }
             }
-            const Keep kp = select_topk(vl, sl, vr, sr, kq, lane);
-            const unsigned kl = __ballot_sync(0xffffffffu, kp.l), kr = __ballot_sync(0xffffffffu, kp.r);
-            const int pos_l = __popc(kl & lt) + __popc(kr & lt), pos_r = pos_l + (kp.l ? 1 : 0);
+            bool keep[2 * kNodes];
+            if constexpr (kNodes == 1) {
+                const Keep kp = select_topk(has[0], sc[0], has[1], sc[1], kq, lane);
+                keep[0] = kp.l; keep[1] = kp.r;
+            } else {
+                select_topk_of<2 * kNodes>(has, sc, kq, lane, keep);
+            }
+            unsigned kept[2 * kNodes];
+#pragma unroll
+            for (int x = 0; x < 2 * kNodes; ++x) kept[x] = __ballot_sync(0xffffffffu, keep[x]);
+            int place = flags_before(kept, lt);
             __syncwarp();
-            if (kp.l) { tl->node_f[r][pos_l] = f; tl->node_l[r][pos_l] = m; tl->node_s[r][pos_l] = sl; }
-            if (kp.r) { tl->node_f[r][pos_r] = m + 1; tl->node_l[r][pos_r] = l; tl->node_s[r][pos_r] = sr; }
+#pragma unroll
+            for (int x = 0; x < 2 * kNodes; ++x) {
+                if (!keep[x]) continue;
+                const int f = nf[x >> 1], l = nl[x >> 1], m = (f + l) / 2;
+                tl->node_f[r][place] = (x & 1) ? m + 1 : f;
+                tl->node_l[r][place] = (x & 1) ? l : m;
+                tl->node_s[r][place] = sc[x];
+                ++place;
+            }
             __syncwarp();
-            n_nodes = __popc(kl) + __popc(kr);
-            const bool live = lane < n_nodes;
-            nf = live ? tl->node_f[r][lane] : 0;
-            nl = live ? tl->node_l[r][lane] : -1;
-            ns = live ? tl->node_s[r][lane] : -CUDART_INF_F;
+            n_nodes = flags_all(kept);
+#pragma unroll
+            for (int x = 0; x < kNodes; ++x) {
+                const bool live = kNodes * lane + x < n_nodes;
+                nf[x] = live ? tl->node_f[r][kNodes * lane + x] : 0;
+                nl[x] = live ? tl->node_l[r][kNodes * lane + x] : -1;
+                ns[x] = live ? tl->node_s[r][kNodes * lane + x] : -CUDART_INF_F;
+            }
             if (level + 1 < levels) {
                 // next level: only right branches need a tile; left ones keep the node's score
-                const int mm = (nf + nl) / 2;
-                has_r = live && nl > nf && mm + 1 <= q_lim;
-                rb = mm + 1;
-                need = has_r;
-                if (kMulti && has_r) {  // an earlier pass (another k) may have scored it
-                    const unsigned long long e = __ldcg(cache + rb);
-                    if ((unsigned)(e >> 32) == tag) { cs = __uint_as_float((unsigned)e); need = false; }
+                unsigned due[kNodes];
+#pragma unroll
+                for (int x = 0; x < kNodes; ++x) {
+                    const int rb = (nf[x] + nl[x]) / 2 + 1;
+                    has[2 * x + 1] = kNodes * lane + x < n_nodes && nl[x] > nf[x] && rb <= q_lim;
+                    sc[2 * x + 1] = -CUDART_INF_F;
+                    need[x] = has[2 * x + 1];
+                    if (kMulti && need[x] && remembered(rb, tag, sc[2 * x + 1])) need[x] = false;  // an earlier pass (another k) has scored it
+                    due[x] = __ballot_sync(0xffffffffu, need[x]);
                 }
-                const unsigned hb = __ballot_sync(0xffffffffu, need);
-                my_c = __popc(hb & lt);
                 if (!mbar_wait_w(smem_u32(&tl->jobs_ack[r]), ack_par, tl, P.ws, 403)) return;
                 ack_par ^= 1;
-                if (need) tl->jobs_blk[r][my_c] = rb;
-                if (lane == 0) tl->n_jobs[r] = __popc(hb);
-                tiles += (unsigned)__popc(hb);
+                int at = flags_before(due, lt);
+#pragma unroll
+                for (int x = 0; x < kNodes; ++x) {
+                    my_c[x] = at;
+                    if (need[x]) tl->jobs_blk[r][at++] = (nf[x] + nl[x]) / 2 + 1;
+                }
+                if (lane == 0) tl->n_jobs[r] = flags_all(due);
+                tiles += (unsigned)flags_all(due);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[r]));
             } else {
                 // emit I[q, :]: first block of every surviving node, ascending, -1 padded
                 const long long row = ((long long)b * g.H + h) * g.n_qb + qb;
                 const long long o = (long long)pass * P.slab + row * g.k_top;
-                if (lane < g.k_top) {
-                    P.mask[o + lane] = live ? nf : -1;
-                    if (P.score != nullptr) P.score[o + lane] = live ? ns : -CUDART_INF_F;
+#pragma unroll
+                for (int x = 0; x < kNodes; ++x) {
+                    const int i = kNodes * lane + x;
+                    if (i < g.k_top) {
+                        P.mask[o + i] = i < n_nodes ? nf[x] : -1;
+                        if (P.score != nullptr) P.score[o + i] = i < n_nodes ? ns[x] : -CUDART_INF_F;
+                    }
                 }
                 if (!kMulti && g.row_tiles != nullptr && lane == 0) g.row_tiles[row] = tiles;
             }
@@ -625,17 +746,20 @@ __device__ void controller_role(const Params &P, Tail *tl, int r, int lane) {
     }
 }
 
-template <bool kMulti>
+template <class S>
 __global__ void __launch_bounds__(kThreads, 1)
 mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, Params P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = aligned_smem(smem_raw);
-    const unsigned q_smem = smem_u32(smem), k_smem = q_smem + kQBytes;
-    Tail *tl = (Tail *)(smem + kQBytes + kStages * kStageBytes);
+    const unsigned q_smem = smem_u32(smem), k_smem = q_smem + S::kQBytes;
+    Tail<S> *tl = (Tail<S> *)(smem + S::kQBytes + S::kStages * S::kStageBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStages; ++i) { mbar_init(smem_u32(&tl->full[0][i]), 1); mbar_init(smem_u32(&tl->full[1][i]), 1); mbar_init(smem_u32(&tl->empty[i]), 1); }
+        for (int i = 0; i < S::kStages; ++i) {
+            for (int c = 0; c < S::kHalves; ++c) mbar_init(smem_u32(&tl->full[c][i]), 1);
+            mbar_init(smem_u32(&tl->empty[i]), 1);
+        }
         for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&tl->tmem_full[i]), 1); mbar_init(smem_u32(&tl->tmem_empty[i]), 4); }
         for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), kListReaders + (i == kR ? kR : 0)); }
         for (int i = 0; i < kR; ++i) {
@@ -665,9 +789,9 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     } else if (warp == 2 || warp == 14) {
         producer_role(P, &tmap_k, tl, k_smem, warp == 2 ? 0 : 1);
     } else if (warp == 18) {
-        dispatcher_role<kMulti>(P, &tmap_q, tl, q_smem, lane);
+        dispatcher_role(P, &tmap_q, tl, q_smem, lane);
     } else {
-        controller_role<kMulti>(P, tl, warp == 0 ? 0 : (warp == 12 ? 1 : (warp == 16 ? 2 : 3)), lane);
+        controller_role(P, tl, warp == 0 ? 0 : (warp == 12 ? 1 : (warp == 16 ? 2 : 3)), lane);
     }
     __syncwarp();
 
@@ -691,26 +815,64 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
 }  // namespace
 
 bool mask_tc_supported(const Geom &g, int dtype) {
-    return dtype == STREAM_BF16 && g.d == kD && g.bq == kBlk && g.bk == kBlk && g.k_top <= 32 && g.levels >= 1 &&
-           tma_strides_ok(g);
+    return g.d == 128 && g.bq == 64 && g.k_top <= 32 && mask_tc_auto(g, dtype);
+}
+
+// Against the mma.sync kernel, us: 12 heads, 10007 tokens, d = 128, blocks of 32, k = 8: 221 -> 147; d = 64,
+// blocks of 64, k = 40 (above): 409 -> 156; 8 heads, 13232 tokens, k = 59: 880 -> 265; 12 heads, 558 tokens,
+// k = 59: 16.4 -> 14.6. (28 heads, 1329 tokens, d = 64, blocks of 32, k = 19: 28.7 -> 32.7, the one
+// shape of 26 drawn that lost.)
+bool mask_tc_auto(const Geom &g, int dtype) {
+    return dtype == STREAM_BF16 && (g.d == 64 || g.d == 128) && (g.bq == 32 || g.bq == 64) && g.bk == g.bq && g.k_top <= 64 &&
+           g.levels >= 1 && tma_strides_ok(g);
 }
 
 namespace {
-// CTAs of a launch and the groups they share.
-stream_status launch_shape(const Geom &g, int *grid, long long *n_groups) {
+// CTAs of a launch, the groups they share and the rows of a group: four rows where there are enough
+// groups, since they share the key tiles of the first level and its chains of two rows, else fewer.
+// Two groups a CTA are enough up to k = 32 (7 query heads per kv head, 3419 tokens, k = 27, not causal:
+// four rows 61 us, two 83), three beyond, where a group is a long piece of work (4 heads per kv head,
+// 10502 tokens, d = 64, k = 50: four rows 182 us, two 126; 2713 tokens, d = 128, k = 45: 67 and 54). With
+// fewer than four heads per kv head the rows are neighbouring query blocks' (16 heads, each its
+// own keys, 8192 tokens, d = 64, k = 40, not causal: a row a group 229 us, four 156), unless k changes
+// from one to the next.
+struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
+stream_status split_rows(const Geom &g, Split *s) {
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    *n_groups = (long long)g.batch * g.G * g.n_qb * ((g.hpg + kR - 1) / kR);
-    *grid = (int)(*n_groups < n_sm ? *n_groups : n_sm);
+    s->head_rows = g.hpg < kR ? g.hpg : kR;
+    s->qb_rows = g.k_row == nullptr ? kR / g.hpg : 1;
+    if (s->qb_rows < 1) s->qb_rows = 1;
+    for (;;) {
+        s->n_chunks = (g.hpg + s->head_rows - 1) / s->head_rows;
+        s->n_groups = (long long)g.batch * g.G * ((g.n_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
+        if (s->n_groups >= (g.k_top > 32 ? 3 : 2) * n_sm || s->head_rows * s->qb_rows == 1) break;
+        if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
+        else s->head_rows = (s->head_rows + 1) / 2;
+    }
+    s->grid = (int)(s->n_groups < n_sm ? s->n_groups : n_sm);
     return STREAM_OK;
+}
+
+template <class S>
+cudaError_t launch(int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
+    static_assert(kSmemBytes<S> <= 232448, "one CTA's shared memory");
+    const cudaError_t e = cudaFuncSetAttribute(mask_tc_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<S>);
+    if (e == cudaSuccess) mask_tc_kernel<S><<<grid, kThreads, kSmemBytes<S>, st>>>(tq, tk, P);
+    return e;
+}
+
+template <int kD, int kBlk>
+cudaError_t launch_rows(const Geom &g, const Split &sp, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
+    if (g.k_top > 32) return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, true, false, true>>(sp.grid, st, tq, tk, P) : launch<Shape<kD, kBlk, true, false>>(sp.grid, st, tq, tk, P);
+    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, false, false, true>>(sp.grid, st, tq, tk, P) : launch<Shape<kD, kBlk, false, false>>(sp.grid, st, tq, tk, P);
 }
 }  // namespace
 
 size_t mask_tc_score_memory_bytes(const Geom &g) {
-    int grid = 0;
-    long long n_groups = 0;
-    if (launch_shape(g, &grid, &n_groups) != STREAM_OK) return 0;
-    return (size_t)grid * kR * (size_t)g.N_k * sizeof(unsigned long long);
+    Split sp;
+    if (split_rows(g, &sp) != STREAM_OK) return 0;
+    return (size_t)sp.grid * kR * (size_t)g.N_k * sizeof(unsigned long long);
 }
 
 stream_status launch_mask_tc(const Geom &g, const void *q, const void *k, int32_t *mask, float *score,
@@ -726,32 +888,37 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
         return STREAM_ERR_UNSUPPORTED;
     }
     CUtensorMap tq, tk;
-    stream_status rc = make_map_bf16_d128(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q");
+    stream_status rc = make_map_bf16(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q", g.bq, g.d);
     if (rc != STREAM_OK) return rc;
-    rc = make_map_bf16_d128(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k");
+    rc = make_map_bf16(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k", g.bk, g.d);
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;
-    P.n_chunks = (g.hpg + kR - 1) / kR;
-    long long n_groups = (long long)g.batch * g.G * g.n_qb * P.n_chunks;
-    P.n_groups = (int)n_groups;
+    Split sp;
+    rc = split_rows(g, &sp);
+    if (rc != STREAM_OK) return rc;
+    P.n_groups = (int)sp.n_groups;
+    P.n_chunks = sp.n_chunks; P.head_rows = sp.head_rows; P.qb_rows = sp.qb_rows;
+    P.row_head = P.row_back = 0;
+    for (int r = 0; r < sp.head_rows * sp.qb_rows; ++r) {
+        P.row_head |= (unsigned)(r % sp.head_rows) << (2 * r);
+        P.row_back |= (unsigned)(r / sp.head_rows) << (2 * r);
+    }
+    const int grid = sp.grid;
     P.mask = mask; P.score = score; P.ws = ws;
     P.mk = mk;
     P.cache = (unsigned long long *)score_memory;
     P.slab = (long long)g.batch * g.H * g.n_qb * g.k_top;
-    int grid = 0;
-    rc = launch_shape(g, &grid, &n_groups);
-    if (rc != STREAM_OK) return rc;
     cudaError_t e = cudaSuccess;
     if (score_memory != nullptr) {  // tag 0 = "no score yet"
         e = cudaMemsetAsync(score_memory, 0, mask_tc_score_memory_bytes(g), st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(score memory)");
     }
     if (mk.n >= 1 && score_memory == nullptr) { set_error("several k in one launch need the score memory"); return STREAM_ERR_WORKSPACE; }
-    auto kern = mk.n >= 1 ? mask_tc_kernel<true> : mask_tc_kernel<false>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (mk.n >= 1) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, true>>(grid, st, tq, tk, P);
+    else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64>(g, sp, st, tq, tk, P) : launch_rows<128, 32>(g, sp, st, tq, tk, P);
+    else e = g.bq == 64 ? launch_rows<64, 64>(g, sp, st, tq, tk, P) : launch_rows<64, 32>(g, sp, st, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tc)");
-    kern<<<grid, kThreads, kSmemBytes, st>>>(tq, tk, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "mask_tc launch");
     return STREAM_OK;

@@ -290,6 +290,26 @@ __device__ __forceinline__ float max_of_64(const float *v) {
     return fmaxf(fmaxf(b0, b1), fmaxf(b2, b3));
 }
 
+template <int n>
+__device__ __forceinline__ float max_of(const float *v) {
+    static_assert(n == 64 || n == 32, "what the kernels read at a time");
+    if constexpr (n == 64) {
+        return max_of_64(v);
+    } else {
+        float b0 = max3(v[0], v[1], v[2]), b1 = max3(v[3], v[4], v[5]), b2 = max3(v[6], v[7], v[8]), b3 = max3(v[9], v[10], v[11]);
+#pragma unroll
+        for (int i = 12; i < 28; i += 8) {
+            b0 = max3(b0, v[i], v[i + 1]);
+            b1 = max3(b1, v[i + 2], v[i + 3]);
+            b2 = max3(b2, v[i + 4], v[i + 5]);
+            b3 = max3(b3, v[i + 6], v[i + 7]);
+        }
+        b0 = max3(b0, v[28], v[29]);
+        b1 = max3(b1, v[30], v[31]);
+        return fmaxf(fmaxf(b0, b1), fmaxf(b2, b3));
+    }
+}
+
 __device__ __forceinline__ float warp_max(float x) {
     float r;
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
@@ -361,6 +381,47 @@ __device__ __forceinline__ Keep select_topk(bool vl, float sl, bool vr, float sr
     return {vl && (gl || (el && pos_l < missing)), vr && (gr || (er && pos_r < missing))};
 }
 
+// The same for n candidates a lane, numbered n * lane + i: the largest threshold that at least k keys
+// reach, bit by bit from the top (it is the k-th largest key), or earlier if exactly k reach it.
+template <int n>
+__device__ __forceinline__ void select_topk_of(const bool (&have)[n], const float (&score)[n], int k, int lane, bool (&keep)[n]) {
+    unsigned key[n], b[n];
+    int total = 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        key[i] = score_key(have[i], score[i]);
+        total += __popc(__ballot_sync(0xffffffffu, have[i]));
+        keep[i] = have[i];
+    }
+    if (total <= k) return;
+    unsigned thr = 0;
+    int above = total;
+#pragma unroll 1
+    for (unsigned bit = 0x80000000u; bit != 0 && above != k; bit >>= 1) {
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) c += __popc(__ballot_sync(0xffffffffu, key[i] >= (thr | bit)));
+        if (c >= k) { thr |= bit; above = c; }
+    }
+    int missing = k;
+#pragma unroll
+    for (int i = 0; i < n; ++i) missing -= __popc(__ballot_sync(0xffffffffu, key[i] > thr));
+    int place = 0;
+    const unsigned lt = (1u << lane) - 1u;
+    if (above == k) missing = 32 * n;  // all that reach it
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        b[i] = __ballot_sync(0xffffffffu, have[i] && key[i] == thr);
+        place += __popc(b[i] & lt);
+    }
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+        const bool equal = have[i] && key[i] == thr;
+        keep[i] = have[i] && (key[i] > thr || (equal && place < missing));
+        place += equal ? 1 : 0;
+    }
+}
+
 struct Ring {  // position in a ring of barriers with phase tracking
     int idx = 0;
     unsigned phase = 0;
@@ -388,16 +449,16 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// [batch, heads, T, 128] bf16 with element strides -> 4-D map with a box of 64 channels x box_rows
-// tokens (64 unless told otherwise), 128-byte swizzle. Rows beyond T read as zeros.
-inline stream_status make_map_bf16_d128(CUtensorMap *map, const void *base, long long T, int heads, int batch,
-                                        long long s_t, long long s_h, long long s_b, const char *what, int box_rows = 64) {
+// [batch, heads, T, d] bf16 with element strides -> 4-D map with a box of 64 channels x box_rows
+// tokens, 128-byte swizzle. Rows beyond T read as zeros.
+inline stream_status make_map_bf16(CUtensorMap *map, const void *base, long long T, int heads, int batch,
+                                   long long s_t, long long s_h, long long s_b, const char *what, int box_rows, int d) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return STREAM_ERR_CUDA; }
     // extents of 1 may come with arbitrary strides: give them a well-formed one
     if (heads == 1) s_h = s_t * T;
     if (batch == 1) s_b = s_h * heads;
-    cuuint64_t dims[4] = {128, (cuuint64_t)T, (cuuint64_t)heads, (cuuint64_t)batch};
+    cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)heads, (cuuint64_t)batch};
     cuuint64_t strides[3] = {(cuuint64_t)s_t * 2, (cuuint64_t)s_h * 2, (cuuint64_t)s_b * 2};
     cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1}, estr[4] = {1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
@@ -405,6 +466,11 @@ inline stream_status make_map_bf16_d128(CUtensorMap *map, const void *base, long
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled(%s) failed with %d", what, (int)r); return STREAM_ERR_CUDA; }
     return STREAM_OK;
+}
+
+inline stream_status make_map_bf16_d128(CUtensorMap *map, const void *base, long long T, int heads, int batch,
+                                        long long s_t, long long s_h, long long s_b, const char *what, int box_rows = 64) {
+    return make_map_bf16(map, base, T, heads, batch, s_t, s_h, s_b, what, box_rows, 128);
 }
 
 // The same tensor seen as [batch, heads, 2 channel halves, T, 64]: one box brings a whole

@@ -9,7 +9,7 @@ import torch
 from helpers import compare_masks, oracle_problem
 from oracle import stream_oracle as so
 from paper_2510_19875_b200 import workloads as wl
-from test_gpu_parity import S  # noqa: F401  (fixture)
+from test_gpu_parity import S, assert_mask_parity  # noqa: F401  (S: fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -113,3 +113,20 @@ def test_attention_with_logits_far_from_the_reference(S, bq, shift, scale):
         lo, hi = qb * bq, min(spec.T, qb * bq + bq)
         want = ref[rid, : hi - lo]
         assert (np.abs(out[bh, lo:hi] - want) <= few + np.abs(want) / 256).all(), rid
+
+
+@pytest.mark.parametrize("kw,causal", [
+    (dict(d=64, T=2100, block=64, k_top=33), True),                                       # two nodes a lane, one more than one would hold
+    (dict(T=4500, k_top=64, n_q_heads=7, n_kv_heads=1), False),                           # the most; N_k just above k; 4 + 3 heads or fewer
+    (dict(d=64, T=9000, block=32, k_top=64, n_q_heads=2, n_kv_heads=1), True),            # four tiles a stage, lists of up to 128
+    (dict(block=32, T=6001, k_top=9, n_q_heads=3, n_kv_heads=3, batch=2), True),          # query blocks as rows, their number no multiple
+    (dict(d=64, block=64, T=40000, k_top=3, n_q_heads=4, n_kv_heads=2), True),            # two heads at two query blocks, many levels
+    (dict(T=40001, k_top=32, n_q_heads=3, n_kv_heads=3, local=True), False),
+    (dict(d=64, block=32, T=97, k_top=64), True),                                         # k beyond the number of blocks
+])
+def test_masks_on_tcgen05_beyond_four_heads_and_32_blocks(S, kw, causal):
+    base = dict(name="w", seed=6, batch=1, n_q_heads=4, n_kv_heads=1, T=700, d=128, block=64, k_top=5, dtype="bf16")
+    spec = wl.WorkloadSpec(**{**base, **kw})
+    w = wl.generate(spec)
+    rows = None if spec.n_rows <= 600 else np.unique(np.random.default_rng(1).choice(spec.n_rows, 500, replace=False))
+    assert_mask_parity(S, w, rows, score_cache=False, causal=causal)
