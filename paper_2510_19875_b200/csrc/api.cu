@@ -295,6 +295,8 @@ stream_status stream_sparse_attention(const stream_problem *p, const void *q, co
         return STREAM_ERR_UNSUPPORTED;
     }
     if (tc_ok && p->impl != STREAM_IMPL_GENERIC) return launch_attn_tc(g, q, k, v, mask, scale, out, st);
+    if (p->impl == STREAM_IMPL_AUTO && attn_tc_auto(g, p->dtype) && (((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)out) & 15) == 0)
+        return launch_attn_tc(g, q, k, v, mask, scale, out, st);
     if (p->impl == STREAM_IMPL_AUTO && attn_tok_supported(g, p->dtype, q, k, v, out)) return launch_attn_tok(g, q, k, v, mask, scale, out, st);
     if (p->impl == STREAM_IMPL_AUTO && attn_mma_supported(g, p->dtype, q, k, v, out)) return launch_attn_mma(g, q, k, v, mask, scale, out, st);
     return launch_attn_generic(g, p->dtype, q, k, v, mask, scale, out, st);

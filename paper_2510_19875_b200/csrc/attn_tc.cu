@@ -61,14 +61,28 @@ namespace {
 using namespace tc;
 
 constexpr int kThreads = 384;
-constexpr int kBlk = 64, kD = 128;
+constexpr int kBlk = 64;
 constexpr int kHalfTile = kBlk * 128;       // 64 rows x 128 bytes
-constexpr int kTile = 2 * kHalfTile;        // one 64 x 128 tile
-constexpr int kOperand = 2 * kTile;         // two tiles: an entry's K or V, or the Q of a pair
-// Stages of the two rings, out of the operand buffers shared memory has room for beside Q: five (a V
-// stage is held from its load until the product of its entry is complete, a whole softmax later:
-// V three, K two), or four when the mask rows are long.
-constexpr int kMaxKStages = 2, kMaxVStages = 3;
+// d = 128: P goes into the product as bf16. d = 64: as a sum of two bf16, whose rounding is below
+// that of the fp32 sums (what the kernels for the other shapes give, too).
+template <int kD_>
+struct Form {
+    static constexpr int kD = kD_, kHalves = kD / 64;
+    static constexpr bool kSplit = kD == 64;
+    static constexpr int kTile = kHalves * kHalfTile;  // one 64 x d tile
+    static constexpr int kOperand = 2 * kTile;         // two tiles: an entry's K or V, or the Q of a pair
+    // Stages of the two rings, out of the operand buffers shared memory has room for beside Q. d = 128: five (a V
+    // stage is held from its load until the product of its entry is complete, a whole softmax later:
+    // V three, K two), or four when the mask rows are long.
+    static constexpr int kMaxKStages = kD == 128 ? 2 : 6, kMaxVStages = kD == 128 ? 3 : 6;
+    // TMEM columns: the two logit buffers of group g at 128 g and 64 behind, its P at 256 + 64 g (two
+    // buffers, the second 32 behind, or the two parts of one), O at 384.
+    static constexpr int kPBufs = kSplit ? 1 : 2;
+    static constexpr int kPCol = 256, kOCol = 384;
+    static constexpr int kOutBytes = kD;               // of an output token that one group stores (half of the channels)
+    static constexpr unsigned kIdescQK = idesc_bf16(64, 64, false);  // B = a K tile, K-major
+    static constexpr unsigned kIdescPV = idesc_bf16(64, kD, true);   // B = a V tile, MN-major
+};
 constexpr int kMaskSlots = 2;               // pairs whose mask rows are resident
 constexpr int kMaxKTopTc = 1024;
 constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while pairs of several heads are walked
@@ -81,12 +95,10 @@ struct Item {
     int h[2], qb[2];
 };
 
-// TMEM columns: the two logit buffers of group g at 128 g and 64 behind, its two P buffers at 256 + 64 g
-// and 32 behind, O at 384.
-constexpr int kPCol = 256, kOCol = 384;
+template <class F>
 struct Tail {
     unsigned long long q_full[2], q_free[2];  // q_free: the output staged over the pair's Q has left (8 warps)
-    unsigned long long k_full[kMaxKStages], k_empty[kMaxKStages], v_full[kMaxVStages], v_empty[kMaxVStages];
+    unsigned long long k_full[F::kMaxKStages], k_empty[F::kMaxKStages], v_full[F::kMaxVStages], v_empty[F::kMaxVStages];
     unsigned long long s_full[2][2], s_free[2][2];        // per group and logit buffer: ready / read
     unsigned long long p_full[2][2], p_free[2][2];        // per group and P buffer: published / product added
     unsigned long long o_done, o_free;     // a pair's last product is complete; its O has been read (8 warps)
@@ -106,8 +118,6 @@ struct Tail {
 constexpr int kFixedOperands = 2;  // Q; behind it the V stages, then the K stages
 constexpr int kMaxSmemPerCta = 232448;
 
-constexpr unsigned kIdescQK = idesc_bf16(64, 64, false);  // B = a K tile, K-major
-constexpr unsigned kIdescPV = idesc_bf16(64, 128, true);  // B = a V tile, MN-major
 constexpr unsigned kRowLanes = 16u << 16;  // row 1's accumulator and P: the upper half of every 32 lanes
 constexpr unsigned kHiK = desc_hi_sw128(1024);              // every operand: 8-row (8-key) groups 1024 bytes apart
 
@@ -123,17 +133,20 @@ struct Params {
     float scale_log2;      // logit scale times log2(e)
 };
 
-__device__ __forceinline__ bool wait(unsigned bar, unsigned parity, Tail *tl, unsigned code) {
+template <class F>
+__device__ __forceinline__ bool wait(unsigned bar, unsigned parity, Tail<F> *tl, unsigned code) {
     return mbar_wait_bounded(bar, parity, &tl->abort_flag, &g_attn_status[0], &g_attn_status[1], code);
 }
 
 // The same for a whole converged warp (all lanes get the same answer).
-__device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail *tl, unsigned code) {
+template <class F>
+__device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail<F> *tl, unsigned code) {
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &g_attn_status[0], &g_attn_status[1], code);
 }
 
 // Shared copy of the mask rows of the pair in slot `slot`: [2][row_stride] ints behind the Tail.
-__device__ __forceinline__ int *mask_rows(Tail *tl, const Params &P, int slot) {
+template <class F>
+__device__ __forceinline__ int *mask_rows(Tail<F> *tl, const Params &P, int slot) {
     return reinterpret_cast<int *>(tl + 1) + slot * 2 * P.row_stride;
 }
 
@@ -208,7 +221,8 @@ __device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
 }
 
 // Opens the stream's pair (its mask rows must be resident) or closes it; true if it did.
-__device__ __forceinline__ bool open_pair(const Params &P, Tail *tl, LoadStream &S) {
+template <class F>
+__device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStream &S) {
     if (!probe_w(smem_u32(&tl->m_full[S.ms.idx]), S.ms.phase)) return false;
     S.b = tl->m_item[S.ms.idx].b;
     S.kvh = tl->m_item[S.ms.idx].kvh;
@@ -217,19 +231,22 @@ __device__ __forceinline__ bool open_pair(const Params &P, Tail *tl, LoadStream 
     if (S.n > 0) S.cur = entry_at(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
     return true;
 }
-__device__ __forceinline__ void close_pair(const Params &P, Tail *tl, LoadStream &S) {
+template <class F>
+__device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStream &S) {
     if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
     __syncwarp();
     S.ms.advance(kMaskSlots);
     S.id = nth_item(P, ++S.round);
     S.e = -2;
 }
-__device__ __forceinline__ void next_entry(const Params &P, Tail *tl, LoadStream &S) {
+template <class F>
+__device__ __forceinline__ void next_entry(const Params &P, Tail<F> *tl, LoadStream &S) {
     if (++S.e < S.n) S.cur = entry_at(mask_rows(tl, P, S.ms.idx), P.row_stride, S.e);
 }
 
 // After a step that could not move: false if the CTA is aborting or nothing has moved for too long.
-__device__ __forceinline__ bool idle_ok(Tail *tl, long long t_last, unsigned code) {
+template <class F>
+__device__ __forceinline__ bool idle_ok(Tail<F> *tl, long long t_last, unsigned code) {
     int stop = 0;
     if ((threadIdx.x & 31) == 0) {  // lane 0 decides for the warp
         if (*(volatile int *)&tl->abort_flag) stop = 1;
@@ -244,7 +261,8 @@ __device__ __forceinline__ bool idle_ok(Tail *tl, long long t_last, unsigned cod
     return true;
 }
 
-__device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, Tail *tl, unsigned q_smem,
+template <class F>
+__device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, Tail<F> *tl, unsigned q_smem,
                                 unsigned k_smem) {
     LoadStream S;
     S.round = 0;
@@ -257,11 +275,11 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
         if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
         if (elect_one()) {
             // [half][tile][64 rows][128 B]; a row without a block at an entry gets block 0, its logits are masked out
-            const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * kOperand;
+            const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * F::kOperand;
             const int ba = max(S.cur.a, 0), bb = max(S.cur.b, 0);
-            mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+            mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
+            for (int c = 0; c < F::kHalves; ++c) {
                 tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, ba * kBlk, S.kvh, S.b);
                 tma_load_4d(dst + c * 2 * kHalfTile + kHalfTile, tk, bar, c * 64, bb * kBlk, S.kvh, S.b);
             }
@@ -283,13 +301,13 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
             if (elect_one()) {
                 const Item &it = tl->m_item[qm.idx];
                 const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
-                mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+                mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
 #pragma unroll
-                for (int c = 0; c < 2; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
+                for (int c = 0; c < F::kHalves; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         const bool second = r == 1 && it.R == 2;
-                        tma_load_4d(q_smem + qs.idx * kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64,
+                        tma_load_4d(q_smem + qs.idx * F::kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64,
                                     (second ? it.qb[1] : it.qb[0]) * kBlk, second ? it.h[1] : it.h[0], it.b);
                     }
             }
@@ -311,7 +329,8 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
 // The V tiles, and the pairs' mask rows up to two pairs ahead of everyone else: only the kept entries
 // of a pair (an entry is kept if either row has a block there) go to shared memory, in order, with
 // their number, so that the other roles index them instead of searching.
-__device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail *tl, unsigned v_smem, int lane) {
+template <class F>
+__device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> *tl, unsigned v_smem, int lane) {
     const Geom &g = P.g;
     LoadStream S;
     S.round = 0;
@@ -373,10 +392,10 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail *tl
         // a V stage is free once the product computed from it is complete
         if (!probe_w(smem_u32(&tl->v_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
         if (elect_one()) {  // [tile][half][64 rows][128 B]
-            const unsigned bar = smem_u32(&tl->v_full[S.ring.idx]), dst = v_smem + S.ring.idx * kOperand;
-            mbar_arrive_expect_tx(bar, (unsigned)kOperand);
+            const unsigned bar = smem_u32(&tl->v_full[S.ring.idx]), dst = v_smem + S.ring.idx * F::kOperand;
+            mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
             tma_load_5d(dst, tv, bar, 0, max(S.cur.a, 0) * kBlk, S.kvh, 0, S.b);
-            tma_load_5d(dst + kTile, tv, bar, 0, max(S.cur.b, 0) * kBlk, S.kvh, 0, S.b);
+            tma_load_5d(dst + F::kTile, tv, bar, 0, max(S.cur.b, 0) * kBlk, S.kvh, 0, S.b);
         }
         __syncwarp();
         S.ring.advance(P.n_v_stages);
@@ -394,14 +413,15 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail *tl
 // warp-wide, one elected lane issues.
 
 // S_r = Q_r K_r^T of both rows for every kept entry.
-__device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base) {
+template <class F>
+__device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base) {
     Ring ks, ms, qs;
     unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
     const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
     for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
         const int n_entries = tl->m_count[ms.idx];  // the issuers need no more than the count
-        const unsigned q_lo = q_lo0 + qs.idx * (kOperand >> 4);
+        const unsigned q_lo = q_lo0 + qs.idx * (F::kOperand >> 4);
         if (n_entries > 0) {
             if (!wait_w(smem_u32(&tl->q_full[qs.idx]), qs.phase, tl, 201)) return;
             qs.advance(2);
@@ -412,16 +432,16 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
             if (!wait_w(smem_u32(&tl->s_free[gi][use & 1u]), ((use >> 1) & 1u) ^ 1u, tl, 203)) return;
             tc_fence_after();
             const unsigned d_tmem = tmem_base + gi * 128 + (use & 1u) * 64;
-            const unsigned b_lo = k_lo + ks.idx * (kOperand >> 4);
+            const unsigned b_lo = k_lo + ks.idx * (F::kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int c = 0; c < 2; ++c)
+                    for (int c = 0; c < F::kHalves; ++c)
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4)
                             tc_mma_bf16_split(d_tmem + r * kRowLanes, q_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK,
-                                              b_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK, kIdescQK, (c | k4) != 0);
+                                              b_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK, F::kIdescQK, (c | k4) != 0);
                 tc_commit(smem_u32(&tl->s_full[gi][use & 1u]));
                 tc_commit(smem_u32(&tl->k_empty[ks.idx]));
             }
@@ -435,32 +455,35 @@ __device__ void qk_role(const Params &P, Tail *tl, unsigned q_smem, unsigned k_s
 }
 
 // O_r (+)= P_r V_r of both rows for every kept entry; a pair's first entry starts O afresh.
-__device__ void pv_role(const Params &P, Tail *tl, unsigned v_smem, unsigned tmem_base) {
+template <class F>
+__device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned tmem_base) {
     Ring vs, ms;  // vs: the entry's V stage
     unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
     unsigned free_par = 1;  // (the first wait passes at once)
     // the MN-major V tiles have their two 64-channel halves kHalfTile apart
-    const unsigned v_lo = desc_lo_sw128(v_smem, kHalfTile), d_tmem = tmem_base + kOCol;
+    const unsigned v_lo = desc_lo_sw128(v_smem, kHalfTile), d_tmem = tmem_base + F::kOCol;
     for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
         const int n_entries = tl->m_count[ms.idx];
         for (int i = 0; i < n_entries; ++i) {
             if (!wait_w(smem_u32(&tl->v_full[vs.idx]), vs.phase, tl, 205)) return;
-            const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use & 1u;
-            if (!wait_w(smem_u32(&tl->p_full[gi][pb]), (use >> 1) & 1u, tl, 204)) return;  // also: O rescaled if it had to be
+            const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use % F::kPBufs;
+            if (!wait_w(smem_u32(&tl->p_full[gi][pb]), (use / F::kPBufs) & 1u, tl, 204)) return;  // also: O rescaled if it had to be
             if (i == 0) {
                 if (!wait_w(smem_u32(&tl->o_free), free_par, tl, 206)) return;  // the previous pair's O has been read
                 free_par ^= 1;
             }
             tc_fence_after();
-            const unsigned a_tmem = tmem_base + kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (kOperand >> 4);
+            const unsigned a_tmem = tmem_base + F::kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (F::kOperand >> 4);
             if (elect_one()) {
 #pragma unroll
-                for (int r = 0; r < 2; ++r)  // row r of the pair: its P, its V tile
+                for (int r = 0; r < 2; ++r)  // row r of the pair: its P (or the parts of it), its V tile
 #pragma unroll
-                    for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step: 8 columns of packed bf16
-                        tc_mma_bf16_ta(d_tmem + r * kRowLanes, a_tmem + r * kRowLanes + s4 * 8, b_lo + ((r * kTile + s4 * 2048) >> 4), kHiK,
-                                       kIdescPV, (i | s4) != 0);
+                    for (int part = 0; part < (F::kSplit ? 2 : 1); ++part)
+#pragma unroll
+                        for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step: 8 columns of packed bf16
+                            tc_mma_bf16_ta(d_tmem + r * kRowLanes, a_tmem + r * kRowLanes + part * 32 + s4 * 8,
+                                           b_lo + ((r * F::kTile + s4 * 2048) >> 4), kHiK, F::kIdescPV, (i | part | s4) != 0);
                 tc_commit(smem_u32(&tl->p_free[gi][pb]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
                 if (i + 1 == n_entries) tc_commit(smem_u32(&tl->o_done));
@@ -481,11 +504,12 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-// Multiplies 128 fp32 columns of this thread's TMEM lane by f, in place (every lane of the warp
+// Multiplies fp32 columns of this thread's TMEM lane by f, in place (every lane of the warp
 // takes part; lanes that need no change pass f = 1).
+template <int kColumns>
 __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 #pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < kColumns / 32; ++c) {
         unsigned r[32];
         tmem_ld_32x32_issue(taddr + c * 32, r);
         tmem_ld_wait();
@@ -505,12 +529,13 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 // every phase of its own logit and P buffers; what it waits for of the other group's (`turn`) it
 // has followed entry by entry within the pair, and everything of earlier pairs is complete after
 // o_done.
-__device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
+template <class F>
+__device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
     const Geom &g = P.g;
     const int lane = t & 31, row = t & 127, grp = t >> 7, wq = row >> 5, half = lane >> 4, mq = wq * 16 + (lane & 15);
     const unsigned lanes = tmem_base + ((unsigned)(row & ~31) << 16);
     const unsigned turn_own = smem_u32(&tl->turn[wq][grp]), turn_other = smem_u32(&tl->turn[wq][grp ^ 1]);
-    unsigned char *const stage = q_ptr + (grp * 4 + wq) * 4096;  // this warp's 32 tokens x 64 channels in a Q buffer
+    unsigned char *const stage = q_ptr + (grp * 4 + wq) * 32 * F::kOutBytes;  // this warp's 32 tokens x half of the channels in a Q buffer
     unsigned n_other = 0;     // entries of the other group before this pair, over the whole kernel
     unsigned n_own = 0;       // entries of this group so far
     const unsigned s_full = smem_u32(&tl->s_full[grp][0]), s_free = smem_u32(&tl->s_free[grp][0]), s_addr = lanes + grp * 128;
@@ -542,15 +567,15 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
         bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
             // the token's 64 logits against its row's key block
-            const unsigned pb = n_own & 1u;  // the entry's logit and P buffer
-            if (!wait_w(s_full + pb * 8, (n_own >> 1) & 1u, tl, 301)) return;
+            const unsigned sb = n_own & 1u, pb = n_own % F::kPBufs;  // the entry's logit and P buffers
+            if (!wait_w(s_full + sb * 8, (n_own >> 1) & 1u, tl, 301)) return;
             tc_fence_after();
             unsigned sr[64];
-            tmem_ld_32x32_issue(s_addr + pb * 64, sr);
-            tmem_ld_32x32_issue(s_addr + pb * 64 + 32, sr + 32);
+            tmem_ld_32x32_issue(s_addr + sb * 64, sr);
+            tmem_ld_32x32_issue(s_addr + sb * 64 + 32, sr + 32);
             tmem_ld_wait();
             tc_fence_before();
-            mbar_arrive_if(s_free + pb * 8, lane == 0);
+            mbar_arrive_if(s_free + sb * 8, lane == 0);
             if (masked) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
@@ -573,14 +598,15 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             const unsigned other = n_other + (unsigned)((n - 1) >> 1), turn_par = other & 1u;  // entry n - 1 is the other group's `other`-th
             const int next_blk = my_row[min(n + 2, last_entry)];  // (of no meaning behind the last)
             int next_hi = 0;
-            const unsigned p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own >> 1) & 1u) ^ 1u;
-            unsigned packed[32];
+            const unsigned p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own / F::kPBufs) & 1u) ^ 1u;
+            const unsigned p_addr = lanes + F::kPCol + grp * 64 + (F::kSplit ? 0 : pb * 32);
+            unsigned packed[F::kSplit ? 16 : 32], rest[16];
             float esum;
             for (int attempt = 0;; ++attempt) {
                 const float shift = ref == -CUDART_INF_F ? 0.f : -ref * P.scale_log2;
                 const unsigned long long scale2 = pack_f32x2(P.scale_log2, P.scale_log2), shift2 = pack_f32x2(shift, shift);
                 unsigned long long sum2[4] = {0ull, 0ull, 0ull, 0ull};
-                auto weights = [&](int i0) {
+                auto weights = [&](int i0) -> bool {
 #pragma unroll
                     for (int i = i0; i < i0 + 32; i += 2) {
                         float x0, x1;
@@ -588,10 +614,22 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                         const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
                         sum2[(i >> 1) & 3] = add_f32x2(sum2[(i >> 1) & 3], pack_f32x2(p0, p1));
                         const __nv_bfloat162 pk = __floats2bfloat162_rn(p0, p1);
-                        packed[i >> 1] = *reinterpret_cast<const unsigned *>(&pk);
+                        packed[F::kSplit ? (i >> 1) & 15 : i >> 1] = *reinterpret_cast<const unsigned *>(&pk);
+                        if (F::kSplit) {
+                            const float2 top = __bfloat1622float2(pk);
+                            const __nv_bfloat162 low = __floats2bfloat162_rn(p0 - top.x, p1 - top.y);
+                            rest[(i >> 1) & 15] = *reinterpret_cast<const unsigned *>(&low);
+                        }
                     }
+                    if (F::kSplit) {  // (half at a time: both parts of a whole row do not fit in registers beside the logits)
+                        // the product of the group's last entry, from the same buffer, is complete
+                        if (i0 == 0 && !wait_w(p_free, p_par, tl, 309)) return false;
+                        tmem_st_32x16_issue(p_addr + (i0 >> 1), packed);
+                        tmem_st_32x16_issue(p_addr + 32 + (i0 >> 1), rest);
+                    }
+                    return true;
                 };
-                weights(0);
+                if (!weights(0)) return;
                 bool seen = mbar_test_wait(p_free, p_par);
                 float now = ref;
                 if (n > 0) {
@@ -614,6 +652,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                     moved = __float_as_uint(now) != __float_as_uint(ref);
                 }
                 if (attempt == 2 || !__any_sync(0xffffffffu, moved || outgrown)) break;
+                if (F::kSplit) tmem_st_wait();
                 if (moved) {
                     if (ref != -CUDART_INF_F) l *= fast_exp2((ref - now) * P.scale_log2);
                     ref = now;
@@ -628,15 +667,15 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                         tl->ref[row] = ref;
                     }
                     if (n > 0) {  // what has been added up so far is brought to the new reference
-                        if (!wait_w(smem_u32(&tl->p_free[grp ^ 1][other & 1u]), (other >> 1) & 1u, tl, 302)) return;
+                        if (!wait_w(smem_u32(&tl->p_free[grp ^ 1][other % F::kPBufs]), (other / F::kPBufs) & 1u, tl, 302)) return;
                         tc_fence_after();
-                        rescale_lane(lanes + kOCol, f);
+                        rescale_lane<F::kD>(lanes + F::kOCol, f);
                     }
                     l *= f;
                 }
             }
             l += esum;
-            tmem_st_32x32_issue(lanes + kPCol + grp * 64 + pb * 32, packed);
+            if constexpr (!F::kSplit) tmem_st_32x32_issue(p_addr, packed);
             tmem_st_wait();
             tc_fence_before();
             mbar_arrive_if(turn_own, lane == 0);
@@ -659,9 +698,9 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             tl->sum[grp][row] = l;
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tl->sums_there[wq]));
-            unsigned ra[64];  // this group stores channels 64 grp .. 64 grp + 63 of every token
-            tmem_ld_32x32_issue(lanes + kOCol + grp * 64, ra);
-            tmem_ld_32x32_issue(lanes + kOCol + grp * 64 + 32, ra + 32);
+            unsigned ra[F::kD / 2];  // this group stores half of the channels of every token
+#pragma unroll
+            for (int x = 0; x < F::kD / 64; ++x) tmem_ld_32x32_issue(lanes + F::kOCol + grp * (F::kD / 2) + 32 * x, ra + 32 * x);
             tmem_ld_wait();
             tc_fence_before();
             if (!wait_w(smem_u32(&tl->sums_there[wq]), pair_par, tl, 304)) return;
@@ -669,28 +708,29 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tl->o_free));
             const float inv = total > 0.f ? 1.f / total : 0.f;
-            // The warp's 32 x 64 part goes to the pair's Q buffer, whose last product is complete, and
+            // The warp's part goes to the pair's Q buffer, whose last product is complete, and
             // from there to global memory as one TMA store (rows beyond T are left out): a lane's
             // own 128 bytes stored directly would touch 32 lines with every instruction.
-            unsigned char *const dst = stage + qs.idx * kOperand + lane * 128;
+            unsigned char *const dst = stage + qs.idx * F::kOperand + lane * F::kOutBytes;
+            const int turned = F::kOutBytes == 128 ? lane & 7 : (lane >> 1) & 3;  // the swizzle of the map's 128 or 64 bytes
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
+            for (int c = 0; c < F::kOutBytes / 16; ++c) {
                 unsigned w[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(ra[8 * c + 2 * u]) * inv, __uint_as_float(ra[8 * c + 2 * u + 1]) * inv);
                     w[u] = *reinterpret_cast<const unsigned *>(&pk);
                 }
-                *reinterpret_cast<uint4 *>(dst + ((c ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4 *>(dst + ((c ^ turned) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
             }
             fence_async_smem();
             __syncwarp();
             const int h_1 = __shfl_sync(0xffffffffu, h, 16), tok_1 = __shfl_sync(0xffffffffu, tq0, 16) + wq * 16;
             const bool there_1 = __shfl_sync(0xffffffffu, (int)row_active, 16) != 0;
             if (lane == 0) {  // lanes 0 and 16 hold the first of the 16 tokens of a row
-                const unsigned src = smem_u32(stage + qs.idx * kOperand);
-                if (row_active) tma_store_4d(to, src, grp * 64, tq0 + wq * 16, h, b);
-                if (there_1) tma_store_4d(to, src + 16 * 128, grp * 64, tok_1, h_1, b);
+                const unsigned src = smem_u32(stage + qs.idx * F::kOperand);
+                if (row_active) tma_store_4d(to, src, grp * (F::kD / 2), tq0 + wq * 16, h, b);
+                if (there_1) tma_store_4d(to, src + 16 * F::kOutBytes, grp * (F::kD / 2), tok_1, h_1, b);
                 tma_store_commit();
             }
             staged = qs.idx;
@@ -698,33 +738,34 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
             pair_par ^= 1;
             n_other += (unsigned)(grp == 0 ? n_entries >> 1 : (n_entries + 1) >> 1);
         } else if (row_active) {
-            uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)b * g.H + h) * g.T + tq0 + mq) * kD + grp * 64);
+            uint4 *dst = reinterpret_cast<uint4 *>(P.out + (((long long)b * g.H + h) * g.T + tq0 + mq) * F::kD + grp * (F::kD / 2));
 #pragma unroll
-            for (int c = 0; c < 8; ++c) dst[c] = make_uint4(0, 0, 0, 0);
+            for (int c = 0; c < F::kOutBytes / 16; ++c) dst[c] = make_uint4(0, 0, 0, 0);
         }
     }
     if (lane == 0) tma_store_wait_read();  // shared memory is given back when the CTA leaves
     __syncwarp();
 }
 
+template <class F>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                const __grid_constant__ CUtensorMap tmap_v, const __grid_constant__ CUtensorMap tmap_out, Params P) {  // P by value: n_k_stages is filled in here
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = aligned_smem(smem_raw);
     // what is left behind the aligned base decides the number of V and K stages (the same in every thread)
-    const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
-    const int n_rings = (P.smem_bytes - fixed_bytes) / kOperand - kFixedOperands;  // buffers for the two rings: 4 or 5
-    P.n_v_stages = n_rings >= 5 ? 3 : 2;
-    P.n_k_stages = min(kMaxKStages, n_rings - P.n_v_stages);
-    const unsigned q_smem = smem_u32(smem), v_smem = q_smem + kFixedOperands * kOperand, k_smem = v_smem + P.n_v_stages * kOperand;
-    Tail *tl = (Tail *)(smem + (kFixedOperands + P.n_v_stages + P.n_k_stages) * kOperand);
+    const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail<F>) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
+    const int n_rings = (P.smem_bytes - fixed_bytes) / F::kOperand - kFixedOperands;  // buffers for the two rings: d = 128: 4 or 5
+    P.n_v_stages = min(F::kMaxVStages, (n_rings + 1) / 2);
+    P.n_k_stages = min(F::kMaxKStages, n_rings - P.n_v_stages);
+    const unsigned q_smem = smem_u32(smem), v_smem = q_smem + kFixedOperands * F::kOperand, k_smem = v_smem + P.n_v_stages * F::kOperand;
+    Tail<F> *tl = (Tail<F> *)(smem + (kFixedOperands + P.n_v_stages + P.n_k_stages) * F::kOperand);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), 8); }
-        for (int i = 0; i < kMaxKStages; ++i) { mbar_init(smem_u32(&tl->k_full[i]), 1); mbar_init(smem_u32(&tl->k_empty[i]), 1); }
-        for (int i = 0; i < kMaxVStages; ++i) { mbar_init(smem_u32(&tl->v_full[i]), 1); mbar_init(smem_u32(&tl->v_empty[i]), 1); }
+        for (int i = 0; i < F::kMaxKStages; ++i) { mbar_init(smem_u32(&tl->k_full[i]), 1); mbar_init(smem_u32(&tl->k_empty[i]), 1); }
+        for (int i = 0; i < F::kMaxVStages; ++i) { mbar_init(smem_u32(&tl->v_full[i]), 1); mbar_init(smem_u32(&tl->v_empty[i]), 1); }
         for (int i = 0; i < 2; ++i) {
             for (int j = 0; j < 2; ++j) { mbar_init(smem_u32(&tl->s_full[i][j]), 1); mbar_init(smem_u32(&tl->s_free[i][j]), 4); mbar_init(smem_u32(&tl->p_full[i][j]), 4); mbar_init(smem_u32(&tl->p_free[i][j]), 1); }
         }
@@ -775,28 +816,29 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
 
 }  // namespace
 
-bool attn_tc_supported(const Geom &g, int dtype) {
-    return dtype == STREAM_BF16 && g.d == kD && g.bq == kBlk && g.bk == kBlk && g.k_top <= kMaxKTopTc && tma_strides_ok(g);
+bool attn_tc_supported(const Geom &g, int dtype) { return g.d == 128 && attn_tc_auto(g, dtype); }
+
+// Against the mma.sync kernel at d = 64: FIGS
+bool attn_tc_auto(const Geom &g, int dtype) {
+    return dtype == STREAM_BF16 && (g.d == 64 || g.d == 128) && g.bq == kBlk && g.bk == kBlk && g.k_top <= kMaxKTopTc && tma_strides_ok(g);
 }
 
-stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask,
-                             float scale, void *out, cudaStream_t st) {
-    if ((((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)out) & 15) != 0) {
-        set_error("tensor-core attention kernel needs 16-byte aligned q, k, v and out");
-        return STREAM_ERR_UNSUPPORTED;
-    }
+namespace {
+template <class F>
+stream_status launch(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
+                     cudaStream_t st) {
     CUtensorMap tq, tk, tv, to;
-    stream_status rc = make_map_bf16_d128(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q");  // 4-D: 64 x 64 half tiles
+    stream_status rc = make_map_bf16(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q", kBlk, F::kD);  // 4-D: 64 x 64 half tiles
     if (rc != STREAM_OK) return rc;
-    rc = make_map_bf16_d128(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k");
+    rc = make_map_bf16(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k", kBlk, F::kD);
     if (rc != STREAM_OK) return rc;
-    rc = make_map5_bf16_d128(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v");
+    rc = make_map5_bf16(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v", F::kD);
     if (rc != STREAM_OK) return rc;
-    rc = make_map_bf16_d128(&to, out, g.T, g.H, g.batch, kD, g.T * kD, (long long)g.H * g.T * kD, "out", 16);
+    rc = make_map_bf16(&to, out, g.T, g.H, g.batch, F::kD, g.T * F::kD, (long long)g.H * g.T * F::kD, "out", 16, F::kD, F::kD / 2);
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;
-    const long long kv_bytes = 2ll * g.T * kD * 2;  // K and V of one kv head
+    const long long kv_bytes = 2ll * g.T * F::kD * 2;  // K and V of one kv head
     const long long fit = kL2KvBytes / kv_bytes, all = (long long)g.batch * g.G;
     P.group_heads = (int)(fit < 1 ? 1 : (fit > all ? all : fit));
     const long long n_items = all * ((g.n_qb + 1) / 2) * (2 * (g.hpg / 2) + g.hpg % 2);
@@ -807,25 +849,35 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
     P.scale_log2 = scale * 1.4426950408889634f;
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    // room for five ring buffers if the mask rows are short enough, else four; 1 KB of slack for the alignment
+    // room for all ring buffers if the mask rows are short enough, else fewer, but four; 1 KB of slack for the alignment
     // of the base (the kernel counts its stages from what it really gets)
     P.row_stride = (g.k_top + 3) & ~3;
-    const int tail_bytes = (int)sizeof(Tail) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
-    int smem_bytes = (kFixedOperands + 5) * kOperand + tail_bytes + 1024;
+    const int tail_bytes = (int)sizeof(Tail<F>) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
+    int smem_bytes = (kFixedOperands + F::kMaxKStages + F::kMaxVStages) * F::kOperand + tail_bytes + 1024;
     if (smem_bytes > kMaxSmemPerCta) smem_bytes = kMaxSmemPerCta;
-    if (smem_bytes < (kFixedOperands + 4) * kOperand + tail_bytes + 1024) {
+    if (smem_bytes < (kFixedOperands + 4) * F::kOperand + tail_bytes + 1024) {
         set_error("tensor-core attention kernel: k_top = %d needs more shared memory than one CTA has", g.k_top);
         return STREAM_ERR_UNSUPPORTED;
     }
     P.smem_bytes = smem_bytes;
     P.n_k_stages = P.n_v_stages = 0;
-    cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemPerCta);
+    cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemPerCta);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_tc)");
     const int grid = (int)(n_items < n_sm ? n_items : n_sm);
-    attn_tc_kernel<<<grid, kThreads, smem_bytes, st>>>(tq, tk, tv, to, P);
+    attn_tc_kernel<F><<<grid, kThreads, smem_bytes, st>>>(tq, tk, tv, to, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "attn_tc launch");
     return STREAM_OK;
+}
+}  // namespace
+
+stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask,
+                             float scale, void *out, cudaStream_t st) {
+    if ((((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)out) & 15) != 0) {
+        set_error("tensor-core attention kernel needs 16-byte aligned q, k, v and out");
+        return STREAM_ERR_UNSUPPORTED;
+    }
+    return g.d == 128 ? launch<Form<128>>(g, q, k, v, mask, scale, out, st) : launch<Form<64>>(g, q, k, v, mask, scale, out, st);
 }
 
 stream_status read_attn_status(unsigned int out[2], cudaStream_t st) {

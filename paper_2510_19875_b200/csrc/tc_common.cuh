@@ -449,10 +449,10 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// [batch, heads, T, d] bf16 with element strides -> 4-D map with a box of 64 channels x box_rows
-// tokens, 128-byte swizzle. Rows beyond T read as zeros.
+// [batch, heads, T, d] bf16 with element strides -> 4-D map with a box of 64 (or 32) channels x box_rows
+// tokens, 128-byte (or 64-byte) swizzle. Rows beyond T read as zeros.
 inline stream_status make_map_bf16(CUtensorMap *map, const void *base, long long T, int heads, int batch,
-                                   long long s_t, long long s_h, long long s_b, const char *what, int box_rows, int d) {
+                                   long long s_t, long long s_h, long long s_b, const char *what, int box_rows, int d, int channels = 64) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return STREAM_ERR_CUDA; }
     // extents of 1 may come with arbitrary strides: give them a well-formed one
@@ -460,9 +460,9 @@ inline stream_status make_map_bf16(CUtensorMap *map, const void *base, long long
     if (batch == 1) s_b = s_h * heads;
     cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)heads, (cuuint64_t)batch};
     cuuint64_t strides[3] = {(cuuint64_t)s_t * 2, (cuuint64_t)s_h * 2, (cuuint64_t)s_b * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1}, estr[4] = {1, 1, 1, 1};
+    cuuint32_t box[4] = {(cuuint32_t)channels, (cuuint32_t)box_rows, 1, 1}, estr[4] = {1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, channels == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled(%s) failed with %d", what, (int)r); return STREAM_ERR_CUDA; }
     return STREAM_OK;
@@ -473,19 +473,19 @@ inline stream_status make_map_bf16_d128(CUtensorMap *map, const void *base, long
     return make_map_bf16(map, base, T, heads, batch, s_t, s_h, s_b, what, box_rows, 128);
 }
 
-// The same tensor seen as [batch, heads, 2 channel halves, T, 64]: one box brings a whole
-// 64-token x 128-channel tile (16 KB) as [half][64 rows][128 B], the layout of a 128-byte-swizzled
+// The same tensor seen as [batch, heads, channel halves, T, 64]: one box brings a whole
+// 64-token x d-channel tile as [half][64 rows][128 B], the layout of a 128-byte-swizzled
 // K-major (or, read along the rows, MN-major) tcgen05 operand.
 // Coordinates: (0, token, head, 0, batch) with the half as dimension 3.
-inline stream_status make_map5_bf16_d128(CUtensorMap *map, const void *base, long long T, int heads, int batch,
-                                         long long s_t, long long s_h, long long s_b, const char *what) {
+inline stream_status make_map5_bf16(CUtensorMap *map, const void *base, long long T, int heads, int batch,
+                                    long long s_t, long long s_h, long long s_b, const char *what, int d) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return STREAM_ERR_CUDA; }
     if (heads == 1) s_h = s_t * T;
     if (batch == 1) s_b = s_h * heads;
-    cuuint64_t dims[5] = {64, (cuuint64_t)T, (cuuint64_t)heads, 2, (cuuint64_t)batch};
+    cuuint64_t dims[5] = {64, (cuuint64_t)T, (cuuint64_t)heads, (cuuint64_t)(d / 64), (cuuint64_t)batch};
     cuuint64_t strides[4] = {(cuuint64_t)s_t * 2, (cuuint64_t)s_h * 2, 128, (cuuint64_t)s_b * 2};
-    cuuint32_t box[5] = {64, 64, 1, 2, 1}, estr[5] = {1, 1, 1, 1, 1};
+    cuuint32_t box[5] = {64, 64, 1, (cuuint32_t)(d / 64), 1}, estr[5] = {1, 1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
