@@ -1,9 +1,8 @@
-// Tensor-core block-sparse attention for sm_100a (Eq. 2 on a Stream mask): bf16, d = 128,
-// 64 x 64 blocks.
+// Tensor-core block-sparse attention for sm_100a (Eq. 2 on a Stream mask): bf16, d = 64 or 128, blocks
+// of 32 or 64. (What follows is said for d = 128 and blocks of 64; Form has the differences.)
 //
-// One persistent CTA per SM works through "pairs": two rows (query blocks) of one kv head - two query
-// heads at one query block, or, where the number of heads per kv head is odd, two neighbouring
-// query blocks of the last head. For every mask entry e the two rows name one key block each (K_0, K_1,
+// One persistent CTA per SM works through "pairs": two rows (query blocks) of one kv head, as a rule two
+// query heads at one query block. For every mask entry e the two rows name one key block each (K_0, K_1,
 // usually different); the tiles arrive by TMA (128-byte swizzle), and each row r has its own products,
 //     S_r = Q_r K_r^T  (64 x 64),     O_r += P_r V_r  (64 x 128),
 // with M = 64: a row's 64 tokens take 16 of every 32 TMEM lanes (token 16 w + i in lane 32 w + 16 r + i),
@@ -61,15 +60,19 @@ namespace {
 using namespace tc;
 
 constexpr int kThreads = 384;
-constexpr int kBlk = 64;
-constexpr int kHalfTile = kBlk * 128;       // 64 rows x 128 bytes
-// d = 128: P goes into the product as bf16. d = 64: as a sum of two bf16, whose rounding is below
-// that of the fp32 sums (what the kernels for the other shapes give, too).
-template <int kD_>
+constexpr int kHalfTile = 64 * 128;       // 64 rows x 128 bytes
+// Blocks of 64: two rows in a unit, one in each half of the lanes. Blocks of 32: four, two stacked in
+// each half: their 64 tokens meet the 64 keys of both rows' blocks, a token keeps its own row's half of
+// the logits, and the other half of its P stays zero.
+// d = 128 in blocks of 64: P goes into the product as bf16. Else: as a sum of two bf16, whose rounding is
+// below that of the fp32 sums (what the kernels for the other shapes give, too).
+template <int kD_, int kBlk_>
 struct Form {
-    static constexpr int kD = kD_, kHalves = kD / 64;
-    static constexpr bool kSplit = kD == 64;
-    static constexpr int kTile = kHalves * kHalfTile;  // one 64 x d tile
+    static constexpr int kD = kD_, kBlk = kBlk_, kHalves = kD / 64;
+    static constexpr int kRows = 128 / kBlk, kStack = 64 / kBlk;  // rows of a unit; those stacked in one half of the lanes
+    static constexpr bool kSplit = !(kD == 128 && kBlk == 64);
+    static constexpr int kPart = kBlk * 128;           // a row's block of one channel half
+    static constexpr int kTile = kHalves * kHalfTile;  // 64 x d: the block of one row or those of two
     static constexpr int kOperand = 2 * kTile;         // two tiles: an entry's K or V, or the Q of a pair
     // Stages of the two rings, out of the operand buffers shared memory has room for beside Q. d = 128: five (a V
     // stage is held from its load until the product of its entry is complete, a whole softmax later:
@@ -90,9 +93,10 @@ constexpr float kLazySum = 68719476736.f;   // 2^36 = 64 * 2^30: the 64 P of an 
 
 // The pair a CTA works on. h[r], qb[r]: head and query block of row r < R (R = 0: a place of the
 // order without a pair).
+template <class F>
 struct Item {
     int b, kvh, R;
-    int h[2], qb[2];
+    int h[F::kRows], qb[F::kRows];
 };
 
 template <class F>
@@ -109,7 +113,7 @@ struct Tail {
     unsigned int tmem_base;
     int abort_flag;
     int m_count[kMaskSlots];  // kept entries of the pair in each mask slot
-    Item m_item[kMaskSlots];  // and the pair itself
+    Item<F> m_item[kMaskSlots];  // and the pair itself
     float ref[128], sum[2][128];
 };
 // Dynamic shared memory: Q (two buffers; a pair's output is staged over its Q) | V stages | K stages |
@@ -144,10 +148,10 @@ __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail<F> *t
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &g_attn_status[0], &g_attn_status[1], code);
 }
 
-// Shared copy of the mask rows of the pair in slot `slot`: [2][row_stride] ints behind the Tail.
+// Shared copy of the mask rows of the pair in slot `slot`: [kRows][row_stride] ints behind the Tail.
 template <class F>
 __device__ __forceinline__ int *mask_rows(Tail<F> *tl, const Params &P, int slot) {
-    return reinterpret_cast<int *>(tl + 1) + slot * 2 * P.row_stride;
+    return reinterpret_cast<int *>(tl + 1) + slot * F::kRows * P.row_stride;
 }
 
 // A CTA's n-th place in the order of pairs. Every second round runs backwards, so that with pairs in
@@ -159,42 +163,40 @@ __device__ __forceinline__ int nth_item(const Params &P, int n) {
 // The order: `group_heads` kv heads at a time, as many as have K and V in L2 together, and within
 // them late query blocks (most kept blocks under a causal mask) first. One kv head after the other,
 // every head's short pairs in between, left the CTAs 11 % apart at T = 4096 (32 / 8 heads, k = 32;
-// 4 % at T = 16384), this order with the turn of nth_item 1 %. Two query blocks make a level: their
-// pairs of heads, and the odd last head's pair of its own two query blocks.
-__device__ __forceinline__ Item decode_item(const Params &P, int id) {
+// 4 % at T = 16384), this order with the turn of nth_item 1 %. A kv head's rows are counted query block by
+// query block, head by head within one, and taken from the last in pairs (fours).
+template <class F>
+__device__ __forceinline__ Item<F> decode_item(const Params &P, int id) {
     const Geom &g = P.g;
-    Item it;
-    const int pairs = g.hpg >> 1, per_level = 2 * pairs + (g.hpg & 1), levels = (g.n_qb + 1) >> 1;
-    const int per_head = levels * per_level, per_group = P.group_heads * per_head;
+    Item<F> it;
+    const int n_rows = g.n_qb * g.hpg, levels = (n_rows + F::kRows - 1) / F::kRows;
+    const int per_group = P.group_heads * levels;
     const int grp = id / per_group, rem = id - grp * per_group;
     const int heads = min(P.group_heads, g.batch * g.G - grp * P.group_heads);
-    const int level = rem / (heads * per_level), in_level = rem - level * heads * per_level;
-    const int head = in_level / per_level, slot = in_level - head * per_level;
-    const int bh = grp * P.group_heads + head, j = levels - 1 - level;
+    const int level = rem / heads, bh = grp * P.group_heads + (rem - level * heads);
     it.kvh = bh % g.G;
     it.b = bh / g.G;
-    if (slot < 2 * pairs) {
-        const int qb = 2 * j + 1 - slot / pairs, h0 = it.kvh * g.hpg + slot % pairs * 2;
-        it.R = qb < g.n_qb ? 2 : 0;
-        it.h[0] = h0; it.h[1] = h0 + 1;
-        it.qb[0] = it.qb[1] = min(qb, g.n_qb - 1);
-    } else {
-        it.R = 2 * j + 1 < g.n_qb ? 2 : 1;
-        it.h[0] = it.h[1] = it.kvh * g.hpg + g.hpg - 1;
-        it.qb[0] = 2 * j; it.qb[1] = min(2 * j + 1, g.n_qb - 1);
+    const int last = n_rows - 1 - level * F::kRows;
+    it.R = min(F::kRows, last + 1);
+#pragma unroll
+    for (int r = 0; r < F::kRows; ++r) {
+        const int row = max(last - r, 0);
+        it.qb[r] = row / g.hpg;
+        it.h[r] = it.kvh * g.hpg + row % g.hpg;
     }
     return it;
 }
 
-// Entry e of the two rows: key block per row (negative = this row has nothing at e). An entry
-// is processed if either row has a block there. `rows` is the pair's shared copy [2][stride].
-struct Entry { int a, b; };
-// The mask loader keeps only the kept entries of a pair, in order, at the front of the two
-// resident rows and leaves their number in the Tail: entry n of a pair is (rows[n], rows[stride + n]).
-__device__ __forceinline__ Entry entry_at(const int *rows, int stride, int n) {
-    Entry x;
-    x.a = rows[n];
-    x.b = rows[stride + n];
+// Entry n of a pair: the key block of each row (negative: this row has nothing there). The mask loader
+// keeps only the entries where some row has a block, in order, at the front of the resident rows, and
+// leaves their number in the Tail.
+template <class F>
+struct Entry { int blk[F::kRows]; };
+template <class F>
+__device__ __forceinline__ Entry<F> entry_at(const int *rows, int stride, int n) {
+    Entry<F> x;
+#pragma unroll
+    for (int r = 0; r < F::kRows; ++r) x.blk[r] = rows[r * stride + n];
     return x;
 }
 
@@ -207,11 +209,12 @@ __device__ __forceinline__ Entry entry_at(const int *rows, int stride, int n) {
 // would take 1400 clocks that way, more than its two chains. Neither blocks on one thing while another could
 // move: every step probes its barrier without waiting. The warps run converged (lane 0's probe
 // result is broadcast) and one elected lane issues.
+template <class F>
 struct LoadStream {
     int round, id;     // pair being walked
     int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
     int n = 0;         // kept entries of the pair
-    Entry cur;
+    Entry<F> cur;
     int b, kvh;
     Ring ring, ms;
 };
@@ -222,17 +225,17 @@ __device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
 
 // Opens the stream's pair (its mask rows must be resident) or closes it; true if it did.
 template <class F>
-__device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStream &S) {
+__device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStream<F> &S) {
     if (!probe_w(smem_u32(&tl->m_full[S.ms.idx]), S.ms.phase)) return false;
     S.b = tl->m_item[S.ms.idx].b;
     S.kvh = tl->m_item[S.ms.idx].kvh;
     S.n = tl->m_count[S.ms.idx];
     S.e = 0;
-    if (S.n > 0) S.cur = entry_at(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
+    if (S.n > 0) S.cur = entry_at<F>(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
     return true;
 }
 template <class F>
-__device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStream &S) {
+__device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStream<F> &S) {
     if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
     __syncwarp();
     S.ms.advance(kMaskSlots);
@@ -240,8 +243,8 @@ __device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStr
     S.e = -2;
 }
 template <class F>
-__device__ __forceinline__ void next_entry(const Params &P, Tail<F> *tl, LoadStream &S) {
-    if (++S.e < S.n) S.cur = entry_at(mask_rows(tl, P, S.ms.idx), P.row_stride, S.e);
+__device__ __forceinline__ void next_entry(const Params &P, Tail<F> *tl, LoadStream<F> &S) {
+    if (++S.e < S.n) S.cur = entry_at<F>(mask_rows(tl, P, S.ms.idx), P.row_stride, S.e);
 }
 
 // After a step that could not move: false if the CTA is aborting or nothing has moved for too long.
@@ -264,7 +267,7 @@ __device__ __forceinline__ bool idle_ok(Tail<F> *tl, long long t_last, unsigned 
 template <class F>
 __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CUtensorMap *tk, Tail<F> *tl, unsigned q_smem,
                                 unsigned k_smem) {
-    LoadStream S;
+    LoadStream<F> S;
     S.round = 0;
     S.id = nth_item(P, 0);
     S.e = -2;
@@ -274,15 +277,14 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
         // a K stage is free once the logits computed from it are complete
         if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
         if (elect_one()) {
-            // [half][tile][64 rows][128 B]; a row without a block at an entry gets block 0, its logits are masked out
+            // [half][row][keys][128 B]; a row without a block at an entry gets block 0, its logits are masked out
             const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * F::kOperand;
-            const int ba = max(S.cur.a, 0), bb = max(S.cur.b, 0);
             mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
 #pragma unroll
-            for (int c = 0; c < F::kHalves; ++c) {
-                tma_load_4d(dst + c * 2 * kHalfTile, tk, bar, c * 64, ba * kBlk, S.kvh, S.b);
-                tma_load_4d(dst + c * 2 * kHalfTile + kHalfTile, tk, bar, c * 64, bb * kBlk, S.kvh, S.b);
-            }
+            for (int c = 0; c < F::kHalves; ++c)
+#pragma unroll
+                for (int r = 0; r < F::kRows; ++r)
+                    tma_load_4d(dst + c * 2 * kHalfTile + r * F::kPart, tk, bar, c * 64, max(S.cur.blk[r], 0) * F::kBlk, S.kvh, S.b);
         }
         __syncwarp();
         S.ring.advance(P.n_k_stages);
@@ -299,17 +301,14 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
         if (tl->m_count[qm.idx] > 0) {
             if (!probe_w(smem_u32(&tl->q_free[qs.idx]), qs.phase ^ 1)) return false;
             if (elect_one()) {
-                const Item &it = tl->m_item[qm.idx];
+                const Item<F> &it = tl->m_item[qm.idx];
                 const unsigned bar = smem_u32(&tl->q_full[qs.idx]);
                 mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
 #pragma unroll
-                for (int c = 0; c < F::kHalves; ++c)  // [half][row][64 tokens][128 B]; a missing second row repeats the first
+                for (int c = 0; c < F::kHalves; ++c)  // [half][row][tokens][128 B] (a missing row has those of another)
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const bool second = r == 1 && it.R == 2;
-                        tma_load_4d(q_smem + qs.idx * F::kOperand + (2 * c + r) * kHalfTile, tq, bar, c * 64,
-                                    (second ? it.qb[1] : it.qb[0]) * kBlk, second ? it.h[1] : it.h[0], it.b);
-                    }
+                    for (int r = 0; r < F::kRows; ++r)
+                        tma_load_4d(q_smem + qs.idx * F::kOperand + c * 2 * kHalfTile + r * F::kPart, tq, bar, c * 64, it.qb[r] * F::kBlk, it.h[r], it.b);
             }
             __syncwarp();
             qs.advance(2);
@@ -332,30 +331,27 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
 template <class F>
 __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> *tl, unsigned v_smem, int lane) {
     const Geom &g = P.g;
-    LoadStream S;
+    LoadStream<F> S;
     S.round = 0;
     S.id = nth_item(P, 0);
     S.e = -2;
     int m_round = 0, m_id = nth_item(P, 0);  // the next pair whose mask rows are due
     bool asked = false;                      // its first 32 entries are on their way to registers
-    Item it;
-    int a0 = -1, b0 = -1;
-    const int32_t *m0 = nullptr, *m1 = nullptr;
+    Item<F> it;
+    int first[F::kRows];
+    const int32_t *row[F::kRows];
     Ring mw;
-    auto fetch = [&](int e, int &a, int &b) {
-        a = b = -1;
-        if (e < g.k_top) {
-            if (it.R >= 1) a = __ldg(m0 + e);
-            if (it.R == 2) b = __ldg(m1 + e);
-        }
+    auto fetch = [&](int e, int (&blk)[F::kRows]) {
+#pragma unroll
+        for (int r = 0; r < F::kRows; ++r) blk[r] = e < g.k_top && r < it.R ? __ldg(row[r] + e) : -1;
     };
     auto mask_step = [&]() -> bool {
         if (m_id >= P.n_items) return false;
         if (!asked) {
-            it = decode_item(P, m_id);
-            m0 = P.mask + (((long long)it.b * g.H + it.h[0]) * g.n_qb + it.qb[0]) * g.k_top;
-            m1 = P.mask + (((long long)it.b * g.H + it.h[1]) * g.n_qb + it.qb[1]) * g.k_top;
-            fetch(lane, a0, b0);
+            it = decode_item<F>(P, m_id);
+#pragma unroll
+            for (int r = 0; r < F::kRows; ++r) row[r] = P.mask + (((long long)it.b * g.H + it.h[r]) * g.n_qb + it.qb[r]) * g.k_top;
+            fetch(lane, first);
             asked = true;
             return true;
         }
@@ -363,14 +359,19 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         int *dst = mask_rows(tl, P, mw.idx);
         int cnt = 0;
         for (int base = 0; base < g.k_top; base += 32) {
-            int a = a0, b = b0;
-            if (base > 0) fetch(base + lane, a, b);
-            const bool kept = a >= 0 || b >= 0;
+            int blk[F::kRows];
+            bool kept = false;
+            if (base > 0) fetch(base + lane, blk);
+#pragma unroll
+            for (int r = 0; r < F::kRows; ++r) {
+                if (base == 0) blk[r] = first[r];
+                kept = kept || blk[r] >= 0;
+            }
             const unsigned bal = __ballot_sync(0xffffffffu, kept);
             if (kept) {
                 const int pos = cnt + __popc(bal & ((1u << lane) - 1u));
-                dst[pos] = a;
-                dst[P.row_stride + pos] = b;
+#pragma unroll
+                for (int r = 0; r < F::kRows; ++r) dst[r * P.row_stride + pos] = blk[r];
             }
             cnt += __popc(bal);
         }
@@ -391,11 +392,12 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         if (S.e >= S.n) { close_pair(P, tl, S); return true; }
         // a V stage is free once the product computed from it is complete
         if (!probe_w(smem_u32(&tl->v_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
-        if (elect_one()) {  // [tile][half][64 rows][128 B]
+        if (elect_one()) {  // [row][half][keys][128 B]
             const unsigned bar = smem_u32(&tl->v_full[S.ring.idx]), dst = v_smem + S.ring.idx * F::kOperand;
             mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
-            tma_load_5d(dst, tv, bar, 0, max(S.cur.a, 0) * kBlk, S.kvh, 0, S.b);
-            tma_load_5d(dst + F::kTile, tv, bar, 0, max(S.cur.b, 0) * kBlk, S.kvh, 0, S.b);
+#pragma unroll
+            for (int r = 0; r < F::kRows; ++r)
+                tma_load_5d(dst + r * F::kHalves * F::kPart, tv, bar, 0, max(S.cur.blk[r], 0) * F::kBlk, S.kvh, 0, S.b);
         }
         __syncwarp();
         S.ring.advance(P.n_v_stages);
@@ -460,8 +462,8 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
     Ring vs, ms;  // vs: the entry's V stage
     unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
     unsigned free_par = 1;  // (the first wait passes at once)
-    // the MN-major V tiles have their two 64-channel halves kHalfTile apart
-    const unsigned v_lo = desc_lo_sw128(v_smem, kHalfTile), d_tmem = tmem_base + F::kOCol;
+    // a row's MN-major V block has its two 64-channel halves kPart apart
+    const unsigned v_lo = desc_lo_sw128(v_smem, F::kPart), d_tmem = tmem_base + F::kOCol;
     for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
         const int n_entries = tl->m_count[ms.idx];
@@ -483,7 +485,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
 #pragma unroll
                         for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step: 8 columns of packed bf16
                             tc_mma_bf16_ta(d_tmem + r * kRowLanes, a_tmem + r * kRowLanes + part * 32 + s4 * 8,
-                                           b_lo + ((r * F::kTile + s4 * 2048) >> 4), kHiK, F::kIdescPV, (i | part | s4) != 0);
+                                           b_lo + ((r * F::kTile + s4 / (F::kBlk / 16) * F::kHalves * F::kPart + s4 % (F::kBlk / 16) * 2048) >> 4), kHiK, F::kIdescPV, (i | part | s4) != 0);
                 tc_commit(smem_u32(&tl->p_free[gi][pb]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
                 if (i + 1 == n_entries) tc_commit(smem_u32(&tl->o_done));
@@ -532,16 +534,28 @@ __device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
 template <class F>
 __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
     const Geom &g = P.g;
-    const int lane = t & 31, row = t & 127, grp = t >> 7, wq = row >> 5, half = lane >> 4, mq = wq * 16 + (lane & 15);
+    const int lane = t & 31, row = t & 127, grp = t >> 7, wq = row >> 5;
+    // this thread's row of the pair, its token of the row's query block, its logits' first column (in stacked
+    // rows: its row's half)
+    const int r_own = (lane >> 4) * F::kStack + (F::kStack == 2 ? wq >> 1 : 0), mq = (F::kStack == 2 ? wq & 1 : wq) * 16 + (lane & 15);
+    const int col = F::kStack == 2 ? (wq >> 1) * 32 : 0;
     const unsigned lanes = tmem_base + ((unsigned)(row & ~31) << 16);
     const unsigned turn_own = smem_u32(&tl->turn[wq][grp]), turn_other = smem_u32(&tl->turn[wq][grp ^ 1]);
     unsigned char *const stage = q_ptr + (grp * 4 + wq) * 32 * F::kOutBytes;  // this warp's 32 tokens x half of the channels in a Q buffer
     unsigned n_other = 0;     // entries of the other group before this pair, over the whole kernel
     unsigned n_own = 0;       // entries of this group so far
-    const unsigned s_full = smem_u32(&tl->s_full[grp][0]), s_free = smem_u32(&tl->s_free[grp][0]), s_addr = lanes + grp * 128;
+    const unsigned s_full = smem_u32(&tl->s_full[grp][0]), s_free = smem_u32(&tl->s_free[grp][0]), s_addr = lanes + grp * 128 + col;
     unsigned pair_par = 0;    // phase of the barriers that complete once per pair with entries
     int staged = -1;          // Q buffer whose staged output may still be on its way out
     Ring ms, qs;
+    if constexpr (F::kStack == 2) {  // P of the keys that are not this row's stays zero
+        unsigned zero[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) zero[i] = 0;
+        tmem_st_32x32_issue(lanes + F::kPCol + grp * 64, zero);
+        tmem_st_32x32_issue(lanes + F::kPCol + grp * 64 + 32, zero);
+        tmem_st_wait();
+    }
     auto release_stage = [&]() {
         if (staged < 0) return;
         if (lane == 0) {
@@ -553,36 +567,36 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
     };
     for (int round = 0; nth_item(P, round) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 305)) return;
-        const Item &it = tl->m_item[ms.idx];
-        const int h = half ? it.h[1] : it.h[0], qb = half ? it.qb[1] : it.qb[0], b = it.b;
-        const int tq0 = qb * kBlk;  // (token numbers fit 32 bits: TMA coordinates)
-        const bool row_active = half < it.R && tq0 + mq < g.T;
+        const Item<F> &it = tl->m_item[ms.idx];
+        const int h = it.h[r_own], qb = it.qb[r_own], b = it.b;
+        const int tq0 = qb * F::kBlk;  // (token numbers fit 32 bits: TMA coordinates)
+        const bool row_active = r_own < it.R && tq0 + mq < g.T;
         const int key_end = row_active ? (g.causal ? tq0 + mq + 1 : (int)g.T) : 0;  // keys this token may attend: those before
         const int n_entries = tl->m_count[ms.idx], last_entry = max(n_entries - 1, 0);
-        const int *my_row = mask_rows(tl, P, ms.idx) + half * P.row_stride;  // this token's row of the pair
+        const int *my_row = mask_rows(tl, P, ms.idx) + r_own * P.row_stride;  // this token's row of the pair
         float ref = -CUDART_INF_F, l = 0.f;
         // the entry's key block of this token's row; the keys of it the token may attend, a prefix of n_hi
-        auto allowed_keys = [&](int blk) { return blk >= 0 ? max(0, min(key_end - blk * kBlk, kBlk)) : 0; };
+        auto allowed_keys = [&](int blk) { return blk >= 0 ? max(0, min(key_end - blk * F::kBlk, F::kBlk)) : 0; };
         int n_hi = allowed_keys(grp < n_entries ? my_row[grp] : -1);
-        bool masked = __any_sync(0xffffffffu, n_hi != kBlk);  // the diagonal block, one across T, a row without one
+        bool masked = __any_sync(0xffffffffu, n_hi != F::kBlk);  // the diagonal block, one across T, a row without one
         for (int n = grp; n < n_entries; n += 2) {  // entry n of a pair belongs to group n % 2
             // the token's 64 logits against its row's key block
             const unsigned sb = n_own & 1u, pb = n_own % F::kPBufs;  // the entry's logit and P buffers
             if (!wait_w(s_full + sb * 8, (n_own >> 1) & 1u, tl, 301)) return;
             tc_fence_after();
-            unsigned sr[64];
-            tmem_ld_32x32_issue(s_addr + sb * 64, sr);
-            tmem_ld_32x32_issue(s_addr + sb * 64 + 32, sr + 32);
+            unsigned sr[F::kBlk];
+#pragma unroll
+            for (int x = 0; x < F::kBlk / 32; ++x) tmem_ld_32x32_issue(s_addr + sb * 64 + 32 * x, sr + 32 * x);
             tmem_ld_wait();
             tc_fence_before();
             mbar_arrive_if(s_free + sb * 8, lane == 0);
             if (masked) {
 #pragma unroll
-                for (int i = 0; i < 64; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
+                for (int i = 0; i < F::kBlk; ++i) sr[i] = i < n_hi ? sr[i] : 0xff800000u;
             }
             // the pair's first entry sets the references of the tokens it has keys for
             if (n == 0) {
-                ref = max_of_64(reinterpret_cast<const float *>(sr));
+                ref = max_of<F::kBlk>(reinterpret_cast<const float *>(sr));
                 tl->ref[row] = ref;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&tl->ref_set[wq]));
@@ -599,7 +613,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
             const int next_blk = my_row[min(n + 2, last_entry)];  // (of no meaning behind the last)
             int next_hi = 0;
             const unsigned p_free = smem_u32(&tl->p_free[grp][pb]), p_par = ((n_own / F::kPBufs) & 1u) ^ 1u;
-            const unsigned p_addr = lanes + F::kPCol + grp * 64 + (F::kSplit ? 0 : pb * 32);
+            const unsigned p_addr = lanes + F::kPCol + grp * 64 + (F::kSplit ? 0 : pb * 32) + col / 2;
             unsigned packed[F::kSplit ? 16 : 32], rest[16];
             float esum;
             for (int attempt = 0;; ++attempt) {
@@ -637,7 +651,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
                     now = *(volatile float *)&tl->ref[row];
                 }
                 next_hi = allowed_keys(next_blk);
-                weights(32);
+                if constexpr (F::kBlk == 64) weights(32);
                 float e0, e1;
                 unpack_f32x2(add_f32x2(add_f32x2(sum2[0], sum2[1]), add_f32x2(sum2[2], sum2[3])), e0, e1);
                 esum = e0 + e1;
@@ -661,7 +675,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
                 if (__any_sync(0xffffffffu, move)) {
                     float f = 1.f;
                     if (move) {
-                        const float mx = max_of_64(reinterpret_cast<const float *>(sr));
+                        const float mx = max_of<F::kBlk>(reinterpret_cast<const float *>(sr));
                         if (ref != -CUDART_INF_F) f = fast_exp2((ref - mx) * P.scale_log2);
                         ref = mx;
                         tl->ref[row] = ref;
@@ -682,7 +696,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
             mbar_arrive_if(smem_u32(&tl->p_full[grp][pb]), lane == 0);
             ++n_own;
             n_hi = next_hi;
-            masked = __any_sync(0xffffffffu, n_hi != kBlk);
+            masked = __any_sync(0xffffffffu, n_hi != F::kBlk);
             release_stage();  // the previous pair's output has long been read
         }
         __syncwarp();
@@ -725,11 +739,12 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
             }
             fence_async_smem();
             __syncwarp();
-            const int h_1 = __shfl_sync(0xffffffffu, h, 16), tok_1 = __shfl_sync(0xffffffffu, tq0, 16) + wq * 16;
+            const int tok = tq0 + (mq & ~15);
+            const int h_1 = __shfl_sync(0xffffffffu, h, 16), tok_1 = __shfl_sync(0xffffffffu, tok, 16);
             const bool there_1 = __shfl_sync(0xffffffffu, (int)row_active, 16) != 0;
             if (lane == 0) {  // lanes 0 and 16 hold the first of the 16 tokens of a row
                 const unsigned src = smem_u32(stage + qs.idx * F::kOperand);
-                if (row_active) tma_store_4d(to, src, grp * (F::kD / 2), tq0 + wq * 16, h, b);
+                if (row_active) tma_store_4d(to, src, grp * (F::kD / 2), tok, h, b);
                 if (there_1) tma_store_4d(to, src + 16 * F::kOutBytes, grp * (F::kD / 2), tok_1, h_1, b);
                 tma_store_commit();
             }
@@ -754,7 +769,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = aligned_smem(smem_raw);
     // what is left behind the aligned base decides the number of V and K stages (the same in every thread)
-    const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail<F>) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
+    const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail<F>) + kMaskSlots * F::kRows * P.row_stride * (int)sizeof(int);
     const int n_rings = (P.smem_bytes - fixed_bytes) / F::kOperand - kFixedOperands;  // buffers for the two rings: d = 128: 4 or 5
     P.n_v_stages = min(F::kMaxVStages, (n_rings + 1) / 2);
     P.n_k_stages = min(F::kMaxKStages, n_rings - P.n_v_stages);
@@ -816,11 +831,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
 
 }  // namespace
 
-bool attn_tc_supported(const Geom &g, int dtype) { return g.d == 128 && attn_tc_auto(g, dtype); }
+bool attn_tc_supported(const Geom &g, int dtype) { return g.d == 128 && g.bq == 64 && attn_tc_auto(g, dtype); }
 
-// Against the mma.sync kernel at d = 64: FIGS
+// Against the mma.sync kernel, us: d = 64: 16 heads, 8192 tokens, k = 40, not causal: 600 -> 208; 6 heads, 12791
+// tokens, k = 5: 57 -> 33. Blocks of 32: 12 heads, 10007 tokens, d = 128, k = 8: 152 -> 72; 32
+// heads, 1416 tokens, d = 64, k = 60: 172 -> 96; 16 heads, 834 tokens, d = 128, k = 30: 51 -> 35.
 bool attn_tc_auto(const Geom &g, int dtype) {
-    return dtype == STREAM_BF16 && (g.d == 64 || g.d == 128) && g.bq == kBlk && g.bk == kBlk && g.k_top <= kMaxKTopTc && tma_strides_ok(g);
+    return dtype == STREAM_BF16 && (g.d == 64 || g.d == 128) && (g.bq == 32 || g.bq == 64) && g.bk == g.bq &&
+           g.k_top <= (g.bq == 64 ? kMaxKTopTc : kMaxKTopTc / 2) && tma_strides_ok(g);
 }
 
 namespace {
@@ -828,11 +846,11 @@ template <class F>
 stream_status launch(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
                      cudaStream_t st) {
     CUtensorMap tq, tk, tv, to;
-    stream_status rc = make_map_bf16(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q", kBlk, F::kD);  // 4-D: 64 x 64 half tiles
+    stream_status rc = make_map_bf16(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q", F::kBlk, F::kD);  // 4-D: a block of one channel half
     if (rc != STREAM_OK) return rc;
-    rc = make_map_bf16(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k", kBlk, F::kD);
+    rc = make_map_bf16(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k", F::kBlk, F::kD);
     if (rc != STREAM_OK) return rc;
-    rc = make_map5_bf16(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v", F::kD);
+    rc = make_map5_bf16(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v", F::kBlk, F::kD);
     if (rc != STREAM_OK) return rc;
     rc = make_map_bf16(&to, out, g.T, g.H, g.batch, F::kD, g.T * F::kD, (long long)g.H * g.T * F::kD, "out", 16, F::kD, F::kD / 2);
     if (rc != STREAM_OK) return rc;
@@ -841,7 +859,7 @@ stream_status launch(const Geom &g, const void *q, const void *k, const void *v,
     const long long kv_bytes = 2ll * g.T * F::kD * 2;  // K and V of one kv head
     const long long fit = kL2KvBytes / kv_bytes, all = (long long)g.batch * g.G;
     P.group_heads = (int)(fit < 1 ? 1 : (fit > all ? all : fit));
-    const long long n_items = all * ((g.n_qb + 1) / 2) * (2 * (g.hpg / 2) + g.hpg % 2);
+    const long long n_items = all * (((long long)g.n_qb * g.hpg + F::kRows - 1) / F::kRows);
     if (n_items > 0x7fffffffLL - (1 << 20)) { set_error("too many rows for 32-bit indexing"); return STREAM_ERR_UNSUPPORTED; }
     P.n_items = (int)n_items;
     P.mask = mask;
@@ -852,7 +870,7 @@ stream_status launch(const Geom &g, const void *q, const void *k, const void *v,
     // room for all ring buffers if the mask rows are short enough, else fewer, but four; 1 KB of slack for the alignment
     // of the base (the kernel counts its stages from what it really gets)
     P.row_stride = (g.k_top + 3) & ~3;
-    const int tail_bytes = (int)sizeof(Tail<F>) + kMaskSlots * 2 * P.row_stride * (int)sizeof(int);
+    const int tail_bytes = (int)sizeof(Tail<F>) + kMaskSlots * F::kRows * P.row_stride * (int)sizeof(int);
     int smem_bytes = (kFixedOperands + F::kMaxKStages + F::kMaxVStages) * F::kOperand + tail_bytes + 1024;
     if (smem_bytes > kMaxSmemPerCta) smem_bytes = kMaxSmemPerCta;
     if (smem_bytes < (kFixedOperands + 4) * F::kOperand + tail_bytes + 1024) {
@@ -877,7 +895,8 @@ stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const 
         set_error("tensor-core attention kernel needs 16-byte aligned q, k, v and out");
         return STREAM_ERR_UNSUPPORTED;
     }
-    return g.d == 128 ? launch<Form<128>>(g, q, k, v, mask, scale, out, st) : launch<Form<64>>(g, q, k, v, mask, scale, out, st);
+    if (g.bq == 64) return g.d == 128 ? launch<Form<128, 64>>(g, q, k, v, mask, scale, out, st) : launch<Form<64, 64>>(g, q, k, v, mask, scale, out, st);
+    return g.d == 128 ? launch<Form<128, 32>>(g, q, k, v, mask, scale, out, st) : launch<Form<64, 32>>(g, q, k, v, mask, scale, out, st);
 }
 
 stream_status read_attn_status(unsigned int out[2], cudaStream_t st) {

@@ -640,9 +640,9 @@ stream_status launch_attn_tok(const Geom &g, const void *q, const void *k, const
     CUtensorMap tq, tk, tv, to;
     stream_status rc = make_map_bf16_d128(&tq, q, g.T, g.H, g.batch, g.qs_t, g.qs_h, g.qs_b, "q", kTok);
     if (rc != STREAM_OK) return rc;
-    rc = make_map5_bf16(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k", 128);
+    rc = make_map5_bf16(&tk, k, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "k", 64, 128);
     if (rc != STREAM_OK) return rc;
-    rc = make_map5_bf16(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v", 128);
+    rc = make_map5_bf16(&tv, v, g.T, g.G, g.batch, g.ks_t, g.ks_h, g.ks_b, "v", 64, 128);
     if (rc != STREAM_OK) return rc;
     rc = make_map_bf16_d128(&to, out, g.T, g.H, g.batch, kD, g.T * kD, (long long)g.H * g.T * kD, "out", 32);
     if (rc != STREAM_OK) return rc;

@@ -474,18 +474,18 @@ inline stream_status make_map_bf16_d128(CUtensorMap *map, const void *base, long
 }
 
 // The same tensor seen as [batch, heads, channel halves, T, 64]: one box brings a whole
-// 64-token x d-channel tile as [half][64 rows][128 B], the layout of a 128-byte-swizzled
+// tile of box_rows tokens x d channels as [half][rows][128 B], the layout of a 128-byte-swizzled
 // K-major (or, read along the rows, MN-major) tcgen05 operand.
 // Coordinates: (0, token, head, 0, batch) with the half as dimension 3.
 inline stream_status make_map5_bf16(CUtensorMap *map, const void *base, long long T, int heads, int batch,
-                                    long long s_t, long long s_h, long long s_b, const char *what, int d) {
+                                    long long s_t, long long s_h, long long s_b, const char *what, int box_rows, int d) {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) { set_error("cuTensorMapEncodeTiled is not available from this driver"); return STREAM_ERR_CUDA; }
     if (heads == 1) s_h = s_t * T;
     if (batch == 1) s_b = s_h * heads;
     cuuint64_t dims[5] = {64, (cuuint64_t)T, (cuuint64_t)heads, (cuuint64_t)(d / 64), (cuuint64_t)batch};
     cuuint64_t strides[4] = {(cuuint64_t)s_t * 2, (cuuint64_t)s_h * 2, 128, (cuuint64_t)s_b * 2};
-    cuuint32_t box[5] = {64, 64, 1, (cuuint32_t)(d / 64), 1}, estr[5] = {1, 1, 1, 1, 1};
+    cuuint32_t box[5] = {64, (cuuint32_t)box_rows, 1, (cuuint32_t)(d / 64), 1}, estr[5] = {1, 1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

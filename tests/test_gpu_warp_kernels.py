@@ -37,6 +37,9 @@ CASES = [  # spec changes, block_q, block_k (None: the spec's block), causal
     (dict(d=128, T=9000, k_top=1, n_q_heads=2, n_kv_heads=1), 1, 64, True),  # (arbitrary masks) whole groups of tokens that keep nothing
     (dict(d=128, T=700, k_top=7, n_q_heads=3, n_kv_heads=1), 5, 64, False),  # rows that straddle 128 tokens
     (dict(d=128, T=33000, k_top=4, n_q_heads=1, n_kv_heads=1), 1, 64, True),  # two windows of 512 key blocks
+    (dict(block=64, T=1003, n_q_heads=3, n_kv_heads=1, k_top=7), None, None, True),   # attention on tcgen05, d = 64: a row alone in its pair
+    (dict(d=128, T=515, n_q_heads=7, n_kv_heads=1), None, None, True),                # blocks of 32: four rows across query blocks, three left over
+    (dict(d=128, T=515, n_q_heads=5, n_kv_heads=1, k_top=512), None, None, False),    # mask rows as long as they go with four to a unit
     (dict(dtype="f32", T=1003, n_q_heads=8), None, None, True),
     (dict(dtype="f32", T=515, d=128, k_top=40, block=16), None, None, True),
     (dict(dtype="f32", T=300, d=256, block=64, k_top=3), None, None, False),
