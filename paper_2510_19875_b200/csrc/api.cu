@@ -363,6 +363,12 @@ size_t stream_host_staging_bytes(const stream_problem *p) {
     return staging_layout(p, g).total;
 }
 
+// A chunk is 16 MB, but a fifth of the heads at most: a copy of one megabyte runs at two thirds of the link's
+// rate, one of 8 MB at 95 %, and a chunk's launches and events take the host 50 us (16 heads with their
+// own keys, 3998 tokens: head by head 1300 us, three at a time 1175; 3011 tokens: 1055 and 893). A last
+// head below 3 MB is not split (8 query heads, 2 kv heads, 1284 tokens: 208 and 180 us).
+constexpr size_t kChunkBytes = 16u << 20, kSplitBytes = 3u << 20;
+
 // Both host entry points: k_row_host == NULL is the fixed-k path.
 static stream_status run_host_impl(const stream_problem *p, const void *q_host, const void *k_host, const void *v_host,
                                    const int32_t *k_row_host, int32_t *mask_host, void *out_host, float scale, void *staging,
@@ -383,12 +389,12 @@ static stream_status run_host_impl(const stream_problem *p, const void *q_host, 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     char *base = (char *)staging;
     const size_t e = elem_size(p->dtype);
-    // One chunk = one kv head of one batch entry with its query heads: nothing else depends on it,
-    // so its copy in, its two kernels and its copy out can overlap with the neighbours'.
+    // One chunk = some kv heads (counted through the batch) with their query heads: nothing else depends
+    // on it, so its copy in, its two kernels and its copy out can overlap with the neighbours'.
     const size_t q_chunk = (size_t)g.hpg * g.T * g.d * e, kv_chunk = (size_t)g.T * g.d * e;
     const size_t m_chunk = (size_t)g.hpg * g.n_qb * g.k_top * sizeof(int32_t);
     stream_problem sub = *p;
-    sub.batch = 1; sub.n_q_heads = g.hpg; sub.n_kv_heads = 1;
+    sub.batch = 1;
     cudaError_t ce;
 #define STREAM_TRY(call, what) do { if ((ce = (call)) != cudaSuccess) return cuda_fail(ce, what); } while (0)
     // the internal streams start after everything already enqueued on the caller's stream
@@ -400,26 +406,34 @@ static stream_status run_host_impl(const stream_problem *p, const void *q_host, 
         STREAM_TRY(cudaMemcpyAsync(base + s.k_row, k_row_host, (size_t)g.n_qb * sizeof(int32_t), cudaMemcpyHostToDevice, hp->in), "H2D k_row");
         k_row_dev = (const int32_t *)(base + s.k_row);
     }
-    const int n_chunks = g.batch * g.G;
+    const int n_heads = g.batch * g.G;
     const size_t q_head = (size_t)g.T * g.d * e, m_head = (size_t)g.n_qb * g.k_top * sizeof(int32_t);
+    const size_t head_in = q_chunk + 2 * kv_chunk;
+    const int want = (int)((kChunkBytes + head_in - 1) / head_in), most = n_heads / 5;
+    const int per_chunk = want < most ? want : (most > 1 ? most : 1);
     int unit = 0;  // running number of the (chunk, heads) units, for the ring of events
-    for (int c = 0; c < n_chunks; ++c) {
+    for (int c = 0, take; c < n_heads; c += take) {
+        const int left = n_heads - c;
+        take = left > per_chunk ? per_chunk : left;
+        // The very last head goes through in two halves of its query heads, if they are not small: what
+        // is left after the last byte has arrived (its kernels and its copy out, which nothing overlaps
+        // any more) is then half as long. Everywhere else the query heads of a kv head stay together,
+        // so that the first level's key tiles serve as many rows as possible.
+        if (take == left && left > 1) take = (left + 1) / 2;
         const size_t ko = (size_t)c * kv_chunk;
-        // The very last chunk goes through in two halves of its query heads: what is left after the
-        // last byte has arrived (its kernels and its copy out, which nothing overlaps any more) is
-        // then half as long. Everywhere else a chunk keeps all its heads together, so that the
-        // first level's key tiles serve as many rows as possible.
-        const int n_units = (c == n_chunks - 1 && g.hpg >= 4) ? 2 : 1;
+        const int n_units = left == 1 && g.hpg >= 4 && head_in >= kSplitBytes ? 2 : 1;
+        const int heads = take * g.hpg;
+        sub.n_kv_heads = take;
         for (int u = 0; u < n_units; ++u, ++unit) {
-            const int h0 = u * ((g.hpg + n_units - 1) / n_units);
-            const int nh = (u == n_units - 1) ? g.hpg - h0 : (g.hpg + n_units - 1) / n_units;
+            const int h0 = u * ((heads + n_units - 1) / n_units);
+            const int nh = (u == n_units - 1) ? heads - h0 : (heads + n_units - 1) / n_units;
             const size_t qo = (size_t)c * q_chunk + (size_t)h0 * q_head, mo = (size_t)c * m_chunk + (size_t)h0 * m_head;
             const size_t q_bytes = (size_t)nh * q_head, m_bytes = (size_t)nh * m_head;
             sub.n_q_heads = nh;
             cudaEvent_t in_done = hp->in_done[unit % kPipeEvents], comp_done = hp->comp_done[unit % kPipeEvents];
             if (u == 0) {
-                STREAM_TRY(cudaMemcpyAsync(base + s.k + ko, (const char *)k_host + ko, kv_chunk, cudaMemcpyHostToDevice, hp->in), "H2D k");
-                STREAM_TRY(cudaMemcpyAsync(base + s.v + ko, (const char *)v_host + ko, kv_chunk, cudaMemcpyHostToDevice, hp->in), "H2D v");
+                STREAM_TRY(cudaMemcpyAsync(base + s.k + ko, (const char *)k_host + ko, (size_t)take * kv_chunk, cudaMemcpyHostToDevice, hp->in), "H2D k");
+                STREAM_TRY(cudaMemcpyAsync(base + s.v + ko, (const char *)v_host + ko, (size_t)take * kv_chunk, cudaMemcpyHostToDevice, hp->in), "H2D v");
             }
             STREAM_TRY(cudaMemcpyAsync(base + s.q + qo, (const char *)q_host + qo, q_bytes, cudaMemcpyHostToDevice, hp->in), "H2D q");
             STREAM_TRY(cudaEventRecord(in_done, hp->in), "cudaEventRecord");

@@ -133,3 +133,22 @@ def test_masks_on_tcgen05_beyond_four_heads_and_32_blocks(S, kw, causal):
     w = wl.generate(spec)
     rows = None if spec.n_rows <= 600 else np.unique(np.random.default_rng(1).choice(spec.n_rows, 500, replace=False))
     assert_mask_parity(S, w, rows, score_cache=False, causal=causal)
+
+
+@pytest.mark.parametrize("kw", [dict(n_q_heads=8, n_kv_heads=8, batch=2, T=300),      # three kv heads to a chunk, across the batch; the last one alone
+                                dict(n_q_heads=11, n_kv_heads=11, T=2001, dtype="f32", d=64, block=32)])
+def test_run_host_with_several_kv_heads_to_a_chunk(S, kw):
+    spec = wl.WorkloadSpec(**{**dict(name="w", seed=8, batch=1, T=700, d=128, block=64, k_top=5, dtype="bf16"), **kw})
+    q, k, v = wl.generate(spec).torch_tensors("cpu")
+    qh, kh, vh = (x.contiguous().pin_memory() for x in (q, k, v))
+    mask = torch.empty(spec.batch, spec.n_q_heads, spec.n_blocks, spec.k_top, dtype=torch.int32, pin_memory=True)
+    out = torch.empty_like(qh).pin_memory()
+    blocks = dict(block_q=spec.block, block_k=spec.block)
+    p = S.make_problem(qh, kh, k_top=spec.k_top, **blocks)
+    staging = torch.empty(S.stream_host_staging_bytes(p), dtype=torch.uint8, device="cuda")
+    S.run_host(qh, kh, vh, mask, out, staging, k_top=spec.k_top, **blocks)
+    torch.cuda.synchronize()
+    q, k, v = q.cuda(), k.cuda(), v.cuda()
+    ref = S.build_mask(q, k, k_top=spec.k_top, **blocks).mask
+    assert torch.equal(mask, ref.cpu())
+    assert (out.float() - S.sparse_attention(q, k, v, ref, **blocks).float().cpu()).abs().max().item() <= TOL[spec.dtype]
