@@ -52,7 +52,9 @@ struct Tail {
     int item;            // the group being worked on
     int n_list;          // blocks in the current level's list
     int n_nodes[kTok];   // surviving nodes per token
-    int n_tiles[kTok];   // tiles the token has needed so far (its own candidates, not the merged list)
+    int n_tiles[kTok];   // tiles the token has needed so far (a warp's ranking keeps them here)
+    unsigned node0[32];  // the initial nodes (the same for every token), and of the group: the places of
+    unsigned place0[32]; // their left | right << 16 candidates in the first level's list
 };
 
 // Dynamic shared memory behind the 1024-byte aligned base:
@@ -82,6 +84,22 @@ __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail *tl, 
 
 __device__ __forceinline__ unsigned pack_node(int f, int len) { return (unsigned)f | ((unsigned)len << 16); }
 
+// Sorts n keys of a thread, largest first (Batcher's odd-even merge sort, unrolled: n = 32: 191
+// exchanges, 64: 543).
+template <int n, int P, int K>
+__device__ __forceinline__ void sort_step(unsigned (&key)[n]) {
+#pragma unroll
+    for (int x = 0; x + K < n; ++x)
+        if (x >= K % P && ((x - K % P) & (2 * K - 1)) < K && x / (2 * P) == (x + K) / (2 * P)) {
+            const unsigned a = key[x], b = key[x + K];
+            key[x] = max(a, b);
+            key[x + K] = min(a, b);
+        }
+    if constexpr (K > 1) sort_step<n, P, K / 2>(key);
+    else if constexpr (2 * P < n) sort_step<n, 2 * P, 2 * P>(key);
+}
+
+template <int kNodes>  // of a token, at most: 16 or 32
 __global__ void __launch_bounds__(kThreads, 1)
 mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, Params P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -113,6 +131,15 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     tc_fence_after();
     const unsigned tmem_base = tl->tmem_base;
 
+    // the level's wanted blocks: a byte each while they fit (plain stores, the same value from all), else a bit
+    unsigned char *const wanted = (unsigned char *)bitmap;
+    const bool bytes = g.N_k <= kBitmapBytes;
+    auto want = [&](int blk) {
+        if (bytes) wanted[blk] = 1;
+        else atomicOr(&bitmap[blk >> 5], 1u << (blk & 31));
+    };
+    constexpr bool kSorted = kNodes == 16;
+
     // role of this warp inside a level
     const bool is_producer = warp == 0;
     const int mma_which = warp == 1 ? 0 : (warp == 3 ? 1 : -1);            // issues the stages with this parity
@@ -120,9 +147,13 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int epi_tok = (warp & 3) * 32 + lane;                            // its token (TMEM lane)
 
     const int kq = g.k_top, levels = g.levels;
+    if (tid < 32) {
+        const int f = (int)(((long long)tid * g.N_k) / kq), end = (int)(((long long)(tid + 1) * g.N_k) / kq);
+        tl->node0[tid] = tid < kq && f < end ? pack_node(f, end - f) : 0u;
+    }
     unsigned seq = 0;     // stages so far over the whole kernel (the same in every thread)
     unsigned q_par = 0;
-    unsigned long long tiles_needed = 0, products = 0;  // per warp (lane 0 adds them up at the end)
+    unsigned long long tiles_needed = 0, products = 0;  // per thread
 
     for (;;) {
         if (tid == 0) tl->item = (int)atomicAdd(&P.ws->work_counter, 1u);
@@ -154,12 +185,15 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         if (warp == 0) {
             if (gl) list[pos_l0] = (unsigned short)f0;
             if (gr) list[pos_r0] = (unsigned short)(m0 + 1);
+            tl->place0[lane] = (unsigned)pos_l0 | ((unsigned)pos_r0 << 16);
             if (lane == 0) tl->n_list = __popc(bl) + __popc(br);
         }
         // the token this thread reads accumulators for
         const long long e_tq = tok0 + epi_tok;
         const bool e_ok = epi_grp >= 0 && e_tq < g.T;
         const int e_qlim = e_ok ? last_valid_block(g, (int)e_tq) : -1;
+        const int key_end = e_ok ? (int)(g.causal ? e_tq + 1 : g.T) : 0;  // keys the token may look at: those before
+        unsigned n_tiles = 0;  // tiles the token has needed so far (its own candidates, not the merged list)
 
         for (int level = 0; level < levels; ++level) {
             __syncthreads();  // the level's list is complete; the ranking of the level before is done
@@ -207,55 +241,53 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     __syncwarp();
                 }
             } else if (epi_grp >= 0) {
-                int cur = 0;  // cursor over this token's nodes (their right branches ascend with the list)
-                const int n_nodes = level > 0 ? tl->n_nodes[epi_tok] : 0;
+                // This token's next candidate: at the first level every allowed block of the list, later the
+                // right branches of its nodes, which ascend with the list: of node `cur`, block `due`.
+                const int n_nodes = level > 0 && e_ok ? tl->n_nodes[epi_tok] : 0;
+                int cur = -1, due = -1;
+                auto advance = [&]() {
+                    due = -1;
+                    while (++cur < n_nodes) {
+                        const unsigned nd = nodes[cur * kPad + epi_tok];
+                        const int f = (int)(nd & 0xffffu), len = (int)(nd >> 16), rb = (2 * f + len - 1) / 2 + 1;
+                        if (len > 1 && rb <= e_qlim) { due = rb; break; }
+                    }
+                };
+                if (level > 0) advance();
                 for (int i = 0; i < n_st; ++i) {
                     const unsigned s = seq + (unsigned)i, buf = s & 3u;
-                    if ((int)(s & 1u) != epi_grp) continue;
+                    // the other group's stage: its blocks are passed over
+                    const int blk2[2] = {list[2 * i], 2 * i + 1 < n_list ? list[2 * i + 1] : 0x7fff0000};
+                    if ((int)(s & 1u) != epi_grp) {
+                        while (level > 0 && due >= 0 && due <= blk2[1]) advance();
+                        continue;
+                    }
                     if (!wait_w(smem_u32(&tl->tmem_full[buf]), (s >> 2) & 1u, tl, P.ws, 605)) break;
                     tc_fence_after();
 #pragma unroll
                     for (int tile = 0; tile < 2; ++tile) {
-                        const int idx = 2 * i + tile;
-                        if (idx >= n_list) break;  // (uniform)
-                        const int blk = list[idx];
-                        int pos = -1;  // where this token keeps the tile's score, if it is one of its candidates
-                        if (level == 0) {
-                            if (e_ok && blk <= e_qlim) pos = idx;
-                        } else if (e_ok) {
-                            while (cur < n_nodes) {
-                                const unsigned nd = nodes[cur * kPad + epi_tok];
-                                const int f = (int)(nd & 0xffffu), len = (int)(nd >> 16);
-                                const int rb = (f + f + len - 1) / 2 + 1;
-                                if (len > 1 && rb <= e_qlim) {
-                                    if (rb == blk) pos = 32 + cur;
-                                    if (rb >= blk) break;
-                                }
-                                ++cur;
-                            }
-                            if (pos >= 0) ++cur;
-                        }
-                        if (__any_sync(0xffffffffu, pos >= 0)) {
-                            const unsigned taddr = tmem_base + buf * 128 + tile * 64 + ((unsigned)((warp & 3) * 32) << 16);
-                            float v[64];
-                            tmem_ld_32x32(taddr, v);
-                            tmem_ld_32x32(taddr + 32, v + 32);
-                            // keys of the block this token may look at: a prefix (inside T, not after the token if causal)
-                            const long long k0 = (long long)blk * kBlk;
-                            long long lim = g.T - k0;
-                            if (g.causal) lim = min(lim, e_tq - k0 + 1);
-                            const int n_hi = (int)max(0ll, min(lim, (long long)kBlk));
-                            if (n_hi != kBlk) {  // the token's own block, or a block across T
+                        const int blk = blk2[tile];
+                        const bool mine = level == 0 ? blk <= e_qlim : blk == due;
+                        if (!__any_sync(0xffffffffu, mine)) continue;  // (a place behind the list is nobody's)
+                        const unsigned taddr = tmem_base + buf * 128 + tile * 64 + ((unsigned)((warp & 3) * 32) << 16);
+                        unsigned v[64];
+                        tmem_ld_32x32_issue(taddr, v);
+                        tmem_ld_32x32_issue(taddr + 32, v + 32);
+                        // (while they are on their way:) where this token keeps the tile's score, what comes next
+                        const int pos = level == 0 ? 2 * i + tile : 32 + cur;
+                        if (mine && level > 0) advance();
+                        // keys of the block this token may look at: a prefix (inside T, not after the token if causal)
+                        const int n_hi = key_end - blk * kBlk;
+                        tmem_ld_wait();
+                        if (__any_sync(0xffffffffu, mine && n_hi < kBlk)) {  // the token's own block, or a block across T
 #pragma unroll
-                                for (int j = 0; j < 64; ++j) v[j] = j < n_hi ? v[j] : -CUDART_INF_F;
-                            }
-                            const float best = max_of_64(v);
-                            if (pos >= 0) scores[pos * kPad + epi_tok] = best;
+                            for (int j = 0; j < 64; ++j) v[j] = j < n_hi ? v[j] : 0xff800000u;
                         }
+                        const float best = max_of_64(reinterpret_cast<const float *>(v));
+                        if (mine) scores[pos * kPad + epi_tok] = best;
                     }
                     tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&tl->tmem_empty[buf]));
+                    mbar_arrive_if(smem_u32(&tl->tmem_empty[buf]), lane == 0);
                 }
             }
             seq += (unsigned)n_st;
@@ -263,8 +295,82 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             __syncthreads();  // every score of the level is in place
             if (*(volatile int *)&tl->abort_flag) break;  // (set only inside the level: the same answer in every thread)
 
-            // ---- ranking: every warp takes eight tokens; lane j holds node j of the token ----
+            // ---- ranking. Up to 16 nodes: a thread per token (the first epilogue group's), which sorts its keys
+            // in registers, 32 tokens a warp at once. More do not fit in registers: a warp per token, a
+            // lane per node, which spends 240 instructions of a warp on every token, 8000 clocks a level of
+            // the 128 against 3000. (32 / 8 heads, 4096 tokens: k = 16 225 us that way, 160 this way; k = 24,
+            // spilled, 304 this way, 224 that way.)
             const bool last = level + 1 == levels;
+            if constexpr (kSorted) {
+            if (epi_grp == 0) {
+                const int t = epi_tok;
+                const int n = !e_ok ? 0 : (level == 0 ? kq : tl->n_nodes[t]);
+                // Everything of the token goes to registers first: its nodes, and the keys of their left and
+                // right candidates (0: there is none).
+                unsigned nd[kNodes], own[2 * kNodes], key[2 * kNodes];
+#pragma unroll
+                for (int j = 0; j < kNodes; ++j) {
+                    nd[j] = 0u;
+                    unsigned at = (unsigned)j | ((unsigned)(32 + j) << 16);
+                    if (level == 0) { nd[j] = tl->node0[j]; at = tl->place0[j]; }
+                    else if (j < n) nd[j] = nodes[j * kPad + t];
+                    const int f = (int)(nd[j] & 0xffffu), len = (int)(nd[j] >> 16), rb = (2 * f + len - 1) / 2 + 1;
+                    const bool vl = j < n && len > 0 && f <= e_qlim, vr = vl && len > 1 && rb <= e_qlim;
+                    own[2 * j] = vl ? __float_as_uint(scores[(at & 0xffffu) * kPad + t]) : 0u;
+                    own[2 * j + 1] = vr ? __float_as_uint(scores[(at >> 16) * kPad + t]) : 0u;
+                    key[2 * j] = score_key(vl, __uint_as_float(own[2 * j]));
+                    key[2 * j + 1] = score_key(vr, __uint_as_float(own[2 * j + 1]));
+                    if (level == 0) n_tiles += (vl ? 1u : 0u) + (vr ? 1u : 0u);
+                }
+                // The k-th largest key, always in the same place of the sorted ones: kNodes - k places that
+                // no candidate can have are taken by keys above all others.
+                unsigned valid_l = 0u, valid_r = 0u;  // (bit j: of node j)
+#pragma unroll
+                for (int j = 0; j < kNodes; ++j) {
+                    valid_l |= (key[2 * j] != 0u ? 1u : 0u) << j;
+                    valid_r |= (key[2 * j + 1] != 0u ? 1u : 0u) << j;
+                    if (j >= kq) key[2 * j] = 0xffffffffu;
+                }
+                sort_step<2 * kNodes, 1, 1>(key);
+                const unsigned thr = key[kNodes - 1];
+                int missing = kNodes;  // (counting the places taken)
+#pragma unroll
+                for (int i = 0; i < kNodes - 1; ++i) missing -= key[i] > thr ? 1 : 0;
+                // what is kept, in order, to its place (nothing is left to be read there)
+                unsigned n_new = 0u;
+#pragma unroll
+                for (int j = 0; j < kNodes; ++j) {
+                    const int f = (int)(nd[j] & 0xffffu), len = (int)(nd[j] >> 16), rb = (2 * f + len - 1) / 2 + 1;
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const bool valid = ((x ? valid_r : valid_l) >> j) & 1u;
+                        const unsigned k = score_key(valid, __uint_as_float(own[2 * j + x]));
+                        const bool equal = valid && k == thr && missing > 0;
+                        missing -= equal ? 1 : 0;
+                        if (equal || (valid && k > thr)) {
+                            nodes[n_new * kPad + t] = x ? pack_node(rb, f + len - rb) : pack_node(f, rb - f);
+                            scores[n_new * kPad + t] = __uint_as_float(own[2 * j + x]);
+                            ++n_new;
+                        }
+                    }
+                }
+                tl->n_nodes[t] = (int)n_new;
+                if (!last) {  // the token's candidates of the next level: the right branch of every node that has one
+#pragma unroll
+                    for (int j = 0; j < kNodes; ++j) {
+                        const unsigned x = j < (int)n_new ? nodes[j * kPad + t] : 0u;
+                        const int f = (int)(x & 0xffffu), len = (int)(x >> 16), rb = (2 * f + len - 1) / 2 + 1;
+                        if (len > 1 && rb <= e_qlim) {
+                            ++n_tiles;
+                            want(rb);
+                        }
+                    }
+                } else if (e_ok) {
+                    tiles_needed += n_tiles;
+                    if (g.row_tiles != nullptr) g.row_tiles[((long long)b * g.H + h) * g.n_qb + e_tq] = n_tiles;
+                }
+            }
+            } else {
             for (int i = 0; i < kTok / (kThreads / 32); ++i) {
                 const int t = warp * (kTok / (kThreads / 32)) + i;
                 const long long tq = tok0 + t;
@@ -305,18 +411,26 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     // the token's candidates of the next level: the right branch of every node that has one
                     const int rb = (nf + nf + nlen - 1) / 2 + 1;
                     const bool has_r = live && nlen > 1 && rb <= q_lim;
-                    if (has_r) atomicOr(&bitmap[rb >> 5], 1u << (rb & 31));
+                    if (has_r) want(rb);
                     const unsigned hb = __ballot_sync(0xffffffffu, has_r);
                     if (lane == 0) { tiles_needed += (unsigned long long)__popc(hb); tl->n_tiles[t] += __popc(hb); }
                 } else {
-                    // emit I[token, :]: first block of every surviving node, ascending, -1 padded
+                    if (lane == 0 && g.row_tiles != nullptr) g.row_tiles[((long long)b * g.H + h) * g.n_qb + tq] = (unsigned)tl->n_tiles[t];
+                }
+            }
+            }
+            if (last) {  // emit I[token, :]: first block of every surviving node, ascending, -1 padded
+                __syncthreads();
+                for (int i = 0; i < kTok / (kThreads / 32); ++i) {
+                    const int t = warp * (kTok / (kThreads / 32)) + i;
+                    const long long tq = tok0 + t;
+                    if (tq >= g.T) break;  // (uniform) tokens beyond T: no row
+                    const bool live = lane < tl->n_nodes[t];
                     const long long o = (((long long)b * g.H + h) * g.n_qb + tq) * g.k_top;
                     if (lane < g.k_top) {
-                        P.mask[o + lane] = live ? nf : -1;
+                        P.mask[o + lane] = live ? (int)(nodes[lane * kPad + t] & 0xffffu) : -1;
                         if (P.score != nullptr) P.score[o + lane] = live ? scores[lane * kPad + t] : -CUDART_INF_F;
                     }
-                    if (g.row_tiles != nullptr && lane == 0)
-                        g.row_tiles[((long long)b * g.H + h) * g.n_qb + tq] = (unsigned)tl->n_tiles[t];
                 }
             }
             if (last) break;
@@ -326,8 +440,18 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 const int n_words = (g.N_k + 31) >> 5;
                 for (int w0 = 0; w0 < n_words; w0 += 32) {
                     const int w = w0 + lane;
-                    unsigned bits = w < n_words ? bitmap[w] : 0u;
-                    if (w < n_words) bitmap[w] = 0u;
+                    unsigned bits = 0u;
+                    if (bytes && w < n_words) {
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            const unsigned y = bitmap[8 * w + x];
+                            bitmap[8 * w + x] = 0u;
+                            bits |= ((y & 1u) | ((y >> 7) & 2u) | ((y >> 14) & 4u) | ((y >> 21) & 8u)) << (4 * x);
+                        }
+                    } else if (w < n_words) {
+                        bits = bitmap[w];
+                        bitmap[w] = 0u;
+                    }
                     const int cnt = __popc(bits);
                     int incl = cnt;
 #pragma unroll
@@ -349,6 +473,8 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         if (*(volatile int *)&tl->abort_flag) break;
         if (warp == 0 && lane == 0) atomicAdd(&P.ws->rows, (unsigned long long)(tq_max - tok0 + 1));
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tiles_needed += __shfl_xor_sync(0xffffffffu, tiles_needed, o);
     if (lane == 0 && (tiles_needed | products) != 0ull) {
         atomicAdd(&P.ws->tiles_scored, tiles_needed);
         atomicAdd(&P.ws->tile_products, products);
@@ -395,10 +521,11 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     P.mask = mask; P.score = score; P.ws = ws;
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    cudaError_t e = cudaFuncSetAttribute(mask_tok_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    auto kern = g.k_top <= 16 ? mask_tok_kernel<16> : mask_tok_kernel<32>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tok)");
     const int grid = (int)(n_items < n_sm ? n_items : n_sm);
-    mask_tok_kernel<<<grid, kThreads, kSmemBytes, st>>>(tq, tk, P);
+    kern<<<grid, kThreads, kSmemBytes, st>>>(tq, tk, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "mask_tok launch");
     return STREAM_OK;
