@@ -61,7 +61,8 @@ struct Tail {
 //   Q tile | key-pair stages | scores [64][kPad] f32 | nodes [32][kPad] u32 | list u16 | bitmap u32 | Tail
 // scores rows 0..31: score of a token's node j (its first allowed block); rows 32..63: score of
 // node j's right branch at the current level. At the first level the 64 rows hold the scores of
-// the (shared) list positions instead. nodes: first block | (blocks in the node << 16).
+// the (shared) list positions instead. nodes: first block | (blocks in the node << 16). With up
+// to 16 nodes rows 16..31 hold the token's candidates of the level instead: block | (its node << 16).
 constexpr int kScoresBytes = 64 * kPad * 4, kNodesBytes = 32 * kPad * 4, kListBytes = kMaxList * 2, kBitmapBytes = kMaxNk / 8;
 constexpr int kSmemBytes = kQBytes + kStages * kStageBytes + kScoresBytes + kNodesBytes + kListBytes + kBitmapBytes +
                            (int)sizeof(Tail) + 1024;
@@ -69,6 +70,8 @@ static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 
 constexpr unsigned kDescHi = desc_hi_sw128(1024);            // K-major, 8-row groups 1024 bytes apart
 constexpr unsigned kIdesc = idesc_bf16(128, 128, false);     // D fp32, A and B bf16 K-major, M = N = 128
+
+constexpr unsigned kNoBlock = 0xffffu;  // (behind every block)
 
 struct Params {
     Geom g;
@@ -83,6 +86,10 @@ __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail *tl, 
 }
 
 __device__ __forceinline__ unsigned pack_node(int f, int len) { return (unsigned)f | ((unsigned)len << 16); }
+// First block of a node's right half (of its left half, for a node of one block the one behind it).
+__device__ __forceinline__ int right_of(unsigned node) { return (int)(((2u * (node & 0xffffu) + (node >> 16) - 1u) >> 1) + 1u); }
+// The score whose score_key this is.
+__device__ __forceinline__ float score_of_key(unsigned key) { return __uint_as_float(key ^ ((key & 0x80000000u) ? 0x80000000u : 0xffffffffu)); }
 
 // Sorts n keys of a thread, largest first (Batcher's odd-even merge sort, unrolled: n = 32: 191
 // exchanges, 64: 543).
@@ -242,24 +249,37 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 }
             } else if (epi_grp >= 0) {
                 // This token's next candidate: at the first level every allowed block of the list, later the
-                // right branches of its nodes, which ascend with the list: of node `cur`, block `due`.
+                // right branches of its nodes, which ascend with the list: block due & 0xffff, of node
+                // due >> 16. (From a ranked token's own list the one behind it is always on its way.)
                 const int n_nodes = level > 0 && e_ok ? tl->n_nodes[epi_tok] : 0;
-                int cur = -1, due = -1;
-                auto advance = [&]() {
-                    due = -1;
-                    while (++cur < n_nodes) {
-                        const unsigned nd = nodes[cur * kPad + epi_tok];
-                        const int f = (int)(nd & 0xffffu), len = (int)(nd >> 16), rb = (2 * f + len - 1) / 2 + 1;
-                        if (len > 1 && rb <= e_qlim) { due = rb; break; }
+                int cur = -1;
+                unsigned due = kNoBlock, next = kNoBlock;
+                auto read_next = [&]() {
+                    ++cur;
+                    if constexpr (kSorted) {
+                        next = cur < kNodes && n_nodes > 0 ? nodes[(kNodes + cur) * kPad + epi_tok] : kNoBlock;
+                    } else {
+                        for (next = kNoBlock; cur < n_nodes; ++cur) {
+                            const unsigned nd = nodes[cur * kPad + epi_tok];
+                            if ((nd >> 16) > 1u && right_of(nd) <= e_qlim) { next = (unsigned)right_of(nd) | ((unsigned)cur << 16); break; }
+                        }
                     }
                 };
-                if (level > 0) advance();
+                auto advance = [&]() {
+                    if (kSorted) due = next;
+                    if (!kSorted || (due & 0xffffu) != kNoBlock) read_next();
+                    if (!kSorted) due = next;
+                };
+                if (level > 0) {
+                    if (kSorted) read_next();
+                    advance();
+                }
                 for (int i = 0; i < n_st; ++i) {
                     const unsigned s = seq + (unsigned)i, buf = s & 3u;
                     // the other group's stage: its blocks are passed over
-                    const int blk2[2] = {list[2 * i], 2 * i + 1 < n_list ? list[2 * i + 1] : 0x7fff0000};
+                    const int blk2[2] = {list[2 * i], 2 * i + 1 < n_list ? list[2 * i + 1] : (int)kNoBlock - 1};
                     if ((int)(s & 1u) != epi_grp) {
-                        while (level > 0 && due >= 0 && due <= blk2[1]) advance();
+                        while ((int)(due & 0xffffu) <= blk2[1]) advance();
                         continue;
                     }
                     if (!wait_w(smem_u32(&tl->tmem_full[buf]), (s >> 2) & 1u, tl, P.ws, 605)) break;
@@ -267,14 +287,14 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
                     for (int tile = 0; tile < 2; ++tile) {
                         const int blk = blk2[tile];
-                        const bool mine = level == 0 ? blk <= e_qlim : blk == due;
+                        const bool mine = level == 0 ? blk <= e_qlim : blk == (int)(due & 0xffffu);
                         if (!__any_sync(0xffffffffu, mine)) continue;  // (a place behind the list is nobody's)
                         const unsigned taddr = tmem_base + buf * 128 + tile * 64 + ((unsigned)((warp & 3) * 32) << 16);
                         unsigned v[64];
                         tmem_ld_32x32_issue(taddr, v);
                         tmem_ld_32x32_issue(taddr + 32, v + 32);
                         // (while they are on their way:) where this token keeps the tile's score, what comes next
-                        const int pos = level == 0 ? 2 * i + tile : 32 + cur;
+                        const int pos = level == 0 ? 2 * i + tile : 32 + (int)(due >> 16);
                         if (mine && level > 0) advance();
                         // keys of the block this token may look at: a prefix (inside T, not after the token if causal)
                         const int n_hi = key_end - blk * kBlk;
@@ -310,61 +330,55 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 unsigned nd[kNodes], own[2 * kNodes], key[2 * kNodes];
 #pragma unroll
                 for (int j = 0; j < kNodes; ++j) {
-                    nd[j] = 0u;
                     unsigned at = (unsigned)j | ((unsigned)(32 + j) << 16);
-                    if (level == 0) { nd[j] = tl->node0[j]; at = tl->place0[j]; }
-                    else if (j < n) nd[j] = nodes[j * kPad + t];
-                    const int f = (int)(nd[j] & 0xffffu), len = (int)(nd[j] >> 16), rb = (2 * f + len - 1) / 2 + 1;
-                    const bool vl = j < n && len > 0 && f <= e_qlim, vr = vl && len > 1 && rb <= e_qlim;
-                    own[2 * j] = vl ? __float_as_uint(scores[(at & 0xffffu) * kPad + t]) : 0u;
-                    own[2 * j + 1] = vr ? __float_as_uint(scores[(at >> 16) * kPad + t]) : 0u;
-                    key[2 * j] = score_key(vl, __uint_as_float(own[2 * j]));
-                    key[2 * j + 1] = score_key(vr, __uint_as_float(own[2 * j + 1]));
-                    if (level == 0) n_tiles += (vl ? 1u : 0u) + (vr ? 1u : 0u);
+                    if (level == 0) { nd[j] = j < n ? tl->node0[j] : 0u; at = tl->place0[j]; }
+                    else nd[j] = j < n ? nodes[j * kPad + t] : 0u;
+                    const bool vl = nd[j] != 0u && (int)(nd[j] & 0xffffu) <= e_qlim, vr = (nd[j] >> 16) > 1u && right_of(nd[j]) <= e_qlim;
+                    own[2 * j] = score_key(vl, vl ? scores[(at & 0xffffu) * kPad + t] : 0.f);
+                    own[2 * j + 1] = score_key(vr, vr ? scores[(at >> 16) * kPad + t] : 0.f);
+                }
+                if (level == 0) {
+#pragma unroll
+                    for (int i = 0; i < 2 * kNodes; ++i) n_tiles += own[i] != 0u ? 1u : 0u;
                 }
                 // The k-th largest key, always in the same place of the sorted ones: kNodes - k places that
                 // no candidate can have are taken by keys above all others.
-                unsigned valid_l = 0u, valid_r = 0u;  // (bit j: of node j)
 #pragma unroll
-                for (int j = 0; j < kNodes; ++j) {
-                    valid_l |= (key[2 * j] != 0u ? 1u : 0u) << j;
-                    valid_r |= (key[2 * j + 1] != 0u ? 1u : 0u) << j;
-                    if (j >= kq) key[2 * j] = 0xffffffffu;
-                }
+                for (int i = 0; i < 2 * kNodes; ++i) key[i] = i % 2 == 0 && i / 2 >= kq ? 0xffffffffu : own[i];
                 sort_step<2 * kNodes, 1, 1>(key);
                 const unsigned thr = key[kNodes - 1];
-                int missing = kNodes;  // (counting the places taken)
+                int above[4] = {0, 0, 0, 0};  // (counting the places taken)
 #pragma unroll
-                for (int i = 0; i < kNodes - 1; ++i) missing -= key[i] > thr ? 1 : 0;
+                for (int i = 0; i < kNodes - 1; ++i) above[i & 3] += key[i] > thr ? 1 : 0;
+                int missing = kNodes - (above[0] + above[1]) - (above[2] + above[3]);
                 // what is kept, in order, to its place (nothing is left to be read there)
                 unsigned n_new = 0u;
 #pragma unroll
-                for (int j = 0; j < kNodes; ++j) {
-                    const int f = (int)(nd[j] & 0xffffu), len = (int)(nd[j] >> 16), rb = (2 * f + len - 1) / 2 + 1;
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        const bool valid = ((x ? valid_r : valid_l) >> j) & 1u;
-                        const unsigned k = score_key(valid, __uint_as_float(own[2 * j + x]));
-                        const bool equal = valid && k == thr && missing > 0;
-                        missing -= equal ? 1 : 0;
-                        if (equal || (valid && k > thr)) {
-                            nodes[n_new * kPad + t] = x ? pack_node(rb, f + len - rb) : pack_node(f, rb - f);
-                            scores[n_new * kPad + t] = __uint_as_float(own[2 * j + x]);
-                            ++n_new;
-                        }
+                for (int i = 0; i < 2 * kNodes; ++i) {
+                    const bool equal = own[i] == thr && thr != 0u && missing > 0;
+                    missing -= equal ? 1 : 0;
+                    if (equal || own[i] > thr) {
+                        const unsigned f = nd[i / 2] & 0xffffu, len = nd[i / 2] >> 16, left = (len + 1u) >> 1;
+                        nodes[n_new * kPad + t] = i & 1 ? (f + left) | ((len - left) << 16) : f | (left << 16);
+                        scores[n_new * kPad + t] = score_of_key(own[i]);
+                        ++n_new;
                     }
                 }
                 tl->n_nodes[t] = (int)n_new;
                 if (!last) {  // the token's candidates of the next level: the right branch of every node that has one
+                    unsigned c = 0u;
 #pragma unroll
                     for (int j = 0; j < kNodes; ++j) {
                         const unsigned x = j < (int)n_new ? nodes[j * kPad + t] : 0u;
-                        const int f = (int)(x & 0xffffu), len = (int)(x >> 16), rb = (2 * f + len - 1) / 2 + 1;
-                        if (len > 1 && rb <= e_qlim) {
-                            ++n_tiles;
+                        const int rb = right_of(x);
+                        if ((x >> 16) > 1u && rb <= e_qlim) {
+                            nodes[(kNodes + c) * kPad + t] = (unsigned)rb | ((unsigned)j << 16);
+                            ++c;
                             want(rb);
                         }
                     }
+                    if (c < (unsigned)kNodes) nodes[(kNodes + c) * kPad + t] = kNoBlock;
+                    n_tiles += c;
                 } else if (e_ok) {
                     tiles_needed += n_tiles;
                     if (g.row_tiles != nullptr) g.row_tiles[((long long)b * g.H + h) * g.n_qb + e_tq] = n_tiles;
