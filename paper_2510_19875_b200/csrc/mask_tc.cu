@@ -47,6 +47,7 @@ constexpr int kMmaWarps = 4;   // they take the stages in turn
 constexpr int kR = 4;          // rows (query heads) per group
 constexpr int kSlots = 8;      // TMEM accumulator slots, one query block of fp32 columns each
 constexpr int kStageKeys = 128;
+constexpr int kFinal = 1 << 16;  // (several k) added to the length of a row's last list
 constexpr int kProducers = 2;     // producer p fills the stage buffers b with b % 2 == p
 constexpr int kListReaders = kProducers + kMmaWarps + 4 * kEpiGroups;  // producer, MMA and epilogue warps; of a first list and the group record also the controllers
 
@@ -175,15 +176,18 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
             return;
         }
         const int b = tl->grp_b, kvh = tl->grp_kvh, R = tl->grp_R, levels = tl->grp_levels;
-        for (int level = 0; level < levels; ++level) {
+        unsigned open = S::kMulti && levels > 1 ? (1u << R) - 1u : 0u;  // (several k) rows with a list to come
+        for (int level = 0; S::kMulti ? level == 0 || open != 0 : level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
                 const int li = level == 0 ? kR : x;
+                if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 102)) return;
                     jr_par[x] ^= 1;
                 }
-                const int n = tl->n_jobs[li];
+                int n = tl->n_jobs[li];
+                if (S::kMulti && n >= kFinal) { n -= kFinal; open &= ~(1u << x); }
                 const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
                 for (int j = 0; j < n; j += S::kTps) {
                     if ((st.idx & (kProducers - 1)) != which) { st.advance(S::kStages); continue; }  // the other producer's buffer
@@ -254,15 +258,20 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
         const int R = tl->grp_R, levels = tl->grp_levels;
         const bool give_back = tl->grp_last != 0;
         unsigned q_due = tl->grp_new_q ? (1u << R) - 1u : 0u;  // rows whose Q tile this warp has yet to see arrive
-        for (int level = 0; level < levels; ++level) {
+        unsigned open = S::kMulti && levels > 1 ? (1u << R) - 1u : 0u;  // (several k) rows with a list to come
+        for (int level = 0; S::kMulti ? level == 0 || open != 0 : level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
                 const int li = level == 0 ? kR : x;
+                if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 203)) return;
                     jr_par[x] ^= 1;
                 }
-                const unsigned n_st = (unsigned)(tl->n_jobs[li] + S::kTps - 1) / S::kTps;  // stages of this list
+                int n = tl->n_jobs[li];
+                const bool final = S::kMulti ? n >= kFinal || levels == 1 : level + 1 == levels;
+                if (S::kMulti && n >= kFinal) { n -= kFinal; open &= ~(1u << x); }
+                const unsigned n_st = (unsigned)(n + S::kTps - 1) / S::kTps;  // stages of this list
                 __syncwarp();
                 if (elect_one()) mbar_arrive(smem_u32(&tl->jobs_ack[li]));  // the count is all this role reads
                 __syncwarp();
@@ -321,7 +330,7 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
                             q_par ^= 1u << r;
                             q_due &= ~(1u << r);
                         }
-                if (give_back && level + 1 == levels) {  // the rows' last products with these Q tiles
+                if (give_back && final) {  // the rows' last products with these Q tiles
                     if (elect_one())
                         for (int r = r0; r < r1; ++r) tc_commit(smem_u32(&tl->q_free[r]));
                     __syncwarp();
@@ -411,17 +420,20 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
             last_to = to;
             return true;
         };
-        for (int level = 0; level < levels; ++level) {
+        unsigned open = S::kMulti && levels > 1 ? (1u << R) - 1u : 0u;  // (several k) rows with a list to come
+        for (int level = 0; S::kMulti ? level == 0 || open != 0 : level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
                 const int li = level == 0 ? kR : x;
+                if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 302)) return;
                     jr_par[x] ^= 1;
                 }
                 // All there is to read of the list, at once: a look at it chain by chain, with the
                 // comparisons, was a good part of what a warp spends on a chain.
-                const int n = tl->n_jobs[li];
+                int n = tl->n_jobs[li];
+                if (S::kMulti && n >= kFinal) { n -= kFinal; open &= ~(1u << x); }
                 const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
 #pragma unroll
                 for (int y = 0; y < S::kListRegs; ++y) {
@@ -460,7 +472,7 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                 last_to = smem_u32(&tl->no_part);
                 // this list is done for rows r0..r1: tell their controllers
                 __syncwarp();
-                if (lane == 0)
+                if (lane == 0 && (!S::kMulti || level == 0 || n > 0))
                     for (int r = level == 0 ? 0 : x; r < r1; ++r) mbar_arrive(smem_u32(level == 0 ? &tl->first_done[set][r] : &tl->scores_done[r]));
             }
         }
@@ -649,6 +661,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
         }
         bool need[kNodes];                // the right candidate's score comes from the list
         int my_c[kNodes], n_nodes = 0;
+        bool listed = true;               // the level's list holds something (else nobody reports on it)
         for (int level = 0; level < levels; ++level) {
             if (level == 0) {
                 if (!mbar_wait_w(smem_u32(&tl->first_done[set][r]), (first_par >> set) & 1u, tl, P.ws, 408)) return;
@@ -661,8 +674,10 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
                     if (kMulti) __stcg(cache + ((x & 1) ? (nf[x >> 1] + nl[x >> 1]) / 2 + 1 : nf[x >> 1]), cache_pack(tag, sc[x]));
                 }
             } else {
-                if (!mbar_wait_w(smem_u32(&tl->scores_done[r]), sd_par, tl, P.ws, 401)) return;
-                sd_par ^= 1;
+                if (!kMulti || listed) {
+                    if (!mbar_wait_w(smem_u32(&tl->scores_done[r]), sd_par, tl, P.ws, 401)) return;
+                    sd_par ^= 1;
+                }
 #pragma unroll
                 for (int x = 0; x < kNodes; ++x) {
                     has[2 * x] = kNodes * lane + x < n_nodes;
@@ -715,6 +730,10 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
                     if (kMulti && need[x] && remembered(rb, tag, sc[2 * x + 1])) need[x] = false;  // an earlier pass (another k) has scored it
                     due[x] = __ballot_sync(0xffffffffu, need[x]);
                 }
+                // (several k) An empty list is left out, but for the row's last, which says that it is.
+                const bool final = kMulti && level + 2 == levels;
+                listed = flags_all(due) > 0;
+                if (kMulti && !listed && !final) continue;
                 if (!mbar_wait_w(smem_u32(&tl->jobs_ack[r]), ack_par, tl, P.ws, 403)) return;
                 ack_par ^= 1;
                 int at = flags_before(due, lt);
@@ -723,7 +742,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
                     my_c[x] = at;
                     if (need[x]) tl->jobs_blk[r][at++] = (nf[x] + nl[x]) / 2 + 1;
                 }
-                if (lane == 0) tl->n_jobs[r] = flags_all(due);
+                if (lane == 0) tl->n_jobs[r] = flags_all(due) + (final ? kFinal : 0);
                 tiles += (unsigned)flags_all(due);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[r]));
