@@ -166,7 +166,7 @@ __device__ __forceinline__ unsigned long long cache_pack(unsigned tag, float s) 
 template <class S>
 __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *tl, unsigned k_smem, int which) {
     Ring st;
-    unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
+    unsigned grp_par = 0, jr_par = 0;  // jr_par: bit by bit for the rows
     unsigned long long fetched = 0;  // tiles this warp has asked TMA for
     for (;;) {
         if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 101)) return;
@@ -183,8 +183,8 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
                 const int li = level == 0 ? kR : x;
                 if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
-                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 102)) return;
-                    jr_par[x] ^= 1;
+                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), (jr_par >> x) & 1u, tl, P.ws, 102)) return;
+                    jr_par ^= 1u << x;
                 }
                 int n = tl->n_jobs[li];
                 if (S::kMulti && n >= kFinal) { n -= kFinal; open &= ~(1u << x); }
@@ -245,7 +245,7 @@ __device__ __forceinline__ int chain_slot(int level, int r, unsigned stage) {
 
 template <class S>
 __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned k_smem, unsigned tmem_base, int which) {
-    unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
+    unsigned grp_par = 0, jr_par = 0;  // jr_par: bit by bit for the rows
     unsigned q_par = 0;       // bit r: phase of row r's next Q tile
     unsigned stage_seq = 0;   // stages so far, over the whole kernel (the same in every role)
     unsigned slot_par = 0;    // bit i: phase of the next use of this warp's slot i
@@ -265,8 +265,8 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
                 const int li = level == 0 ? kR : x;
                 if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
-                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 203)) return;
-                    jr_par[x] ^= 1;
+                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), (jr_par >> x) & 1u, tl, P.ws, 203)) return;
+                    jr_par ^= 1u << x;
                 }
                 int n = tl->n_jobs[li];
                 const bool final = S::kMulti ? n >= kFinal || levels == 1 : level + 1 == levels;
@@ -348,7 +348,7 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
 template <class S>
 __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, int wq, int grp, int lane) {
     const Geom &g = P.g;
-    unsigned grp_par = 0, jr_par[kR] = {0, 0, 0, 0};
+    unsigned grp_par = 0, jr_par = 0;  // jr_par: bit by bit for the rows
     unsigned stage_seq = 0;
     unsigned full_par = 0;  // bit w: phase of the next use of issuing warp w's slot `grp`
     constexpr int kBlk = S::kBlk;
@@ -427,8 +427,8 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                 const int li = level == 0 ? kR : x;
                 if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
-                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), jr_par[x], tl, P.ws, 302)) return;
-                    jr_par[x] ^= 1;
+                    if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), (jr_par >> x) & 1u, tl, P.ws, 302)) return;
+                    jr_par ^= 1u << x;
                 }
                 // All there is to read of the list, at once: a look at it chain by chain, with the
                 // comparisons, was a good part of what a warp spends on a chain.
@@ -860,7 +860,8 @@ struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
 stream_status split_rows(const Geom &g, Split *s) {
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    s->head_rows = g.hpg < kR ? g.hpg : kR;
+    s->n_chunks = (g.hpg + kR - 1) / kR;
+    s->head_rows = (g.hpg + s->n_chunks - 1) / s->n_chunks;  // (six heads as 3 + 3, not 4 + 2: 139 -> 135 us at 10007 tokens in blocks of 32, 115 -> 107 at 8221)
     s->qb_rows = g.k_row == nullptr ? kR / g.hpg : 1;
     if (s->qb_rows < 1) s->qb_rows = 1;
     for (;;) {
