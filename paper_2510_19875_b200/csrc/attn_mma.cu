@@ -1,5 +1,5 @@
 // Block-sparse attention (Eq. 2 on a Stream mask) on mma.sync for the bf16 shapes that the tcgen05
-// kernel does not take: d = 64 / 128 / 256, any block sizes up to 64, per-token masks among them.
+// kernels do not take: d = 64 / 128 / 256, any block sizes up to 64, per-token masks among them.
 //
 // A warp owns 16 query tokens: their Q fragments (registers; shared memory for d = 256), their
 // output accumulators and softmax statistics. Key and value tiles come to shared memory by
@@ -24,7 +24,8 @@
 // Bound: the latency of dependent steps at 8 to 16 warps per SM (issue slots 41 % busy, mma pipe 23
 // to 35 %); hence the register limits below (12 heads, T = 10007, blocks of 32, d = 128, k = 8: 180
 // us at two CTAs of four warps per SM, 152 at three; 3220 on the fp32-FMA kernel. 16 heads,
-// T = 8192, d = 64, k = 40, not causal: 669 us at two, 600 at four; 4640).
+// T = 8192, d = 64, k = 40, not causal: 669 us at two, 600 at four; 4640. Both have gone to attn_tc.cu since; left
+// are d = 256, blocks other than 32 and 64, block_q != block_k, per-token masks beside attn_tok.cu's).
 #include "warp_common.cuh"
 
 namespace stream {

@@ -8,9 +8,10 @@
 // stages; one tcgen05.mma chain per (stage, row) computes the keys (128 x d) x Q_row^T (d x block)
 // into a TMEM slot of as many columns (on the first level one chain for two rows: a chain of one is
 // bound by its operands' way out of shared memory, 48 clocks a step of 16 channels against 64 for
-// both); four epilogue warps reduce the slot to the masked tile maxima (Eq. 4 under C). There are two such groups of four, each serving one of every issuing warp's
-// two slots: the fixed cost of a hand-over (wait, fences, arrive) is larger than the reduction
-// itself, and one group alone would be the longest stage of the pipeline. A controller warp per
+// both); four epilogue warps reduce the slot to the masked tile maxima (Eq. 4 under C). There are two
+// such groups of four, each serving one of every issuing warp's two slots: the fixed cost of a
+// hand-over (wait, fences, arrive) is larger than the reduction itself, and one group alone would be
+// the longest stage of the pipeline. A controller warp per
 // row keeps the row's nodes in registers, ranks the 2k branch scores (higher score, then lower block
 // index), compacts the survivors with ballots and publishes the next level's fetch list. The
 // first level's representatives are the same for every row of a group, so one fetched stage
@@ -24,6 +25,10 @@
 // last products are complete, so that the first tiles of the next group arrive behind the last
 // products of this one. (One warp doing all of it, and ranking all four rows, kept the issuing
 // warps waiting for a group or a list for 17 % (T = 16384, k = 16) to 29 % (several k) of the time.)
+//
+// What bounds it: the chip's power limit (1500 MHz at T = 131072, 1590 at 16384, of 1965) with the tensor cores
+// busy 70 to 76 % of the clocks; beside them the way of a stage (a third of it transfer) and the
+// serial round of a row's level, list to ranked list, about 3500 clocks.
 //
 // Roles (608 threads): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
 // 3, 13, 17 MMA issuers (warp 1 owns TMEM), warp 18 dispatcher (groups, first lists, Q tiles), warps 0,
