@@ -479,8 +479,12 @@ stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void 
     const long long rows = (long long)g.batch * g.H * g.n_qb;
     // Sixteen warps when every row has an SM to itself anyway: a level's tiles then spread over more
     // warps (64 rows, fp32, d = 64, blocks of 32, k = 8: 34.9 us with eight, 32.9 with sixteen, before the
-    // divisions went; 28.9 now).
-    if (rows <= sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
+    // divisions went; 28.9 now). With up to two rows an SM, too, if the first level has a tile part for
+    // each of them (fp32: 208 rows, blocks of 64, k = 8: four warps 92.8 us, sixteen 59.7; 181 rows, blocks
+    // of 16, k = 15, d = 128: 118 and 78; 282 rows with 12 parts each: 26.6 and 30.8). With three rows an SM
+    // four warps are the better (343 rows, blocks of 16, k = 8: 42.9 us, sixteen 63.5).
+    const int parts = 2 * g.k_top * ((g.bq + 31) / 32) * ((g.bk + kKeysPerUnit - 1) / kKeysPerUnit);
+    if (rows <= (parts >= kWideWarps ? 2 : 1) * (long long)sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
     return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
 }
 
