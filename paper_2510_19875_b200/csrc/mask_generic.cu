@@ -299,7 +299,9 @@ struct Slots {
     __device__ unsigned *key() const { return (unsigned *)at + 2 * n; }
 };
 
-template <class P, int W>
+// kCluster: a row's tiles are dealt to the CTAs of a cluster (a power of two of them). Each keeps all the slots, scores
+// those that are its own, hands their keys to the others, and ranks like them.
+template <class P, int W, bool kCluster>
 __global__ void __launch_bounds__(W * 32, W == kWideWarps ? 1 : P::kCtas)
 mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P::Elem *__restrict__ q,
                  const typename P::Elem *__restrict__ k, int32_t *__restrict__ mask, float *__restrict__ score, WorkspaceHeader *ws) {
@@ -310,11 +312,12 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
     unsigned *keep = (unsigned *)words + 7 * n_max;  // a bit per slot
     // several k: scores of this row by key block, NaN = not scored yet (a score does not depend on k)
     float *cache = mk.use_cache ? (float *)(keep + n_max / 32) : nullptr;
-    __shared__ int s_list, s_valid;
+    __shared__ int s_list, s_valid, s_all;  // s_all (clusters): listed by any of the CTAs
+    const unsigned n_cta = kCluster ? cluster_size() : 1u, cta = kCluster ? cluster_rank() : 0u;
 
     const int tid = threadIdx.x, n_thr = blockDim.x;
     // heaviest rows (late query blocks) first
-    const long long row_rev = blockIdx.x;
+    const long long row_rev = blockIdx.x / n_cta;
     const int qb = g.n_qb - 1 - (int)(row_rev / ((long long)g.batch * g.H));
     const int bh = (int)(row_rev % ((long long)g.batch * g.H));
     const int b = bh / g.H, h = bh % g.H, kvh = h / g.hpg;
@@ -333,7 +336,8 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
     auto put = [&](const Slots &s, int c, bool ok, int fst, int lst, unsigned known, bool want) {
         if (ok && known == 0u && want) {
             if (cache != nullptr && !isnan(cache[fst])) known = key_of(cache[fst]);
-            else list[atomicAdd(&s_list, 1)] = c;
+            else if (!kCluster || (((unsigned)c >> 1) & (n_cta - 1u)) == cta) list[atomicAdd(&s_list, 1)] = c;
+            if (kCluster) atomicAdd(&s_all, 1);
         }
         s.first()[c] = fst;
         s.last()[c] = ok ? lst : fst - 1;
@@ -357,7 +361,7 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
         const int kq = mk.n > 0 ? mk.k[pass] : row_k(g, qb);  // this pass's k (= k_top unless told otherwise)
         const int levels = row_levels(g, kq);
         __syncthreads();  // the previous pass is done with the slots
-        if (tid == 0) { s_list = 0; s_valid = 0; }
+        if (tid == 0) { s_list = 0; s_valid = 0; s_all = 0; }
         __syncthreads();
         // initial nodes tiling [0, N_k); those without an allowed block are absent. With no level to
         // go through (one key block) they are the result, and need a score only if it is asked for.
@@ -375,11 +379,22 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
 
         for (int level = 0;; ++level) {
             const Slots cur = {words + par * 3 * n_max, n_max}, nxt = {words + (par ^ 1) * 3 * n_max, n_max};
-            const int n_list = s_list, n_valid = s_valid, n_words = (n_slots + 31) >> 5;
+            if (kCluster) cluster_arrive();  // the level's slots are written
+            const int n_list = s_list, n_valid = s_valid, n_all = kCluster ? s_all : n_list, n_words = (n_slots + 31) >> 5;
             P::score(g, smem, kp, qb, list, n_list, cur.first(), cur.key());
-            if (level < levels) tiles += (unsigned)n_list;
+            if (level < levels) tiles += (unsigned)n_all;
             __syncthreads();  // every key of the level is in place
-            if (tid == 0) { s_list = 0; s_valid = 0; }
+            if (kCluster) {
+                cluster_wait();
+                for (int i = tid; i < n_list * (int)n_cta; i += n_thr) {
+                    const int slot = list[i / (int)n_cta];
+                    const unsigned to = (unsigned)i % n_cta;
+                    if (to != cta) store_in_cluster(&cur.key()[slot], to, cur.key()[slot]);
+                }
+                cluster_arrive();
+                cluster_wait();
+            }
+            if (tid == 0) { s_list = 0; s_valid = 0; s_all = 0; }
             if (cache != nullptr)
                 for (int i = tid; i < n_list; i += n_thr) cache[cur.first()[list[i]]] = score_of(cur.key()[list[i]]);
             // Top-k by rank: a candidate is beaten by a higher score, or an equal one in a lower slot.
@@ -425,6 +440,7 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
                 if (!((keep[w] >> (c & 31)) & 1u)) continue;
                 int pos = __popc(keep[w] & ((1u << (c & 31)) - 1u));
                 for (int u = 0; u < w; ++u) pos += __popc(keep[u]);
+                if (last && cta != 0u) continue;
                 if (last) {
                     mask[o + pos] = cur.first()[c];
                     if (score != nullptr) score[o + pos] = score_of(cur.key()[c]);
@@ -433,7 +449,7 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
                 }
             }
             if (last) {
-                for (int j = n_kept + tid; j < g.k_top; j += n_thr) {
+                for (int j = n_kept + tid; j < g.k_top && cta == 0u; j += n_thr) {
                     mask[o + j] = -1;
                     if (score != nullptr) score[o + j] = -CUDART_INF_F;
                 }
@@ -445,7 +461,7 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
             __syncthreads();
         }
     }
-    if (tid == 0) {
+    if (tid == 0 && cta == 0u) {
         atomicAdd(&ws->tiles_scored, (unsigned long long)tiles);
         atomicAdd(&ws->rows, 1ull);
         if (g.row_tiles != nullptr) g.row_tiles[row] = tiles;
@@ -454,21 +470,31 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
 
 constexpr size_t kMaxDynamicSmem = 227 * 1024 - 1024;  // (the kernel has a few static words too)
 
-template <class P, int W>
+template <class P, int W, bool kCluster = false>
 stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, int32_t *mask, float *score, WorkspaceHeader *ws,
-                       cudaStream_t st) {
+                       cudaStream_t st, int n_cta = 1) {
     const long long rows = (long long)g.batch * g.H * g.n_qb;
     const int n_max = (2 * g.k_top + 31) & ~31;
     const size_t score_bytes = P::smem_bytes(g, W);
     size_t smem = score_bytes + (size_t)(7 * n_max + n_max / 32) * 4;
     mk.use_cache = mk.n > 1 && smem + sizeof(float) * (size_t)g.N_k <= kMaxDynamicSmem;
     if (mk.use_cache) smem += sizeof(float) * (size_t)g.N_k;
-    auto kern = mask_rows_kernel<P, W>;
+    auto kern = mask_rows_kernel<P, W, kCluster>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_rows)");
-    kern<<<(unsigned)rows, W * 32, smem, st>>>(g, mk, (int)score_bytes, n_max, (const typename P::Elem *)q,
-                                               (const typename P::Elem *)k, mask, score, ws);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute cluster[1] = {};
+    c.gridDim = dim3((unsigned)(rows * n_cta));
+    c.blockDim = dim3(W * 32);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cluster[0].id = cudaLaunchAttributeClusterDimension;
+    cluster[0].val.clusterDim.x = (unsigned)n_cta;
+    cluster[0].val.clusterDim.y = cluster[0].val.clusterDim.z = 1;
+    c.attrs = cluster;
+    c.numAttrs = kCluster ? 1 : 0;
+    e = cudaLaunchKernelEx(&c, kern, g, mk, (int)score_bytes, n_max, (const typename P::Elem *)q, (const typename P::Elem *)k, mask, score, ws);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "mask_rows launch");
     return STREAM_OK;
 }
@@ -484,6 +510,12 @@ stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void 
     // of 16, k = 15, d = 128: 118 and 78; 282 rows with 12 parts each: 26.6 and 30.8). With three rows an SM
     // four warps are the better (343 rows, blocks of 16, k = 8: 42.9 us, sixteen 63.5).
     const int parts = 2 * g.k_top * ((g.bq + 31) / 32) * ((g.bk + kKeysPerUnit - 1) / kKeysPerUnit);
+    // Fewer rows than half of the SMs: a row over two, four or eight of them, while each has a tile part for
+    // every scheduler (fp32, 28 rows, blocks of 64, k = 11: 65.2 -> 31.3 us; 55 rows, blocks of 32, d = 128, k = 9:
+    // 55.3 -> 43.7; the 64 rows above: 28.7 -> 24.6).
+    int n_cta = 1;
+    while (n_cta < 8 && rows * 2 * n_cta <= sm_count_or_default() && parts >= 8 * n_cta) n_cta *= 2;
+    if (n_cta > 1 && mk.n <= 1) return launch_w<P, kWideWarps, true>(g, mk, q, k, mask, score, ws, st, n_cta);
     if (rows <= (parts >= kWideWarps ? 2 : 1) * (long long)sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
     return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
 }

@@ -53,6 +53,27 @@ __device__ __forceinline__ void group_sync(int id, int threads) {
     else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+// The CTAs of a cluster: their number, this one's; a barrier in two halves (what was written before the
+// first is seen behind the second, in the other CTAs' shared memory too); a word of another's
+// shared memory, at the place of one of this CTA's own.
+__device__ __forceinline__ unsigned cluster_size() {
+    unsigned n;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+    return n;
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void store_in_cluster(unsigned *own, unsigned cta, unsigned value) {
+    unsigned at;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(own)), "r"(cta));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(value) : "memory");
+}
+
 // Which of the 8 16-byte columns of a 128-byte line a bf16 row keeps chunk c of that line in: c ^
 // swz_rows(row). Read as mma operands, 8 lanes (two rows r, r + 1, four consecutive chunks each)
 // then meet 8 different columns.

@@ -42,6 +42,8 @@ CASES = [  # spec changes, block_q, block_k (None: the spec's block), causal
     (dict(d=128, T=515, n_q_heads=5, n_kv_heads=1, k_top=512), None, None, False),    # mask rows as long as they go with four to a unit
     (dict(dtype="f32", T=1003, n_q_heads=8), None, None, True),
     (dict(dtype="f32", T=515, d=128, k_top=40, block=16), None, None, True),
+    (dict(dtype="f32", T=300, block=64, n_q_heads=1, n_kv_heads=1, k_top=8), None, None, True),    # a row over eight CTAs
+    (dict(dtype="f32", T=2047, n_q_heads=1, n_kv_heads=1, k_top=7), None, None, False),            # over two
     (dict(dtype="f32", T=300, d=256, block=64, k_top=3), None, None, False),
     (dict(dtype="f32", T=300, d=16, k_top=3), 1, 24, True),
 ]
