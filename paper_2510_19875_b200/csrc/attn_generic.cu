@@ -63,7 +63,8 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
     if (kAsync) cp_async_commit();
 }
 
-template <typename T, int D, int QW, bool kAsync>
+// kCluster: the row's tiles are dealt to the groups of all CTAs of a cluster, which read each other's parts at the end.
+template <typename T, int D, int QW, bool kAsync, bool kCluster>
 __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, int splits, const T *__restrict__ q,
                                                            const T *__restrict__ k, const T *__restrict__ v,
                                                            const int32_t *__restrict__ mask, float scale, T *__restrict__ out) {
@@ -76,7 +77,9 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
     const int kq = lane >> 2, kk = lane & 3;   // Q K^T
     const int ro = lane >> 3, co = lane & 7;   // P V
     // late (longer) rows first
-    const int bh = blockIdx.x / g.n_qb, qb = g.n_qb - 1 - (int)(blockIdx.x % g.n_qb);
+    const unsigned n_cta = kCluster ? cluster_size() : 1u, cta = kCluster ? cluster_rank() : 0u, row = blockIdx.x / n_cta;
+    const int bh = (int)(row / (unsigned)g.n_qb), qb = g.n_qb - 1 - (int)(row % (unsigned)g.n_qb);
+    const int turn = (int)cta * splits + grp, groups = (int)n_cta * splits;  // this group's turn among all of the row's
     const int b = bh / g.H, h = bh % g.H, kvh = h / g.hpg;
     const T *qp = q + b * g.qs_b + h * g.qs_h;
     const T *kp = k + b * g.ks_b + kvh * g.ks_h, *vp = v + b * g.ks_b + kvh * g.ks_h;
@@ -120,12 +123,12 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
     const float *qw = Qs + (size_t)mw * QW * D;
 
     const int n_sub = (g.bk + kKeys - 1) / kKeys, n_tiles = s_n * n_sub;
-    if (grp < n_tiles) {
-        fetch<T, D, kAsync, true>(g, ks, kp, list[grp / n_sub], grp % n_sub * kKeys, g_tid, g_thr);
-        fetch<T, D, kAsync, false>(g, vs, vp, list[grp / n_sub], grp % n_sub * kKeys, g_tid, g_thr);
+    if (turn < n_tiles) {
+        fetch<T, D, kAsync, true>(g, ks, kp, list[turn / n_sub], turn % n_sub * kKeys, g_tid, g_thr);
+        fetch<T, D, kAsync, false>(g, vs, vp, list[turn / n_sub], turn % n_sub * kKeys, g_tid, g_thr);
     }
-    for (int i0 = grp; i0 < n_tiles; i0 += splits) {
-        const int r = list[i0 / n_sub], n0 = i0 % n_sub * kKeys, nxt = i0 + splits;
+    for (int i0 = turn; i0 < n_tiles; i0 += groups) {
+        const int r = list[i0 / n_sub], n0 = i0 % n_sub * kKeys, nxt = i0 + groups;
         const long long k0 = (long long)r * g.bk + n0;
         const int n_keys = (int)max(0ll, min((long long)min(g.bk - n0, kKeys), g.T - k0));
         if (kAsync) cp_async_wait<1>();
@@ -239,6 +242,45 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
                 *(float4 *)(part + 2 * QW + (ro * RO + i) * Sh::kRowPitch + 4 * co + 32 * j) =
                     make_float4(o[i][4 * j], o[i][4 * j + 1], o[i][4 * j + 2], o[i][4 * j + 3]);
     }
+    if constexpr (kCluster) {
+        cluster_arrive();
+        cluster_wait();
+        const size_t step = (size_t)m_warps * Sh::kPart;  // to the same row of the CTA's next group
+        float *const weight = (float *)smem + (size_t)splits * step;  // [row][group]
+        for (int m = tid; m < m_warps * QW; m += blockDim.x) {
+            const float *first = (const float *)smem + (size_t)(m / QW) * Sh::kPart + m % QW;
+            float *const w = weight + m * groups;
+            float top = -CUDART_INF_F, total = 0.f;
+            for (int s = 0; s < groups; ++s) {
+                w[s] = load_in_cluster(first + s % splits * step, (unsigned)(s / splits));
+                top = fmaxf(top, w[s]);
+            }
+            const float ref = top == -CUDART_INF_F ? 0.f : top;
+            for (int s = 0; s < groups; ++s) {
+                w[s] = w[s] == -CUDART_INF_F ? 0.f : expf(w[s] - ref);
+                total += w[s] * load_in_cluster(first + s % splits * step + QW, (unsigned)(s / splits));
+            }
+            const float inv = total > 0.f ? 1.f / total : 0.f;
+            for (int s = 0; s < groups; ++s) w[s] *= inv;
+        }
+        __syncthreads();
+        for (int idx = tid + (int)cta * (int)blockDim.x; idx < m_warps * QW * (D / 4); idx += (int)(n_cta * blockDim.x)) {
+            const int m = idx / (D / 4), c = idx % (D / 4) * 4;
+            const long long tq = (long long)qb * g.bq + m;
+            if (m >= g.bq || tq >= g.T) continue;
+            const float *first = (const float *)smem + (size_t)(m / QW) * Sh::kPart + 2 * QW + (m % QW) * Sh::kRowPitch + c;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int s = 0; s < groups; ++s) {
+                const float f = weight[m * groups + s];
+                const float4 y = load4_in_cluster(first + s % splits * step, (unsigned)(s / splits));
+                x.x = fmaf(f, y.x, x.x); x.y = fmaf(f, y.y, x.y); x.z = fmaf(f, y.z, x.z); x.w = fmaf(f, y.w, x.w);
+            }
+            store4(out + ((long long)bh * g.T + tq) * D + c, x);
+        }
+        cluster_arrive();  // (nobody leaves while its part may still be read)
+        cluster_wait();
+        return;
+    }
     __syncthreads();
     for (int m = tid; m < m_warps * QW; m += blockDim.x) {
         float *first = (float *)smem + (size_t)(m / QW) * Sh::kPart + m % QW;
@@ -278,20 +320,36 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     const int m_warps = (g.bq + QW - 1) / QW;
     const long long rows = (long long)g.batch * g.H * g.n_qb;
     // Four warps a CTA, so that several CTAs share an SM; eight when every row has an SM to itself
-    // anyway.
-    int splits = (rows <= sm_count_or_default() ? 8 : 4) / m_warps;
+    // anyway. Fewer rows than half of the SMs: a row over two, four or eight CTAs, while each has a tile part for
+    // every scheduler (28 rows, blocks of 64, k = 11, d = 64: 65.4 -> 34.8 us; 55 rows, blocks of 32, k = 9, d = 128:
+    // 38.9 -> 30.7; 64 rows, blocks of 32, k = 8: 18.4 either way).
+    const int n_sm = sm_count_or_default(), tiles = g.k_top * ((g.bk + kKeys - 1) / kKeys);
+    int splits = (rows <= n_sm ? 8 : 4) / m_warps, n_cta = 1;
+    while (n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta) n_cta *= 2;
+    if (n_cta > 1 && splits > (tiles + n_cta - 1) / n_cta) splits = (tiles + n_cta - 1) / n_cta;
     auto bytes = [&](int s) {
         const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * (Sh::kPBytes + QW * 4) + (size_t)g.k_top * 4;
-        const size_t sum = (size_t)m_warps * s * Sh::kPart * 4;
+        const size_t sum = (size_t)m_warps * s * Sh::kPart * 4 + (n_cta > 1 ? (size_t)m_warps * QW * s * n_cta * 4 : 0);
         return walk > sum ? walk : sum;
     };
     while (splits > 1 && bytes(splits) > 220 * 1024) splits /= 2;
     const size_t smem = bytes(splits);
-    auto kern = attn_generic_kernel<T, D, QW, kAsync>;
+    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kAsync, true> : attn_generic_kernel<T, D, QW, kAsync, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
-    kern<<<(unsigned)rows, m_warps * splits * 32, smem, st>>>(g, m_warps, splits, (const T *)q, (const T *)k, (const T *)v, mask, scale, (T *)out);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute cluster[1] = {};
+    c.gridDim = dim3((unsigned)(rows * n_cta));
+    c.blockDim = dim3((unsigned)(m_warps * splits * 32));
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cluster[0].id = cudaLaunchAttributeClusterDimension;
+    cluster[0].val.clusterDim.x = (unsigned)n_cta;
+    cluster[0].val.clusterDim.y = cluster[0].val.clusterDim.z = 1;
+    c.attrs = cluster;
+    c.numAttrs = n_cta > 1 ? 1 : 0;
+    e = cudaLaunchKernelEx(&c, kern, g, m_warps, splits, (const T *)q, (const T *)k, (const T *)v, mask, scale, (T *)out);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "attn_generic launch");
     return STREAM_OK;
 }

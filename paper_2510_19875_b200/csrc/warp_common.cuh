@@ -68,10 +68,24 @@ __device__ __forceinline__ unsigned cluster_rank() {
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-__device__ __forceinline__ void store_in_cluster(unsigned *own, unsigned cta, unsigned value) {
+__device__ __forceinline__ unsigned address_in_cluster(const void *own, unsigned cta) {
     unsigned at;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(own)), "r"(cta));
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(value) : "memory");
+    return at;
+}
+__device__ __forceinline__ void store_in_cluster(unsigned *own, unsigned cta, unsigned value) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(address_in_cluster(own, cta)), "r"(value) : "memory");
+}
+__device__ __forceinline__ float load_in_cluster(const float *own, unsigned cta) {
+    float x;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(address_in_cluster(own, cta)) : "memory");
+    return x;
+}
+__device__ __forceinline__ float4 load4_in_cluster(const float *own, unsigned cta) {
+    float4 x;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(address_in_cluster(own, cta)) : "memory");
+    return x;
 }
 
 // Which of the 8 16-byte columns of a 128-byte line a bf16 row keeps chunk c of that line in: c ^
