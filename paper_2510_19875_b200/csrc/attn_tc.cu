@@ -137,12 +137,7 @@ struct Params {
     float scale_log2;      // logit scale times log2(e)
 };
 
-template <class F>
-__device__ __forceinline__ bool wait(unsigned bar, unsigned parity, Tail<F> *tl, unsigned code) {
-    return mbar_wait_bounded(bar, parity, &tl->abort_flag, &g_attn_status[0], &g_attn_status[1], code);
-}
-
-// The same for a whole converged warp (all lanes get the same answer).
+// Bounded wait of a whole converged warp (all lanes get the same answer).
 template <class F>
 __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail<F> *tl, unsigned code) {
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &g_attn_status[0], &g_attn_status[1], code);

@@ -59,17 +59,10 @@ __device__ __forceinline__ bool mbar_test_wait(unsigned bar, unsigned parity) {
     return ok != 0;
 }
 
-// Bounded wait on an mbarrier phase. Returns false if the CTA is aborting, or if this wait ran
+// The part of a bounded wait on an mbarrier phase behind its first look. Returns false if the CTA is aborting, or if this wait ran
 // out, in which case it raises the CTA's abort flag and records `code` (first one wins) with the
 // block index in the two error words.
-// (A kernel that moves registers between its warpgroups with setmaxnreg cannot call a separate
-// function from the regions with different register counts: it defines STREAM_INLINE_SLOW_WAIT.)
-#ifdef STREAM_INLINE_SLOW_WAIT
-#define STREAM_SLOW_WAIT_ATTR __forceinline__
-#else
-#define STREAM_SLOW_WAIT_ATTR __noinline__
-#endif
-static __device__ STREAM_SLOW_WAIT_ATTR bool mbar_wait_slow(unsigned bar, unsigned parity, int *abort_flag, unsigned *err_code,
+static __device__ __noinline__ bool mbar_wait_slow(unsigned bar, unsigned parity, int *abort_flag, unsigned *err_code,
                                                    unsigned *err_info, unsigned code, long long limit) {
     const long long t0 = clock64();
     for (;;) {
@@ -82,11 +75,6 @@ static __device__ STREAM_SLOW_WAIT_ATTR bool mbar_wait_slow(unsigned bar, unsign
         }
     }
 }
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity, int *abort_flag, unsigned *err_code,
-                                                  unsigned *err_info, unsigned code, long long limit = kWaitCycles) {
-    if (mbar_try_wait(bar, parity)) return true;  // the common case costs one instruction
-    return mbar_wait_slow(bar, parity, abort_flag, err_code, err_info, code, limit);
-}
 
 // True in exactly one lane of a converged warp (the same lane every time).
 __device__ __forceinline__ bool elect_one() {
@@ -95,7 +83,7 @@ __device__ __forceinline__ bool elect_one() {
     return pred != 0;
 }
 
-// mbar_wait_bounded for a whole converged warp: every lane waits, and all lanes get the same
+// Bounded wait of a whole converged warp: every lane waits, and all lanes get the same
 // answer (false as soon as one lane saw the abort flag or ran out of time), so that the warp
 // stays converged for the elect_one() that follows.
 __device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, int *abort_flag, unsigned *err_code,
@@ -257,14 +245,6 @@ __device__ __forceinline__ void tmem_ld_32x8_issue(unsigned taddr, unsigned *r) 
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)
                  : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld_32x32(unsigned taddr, float *v) {
-    unsigned r[32];
-    tmem_ld_32x32_issue(taddr, r);
-    tmem_ld_wait();
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Maximum of three in one instruction.
