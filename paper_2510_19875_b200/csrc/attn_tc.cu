@@ -231,6 +231,7 @@ __device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStre
 }
 template <class F>
 __device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStream<F> &S) {
+    __syncwarp();  // (every lane has read what it needs of the slot; so wherever one lane arrives for its warp)
     if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
     __syncwarp();
     S.ms.advance(kMaskSlots);
@@ -445,6 +446,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
             __syncwarp();
             ks.advance(P.n_k_stages);
         }
+        __syncwarp();
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
         ms.advance(kMaskSlots);
@@ -488,6 +490,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
             __syncwarp();
             vs.advance(P.n_v_stages);
         }
+        __syncwarp();
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
         ms.advance(kMaskSlots);
@@ -687,6 +690,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
             if constexpr (!F::kSplit) tmem_st_32x32_issue(p_addr, packed);
             tmem_st_wait();
             tc_fence_before();
+            __syncwarp();  // lane 0 speaks for all lanes: their references and P come before its arrivals
             mbar_arrive_if(turn_own, lane == 0);
             mbar_arrive_if(smem_u32(&tl->p_full[grp][pb]), lane == 0);
             ++n_own;

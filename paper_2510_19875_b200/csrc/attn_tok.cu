@@ -211,6 +211,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tq, const CUte
             return true;
         }
         if (S.e >= S.n && !(is_k && q_due)) {
+            __syncwarp();
             if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
             __syncwarp();
             S.ms.advance(kMaskSlots);
@@ -297,6 +298,7 @@ __device__ void qk_role(Tail *tl, unsigned q_smem, unsigned k_smem, unsigned tme
             __syncwarp();
             ks.advance(kKStages);
         }
+        __syncwarp();
         if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));
         __syncwarp();
         ms.advance(kMaskSlots);
@@ -337,6 +339,7 @@ __device__ void pv_role(Tail *tl, unsigned v_smem, unsigned tmem_base) {
             __syncwarp();
             vs.advance(kVStages);
         }
+        __syncwarp();
         if (elect_one()) {
             if (last) tc_commit(smem_u32(&tl->o_done));
             mbar_arrive(smem_u32(&tl->m_empty[ms.idx]));

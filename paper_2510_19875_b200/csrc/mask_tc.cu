@@ -226,7 +226,8 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
                     __syncwarp();
                     st.advance(S::kStages);
                 }
-                if (elect_one()) mbar_arrive(smem_u32(&tl->jobs_ack[li]));  // done reading this list
+                __syncwarp();  // done reading this list, in every lane
+                if (elect_one()) mbar_arrive(smem_u32(&tl->jobs_ack[li]));
                 __syncwarp();
             }
         }
@@ -455,6 +456,7 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                     for (int y = 0; y < S::kListRegs; ++y)
                         masked[z][y] = __ballot_sync(0xffffffffu, my_blk[y] < 0 || my_blk[y] >= whole || my_blk[y] == diag);
                 }
+                __syncwarp();  // (lane 0 speaks for what every lane has read)
                 mbar_arrive_if(smem_u32(&tl->jobs_ack[li]), lane == 0);
                 const unsigned s_end = stage_seq + (unsigned)(n + S::kTps - 1) / S::kTps;
                 // First level: every stage serves all rows, rows grp, grp + 2 are this group's, and each

@@ -120,6 +120,36 @@ def test_attention_with_logits_far_from_the_reference(S, bq, shift, scale):
         assert (np.abs(out[bh, lo:hi] - want) <= few + np.abs(want) / 256).all(), rid
 
 
+@pytest.mark.parametrize("d,bq,bk", [(128, 64, 64), (64, 64, 64), (128, 32, 32), (64, 32, 32), (128, 1, 64)])
+def test_attention_with_references_that_move_at_many_entries(S, d, bq, bk):
+    """The logits of a token grow, fall or stay from block to block, each lane of a warp in its own way: the
+    tcgen05 attention kernels hand the references that move on between two groups of warps, lane by
+    lane. One stale reference and a weight is off by 2^30 or more; and every launch gives the same bits."""
+    spec = wl.WorkloadSpec("moves", 10, 1, 3, 1, 900, d, bk, 6, "bf16")
+    w = wl.generate(spec)
+    q, k, v = w.torch_tensors("cpu")
+    u = torch.ones(d) / d ** 0.5
+    slope = torch.from_numpy(np.random.default_rng(5).uniform(-1, 1, size=(1, 3, spec.T, 1)).astype(np.float32))
+    level = torch.arange(spec.T)[:, None] // bk * (bk / 64)  # a slope of 1: 30 a block of 64, 43 in the exponents of two
+    w.q = wl.to_bf16_bits((q.float() + d ** 0.5 * slope * u).numpy())
+    w.k = wl.to_bf16_bits((k.float() * 0.5 + 30 * level * u).numpy())
+    q, k, v = w.torch_tensors("cuda")
+    p = oracle_problem(spec, block_q=bq, block_k=bk)
+    nqb = so.num_query_blocks(p)
+    mask = np.random.default_rng(6).integers(0, spec.n_blocks, size=(spec.n_q_heads * nqb, spec.k_top)).astype(np.int32)
+    blocks = torch.from_numpy(mask.reshape(1, spec.n_q_heads, nqb, spec.k_top)).cuda()
+    outs = [S.sparse_attention(q, k, v, blocks, block_q=bq, block_k=bk) for _ in range(20)]
+    S.stream_check_device_status()
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
+    out = outs[0].float().cpu().numpy().reshape(-1, spec.T, d)
+    ref = so.sparse_attention_rows(p, w.q, w.k, w.v, mask, None)
+    few = 2e-3 + (5 / 256 if (d, bq) == (128, 64) else 0)  # as above: logits of up to 450
+    for rid in range(len(mask)):
+        bh, qb = divmod(rid, nqb)
+        lo, hi = qb * bq, min(spec.T, qb * bq + bq)
+        want = ref[rid, : hi - lo]
+        assert (np.abs(out[bh, lo:hi] - want) <= few + np.abs(want) / 256).all(), rid
+
 @pytest.mark.parametrize("kw,causal", [
     (dict(d=64, T=2100, block=64, k_top=33), True),                                       # two nodes a lane, one more than one would hold
     (dict(T=4500, k_top=64, n_q_heads=7, n_kv_heads=1), False),                           # the most; N_k just above k; 4 + 3 heads or fewer
