@@ -37,6 +37,7 @@ constexpr int kMaxBlock = 64;
 constexpr int kWindow = 128;          // merged: key blocks per window
 constexpr int kMergedWarps = 4;       // merged: warps (16 tokens each) per group
 constexpr int kMaxRows = 16 * kMergedWarps;
+constexpr size_t kMaxDynamicSmem = 227 * 1024 - 2048;  // (the merged walk's bits are static)
 
 struct Params {
     Geom g;
@@ -413,13 +414,18 @@ stream_status launch(Params P, cudaStream_t st) {
     P.n_tb = (int)((g.T + kMaxRows - 1) / kMaxRows);
     const long long ctas = (long long)g.batch * g.H * (P.merged ? P.n_tb : g.n_qb);
     // Four warps a CTA (eight when there are too few CTAs to give every SM several): whole groups of
-    // m_warps, the splits.
+    // m_warps, the splits, as many of them as shared memory has room for (a group of one warp, tiles of 64 keys,
+    // d = 256: three).
     const bool wide = ctas < 3ll * sm_count_or_default();
+    auto bytes = [&](int splits) {
+        size_t walk = (size_t)splits * 2 * W::kTileBytes + (size_t)(P.merged ? kWindow : ((g.k_top + 3) & ~3)) * 4;
+        if (W::kQRegs == 0) walk += (size_t)P.m_warps * 16 * D * 2;
+        const size_t part = (size_t)(splits - 1) * P.m_warps * (D / 2 + 4) * 32 * 4;
+        return walk > part ? walk : part;
+    };
     P.splits = (wide ? 8 : 4) / P.m_warps;
-    size_t smem = (size_t)P.splits * 2 * W::kTileBytes + (size_t)(P.merged ? kWindow : ((g.k_top + 3) & ~3)) * 4;
-    if (W::kQRegs == 0) smem += (size_t)P.m_warps * 16 * D * 2;
-    const size_t part = (size_t)(P.splits - 1) * P.m_warps * (D / 2 + 4) * 32 * 4;
-    if (part > smem) smem = part;
+    while (P.splits > 1 && bytes(P.splits) > kMaxDynamicSmem) --P.splits;
+    const size_t smem = bytes(P.splits);
     auto kern = wide ? attn_mma_kernel<D, BK, 8> : attn_mma_kernel<D, BK, 4>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_mma)");

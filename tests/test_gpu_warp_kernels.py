@@ -40,6 +40,11 @@ CASES = [  # spec changes, block_q, block_k (None: the spec's block), causal
     (dict(block=64, T=1003, n_q_heads=3, n_kv_heads=1, k_top=7), None, None, True),   # attention on tcgen05, d = 64: a row alone in its pair
     (dict(d=128, T=515, n_q_heads=7, n_kv_heads=1), None, None, True),                # blocks of 32: four rows across query blocks, three left over
     (dict(d=128, T=515, n_q_heads=5, n_kv_heads=1, k_top=512), None, None, False),    # mask rows as long as they go with four to a unit
+    (dict(d=128, T=515, k_top=7), 16, 64, True),                       # 16 tokens a row, 64 keys a tile: groups as shared memory allows
+    (dict(d=256, T=515, k_top=7), 16, 32, True),
+    (dict(d=256, T=515, k_top=7), 16, 64, False),
+    (dict(d=256, T=515, k_top=7), 32, 64, True),
+    (dict(d=256, T=2003, k_top=4, n_q_heads=8), 16, 64, True),         # the same with more rows than three an SM
     (dict(dtype="f32", T=1003, n_q_heads=8), None, None, True),
     (dict(dtype="f32", T=515, d=128, k_top=40, block=16), None, None, True),
     (dict(dtype="f32", T=300, block=64, n_q_heads=1, n_kv_heads=1, k_top=8), None, None, True),    # a row over eight CTAs
