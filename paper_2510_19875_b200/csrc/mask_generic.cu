@@ -470,13 +470,20 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
 
 constexpr size_t kMaxDynamicSmem = 227 * 1024 - 1024;  // (the kernel has a few static words too)
 
+// Shared memory of a row with W warps: what scoring takes, the slots, the list, a bit per slot.
+template <class P>
+size_t row_bytes(const Geom &g, int warps) {
+    const int n_max = (2 * g.k_top + 31) & ~31;
+    return P::smem_bytes(g, warps) + (size_t)(7 * n_max + n_max / 32) * 4;
+}
+
 template <class P, int W, bool kCluster = false>
 stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, int32_t *mask, float *score, WorkspaceHeader *ws,
                        cudaStream_t st, int n_cta = 1) {
     const long long rows = (long long)g.batch * g.H * g.n_qb;
     const int n_max = (2 * g.k_top + 31) & ~31;
     const size_t score_bytes = P::smem_bytes(g, W);
-    size_t smem = score_bytes + (size_t)(7 * n_max + n_max / 32) * 4;
+    size_t smem = row_bytes<P>(g, W);
     mk.use_cache = mk.n > 1 && smem + sizeof(float) * (size_t)g.N_k <= kMaxDynamicSmem;
     if (mk.use_cache) smem += sizeof(float) * (size_t)g.N_k;
     auto kern = mask_rows_kernel<P, W, kCluster>;
@@ -515,8 +522,10 @@ stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void 
     // 55.3 -> 43.7; the 64 rows above: 28.7 -> 24.6).
     int n_cta = 1;
     while (n_cta < 8 && rows * 2 * n_cta <= sm_count_or_default() && parts >= 8 * n_cta) n_cta *= 2;
-    if (n_cta > 1 && mk.n <= 1) return launch_w<P, kWideWarps, true>(g, mk, q, k, mask, score, ws, st, n_cta);
-    if (rows <= (parts >= kWideWarps ? 2 : 1) * (long long)sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
+    // (d = 256 in fp32, blocks above 32 and k above 624: sixteen warps do not fit, four do)
+    const bool fits = row_bytes<P>(g, kWideWarps) <= kMaxDynamicSmem;
+    if (fits && n_cta > 1 && mk.n <= 1) return launch_w<P, kWideWarps, true>(g, mk, q, k, mask, score, ws, st, n_cta);
+    if (fits && rows <= (parts >= kWideWarps ? 2 : 1) * (long long)sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
     return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
 }
 

@@ -51,6 +51,7 @@ CASES = [  # spec changes, block_q, block_k (None: the spec's block), causal
     (dict(dtype="f32", T=2047, n_q_heads=1, n_kv_heads=1, k_top=7), None, None, False),            # over two
     (dict(dtype="f32", T=300, d=256, block=64, k_top=3), None, None, False),
     (dict(dtype="f32", T=300, d=16, k_top=3), 1, 24, True),
+    (dict(dtype="f32", T=300, d=256, block=64, n_q_heads=1, n_kv_heads=1, k_top=1024), None, None, True),  # sixteen warps a row do not fit
 ]
 
 
@@ -88,6 +89,19 @@ def test_masks_and_attention_at_tile_edges(S, kw, bq, bk, causal):
             bh, qb = divmod(int(rid), nqb)
             lo, hi = qb * BQ, min(spec.T, qb * BQ + BQ)
             assert np.abs(out[bh, lo:hi] - ref[i, : hi - lo]).max() <= TOL[spec.dtype], rid
+
+
+@pytest.mark.parametrize("k_top", [624, 1024])  # the largest k at which sixteen warps a row fit, the largest there is
+@pytest.mark.parametrize("dtype,impl", [("f32", "auto"), ("bf16", "generic")])
+def test_masks_of_few_rows_at_the_largest_k(S, dtype, impl, k_top):
+    """d = 256 in blocks of 64 on the fp32-FMA form, 76 rows: one k, and two k in one call."""
+    spec = wl.WorkloadSpec("k", 12, 1, 1, 1, 4801, 256, 64, k_top, dtype)
+    w = wl.generate(spec)
+    assert_mask_parity(S, w, None, impl=impl)
+    q, k, _ = w.torch_tensors("cuda")
+    both = S.build_masks(q, k, [3, k_top], block_q=64, block_k=64, impl=impl).mask
+    for got, kq in zip(both, (3, k_top)):
+        assert torch.equal(got[..., :kq], S.build_mask(q, k, block_q=64, block_k=64, k_top=kq, impl=impl).mask)
 
 
 @pytest.mark.parametrize("bq", [64, 1])
