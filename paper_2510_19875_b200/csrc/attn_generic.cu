@@ -21,6 +21,7 @@ using namespace wp;
 
 constexpr int kMaxBlock = 64;
 constexpr int kKeys = 32;  // keys of a tile
+constexpr size_t kMaxDynamicSmem = 220 * 1024;
 
 template <typename T>
 __device__ __forceinline__ void store4(T *dst, float4 x);
@@ -332,10 +333,10 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
         const size_t sum = (size_t)m_warps * s * Sh::kPart * 4 + (n_cta > 1 ? (size_t)m_warps * QW * s * n_cta * 4 : 0);
         return walk > sum ? walk : sum;
     };
-    while (splits > 1 && bytes(splits) > 220 * 1024) splits /= 2;
+    while (splits > 1 && bytes(splits) > kMaxDynamicSmem) splits /= 2;
     const size_t smem = bytes(splits);
     auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kAsync, true> : attn_generic_kernel<T, D, QW, kAsync, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
     cudaLaunchConfig_t c = {};
     cudaLaunchAttribute cluster[1] = {};

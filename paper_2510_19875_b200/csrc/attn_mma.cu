@@ -427,7 +427,7 @@ stream_status launch(Params P, cudaStream_t st) {
     while (P.splits > 1 && bytes(P.splits) > kMaxDynamicSmem) --P.splits;
     const size_t smem = bytes(P.splits);
     auto kern = wide ? attn_mma_kernel<D, BK, 8> : attn_mma_kernel<D, BK, 4>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_mma)");
     kern<<<(unsigned)ctas, P.m_warps * P.splits * 32, smem, st>>>(P);
     e = cudaGetLastError();

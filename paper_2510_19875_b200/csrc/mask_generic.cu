@@ -487,7 +487,7 @@ stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, i
     mk.use_cache = mk.n > 1 && smem + sizeof(float) * (size_t)g.N_k <= kMaxDynamicSmem;
     if (mk.use_cache) smem += sizeof(float) * (size_t)g.N_k;
     auto kern = mask_rows_kernel<P, W, kCluster>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_rows)");
     cudaLaunchConfig_t c = {};
     cudaLaunchAttribute cluster[1] = {};

@@ -92,7 +92,8 @@ stream_status launch_vertical(const Geom &g, const int32_t *mask, const float *s
         return STREAM_ERR_UNSUPPORTED;
     }
     const size_t smem = (size_t)n_kb * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(vertical_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(vertical_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxBins * (int)sizeof(float));  // (not this call's need: another thread may be launching too)
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(vertical)");
     const int heads = g.batch * g.H;
     e = cudaMemsetAsync(vertical, 0, (size_t)heads * n_kb * sizeof(float), st);

@@ -102,6 +102,13 @@ __device__ __forceinline__ float score_of(unsigned key) {
     return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
 }
 
+// Allows a kernel the dynamic shared memory `most`, whatever this launch takes: the limit belongs to the kernel,
+// and one set to the need of a launch would be in the way of another thread's.
+template <class Kernel>
+cudaError_t allow_smem(Kernel *kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 inline bool rows_16_byte_aligned(const void *base, long long s_t, long long s_h, long long s_b, int elem) {
     const long long per = 16 / elem;
     return ((uintptr_t)base & 15) == 0 && s_t % per == 0 && s_h % per == 0 && s_b % per == 0;

@@ -2,6 +2,8 @@
 attention on tcgen05) against the CPU oracle, at the sizes where their tiles,
 remainders and launch shapes change: masks bit for bit outside near-ties, attention within
 tolerance, also on arbitrary masks (holes, empty rows, a block twice in a row)."""
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 import torch
@@ -203,3 +205,46 @@ def test_run_host_with_several_kv_heads_to_a_chunk(S, kw):
     ref = S.build_mask(q, k, k_top=spec.k_top, **blocks).mask
     assert torch.equal(mask, ref.cpu())
     assert (out.float() - S.sparse_attention(q, k, v, ref, **blocks).float().cpu()).abs().max().item() <= TOL[spec.dtype]
+
+
+@pytest.mark.parametrize("dtype,d,bq", [(torch.float32, 64, 64), (torch.bfloat16, 256, 64)])  # fp32 FMA, mma.sync
+def test_threads_with_different_sizes_on_one_kernel(S, dtype, d, bq):
+    """Threads with streams and outputs of their own launch the same kernels, some with rows of 2 blocks, some of 1024:
+    no thread's launch may take from another the shared memory that it needs."""
+    torch.manual_seed(3)
+    q, k, v = (torch.randn(1, 80, 64, d, device="cuda", dtype=dtype) for _ in range(3))
+
+    class Thread:
+        def __init__(self, k_top):
+            self.p = S.make_problem(q, k, block_q=bq, block_k=64, k_top=k_top)
+            self.stream = torch.cuda.Stream()
+            self.mask = torch.empty(1, 80, 64 // bq, k_top, dtype=torch.int32, device="cuda")
+            self.out, self.ws = torch.empty_like(q), torch.empty(256, dtype=torch.uint8, device="cuda")
+            self.vertical = torch.empty(1, 80, 1, device="cuda")
+
+        def once(self):
+            S.stream_build_mask(self.p, q, k, self.mask, None, self.ws, 256, self.stream)
+            S.stream_sparse_attention(self.p, q, k, v, self.mask, 0.0, self.out, self.stream)
+            S.stream_vertical_scores(self.p, self.mask, None, self.vertical, None, self.ws, 256, self.stream)
+
+        def run(self, n=2000):
+            for i in range(n):
+                self.once()
+                if i % 100 == 0:
+                    self.stream.synchronize()
+
+    threads = [Thread(k_top) for k_top in (2, 1024, 2, 1024)]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.once()
+    torch.cuda.synchronize()
+    want = [(t.mask.clone(), t.out.clone(), t.vertical.clone()) for t in threads]
+    for t in threads:
+        t.mask.fill_(-7), t.out.zero_(), t.vertical.zero_()
+    torch.cuda.synchronize()
+    with ThreadPoolExecutor(len(threads)) as pool:
+        for done in [pool.submit(t.run) for t in threads]:
+            done.result()
+    torch.cuda.synchronize()
+    for t, ref in zip(threads, want):
+        assert all(torch.equal(a, b) for a, b in zip((t.mask, t.out, t.vertical), ref))
