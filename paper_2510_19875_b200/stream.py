@@ -8,6 +8,7 @@ streams only.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 import struct
@@ -277,10 +278,12 @@ def make_problem(q: torch.Tensor, k: torch.Tensor, *, block_q: int, block_k: int
     (q_b, q_h, q_t, q_d), (k_b, k_h, k_t, k_d) = q.stride(), k.stride()
     if q_d != 1 or k_d != 1:
         raise ValueError("innermost stride must be 1")
-    # (packed at once: field by field the struct takes three times as long)
-    return StreamProblem.from_buffer_copy(_PROBLEM.pack(
-        qs[0], qs[1], ks[1], qs[2], qs[3], block_q, block_k, k_top, int(causal),
-        STREAM_F32 if dtype is torch.float32 else STREAM_BF16, IMPL[impl], q_b, q_h, q_t, k_b, k_h, k_t))
+    fields = (qs[0], qs[1], ks[1], qs[2], qs[3], block_q, block_k, k_top, int(causal),
+              STREAM_F32 if dtype is torch.float32 else STREAM_BF16, IMPL[impl], q_b, q_h, q_t, k_b, k_h, k_t)
+    try:  # (packed at once: field by field the struct takes three times as long)
+        return StreamProblem.from_buffer_copy(_PROBLEM.pack(*fields))
+    except struct.error:  # not whole numbers, or none that fit: as ctypes takes them
+        return StreamProblem(*fields)
 
 
 def n_query_blocks(p: StreamProblem) -> int:
@@ -361,7 +364,7 @@ def build_masks(q: torch.Tensor, k: torch.Tensor, k_list, *, block_q: int, block
     once per k and does not reuse tile scores between them)."""
     if not q.is_cuda or not k.is_cuda:
         raise ValueError("q and k must be CUDA tensors (there is no CPU path)")
-    ks = [int(x) for x in k_list]
+    ks = array.array("i", [int(x) for x in k_list])  # (an entry beyond 32 bits is an error)
     p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=max(ks), causal=causal, impl=impl)
     shape = (len(ks), p.batch, p.n_q_heads, n_query_blocks(p), p.k_top)
     mask = _empty(shape, torch.int32, q.device)
@@ -370,8 +373,7 @@ def build_masks(q: torch.Tensor, k: torch.Tensor, k_list, *, block_q: int, block
     if n_ws == 0:
         raise StreamError(STREAM_ERR_INVALID_ARG, stream_last_error())
     ws = _empty((n_ws,), torch.uint8, q.device)
-    k_host = (ctypes.c_int32 * len(ks))(*ks)
-    stream_build_mask_multi(p, q, k, len(ks), ctypes.addressof(k_host), mask, scores, ws, n_ws, stream)
+    stream_build_mask_multi(p, q, k, len(ks), ks.buffer_info()[0], mask, scores, ws, n_ws, stream)
     return MaskResult(mask, scores, ws)
 
 

@@ -187,3 +187,15 @@ def test_k_schedule_and_variable_k_reject_bad_arguments(S):
     with pytest.raises(S.StreamError) as e:  # a missing schedule is an error, not the fixed-k build
         S.stream_build_mask_var(p, 256, 256, None, 256, None, 256, 256, stream=0)
     assert e.value.status == S.STREAM_ERR_INVALID_ARG
+
+
+def test_sizes_beyond_32_bits_are_the_librarys_to_refuse(S):
+    import torch
+
+    q = torch.zeros(1, 4, 256, 128)
+    for bad in (2**31, 2**40, -2**33):
+        for kw in (dict(block_q=bad), dict(block_k=bad), dict(k_top=bad)):
+            p = S.make_problem(q, q, **{**dict(block_q=64, block_k=64, k_top=4), **kw})
+            assert S.stream_workspace_bytes(p) == 0
+    with pytest.raises(TypeError):
+        S.make_problem(q, q, block_q=64.0, block_k=64, k_top=4)

@@ -248,3 +248,10 @@ def test_threads_with_different_sizes_on_one_kernel(S, dtype, d, bq):
     torch.cuda.synchronize()
     for t, ref in zip(threads, want):
         assert all(torch.equal(a, b) for a, b in zip((t.mask, t.out, t.vertical), ref))
+
+
+def test_a_list_of_k_beyond_32_bits_is_refused(S):
+    q = torch.zeros(1, 1, 256, 64, device="cuda")
+    for bad in ([2**32 + 4, 2], [2, 2**31]):
+        with pytest.raises(OverflowError):
+            S.build_masks(q, q, bad, block_q=32, block_k=32)
