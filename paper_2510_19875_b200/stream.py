@@ -342,7 +342,7 @@ def build_mask(q: torch.Tensor, k: torch.Tensor, *, block_q: int, block_k: int, 
     if not q.is_cuda or not k.is_cuda:
         raise ValueError("q and k must be CUDA tensors (there is no CPU path)")
     p = make_problem(q, k, block_q=block_q, block_k=block_k, k_top=k_top, causal=causal, impl=impl)
-    header = _header_bytes(p)
+    header = _header_bytes(p) if workspace is None else 0  # (with a workspace the call itself says what is wrong with the problem)
     device, shape = q.device, (p.batch, p.n_q_heads, n_query_blocks(p), k_top)
     mask = mask_out if mask_out is not None else _empty(shape, torch.int32, device)
     scores = _empty(shape, torch.float32, device) if want_scores else None
@@ -354,7 +354,7 @@ def build_mask(q: torch.Tensor, k: torch.Tensor, *, block_q: int, block_k: int, 
         if not k_row.is_cuda or k_row.dtype != torch.int32 or not k_row.is_contiguous() or tuple(k_row.shape) != (shape[2],):
             raise ValueError(f"k_row must be a contiguous int32 CUDA tensor of shape ({shape[2]},)")
         stream_build_mask_var(p, q, k, k_row, mask, scores, workspace, workspace.numel(), stream)
-    return MaskResult(mask, scores, workspace, header)
+    return MaskResult(mask, scores, workspace, header or _header_bytes(p))
 
 
 def build_masks(q: torch.Tensor, k: torch.Tensor, k_list, *, block_q: int, block_k: int, causal: bool = True,

@@ -255,3 +255,13 @@ def test_a_list_of_k_beyond_32_bits_is_refused(S):
     for bad in ([2**32 + 4, 2], [2, 2**31]):
         with pytest.raises(OverflowError):
             S.build_masks(q, q, bad, block_q=32, block_k=32)
+
+
+def test_a_mask_build_with_a_workspace_says_why_it_is_refused(S):
+    q = torch.zeros(1, 1, 256, 64, device="cuda")
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    for kw, status in ((dict(k_top=2000), S.STREAM_ERR_UNSUPPORTED), (dict(k_top=2, block_k=65), S.STREAM_ERR_UNSUPPORTED),
+                       (dict(k_top=0), S.STREAM_ERR_INVALID_ARG)):
+        with pytest.raises(S.StreamError) as e:
+            S.build_mask(q, q, workspace=ws, **{**dict(block_q=32, block_k=32), **kw})
+        assert e.value.status == status
