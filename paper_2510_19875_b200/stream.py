@@ -132,12 +132,19 @@ def _addr(x):
     return None if x is None else int(x)
 
 
+try:  # the current stream by its handle: a Stream object for it takes 3 us to make
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream, _cuda_getDevice as _current_device
+except ImportError:  # (torch does not promise these names)
+    _raw_stream = None
+
+
 def _stream_handle(stream) -> int:
     if stream is None:
-        # the current device's current stream, by its handle: a Stream object for it takes 3 us to make
+        if _raw_stream is None:
+            return torch.cuda.current_stream().cuda_stream
         if not torch.cuda.is_initialized():
             torch.cuda.init()
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        return _raw_stream(_current_device())
     return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
 
 

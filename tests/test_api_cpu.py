@@ -199,3 +199,14 @@ def test_sizes_beyond_32_bits_are_the_librarys_to_refuse(S):
             assert S.stream_workspace_bytes(p) == 0
     with pytest.raises(TypeError):
         S.make_problem(q, q, block_q=64.0, block_k=64, k_top=4)
+
+
+def test_the_current_stream_without_torchs_private_names(S, monkeypatch):
+    import torch
+
+    class Stream:
+        cuda_stream = 77
+
+    monkeypatch.setattr(S, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    assert S._stream_handle(None) == 77 and S._stream_handle(5) == 5
