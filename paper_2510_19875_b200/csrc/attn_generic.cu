@@ -44,16 +44,35 @@ struct Shape {
 };
 
 // A [32][D] fp32 tile: keys n0 .. n0 + 31 of block r.
-template <typename T, int D, bool kAsync, bool kIsK>
+template <typename T, int D, Load kLoad, bool kIsK>
 __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T *base, int r, int n0, int thr, int n_thr) {
-    constexpr int per_row = D / 4;
-    for (int idx = thr; idx < kKeys * per_row; idx += n_thr) {
+    constexpr int per_row = D / 4, n_copies = kKeys * per_row;
+    if constexpr (kLoad == Load::kWide) {  // eight loads of a thread on their way at a time, not one value after the other
+        const long long tk0 = (long long)r * g.bk + n0;
+        const int n_in = (int)max(0ll, min((long long)min(g.bk - n0, kKeys), g.T - tk0));  // keys of the tile; the rest become zeros
+        constexpr int most = n_copies / 32 < 8 ? n_copies / 32 : 8;
+        for (int first = thr; first < n_copies; first += most * n_thr) {
+            uint2 x[most];
+#pragma unroll
+            for (int i = 0; i < most; ++i) {
+                const int idx = first + i * n_thr, n = idx / per_row, c = idx % per_row;
+                x[i] = n < n_in ? __ldg((const uint2 *)(base + (tk0 + n) * g.ks_t + c * 4)) : make_uint2(0, 0);
+            }
+#pragma unroll
+            for (int i = 0; i < most; ++i) {
+                const int idx = first + i * n_thr, n = idx / per_row, c = idx % per_row;
+                if (idx < n_copies) *(float4 *)(dst + n * D * 4 + ((kIsK ? c ^ (n & Shape<D, 32>::kSwz) : c) << 4)) = widen4(x[i]);
+            }
+        }
+        return;
+    }
+    for (int idx = thr; idx < n_copies; idx += n_thr) {
         const int n = idx / per_row, c = idx % per_row;
         const long long tk = (long long)r * g.bk + n0 + n;
         const bool in = n0 + n < g.bk && tk < g.T;  // the rest become zeros
         unsigned char *to = dst + n * D * 4 + ((kIsK ? c ^ (n & Shape<D, 32>::kSwz) : c) << 4);
         const T *src = base + (in ? tk : 0) * g.ks_t + c * 4;
-        if (kAsync) {
+        if (kLoad == Load::kCopy16) {
             cp_async16(smem_addr(to), src, in ? 16 : 0);
         } else {
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -61,15 +80,16 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
             *(float4 *)to = x;
         }
     }
-    if (kAsync) cp_async_commit();
+    if (kLoad == Load::kCopy16) cp_async_commit();
 }
 
 // kCluster: the row's tiles are dealt to the groups of all CTAs of a cluster, which read each other's parts at the end.
-template <typename T, int D, int QW, bool kAsync, bool kCluster>
+template <typename T, int D, int QW, Load kLoad, bool kCluster>
 __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, int splits, const T *__restrict__ q,
                                                            const T *__restrict__ k, const T *__restrict__ v,
                                                            const int32_t *__restrict__ mask, float scale, T *__restrict__ out) {
     using Sh = Shape<D, QW>;
+    constexpr bool kAsync = kLoad == Load::kCopy16;
     constexpr int RQ = QW / 8, RO = QW / 4, CO = D < 32 ? 1 : D / 32;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_n;
@@ -125,8 +145,8 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
 
     const int n_sub = (g.bk + kKeys - 1) / kKeys, n_tiles = s_n * n_sub;
     if (turn < n_tiles) {
-        fetch<T, D, kAsync, true>(g, ks, kp, list[turn / n_sub], turn % n_sub * kKeys, g_tid, g_thr);
-        fetch<T, D, kAsync, false>(g, vs, vp, list[turn / n_sub], turn % n_sub * kKeys, g_tid, g_thr);
+        fetch<T, D, kLoad, true>(g, ks, kp, list[turn / n_sub], turn % n_sub * kKeys, g_tid, g_thr);
+        fetch<T, D, kLoad, false>(g, vs, vp, list[turn / n_sub], turn % n_sub * kKeys, g_tid, g_thr);
     }
     for (int i0 = turn; i0 < n_tiles; i0 += groups) {
         const int r = list[i0 / n_sub], n0 = i0 % n_sub * kKeys, nxt = i0 + groups;
@@ -155,7 +175,7 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
             fma_channel<RQ>(s, a, x, &float4::w);
         }
         group_sync(1 + grp, g_thr);  // everybody is done with the K tile
-        if (nxt < n_tiles) fetch<T, D, kAsync, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
+        if (nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
         else if (kAsync) cp_async_commit();
         // online softmax; the four lanes of a query share its keys
         bool moved = false;
@@ -218,7 +238,7 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
             }
         }
         group_sync(1 + grp, g_thr);  // done with the V tile and with P
-        if (nxt < n_tiles) fetch<T, D, kAsync, false>(g, vs, vp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
+        if (nxt < n_tiles) fetch<T, D, kLoad, false>(g, vs, vp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
     }
     if (kAsync) cp_async_wait<0>();
 
@@ -314,7 +334,7 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
     }
 }
 
-template <typename T, int D, int QW, bool kAsync>
+template <typename T, int D, int QW, Load kLoad>
 stream_status launch_qw(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
                      cudaStream_t st) {
     using Sh = Shape<D, QW>;
@@ -335,7 +355,7 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     };
     while (splits > 1 && bytes(splits) > kMaxDynamicSmem) splits /= 2;
     const size_t smem = bytes(splits);
-    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kAsync, true> : attn_generic_kernel<T, D, QW, kAsync, false>;
+    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, true> : attn_generic_kernel<T, D, QW, kLoad, false>;
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
     cudaLaunchConfig_t c = {};
@@ -355,23 +375,25 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     return STREAM_OK;
 }
 
-template <typename T, int D, bool kAsync>
+template <typename T, int D, Load kLoad>
 stream_status launch(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
                      cudaStream_t st) {
     // 32 tokens a warp are 64 accumulators a lane at d = 64; not where half of them would be padding
-    if (D <= 64 && g.bq > 16) return launch_qw<T, D, 32, kAsync>(g, q, k, v, mask, scale, out, st);
-    return launch_qw<T, D, 16, kAsync>(g, q, k, v, mask, scale, out, st);
+    if constexpr (D <= 64) {
+        if (g.bq > 16) return launch_qw<T, D, 32, kLoad>(g, q, k, v, mask, scale, out, st);
+    }
+    return launch_qw<T, D, 16, kLoad>(g, q, k, v, mask, scale, out, st);
 }
 
-template <typename T, bool kAsync>
+template <typename T, Load kLoad>
 stream_status dispatch_d(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask, float scale, void *out,
                          cudaStream_t st) {
     switch (g.d) {
-        case 16: return launch<T, 16, kAsync>(g, q, k, v, mask, scale, out, st);
-        case 32: return launch<T, 32, kAsync>(g, q, k, v, mask, scale, out, st);
-        case 64: return launch<T, 64, kAsync>(g, q, k, v, mask, scale, out, st);
-        case 128: return launch<T, 128, kAsync>(g, q, k, v, mask, scale, out, st);
-        case 256: return launch<T, 256, kAsync>(g, q, k, v, mask, scale, out, st);
+        case 16: return launch<T, 16, kLoad>(g, q, k, v, mask, scale, out, st);
+        case 32: return launch<T, 32, kLoad>(g, q, k, v, mask, scale, out, st);
+        case 64: return launch<T, 64, kLoad>(g, q, k, v, mask, scale, out, st);
+        case 128: return launch<T, 128, kLoad>(g, q, k, v, mask, scale, out, st);
+        case 256: return launch<T, 256, kLoad>(g, q, k, v, mask, scale, out, st);
     }
     set_error("generic attention kernel: head dim %d not in {16, 32, 64, 128, 256}", g.d);
     return STREAM_ERR_UNSUPPORTED;
@@ -385,10 +407,13 @@ stream_status launch_attn_generic(const Geom &g, int dtype, const void *q, const
         set_error("generic attention kernel: block sizes up to %d (got %d, %d)", kMaxBlock, g.bq, g.bk);
         return STREAM_ERR_UNSUPPORTED;
     }
-    if (dtype != STREAM_F32) return dispatch_d<__nv_bfloat16, false>(g, q, k, v, mask, scale, out, st);
+    if (dtype != STREAM_F32) {
+        if (rows_aligned(k, g.ks_t, g.ks_h, g.ks_b, 2, 8) && ((uintptr_t)v & 7) == 0) return dispatch_d<__nv_bfloat16, Load::kWide>(g, q, k, v, mask, scale, out, st);
+        return dispatch_d<__nv_bfloat16, Load::kScalars>(g, q, k, v, mask, scale, out, st);
+    }
     const bool aligned = rows_16_byte_aligned(k, g.ks_t, g.ks_h, g.ks_b, 4) && ((uintptr_t)v & 15) == 0;
-    if (aligned) return dispatch_d<float, true>(g, q, k, v, mask, scale, out, st);
-    return dispatch_d<float, false>(g, q, k, v, mask, scale, out, st);
+    if (aligned) return dispatch_d<float, Load::kCopy16>(g, q, k, v, mask, scale, out, st);
+    return dispatch_d<float, Load::kScalars>(g, q, k, v, mask, scale, out, st);
 }
 
 }  // namespace stream

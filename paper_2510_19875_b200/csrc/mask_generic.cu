@@ -55,13 +55,14 @@ struct Allowed {
 // ----------------------------------------------------------------------------------------------
 // Lane (kq = lane / 4, kk = lane % 4) holds queries kq + 8 i (i < RQ) x keys kk + 4 j (j < 8): per
 // four channels RQ + 8 16-byte shared loads (conflict-free, broadcast over the lanes) feed 32 RQ FMA.
-template <typename T, int D, int RQ, bool kAsync>
+template <typename T, int D, int RQ, Load kLoad>
 struct FmaScore {
     using Elem = T;
+    static constexpr bool kRegisters = kLoad == Load::kWide || kLoad == Load::kScalars;
     static constexpr int kSQ = 8 * RQ, kCh = D < 32 ? D : 32, kChunks = D / kCh;
     static constexpr int kRowBytes = kCh * 4, kBufBytes = kKeysPerUnit * kRowBytes, kRing = 2;
     static constexpr int kSwz = kCh / 4 - 1;
-    static constexpr int kWarps = 4, kCtas = 4;  // warps of a row, CTAs an SM should hold
+    static constexpr int kWarps = 4, kCtas = kRegisters && RQ == 4 && D >= 64 ? 3 : 4;  // warps of a row, CTAs an SM should hold
 
     static int q_parts(const Geom &g) { return (g.bq + kSQ - 1) / kSQ; }
     static size_t smem_bytes(const Geom &g, int warps) {
@@ -104,29 +105,60 @@ struct FmaScore {
             x.ks = sub - x.qs * nk;
             return x;
         };
+        // Chunk q (channels cc) on its way: to its buffer, or (bf16) to registers, from where `put` takes it to the
+        // buffer behind the products of the chunk before. (Keys beyond the block are never looked at. Loaded and
+        // stored at once, element by element, a chunk waited for its loads.)
+        constexpr int kPerKey = kCh / 4, kCopies = kKeysPerUnit * kPerKey / 32;
+        uint2 raw[kRegisters ? kCopies : 1];
+        auto place = [&](int q, int n, int c4) { return (q & 1) * kBufBytes + n * kRowBytes + ((c4 ^ (n & kSwz)) << 4); };
         auto issue = [&](const Unit &x, int q, int cc) {
-            const int n0 = x.ks * kKeysPerUnit;
-            constexpr int per_key = kCh / 4;
+            const int n0 = x.ks * kKeysPerUnit, n_end = min(g.bk - n0, kKeysPerUnit);
             const int last = (int)min((long long)g.bk, g.T - (long long)x.r * g.bk) - n0 - 1;  // (the tile's last key inside T stands in for those beyond)
             const T *base = kp + ((long long)x.r * g.bk + n0) * g.ks_t + cc * kCh;
+            if constexpr (kLoad == Load::kCopy4) {
+                constexpr int n_step = 32 / kCh;  // keys a warp copies at a time
+                const int c = lane % kCh;
+                const unsigned dst = buf_s + (q & 1) * kBufBytes + (c & 3) * 4;
+                const long long step = n_step * g.ks_t;
+                int n = lane / kCh;
+                const T *src = base + (long long)min(n, last) * g.ks_t + c;
+                if (last + 1 >= n_end) {
+#pragma unroll 8
+                    for (; n < n_end; n += n_step, src += step) cp_async4(dst + n * kRowBytes + (((c >> 2) ^ (n & kSwz)) << 4), src);
+                } else {
+                    for (; n < n_end; n += n_step) {
+                        cp_async4(dst + n * kRowBytes + (((c >> 2) ^ (n & kSwz)) << 4), src);
+                        src = base + (long long)min(n + n_step, last) * g.ks_t + c;
+                    }
+                }
+            } else {
 #pragma unroll
-            for (int i = 0; i < kKeysPerUnit * per_key / 32; ++i) {
-                const int idx = i * 32 + lane, n = idx / per_key, c4 = idx % per_key;
-                const int dst = (q & 1) * kBufBytes + n * kRowBytes + ((c4 ^ (n & kSwz)) << 4);
-                if (n0 + n < g.bk) {  // (keys beyond the block are never looked at)
+                for (int i = 0; i < kCopies; ++i) {
+                    const int idx = i * 32 + lane, n = idx / kPerKey, c4 = idx % kPerKey;
                     const T *src = base + (long long)min(n, last) * g.ks_t + c4 * 4;
-                    if (kAsync) {
-                        cp_async16(buf_s + dst, src, 16);
-                    } else {
-                        *(float4 *)(buf + dst) = make_float4(to_float(src[0]), to_float(src[1]), to_float(src[2]), to_float(src[3]));
+                    if (n < n_end) {
+                        if constexpr (kLoad == Load::kCopy16) cp_async16(buf_s + place(q, n, c4), src, 16);
+                        else if constexpr (kLoad == Load::kWide) raw[i] = __ldg((const uint2 *)src);
+                        else raw[i] = load4(src);
                     }
                 }
             }
-            if (kAsync) cp_async_commit();
+            if (!kRegisters) cp_async_commit();
+        };
+        auto put = [&](int q) {
+#pragma unroll
+            for (int i = 0; i < kCopies; ++i) {
+                const int idx = i * 32 + lane, n = idx / kPerKey, c4 = idx % kPerKey;
+                *(float4 *)(buf + place(q, n, c4)) = widen4(raw[i]);
+            }
         };
 
         Unit cur = {}, ahead = {};  // the unit being scored, the one being fetched
-        if (n_chunks > 0) { ahead = unit(warp); issue(ahead, 0, 0); }
+        if (n_chunks > 0) {
+            ahead = unit(warp);
+            issue(ahead, 0, 0);
+            if constexpr (kRegisters) put(0);
+        }
         float acc[RQ][8];
         for (int q = 0; q < n_chunks; ++q) {
             const int cc = q % kChunks;
@@ -135,8 +167,8 @@ struct FmaScore {
                 if (cc == kChunks - 1) ahead = unit(warp + (q + 1) / kChunks * warps);
                 __syncwarp();  // every lane is done with the buffer's previous chunk
                 issue(ahead, q + 1, (q + 1) % kChunks);
-                if (kAsync) cp_async_wait<1>();
-            } else if (kAsync) {
+                if (!kRegisters) cp_async_wait<1>();
+            } else if (!kRegisters) {
                 cp_async_wait<0>();
             }
             __syncwarp();
@@ -165,6 +197,9 @@ struct FmaScore {
                 fma_channel<RQ>(acc, a, b, &float4::y);
                 fma_channel<RQ>(acc, a, b, &float4::z);
                 fma_channel<RQ>(acc, a, b, &float4::w);
+            }
+            if constexpr (kRegisters) {
+                if (q + 1 < n_chunks) put(q + 1);
             }
             if (cc == kChunks - 1) {
                 float best = -CUDART_INF_F;
@@ -529,25 +564,25 @@ stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void 
     return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
 }
 
-template <typename T, int RQ, bool kAsync>
+template <typename T, int RQ, Load kLoad>
 stream_status fma_d(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score,
                     WorkspaceHeader *ws, cudaStream_t st) {
     switch (g.d) {
-        case 16: return launch<FmaScore<T, 16, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
-        case 32: return launch<FmaScore<T, 32, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
-        case 64: return launch<FmaScore<T, 64, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
-        case 128: return launch<FmaScore<T, 128, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
-        case 256: return launch<FmaScore<T, 256, RQ, kAsync>>(g, mk, q, k, mask, score, ws, st);
+        case 16: return launch<FmaScore<T, 16, RQ, kLoad>>(g, mk, q, k, mask, score, ws, st);
+        case 32: return launch<FmaScore<T, 32, RQ, kLoad>>(g, mk, q, k, mask, score, ws, st);
+        case 64: return launch<FmaScore<T, 64, RQ, kLoad>>(g, mk, q, k, mask, score, ws, st);
+        case 128: return launch<FmaScore<T, 128, RQ, kLoad>>(g, mk, q, k, mask, score, ws, st);
+        case 256: return launch<FmaScore<T, 256, RQ, kLoad>>(g, mk, q, k, mask, score, ws, st);
     }
     set_error("generic mask kernel: head dim %d not in {16, 32, 64, 128, 256}", g.d);
     return STREAM_ERR_UNSUPPORTED;
 }
 
-template <typename T, bool kAsync>
+template <typename T, Load kLoad>
 stream_status fma_rq(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score,
                      WorkspaceHeader *ws, cudaStream_t st) {
-    if (g.bq <= 16) return fma_d<T, 2, kAsync>(g, mk, q, k, mask, score, ws, st);  // 16 queries per warp instead of 32
-    return fma_d<T, 4, kAsync>(g, mk, q, k, mask, score, ws, st);
+    if (g.bq <= 16) return fma_d<T, 2, kLoad>(g, mk, q, k, mask, score, ws, st);  // 16 queries per warp instead of 32
+    return fma_d<T, 4, kLoad>(g, mk, q, k, mask, score, ws, st);
 }
 
 template <int MT>
@@ -571,8 +606,8 @@ stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dty
     const int e = dtype == STREAM_F32 ? 4 : 2;
     const bool k_aligned = rows_16_byte_aligned(k, g.ks_t, g.ks_h, g.ks_b, e);
     if (dtype == STREAM_F32) {
-        if (k_aligned) return fma_rq<float, true>(g, mk, q, k, mask, score, ws, st);
-        return fma_rq<float, false>(g, mk, q, k, mask, score, ws, st);
+        if (k_aligned) return fma_rq<float, Load::kCopy16>(g, mk, q, k, mask, score, ws, st);
+        return fma_rq<float, Load::kCopy4>(g, mk, q, k, mask, score, ws, st);
     }
     // d = 16 and 32 would leave most of an mma's channels or lanes unused: they stay on the FMA form
     if (allow_mma && (g.d == 64 || g.d == 128 || g.d == 256) && k_aligned && g.ks_t < (1 << 24) &&
@@ -581,7 +616,8 @@ stream_status launch_mask_generic_multi(const Geom &g, const MultiK &mk, int dty
         if (g.bq <= 32) return mma_d<2>(g, mk, q, k, mask, score, ws, st);
         return mma_d<4>(g, mk, q, k, mask, score, ws, st);
     }
-    return fma_rq<__nv_bfloat16, false>(g, mk, q, k, mask, score, ws, st);
+    if (rows_aligned(k, g.ks_t, g.ks_h, g.ks_b, 2, 8)) return fma_rq<__nv_bfloat16, Load::kWide>(g, mk, q, k, mask, score, ws, st);
+    return fma_rq<__nv_bfloat16, Load::kScalars>(g, mk, q, k, mask, score, ws, st);
 }
 
 stream_status launch_mask_generic(const Geom &g, int dtype, bool allow_mma, const void *q, const void *k, int32_t *mask,

@@ -2,6 +2,8 @@
 #pragma once
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace stream {
@@ -12,6 +14,9 @@ __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)
 // 16 bytes global -> shared without a register; bytes = 0 writes zeros and reads nothing.
 __device__ __forceinline__ void cp_async16(unsigned dst, const void *src, int bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(unsigned dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -109,9 +114,27 @@ cudaError_t allow_smem(Kernel *kern, size_t most) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
+// How the fp32-FMA kernels bring keys and values to shared memory: 16 or 4 bytes at a time by cp.async (fp32),
+// 8 at a time through registers (bf16, widened on the way), element by element (rows off these boundaries).
+enum class Load { kCopy16, kCopy4, kWide, kScalars };
+
+// Four bf16 in a row, element by element; as fp32.
+__device__ __forceinline__ uint2 load4(const __nv_bfloat16 *src) {
+    const unsigned short *x = (const unsigned short *)src;
+    const unsigned a = __ldg(x), b = __ldg(x + 1), c = __ldg(x + 2), d = __ldg(x + 3);
+    return make_uint2(a | (b << 16), c | (d << 16));
+}
+__device__ __forceinline__ float4 widen4(uint2 x) {
+    return make_float4(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xffff0000u), __uint_as_float(x.y << 16),
+                       __uint_as_float(x.y & 0xffff0000u));
+}
+
+inline bool rows_aligned(const void *base, long long s_t, long long s_h, long long s_b, int elem, int bytes) {
+    const long long per = bytes / elem;
+    return ((uintptr_t)base & (bytes - 1)) == 0 && s_t % per == 0 && s_h % per == 0 && s_b % per == 0;
+}
 inline bool rows_16_byte_aligned(const void *base, long long s_t, long long s_h, long long s_b, int elem) {
-    const long long per = 16 / elem;
-    return ((uintptr_t)base & 15) == 0 && s_t % per == 0 && s_h % per == 0 && s_b % per == 0;
+    return rows_aligned(base, s_t, s_h, s_b, elem, 16);
 }
 
 // SMs of the current device (148 if it cannot be asked): only used to choose launch shapes.

@@ -54,6 +54,8 @@ CASES = [  # spec changes, block_q, block_k (None: the spec's block), causal
     (dict(dtype="f32", T=300, d=256, block=64, k_top=3), None, None, False),
     (dict(dtype="f32", T=300, d=16, k_top=3), 1, 24, True),
     (dict(dtype="f32", T=300, d=256, block=64, n_q_heads=1, n_kv_heads=1, k_top=1024), None, None, True),  # sixteen warps a row do not fit
+    (dict(d=16, T=1003, block=24), None, None, True),                  # bf16 on the fp32-FMA kernels
+    (dict(d=32, T=515, n_q_heads=16), 8, 64, False),
 ]
 
 
@@ -104,6 +106,28 @@ def test_masks_of_few_rows_at_the_largest_k(S, dtype, impl, k_top):
     both = S.build_masks(q, k, [3, k_top], block_q=64, block_k=64, impl=impl).mask
     for got, kq in zip(both, (3, k_top)):
         assert torch.equal(got[..., :kq], S.build_mask(q, k, block_q=64, block_k=64, k_top=kq, impl=impl).mask)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("d,bq,bk", [(16, 48, 24), (64, 20, 64), (128, 16, 48), (256, 64, 16)])
+@pytest.mark.parametrize("pitch,start", [(1, 0), (2, 2), (4, 4), (8, 1)])  # elements between rows, in front of the first
+def test_rows_off_the_vector_loads_give_the_same_bits(S, dtype, d, bq, bk, pitch, start):
+    """The fp32-FMA kernels read keys and values 16, 8 or 4 bytes at a time, or one by one, as the rows lie; the sums are the
+    same, and nothing beside the rows is used (NaN there)."""
+    torch.manual_seed(d + pitch)
+
+    def rows(heads):
+        room = torch.full((start + heads * 403 * (d + pitch),), float("nan"), device="cuda", dtype=dtype)
+        x = room[start:].view(1, heads, 403, d + pitch)[..., :d]
+        x.copy_(torch.randn(1, heads, 403, d, device="cuda"))
+        return x
+
+    q, k, v = rows(4), rows(2), rows(2)
+    kw = dict(block_q=bq, block_k=bk, impl="generic")
+    plain = [x.contiguous() for x in (q, k, v)]
+    got, ref = (S.build_mask(x, y, k_top=7, want_scores=True, **kw) for x, y in ((q, k), plain[:2]))
+    assert torch.equal(got.mask, ref.mask) and torch.equal(got.scores, ref.scores)
+    assert torch.equal(S.sparse_attention(q, k, v, ref.mask, **kw), S.sparse_attention(*plain, ref.mask, **kw))
 
 
 @pytest.mark.parametrize("bq", [64, 1])
