@@ -344,10 +344,15 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     // anyway. Fewer rows than half of the SMs: a row over two, four or eight CTAs, while each has a tile part for
     // every scheduler (28 rows, blocks of 64, k = 11, d = 64: 65.4 -> 34.8 us; 55 rows, blocks of 32, k = 9, d = 128:
     // 38.9 -> 30.7; 64 rows, blocks of 32, k = 8: 18.4 either way).
-    const int n_sm = sm_count_or_default(), tiles = g.k_top * ((g.bk + kKeys - 1) / kKeys);
+    // T may have fewer blocks than k_top, and what counts are those that are there: a CTA of a cluster has two tile
+    // parts at least, a group half of one (16 rows, T = 29, blocks of 48, k = 9, d = 16: 32 -> 10 us); with many
+    // rows an idle group takes another CTA's shared memory (2500 rows, k = 1, d = 128, rows off 16 bytes: 397 -> 316).
+    const int n_sm = sm_count_or_default(), n_sub = (g.bk + kKeys - 1) / kKeys, tiles = g.k_top * n_sub;
+    const int there = (int)std::min((long long)g.k_top, (g.T + g.bk - 1) / g.bk) * n_sub;
     int splits = (rows <= n_sm ? 8 : 4) / m_warps, n_cta = 1;
-    while (n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta) n_cta *= 2;
-    if (n_cta > 1 && splits > (tiles + n_cta - 1) / n_cta) splits = (tiles + n_cta - 1) / n_cta;
+    while (n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta && there >= 3 && there >= 2 * n_cta) n_cta *= 2;
+    if (n_cta > 1) splits = std::min({splits, (tiles + n_cta - 1) / n_cta, 2 * ((there + n_cta - 1) / n_cta)});
+    else if (rows > n_sm) splits = std::min(splits, rows > 4ll * n_sm ? there : 2 * there);
     auto bytes = [&](int s) {
         const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * (Sh::kPBytes + QW * 4) + (size_t)g.k_top * 4;
         const size_t sum = (size_t)m_warps * s * Sh::kPart * 4 + (n_cta > 1 ? (size_t)m_warps * QW * s * n_cta * 4 : 0);
