@@ -17,7 +17,9 @@
  *   - Tensors: Q is [batch, n_q_heads, T, d], K and V are [batch, n_kv_heads, T, d], addressed
  *     with the element strides in the problem struct (innermost stride 1). Query head h reads
  *     kv head h / (n_q_heads / n_kv_heads). dtype is fp32 or bf16 for Q, K, V and the attention
- *     output alike. Inputs must be finite.
+ *     output alike. Inputs must be finite, all of them: a kernel may multiply keys and values
+ *     that a row does not keep by a weight of zero (the tcgen05 and mma.sync kernels do), and zero
+ *     times an infinity or a NaN is a NaN.
  *   - A "row" is one (batch, query head, query block); there are ceil(T / block_q) query
  *     blocks. The mask is int32 [batch, n_q_heads, ceil(T / block_q), k_top], contiguous: per
  *     row the kept key-block indices (0-based; block r covers tokens r*block_k ..), strictly

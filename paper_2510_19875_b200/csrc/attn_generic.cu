@@ -5,7 +5,7 @@
 // accumulators would not fit) against 32 keys at a time; ceil(block_q / QW) warps make a group that
 // walks a sequence of key tiles, and the groups of a CTA take the row's tiles in turn, each with
 // softmax statistics and accumulators of its own, added up at the end. One K and one V buffer
-// per group, filled by cp.async: the next K tile arrives behind softmax and P V, the next V tile
+// per group, filled by cp.async (bf16, and rows off 16 bytes: through registers): the next K tile arrives behind softmax and P V, the next V tile
 // behind the next Q K^T. Inner loops read shared memory 16 bytes at a time, conflict-free:
 //   Q K^T   lane (kq, kk): queries kq + 8 i x keys kk + 4 j; QW / 8 + 8 loads per 4 QW FMA
 //   P V     lane (ro, co): QW / 4 consecutive queries x channels 4 co + 32 i, P kept key-major
@@ -346,7 +346,7 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     // 38.9 -> 30.7; 64 rows, blocks of 32, k = 8: 18.4 either way).
     // T may have fewer blocks than k_top, and what counts are those that are there: a CTA of a cluster has two tile
     // parts at least, a group half of one (16 rows, T = 29, blocks of 48, k = 9, d = 16: 32 -> 10 us); with many
-    // rows an idle group takes another CTA's shared memory (2500 rows, k = 1, d = 128, rows off 16 bytes: 397 -> 316).
+    // rows an idle group takes another CTA's shared memory (2500 rows, k = 1, d = 128, rows off 16 bytes: 397 -> 223).
     const int n_sm = sm_count_or_default(), n_sub = (g.bk + kKeys - 1) / kKeys, tiles = g.k_top * n_sub;
     const int there = (int)std::min((long long)g.k_top, (g.T + g.bk - 1) / g.bk) * n_sub;
     int splits = (rows <= n_sm ? 8 : 4) / m_warps, n_cta = 1;

@@ -23,9 +23,9 @@
 //           (d = 128 with blocks of 64 keys: attn_tok.cu.)
 // Bound: the latency of dependent steps at 8 to 16 warps per SM (issue slots 41 % busy, mma pipe 23
 // to 35 %); hence the register limits below (12 heads, T = 10007, blocks of 32, d = 128, k = 8: 180
-// us at two CTAs of four warps per SM, 152 at three; 3220 on the fp32-FMA kernel. 16 heads,
-// T = 8192, d = 64, k = 40, not causal: 669 us at two, 600 at four; 4640. Both have gone to attn_tc.cu since; left
-// are d = 256, blocks other than 32 and 64, block_q != block_k, per-token masks beside attn_tok.cu's).
+// us at two CTAs of four warps per SM, 152 at three, 3220 on the fp32-FMA kernel; 16 heads, T = 8192, d = 64,
+// k = 40, not causal: 669, 600 at four, 4640). It serves d = 256, blocks other than 32 and 64, block_q !=
+// block_k, and per-token masks beside attn_tok.cu's.
 #include "warp_common.cuh"
 
 namespace stream {

@@ -20,8 +20,7 @@
 // product takes it as its A operand. The logits are given back as soon as they are in registers.
 // A group has two buffers of logits and two of P: its next logits are there when it comes for them
 // (with one buffer 421 against 411 us at T = 16384), and P need not wait for the product before. (Three logit buffers with P in
-// their place instead hold a buffer through Q K^T, softmax and P V: 1470 clocks an entry, this
-// split 1330.)
+// their place instead hold a buffer through Q K^T, softmax and P V: 140 clocks an entry more.)
 //
 // `ref` is a per-token reference kept instead of the exact running maximum (bf16 P and fp32 sums
 // keep their relative precision whatever the reference, as long as nothing overflows): the
@@ -34,9 +33,9 @@
 // half of the channels each.
 //
 // What bounds it: an entry's products keep the tensor cores busy for 1050 clocks, its softmax work is
-// about 2000 of one group's, and the chip runs at its power limit; an entry takes 1500 clocks at
-// 1660 MHz. (With P in shared memory, 64 KB of stores and proxy fences, and one O per group: 1560 at
-// the lower clock.)
+// about 2000 of one group's, and the chip runs at its power limit; an entry takes 1350 to
+// 1450 clocks at 1600 to 1660 MHz. (With P in shared memory, 64 KB of stores and proxy fences, and one O
+// per group: 1560 at 1475 MHz.)
 //
 // Roles (384 threads): warp 0 brings the K and Q tiles by TMA, warp 2 the V tiles and, ahead of
 // everyone else, the pairs' mask rows; warp 1 issues the Q K^T chains and owns TMEM; warp 3 issues
@@ -117,7 +116,7 @@ struct Tail {
     float ref[128], sum[2][128];
 };
 // Dynamic shared memory: Q (two buffers; a pair's output is staged over its Q) | V stages | K stages |
-// Tail | mask rows [kMaskSlots][2][row_stride] (-1 where a row has nothing), the operands 1024-byte
+// Tail | mask rows [kMaskSlots][kRows][row_stride] (-1 where a row has nothing), the operands 1024-byte
 // aligned.
 constexpr int kFixedOperands = 2;  // Q; behind it the V stages, then the K stages
 constexpr int kMaxSmemPerCta = 232448;

@@ -76,7 +76,7 @@ bool mask_tok_supported(const Geom &g, int dtype);
 stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32_t *mask, float *score,
                               WorkspaceHeader *ws, cudaStream_t st);
 bool attn_tc_supported(const Geom &g, int dtype);  // d = 128, blocks of 64
-bool attn_tc_auto(const Geom &g, int dtype);       // and d = 64
+bool attn_tc_auto(const Geom &g, int dtype);       // and d = 64, and blocks of 32
 stream_status launch_attn_tc(const Geom &g, const void *q, const void *k, const void *v, const int32_t *mask,
                              float scale, void *out, cudaStream_t st);
 // bad_flag: device word that gets bit 0 set if a mask entry is >= the number of key blocks.

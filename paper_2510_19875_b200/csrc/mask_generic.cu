@@ -16,11 +16,10 @@
 // SM several rows: the 7 to 16 tiles of a level leave eight warps unequal work (12 heads,
 // T = 10007, blocks of 32, d = 128, bf16, k = 8: 310 us with eight warps a row, 222 with four; 8
 // heads, T = 5003, blocks of 32, d = 64, fp32: 246 and 216, and 181 since a unit's divisions are done
-// once and not with every chunk). The kernel this one replaced put 256
-// threads on one padded 64 x 64 tile at a time, with scalar loads and four barriers per tile: 5294
-// and 812 us for the same two. (The bf16 shape has gone to mask_tc.cu since; what is left to the MMA form is
-// d = 256, blocks other than 32 and 64, block_q != block_k, k above 64: 12 heads, T = 5676, d = 256, blocks of
-// 64, k = 33, mask and attention: 12192 -> 1065 us; 6 heads, T = 17577, blocks of 16: 37015 -> 793.)
+// once and not with every chunk). Against 256 threads on one padded 64 x 64 tile at a time, with scalar
+// loads and four barriers per tile: the fp32 shape 812 -> 181 us; with the attention, 12 heads, T = 5676, d = 256,
+// blocks of 64, k = 33, bf16: 12192 -> 1065; 6 heads, T = 17577, blocks of 16: 37015 -> 793. (The MMA form
+// serves d = 256, blocks other than 32 and 64, block_q != block_k and k above 64.)
 //
 // Follows Algorithm 2 with two exact shortcuts: branches without an allowed block are dropped (they
 // score -inf and can never displace a finite score), and a left branch inherits its parent's score
