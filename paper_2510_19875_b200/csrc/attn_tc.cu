@@ -87,7 +87,6 @@ struct Form {
 };
 constexpr int kMaskSlots = 2;               // pairs whose mask rows are resident
 constexpr int kMaxKTopTc = 1024;
-constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while pairs of several heads are walked
 constexpr float kLazySum = 68719476736.f;   // 2^36 = 64 * 2^30: the 64 P of an entry add up to more only if one of them exceeds 2^30 (its logit has outgrown the reference by 30 in log2 units)
 
 // The pair a CTA works on. h[r], qb[r]: head and query block of row r < R (R = 0: a place of the
@@ -146,12 +145,6 @@ __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail<F> *t
 template <class F>
 __device__ __forceinline__ int *mask_rows(Tail<F> *tl, const Params &P, int slot) {
     return reinterpret_cast<int *>(tl + 1) + slot * F::kRows * P.row_stride;
-}
-
-// A CTA's n-th place in the order of pairs. Every second round runs backwards, so that with pairs in
-// order of falling length every CTA gets about the same sum.
-__device__ __forceinline__ int nth_item(const Params &P, int n) {
-    return n * (int)gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
 }
 
 // The order: `group_heads` kv heads at a time, as many as have K and V in L2 together, and within
@@ -213,10 +206,6 @@ struct LoadStream {
     Ring ring, ms;
 };
 
-__device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
-    return __shfl_sync(0xffffffffu, (int)mbar_test_wait(bar, parity), 0) != 0;
-}
-
 // Opens the stream's pair (its mask rows must be resident) or closes it; true if it did.
 template <class F>
 __device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStream<F> &S) {
@@ -234,7 +223,7 @@ __device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStr
     if (elect_one()) mbar_arrive(smem_u32(&tl->m_empty[S.ms.idx]));
     __syncwarp();
     S.ms.advance(kMaskSlots);
-    S.id = nth_item(P, ++S.round);
+    S.id = nth_item(++S.round);
     S.e = -2;
 }
 template <class F>
@@ -264,7 +253,7 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
                                 unsigned k_smem) {
     LoadStream<F> S;
     S.round = 0;
-    S.id = nth_item(P, 0);
+    S.id = nth_item(0);
     S.e = -2;
     auto step = [&]() -> bool {
         if (S.e == -2) return open_pair(P, tl, S);
@@ -290,7 +279,7 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
     // as a rule: asked for behind the pair's first K tiles they came 1200 clocks late. (A pair's mask
     // slot stays until this warp has closed the pair on the K side, which a pair's Q precedes.)
     Ring qs, qm;
-    int q_round = 0, q_id = nth_item(P, 0);
+    int q_round = 0, q_id = nth_item(0);
     auto q_step = [&]() -> bool {
         if (q_id >= P.n_items || !probe_w(smem_u32(&tl->m_full[qm.idx]), qm.phase)) return false;
         if (tl->m_count[qm.idx] > 0) {
@@ -309,7 +298,7 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
             qs.advance(2);
         }
         qm.advance(kMaskSlots);
-        q_id = nth_item(P, ++q_round);
+        q_id = nth_item(++q_round);
         return true;
     };
     long long t_last = clock64();
@@ -328,9 +317,9 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
     const Geom &g = P.g;
     LoadStream<F> S;
     S.round = 0;
-    S.id = nth_item(P, 0);
+    S.id = nth_item(0);
     S.e = -2;
-    int m_round = 0, m_id = nth_item(P, 0);  // the next pair whose mask rows are due
+    int m_round = 0, m_id = nth_item(0);  // the next pair whose mask rows are due
     bool asked = false;                      // its first 32 entries are on their way to registers
     Item<F> it;
     int first[F::kRows];
@@ -378,7 +367,7 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         }
         __syncwarp();
         mw.advance(kMaskSlots);
-        m_id = nth_item(P, ++m_round);
+        m_id = nth_item(++m_round);
         asked = false;
         return true;
     };
@@ -415,7 +404,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
     Ring ks, ms, qs;
     unsigned cnt[2] = {0, 0};  // entries each group has had over the whole kernel
     const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
-    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
+    for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
         const int n_entries = tl->m_count[ms.idx];  // the issuers need no more than the count
         const unsigned q_lo = q_lo0 + qs.idx * (F::kOperand >> 4);
@@ -460,7 +449,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
     unsigned free_par = 1;  // (the first wait passes at once)
     // a row's MN-major V block has its two 64-channel halves kPart apart
     const unsigned v_lo = desc_lo_sw128(v_smem, F::kPart), d_tmem = tmem_base + F::kOCol;
-    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
+    for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
         const int n_entries = tl->m_count[ms.idx];
         for (int i = 0; i < n_entries; ++i) {
@@ -494,29 +483,6 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
         __syncwarp();
         ms.advance(kMaskSlots);
     }
-}
-
-// 2^x by the special-function unit (relative error about 2^-22; -inf gives 0).
-__device__ __forceinline__ float fast_exp2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Multiplies fp32 columns of this thread's TMEM lane by f, in place (every lane of the warp
-// takes part; lanes that need no change pass f = 1).
-template <int kColumns>
-__device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
-#pragma unroll 1
-    for (int c = 0; c < kColumns / 32; ++c) {
-        unsigned r[32];
-        tmem_ld_32x32_issue(taddr + c * 32, r);
-        tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
-        tmem_st_32x32_issue(taddr + c * 32, r);
-    }
-    tmem_st_wait();
 }
 
 // One softmax group: four warps, thread = TMEM lane `row`, token `mq` of the pair's row `half`, for the
@@ -562,7 +528,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail<F> *tl
         __syncwarp();
         staged = -1;
     };
-    for (int round = 0; nth_item(P, round) < P.n_items; ++round) {
+    for (int round = 0; nth_item(round) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 305)) return;
         const Item<F> &it = tl->m_item[ms.idx];
         const int h = it.h[r_own], qb = it.qb[r_own], b = it.b;
@@ -813,18 +779,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     }
     __syncwarp();
 
-    // Teardown. After an abort, copies and MMAs may still be in flight: leave them a bounded time
-    // to land before shared memory and TMEM are given back.
-    if (*(volatile int *)&tl->abort_flag) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) { }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc_512(tmem_base);
-    }
+    leave(&tl->abort_flag, tmem_base, warp == 1);
 }
 
 }  // namespace

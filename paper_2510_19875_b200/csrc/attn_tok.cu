@@ -83,7 +83,7 @@ constexpr unsigned kHi = desc_hi_sw128(1024);
 struct Params {
     Geom g;
     int n_items, n_tb;     // groups of 128 tokens, of one head
-    int group_heads;       // kv heads (of the batch * G) whose items are walked together
+    int group_heads;       // kv heads (of the batch * G) whose items are walked together, late tokens (most blocks) first
     const int32_t *mask;
     __nv_bfloat16 *out;
     float scale_log2;
@@ -91,15 +91,6 @@ struct Params {
 
 __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail *tl, unsigned code) {
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &g_attn_tok_status[0], &g_attn_tok_status[1], code);
-}
-__device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
-    return __shfl_sync(0xffffffffu, (int)mbar_test_wait(bar, parity), 0) != 0;
-}
-
-// A CTA's n-th item: late tokens (most blocks) first over as many kv heads as have K and V in L2
-// together, back and forth over the CTAs, as in attn_tc.cu.
-__device__ __forceinline__ int nth_item(const Params &P, int n) {
-    return n * (int)gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -109,7 +100,7 @@ __device__ void mask_role(const Params &P, Tail *tl, int lane) {
     const Geom &g = P.g;
     const int n_kb = (int)((g.T + kBlk - 1) / kBlk);
     Ring ms;
-    for (int round = 0, id; (id = nth_item(P, round)) < P.n_items; ++round) {
+    for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         const int per_group = P.group_heads * g.hpg * P.n_tb, grp = id / per_group, rem = id - grp * per_group;
         const int heads = min(P.group_heads, g.batch * g.G - grp * P.group_heads) * g.hpg;  // query heads of the group
         const int tb = P.n_tb - 1 - rem / heads, bh = grp * P.group_heads * g.hpg + rem % heads;  // (heads of a kv head are neighbours)
@@ -331,8 +322,7 @@ __device__ void pv_role(Tail *tl, unsigned v_smem, unsigned tmem_base) {
                 for (int part = 0; part < 2; ++part)  // the rounded weights, the rest
 #pragma unroll
                     for (int s4 = 0; s4 < 4; ++s4)    // 16 keys per step: 8 columns of packed bf16
-                        tc_mma_bf16_ta_masked(d_tmem, a_tmem + part * 32 + s4 * 8, b_lo + ((s4 * 2048) >> 4), kHi, kIdescPV,
-                                              (u | part | s4) != 0, 0u, 0u, 0u, 0u);
+                        tc_mma_bf16_ta(d_tmem, a_tmem + part * 32 + s4 * 8, b_lo + ((s4 * 2048) >> 4), kHi, kIdescPV, (u | part | s4) != 0);
                 tc_commit(smem_u32(&tl->p_free[gi][pb]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
             }
@@ -347,26 +337,6 @@ __device__ void pv_role(Tail *tl, unsigned v_smem, unsigned tmem_base) {
         __syncwarp();
         ms.advance(kMaskSlots);
     }
-}
-
-__device__ __forceinline__ float fast_exp2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Multiplies 128 fp32 columns of this thread's TMEM lane by f, in place (every lane takes part).
-__device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-        unsigned r[32];
-        tmem_ld_32x32_issue(taddr + c * 32, r);
-        tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
-        tmem_st_32x32_issue(taddr + c * 32, r);
-    }
-    tmem_st_wait();
 }
 
 __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, unsigned char *q_ptr, unsigned tmem_base, int t) {
@@ -499,7 +469,7 @@ __device__ void softmax_role(const Params &P, const CUtensorMap *to, Tail *tl, u
                     if (u > 0 && __any_sync(0xffffffffu, f != 1.f)) {  // what has been added up so far is brought to the new reference
                         if (!wait_w(smem_u32(&tl->p_free[grp ^ 1][other & 1u]), (other >> 1) & 1u, tl, 325)) return;
                         tc_fence_after();
-                        rescale_lane(lanes + kOCol, f);
+                        rescale_lane<kD>(lanes + kOCol, f);
                     }
                     l *= f;
                 }
@@ -614,21 +584,8 @@ attn_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         softmax_role(P, &tmap_out, tl, smem, tmem_base, (int)threadIdx.x - 128);
     }
     __syncwarp();
-    // Teardown. After an abort, copies and MMAs may still be in flight: leave them a bounded time
-    // to land before shared memory and TMEM are given back.
-    if (*(volatile int *)&tl->abort_flag) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) { }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc_512(tmem_base);
-    }
+    leave(&tl->abort_flag, tmem_base, warp == 1);
 }
-
-constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while several heads are walked
 
 }  // namespace
 

@@ -95,6 +95,13 @@ stream_status read_attn_tok_status(unsigned int out[2], cudaStream_t st);
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 
+// 2^x by the special-function unit (relative error about 2^-22; -inf gives 0).
+__device__ __forceinline__ float fast_exp2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Levels until every node is a single block: nodes start with at most ceil(N_k / k) blocks and
 // the larger half of n blocks has ceil(n / 2). With N_k > 1 the first level always runs (it is
 // where scores are first computed), matching n_it = ceil(log2 N_k) >= 1.

@@ -822,18 +822,7 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     }
     __syncwarp();
 
-    // Teardown. After an abort, copies and MMAs may still be in flight: give every stage and slot
-    // barrier a bounded chance to complete before shared memory and TMEM are given back.
-    if (*(volatile int *)&tl->abort_flag) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < (1ll << 22)) { }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc_512(tmem_base);
-    }
+    leave(&tl->abort_flag, tmem_base, warp == 1);
 }
 
 // ----------------------------------------------------------------------------------------------

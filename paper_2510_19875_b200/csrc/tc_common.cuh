@@ -59,6 +59,11 @@ __device__ __forceinline__ bool mbar_test_wait(unsigned bar, unsigned parity) {
     return ok != 0;
 }
 
+// The same for a whole converged warp: lane 0's answer.
+__device__ __forceinline__ bool probe_w(unsigned bar, unsigned parity) {
+    return __shfl_sync(0xffffffffu, (int)mbar_test_wait(bar, parity), 0) != 0;
+}
+
 // The part of a bounded wait on an mbarrier phase behind its first look. Returns false if the CTA is aborting, or if this wait ran
 // out, in which case it raises the CTA's abort flag and records `code` (first one wins) with the
 // block index in the two error words.
@@ -160,18 +165,6 @@ __device__ __forceinline__ void tc_mma_bf16_ta(unsigned d_tmem, unsigned a_tmem,
         : "memory");
 }
 
-// With A from TMEM, M = 128 and an output-lane mask: bit i of the
-// 128-bit vector {m0 (lanes 0..31), m1, m2, m3} set = accumulator lane i is left untouched.
-__device__ __forceinline__ void tc_mma_bf16_ta_masked(unsigned d_tmem, unsigned a_tmem, unsigned b_lo, unsigned b_hi,
-                                                      unsigned idesc, unsigned accumulate, unsigned m0, unsigned m1,
-                                                      unsigned m2, unsigned m3) {
-    asm volatile(
-        "{\n.reg .pred p;\n.reg .b64 db;\nmov.b64 db, {%2, %3};\nsetp.ne.b32 p, %5, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, {%6, %7, %8, %9}, p;\n}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(m0), "r"(m1), "r"(m2), "r"(m3)
-        : "memory");
-}
-
 // Two fp32 in a register pair: one instruction for both.
 __device__ __forceinline__ unsigned long long pack_u32x2(unsigned a, unsigned b) {
     unsigned long long r;
@@ -245,6 +238,22 @@ __device__ __forceinline__ void tmem_ld_32x8_issue(unsigned taddr, unsigned *r) 
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)
                  : "memory");
+}
+
+// Multiplies fp32 columns of this thread's TMEM lane by f, in place (every lane of the warp
+// takes part; lanes that need no change pass f = 1).
+template <int kColumns>
+__device__ __forceinline__ void rescale_lane(unsigned taddr, float f) {
+#pragma unroll 1
+    for (int c = 0; c < kColumns / 32; ++c) {
+        unsigned r[32];
+        tmem_ld_32x32_issue(taddr + c * 32, r);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
+        tmem_st_32x32_issue(taddr + c * 32, r);
+    }
+    tmem_st_wait();
 }
 
 // Maximum of three in one instruction.
@@ -399,6 +408,28 @@ __device__ __forceinline__ void select_topk_of(const bool (&have)[n], const floa
         const bool equal = have[i] && key[i] == thr;
         keep[i] = have[i] && (key[i] > thr || (equal && place < missing));
         place += equal ? 1 : 0;
+    }
+}
+
+// A CTA's n-th place in an order of items. Every second round runs backwards, so that with items in
+// order of falling length every CTA gets about the same sum.
+__device__ __forceinline__ int nth_item(int n) {
+    return n * (int)gridDim.x + ((n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+}
+constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 126 MB L2 while items of several heads are walked
+
+// The end of a kernel, of all its threads; `owner`: the warp that has allocated TMEM. After an abort, copies and
+// MMAs may still be in flight: they have a bounded time to land before shared memory and TMEM are given back.
+__device__ __forceinline__ void leave(const int *abort_flag, unsigned tmem_base, bool owner) {
+    if (*(const volatile int *)abort_flag) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1ll << 22)) { }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (owner) {
+        tc_fence_after();
+        tmem_dealloc_512(tmem_base);
     }
 }
 

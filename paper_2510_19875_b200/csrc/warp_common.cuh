@@ -35,13 +35,6 @@ __device__ __forceinline__ float warp_max(float x) {
     return r;
 }
 
-// 2^x by the special-function unit (relative error about 2^-22; -inf gives 0).
-__device__ __forceinline__ float fast_exp2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // One channel of an RQ x 8 tile: acc += a b^T. (Channel by channel, so that an accumulator's next
 // addition is 8 RQ instructions away; four in a row on one accumulator wait for each other.)
 template <int RQ>
