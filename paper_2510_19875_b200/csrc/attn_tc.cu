@@ -34,7 +34,8 @@
 //
 // What bounds it: an entry's products keep the tensor cores busy for 1050 clocks, its softmax work is
 // about 2000 of one group's, and the chip runs at its power limit; an entry takes 1350 to
-// 1450 clocks at 1600 to 1660 MHz. (With P in shared memory, 64 KB of stores and proxy fences, and one O
+// 1450 clocks at 1600 to 1660 MHz. (What an issuing warp does between two chains counts all the same: one look at both of
+// its barriers instead of two, and one commit fewer, 16384 tokens, k = 16: 408 -> 396 us; 131072, k = 32: 6190 -> 6070.) (With P in shared memory, 64 KB of stores and proxy fences, and one O
 // per group: 1560 at 1475 MHz.)
 //
 // Roles (384 threads): warp 0 brings the K and Q tiles by TMA, warp 2 the V tiles and, ahead of
@@ -77,6 +78,9 @@ struct Form {
     // stage is held from its load until the product of its entry is complete, a whole softmax later:
     // V three, K two), or four when the mask rows are long.
     static constexpr int kMaxKStages = kD == 128 ? 2 : 6, kMaxVStages = kD == 128 ? 3 : 6;
+    // Two K stages: one is free when the logits of the entry before last are there, which their own barrier says (its next
+    // use is at least two entries later). More: a barrier of the stage's own, and a commit more for the issuing warp.
+    static constexpr bool kKByLogits = kMaxKStages == 2;
     // TMEM columns: the two logit buffers of group g at 128 g and 64 behind, its P at 256 + 64 g (two
     // buffers, the second 32 behind, or the two parts of one), O at 384.
     static constexpr int kPBufs = kSplit ? 1 : 2;
@@ -139,6 +143,14 @@ struct Params {
 template <class F>
 __device__ __forceinline__ bool wait_w(unsigned bar, unsigned parity, Tail<F> *tl, unsigned code) {
     return mbar_wait_warp(bar, parity, &tl->abort_flag, &g_attn_status[0], &g_attn_status[1], code);
+}
+
+// The same for two barriers, in one look where both phases are complete: for an issuing warp, which has a chain to
+// issue every 700 clocks, each look of its own was 100 of them.
+template <class F>
+__device__ __forceinline__ bool wait_both_w(unsigned bar_a, unsigned parity_a, unsigned code_a, unsigned bar_b, unsigned parity_b, unsigned code_b, Tail<F> *tl) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_both(bar_a, parity_a, bar_b, parity_b))) return true;
+    return wait_w(bar_a, parity_a, tl, code_a) && wait_w(bar_b, parity_b, tl, code_b);
 }
 
 // Shared copy of the mask rows of the pair in slot `slot`: [kRows][row_stride] ints behind the Tail.
@@ -255,11 +267,20 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
     S.round = 0;
     S.id = nth_item(0);
     S.e = -2;
+    // (kKByLogits) the last two entries, the older one in the stage that is next: the barrier of their logits (0: none), its phase
+    unsigned cnt[2] = {0, 0}, bar_old = 0, bar_new = 0, par_old = 0, par_new = 0;
     auto step = [&]() -> bool {
         if (S.e == -2) return open_pair(P, tl, S);
         if (S.e >= S.n) { close_pair(P, tl, S); return true; }
         // a K stage is free once the logits computed from it are complete
-        if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
+        if constexpr (F::kKByLogits) {
+            if (bar_old != 0 && !probe_w(bar_old, par_old)) return false;
+            const unsigned gi = (unsigned)(S.e & 1), use = gi ? cnt[1]++ : cnt[0]++;
+            bar_old = bar_new; par_old = par_new;
+            bar_new = smem_u32(&tl->s_full[gi][use & 1u]); par_new = (use >> 1) & 1u;
+        } else {
+            if (!probe_w(smem_u32(&tl->k_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
+        }
         if (elect_one()) {
             // [half][row][keys][128 B]; a row without a block at an entry gets block 0, its logits are masked out
             const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * F::kOperand;
@@ -413,9 +434,8 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
             qs.advance(2);
         }
         for (int i = 0; i < n_entries; ++i) {
-            if (!wait_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, tl, 202)) return;
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++;  // entry i of a pair belongs to group i % 2
-            if (!wait_w(smem_u32(&tl->s_free[gi][use & 1u]), ((use >> 1) & 1u) ^ 1u, tl, 203)) return;
+            if (!wait_both_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, 202, smem_u32(&tl->s_free[gi][use & 1u]), ((use >> 1) & 1u) ^ 1u, 203, tl)) return;
             tc_fence_after();
             const unsigned d_tmem = tmem_base + gi * 128 + (use & 1u) * 64;
             const unsigned b_lo = k_lo + ks.idx * (F::kOperand >> 4);
@@ -429,7 +449,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
                             tc_mma_bf16_split(d_tmem + r * kRowLanes, q_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK,
                                               b_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK, F::kIdescQK, (c | k4) != 0);
                 tc_commit(smem_u32(&tl->s_full[gi][use & 1u]));
-                tc_commit(smem_u32(&tl->k_empty[ks.idx]));
+                if (!F::kKByLogits) tc_commit(smem_u32(&tl->k_empty[ks.idx]));
             }
             __syncwarp();
             ks.advance(P.n_k_stages);
@@ -453,9 +473,9 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
         const int n_entries = tl->m_count[ms.idx];
         for (int i = 0; i < n_entries; ++i) {
-            if (!wait_w(smem_u32(&tl->v_full[vs.idx]), vs.phase, tl, 205)) return;
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use % F::kPBufs;
-            if (!wait_w(smem_u32(&tl->p_full[gi][pb]), (use / F::kPBufs) & 1u, tl, 204)) return;  // also: O rescaled if it had to be
+            // (P is there: also, O is rescaled if it had to be)
+            if (!wait_both_w(smem_u32(&tl->v_full[vs.idx]), vs.phase, 205, smem_u32(&tl->p_full[gi][pb]), (use / F::kPBufs) & 1u, 204, tl)) return;
             if (i == 0) {
                 if (!wait_w(smem_u32(&tl->o_free), free_par, tl, 206)) return;  // the previous pair's O has been read
                 free_par ^= 1;

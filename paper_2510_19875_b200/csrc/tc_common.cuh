@@ -35,6 +35,18 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity) {
     return ok != 0;
 }
 
+// Two barriers' phases at once: the second look is on its way while the first is.
+__device__ __forceinline__ bool mbar_try_wait_both(unsigned bar_a, unsigned parity_a, unsigned bar_b, unsigned parity_b) {
+    unsigned ok;
+    asm volatile(
+        "{\n.reg .pred p, q;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 q, [%3], %4;\nand.pred p, p, q;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar_a), "r"(parity_a), "r"(bar_b), "r"(parity_b)
+        : "memory");
+    return ok != 0;
+}
+
 // The same, but the hardware may keep the thread suspended for up to `ns` nanoseconds while the
 // phase is incomplete, instead of returning at once: far fewer shared-memory transactions than
 // polling, and the shared-memory port is what these kernels run against.
