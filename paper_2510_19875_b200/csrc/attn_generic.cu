@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
     constexpr int RQ = QW / 8, RO = QW / 4, CO = D < 32 ? 1 : D / 32;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_n;
+    after_previous_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = warp / m_warps, mw = warp % m_warps, g_thr = m_warps * 32, g_tid = tid - grp * g_thr;
     const int kq = lane >> 2, kk = lane & 3;   // Q K^T
@@ -363,19 +364,8 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, true> : attn_generic_kernel<T, D, QW, kLoad, false>;
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
-    cudaLaunchConfig_t c = {};
-    cudaLaunchAttribute cluster[1] = {};
-    c.gridDim = dim3((unsigned)(rows * n_cta));
-    c.blockDim = dim3((unsigned)(m_warps * splits * 32));
-    c.dynamicSmemBytes = smem;
-    c.stream = st;
-    cluster[0].id = cudaLaunchAttributeClusterDimension;
-    cluster[0].val.clusterDim.x = (unsigned)n_cta;
-    cluster[0].val.clusterDim.y = cluster[0].val.clusterDim.z = 1;
-    c.attrs = cluster;
-    c.numAttrs = n_cta > 1 ? 1 : 0;
-    e = cudaLaunchKernelEx(&c, kern, g, m_warps, splits, (const T *)q, (const T *)k, (const T *)v, mask, scale, (T *)out);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = launch_kernel(kern, (unsigned)(rows * n_cta), (unsigned)(m_warps * splits * 32), smem, st, (unsigned)n_cta, g, m_warps, splits, (const T *)q,
+                      (const T *)k, (const T *)v, mask, scale, (T *)out);
     if (e != cudaSuccess) return cuda_fail(e, "attn_generic launch");
     return STREAM_OK;
 }

@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 4 ? ctas_per_sm<D, BK>() 
     __shared__ unsigned row_bits[kMaxRows][kWindow / 32];  // merged: the window's blocks each row keeps
     __shared__ unsigned any_bits[kWindow / 32];
     const Geom &g = P.g;
+    after_previous_kernel();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, t = lane & 3;
     const int grp = warp / P.m_warps, mw = warp % P.m_warps, g_thr = P.m_warps * 32, g_tid = tid - grp * g_thr;
 
@@ -429,8 +430,7 @@ stream_status launch(Params P, cudaStream_t st) {
     auto kern = wide ? attn_mma_kernel<D, BK, 8> : attn_mma_kernel<D, BK, 4>;
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_mma)");
-    kern<<<(unsigned)ctas, P.m_warps * P.splits * 32, smem, st>>>(P);
-    e = cudaGetLastError();
+    e = launch_kernel(kern, (unsigned)ctas, P.m_warps * P.splits * 32, smem, st, 1, P);
     if (e != cudaSuccess) return cuda_fail(e, "attn_mma launch");
     return STREAM_OK;
 }

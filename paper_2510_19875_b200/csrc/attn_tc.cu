@@ -785,6 +785,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = tl->tmem_base;
+    after_previous_kernel();
 
     if (warp == 0) {
         k_producer_role(P, &tmap_q, &tmap_k, tl, q_smem, k_smem);
@@ -855,8 +856,7 @@ stream_status launch(const Geom &g, const void *q, const void *k, const void *v,
     cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmemPerCta);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_tc)");
     const int grid = (int)(n_items < n_sm ? n_items : n_sm);
-    attn_tc_kernel<F><<<grid, kThreads, smem_bytes, st>>>(tq, tk, tv, to, P);
-    e = cudaGetLastError();
+    e = launch_kernel(attn_tc_kernel<F>, grid, kThreads, smem_bytes, st, 1, tq, tk, tv, to, P);
     if (e != cudaSuccess) return cuda_fail(e, "attn_tc launch");
     return STREAM_OK;
 }

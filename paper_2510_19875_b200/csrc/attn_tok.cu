@@ -572,6 +572,7 @@ attn_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = tl->tmem_base;
+    after_previous_kernel();
     if (warp == 0) {
         producer_role(P, &tmap_q, &tmap_k, &tmap_v, tl, q_smem, k_smem, v_smem);
     } else if (warp == 1) {
@@ -622,8 +623,7 @@ stream_status launch_attn_tok(const Geom &g, const void *q, const void *k, const
     cudaError_t e = cudaFuncSetAttribute(attn_tok_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_tok)");
     const int grid = (int)(n_items < n_sm ? n_items : n_sm);
-    attn_tok_kernel<<<grid, kThreads, kSmemBytes, st>>>(tq, tk, tv, to, P);
-    e = cudaGetLastError();
+    e = launch_kernel(attn_tok_kernel, grid, kThreads, kSmemBytes, st, 1, tq, tk, tv, to, P);
     if (e != cudaSuccess) return cuda_fail(e, "attn_tok launch");
     return STREAM_OK;
 }

@@ -347,6 +347,7 @@ mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P
     // several k: scores of this row by key block, NaN = not scored yet (a score does not depend on k)
     float *cache = mk.use_cache ? (float *)(keep + n_max / 32) : nullptr;
     __shared__ int s_list, s_valid, s_all;  // s_all (clusters): listed by any of the CTAs
+    after_previous_kernel();
     const unsigned n_cta = kCluster ? cluster_size() : 1u, cta = kCluster ? cluster_rank() : 0u;
 
     const int tid = threadIdx.x, n_thr = blockDim.x;
@@ -523,19 +524,8 @@ stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, i
     auto kern = mask_rows_kernel<P, W, kCluster>;
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_rows)");
-    cudaLaunchConfig_t c = {};
-    cudaLaunchAttribute cluster[1] = {};
-    c.gridDim = dim3((unsigned)(rows * n_cta));
-    c.blockDim = dim3(W * 32);
-    c.dynamicSmemBytes = smem;
-    c.stream = st;
-    cluster[0].id = cudaLaunchAttributeClusterDimension;
-    cluster[0].val.clusterDim.x = (unsigned)n_cta;
-    cluster[0].val.clusterDim.y = cluster[0].val.clusterDim.z = 1;
-    c.attrs = cluster;
-    c.numAttrs = kCluster ? 1 : 0;
-    e = cudaLaunchKernelEx(&c, kern, g, mk, (int)score_bytes, n_max, (const typename P::Elem *)q, (const typename P::Elem *)k, mask, score, ws);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = launch_kernel(kern, (unsigned)(rows * n_cta), W * 32, smem, st, (unsigned)n_cta, g, mk, (int)score_bytes, n_max, (const typename P::Elem *)q,
+                      (const typename P::Elem *)k, mask, score, ws);
     if (e != cudaSuccess) return cuda_fail(e, "mask_rows launch");
     return STREAM_OK;
 }

@@ -804,6 +804,7 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = tl->tmem_base;
+    after_previous_kernel();
 
     // One call of each role, so that its code is in the instruction cache once, and the roles dealt so
     // that a scheduler (warp % 4) runs little beside its two epilogue warps: three copies of the
@@ -875,8 +876,7 @@ template <class S>
 cudaError_t launch(int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
     static_assert(kSmemBytes<S> <= 232448, "one CTA's shared memory");
     const cudaError_t e = cudaFuncSetAttribute(mask_tc_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<S>);
-    if (e == cudaSuccess) mask_tc_kernel<S><<<grid, kThreads, kSmemBytes<S>, st>>>(tq, tk, P);
-    return e;
+    return e == cudaSuccess ? launch_kernel(mask_tc_kernel<S>, grid, kThreads, kSmemBytes<S>, st, 1, tq, tk, P) : e;
 }
 
 template <int kD, int kBlk>
@@ -943,8 +943,6 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     if (mk.n >= 1) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, true>>(grid, st, tq, tk, P);
     else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64>(g, sp, st, tq, tk, P) : launch_rows<128, 32>(g, sp, st, tq, tk, P);
     else e = g.bq == 64 ? launch_rows<64, 64>(g, sp, st, tq, tk, P) : launch_rows<64, 32>(g, sp, st, tq, tk, P);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tc)");
-    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "mask_tc launch");
     return STREAM_OK;
 }

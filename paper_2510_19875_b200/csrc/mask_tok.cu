@@ -139,6 +139,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = tl->tmem_base;
+    after_previous_kernel();
 
     // the level's wanted blocks: a byte each while they fit (plain stores, the same value from all), else a bit
     unsigned char *const wanted = (unsigned char *)bitmap;
@@ -530,8 +531,7 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tok)");
     const int grid = (int)(n_items < n_sm ? n_items : n_sm);
-    kern<<<grid, kThreads, kSmemBytes, st>>>(tq, tk, P);
-    e = cudaGetLastError();
+    e = launch_kernel(kern, grid, kThreads, kSmemBytes, st, 1, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tok launch");
     return STREAM_OK;
 }
