@@ -114,6 +114,7 @@ struct Tail {
     int first_blk[S::kMaxJobs], jobs_blk[kR][S::kMaxRowJobs];
     float first_part[2][kR][S::kMaxJobs][S::kParts], part[kR][S::kMaxRowJobs][S::kParts];
     float no_part;   // (written before a list's first tile, not read)
+    alignas(16) unsigned keys[kR][S::kNodes == 1 ? 64 : 4];  // a row's candidates while it ranks them
     int node_f[kR][32 * S::kNodes], node_l[kR][32 * S::kNodes];
     float node_s[kR][32 * S::kNodes];
 };
@@ -697,7 +698,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
             }
             bool keep[2 * kNodes];
             if constexpr (kNodes == 1) {
-                const Keep kp = select_topk(has[0], sc[0], has[1], sc[1], kq, lane);
+                const Keep kp = select_topk_counting(has[0], sc[0], has[1], sc[1], kq, level == 0 ? kq : n_nodes, lane, tl->keys[r]);
                 keep[0] = kp.l; keep[1] = kp.r;
             } else {
                 select_topk_of<2 * kNodes>(has, sc, kq, lane, keep);
