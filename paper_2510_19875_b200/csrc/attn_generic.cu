@@ -84,8 +84,13 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
 }
 
 // kCluster: the row's tiles are dealt to the groups of all CTAs of a cluster, which read each other's parts at the end.
-template <typename T, int D, int QW, Load kLoad, bool kCluster>
-__global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, int splits, const T *__restrict__ q,
+// kFour: the build for four warps and three CTAs an SM (four at d = 32), within their registers. Unbounded, ptxas takes
+// over 200 a thread at d = 64 and two CTAs are all an SM holds; at d = 128 and 256 a bound of one CTA lets it take more
+// than it would (8 heads, 5000 tokens, d = 128, blocks of 32: 294 -> 274 us; blocks of 16, k = 16: 482 -> 427).
+// p_in_k: P lies over the group's K tile, and both next tiles are fetched behind P V: what a warp then waits for its tiles the other
+// two CTAs' warps cover.
+template <typename T, int D, int QW, Load kLoad, bool kCluster, bool kFour>
+__global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) : (D >= 128 ? 1 : 0)) attn_generic_kernel(Geom g, int m_warps, int splits, bool p_in_k, const T *__restrict__ q,
                                                            const T *__restrict__ k, const T *__restrict__ v,
                                                            const int32_t *__restrict__ mask, float scale, T *__restrict__ out) {
     using Sh = Shape<D, QW>;
@@ -111,8 +116,8 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
     float *Qs = (float *)smem;
     unsigned char *ks = smem + (size_t)m_warps * QW * D * 4 + (size_t)grp * 2 * Sh::kTileBytes, *vs = ks + Sh::kTileBytes;
     unsigned char *pw = smem + (size_t)m_warps * QW * D * 4 + (size_t)splits * 2 * Sh::kTileBytes;
-    float *Ps = (float *)(pw + (size_t)warp * Sh::kPBytes);
-    pw += (size_t)m_warps * splits * Sh::kPBytes;
+    float *Ps = (float *)(p_in_k ? ks + (size_t)mw * Sh::kPBytes : pw + (size_t)warp * Sh::kPBytes);
+    if (!p_in_k) pw += (size_t)m_warps * splits * Sh::kPBytes;
     float *factor = (float *)pw + warp * QW;
     int *list = (int *)((float *)pw + m_warps * splits * QW);
 
@@ -176,8 +181,10 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
             fma_channel<RQ>(s, a, x, &float4::w);
         }
         group_sync(1 + grp, g_thr);  // everybody is done with the K tile
-        if (nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
-        else if (kAsync) cp_async_commit();
+        if (!p_in_k) {
+            if (nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
+            else if (kAsync) cp_async_commit();
+        }
         // online softmax; the four lanes of a query share its keys
         bool moved = false;
 #pragma unroll
@@ -209,7 +216,8 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
             moved |= alpha != 1.f;
         }
         moved = __any_sync(0xffffffffu, moved);
-        if (kAsync) cp_async_wait<1>();
+        if (kAsync && p_in_k) cp_async_wait<0>();
+        else if (kAsync) cp_async_wait<1>();
         group_sync(1 + grp, g_thr);  // the V tile and this warp's P are there
         if (moved) {
 #pragma unroll
@@ -239,6 +247,7 @@ __global__ void __launch_bounds__(256) attn_generic_kernel(Geom g, int m_warps, 
             }
         }
         group_sync(1 + grp, g_thr);  // done with the V tile and with P
+        if (p_in_k && nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
         if (nxt < n_tiles) fetch<T, D, kLoad, false>(g, vs, vp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
     }
     if (kAsync) cp_async_wait<0>();
@@ -354,17 +363,23 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     while (n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta && there >= 3 && there >= 2 * n_cta) n_cta *= 2;
     if (n_cta > 1) splits = std::min({splits, (tiles + n_cta - 1) / n_cta, 2 * ((there + n_cta - 1) / n_cta)});
     else if (rows > n_sm) splits = std::min(splits, rows > 4ll * n_sm ? there : 2 * there);
+    // Three CTAs an SM where that is enough rows for (d = 64, one warp a group; us before and after): 8 heads, blocks of 32, k = 8,
+    // 5003 tokens 125 -> 108, 1500 (376 rows) 52 -> 38; blocks of 16, 5000 tokens 115 -> 94. With 328 rows, k = 16, it was 61 -> 69:
+    // two CTAs an SM nearly hold them. Two warps a group (blocks of 64) have no room for their P there.
+    const bool p_in_k = D == 64 && m_warps * Sh::kPBytes <= Sh::kTileBytes && 2 * rows > 5ll * n_sm;
     auto bytes = [&](int s) {
-        const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * (Sh::kPBytes + QW * 4) + (size_t)g.k_top * 4;
+        const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * ((p_in_k ? 0 : Sh::kPBytes) + QW * 4) + (size_t)g.k_top * 4;
         const size_t sum = (size_t)m_warps * s * Sh::kPart * 4 + (n_cta > 1 ? (size_t)m_warps * QW * s * n_cta * 4 : 0);
         return walk > sum ? walk : sum;
     };
     while (splits > 1 && bytes(splits) > kMaxDynamicSmem) splits /= 2;
     const size_t smem = bytes(splits);
-    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, true> : attn_generic_kernel<T, D, QW, kLoad, false>;
+    constexpr bool kTight = (D == 64 || D == 32) && QW == 32;
+    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, true, false> : attn_generic_kernel<T, D, QW, kLoad, false, false>;
+    if (kTight && n_cta == 1 && m_warps * splits <= 4 && (p_in_k || D == 32)) kern = attn_generic_kernel<T, D, QW, kLoad, false, kTight>;
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
-    e = launch_kernel(kern, (unsigned)(rows * n_cta), (unsigned)(m_warps * splits * 32), smem, st, (unsigned)n_cta, g, m_warps, splits, (const T *)q,
+    e = launch_kernel(kern, (unsigned)(rows * n_cta), (unsigned)(m_warps * splits * 32), smem, st, (unsigned)n_cta, g, m_warps, splits, p_in_k, (const T *)q,
                       (const T *)k, (const T *)v, mask, scale, (T *)out);
     if (e != cudaSuccess) return cuda_fail(e, "attn_generic launch");
     return STREAM_OK;
