@@ -61,7 +61,10 @@ struct FmaScore {
     static constexpr int kSQ = 8 * RQ, kCh = D < 32 ? D : 32, kChunks = D / kCh;
     static constexpr int kRowBytes = kCh * 4, kBufBytes = kKeysPerUnit * kRowBytes, kRing = 2;
     static constexpr int kSwz = kCh / 4 - 1;
-    static constexpr int kWarps = 4, kCtas = kRegisters && RQ == 4 && D >= 64 ? 3 : 4;  // warps of a row, CTAs an SM should hold
+    // Warps of a row, CTAs an SM should hold. Rows of up to 16 queries have half the register tile, and a fifth CTA pays (fp32, us: 8
+    // heads, 4000 tokens, d = 128, blocks of 16, k = 16: 595 -> 555; 6 heads, 5000 tokens, d = 64, k = 8: 240 -> 223; 4 heads, 5500
+    // tokens, d = 32, k = 6: 101 -> 89); 32 queries spill with it (181 -> 217).
+    static constexpr int kWarps = 4, kCtas = RQ == 2 ? (kRegisters ? 4 : 5) : (kRegisters && D >= 64 ? 3 : 4);
 
     static int q_parts(const Geom &g) { return (g.bq + kSQ - 1) / kSQ; }
     static size_t smem_bytes(const Geom &g, int warps) {
