@@ -9,9 +9,9 @@
 // behind the next Q K^T. Inner loops read shared memory 16 bytes at a time, conflict-free:
 //   Q K^T   lane (kq, kk): queries kq + 8 i x keys kk + 4 j; QW / 8 + 8 loads per 4 QW FMA
 //   P V     lane (ro, co): QW / 4 consecutive queries x channels 4 co + 32 i, P kept key-major
-// Bound: FMA issue and its latency at 8 warps per SM (issue slots 53 % busy; a bare FMA loop measures
-// 66 of the 74.5 TFLOP/s). The kernel this one replaced padded every tile to 64 x 64 and loaded
-// scalars: 8 heads, T = 5003, blocks of 32, d = 64, k = 8: 599 -> 150 us; one head, T = 2048: 82 -> 18 us.
+// Bound: FMA issue and its latency at 8 to 12 warps per SM (a bare FMA loop measures 66 of the 74.5 TFLOP/s; 8 heads,
+// T = 5003, blocks of 32, d = 64, k = 8: 108 us, 24). The kernel this one replaced padded every tile to 64 x 64 and loaded
+// scalars: 8 heads, T = 5003, blocks of 32, d = 64, k = 8: 599 -> 150 us, and 108 since; one head, T = 2048: 82 -> 18 us.
 #include "warp_common.cuh"
 
 namespace stream {
