@@ -56,7 +56,7 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
 #pragma unroll
             for (int i = 0; i < most; ++i) {
                 const int idx = first + i * n_thr, n = idx / per_row, c = idx % per_row;
-                x[i] = n < n_in ? __ldg((const uint2 *)(base + (tk0 + n) * g.ks_t + c * 4)) : make_uint2(0, 0);
+                x[i] = n < n_in ? *(const uint2 *)(base + (tk0 + n) * g.ks_t + c * 4) : make_uint2(0, 0);
             }
 #pragma unroll
             for (int i = 0; i < most; ++i) {
@@ -90,9 +90,8 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
 // p_in_k: P lies over the group's K tile, and both next tiles are fetched behind P V: what a warp then waits for its tiles the other
 // two CTAs' warps cover.
 template <typename T, int D, int QW, Load kLoad, bool kCluster, bool kFour>
-__global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) : (D >= 128 ? 1 : 0)) attn_generic_kernel(Geom g, int m_warps, int splits, bool p_in_k, const T *__restrict__ q,
-                                                           const T *__restrict__ k, const T *__restrict__ v,
-                                                           const int32_t *__restrict__ mask, float scale, T *__restrict__ out) {
+__global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) : (D >= 128 ? 1 : 0)) attn_generic_kernel(Geom g, int m_warps, int splits, bool p_in_k, const T *q, const T *k, const T *v,
+                                                           const int32_t *mask, float scale, T *__restrict__ out) {
     using Sh = Shape<D, QW>;
     constexpr bool kAsync = kLoad == Load::kCopy16;
     constexpr int RQ = QW / 8, RO = QW / 4, CO = D < 32 ? 1 : D / 32;

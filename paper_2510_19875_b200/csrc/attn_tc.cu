@@ -348,7 +348,7 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
     Ring mw;
     auto fetch = [&](int e, int (&blk)[F::kRows]) {
 #pragma unroll
-        for (int r = 0; r < F::kRows; ++r) blk[r] = e < g.k_top && r < it.R ? __ldg(row[r] + e) : -1;
+        for (int r = 0; r < F::kRows; ++r) blk[r] = e < g.k_top && r < it.R ? row[r][e] : -1;
     };
     auto mask_step = [&]() -> bool {
         if (m_id >= P.n_items) return false;

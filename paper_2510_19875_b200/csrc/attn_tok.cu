@@ -126,7 +126,7 @@ __device__ void mask_role(const Params &P, Tail *tl, int lane) {
                 for (int i0 = 0; i0 < n_entries; i0 += 128) {
                     int e[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) e[u] = i0 + u * 32 + lane < n_entries ? __ldg(m + i0 + u * 32 + lane) : -1;
+                    for (int u = 0; u < 4; ++u) e[u] = i0 + u * 32 + lane < n_entries ? m[i0 + u * 32 + lane] : -1;
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int i = i0 + u * 32 + lane, rel = e[u] - s.block0;

@@ -97,7 +97,9 @@ stream_status read_attn_tok_status(unsigned int out[2], cudaStream_t st);
 // The library's kernels are launched as programmatic dependents: a kernel may begin while the one before it on the stream
 // still runs, as far as this point, behind which that one (and with it all before it) is complete and its
 // results are there. So launch latency, barrier setup and TMEM allocation are not waited for. Every thread comes by before it
-// touches global memory (read-only loads, which the compiler may move, stand under conditions behind it).
+// touches global memory, and reads it with ordinary loads, cp.async or TMA only: no __ldg and no const __restrict__ inputs.
+// Those are for data that nobody writes while the kernel lives, and this one lives while the kernel before still
+// writes the mask it reads; such loads may also be moved up across the wait or find a line from before it.
 __device__ __forceinline__ void after_previous_kernel() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -140,7 +140,7 @@ struct FmaScore {
                     const T *src = base + (long long)min(n, last) * g.ks_t + c4 * 4;
                     if (n < n_end) {
                         if constexpr (kLoad == Load::kCopy16) cp_async16(buf_s + place(q, n, c4), src, 16);
-                        else if constexpr (kLoad == Load::kWide) raw[i] = __ldg((const uint2 *)src);
+                        else if constexpr (kLoad == Load::kWide) raw[i] = *(const uint2 *)src;
                         else raw[i] = load4(src);
                     }
                 }
@@ -276,7 +276,7 @@ struct MmaScore {
             for (int c = 0; c < kAhead; ++c)
 #pragma unroll
                 for (int n = 0; n < 4; ++n)
-                    if (n * 8 < n_left) b[c][n] = __ldg((const uint4 *)(row0 + row[n] + 32 * c));
+                    if (n * 8 < n_left) b[c][n] = *(const uint4 *)(row0 + row[n] + 32 * c);
 #pragma unroll
             for (int c = 0; c < kGroups; ++c) {
                 uint4 (&x)[4] = b[c % kAhead];
@@ -295,7 +295,7 @@ struct MmaScore {
                 }
 #pragma unroll
                 for (int n = 0; n < 4; ++n)
-                    if (c + kAhead < kGroups && n * 8 < n_left) x[n] = __ldg((const uint4 *)(row0 + row[n] + 32 * (c + kAhead)));
+                    if (c + kAhead < kGroups && n * 8 < n_left) x[n] = *(const uint4 *)(row0 + row[n] + 32 * (c + kAhead));
             }
             float best = -CUDART_INF_F;
             const Allowed ok(g, qb, r);
@@ -340,8 +340,8 @@ struct Slots {
 // those that are its own, hands their keys to the others, and ranks like them.
 template <class P, int W, bool kCluster>
 __global__ void __launch_bounds__(W * 32, W == kWideWarps ? 1 : P::kCtas)
-mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P::Elem *__restrict__ q,
-                 const typename P::Elem *__restrict__ k, int32_t *__restrict__ mask, float *__restrict__ score, WorkspaceHeader *ws) {
+mask_rows_kernel(Geom g, MultiK mk, int score_bytes, int n_max, const typename P::Elem *q,
+                 const typename P::Elem *k, int32_t *__restrict__ mask, float *__restrict__ score, WorkspaceHeader *ws) {
     extern __shared__ __align__(16) unsigned char smem[];
     int *words = (int *)(smem + score_bytes);  // n_max: slots, a multiple of 32
     int par = 0;                               // the present level's slots: the first or the second set

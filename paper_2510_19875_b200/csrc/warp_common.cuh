@@ -114,7 +114,7 @@ enum class Load { kCopy16, kCopy4, kWide, kScalars };
 // Four bf16 in a row, element by element; as fp32.
 __device__ __forceinline__ uint2 load4(const __nv_bfloat16 *src) {
     const unsigned short *x = (const unsigned short *)src;
-    const unsigned a = __ldg(x), b = __ldg(x + 1), c = __ldg(x + 2), d = __ldg(x + 3);
+    const unsigned a = x[0], b = x[1], c = x[2], d = x[3];
     return make_uint2(a | (b << 16), c | (d << 16));
 }
 __device__ __forceinline__ float4 widen4(uint2 x) {

@@ -1,0 +1,53 @@
+"""Kernels that begin while the one before them on the stream still runs: chains of calls without anything in between."""
+import gc
+
+import pytest
+import torch
+
+from test_gpu_parity import S  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+# dtype, heads, T, d, block_q, block_k: a form of every attention kernel
+FORMS = [
+    (torch.bfloat16, 16, 3000, 128, 64, 64), (torch.bfloat16, 8, 1500, 64, 64, 64),   # tcgen05
+    (torch.bfloat16, 8, 1500, 128, 32, 32), (torch.bfloat16, 8, 1500, 64, 32, 32),    # tcgen05, blocks of 32
+    (torch.bfloat16, 4, 1100, 128, 1, 64),                                            # tcgen05, per-token masks
+    (torch.bfloat16, 8, 1100, 256, 64, 64), (torch.bfloat16, 4, 700, 64, 1, 16),      # mma.sync, and its merged walk
+    (torch.float32, 8, 1500, 64, 32, 32), (torch.float32, 8, 1000, 64, 32, 32),       # fp32, P over the key tile or not
+    (torch.float32, 8, 1500, 32, 32, 32), (torch.float32, 4, 1100, 128, 32, 32),
+    (torch.float32, 2, 700, 64, 32, 32),                                              # a row over a cluster
+]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def leave_no_garbage():  # (what follows counts the allocator's bytes around a call: no collection may fall there)
+    yield
+    gc.collect()
+
+
+@pytest.mark.parametrize("dtype,heads,T,d,block_q,block_k", FORMS)
+def test_attentions_that_feed_each_other(S, dtype, heads, T, d, block_q, block_k):
+    """Every output is the queries or the values of the next call, and its buffer is written again two or three calls later: a
+    kernel has to see the results of the one before, and of those before that, and may not write what they still read."""
+    torch.manual_seed(d + block_q)
+    q, k, v = (torch.randn(1, heads, T, d, device="cuda").to(dtype) for _ in range(3))
+    kw = dict(block_q=block_q, block_k=block_k)
+    mask = S.build_mask(q, k, k_top=5, **kw).mask
+    calls = [("q", "v", "a"), ("a", "v", "b"), ("b", "a", "c"), ("c", "b", "a"), ("a", "c", "b"), ("q", "b", "c"), ("c", "a", "a2"), ("a2", "c", "a")]
+
+    def chain(wait):
+        x = dict(q=q, v=v, **{n: torch.full_like(q, float("nan")) for n in ("a", "b", "c", "a2")})
+        torch.cuda.synchronize()
+        for at_q, at_v, to in calls * 3:
+            S.sparse_attention(x[at_q], k, x[at_v], mask, out=x[to], **kw)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return x
+
+    want = chain(True)
+    for _ in range(3):
+        got = chain(False)
+        for n in ("a", "b", "c", "a2"):
+            assert torch.isfinite(want[n]).all() and torch.equal(got[n], want[n]), n
