@@ -18,7 +18,9 @@ void set_error(const char *fmt, ...) {
     va_end(ap);
 }
 
+// Reports e, and takes it off the runtime's record: the next launch that asks for its own error would find it there.
 stream_status cuda_fail(cudaError_t e, const char *what) {
+    (void)cudaGetLastError();
     set_error("%s: %s", what, cudaGetErrorString(e));
     return STREAM_ERR_CUDA;
 }

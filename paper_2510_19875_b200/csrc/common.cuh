@@ -126,8 +126,7 @@ cudaError_t launch_kernel(void (*kern)(K...), unsigned grid, unsigned threads, s
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
     }
-    const cudaError_t e = cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...);
-    return e == cudaSuccess ? cudaGetLastError() : e;
+    return cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...);
 }
 
 __device__ __forceinline__ float to_float(float x) { return x; }

@@ -1,4 +1,5 @@
 """Kernels that begin while the one before them on the stream still runs: chains of calls without anything in between."""
+import ctypes
 import gc
 
 import pytest
@@ -51,3 +52,26 @@ def test_attentions_that_feed_each_other(S, dtype, heads, T, d, block_q, block_k
         got = chain(False)
         for n in ("a", "b", "c", "a2"):
             assert torch.isfinite(want[n]).all() and torch.equal(got[n], want[n]), n
+
+
+def test_a_call_that_failed_does_not_fail_the_next(S):
+    """A synchronisation on a stream that is being captured is refused on the host. The refusal is that call's alone: the
+    calls after it report their own errors, none here."""
+    torch.manual_seed(0)
+    q, k, v = (torch.randn(1, 2, 300, 64, device="cuda") for _ in range(3))
+    kw = dict(block_q=32, block_k=32)
+    mask = S.build_mask(q, k, k_top=4, **kw).mask
+    want = S.sparse_attention(q, k, v, mask, **kw)
+    torch.cuda.synchronize()
+    rt = ctypes.CDLL("libcudart.so.12")  # the one that torch has loaded
+    side, graph = torch.cuda.Stream(), ctypes.c_void_p()
+    for call in (lambda: S.sparse_attention(q, k, v, mask, **kw), lambda: S.build_mask(q, k, k_top=4, **kw).mask,
+                 lambda: S.mask_difference(mask, mask)[0]):
+        assert rt.cudaStreamBeginCapture(ctypes.c_void_p(side.cuda_stream), 2) == 0  # (relaxed: other streams go on as ever)
+        with pytest.raises(S.StreamError):
+            S.stream_check_device_status(side)
+        assert rt.cudaStreamEndCapture(ctypes.c_void_p(side.cuda_stream), ctypes.byref(graph)) != 0  # the capture is lost
+        rt.cudaGetLastError()  # (that error is this test's own)
+        call()
+        torch.cuda.synchronize()
+    assert torch.equal(S.sparse_attention(q, k, v, mask, **kw), want)
