@@ -83,18 +83,32 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
     if (kLoad == Load::kCopy16) cp_async_commit();
 }
 
-// kCluster: the row's tiles are dealt to the groups of all CTAs of a cluster, which read each other's parts at the end.
-// kFour: the build for four warps and three CTAs an SM (four at d = 32), within their registers. Unbounded, ptxas takes
-// over 200 a thread at d = 64 and two CTAs are all an SM holds; at d = 128 and 256 a bound of one CTA lets it take more
-// than it would (8 heads, 5000 tokens, d = 128, blocks of 32: 294 -> 274 us; blocks of 16, k = 16: 482 -> 427).
-// p_in_k: P lies over the group's K tile, and both next tiles are fetched behind P V: what a warp then waits for its tiles the other
-// two CTAs' warps cover.
-template <typename T, int D, int QW, Load kLoad, bool kCluster, bool kFour>
-__global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) : (D >= 128 ? 1 : 0)) attn_generic_kernel(Geom g, int m_warps, int splits, bool p_in_k, const T *q, const T *k, const T *v,
-                                                           const int32_t *mask, float scale, T *__restrict__ out) {
+// The builds of the kernel. kRow: a row by a CTA. kCluster: its tiles are dealt to the groups of all CTAs of a cluster, which
+// read each other's parts at the end. kPInK (d = 64, one warp a group): P lies over the group's K tile, which makes room for a
+// third CTA an SM, and both next tiles are fetched behind P V: what a warp then waits for its tiles the other two CTAs' warps
+// cover. kMoreCtas (d = 32): kRow within the registers of four CTAs an SM.
+enum class Build { kRow, kCluster, kPInK, kMoreCtas };
+
+// Threads of a CTA at most, and the CTAs an SM whose registers a thread is held to (0: unbounded). Unbounded, ptxas takes over
+// 200 at d = 64 and two CTAs are all an SM holds; at d = 128 and 256 a bound of one CTA lets it take more than
+// it would (8 heads, 5000 tokens, d = 128, blocks of 32: 294 -> 274 us; blocks of 16, k = 16: 482 -> 427), but at d = 256 a
+// cluster's kernel then spills (2 heads, 600 tokens: 57.4 -> 59.4).
+template <int D, int QW, Build kBuild>
+struct Bounds {
+    static constexpr bool kTight = kBuild == Build::kMoreCtas || (kBuild == Build::kPInK && QW == 32);
+    static constexpr int kThreads = kTight ? 128 : 256;
+    static constexpr int kCtas = kTight ? (kBuild == Build::kPInK ? 3 : 4) : (D == 128 || (D == 256 && kBuild == Build::kRow) ? 1 : 0);
+};
+
+template <typename T, int D, int QW, Load kLoad, Build kBuild>
+__global__ void __launch_bounds__(Bounds<D, QW, kBuild>::kThreads, Bounds<D, QW, kBuild>::kCtas)
+attn_generic_kernel(Geom g, int m_warps, int splits, const T *q, const T *k, const T *v, const int32_t *mask, float scale, T *__restrict__ out) {
+    constexpr bool kCluster = kBuild == Build::kCluster, kPInK = kBuild == Build::kPInK;
     using Sh = Shape<D, QW>;
     constexpr bool kAsync = kLoad == Load::kCopy16;
     constexpr int RQ = QW / 8, RO = QW / 4, CO = D < 32 ? 1 : D / 32;
+    // (d = 128, us, at 2 and 4: 278.5 against 272.9 for 8 heads, 5000 tokens, blocks of 32; the other dimensions have no registers for it)
+    constexpr int kUnrollQK = D == 128 ? 4 : 2, kUnrollPV = D == 128 ? 8 : 4;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_n;
     after_previous_kernel();
@@ -115,8 +129,8 @@ __global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) :
     float *Qs = (float *)smem;
     unsigned char *ks = smem + (size_t)m_warps * QW * D * 4 + (size_t)grp * 2 * Sh::kTileBytes, *vs = ks + Sh::kTileBytes;
     unsigned char *pw = smem + (size_t)m_warps * QW * D * 4 + (size_t)splits * 2 * Sh::kTileBytes;
-    float *Ps = (float *)(p_in_k ? ks + (size_t)mw * Sh::kPBytes : pw + (size_t)warp * Sh::kPBytes);
-    if (!p_in_k) pw += (size_t)m_warps * splits * Sh::kPBytes;
+    float *Ps = (float *)(kPInK ? ks + (size_t)mw * Sh::kPBytes : pw + (size_t)warp * Sh::kPBytes);
+    if (!kPInK) pw += (size_t)m_warps * splits * Sh::kPBytes;
     float *factor = (float *)pw + warp * QW;
     int *list = (int *)((float *)pw + m_warps * splits * QW);
 
@@ -164,7 +178,7 @@ __global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) :
         for (int i = 0; i < RQ; ++i)
 #pragma unroll
             for (int j = 0; j < 8; ++j) s[i][j] = 0.f;
-#pragma unroll 2
+#pragma unroll kUnrollQK
         for (int c4 = 0; c4 < D / 4; ++c4) {
             float4 a[RQ], x[8];
 #pragma unroll
@@ -180,7 +194,7 @@ __global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) :
             fma_channel<RQ>(s, a, x, &float4::w);
         }
         group_sync(1 + grp, g_thr);  // everybody is done with the K tile
-        if (!p_in_k) {
+        if (!kPInK) {
             if (nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
             else if (kAsync) cp_async_commit();
         }
@@ -215,7 +229,7 @@ __global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) :
             moved |= alpha != 1.f;
         }
         moved = __any_sync(0xffffffffu, moved);
-        if (kAsync && p_in_k) cp_async_wait<0>();
+        if (kAsync && kPInK) cp_async_wait<0>();
         else if (kAsync) cp_async_wait<1>();
         group_sync(1 + grp, g_thr);  // the V tile and this warp's P are there
         if (moved) {
@@ -227,7 +241,7 @@ __global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) :
             }
         }
         if (D >= 32 || co * 4 < D) {
-#pragma unroll 4
+#pragma unroll kUnrollPV
             for (int n = 0; n < n_keys; ++n) {
                 float p[RO];
 #pragma unroll
@@ -246,7 +260,7 @@ __global__ void __launch_bounds__(kFour ? 128 : 256, kFour ? (D == 64 ? 3 : 4) :
             }
         }
         group_sync(1 + grp, g_thr);  // done with the V tile and with P
-        if (p_in_k && nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
+        if (kPInK && nxt < n_tiles) fetch<T, D, kLoad, true>(g, ks, kp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
         if (nxt < n_tiles) fetch<T, D, kLoad, false>(g, vs, vp, list[nxt / n_sub], nxt % n_sub * kKeys, g_tid, g_thr);
     }
     if (kAsync) cp_async_wait<0>();
@@ -373,12 +387,16 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     };
     while (splits > 1 && bytes(splits) > kMaxDynamicSmem) splits /= 2;
     const size_t smem = bytes(splits);
-    constexpr bool kTight = (D == 64 || D == 32) && QW == 32;
-    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, true, false> : attn_generic_kernel<T, D, QW, kLoad, false, false>;
-    if (kTight && n_cta == 1 && m_warps * splits <= 4 && (p_in_k || D == 32)) kern = attn_generic_kernel<T, D, QW, kLoad, false, kTight>;
+    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, Build::kCluster> : attn_generic_kernel<T, D, QW, kLoad, Build::kRow>;
+    if constexpr (D == 64) {
+        if (p_in_k) kern = attn_generic_kernel<T, D, QW, kLoad, Build::kPInK>;
+    }
+    if constexpr (D == 32 && QW == 32) {
+        if (n_cta == 1 && m_warps * splits <= 4) kern = attn_generic_kernel<T, D, QW, kLoad, Build::kMoreCtas>;
+    }
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
-    e = launch_kernel(kern, (unsigned)(rows * n_cta), (unsigned)(m_warps * splits * 32), smem, st, (unsigned)n_cta, g, m_warps, splits, p_in_k, (const T *)q,
+    e = launch_kernel(kern, (unsigned)(rows * n_cta), (unsigned)(m_warps * splits * 32), smem, st, (unsigned)n_cta, g, m_warps, splits, (const T *)q,
                       (const T *)k, (const T *)v, mask, scale, (T *)out);
     if (e != cudaSuccess) return cuda_fail(e, "attn_generic launch");
     return STREAM_OK;
