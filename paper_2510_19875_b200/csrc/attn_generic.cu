@@ -22,6 +22,7 @@ using namespace wp;
 constexpr int kMaxBlock = 64;
 constexpr int kKeys = 32;  // keys of a tile
 constexpr size_t kMaxDynamicSmem = 220 * 1024;
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerCtaReserved = 1024 + 128;  // (128: the kernel's static words)
 
 template <typename T>
 __device__ __forceinline__ void store4(T *dst, float4 x);
@@ -84,26 +85,27 @@ __device__ __forceinline__ void fetch(const Geom &g, unsigned char *dst, const T
 }
 
 // The builds of the kernel. kRow: a row by a CTA. kCluster: its tiles are dealt to the groups of all CTAs of a cluster, which
-// read each other's parts at the end. kPInK (d = 64, one warp a group): P lies over the group's K tile, which makes room for a
-// third CTA an SM, and both next tiles are fetched behind P V: what a warp then waits for its tiles the other two CTAs' warps
-// cover. kMoreCtas (d = 32): kRow within the registers of four CTAs an SM.
-enum class Build { kRow, kCluster, kPInK, kMoreCtas };
+// read each other's parts at the end. kThree, kFour: as kRow, with three or four CTAs of four warps an SM where the registers of
+// kRow let an SM hold two. kThree at d = 64 (one warp a group): P lies over the group's K tile, for the room of the third, and both
+// next tiles are fetched behind P V: what a warp then waits for its tiles the other two CTAs' warps cover.
+enum class Build { kRow, kCluster, kThree, kFour };
 
-// Threads of a CTA at most, and the CTAs an SM whose registers a thread is held to (0: unbounded). Unbounded, ptxas takes over
-// 200 at d = 64 and two CTAs are all an SM holds; at d = 128 and 256 a bound of one CTA lets it take more than
-// it would (8 heads, 5000 tokens, d = 128, blocks of 32: 294 -> 274 us; blocks of 16, k = 16: 482 -> 427), but at d = 256 a
-// cluster's kernel then spills (2 heads, 600 tokens: 57.4 -> 59.4).
+// Threads of a CTA at most, and the CTAs an SM whose registers a thread is held to (0: unbounded). Unbounded, ptxas takes 200 to 250
+// at d = 32 and 64. Held to three CTAs d = 32 spills nothing and d = 64 20 to 90 bytes; to four, d = 32 spills 70 to
+// 150. At d = 128 and 256 a bound of one CTA lets it take more than it would (8 heads, 5000 tokens, d = 128, blocks of
+// 32: 294 -> 274 us; blocks of 16, k = 16: 482 -> 427), but at d = 256 a cluster's kernel then spills (2 heads, 600
+// tokens: 57.4 -> 59.4).
 template <int D, int QW, Build kBuild>
 struct Bounds {
-    static constexpr bool kTight = kBuild == Build::kMoreCtas || (kBuild == Build::kPInK && QW == 32);
+    static constexpr bool kTight = kBuild == Build::kThree || kBuild == Build::kFour;
     static constexpr int kThreads = kTight ? 128 : 256;
-    static constexpr int kCtas = kTight ? (kBuild == Build::kPInK ? 3 : 4) : (D == 128 || (D == 256 && kBuild == Build::kRow) ? 1 : 0);
+    static constexpr int kCtas = kTight ? (kBuild == Build::kThree ? 3 : 4) : (D == 128 || (D == 256 && kBuild == Build::kRow) ? 1 : 0);
 };
 
 template <typename T, int D, int QW, Load kLoad, Build kBuild>
 __global__ void __launch_bounds__(Bounds<D, QW, kBuild>::kThreads, Bounds<D, QW, kBuild>::kCtas)
 attn_generic_kernel(Geom g, int m_warps, int splits, const T *q, const T *k, const T *v, const int32_t *mask, float scale, T *__restrict__ out) {
-    constexpr bool kCluster = kBuild == Build::kCluster, kPInK = kBuild == Build::kPInK;
+    constexpr bool kCluster = kBuild == Build::kCluster, kPInK = kBuild == Build::kThree && D == 64;
     using Sh = Shape<D, QW>;
     constexpr bool kAsync = kLoad == Load::kCopy16;
     constexpr int RQ = QW / 8, RO = QW / 4, CO = D < 32 ? 1 : D / 32;
@@ -376,23 +378,38 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     while (n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta && there >= 3 && there >= 2 * n_cta) n_cta *= 2;
     if (n_cta > 1) splits = std::min({splits, (tiles + n_cta - 1) / n_cta, 2 * ((there + n_cta - 1) / n_cta)});
     else if (rows > n_sm) splits = std::min(splits, rows > 4ll * n_sm ? there : 2 * there);
-    // Three CTAs an SM where that is enough rows for (d = 64, one warp a group; us before and after): 8 heads, blocks of 32, k = 8,
-    // 5003 tokens 125 -> 108, 1500 (376 rows) 52 -> 38; blocks of 16, 5000 tokens 115 -> 94. With 328 rows, k = 16, it was 61 -> 69:
-    // two CTAs an SM nearly hold them. Two warps a group (blocks of 64) have no room for their P there.
-    const bool p_in_k = D == 64 && m_warps * Sh::kPBytes <= Sh::kTileBytes && 2 * rows > 5ll * n_sm;
-    auto bytes = [&](int s) {
+    auto bytes = [&](int s, bool p_in_k) {
         const size_t walk = (size_t)m_warps * QW * D * 4 + (size_t)s * 2 * Sh::kTileBytes + (size_t)m_warps * s * ((p_in_k ? 0 : Sh::kPBytes) + QW * 4) + (size_t)g.k_top * 4;
         const size_t sum = (size_t)m_warps * s * Sh::kPart * 4 + (n_cta > 1 ? (size_t)m_warps * QW * s * n_cta * 4 : 0);
         return walk > sum ? walk : sum;
     };
-    while (splits > 1 && bytes(splits) > kMaxDynamicSmem) splits /= 2;
-    const size_t smem = bytes(splits);
-    auto kern = n_cta > 1 ? attn_generic_kernel<T, D, QW, kLoad, Build::kCluster> : attn_generic_kernel<T, D, QW, kLoad, Build::kRow>;
-    if constexpr (D == 64) {
-        if (p_in_k) kern = attn_generic_kernel<T, D, QW, kLoad, Build::kPInK>;
+    while (splits > 1 && bytes(splits, false) > kMaxDynamicSmem) splits /= 2;
+    // More than two CTAs an SM: a round of rows then takes 1.4 times as long, so it is a matter of rounds (us at two, at
+    // three; 8 heads, blocks of 32, k = 8). d = 64: 376 rows 49.7, 38.3; 480 to 600 are two rounds either way, 480 52.3, 61.6; 592
+    // 53.1, 66.8; 640 74.1, 68.2; 1256 123.6, 108.1. d = 32: 160 rows 17.9, 22.7; 400 34.1, 23.9; 592 34.9, 42.0;
+    // 752 50.6, 43.6; 3000 177.6, 149.4; bf16 and rows off 16 bytes alike. Four only for groups of two warps at d = 32 (blocks of
+    // 64; two, three, four): 480 rows 113, 104, 100; 720 168, 146, 157; 1000 223, 202, 183. Where the rows have work
+    // for two warps only (k = 1 and 2), smaller CTAs fill the SM by themselves (2400 rows, k = 2, d = 64: 81.8, 85.9).
+    // A causal head's first rows have fewer than k blocks and come last: a third of them off the count puts the lines right
+    // (d = 64, causal: 304 rows, k = 8, 36.9, 37.8; 336, k = 16, 62.1, 69.0; 344 69.9, 69.1; 480 93.7, 83.2; not causal: 304 rows, k = 8, 44.4, 37.7).
+    const int warps = m_warps * splits;
+    const long long first = std::min((long long)g.n_qb, (long long)g.k_top * g.bk / g.bq);
+    const long long full = g.causal ? rows - (long long)g.batch * g.H * first / 3 : rows;
+    Build build = n_cta > 1 ? Build::kCluster : Build::kRow;
+    if ((D == 64 || (D == 32 && QW == 32)) && n_cta == 1 && (warps == 3 || warps == 4) && full > 2ll * n_sm) {
+        auto fit = [&](size_t ctas) { return ctas * (bytes(splits, D == 64) + kSmemPerCtaReserved) <= kSmemPerSm; };
+        const bool three = (D == 32 || m_warps * Sh::kPBytes <= Sh::kTileBytes) && fit(3), four = D == 32 && m_warps == 2 && fit(4);
+        const bool two_rounds = full > 3ll * n_sm && full <= 4ll * n_sm;  // (with three as with two)
+        if (four && (two_rounds || full > 6ll * n_sm)) build = Build::kFour;
+        else if (three && !two_rounds) build = Build::kThree;
+    }
+    const size_t smem = bytes(splits, D == 64 && build == Build::kThree);
+    auto kern = build == Build::kCluster ? attn_generic_kernel<T, D, QW, kLoad, Build::kCluster> : attn_generic_kernel<T, D, QW, kLoad, Build::kRow>;
+    if constexpr (D == 64 || (D == 32 && QW == 32)) {
+        if (build == Build::kThree) kern = attn_generic_kernel<T, D, QW, kLoad, Build::kThree>;
     }
     if constexpr (D == 32 && QW == 32) {
-        if (n_cta == 1 && m_warps * splits <= 4) kern = attn_generic_kernel<T, D, QW, kLoad, Build::kMoreCtas>;
+        if (build == Build::kFour) kern = attn_generic_kernel<T, D, QW, kLoad, Build::kFour>;
     }
     cudaError_t e = allow_smem(kern, kMaxDynamicSmem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(attn_generic)");
