@@ -81,6 +81,10 @@ struct Form {
     // Two K stages: one is free when the logits of the entry before last are there, which their own barrier says (its next
     // use is at least two entries later). More: a barrier of the stage's own, and a commit more for the issuing warp.
     static constexpr bool kKByLogits = kMaxKStages == 2;
+    // Of `rings` buffers (the host sees to kMinRings at least): the stages of V, of K.
+    static constexpr int kMinRings = 4;
+    static __host__ __device__ constexpr int v_stages(int rings) { return kMaxVStages < (rings + 1) / 2 ? kMaxVStages : (rings + 1) / 2; }
+    static __host__ __device__ constexpr int k_stages(int rings) { return kMaxKStages < rings - v_stages(rings) ? kMaxKStages : rings - v_stages(rings); }
     // TMEM columns: the two logit buffers of group g at 128 g and 64 behind, its P at 256 + 64 g (two
     // buffers, the second 32 behind, or the two parts of one), O at 384.
     static constexpr int kPBufs = kSplit ? 1 : 2;
@@ -104,7 +108,7 @@ struct Item {
 template <class F>
 struct Tail {
     unsigned long long q_full[2], q_free[2];  // q_free: the output staged over the pair's Q has left (8 warps)
-    unsigned long long k_full[F::kMaxKStages], k_empty[F::kMaxKStages], v_full[F::kMaxVStages], v_empty[F::kMaxVStages];
+    unsigned long long k_full[F::kMaxKStages], k_empty[F::kMaxKStages] /* (kKByLogits: not used) */, v_full[F::kMaxVStages], v_empty[F::kMaxVStages];
     unsigned long long s_full[2][2], s_free[2][2];        // per group and logit buffer: ready / read
     unsigned long long p_full[2][2], p_free[2][2];        // per group and P buffer: published / product added
     unsigned long long o_done, o_free;     // a pair's last product is complete; its O has been read (8 warps)
@@ -755,8 +759,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     // what is left behind the aligned base decides the number of V and K stages (the same in every thread)
     const int fixed_bytes = (int)(smem - smem_raw) + (int)sizeof(Tail<F>) + kMaskSlots * F::kRows * P.row_stride * (int)sizeof(int);
     const int n_rings = (P.smem_bytes - fixed_bytes) / F::kOperand - kFixedOperands;  // buffers for the two rings: d = 128: 4 or 5
-    P.n_v_stages = min(F::kMaxVStages, (n_rings + 1) / 2);
-    P.n_k_stages = min(F::kMaxKStages, n_rings - P.n_v_stages);
+    static_assert(!F::kKByLogits || (F::k_stages(F::kMinRings) == 2 && F::k_stages(F::kMinRings + 1) == 2), "two K stages, with however many buffers");
+    P.n_v_stages = F::v_stages(n_rings);
+    P.n_k_stages = F::k_stages(n_rings);
     const unsigned q_smem = smem_u32(smem), v_smem = q_smem + kFixedOperands * F::kOperand, k_smem = v_smem + P.n_v_stages * F::kOperand;
     Tail<F> *tl = (Tail<F> *)(smem + (kFixedOperands + P.n_v_stages + P.n_k_stages) * F::kOperand);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -847,7 +852,7 @@ stream_status launch(const Geom &g, const void *q, const void *k, const void *v,
     const int tail_bytes = (int)sizeof(Tail<F>) + kMaskSlots * F::kRows * P.row_stride * (int)sizeof(int);
     int smem_bytes = (kFixedOperands + F::kMaxKStages + F::kMaxVStages) * F::kOperand + tail_bytes + 1024;
     if (smem_bytes > kMaxSmemPerCta) smem_bytes = kMaxSmemPerCta;
-    if (smem_bytes < (kFixedOperands + 4) * F::kOperand + tail_bytes + 1024) {
+    if (smem_bytes < (kFixedOperands + F::kMinRings) * F::kOperand + tail_bytes + 1024) {
         set_error("tensor-core attention kernel: k_top = %d needs more shared memory than one CTA has", g.k_top);
         return STREAM_ERR_UNSUPPORTED;
     }
