@@ -75,3 +75,70 @@ def test_a_call_that_failed_does_not_fail_the_next(S):
         call()
         torch.cuda.synchronize()
     assert torch.equal(S.sparse_attention(q, k, v, mask, **kw), want)
+
+
+@pytest.mark.parametrize("dtype,heads,T,d,block_q,block_k", FORMS)
+def test_capture_in_a_graph(S, dtype, heads, T, d, block_q, block_k):
+    """Two passes of mask and attention and a second attention behind them, captured once, replayed on changed inputs."""
+    torch.manual_seed(d)
+    kw = dict(block_q=block_q, block_k=block_k)
+    inputs = [tuple(torch.randn(1, heads, T, d, device="cuda").to(dtype) for _ in range(3)) for _ in range(2)]
+    want = []
+    for q, k, v in inputs:
+        mask = S.build_mask(q, k, k_top=5, **kw).mask
+        out = S.sparse_attention(q, k, v, mask, **kw)
+        torch.cuda.synchronize()
+        want.append((mask, out, S.sparse_attention(out, k, v, mask, **kw)))
+        torch.cuda.synchronize()
+    q, k, v = (x.clone() for x in inputs[0])
+    mask, out, out2 = (torch.empty_like(x) for x in want[0])
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(2):
+            S.build_mask(q, k, k_top=5, mask_out=mask, workspace=ws, **kw)
+            S.sparse_attention(q, k, v, mask, out=out, **kw)
+            S.sparse_attention(out, k, v, mask, out=out2, **kw)
+    for i in (0, 1, 1, 0):
+        for dst, src in zip((q, k, v), inputs[i]):
+            dst.copy_(src)
+        mask.fill_(-7)
+        out.zero_()
+        out2.zero_()
+        graph.replay()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(mask, want[i][0]) and torch.equal(out, want[i][1]) and torch.equal(out2, want[i][2])
+
+
+def test_capture_of_several_k_one_k_a_row_and_the_library_s_scratch(S):
+    torch.manual_seed(3)
+    kw = dict(block_q=64, block_k=64)
+    inputs = [tuple(torch.randn(1, h, 3000, 128, device="cuda").bfloat16() for h in (8, 2)) for _ in range(2)]
+    q, k = (x.clone() for x in inputs[0])
+    p = S.make_problem(q, k, k_top=12, **kw)
+    k_row = S.k_schedule(p, 1 / 4).cuda()
+    static = torch.empty(1, 8, S.n_query_blocks(p), 12, dtype=torch.int32, device="cuda")
+
+    def calls():
+        S.stream_build_mask_static(p, q, k, static, None)
+        return [static, S.build_masks(q, k, [12, 3, 7], **kw).mask, S.build_masks(q, k, [12, 3, 7], share=False, **kw).mask,
+                S.build_mask(q, k, k_top=12, k_row=k_row, **kw).mask]
+
+    want = []
+    for i in (0, 1):  # (the first call on the library's scratch asks for its address, which no capture allows)
+        q.copy_(inputs[i][0])
+        k.copy_(inputs[i][1])
+        want.append([x.clone() for x in calls()])
+        torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = calls()
+    for i in (1, 0, 1):
+        q.copy_(inputs[i][0])
+        k.copy_(inputs[i][1])
+        for x in got:
+            x.fill_(-7)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want[i]))

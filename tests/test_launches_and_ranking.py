@@ -43,8 +43,9 @@ def test_equal_scores_keep_the_first(S, block, T, k_top):
 @pytest.mark.parametrize("dtype,d,block_q,block_k", [(torch.bfloat16, 128, 64, 64), (torch.bfloat16, 64, 32, 32), (torch.float32, 64, 32, 32),
                                                      (torch.bfloat16, 256, 64, 64), (torch.bfloat16, 128, 1, 64)])
 def test_launches_that_share_buffers_wait_for_each_other(S, dtype, d, block_q, block_k):
-    """Two inputs in turn through one mask, one output and one workspace, without a synchronisation in between: every kernel begins
-    while the one before still runs, and has to see its results and leave its inputs alone until it is done."""
+    """Two inputs in turn through one mask, one output and one workspace, without a synchronisation in between. The attention begins
+    while the mask build still runs and has to see its result; copies and memsets stand between all others (chains of
+    kernels alone: test_dependent_launches.py)."""
     torch.manual_seed(d)
     kw = dict(block_q=block_q, block_k=block_k)
     inputs = [tuple(torch.randn(1, h, 1100, d, device="cuda").to(dtype) for h in (8, 2, 2)) for _ in range(2)]
@@ -63,7 +64,7 @@ def test_launches_that_share_buffers_wait_for_each_other(S, dtype, d, block_q, b
         S.build_mask(q, k, k_top=4, mask_out=mask, workspace=ws, **kw)
         S.sparse_attention(q, k, v, mask, out=out, **kw)
         got.append((mask.clone(), out.clone()))
-        S.sparse_attention(q, k, v, mask, out=out, **kw)  # (two of the same kind, one after the other)
+        S.sparse_attention(q, k, v, mask, out=out, **kw)  # (behind the copies: what it writes again, the next round's kernels find)
     torch.cuda.synchronize()
     for i, pair in enumerate(got):
         assert all(torch.equal(a, b) for a, b in zip(pair, want[i % 2])), i
