@@ -6,11 +6,12 @@
 // walks a sequence of key tiles, and the groups of a CTA take the row's tiles in turn, each with
 // softmax statistics and accumulators of its own, added up at the end. One K and one V buffer
 // per group, filled by cp.async (bf16, and rows off 16 bytes: through registers): the next K tile arrives behind softmax and P V, the next V tile
-// behind the next Q K^T. Inner loops read shared memory 16 bytes at a time, conflict-free:
+// behind the next Q K^T (with three CTAs an SM at d = 64 both are asked for behind P V, and nothing covers them but the
+// other CTAs). Inner loops read shared memory 16 bytes at a time, conflict-free:
 //   Q K^T   lane (kq, kk): queries kq + 8 i x keys kk + 4 j; QW / 8 + 8 loads per 4 QW FMA
 //   P V     lane (ro, co): QW / 4 consecutive queries x channels 4 co + 32 i, P kept key-major
-// Bound: FMA issue and its latency at 8 to 12 warps per SM (a bare FMA loop measures 66 of the 74.5 TFLOP/s; 8 heads,
-// T = 5003, blocks of 32, d = 64, k = 8: 108 us, 24). The kernel this one replaced padded every tile to 64 x 64 and loaded
+// Bound: latency. 8 to 12 warps an SM wait for their tiles, for each other and for the merge of a row's four parts after two tiles
+// each (8 heads, T = 5003, blocks of 32, d = 64, k = 8: 108 us, 24 TFLOP/s; a bare FMA loop reaches 66 of 74.5). The kernel this one replaced padded every tile to 64 x 64 and loaded
 // scalars: 8 heads, T = 5003, blocks of 32, d = 64, k = 8: 599 -> 150 us, and 108 since; one head, T = 2048: 82 -> 18 us.
 #include "warp_common.cuh"
 
@@ -368,7 +369,8 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     // Four warps a CTA, so that several CTAs share an SM; eight when every row has an SM to itself
     // anyway. Fewer rows than half of the SMs: a row over two, four or eight CTAs, while each has a tile part for
     // every scheduler (28 rows, blocks of 64, k = 11, d = 64: 65.4 -> 34.8 us; 55 rows, blocks of 32, k = 9, d = 128:
-    // 38.9 -> 30.7; 64 rows, blocks of 32, k = 8: 18.4 either way).
+    // 38.9 -> 30.7; 32 rows of blocks of 32, k = 8: 18.2, and 15.7 in a CTA each, which begins while the kernel before
+    // it still runs, as no cluster does; 64 rows, k = 8: 18.4 and 15.8, k = 16: 22.5 and 26.7).
     // T may have fewer blocks than k_top, and what counts are those that are there: a CTA of a cluster has two tile
     // parts at least, a group half of one (16 rows, T = 29, blocks of 48, k = 9, d = 16: 32 -> 10 us); with many
     // rows an idle group takes another CTA's shared memory (2500 rows, k = 1, d = 128, rows off 16 bytes: 397 -> 223).

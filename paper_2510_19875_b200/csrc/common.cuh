@@ -94,7 +94,7 @@ stream_status launch_attn_tok(const Geom &g, const void *q, const void *k, const
 stream_status read_attn_status(unsigned int out[2], cudaStream_t st);
 stream_status read_attn_tok_status(unsigned int out[2], cudaStream_t st);
 
-// The library's kernels are launched as programmatic dependents: a kernel may begin while the one before it on the stream
+// The kernels of mask builds and attention, but for clusters, are launched as programmatic dependents: a kernel may begin while the one before it on the stream
 // still runs, as far as this point, behind which that one (and with it all before it) is complete and its
 // results are there. So launch latency, barrier setup and TMEM allocation are not waited for. Every thread comes by before it
 // touches global memory, and reads it with ordinary loads, cp.async or TMA only: no __ldg and no const __restrict__ inputs.

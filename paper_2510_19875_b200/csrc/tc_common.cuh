@@ -338,8 +338,8 @@ __host__ __device__ constexpr unsigned idesc_bf16(unsigned M, unsigned N, bool b
 // keep the k best by (score descending, candidate index ascending), the candidates numbered
 // 2 * lane (left) and 2 * lane + 1 (right); k <= 32.
 //
-// The k-th largest score is found with a sorting network instead of counting ranks (4096
-// comparisons, which made this the longest step of a row's level): the scores become unsigned
+// The k-th largest score is found with a sorting network (a first form counted ranks in one chain of 4096
+// comparisons; it is the chain that was slow, see select_topk_counting): the scores become unsigned
 // keys of the same order (-0 first brought to +0, so that equal floats give equal keys; an absent
 // candidate gets key 0, below every score), the 32 left keys are sorted descending and the 32
 // right keys ascending across the lanes (one bitonic network, 15 exchange steps, both registers
