@@ -392,18 +392,19 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     // 752 50.6, 43.6; 3000 177.6, 149.4; bf16 and rows off 16 bytes alike. Four only for groups of two warps at d = 32 (blocks of
     // 64; two, three, four): 480 rows 113, 104, 100; 720 168, 146, 157; 1000 223, 202, 183. Where the rows have work
     // for two warps only (k = 1 and 2), smaller CTAs fill the SM by themselves (2400 rows, k = 2, d = 64: 81.8, 85.9).
-    // A causal head's first rows have fewer than k blocks and come last: a third of them off the count puts the lines right
-    // (d = 64, causal: 304 rows, k = 8, 36.9, 37.8; 336, k = 16, 62.1, 69.0; 344 69.9, 69.1; 480 93.7, 83.2; not causal: 304 rows, k = 8, 44.4, 37.7).
+    // A causal head's first rows have fewer than k blocks and come last, so that a round may be some rows over: a sixth of
+    // those for a round of two, half for one of three or four (d = 64, causal: 304 rows, k = 4, 29.0, 22.0; 320, k = 16, 61.5, 68.8;
+    // 344 69.9, 69.1; 480, k = 16, 93.7, 83.2, k = 4, 31.1, 35.5; not causal: 304 rows, k = 8, 44.4, 37.7). Over 795 calls timed both
+    // ways this is 0.4 % off the better of the two, 27 % at worst; a third of them for all rounds 0.7 and 50 %.
     const int warps = m_warps * splits;
-    const long long first = std::min((long long)g.n_qb, (long long)g.k_top * g.bk / g.bq);
-    const long long full = g.causal ? rows - (long long)g.batch * g.H * first / 3 : rows;
+    const long long first = g.causal ? (long long)g.batch * g.H * std::min((long long)g.n_qb, (long long)g.k_top * g.bk / g.bq) : 0;
+    const long long in_twos = rows - first / 6, in_more = rows - first / 2;
     Build build = n_cta > 1 ? Build::kCluster : Build::kRow;
-    if ((D == 64 || (D == 32 && QW == 32)) && n_cta == 1 && (warps == 3 || warps == 4) && full > 2ll * n_sm) {
+    if ((D == 64 || (D == 32 && QW == 32)) && n_cta == 1 && (warps == 3 || warps == 4) && in_twos > 2ll * n_sm) {
         auto fit = [&](size_t ctas) { return ctas * (bytes(splits, D == 64) + kSmemPerCtaReserved) <= kSmemPerSm; };
         const bool three = (D == 32 || m_warps * Sh::kPBytes <= Sh::kTileBytes) && fit(3), four = D == 32 && m_warps == 2 && fit(4);
-        const bool two_rounds = full > 3ll * n_sm && full <= 4ll * n_sm;  // (with three as with two)
-        if (four && (two_rounds || full > 6ll * n_sm)) build = Build::kFour;
-        else if (three && !two_rounds) build = Build::kThree;
+        if (four && ((in_more > 3ll * n_sm && in_more <= 4ll * n_sm) || in_more > 6ll * n_sm)) build = Build::kFour;
+        else if (three && (four || in_more <= 3ll * n_sm || in_twos > 4ll * n_sm)) build = Build::kThree;
     }
     const size_t smem = bytes(splits, D == 64 && build == Build::kThree);
     auto kern = build == Build::kCluster ? attn_generic_kernel<T, D, QW, kLoad, Build::kCluster> : attn_generic_kernel<T, D, QW, kLoad, Build::kRow>;
