@@ -76,7 +76,9 @@ typedef struct {
 
 /* Counters a mask build leaves in the first bytes of its workspace. */
 typedef struct {
-    uint64_t tiles_scored; /* (row, representative key block) tiles whose score was computed */
+    uint64_t tiles_scored; /* (row, representative key block) tiles whose score was computed. (Where no scores are
+                              asked for, a row with no more allowed blocks than k needs none: it keeps
+                              them all. Its tiles are counted all the same.) */
     uint64_t rows;         /* rows finished */
     uint32_t error;        /* 0, or a code saying which bounded wait ran out (kernel returned early) */
     uint32_t error_info;

@@ -68,6 +68,8 @@ bool mask_tc_supported(const Geom &g, int dtype);  // d = 128, blocks of 64, k_t
 bool mask_tc_auto(const Geom &g, int dtype);       // what the kernel is the better choice for beyond that
 stream_status launch_mask_tc(const Geom &g, const void *q, const void *k, int32_t *mask, float *score,
                              WorkspaceHeader *ws, cudaStream_t st);
+// A build all of whose rows keep every block they are allowed (whole_query_blocks(g) == g.n_qb), no scores asked for.
+stream_status launch_mask_whole(const Geom &g, int32_t *mask, WorkspaceHeader *ws, cudaStream_t st);
 // Several k in one launch (mk.n >= 1: mask / score are [mk.n][rows][k_top]); with score_memory
 // (mask_tc_score_memory_bytes(g) bytes, device) a (row, block) tile is scored once for all k.
 size_t mask_tc_score_memory_bytes(const Geom &g);
@@ -167,6 +169,21 @@ __host__ __device__ inline int last_valid_block(const Geom &g, int qb) {
     long long last_tok = g.causal ? ((long long)qb * g.bq + g.bq - 1) : (g.T - 1);
     if (last_tok > g.T - 1) last_tok = g.T - 1;
     return (int)(last_tok / g.bk);
+}
+
+// A row whose allowed blocks are no more than its k keeps them all, whatever their scores: Algorithm 2 then drops nothing on any
+// level. How many query blocks, from the first, have such rows (bq == bk, or all of them alike): 0 unless k is the same for all.
+inline int whole_query_blocks(const Geom &g) {
+    if (g.k_row != nullptr) return 0;
+    const int k = g.k_override > 0 ? g.k_override : g.k_top;
+    if (last_valid_block(g, g.n_qb - 1) < k) return g.n_qb;
+    return g.causal && g.bq == g.bk ? k : 0;
+}
+
+// A warp writes such a row of n blocks: 0 .. n - 1, -1 padded, and what scoring it would have counted.
+__device__ __forceinline__ void write_whole_row(const Geom &g, long long row, int n, int lane, int32_t *mask) {
+    for (int i = lane; i < g.k_top; i += 32) mask[row * g.k_top + i] = i < n ? i : -1;
+    if (lane == 0 && g.row_tiles != nullptr) g.row_tiles[row] = g.levels > 0 ? (unsigned)n : 0u;
 }
 
 }  // namespace stream

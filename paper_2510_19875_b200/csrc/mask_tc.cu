@@ -15,8 +15,8 @@
 // row keeps the row's nodes in registers, ranks the 2k branch scores (higher score, then lower block
 // index), compacts the survivors with ballots and publishes the next level's fetch list. The
 // first level's representatives are the same for every row of a group, so one fetched stage
-// serves all its rows; from the second level on a left branch inherits its parent's score and
-// only right branches are fetched. With several k per call a group runs the hierarchy once per
+// serves all its rows (levels that cannot drop anything are passed over before it: FirstNodes); from the second
+// level on a left branch inherits its parent's score and only right branches are fetched. With several k per call a group runs the hierarchy once per
 // k on the same Q tiles and fetches only blocks whose score it does not have yet.
 //
 // Nothing of a group's beginning waits for the end of the group before: a dispatcher warp has the next
@@ -105,9 +105,11 @@ struct Tail {
     unsigned int tmem_base;
     int abort_flag;
     int grp_id, grp_b, grp_kvh, grp_qb, grp_h0, grp_R;
-    int grp_levels;  // levels of this group's rows (they share the query block, hence k)
+    int grp_levels;  // levels of this group's rows that have something to rank (they share the query block, hence k)
     int grp_k, grp_pass;
-    unsigned grp_on[2 * S::kNodes];  // bit i of [2 x], [2 x + 1]: the left, right candidate of initial node kNodes i + x is on the first list
+    int grp_nodes, grp_f[32 * S::kNodes], grp_l[32 * S::kNodes];  // the nodes before the first of them: first and last block
+    int split_f[32 * S::kNodes], split_l[32 * S::kNodes];         // (the dispatcher's own, on the way there)
+    unsigned grp_on[2 * S::kNodes];  // bit i of [2 x], [2 x + 1]: the left, right candidate of node kNodes i + x is on the first list
     int grp_new_q;   // 0: another pass over the same rows (several k), the Q tiles are already there
     int grp_last;    // the last pass over these rows: the Q tiles are given back
     int n_jobs[kR + 1];
@@ -140,6 +142,7 @@ constexpr unsigned kIdescTwo = idesc_bf16(128, 2 * S::kBlk, false);
 struct Params {
     Geom g;
     int n_groups, n_chunks;
+    int first_qb;  // the rows of the query blocks before it keep all they are allowed, and belong to no group
     // A group's rows: head_rows query heads, at each of qb_rows query blocks (more than one only where
     // all heads of the kv head are in the group): row r is head r % head_rows at the group's query
     // block minus r / head_rows, which row_head and row_back hold in two bits a row.
@@ -490,19 +493,6 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
 // Dispatcher and controllers ------------------------------------------------------------------------
 // kMulti: several k per group with the score memory; false compiles the plain single-pass form.
 
-// The two candidates of an initial node (the same for every row of a group).
-struct FirstNode {
-    int f, l, m;
-    bool vl, vr;
-    __device__ FirstNode(const Geom &g, int kq, int q_lim, int i) {
-        f = (int)(((long long)i * g.N_k) / kq);
-        l = (int)(((long long)(i + 1) * g.N_k) / kq) - 1;
-        m = (f + l) / 2;
-        vl = i < kq && f <= l && f <= q_lim;
-        vr = vl && m + 1 <= l && m + 1 <= q_lim;
-    }
-};
-
 // Places of a warp's flags, n of them a lane, in lane order: those before this lane's; all of them.
 template <int n>
 __device__ __forceinline__ int flags_before(const unsigned (&ballots)[n], unsigned lt) {
@@ -514,11 +504,83 @@ __device__ __forceinline__ int flags_before(const unsigned (&ballots)[n], unsign
 template <int n>
 __device__ __forceinline__ int flags_all(const unsigned (&ballots)[n]) { return flags_before(ballots, 0xffffffffu); }
 
-// Is block blk a first-level candidate of a build with k = kq?
-__device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int blk) {
+// Is block blk a candidate of the first list of a build with k = kq, whose nodes have been split `splits` times?
+__device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int splits, int blk) {
     const int i = (int)(((long long)(blk + 1) * kq - 1) / g.N_k);  // the node that holds blk: the last that begins at or before it
-    const int f = (int)(((long long)i * g.N_k) / kq), l = (int)(((long long)(i + 1) * g.N_k) / kq) - 1;
+    int f = (int)(((long long)i * g.N_k) / kq), l = (int)(((long long)(i + 1) * g.N_k) / kq) - 1;
+    for (int x = 0; x < splits; ++x) {
+        const int m = (f + l) / 2;
+        if (blk <= m) l = m;
+        else f = m + 1;
+    }
     return blk == f || blk == (f + l) / 2 + 1;
+}
+
+// The nodes of query block `qb`'s rows (their last allowed block: q_lim) before the first level that ranks anything; n of them.
+// A level with no more than kq allowed candidates keeps them all whatever their scores, so its scores are not waited for:
+// its candidates are split on, and what there is to score of them comes with the next level's (a left branch has its
+// parent's score), in the one list that all rows of a group share. So it is with the first level of every row that may look at half of
+// the blocks at most, the first two where it is a quarter. `splits`: such levels. The last level always has its list. (us, mask build
+// with all levels ranked and now: 32 / 8 heads, 4096 tokens, k = 32: 71.4, 50.7; 16384, k = 16: 526, 492; 131072, k = 32: 12050,
+// 11620; four layers of 9999, 28 / 4 heads, k = 16: 994, 914; 12 / 2 heads, 10007 tokens in blocks of 32, k = 8: 129.6, 116.7.)
+template <class S>
+struct FirstNodes {
+    int f[S::kNodes], l[S::kNodes];  // this lane's (l < f: none)
+    int n, splits;
+    bool left[S::kNodes], right[S::kNodes];  // candidates: first half, second half
+    __device__ __forceinline__ FirstNodes(const Geom &g, int kq, int levels, int q_lim, int lane, int *room_f, int *room_l) {
+        const unsigned lt = (1u << lane) - 1u;
+        unsigned ballots[2 * S::kNodes];
+#pragma unroll
+        for (int x = 0; x < S::kNodes; ++x) {
+            const int i = S::kNodes * lane + x;
+            f[x] = (int)(((long long)i * g.N_k) / kq);
+            l[x] = i < kq ? (int)(((long long)(i + 1) * g.N_k) / kq) - 1 : f[x] - 1;
+        }
+        n = kq;
+        for (splits = 0;; ++splits) {
+#pragma unroll
+            for (int x = 0; x < S::kNodes; ++x) {
+                const int m = (f[x] + l[x]) / 2;
+                left[x] = f[x] <= l[x] && f[x] <= q_lim;
+                right[x] = left[x] && m + 1 <= l[x] && m + 1 <= q_lim;
+                ballots[2 * x] = __ballot_sync(0xffffffffu, left[x]);
+                ballots[2 * x + 1] = __ballot_sync(0xffffffffu, right[x]);
+            }
+            const int total = flags_all(ballots);
+            if (total > kq || splits + 1 >= levels) return;
+            int place = flags_before(ballots, lt);
+            __syncwarp();
+#pragma unroll
+            for (int x = 0; x < S::kNodes; ++x) {
+                const int m = (f[x] + l[x]) / 2;
+                if (left[x]) { room_f[place] = f[x]; room_l[place++] = m; }
+                if (right[x]) { room_f[place] = m + 1; room_l[place++] = l[x]; }
+            }
+            __syncwarp();
+            n = total;
+#pragma unroll
+            for (int x = 0; x < S::kNodes; ++x) {
+                const int i = S::kNodes * lane + x;
+                f[x] = i < n ? room_f[i] : 0;
+                l[x] = i < n ? room_l[i] : -1;
+            }
+        }
+    }
+};
+
+// The rows that keep all blocks they are allowed (P.first_qb): a warp a row, all warps of the launch that call this.
+__device__ __forceinline__ void whole_rows(const Params &P, int warp, int n_warps, int lane) {
+    const Geom &g = P.g;
+    const int heads = g.batch * g.H, n = heads * P.first_qb;
+    for (int i = (int)blockIdx.x * n_warps + warp; i < n; i += (int)gridDim.x * n_warps) {
+        const int bh = i / P.first_qb, qb = i - bh * P.first_qb;
+        write_whole_row(g, (long long)bh * g.n_qb + qb, last_valid_block(g, qb) + 1, lane, P.mask);
+    }
+    if (blockIdx.x == 0 && warp == 0 && lane == 0 && n > 0) {
+        atomicAdd(&P.ws->tiles_scored, (unsigned long long)heads * (unsigned long long)P.first_qb * (unsigned long long)(P.first_qb + 1) / 2ull);
+        atomicAdd(&P.ws->rows, (unsigned long long)n);
+    }
 }
 
 template <class S>
@@ -527,6 +589,7 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
     constexpr bool kMulti = S::kMulti;
     constexpr int kNodes = S::kNodes;
     const unsigned lt = (1u << lane) - 1u;
+    int splits_of = 0;  // lane i: of the group's pass i
     unsigned ack_par = 1, q_par = (1u << kR) - 1u;  // (the first waits pass at once)
     unsigned long long fetched = 0;  // Q tiles asked of TMA
     int next = -1;  // (lane 0) the next group's number, if it has been fetched
@@ -541,32 +604,36 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
         if (lane == 0 && id + 2 * (int)gridDim.x < P.n_groups) next = (int)atomicAdd(&P.ws->work_counter, 1u);
         int b = 0, kvh = 0, qb = 0, h0 = 0, R = 0;
         if (!done) {
-            const int per = (g.n_qb + P.qb_rows - 1) / P.qb_rows * P.n_chunks;
+            const int per = (g.n_qb - P.first_qb + P.qb_rows - 1) / P.qb_rows * P.n_chunks;
             const int bkv = id / per, rem = id % per;
             b = bkv / g.G; kvh = bkv % g.G;
             qb = g.n_qb - 1 - rem / P.n_chunks * P.qb_rows;  // late (expensive) query blocks first
             const int chunk = rem % P.n_chunks;
             h0 = kvh * g.hpg + chunk * P.head_rows;
-            R = min(P.head_rows, g.hpg - chunk * P.head_rows) * min(P.qb_rows, qb + 1);
+            R = min(P.head_rows, g.hpg - chunk * P.head_rows) * min(P.qb_rows, qb - P.first_qb + 1);
         }
         const int q_lim = last_valid_block(g, qb);
         const int n_pass = (!kMulti || done) ? 1 : P.mk.n;
         for (int pass = 0; pass < n_pass; ++pass) {
             const int kq = done ? g.k_top : (kMulti ? P.mk.k[pass] : row_k(g, qb));
+            const int levels = row_levels(g, kq);
+            const FirstNodes<S> nodes(g, kq, levels, q_lim, lane, tl->split_f, tl->split_l);
             bool on[2 * kNodes];  // goes on the list
             int cand[2 * kNodes];
             unsigned ballots[2 * kNodes];
 #pragma unroll
             for (int x = 0; x < kNodes; ++x) {
-                const FirstNode fn(g, kq, q_lim, kNodes * lane + x);
-                cand[2 * x] = fn.f; cand[2 * x + 1] = fn.m + 1;
-                on[2 * x] = fn.vl && !done; on[2 * x + 1] = fn.vr && !done;
+                cand[2 * x] = nodes.f[x]; cand[2 * x + 1] = (nodes.f[x] + nodes.l[x]) / 2 + 1;
+                on[2 * x] = nodes.left[x] && !done; on[2 * x + 1] = nodes.right[x] && !done;
             }
             // Not what an earlier pass has had on its first list: every row has that score. (What rows have
             // met on later levels is for their controllers to know, which may still be at it.)
-            for (int e = 0; kMulti && e < pass; ++e)
+            for (int e = 0; kMulti && e < pass; ++e) {
+                const int splits = __shfl_sync(0xffffffffu, splits_of, e);
 #pragma unroll
-                for (int x = 0; x < 2 * kNodes; ++x) on[x] = on[x] && !on_first_list(g, P.mk.k[e], cand[x]);
+                for (int x = 0; x < 2 * kNodes; ++x) on[x] = on[x] && !on_first_list(g, P.mk.k[e], splits, cand[x]);
+            }
+            if (kMulti && lane == pass) splits_of = nodes.splits;
 #pragma unroll
             for (int x = 0; x < 2 * kNodes; ++x) ballots[x] = __ballot_sync(0xffffffffu, on[x]);
             int place = flags_before(ballots, lt);
@@ -575,11 +642,13 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
 #pragma unroll
             for (int x = 0; x < 2 * kNodes; ++x)
                 if (on[x]) tl->first_blk[place++] = cand[x];
+#pragma unroll
+            for (int x = 0; x < kNodes; ++x) { tl->grp_f[kNodes * lane + x] = nodes.f[x]; tl->grp_l[kNodes * lane + x] = nodes.l[x]; }
             if (lane == 0) {
                 tl->n_jobs[kR] = flags_all(ballots);
                 tl->grp_id = done ? -1 : id; tl->grp_b = b; tl->grp_kvh = kvh; tl->grp_qb = qb; tl->grp_h0 = h0; tl->grp_R = R;
-                tl->grp_levels = row_levels(g, kq);
-                tl->grp_k = kq; tl->grp_pass = pass;
+                tl->grp_levels = levels - nodes.splits;
+                tl->grp_k = kq; tl->grp_pass = pass; tl->grp_nodes = nodes.n;
 #pragma unroll
                 for (int x = 0; x < 2 * kNodes; ++x) tl->grp_on[x] = ballots[x];
                 tl->grp_new_q = pass == 0;
@@ -631,10 +700,13 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
         const unsigned set = grp_par;
         grp_par ^= 1;
         const int id = tl->grp_id, b = tl->grp_b, qb = S::kQbRows ? tl->grp_qb - (int)((P.row_back >> (2 * r)) & 3u) : tl->grp_qb, h = tl->grp_h0 + (S::kQbRows ? (int)((P.row_head >> (2 * r)) & 3u) : r), R = tl->grp_R, levels = tl->grp_levels;
-        const int kq = tl->grp_k, pass = tl->grp_pass;
+        const int kq = tl->grp_k, pass = tl->grp_pass, first_nodes = tl->grp_nodes;
         unsigned on[2 * kNodes];
+        int nf[kNodes], nl[kNodes];       // this lane's nodes
 #pragma unroll
         for (int x = 0; x < 2 * kNodes; ++x) on[x] = tl->grp_on[x];
+#pragma unroll
+        for (int x = 0; x < kNodes; ++x) { nf[x] = tl->grp_f[kNodes * lane + x]; nl[x] = tl->grp_l[kNodes * lane + x]; }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ack[kR]));  // (the list itself is not needed)
         if (id < 0) {
@@ -649,21 +721,19 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
         const unsigned tag = (unsigned)id + 1u;  // marks this group's entries of the score memory (0 = never written)
         // A level's candidates, in ascending order: left and right of every node. cand: what they keep if
         // they survive (first and last block, score); have: it is there.
-        int nf[kNodes], nl[kNodes];       // this lane's nodes
-        float ns[kNodes];
+        float ns[kNodes];                 // its nodes' scores
         bool has[2 * kNodes];
         float sc[2 * kNodes];
         unsigned tiles = 0;               // (row, block) tiles that had no score yet
 #pragma unroll
         for (int x = 0; x < kNodes; ++x) {
-            const FirstNode fn(g, kq, q_lim, kNodes * lane + x);
-            nf[x] = fn.f; nl[x] = fn.l;
-            has[2 * x] = fn.vl; has[2 * x + 1] = fn.vr;
-            bool miss_l = fn.vl, miss_r = fn.vr;
+            const int rb = (nf[x] + nl[x]) / 2 + 1;
+            bool miss_l = nf[x] <= nl[x] && nf[x] <= q_lim, miss_r = miss_l && rb <= nl[x] && rb <= q_lim;
+            has[2 * x] = miss_l; has[2 * x + 1] = miss_r;
             sc[2 * x] = sc[2 * x + 1] = -CUDART_INF_F;
             if (kMulti) {
-                if (fn.vl && remembered(fn.f, tag, sc[2 * x])) miss_l = false;
-                if (fn.vr && remembered(fn.m + 1, tag, sc[2 * x + 1])) miss_r = false;
+                if (miss_l && remembered(nf[x], tag, sc[2 * x])) miss_l = false;
+                if (miss_r && remembered(rb, tag, sc[2 * x + 1])) miss_r = false;
             }
             tiles += (unsigned)(__popc(__ballot_sync(0xffffffffu, miss_l)) + __popc(__ballot_sync(0xffffffffu, miss_r)));
         }
@@ -698,7 +768,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
             }
             bool keep[2 * kNodes];
             if constexpr (kNodes == 1) {
-                const Keep kp = select_topk_counting(has[0], sc[0], has[1], sc[1], kq, level == 0 ? kq : n_nodes, lane, tl->keys[r]);
+                const Keep kp = select_topk_counting(has[0], sc[0], has[1], sc[1], kq, level == 0 ? first_nodes : n_nodes, lane, tl->keys[r]);
                 keep[0] = kp.l; keep[1] = kp.r;
             } else {
                 select_topk_of<2 * kNodes>(has, sc, kq, lane, keep);
@@ -812,6 +882,7 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     // issuing role and two of the controllers', spread over all schedulers, cost a quarter of the
     // kernel's time in instruction fetches.
     if (warp >= 4 && warp < 12) {
+        if constexpr (!S::kMulti) whole_rows(P, warp - 4, 8, lane);  // (they have nothing to reduce yet)
         epilogue_role(P, tl, tmem_base, warp & 3, (warp - 4) >> 2, lane);
     } else if (warp == 1 || warp == 3 || warp == 13 || warp == 17) {
         mma_role(P, tl, q_smem, k_smem, tmem_base, warp == 1 ? 0 : (warp == 3 ? 1 : (warp == 13 ? 2 : 3)));
@@ -855,7 +926,7 @@ namespace {
 // own keys, 8192 tokens, d = 64, k = 40, not causal: a row a group 229 us, four 156), unless k changes
 // from one to the next.
 struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
-stream_status split_rows(const Geom &g, Split *s) {
+stream_status split_rows(const Geom &g, int first_qb, Split *s) {
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
     s->n_chunks = (g.hpg + kR - 1) / kR;
@@ -864,7 +935,7 @@ stream_status split_rows(const Geom &g, Split *s) {
     if (s->qb_rows < 1) s->qb_rows = 1;
     for (;;) {
         s->n_chunks = (g.hpg + s->head_rows - 1) / s->head_rows;
-        s->n_groups = (long long)g.batch * g.G * ((g.n_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
+        s->n_groups = (long long)g.batch * g.G * ((g.n_qb - first_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
         if (s->n_groups >= (g.k_top > 32 ? 3 : 2) * n_sm || s->head_rows * s->qb_rows == 1) break;
         if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
         else s->head_rows = (s->head_rows + 1) / 2;
@@ -889,7 +960,7 @@ cudaError_t launch_rows(const Geom &g, const Split &sp, cudaStream_t st, const C
 
 size_t mask_tc_score_memory_bytes(const Geom &g) {
     Split sp;
-    if (split_rows(g, &sp) != STREAM_OK) return 0;
+    if (split_rows(g, 0, &sp) != STREAM_OK) return 0;
     return (size_t)sp.grid * kR * (size_t)g.N_k * sizeof(unsigned long long);
 }
 
@@ -912,8 +983,11 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;
+    // The rows of one build that keep every block they are allowed, with no score asked for, need no products.
+    P.first_qb = mk.n == 0 && score == nullptr ? whole_query_blocks(g) : 0;
+    if (P.first_qb == g.n_qb) return launch_mask_whole(g, mask, ws, st);
     Split sp;
-    rc = split_rows(g, &sp);
+    rc = split_rows(g, P.first_qb, &sp);
     if (rc != STREAM_OK) return rc;
     P.n_groups = (int)sp.n_groups;
     P.n_chunks = sp.n_chunks; P.head_rows = sp.head_rows; P.qb_rows = sp.qb_rows;
