@@ -172,18 +172,32 @@ __host__ __device__ inline int last_valid_block(const Geom &g, int qb) {
 }
 
 // A row whose allowed blocks are no more than its k keeps them all, whatever their scores: Algorithm 2 then drops nothing on any
-// level. How many query blocks, from the first, have such rows (bq == bk, or all of them alike): 0 unless k is the same for all.
+// level. How many query blocks, from the first, have such rows: 0 unless k is the same for all.
 inline int whole_query_blocks(const Geom &g) {
     if (g.k_row != nullptr) return 0;
     const int k = g.k_override > 0 ? g.k_override : g.k_top;
     if (last_valid_block(g, g.n_qb - 1) < k) return g.n_qb;
-    return g.causal && g.bq == g.bk ? k : 0;
+    return g.causal ? (int)((long long)k * g.bk / g.bq) : 0;
 }
 
-// A warp writes such a row of n blocks: 0 .. n - 1, -1 padded, and what scoring it would have counted.
-__device__ __forceinline__ void write_whole_row(const Geom &g, long long row, int n, int lane, int32_t *mask) {
-    for (int i = lane; i < g.k_top; i += 32) mask[row * g.k_top + i] = i < n ? i : -1;
-    if (lane == 0 && g.row_tiles != nullptr) g.row_tiles[row] = g.levels > 0 ? (unsigned)n : 0u;
+// Writes the rows of every head's first n_qb query blocks as such: their allowed blocks, -1 padded, and what scoring them would have
+// counted, whose sum for this thread it returns. Thread `at` of n_threads that do so.
+__device__ __forceinline__ unsigned long long write_whole_rows(const Geom &g, int n_qb, unsigned at, unsigned n_threads, int32_t *mask) {
+    const unsigned per_head = (unsigned)n_qb * (unsigned)g.k_top;
+    const unsigned long long n = (unsigned long long)g.batch * g.H * per_head;
+    unsigned long long tiles = 0;
+    for (unsigned long long x = at; x < n; x += n_threads) {
+        const unsigned head = (unsigned)(x / per_head), rest = (unsigned)(x - (unsigned long long)head * per_head), qb = rest / (unsigned)g.k_top, i = rest - qb * (unsigned)g.k_top;
+        const long long row = (long long)head * g.n_qb + qb;
+        const int n_blocks = last_valid_block(g, (int)qb) + 1;
+        mask[row * g.k_top + i] = (int)i < n_blocks ? (int)i : -1;
+        if (i == 0u) {
+            const unsigned t = g.levels > 0 ? (unsigned)n_blocks : 0u;
+            tiles += t;
+            if (g.row_tiles != nullptr) g.row_tiles[row] = t;
+        }
+    }
+    return tiles;
 }
 
 }  // namespace stream

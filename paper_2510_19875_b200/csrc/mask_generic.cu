@@ -590,27 +590,22 @@ stream_status mma_d(const Geom &g, const MultiK &mk, const void *q, const void *
 // ----------------------------------------------------------------------------------------------
 // Builds that drop nothing
 // ----------------------------------------------------------------------------------------------
-// No row has more allowed blocks than it may keep: every row is its allowed blocks, and no key is read. A warp a row; bound by
-// the launch (32 heads, 1000 tokens in blocks of 64, k = 16: 24.0 us with all scores computed, 13.1 a call in a loop, the host's part).
+// No row has more allowed blocks than it may keep: every row is its allowed blocks, and no key is read. Bound by the launch (32
+// heads, 1000 tokens in blocks of 64, k = 16: 24.0 us with all scores computed, 13.1 a call in a loop, the host's part).
 constexpr int kWholeThreads = 256;
 __global__ void __launch_bounds__(kWholeThreads) mask_whole_kernel(Geom g, int32_t *mask, WorkspaceHeader *ws) {
     after_previous_kernel();
-    const int lane = threadIdx.x & 31, warps = kWholeThreads / 32;
-    const long long rows = (long long)g.batch * g.H * g.n_qb, step = (long long)gridDim.x * warps;
-    unsigned long long tiles = 0;
-    for (long long row = (long long)blockIdx.x * warps + (threadIdx.x >> 5); row < rows; row += step) {
-        const int n = last_valid_block(g, (int)(row % g.n_qb)) + 1;
-        write_whole_row(g, row, n, lane, mask);
-        tiles += (unsigned long long)n;
-    }
-    if (lane == 0 && g.levels > 0 && tiles > 0) atomicAdd(&ws->tiles_scored, tiles);
-    if (blockIdx.x == 0 && threadIdx.x == 0) ws->rows = (unsigned long long)rows;
+    unsigned long long tiles = write_whole_rows(g, g.n_qb, blockIdx.x * kWholeThreads + threadIdx.x, gridDim.x * kWholeThreads, mask);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tiles += __shfl_xor_sync(0xffffffffu, tiles, o);
+    if ((threadIdx.x & 31) == 0 && tiles > 0) atomicAdd(&ws->tiles_scored, tiles);
+    if (blockIdx.x == 0 && threadIdx.x == 0) ws->rows = (unsigned long long)g.batch * g.H * g.n_qb;
 }
 
 }  // namespace
 
 stream_status launch_mask_whole(const Geom &g, int32_t *mask, WorkspaceHeader *ws, cudaStream_t st) {
-    const long long rows = (long long)g.batch * g.H * g.n_qb, blocks = (rows * 32 + kWholeThreads - 1) / kWholeThreads, most = 8 * sm_count_or_default();
+    const long long rows = (long long)g.batch * g.H * g.n_qb, blocks = (rows * g.k_top + kWholeThreads - 1) / kWholeThreads, most = 8 * sm_count_or_default();
     const cudaError_t e = launch_kernel(mask_whole_kernel, (unsigned)(blocks < most ? blocks : most), kWholeThreads, 0, st, 1, g, mask, ws);
     return e == cudaSuccess ? STREAM_OK : cuda_fail(e, "mask_whole launch");
 }

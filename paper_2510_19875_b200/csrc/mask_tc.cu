@@ -493,17 +493,6 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
 // Dispatcher and controllers ------------------------------------------------------------------------
 // kMulti: several k per group with the score memory; false compiles the plain single-pass form.
 
-// Places of a warp's flags, n of them a lane, in lane order: those before this lane's; all of them.
-template <int n>
-__device__ __forceinline__ int flags_before(const unsigned (&ballots)[n], unsigned lt) {
-    int c = 0;
-#pragma unroll
-    for (int i = 0; i < n; ++i) c += __popc(ballots[i] & lt);
-    return c;
-}
-template <int n>
-__device__ __forceinline__ int flags_all(const unsigned (&ballots)[n]) { return flags_before(ballots, 0xffffffffu); }
-
 // Is block blk a candidate of the first list of a build with k = kq, whose nodes have been split `splits` times?
 __device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int splits, int blk) {
     const int i = (int)(((long long)(blk + 1) * kq - 1) / g.N_k);  // the node that holds blk: the last that begins at or before it
@@ -514,73 +503,6 @@ __device__ __forceinline__ bool on_first_list(const Geom &g, int kq, int splits,
         else f = m + 1;
     }
     return blk == f || blk == (f + l) / 2 + 1;
-}
-
-// The nodes of query block `qb`'s rows (their last allowed block: q_lim) before the first level that ranks anything; n of them.
-// A level with no more than kq allowed candidates keeps them all whatever their scores, so its scores are not waited for:
-// its candidates are split on, and what there is to score of them comes with the next level's (a left branch has its
-// parent's score), in the one list that all rows of a group share. So it is with the first level of every row that may look at half of
-// the blocks at most, the first two where it is a quarter. `splits`: such levels. The last level always has its list. (us, mask build
-// with all levels ranked and now: 32 / 8 heads, 4096 tokens, k = 32: 71.4, 50.7; 16384, k = 16: 526, 492; 131072, k = 32: 12050,
-// 11620; four layers of 9999, 28 / 4 heads, k = 16: 994, 914; 12 / 2 heads, 10007 tokens in blocks of 32, k = 8: 129.6, 116.7.)
-template <class S>
-struct FirstNodes {
-    int f[S::kNodes], l[S::kNodes];  // this lane's (l < f: none)
-    int n, splits;
-    bool left[S::kNodes], right[S::kNodes];  // candidates: first half, second half
-    __device__ __forceinline__ FirstNodes(const Geom &g, int kq, int levels, int q_lim, int lane, int *room_f, int *room_l) {
-        const unsigned lt = (1u << lane) - 1u;
-        unsigned ballots[2 * S::kNodes];
-#pragma unroll
-        for (int x = 0; x < S::kNodes; ++x) {
-            const int i = S::kNodes * lane + x;
-            f[x] = (int)(((long long)i * g.N_k) / kq);
-            l[x] = i < kq ? (int)(((long long)(i + 1) * g.N_k) / kq) - 1 : f[x] - 1;
-        }
-        n = kq;
-        for (splits = 0;; ++splits) {
-#pragma unroll
-            for (int x = 0; x < S::kNodes; ++x) {
-                const int m = (f[x] + l[x]) / 2;
-                left[x] = f[x] <= l[x] && f[x] <= q_lim;
-                right[x] = left[x] && m + 1 <= l[x] && m + 1 <= q_lim;
-                ballots[2 * x] = __ballot_sync(0xffffffffu, left[x]);
-                ballots[2 * x + 1] = __ballot_sync(0xffffffffu, right[x]);
-            }
-            const int total = flags_all(ballots);
-            if (total > kq || splits + 1 >= levels) return;
-            int place = flags_before(ballots, lt);
-            __syncwarp();
-#pragma unroll
-            for (int x = 0; x < S::kNodes; ++x) {
-                const int m = (f[x] + l[x]) / 2;
-                if (left[x]) { room_f[place] = f[x]; room_l[place++] = m; }
-                if (right[x]) { room_f[place] = m + 1; room_l[place++] = l[x]; }
-            }
-            __syncwarp();
-            n = total;
-#pragma unroll
-            for (int x = 0; x < S::kNodes; ++x) {
-                const int i = S::kNodes * lane + x;
-                f[x] = i < n ? room_f[i] : 0;
-                l[x] = i < n ? room_l[i] : -1;
-            }
-        }
-    }
-};
-
-// The rows that keep all blocks they are allowed (P.first_qb): a warp a row, all warps of the launch that call this.
-__device__ __forceinline__ void whole_rows(const Params &P, int warp, int n_warps, int lane) {
-    const Geom &g = P.g;
-    const int heads = g.batch * g.H, n = heads * P.first_qb;
-    for (int i = (int)blockIdx.x * n_warps + warp; i < n; i += (int)gridDim.x * n_warps) {
-        const int bh = i / P.first_qb, qb = i - bh * P.first_qb;
-        write_whole_row(g, (long long)bh * g.n_qb + qb, last_valid_block(g, qb) + 1, lane, P.mask);
-    }
-    if (blockIdx.x == 0 && warp == 0 && lane == 0 && n > 0) {
-        atomicAdd(&P.ws->tiles_scored, (unsigned long long)heads * (unsigned long long)P.first_qb * (unsigned long long)(P.first_qb + 1) / 2ull);
-        atomicAdd(&P.ws->rows, (unsigned long long)n);
-    }
 }
 
 template <class S>
@@ -617,7 +539,7 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
         for (int pass = 0; pass < n_pass; ++pass) {
             const int kq = done ? g.k_top : (kMulti ? P.mk.k[pass] : row_k(g, qb));
             const int levels = row_levels(g, kq);
-            const FirstNodes<S> nodes(g, kq, levels, q_lim, lane, tl->split_f, tl->split_l);
+            const FirstNodes<kNodes> nodes(g, kq, levels, q_lim, lane, tl->split_f, tl->split_l);
             bool on[2 * kNodes];  // goes on the list
             int cand[2 * kNodes];
             unsigned ballots[2 * kNodes];
@@ -882,7 +804,13 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     // issuing role and two of the controllers', spread over all schedulers, cost a quarter of the
     // kernel's time in instruction fetches.
     if (warp >= 4 && warp < 12) {
-        if constexpr (!S::kMulti) whole_rows(P, warp - 4, 8, lane);  // (they have nothing to reduce yet)
+        if constexpr (!S::kMulti) {  // (they have nothing to reduce yet)
+            if (P.first_qb > 0) {
+                const unsigned long long tiles = write_whole_rows(P.g, P.first_qb, blockIdx.x * 256u + threadIdx.x - 128u, gridDim.x * 256u, P.mask);
+                if (tiles > 0) atomicAdd(&P.ws->tiles_scored, tiles);
+                if (blockIdx.x == 0 && threadIdx.x == 128) atomicAdd(&P.ws->rows, (unsigned long long)P.g.batch * P.g.H * P.first_qb);
+            }
+        }
         epilogue_role(P, tl, tmem_base, warp & 3, (warp - 4) >> 2, lane);
     } else if (warp == 1 || warp == 3 || warp == 13 || warp == 17) {
         mma_role(P, tl, q_smem, k_smem, tmem_base, warp == 1 ? 0 : (warp == 3 ? 1 : (warp == 13 ? 2 : 3)));

@@ -55,8 +55,11 @@ struct Tail {
     int n_list;          // blocks in the current level's list
     int n_nodes[kTok];   // surviving nodes per token
     int n_tiles[kTok];   // tiles the token has needed so far (a warp's ranking keeps them here)
-    unsigned node0[32];  // the initial nodes (the same for every token), and of the group: the places of
-    unsigned place0[32]; // their left | right << 16 candidates in the first level's list
+    // Of the group, the same for every token: its levels that rank anything, the nodes before the first of
+    // them, the places of their left | right << 16 candidates in its list.
+    int n_levels, n_node0;
+    unsigned node0[32], place0[32];
+    int split_f[32], split_l[32];  // (on the way to the nodes)
 };
 
 // Dynamic shared memory behind the 1024-byte aligned base:
@@ -77,7 +80,8 @@ constexpr unsigned kNoBlock = 0xffffu;  // (behind every block)
 
 struct Params {
     Geom g;
-    int n_items, n_tb;   // groups; groups per head (ceil(T / 128))
+    int n_items, n_tb;   // groups; groups per head (ceil(T / 128)), but for
+    int first_tb;        // those before this one, whose tokens keep all blocks they are allowed
     int32_t *mask;
     float *score;
     WorkspaceHeader *ws;
@@ -156,14 +160,16 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int epi_grp = (warp >= 4 && warp < 12) ? (warp - 4) >> 2 : -1;   // reads the stages with this parity
     const int epi_tok = (warp & 3) * 32 + lane;                            // its token (TMEM lane)
 
-    const int kq = g.k_top, levels = g.levels;
-    if (tid < 32) {
-        const int f = (int)(((long long)tid * g.N_k) / kq), end = (int)(((long long)(tid + 1) * g.N_k) / kq);
-        tl->node0[tid] = tid < kq && f < end ? pack_node(f, end - f) : 0u;
-    }
+    const int kq = g.k_top;
     unsigned seq = 0;     // stages so far over the whole kernel (the same in every thread)
     unsigned q_par = 0;
     unsigned long long tiles_needed = 0, products = 0;  // per thread
+
+    // Warps without a part in the levels write the tokens' rows that belong to no group, beside the first one.
+    if (P.first_tb > 0 && (warp == 2 || warp >= 12)) {
+        tiles_needed += write_whole_rows(g, P.first_tb * kTok, blockIdx.x * 160u + (warp == 2 ? 0u : warp - 11u) * 32u + lane, gridDim.x * 160u, P.mask);
+        if (blockIdx.x == 0 && tid == 64) atomicAdd(&P.ws->rows, (unsigned long long)g.batch * g.H * P.first_tb * kTok);
+    }
 
     for (;;) {
         if (tid == 0) tl->item = (int)atomicAdd(&P.ws->work_counter, 1u);
@@ -171,7 +177,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int id = tl->item;
         if (id >= P.n_items || *(volatile int *)&tl->abort_flag) break;
         // head by head (the keys of one kv head stay in L2), late token groups (most allowed blocks) first
-        const int bh = id / P.n_tb, tb = P.n_tb - 1 - id % P.n_tb;
+        const int bh = id / P.n_tb, tb = P.first_tb + P.n_tb - 1 - id % P.n_tb;
         const int b = bh / g.H, h = bh % g.H, kvh = h / g.hpg;
         const long long tok0 = (long long)tb * kTok;
         const long long tq_max = min(tok0 + kTok - 1, g.T - 1);
@@ -186,17 +192,16 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
             __syncwarp();
         }
-        // initial nodes (the same for every token) and the first level's shared list
-        const int f0 = (int)(((long long)lane * g.N_k) / kq), l0 = (int)(((long long)(lane + 1) * g.N_k) / kq) - 1;
-        const int m0 = (f0 + l0) / 2;
-        const bool gl = lane < kq && f0 <= l0 && f0 <= q_lim_max, gr = gl && m0 + 1 <= l0 && m0 + 1 <= q_lim_max;
-        const unsigned bl = __ballot_sync(0xffffffffu, gl), br = __ballot_sync(0xffffffffu, gr);
-        const int pos_l0 = __popc(bl & lt) + __popc(br & lt), pos_r0 = pos_l0 + (gl ? 1 : 0);
+        // the nodes before the first level that ranks anything, and its list: the same for every token
         if (warp == 0) {
-            if (gl) list[pos_l0] = (unsigned short)f0;
-            if (gr) list[pos_r0] = (unsigned short)(m0 + 1);
-            tl->place0[lane] = (unsigned)pos_l0 | ((unsigned)pos_r0 << 16);
-            if (lane == 0) tl->n_list = __popc(bl) + __popc(br);
+            const FirstNodes<1> first(g, kq, g.levels, q_lim_max, lane, tl->split_f, tl->split_l);
+            const unsigned ballots[2] = {__ballot_sync(0xffffffffu, first.left[0]), __ballot_sync(0xffffffffu, first.right[0])};
+            const int pos_l = flags_before(ballots, lt), pos_r = pos_l + (first.left[0] ? 1 : 0);
+            if (first.left[0]) list[pos_l] = (unsigned short)first.f[0];
+            if (first.right[0]) list[pos_r] = (unsigned short)((first.f[0] + first.l[0]) / 2 + 1);
+            tl->node0[lane] = first.f[0] <= first.l[0] ? pack_node(first.f[0], first.l[0] - first.f[0] + 1) : 0u;
+            tl->place0[lane] = (unsigned)pos_l | ((unsigned)pos_r << 16);
+            if (lane == 0) { tl->n_list = flags_all(ballots); tl->n_node0 = first.n; tl->n_levels = g.levels - first.splits; }
         }
         // the token this thread reads accumulators for
         const long long e_tq = tok0 + epi_tok;
@@ -205,8 +210,9 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int key_end = e_ok ? (int)(g.causal ? e_tq + 1 : g.T) : 0;  // keys the token may look at: those before
         unsigned n_tiles = 0;  // tiles the token has needed so far (its own candidates, not the merged list)
 
-        for (int level = 0; level < levels; ++level) {
+        for (int level = 0;; ++level) {
             __syncthreads();  // the level's list is complete; the ranking of the level before is done
+            const bool last = level + 1 == tl->n_levels;
             const int n_list = tl->n_list, n_st = (n_list + 1) >> 1;
 
             if (is_producer) {
@@ -323,11 +329,10 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // lane per node, which spends 240 instructions of a warp on every token, 8000 clocks a level of
             // the 128 against 3000. (32 / 8 heads, 4096 tokens: k = 16 225 us that way, 160 this way; k = 24,
             // spilled, 304 this way, 224 that way.)
-            const bool last = level + 1 == levels;
             if constexpr (kSorted) {
             if (epi_grp == 0) {
                 const int t = epi_tok;
-                const int n = !e_ok ? 0 : (level == 0 ? kq : tl->n_nodes[t]);
+                const int n = !e_ok ? 0 : (level == 0 ? tl->n_node0 : tl->n_nodes[t]);
                 // Everything of the token goes to registers first: its nodes, and the keys of their left and
                 // right candidates (0: there is none).
                 unsigned nd[kNodes], own[2 * kNodes], key[2 * kNodes];
@@ -397,10 +402,11 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 bool vl, vr;
                 float sl = -CUDART_INF_F, sr = -CUDART_INF_F;
                 if (level == 0) {
-                    f = f0; l = l0; m = m0;
-                    vl = gl && f0 <= q_lim; vr = gr && m0 + 1 <= q_lim;
-                    if (vl) sl = scores[pos_l0 * kPad + t];
-                    if (vr) sr = scores[pos_r0 * kPad + t];
+                    const unsigned nd = tl->node0[lane], at = tl->place0[lane];
+                    f = (int)(nd & 0xffffu); l = f + (int)(nd >> 16) - 1; m = (f + l) / 2;
+                    vl = nd != 0u && f <= q_lim; vr = vl && l > f && m + 1 <= q_lim;
+                    if (vl) sl = scores[(at & 0xffffu) * kPad + t];
+                    if (vr) sr = scores[(at >> 16) * kPad + t];
                     const int n0 = __popc(__ballot_sync(0xffffffffu, vl)) + __popc(__ballot_sync(0xffffffffu, vr));
                     if (lane == 0) { tiles_needed += (unsigned long long)n0; tl->n_tiles[t] = n0; }
                 } else {
@@ -521,7 +527,11 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     if (rc != STREAM_OK) return rc;
     Params P;
     P.g = g;
-    P.n_tb = (int)((g.T + kTok - 1) / kTok);
+    // tokens that keep every block they are allowed, with no score asked for, need no products: whole groups of them have none
+    const int whole = score == nullptr ? whole_query_blocks(g) : 0;
+    if (whole == g.n_qb) return launch_mask_whole(g, mask, ws, st);
+    P.first_tb = whole / kTok;
+    P.n_tb = (int)((g.T + kTok - 1) / kTok) - P.first_tb;
     const long long n_items = (long long)g.batch * g.H * P.n_tb;
     P.n_items = (int)n_items;
     P.mask = mask; P.score = score; P.ws = ws;

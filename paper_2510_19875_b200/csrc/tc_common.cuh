@@ -452,6 +452,71 @@ __device__ __forceinline__ void select_topk_of(const bool (&have)[n], const floa
     }
 }
 
+// Places of a warp's flags, n of them a lane, in lane order: those before this lane's; all of them.
+template <int n>
+__device__ __forceinline__ int flags_before(const unsigned (&ballots)[n], unsigned lt) {
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) c += __popc(ballots[i] & lt);
+    return c;
+}
+template <int n>
+__device__ __forceinline__ int flags_all(const unsigned (&ballots)[n]) { return flags_before(ballots, 0xffffffffu); }
+
+// The nodes of a row, kNodes a lane of a warp, before the first level that ranks anything; n of them. q_lim: the row's last allowed
+// block, or that of the last of several rows.
+// A level with no more than kq allowed candidates keeps them all whatever their scores, so its scores are not waited for:
+// its candidates are split on, and what there is to score of them comes with the next level's (a left branch has its
+// parent's score), in the one list that all rows of a group share. So it is with the first level of every row that may look at half of
+// the blocks at most, the first two where it is a quarter. `splits`: such levels. The last level always has its list. (us, mask build
+// with all levels ranked and now: 32 / 8 heads, 4096 tokens, k = 32: 71.4, 50.7; 16384, k = 16: 526, 492; 131072, k = 32: 12050,
+// 11620; four layers of 9999, 28 / 4 heads, k = 16: 994, 914; 12 / 2 heads, 10007 tokens in blocks of 32, k = 8: 129.6, 116.7.)
+template <int kNodes>
+struct FirstNodes {
+    int f[kNodes], l[kNodes];  // this lane's (l < f: none)
+    int n, splits;
+    bool left[kNodes], right[kNodes];  // candidates: first half, second half
+    __device__ __forceinline__ FirstNodes(const Geom &g, int kq, int levels, int q_lim, int lane, int *room_f, int *room_l) {
+        const unsigned lt = (1u << lane) - 1u;
+        unsigned ballots[2 * kNodes];
+#pragma unroll
+        for (int x = 0; x < kNodes; ++x) {
+            const int i = kNodes * lane + x;
+            f[x] = (int)(((long long)i * g.N_k) / kq);
+            l[x] = i < kq ? (int)(((long long)(i + 1) * g.N_k) / kq) - 1 : f[x] - 1;
+        }
+        n = kq;
+        for (splits = 0;; ++splits) {
+#pragma unroll
+            for (int x = 0; x < kNodes; ++x) {
+                const int m = (f[x] + l[x]) / 2;
+                left[x] = f[x] <= l[x] && f[x] <= q_lim;
+                right[x] = left[x] && m + 1 <= l[x] && m + 1 <= q_lim;
+                ballots[2 * x] = __ballot_sync(0xffffffffu, left[x]);
+                ballots[2 * x + 1] = __ballot_sync(0xffffffffu, right[x]);
+            }
+            const int total = flags_all(ballots);
+            if (total > kq || splits + 1 >= levels) return;
+            int place = flags_before(ballots, lt);
+            __syncwarp();
+#pragma unroll
+            for (int x = 0; x < kNodes; ++x) {
+                const int m = (f[x] + l[x]) / 2;
+                if (left[x]) { room_f[place] = f[x]; room_l[place++] = m; }
+                if (right[x]) { room_f[place] = m + 1; room_l[place++] = l[x]; }
+            }
+            __syncwarp();
+            n = total;
+#pragma unroll
+            for (int x = 0; x < kNodes; ++x) {
+                const int i = kNodes * lane + x;
+                f[x] = i < n ? room_f[i] : 0;
+                l[x] = i < n ? room_l[i] : -1;
+            }
+        }
+    }
+};
+
 // A CTA's n-th place in an order of items. Every second round runs backwards, so that with items in
 // order of falling length every CTA gets about the same sum.
 __device__ __forceinline__ int nth_item(int n) {

@@ -42,6 +42,13 @@ def test_masks_without_scores(S, kw):
     check(S, kw)
 
 
+# A row per token, 128 tokens a group: some groups, half of one, all of them kept whole; up to 16 nodes and more
+@pytest.mark.parametrize("T,k,H,G,causal", [(2100, 16, 2, 1, True), (2100, 17, 2, 1, True), (1500, 5, 2, 2, True), (1500, 23, 1, 1, True), (1500, 23, 1, 1, False),
+                                            (1500, 24, 1, 1, True), (3000, 11, 2, 1, True), (4200, 32, 1, 1, True), (4200, 1, 1, 1, True), (130, 1, 2, 1, True), (2000, 9, 1, 1, False)])
+def test_masks_of_tokens_without_scores(S, T, k, H, G, causal):
+    check(S, dict(T=T, k_top=k, n_q_heads=H, n_kv_heads=G, d=128, block=64, causal=causal), impl="tensor", block_q=1, block_k=64)
+
+
 @pytest.mark.parametrize("causal", [True, False])
 def test_rows_kept_whole_do_not_depend_on_the_numbers(S, causal):
     """Queries and keys of infinities and NaN: a row that keeps all it may keeps them whatever their scores."""
