@@ -517,8 +517,8 @@ size_t row_bytes(const Geom &g, int warps) {
 
 template <class P, int W, bool kCluster = false>
 stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, int32_t *mask, float *score, WorkspaceHeader *ws,
-                       cudaStream_t st, int n_cta = 1) {
-    const long long rows = (long long)g.batch * g.H * g.n_qb;
+                       cudaStream_t st, int first_qb, int n_cta = 1) {
+    const long long rows = (long long)g.batch * g.H * (g.n_qb - first_qb);
     const int n_max = (2 * g.k_top + 31) & ~31;
     const size_t score_bytes = P::smem_bytes(g, W);
     size_t smem = row_bytes<P>(g, W);
@@ -536,7 +536,17 @@ stream_status launch_w(const Geom &g, MultiK mk, const void *q, const void *k, i
 template <class P>
 stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void *k, int32_t *mask, float *score, WorkspaceHeader *ws,
                      cudaStream_t st) {
-    const long long rows = (long long)g.batch * g.H * g.n_qb;
+    // Rows that keep all blocks they are allowed, with no score asked for, are written by a kernel of their own (they are the last of
+    // the launch's order). Not where they are few, or where all rows run at once anyway: a launch more is 2 us (16 heads, T = 2000, fp32,
+    // blocks of 32, k = 24: 145 -> 135 us), and the
+    // row kernel does not bear a way out of its beginning (fp32, T = 5003: 178 -> 189 us by the compiler's other choices).
+    int first_qb = mk.n == 0 && score == nullptr ? whole_query_blocks(g) : 0;
+    if (first_qb < g.n_qb && (4 * first_qb < g.n_qb || (long long)g.batch * g.H * (g.n_qb - first_qb) < 4 * sm_count_or_default())) first_qb = 0;
+    if (first_qb > 0) {
+        const stream_status rc = launch_mask_whole(g, first_qb, mask, ws, st);
+        if (rc != STREAM_OK || first_qb == g.n_qb) return rc;
+    }
+    const long long rows = (long long)g.batch * g.H * (g.n_qb - first_qb);
     // Sixteen warps when every row has an SM to itself anyway: a level's tiles then spread over more
     // warps (64 rows, fp32, d = 64, blocks of 32, k = 8: 34.9 us with eight, 32.9 with sixteen, before the
     // divisions went; 28.9 now). With up to two rows an SM, too, if the first level has a tile part for
@@ -551,9 +561,9 @@ stream_status launch(const Geom &g, const MultiK &mk, const void *q, const void 
     while (n_cta < 8 && rows * 2 * n_cta <= sm_count_or_default() && parts >= 8 * n_cta) n_cta *= 2;
     // (d = 256 in fp32, blocks above 32 and k above 624: sixteen warps do not fit, four do)
     const bool fits = row_bytes<P>(g, kWideWarps) <= kMaxDynamicSmem;
-    if (fits && n_cta > 1 && mk.n <= 1) return launch_w<P, kWideWarps, true>(g, mk, q, k, mask, score, ws, st, n_cta);
-    if (fits && rows <= (parts >= kWideWarps ? 2 : 1) * (long long)sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st);
-    return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st);
+    if (fits && n_cta > 1 && mk.n <= 1) return launch_w<P, kWideWarps, true>(g, mk, q, k, mask, score, ws, st, first_qb, n_cta);
+    if (fits && rows <= (parts >= kWideWarps ? 2 : 1) * (long long)sm_count_or_default()) return launch_w<P, kWideWarps>(g, mk, q, k, mask, score, ws, st, first_qb);
+    return launch_w<P, P::kWarps>(g, mk, q, k, mask, score, ws, st, first_qb);
 }
 
 template <typename T, int RQ, Load kLoad>
@@ -593,20 +603,16 @@ stream_status mma_d(const Geom &g, const MultiK &mk, const void *q, const void *
 // No row has more allowed blocks than it may keep: every row is its allowed blocks, and no key is read. Bound by the launch (32
 // heads, 1000 tokens in blocks of 64, k = 16: 24.0 us with all scores computed, 13.1 a call in a loop, the host's part).
 constexpr int kWholeThreads = 256;
-__global__ void __launch_bounds__(kWholeThreads) mask_whole_kernel(Geom g, int32_t *mask, WorkspaceHeader *ws) {
+__global__ void __launch_bounds__(kWholeThreads) mask_whole_kernel(Geom g, int n_qb, int32_t *mask, WorkspaceHeader *ws) {
     after_previous_kernel();
-    unsigned long long tiles = write_whole_rows(g, g.n_qb, blockIdx.x * kWholeThreads + threadIdx.x, gridDim.x * kWholeThreads, mask);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tiles += __shfl_xor_sync(0xffffffffu, tiles, o);
-    if ((threadIdx.x & 31) == 0 && tiles > 0) atomicAdd(&ws->tiles_scored, tiles);
-    if (blockIdx.x == 0 && threadIdx.x == 0) ws->rows = (unsigned long long)g.batch * g.H * g.n_qb;
+    write_whole_rows(g, n_qb, (int)(blockIdx.x * kWholeThreads + threadIdx.x) / 32, (int)gridDim.x * (kWholeThreads / 32), (int)threadIdx.x & 31, mask, ws);
 }
 
 }  // namespace
 
-stream_status launch_mask_whole(const Geom &g, int32_t *mask, WorkspaceHeader *ws, cudaStream_t st) {
-    const long long rows = (long long)g.batch * g.H * g.n_qb, blocks = (rows * g.k_top + kWholeThreads - 1) / kWholeThreads, most = 8 * sm_count_or_default();
-    const cudaError_t e = launch_kernel(mask_whole_kernel, (unsigned)(blocks < most ? blocks : most), kWholeThreads, 0, st, 1, g, mask, ws);
+stream_status launch_mask_whole(const Geom &g, int n_qb, int32_t *mask, WorkspaceHeader *ws, cudaStream_t st) {
+    const long long blocks = (whole_pieces(g, n_qb) + kWholeThreads / 32 - 1) / (kWholeThreads / 32), most = 8 * sm_count_or_default();
+    const cudaError_t e = launch_kernel(mask_whole_kernel, (unsigned)(blocks < most ? blocks : most), kWholeThreads, 0, st, 1, g, n_qb, mask, ws);
     return e == cudaSuccess ? STREAM_OK : cuda_fail(e, "mask_whole launch");
 }
 

@@ -804,13 +804,6 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     // issuing role and two of the controllers', spread over all schedulers, cost a quarter of the
     // kernel's time in instruction fetches.
     if (warp >= 4 && warp < 12) {
-        if constexpr (!S::kMulti) {  // (they have nothing to reduce yet)
-            if (P.first_qb > 0) {
-                const unsigned long long tiles = write_whole_rows(P.g, P.first_qb, blockIdx.x * 256u + threadIdx.x - 128u, gridDim.x * 256u, P.mask);
-                if (tiles > 0) atomicAdd(&P.ws->tiles_scored, tiles);
-                if (blockIdx.x == 0 && threadIdx.x == 128) atomicAdd(&P.ws->rows, (unsigned long long)P.g.batch * P.g.H * P.first_qb);
-            }
-        }
         epilogue_role(P, tl, tmem_base, warp & 3, (warp - 4) >> 2, lane);
     } else if (warp == 1 || warp == 3 || warp == 13 || warp == 17) {
         mma_role(P, tl, q_smem, k_smem, tmem_base, warp == 1 ? 0 : (warp == 3 ? 1 : (warp == 13 ? 2 : 3)));
@@ -818,6 +811,11 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         producer_role(P, &tmap_k, tl, k_smem, warp == 2 ? 0 : 1);
     } else if (warp == 18) {
         dispatcher_role(P, &tmap_q, tl, q_smem, lane);
+        // the rows without products, beside the CTA's last group (at the beginning, by warps that the first group needs: 58.4 -> 59.1 us,
+        // 28 / 4 heads, 3000 tokens, k = 8)
+        if constexpr (!S::kMulti) {
+            if (P.first_qb > 0) write_whole_rows(P.g, P.first_qb, (int)blockIdx.x, (int)gridDim.x, lane, P.mask, P.ws);
+        }
     } else {
         controller_role(P, tl, warp == 0 ? 0 : (warp == 12 ? 1 : (warp == 16 ? 2 : 3)), lane);
     }
@@ -880,9 +878,9 @@ cudaError_t launch(int grid, cudaStream_t st, const CUtensorMap &tq, const CUten
 }
 
 template <int kD, int kBlk>
-cudaError_t launch_rows(const Geom &g, const Split &sp, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
-    if (g.k_top > 32) return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, true, false, true>>(sp.grid, st, tq, tk, P) : launch<Shape<kD, kBlk, true, false>>(sp.grid, st, tq, tk, P);
-    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, false, false, true>>(sp.grid, st, tq, tk, P) : launch<Shape<kD, kBlk, false, false>>(sp.grid, st, tq, tk, P);
+cudaError_t launch_rows(const Geom &g, const Split &sp, int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
+    if (g.k_top > 32) return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, true, false, true>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, true, false>>(grid, st, tq, tk, P);
+    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, false, false, true>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, false, false>>(grid, st, tq, tk, P);
 }
 }  // namespace
 
@@ -913,7 +911,7 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     P.g = g;
     // The rows of one build that keep every block they are allowed, with no score asked for, need no products.
     P.first_qb = mk.n == 0 && score == nullptr ? whole_query_blocks(g) : 0;
-    if (P.first_qb == g.n_qb) return launch_mask_whole(g, mask, ws, st);
+    if (P.first_qb == g.n_qb) return launch_mask_whole(g, g.n_qb, mask, ws, st);
     Split sp;
     rc = split_rows(g, P.first_qb, &sp);
     if (rc != STREAM_OK) return rc;
@@ -924,7 +922,9 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
         P.row_head |= (unsigned)(r % sp.head_rows) << (2 * r);
         P.row_back |= (unsigned)(r / sp.head_rows) << (2 * r);
     }
-    const int grid = sp.grid;
+    // (more CTAs than groups where they have rows to write)
+    const long long writers = P.first_qb > 0 ? whole_pieces(g, P.first_qb) / 4 : 0;
+    const int grid = writers > sp.grid ? (int)(writers < sm_count() ? writers : sm_count()) : sp.grid;
     P.mask = mask; P.score = score; P.ws = ws;
     // The largest k first: its nodes are the smallest, and where the numbers divide it meets all blocks that
     // the others would, in longer lists than theirs (8, 16, 32 at 32768 tokens: 2360 us, in rising order 2570).
@@ -944,8 +944,8 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     }
     if (mk.n >= 1 && score_memory == nullptr) { set_error("several k in one launch need the score memory"); return STREAM_ERR_WORKSPACE; }
     if (mk.n >= 1) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, true>>(grid, st, tq, tk, P);
-    else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64>(g, sp, st, tq, tk, P) : launch_rows<128, 32>(g, sp, st, tq, tk, P);
-    else e = g.bq == 64 ? launch_rows<64, 64>(g, sp, st, tq, tk, P) : launch_rows<64, 32>(g, sp, st, tq, tk, P);
+    else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64>(g, sp, grid, st, tq, tk, P) : launch_rows<128, 32>(g, sp, grid, st, tq, tk, P);
+    else e = g.bq == 64 ? launch_rows<64, 64>(g, sp, grid, st, tq, tk, P) : launch_rows<64, 32>(g, sp, grid, st, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tc launch");
     return STREAM_OK;
 }

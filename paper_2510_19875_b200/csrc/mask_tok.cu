@@ -167,8 +167,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     // Warps without a part in the levels write the tokens' rows that belong to no group, beside the first one.
     if (P.first_tb > 0 && (warp == 2 || warp >= 12)) {
-        tiles_needed += write_whole_rows(g, P.first_tb * kTok, blockIdx.x * 160u + (warp == 2 ? 0u : warp - 11u) * 32u + lane, gridDim.x * 160u, P.mask);
-        if (blockIdx.x == 0 && tid == 64) atomicAdd(&P.ws->rows, (unsigned long long)g.batch * g.H * P.first_tb * kTok);
+        write_whole_rows(g, P.first_tb * kTok, (int)blockIdx.x * 5 + (warp == 2 ? 0 : warp - 11), (int)gridDim.x * 5, lane, P.mask, P.ws);
     }
 
     for (;;) {
@@ -529,7 +528,7 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     P.g = g;
     // tokens that keep every block they are allowed, with no score asked for, need no products: whole groups of them have none
     const int whole = score == nullptr ? whole_query_blocks(g) : 0;
-    if (whole == g.n_qb) return launch_mask_whole(g, mask, ws, st);
+    if (whole == g.n_qb) return launch_mask_whole(g, g.n_qb, mask, ws, st);
     P.first_tb = whole / kTok;
     P.n_tb = (int)((g.T + kTok - 1) / kTok) - P.first_tb;
     const long long n_items = (long long)g.batch * g.H * P.n_tb;
@@ -540,7 +539,8 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     auto kern = g.k_top <= 16 ? mask_tok_kernel<16> : mask_tok_kernel<32>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tok)");
-    const int grid = (int)(n_items < n_sm ? n_items : n_sm);
+    const long long writers = P.first_tb > 0 ? (whole_pieces(g, P.first_tb * kTok) + 4) / 5 : 0, ctas = n_items > writers ? n_items : writers;
+    const int grid = (int)(ctas < n_sm ? ctas : n_sm);
     e = launch_kernel(kern, grid, kThreads, kSmemBytes, st, 1, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tok launch");
     return STREAM_OK;

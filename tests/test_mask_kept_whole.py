@@ -49,6 +49,16 @@ def test_masks_of_tokens_without_scores(S, T, k, H, G, causal):
     check(S, dict(T=T, k_top=k, n_q_heads=H, n_kv_heads=G, d=128, block=64, causal=causal), impl="tensor", block_q=1, block_k=64)
 
 
+# The kernels of all other shapes: fp32 and mma.sync, a row over a cluster, sixteen warps, four; one key block; block_q != block_k
+@pytest.mark.parametrize("T,k,H,G,d,bq,bk,dtype,causal", [
+    (900, 7, 1, 1, 64, 32, 32, "f32", True), (2048, 8, 1, 1, 64, 32, 32, "f32", True), (1500, 12, 2, 1, 32, 32, 32, "f32", True), (3000, 9, 4, 2, 64, 32, 32, "f32", True),
+    (3000, 24, 4, 1, 128, 16, 16, "f32", True), (1000, 40, 2, 2, 128, 16, 32, "f32", False), (1000, 20, 3, 1, 64, 24, 48, "f32", True), (500, 6, 2, 1, 64, 64, 16, "f32", True),
+    (30, 3, 2, 1, 64, 32, 32, "f32", True), (2500, 11, 4, 2, 256, 64, 64, "bf16", True), (2500, 70, 4, 2, 128, 16, 16, "bf16", True), (2500, 160, 4, 2, 128, 16, 16, "bf16", True),
+    (5000, 50, 8, 2, 256, 64, 64, "bf16", True), (3000, 24, 16, 4, 64, 32, 32, "f32", True)])
+def test_masks_of_other_shapes_without_scores(S, T, k, H, G, d, bq, bk, dtype, causal):
+    check(S, dict(T=T, k_top=k, n_q_heads=H, n_kv_heads=G, d=d, block=bk, causal=causal), dtype=dtype, block_q=bq, block_k=bk)
+
+
 @pytest.mark.parametrize("causal", [True, False])
 def test_rows_kept_whole_do_not_depend_on_the_numbers(S, causal):
     """Queries and keys of infinities and NaN: a row that keeps all it may keeps them whatever their scores."""
