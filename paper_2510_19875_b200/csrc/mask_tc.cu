@@ -514,16 +514,18 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
     int splits_of = 0;  // lane i: of the group's pass i
     unsigned ack_par = 1, q_par = (1u << kR) - 1u;  // (the first waits pass at once)
     unsigned long long fetched = 0;  // Q tiles asked of TMA
-    int next = -1;  // (lane 0) the next group's number, if it has been fetched
+    // (lane 0) the next group's number, if it has been fetched. The first one's is the CTA's own, the counter deals those behind.
+    int next = (int)blockIdx.x;
+    auto fetch = [&] { return (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u)); };
     for (;;) {
         // the previous list and record have been read by everybody
         if (!mbar_wait_w(smem_u32(&tl->jobs_ack[kR]), ack_par, tl, P.ws, 402)) return;
-        if (lane == 0 && next < 0) next = (int)atomicAdd(&P.ws->work_counter, 1u);
+        if (lane == 0 && next < 0) next = fetch();
         const int id = __shfl_sync(0xffffffffu, next, 0);
         const bool done = id >= P.n_groups || *(volatile int *)&tl->abort_flag;
         // the one after it a group ahead, unless that could leave another CTA without work
         next = -1;
-        if (lane == 0 && id + 2 * (int)gridDim.x < P.n_groups) next = (int)atomicAdd(&P.ws->work_counter, 1u);
+        if (lane == 0 && id + 2 * (int)gridDim.x < P.n_groups) next = fetch();
         int b = 0, kvh = 0, qb = 0, h0 = 0, R = 0;
         if (!done) {
             const int per = (g.n_qb - P.first_qb + P.qb_rows - 1) / P.qb_rows * P.n_chunks;

@@ -51,7 +51,7 @@ struct Tail {
     unsigned long long full[kStages], empty[kStages], tmem_full[kStages], tmem_empty[kStages], q_full;
     unsigned int tmem_base;
     int abort_flag;
-    int item;            // the group being worked on
+    int item;            // the next group
     int n_list;          // blocks in the current level's list
     int n_nodes[kTok];   // surviving nodes per token
     int n_tiles[kTok];   // tiles the token has needed so far (a warp's ranking keeps them here)
@@ -170,10 +170,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         write_whole_rows(g, P.first_tb * kTok, (int)blockIdx.x * 5 + (warp == 2 ? 0 : warp - 11), (int)gridDim.x * 5, lane, P.mask, P.ws);
     }
 
-    for (;;) {
-        if (tid == 0) tl->item = (int)atomicAdd(&P.ws->work_counter, 1u);
-        __syncthreads();
-        const int id = tl->item;
+    for (int id = (int)blockIdx.x;;) {  // (the first group is the CTA's own, the counter deals those behind)
         if (id >= P.n_items || *(volatile int *)&tl->abort_flag) break;
         // head by head (the keys of one kv head stay in L2), late token groups (most allowed blocks) first
         const int bh = id / P.n_tb, tb = P.first_tb + P.n_tb - 1 - id % P.n_tb;
@@ -214,6 +211,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const bool last = level + 1 == tl->n_levels;
             const int n_list = tl->n_list, n_st = (n_list + 1) >> 1;
 
+            if (warp == 13 && lane == 0 && level == 0) tl->item = (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
             if (is_producer) {
                 for (int i = 0; i < n_st; ++i) {
                     const unsigned s = seq + (unsigned)i, buf = s & 3u;
@@ -494,6 +492,8 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
         if (*(volatile int *)&tl->abort_flag) break;
         if (warp == 0 && lane == 0) atomicAdd(&P.ws->rows, (unsigned long long)(tq_max - tok0 + 1));
+        id = tl->item;
+        __syncthreads();
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tiles_needed += __shfl_xor_sync(0xffffffffu, tiles_needed, o);
