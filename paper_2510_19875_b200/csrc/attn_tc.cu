@@ -12,6 +12,14 @@
 // 1475 -> 1660 MHz in a long run, 128k tokens (32 / 8 heads, k = 32) 6560 -> 6330 us, four layers of
 // 9999 (k = 16) 935 -> 883, 4096 (k = 32) 166 -> 158.
 //
+// Where both rows name a block (`shared` entries: the two rows' lists are matched before they are walked, shared blocks first) its
+// K and V tiles are fetched once and serve both rows' products: at the power limit the bytes that an entry brings from L2 are as
+// good as clocks. Of a row's blocks the other head has 80 % at T = 4096, k = 32, 59 % at 16384, k = 16, 16 % at 131072, k = 32
+// (inputs with a sink and local windows or anchors): 144.3 -> 136.5, 406 -> 380, 6010 -> 5917 us; four layers of 9999 842 -> 824.
+// (d = 64, whose tiles are half as long, loses 1 % and is left. One product with M = 128 for both rows on top of it: Q has to lie in
+// TMEM for that, in the place of a second buffer of P, and the two shapes of product into O wait for one another or go
+// under lane masks: 126.5, 380, 5912, but 850 us for short lists that took 834.)
+//
 // Two softmax groups of four warps take a pair's entries in turn (its n-th kept entry belongs to
 // group n % 2, so that a pair's arithmetic does not depend on what the CTA did before), so
 // that one group's chain of waits, TMEM loads and exponentials runs beside the other's. A thread
@@ -71,6 +79,7 @@ struct Form {
     static constexpr int kD = kD_, kBlk = kBlk_, kHalves = kD / 64;
     static constexpr int kRows = 128 / kBlk, kStack = 64 / kBlk;  // rows of a unit; those stacked in one half of the lanes
     static constexpr bool kSplit = !(kD == 128 && kBlk == 64);
+    static constexpr bool kShare = kD == 128 && kBlk == 64;  // a block that both rows name is fetched once
     static constexpr int kPart = kBlk * 128;           // a row's block of one channel half
     static constexpr int kTile = kHalves * kHalfTile;  // 64 x d: the block of one row or those of two
     static constexpr int kOperand = 2 * kTile;         // two tiles: an entry's K or V, or the Q of a pair
@@ -118,7 +127,7 @@ struct Tail {
     unsigned long long m_full[kMaskSlots], m_empty[kMaskSlots];
     unsigned int tmem_base;
     int abort_flag;
-    int m_count[kMaskSlots];  // kept entries of the pair in each mask slot
+    int m_count[kMaskSlots], m_shared[kMaskSlots];  // entries of the pair in each mask slot; the first of them, whose block is both rows'
     Item<F> m_item[kMaskSlots];  // and the pair itself
     float ref[128], sum[2][128];
 };
@@ -216,7 +225,7 @@ template <class F>
 struct LoadStream {
     int round, id;     // pair being walked
     int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
-    int n = 0;         // kept entries of the pair
+    int n = 0, shared = 0;  // entries of the pair; those whose block is both rows'
     Entry<F> cur;
     int b, kvh;
     Ring ring, ms;
@@ -229,6 +238,7 @@ __device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStre
     S.b = tl->m_item[S.ms.idx].b;
     S.kvh = tl->m_item[S.ms.idx].kvh;
     S.n = tl->m_count[S.ms.idx];
+    S.shared = tl->m_shared[S.ms.idx];
     S.e = 0;
     if (S.n > 0) S.cur = entry_at<F>(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
     return true;
@@ -288,12 +298,13 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
         if (elect_one()) {
             // [half][row][keys][128 B]; a row without a block at an entry gets block 0, its logits are masked out
             const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * F::kOperand;
-            mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
+            const bool both = F::kShare && S.e < S.shared;  // (in row 0's place)
+            mbar_arrive_expect_tx(bar, (unsigned)(both ? F::kTile : F::kOperand));
 #pragma unroll
             for (int c = 0; c < F::kHalves; ++c)
 #pragma unroll
                 for (int r = 0; r < F::kRows; ++r)
-                    tma_load_4d(dst + c * 2 * kHalfTile + r * F::kPart, tk, bar, c * 64, max(S.cur.blk[r], 0) * F::kBlk, S.kvh, S.b);
+                    if (r == 0 || !both) tma_load_4d(dst + c * 2 * kHalfTile + r * F::kPart, tk, bar, c * 64, max(S.cur.blk[r], 0) * F::kBlk, S.kvh, S.b);
         }
         __syncwarp();
         S.ring.advance(P.n_k_stages);
@@ -334,6 +345,69 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
     }
 }
 
+// Is x among the ascending 32 kRegs values of a warp, value 32 r + i in register r of lane i?
+template <int kRegs>
+__device__ __forceinline__ bool among(const int (&v)[kRegs], int x) {
+    auto at = [&](int i) {
+        const int low = __shfl_sync(0xffffffffu, v[0], i & 31);
+        if (kRegs == 1) return low;
+        const int high = __shfl_sync(0xffffffffu, v[kRegs - 1], i & 31);  // (every lane takes part in both)
+        return i < 32 ? low : high;
+    };
+    int pos = 0;
+#pragma unroll
+    for (int step = 16 * kRegs; step > 0; step >>= 1) pos += at(pos + step - 1) < x ? step : 0;
+    return at(pos) == x;
+}
+
+// A pair's entries out of its rows' blocks, entry 32 x + lane in a[x], b[x] (negative: none): first those that both rows name, then the
+// rest of both side by side, -1 behind the shorter one. false: the rows are not ascending, as a mask build's are,
+// and nothing is written.
+template <int kRegs>
+__device__ __forceinline__ bool align_rows(const int (&a)[kRegs], const int (&b)[kRegs], int lane, int *to_a, int *to_b, int &count, int &shared) {
+    const unsigned lt = (1u << lane) - 1u;
+    int ka[kRegs], kb[kRegs];  // (none: behind all)
+    bool sorted = true;
+#pragma unroll
+    for (int x = 0; x < kRegs; ++x) { ka[x] = a[x] < 0 ? 0x7fffffff : a[x]; kb[x] = b[x] < 0 ? 0x7fffffff : b[x]; }
+#pragma unroll
+    for (int x = 0; x < kRegs; ++x) {
+        int na = __shfl_down_sync(0xffffffffu, ka[x], 1), nb = __shfl_down_sync(0xffffffffu, kb[x], 1);
+        if (kRegs > 1 && x + 1 < kRegs) {
+            const int ha = __shfl_sync(0xffffffffu, ka[kRegs - 1], 0), hb = __shfl_sync(0xffffffffu, kb[kRegs - 1], 0);
+            if (lane == 31) { na = ha; nb = hb; }
+        } else if (lane == 31) {
+            na = nb = 0x7fffffff;
+        }
+        sorted = sorted && (ka[x] < na || na == 0x7fffffff) && (kb[x] < nb || nb == 0x7fffffff);
+    }
+    // (the last clause: nothing follows an absent entry)
+    if (!__all_sync(0xffffffffu, sorted)) return false;
+    unsigned sa[kRegs], ua[kRegs], ub[kRegs];
+    int n_sa = 0, n_ua = 0, n_ub = 0;
+#pragma unroll
+    for (int x = 0; x < kRegs; ++x) {
+        const bool in_b = among(kb, ka[x]) && a[x] >= 0, in_a = among(ka, kb[x]) && b[x] >= 0;
+        sa[x] = __ballot_sync(0xffffffffu, in_b);
+        ua[x] = __ballot_sync(0xffffffffu, a[x] >= 0 && !in_b);
+        ub[x] = __ballot_sync(0xffffffffu, b[x] >= 0 && !in_a);
+        n_sa += __popc(sa[x]); n_ua += __popc(ua[x]); n_ub += __popc(ub[x]);
+    }
+    shared = n_sa;
+    count = n_sa + max(n_ua, n_ub);
+    int at_s = 0, at_a = n_sa, at_b = n_sa;
+#pragma unroll
+    for (int x = 0; x < kRegs; ++x) {
+        if ((sa[x] >> lane) & 1u) to_a[at_s + __popc(sa[x] & lt)] = to_b[at_s + __popc(sa[x] & lt)] = a[x];
+        if ((ua[x] >> lane) & 1u) to_a[at_a + __popc(ua[x] & lt)] = a[x];
+        if ((ub[x] >> lane) & 1u) to_b[at_b + __popc(ub[x] & lt)] = b[x];
+        at_s += __popc(sa[x]); at_a += __popc(ua[x]); at_b += __popc(ub[x]);
+    }
+    for (int i = at_a + lane; i < count; i += 32) to_a[i] = -1;
+    for (int i = at_b + lane; i < count; i += 32) to_b[i] = -1;
+    return true;
+}
+
 // The V tiles, and the pairs' mask rows up to two pairs ahead of everyone else: only the kept entries
 // of a pair (an entry is kept if either row has a block there) go to shared memory, in order, with
 // their number, so that the other roles index them instead of searching.
@@ -366,8 +440,20 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         }
         if (!probe_w(smem_u32(&tl->m_empty[mw.idx]), mw.phase ^ 1)) return false;
         int *dst = mask_rows(tl, P, mw.idx);
-        int cnt = 0;
-        for (int base = 0; base < g.k_top; base += 32) {
+        int cnt = 0, shared = 0;
+        bool done = false;
+        if constexpr (F::kShare) {
+            if (g.k_top <= 32) {
+                const int a[1] = {first[0]}, b[1] = {first[1]};
+                done = align_rows(a, b, lane, dst, dst + P.row_stride, cnt, shared);
+            } else if (g.k_top <= 64) {
+                int second[2];
+                fetch(lane + 32, second);
+                const int a[2] = {first[0], second[0]}, b[2] = {first[1], second[1]};
+                done = align_rows(a, b, lane, dst, dst + P.row_stride, cnt, shared);
+            }
+        }
+        for (int base = 0; base < g.k_top && !done; base += 32) {
             int blk[F::kRows];
             bool kept = false;
             if (base > 0) fetch(base + lane, blk);
@@ -387,6 +473,7 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         __syncwarp();
         if (lane == 0) {
             tl->m_count[mw.idx] = cnt;
+            tl->m_shared[mw.idx] = shared;
             tl->m_item[mw.idx] = it;
             mbar_arrive(smem_u32(&tl->m_full[mw.idx]));
         }
@@ -403,10 +490,11 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         if (!probe_w(smem_u32(&tl->v_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
         if (elect_one()) {  // [row][half][keys][128 B]
             const unsigned bar = smem_u32(&tl->v_full[S.ring.idx]), dst = v_smem + S.ring.idx * F::kOperand;
-            mbar_arrive_expect_tx(bar, (unsigned)F::kOperand);
+            const bool both = F::kShare && S.e < S.shared;
+            mbar_arrive_expect_tx(bar, (unsigned)(both ? F::kTile : F::kOperand));
 #pragma unroll
             for (int r = 0; r < F::kRows; ++r)
-                tma_load_5d(dst + r * F::kHalves * F::kPart, tv, bar, 0, max(S.cur.blk[r], 0) * F::kBlk, S.kvh, 0, S.b);
+                if (r == 0 || !both) tma_load_5d(dst + r * F::kHalves * F::kPart, tv, bar, 0, max(S.cur.blk[r], 0) * F::kBlk, S.kvh, 0, S.b);
         }
         __syncwarp();
         S.ring.advance(P.n_v_stages);
@@ -431,7 +519,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
     const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
     for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
-        const int n_entries = tl->m_count[ms.idx];  // the issuers need no more than the count
+        const int n_entries = tl->m_count[ms.idx], shared = tl->m_shared[ms.idx];  // the issuers need no more than the counts
         const unsigned q_lo = q_lo0 + qs.idx * (F::kOperand >> 4);
         if (n_entries > 0) {
             if (!wait_w(smem_u32(&tl->q_full[qs.idx]), qs.phase, tl, 201)) return;
@@ -442,7 +530,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
             if (!wait_both_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, 202, smem_u32(&tl->s_free[gi][use & 1u]), ((use >> 1) & 1u) ^ 1u, 203, tl)) return;
             tc_fence_after();
             const unsigned d_tmem = tmem_base + gi * 128 + (use & 1u) * 64;
-            const unsigned b_lo = k_lo + ks.idx * (F::kOperand >> 4);
+            const unsigned b_lo = k_lo + ks.idx * (F::kOperand >> 4), row_1 = F::kShare && i < shared ? 0u : (unsigned)kHalfTile >> 4;
             if (elect_one()) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
@@ -451,7 +539,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4)
                             tc_mma_bf16_split(d_tmem + r * kRowLanes, q_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK,
-                                              b_lo + (((2 * c + r) * kHalfTile + k4 * 32) >> 4), kHiK, F::kIdescQK, (c | k4) != 0);
+                                              b_lo + r * row_1 + ((2 * c * kHalfTile + k4 * 32) >> 4), kHiK, F::kIdescQK, (c | k4) != 0);
                 tc_commit(smem_u32(&tl->s_full[gi][use & 1u]));
                 if (!F::kKByLogits) tc_commit(smem_u32(&tl->k_empty[ks.idx]));
             }
@@ -475,7 +563,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
     const unsigned v_lo = desc_lo_sw128(v_smem, F::kPart), d_tmem = tmem_base + F::kOCol;
     for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
-        const int n_entries = tl->m_count[ms.idx];
+        const int n_entries = tl->m_count[ms.idx], shared = tl->m_shared[ms.idx];
         for (int i = 0; i < n_entries; ++i) {
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use % F::kPBufs;
             // (P is there: also, O is rescaled if it had to be)
@@ -485,7 +573,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
                 free_par ^= 1;
             }
             tc_fence_after();
-            const unsigned a_tmem = tmem_base + F::kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (F::kOperand >> 4);
+            const unsigned a_tmem = tmem_base + F::kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (F::kOperand >> 4), row_1 = F::kShare && i < shared ? 0u : (unsigned)F::kTile >> 4;
             if (elect_one()) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)  // row r of the pair: its P (or the parts of it), its V tile
@@ -494,7 +582,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
 #pragma unroll
                         for (int s4 = 0; s4 < 4; ++s4)  // 16 keys per step: 8 columns of packed bf16
                             tc_mma_bf16_ta(d_tmem + r * kRowLanes, a_tmem + r * kRowLanes + part * 32 + s4 * 8,
-                                           b_lo + ((r * F::kTile + s4 / (F::kBlk / 16) * F::kHalves * F::kPart + s4 % (F::kBlk / 16) * 2048) >> 4), kHiK, F::kIdescPV, (i | part | s4) != 0);
+                                           b_lo + r * row_1 + ((s4 / (F::kBlk / 16) * F::kHalves * F::kPart + s4 % (F::kBlk / 16) * 2048) >> 4), kHiK, F::kIdescPV, (i | part | s4) != 0);
                 tc_commit(smem_u32(&tl->p_free[gi][pb]));
                 tc_commit(smem_u32(&tl->v_empty[vs.idx]));
                 if (i + 1 == n_entries) tc_commit(smem_u32(&tl->o_done));
