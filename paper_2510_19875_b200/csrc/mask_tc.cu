@@ -142,6 +142,7 @@ constexpr unsigned kIdescTwo = idesc_bf16(128, 2 * S::kBlk, false);
 struct Params {
     Geom g;
     int n_groups, n_chunks;
+    int walked_heads;  // kv heads (of the batch * G) whose groups are walked together
     int first_qb;  // the rows of the query blocks before it keep all they are allowed, and belong to no group
     // A group's rows: head_rows query heads, at each of qb_rows query blocks (more than one only where
     // all heads of the kv head are in the group): row r is head r % head_rows at the group's query
@@ -528,11 +529,13 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
         if (lane == 0 && id + 2 * (int)gridDim.x < P.n_groups) next = fetch();
         int b = 0, kvh = 0, qb = 0, h0 = 0, R = 0;
         if (!done) {
-            const int per = (g.n_qb - P.first_qb + P.qb_rows - 1) / P.qb_rows * P.n_chunks;
-            const int bkv = id / per, rem = id % per;
+            // late (expensive) query blocks of all the heads walked together first
+            const int levels = (g.n_qb - P.first_qb + P.qb_rows - 1) / P.qb_rows, per = P.walked_heads * levels * P.n_chunks;
+            const int walk = id / per, rem = id - walk * per, heads = min(P.walked_heads, g.batch * g.G - walk * P.walked_heads);
+            const int level = rem / (heads * P.n_chunks), at = rem - level * heads * P.n_chunks, head = at / P.n_chunks, chunk = at - head * P.n_chunks;
+            const int bkv = walk * P.walked_heads + head;
             b = bkv / g.G; kvh = bkv % g.G;
-            qb = g.n_qb - 1 - rem / P.n_chunks * P.qb_rows;  // late (expensive) query blocks first
-            const int chunk = rem % P.n_chunks;
+            qb = g.n_qb - 1 - level * P.qb_rows;
             h0 = kvh * g.hpg + chunk * P.head_rows;
             R = min(P.head_rows, g.hpg - chunk * P.head_rows) * min(P.qb_rows, qb - P.first_qb + 1);
         }
@@ -918,6 +921,7 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     rc = split_rows(g, P.first_qb, &sp);
     if (rc != STREAM_OK) return rc;
     P.n_groups = (int)sp.n_groups;
+    P.walked_heads = walked_heads(g);
     P.n_chunks = sp.n_chunks; P.head_rows = sp.head_rows; P.qb_rows = sp.qb_rows;
     P.row_head = P.row_back = 0;
     for (int r = 0; r < sp.head_rows * sp.qb_rows; ++r) {

@@ -81,6 +81,7 @@ constexpr unsigned kNoBlock = 0xffffu;  // (behind every block)
 struct Params {
     Geom g;
     int n_items, n_tb;   // groups; groups per head (ceil(T / 128)), but for
+    int walked_heads;    // heads (of the batch * H) whose groups are walked together
     int first_tb;        // those before this one, whose tokens keep all blocks they are allowed
     int32_t *mask;
     float *score;
@@ -172,8 +173,9 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     for (int id = (int)blockIdx.x;;) {  // (the first group is the CTA's own, the counter deals those behind)
         if (id >= P.n_items || *(volatile int *)&tl->abort_flag) break;
-        // head by head (the keys of one kv head stay in L2), late token groups (most allowed blocks) first
-        const int bh = id / P.n_tb, tb = P.first_tb + P.n_tb - 1 - id % P.n_tb;
+        // late token groups (most allowed blocks) of all the heads walked together first
+        const int per = P.walked_heads * P.n_tb, walk = id / per, rem = id - walk * per, heads = min(P.walked_heads, g.batch * g.H - walk * P.walked_heads);
+        const int level = rem / heads, bh = walk * P.walked_heads + rem - level * heads, tb = P.first_tb + P.n_tb - 1 - level;
         const int b = bh / g.H, h = bh % g.H, kvh = h / g.hpg;
         const long long tok0 = (long long)tb * kTok;
         const long long tq_max = min(tok0 + kTok - 1, g.T - 1);
@@ -533,6 +535,7 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     P.n_tb = (int)((g.T + kTok - 1) / kTok) - P.first_tb;
     const long long n_items = (long long)g.batch * g.H * P.n_tb;
     P.n_items = (int)n_items;
+    P.walked_heads = walked_heads(g) * g.hpg;
     P.mask = mask; P.score = score; P.ws = ws;
     const int n_sm = sm_count();
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }

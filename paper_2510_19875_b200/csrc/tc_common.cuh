@@ -615,6 +615,17 @@ inline bool tma_strides_ok(const Geom &g) {
     return ok(g.qs_t) && ok(g.qs_h) && ok(g.qs_b) && ok(g.ks_t) && ok(g.ks_h) && ok(g.ks_b);
 }
 
+// kv heads whose groups a mask kernel walks together: as many as have their keys in 32 MB of L2 (there are 126 MB; queries stream by).
+// One head after the other, the last one's long groups began when most CTAs were about to finish (us: 28 / 4 heads, 1500 tokens, k = 5:
+// 36.1 -> 29.2; 12 / 2 heads, 5000 tokens in blocks of 32, k = 8: 60.7 -> 55.3; three k at 5000 tokens, 28 / 4 heads: 179.6 -> 144.5,
+// at 12845, 12 / 2 heads: 288 -> 240; three layers of 11851, 8 / 2 heads, k = 21: 303 -> 271; per token, 32 / 8 heads, 4096 tokens,
+// k = 16: 119.5 -> 108.6. With 32 / 8 heads and 16000 tokens or more it makes no difference, but for three k at 16000: 879 -> 892. Half
+// or a quarter of the 32 MB gives the middle sizes' gain away: 271 -> 299).
+inline int walked_heads(const Geom &g) {
+    const long long fit = (32ll << 20) / (g.T * g.d * 2), all = (long long)g.batch * g.G;
+    return (int)(fit < 1 ? 1 : (fit > all ? all : fit));
+}
+
 inline int sm_count() {
     static int n_sm = 0;
     if (n_sm == 0) {
