@@ -873,7 +873,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
         tl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc_512(smem_u32(&tl->tmem_base));  // all columns: one CTA per SM
+    if (warp == 1) tmem_alloc(smem_u32(&tl->tmem_base));  // all columns: one CTA per SM
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

@@ -567,7 +567,7 @@ attn_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x < kTok) tl->ref[threadIdx.x] = -CUDART_INF_F;
-    if (warp == 1) tmem_alloc_512(smem_u32(&tl->tmem_base));
+    if (warp == 1) tmem_alloc(smem_u32(&tl->tmem_base));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

@@ -30,7 +30,7 @@
 // busy 70 to 76 % of the clocks; beside them the way of a stage (a third of it transfer) and the
 // serial round of a row's level, list to ranked list, about 3500 clocks.
 //
-// Roles (608 threads): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
+// Roles (608 threads; builds of two CTAs an SM have 384, one producer, two issuers and one epilogue group): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
 // 3, 13, 17 MMA issuers (warp 1 owns TMEM), warp 18 dispatcher (groups, first lists, Q tiles), warps 0,
 // 12, 16, 15 the controllers of rows 0..3, warps 4..7 and 8..11 the two epilogue groups (TMEM lane
 // quarter = warp % 4). All roles walk the same fixed unit order (level 1: stage-major, row-minor;
@@ -46,21 +46,24 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 608;
-constexpr int kEpiGroups = 2;  // group g reduces the chains that land in slot g of their issuing warp
-constexpr int kMmaWarps = 4;   // they take the stages in turn
 constexpr int kR = 4;          // rows (query heads) per group
-constexpr int kSlots = 8;      // TMEM accumulator slots, one query block of fp32 columns each
 constexpr int kStageKeys = 128;
 constexpr int kFinal = 1 << 16;  // (several k) added to the length of a row's last list
-constexpr int kProducers = 2;     // producer p fills the stage buffers b with b % 2 == p
-constexpr int kListReaders = kProducers + kMmaWarps + 4 * kEpiGroups;  // producer, MMA and epilogue warps; of a first list and the group record also the controllers
 
 // What a build of the kernel is for: head dimension, block size, two nodes a lane (k_top up to 64) or one
-// (up to 32), several k with the score memory, rows of several query blocks in a group.
-template <int kD_, int kBlk_, bool kWide_, bool kMulti_, bool kQbRows_ = false>
+// (up to 32), several k with the score memory, rows of several query blocks in a group, two CTAs an SM (where Q and key tiles
+// are small enough).
+template <int kD_, int kBlk_, bool kWide_, bool kMulti_, bool kQbRows_ = false, bool kTwo_ = false>
 struct Shape {
     static constexpr int kD = kD_, kBlk = kBlk_;
+    static constexpr bool kTwo = kTwo_;
+    static constexpr int kThreads = kTwo ? 384 : 608;
+    static constexpr int kEpiGroups = kTwo ? 1 : 2;  // two: group g reduces the chains that land in slot g of their issuing warp; one: all
+    static constexpr int kMmaWarps = kTwo ? 2 : 4;   // they take the stages in turn
+    static constexpr int kProducers = kTwo ? 1 : 2;  // producer p fills the stage buffers b with b % kProducers == p
+    static constexpr int kSlots = 2 * kMmaWarps;     // TMEM accumulator slots, one query block of fp32 columns each: two private ones per issuing warp
+    static constexpr int kTmemColumns = kTwo ? kSlots * kBlk_ : 512;
+    static constexpr int kListReaders = kProducers + kMmaWarps + 4 * kEpiGroups;  // producer, MMA and epilogue warps; of a first list and the group record also the controllers
     static constexpr bool kMulti = kMulti_, kQbRows = kQbRows_;
     static constexpr int kMaskRows = kQbRows ? kR / kEpiGroups : 1;  // of the rows an epilogue group has of a list, those with masks of their own
     static constexpr int kHalves = kD / 64;                 // 64-channel halves (128 bytes a row)
@@ -69,7 +72,7 @@ struct Shape {
     static constexpr int kTile = kBlk * 128;                // a tile's part of one half
     static constexpr int kStageHalf = kStageKeys * 128;
     static constexpr int kStageBytes = kHalves * kStageHalf;
-    static constexpr int kStages = 128 * 1024 / kStageBytes;  // 128 KB of keys on their way
+    static constexpr int kStages = (kTwo ? 64 : 128) * 1024 / kStageBytes;  // 128 KB of keys on their way to an SM
     static constexpr int kQBytes = kHalves * kR * kTile;    // [channel half][row]
     static constexpr int kNodes = kWide_ ? 2 : 1;           // nodes a lane of a controller holds
     static constexpr int kMaxJobs = 64 * kNodes;            // first list: two candidates per node
@@ -81,13 +84,12 @@ struct Shape {
     // to warp s % kMmaWarps and lands in buffer s % kStages, and a warp's chains alternate between its
     // own two slots. The other issuing warps touch none of its barriers.
     static_assert(kStages % kMmaWarps == 0, "a stage buffer must always meet the same issuing warp");
-    static_assert(kSlots == 2 * kMmaWarps, "two private TMEM slots per issuing warp");
 };
 
 template <class S>
 struct Tail {
     unsigned long long full[S::kHalves][S::kStages];  // by channel half
-    unsigned long long empty[S::kStages], tmem_full[kSlots], tmem_empty[kSlots];
+    unsigned long long empty[S::kStages], tmem_full[S::kSlots], tmem_empty[S::kSlots];
     // Per row: its Q tile is there; the last products of a group with it are complete (one commit of
     // every issuing warp).
     unsigned long long q_full[kR], q_free[kR];
@@ -116,7 +118,7 @@ struct Tail {
     int first_blk[S::kMaxJobs], jobs_blk[kR][S::kMaxRowJobs];
     float first_part[2][kR][S::kMaxJobs][S::kParts], part[kR][S::kMaxRowJobs][S::kParts];
     float no_part;   // (written before a list's first tile, not read)
-    alignas(16) unsigned keys[kR][S::kNodes == 1 ? 64 : 4];  // a row's candidates while it ranks them
+    alignas(16) unsigned keys[kR][S::kNodes == 1 ? 64 : 1];  // a row's candidates while it ranks them
     int node_f[kR][32 * S::kNodes], node_l[kR][32 * S::kNodes];
     float node_s[kR][32 * S::kNodes];
 };
@@ -200,7 +202,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
                 if (S::kMulti && n >= kFinal) { n -= kFinal; open &= ~(1u << x); }
                 const int *const list = level == 0 ? tl->first_blk : tl->jobs_blk[x];
                 for (int j = 0; j < n; j += S::kTps) {
-                    if ((st.idx & (kProducers - 1)) != which) { st.advance(S::kStages); continue; }  // the other producer's buffer
+                    if ((st.idx & (S::kProducers - 1)) != which) { st.advance(S::kStages); continue; }  // the other producer's buffer
                     bool there[S::kTps];
                     int blk[S::kTps];
                     unsigned tiles = 0;
@@ -250,8 +252,9 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
 // other's chains: on the first level chain r of a stage goes to slot r % 2, later (one chain per
 // stage) the chain of stage s goes to slot (s / kMmaWarps) % 2. Both sides keep one phase bit per
 // slot they use.
+template <class S>
 __device__ __forceinline__ int chain_slot(int level, int r, unsigned stage) {
-    return level == 0 ? (r & 1) : (int)((stage / kMmaWarps) & 1u);
+    return level == 0 ? (r & 1) : (int)((stage / S::kMmaWarps) & 1u);
 }
 
 template <class S>
@@ -289,12 +292,12 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
                 const int r0 = level == 0 ? 0 : x, r1 = level == 0 ? R : x + 1;
                 const unsigned s_end = stage_seq + n_st;
                 // this warp's stages of the list: s = which (mod kMmaWarps)
-                for (unsigned s = stage_seq + (((unsigned)which - stage_seq) & (kMmaWarps - 1)); s < s_end; s += kMmaWarps) {
-                    const unsigned sidx = S::kStages == kMmaWarps ? (unsigned)which : s % S::kStages, a_lo = a_lo0 + sidx * (S::kStageBytes >> 4);
+                for (unsigned s = stage_seq + (((unsigned)which - stage_seq) & (S::kMmaWarps - 1)); s < s_end; s += S::kMmaWarps) {
+                    const unsigned sidx = S::kStages == S::kMmaWarps ? (unsigned)which : s % S::kStages, a_lo = a_lo0 + sidx * (S::kStageBytes >> 4);
                     for (int r = r0; r < r1; r += 2) {
                         // first level: rows r and r + 1 in one chain, each in its slot
                         const bool two = level == 0 && r + 1 < r1;
-                        const int sl = chain_slot(level, r, s);
+                        const int sl = chain_slot<S>(level, r, s);
                         const int slot = 2 * which + sl;
                         const unsigned rows = two ? 3u << r : 1u << r;
                         for (int i = r; (q_due & rows) != 0; ++i) {
@@ -361,13 +364,13 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
     const Geom &g = P.g;
     unsigned grp_par = 0, jr_par = 0;  // jr_par: bit by bit for the rows
     unsigned stage_seq = 0;
-    unsigned full_par = 0;  // bit w: phase of the next use of issuing warp w's slot `grp`
+    unsigned full_par = 0;  // bit 2 w + i: phase of the next use of issuing warp w's slot i
     constexpr int kBlk = S::kBlk;
     const int tile = wq / S::kParts;                       // which tile of the stage this warp's lanes hold
     const int key = (wq % S::kParts) * 32 + lane;          // key index inside the tile
-    // of this group's slot of issuing warp 0; the others' follow at 16 bytes (slot 2 * warp + grp)
-    const unsigned full_bar = smem_u32(&tl->tmem_full[grp]), empty_bar = smem_u32(&tl->tmem_empty[grp]);
-    const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16) + grp * kBlk;
+    constexpr int kMmaWarps = S::kMmaWarps, kEpiGroups = S::kEpiGroups;
+    const unsigned full_bar = smem_u32(&tl->tmem_full[0]), empty_bar = smem_u32(&tl->tmem_empty[0]);
+    const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16);
     const int whole_blocks = (int)(g.T / kBlk);
     for (;;) {
         if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 301)) return;
@@ -388,14 +391,17 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
         int my_blk[S::kListRegs];
         unsigned masked[S::kMaskRows][S::kListRegs];
         // One chain of this group: the list's stage i, the kernel's stage s, row r, the y-th, where the maximum goes.
-        auto reduce = [&](unsigned s, unsigned i, int r, int y, unsigned to) -> bool {
-            const unsigned owner = s & (kMmaWarps - 1);
-            if (!mbar_wait_w(full_bar + owner * 16, (full_par >> owner) & 1u, tl, P.ws, 303)) return false;
-            full_par ^= 1u << owner;
+        auto reduce = [&](unsigned s, unsigned i, int r, int y, unsigned slot, unsigned to) -> bool {
+            const unsigned at = 2 * (s & (kMmaWarps - 1)) + slot;
+            if (!mbar_wait_w(full_bar + at * 8, (full_par >> at) & 1u, tl, P.ws, 303)) return false;
+            full_par ^= 1u << at;
             tc_fence_after();
             float best = -CUDART_INF_F;
-            const unsigned taddr = t_lane + owner * (2 * kBlk);
-            const unsigned m0 = y ? masked[S::kMaskRows - 1][0] : masked[0][0], m1 = y ? masked[S::kMaskRows - 1][S::kListRegs - 1] : masked[0][S::kListRegs - 1];
+            const unsigned taddr = t_lane + at * kBlk;
+            unsigned m0 = masked[0][0], m1 = masked[0][S::kListRegs - 1];
+#pragma unroll
+            for (int z = 1; z < S::kMaskRows; ++z)
+                if (y == z) { m0 = masked[z][0]; m1 = masked[z][S::kListRegs - 1]; }
             const bool whole = (((S::kListRegs > 1 && i >= 32 ? m1 : m0) >> (i & 31)) & 1u) == 0;
             if (whole) {
                 unsigned v[kBlk];
@@ -405,7 +411,7 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                 tmem_ld_wait();
                 // the slot goes back as soon as it is in registers: its issuing warp waits for it
                 tc_fence_before();
-                mbar_arrive_if(empty_bar + owner * 16, lane == 0);
+                mbar_arrive_if(empty_bar + at * 8, lane == 0);
                 best = max_of<kBlk>(reinterpret_cast<const float *>(v));
             } else {
                 put();
@@ -425,7 +431,7 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                     }
                 }
                 tc_fence_before();
-                mbar_arrive_if(empty_bar + owner * 16, lane == 0);
+                mbar_arrive_if(empty_bar + at * 8, lane == 0);
             }
             last = best;
             last_to = to;
@@ -451,12 +457,12 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                     const int at = S::kTps * (32 * y + lane) + tile;
                     my_blk[y] = at < n ? list[at] : -1;
                 }
-                const int r0 = level == 0 ? grp : x, r1 = level == 0 ? R : x + 1;
+                const int r0 = level == 0 ? (kEpiGroups == 2 ? grp : 0) : x, r1 = level == 0 ? R : x + 1;
 #pragma unroll
                 for (int z = 0; z < S::kMaskRows; ++z) {
                     if (z > 0 && level > 0) continue;
                     // key blocks without a mask: those before `whole`, but for the diagonal one
-                    const int qb = qb_of(r0 + 2 * z), whole = qb < whole_blocks ? whole_blocks : 0, diag = g.causal ? qb : -1;
+                    const int qb = qb_of(r0 + kEpiGroups * z), whole = qb < whole_blocks ? whole_blocks : 0, diag = g.causal ? qb : -1;
 #pragma unroll
                     for (int y = 0; y < S::kListRegs; ++y)
                         masked[z][y] = __ballot_sync(0xffffffffu, my_blk[y] < 0 || my_blk[y] >= whole || my_blk[y] == diag);
@@ -473,11 +479,12 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
                 const unsigned part = smem_u32(level == 0 ? tl->first_part[set][0] : tl->part[x]) + wq * 4;  // (four warps: the kTps * kParts parts of a stage in order)
                 const unsigned row_step = level == 0 ? S::kMaxJobs * S::kParts * 4 : 0;
                 for (unsigned base = level == 0 ? stage_seq : stage_seq & ~(unsigned)(kMmaWarps - 1); base < s_end; base += kMmaWarps) {
-                    if (level > 0 && (int)((base / kMmaWarps) & 1u) != grp) continue;
+                    const unsigned later = (base / kMmaWarps) & 1u;  // the slot of a chain behind the first level
+                    if (kEpiGroups == 2 && level > 0 && (int)later != grp) continue;
                     const unsigned lo = max(base, stage_seq), hi = min(base + kMmaWarps, s_end);
-                    for (int r = r0; r < r1; r += 2)
+                    for (int r = r0; r < r1; r += kEpiGroups)
                         for (unsigned s = lo; s < hi; ++s)
-                            if (!reduce(s, s - stage_seq, r, S::kQbRows && r > r0, part + r * row_step + (s - stage_seq) * 16)) return;
+                            if (!reduce(s, s - stage_seq, r, S::kQbRows ? (r - r0) / kEpiGroups : 0, level == 0 ? (unsigned)r & 1u : later, part + r * row_step + (s - stage_seq) * 16)) return;
                 }
                 stage_seq = s_end;
                 put();
@@ -772,7 +779,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
 }
 
 template <class S>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(S::kThreads, S::kTwo ? 2 : 1)
 mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, Params P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = aligned_smem(smem_raw);
@@ -785,19 +792,17 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             for (int c = 0; c < S::kHalves; ++c) mbar_init(smem_u32(&tl->full[c][i]), 1);
             mbar_init(smem_u32(&tl->empty[i]), 1);
         }
-        for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&tl->tmem_full[i]), 1); mbar_init(smem_u32(&tl->tmem_empty[i]), 4); }
-        for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), kListReaders + (i == kR ? kR : 0)); }
+        for (int i = 0; i < S::kSlots; ++i) { mbar_init(smem_u32(&tl->tmem_full[i]), 1); mbar_init(smem_u32(&tl->tmem_empty[i]), 4); }
+        for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), S::kListReaders + (i == kR ? kR : 0)); }
         for (int i = 0; i < kR; ++i) {
-            mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), kMmaWarps);
-            mbar_init(smem_u32(&tl->first_done[0][i]), 4 * kEpiGroups); mbar_init(smem_u32(&tl->first_done[1][i]), 4 * kEpiGroups); mbar_init(smem_u32(&tl->scores_done[i]), 4 * kEpiGroups);
+            mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), S::kMmaWarps);
+            mbar_init(smem_u32(&tl->first_done[0][i]), 4 * S::kEpiGroups); mbar_init(smem_u32(&tl->first_done[1][i]), 4 * S::kEpiGroups); mbar_init(smem_u32(&tl->scores_done[i]), 4 * S::kEpiGroups);
         }
         tl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
-    if (warp == 1) {  // TMEM: all 512 columns (one CTA per SM)
-        tmem_alloc_512(smem_u32(&tl->tmem_base));
-    }
+    if (warp == 1) tmem_alloc<S::kTmemColumns>(smem_u32(&tl->tmem_base));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -808,13 +813,15 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     // that a scheduler (warp % 4) runs little beside its two epilogue warps: three copies of the
     // issuing role and two of the controllers', spread over all schedulers, cost a quarter of the
     // kernel's time in instruction fetches.
-    if (warp >= 4 && warp < 12) {
+    // (Two CTAs an SM: warp 0 producer, 1 and 2 issuers, 3 dispatcher, 4..7 epilogue, 8..11 controllers.)
+    constexpr bool kTwo = S::kTwo;
+    if (warp >= 4 && warp < (kTwo ? 8 : 12)) {
         epilogue_role(P, tl, tmem_base, warp & 3, (warp - 4) >> 2, lane);
-    } else if (warp == 1 || warp == 3 || warp == 13 || warp == 17) {
-        mma_role(P, tl, q_smem, k_smem, tmem_base, warp == 1 ? 0 : (warp == 3 ? 1 : (warp == 13 ? 2 : 3)));
-    } else if (warp == 2 || warp == 14) {
-        producer_role(P, &tmap_k, tl, k_smem, warp == 2 ? 0 : 1);
-    } else if (warp == 18) {
+    } else if (warp == 1 || warp == (kTwo ? 2 : 3) || (!kTwo && (warp == 13 || warp == 17))) {
+        mma_role(P, tl, q_smem, k_smem, tmem_base, warp == 1 ? 0 : (warp <= 3 ? 1 : (warp == 13 ? 2 : 3)));
+    } else if (warp == (kTwo ? 0 : 2) || (!kTwo && warp == 14)) {
+        producer_role(P, &tmap_k, tl, k_smem, warp <= 2 ? 0 : 1);
+    } else if (warp == (kTwo ? 3 : 18)) {
         dispatcher_role(P, &tmap_q, tl, q_smem, lane);
         // the rows without products, beside the CTA's last group (at the beginning, by warps that the first group needs: 58.4 -> 59.1 us,
         // 28 / 4 heads, 3000 tokens, k = 8)
@@ -822,11 +829,11 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             if (P.first_qb > 0) write_whole_rows(P.g, P.first_qb, (int)blockIdx.x, (int)gridDim.x, lane, P.mask, P.ws);
         }
     } else {
-        controller_role(P, tl, warp == 0 ? 0 : (warp == 12 ? 1 : (warp == 16 ? 2 : 3)), lane);
+        controller_role(P, tl, kTwo ? warp - 8 : (warp == 0 ? 0 : (warp == 12 ? 1 : (warp == 16 ? 2 : 3))), lane);
     }
     __syncwarp();
 
-    leave(&tl->abort_flag, tmem_base, warp == 1);
+    leave<S::kTmemColumns>(&tl->abort_flag, tmem_base, warp == 1);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -857,8 +864,8 @@ namespace {
 // own keys, 8192 tokens, d = 64, k = 40, not causal: a row a group 229 us, four 156), unless k changes
 // from one to the next.
 struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
-stream_status split_rows(const Geom &g, int first_qb, Split *s) {
-    const int n_sm = sm_count();
+stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, Split *s) {
+    const int n_sm = sm_count() * ctas_per_sm;
     if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
     s->n_chunks = (g.hpg + kR - 1) / kR;
     s->head_rows = (g.hpg + s->n_chunks - 1) / s->n_chunks;  // (six heads as 3 + 3, not 4 + 2: 139 -> 135 us at 10007 tokens in blocks of 32, 115 -> 107 at 8221)
@@ -875,23 +882,29 @@ stream_status split_rows(const Geom &g, int first_qb, Split *s) {
     return STREAM_OK;
 }
 
+// Two CTAs an SM for the shapes whose Q and key tiles leave room for it. With lists of a few stages every role of a lone CTA waits for the
+// others most of the time; two groups fill each other's gaps (us, one and two: 12 / 2 heads, 10007 tokens in blocks of 32,
+// k = 8: 114.9, 94.1; 6 / 2 heads, 20000, k = 16: 166, 147.5; d = 64: 32 / 8 heads, 4000 tokens, k = 16: 76.0, 65.6; 16 heads,
+// 8192 tokens, k = 40, not causal: 157.2, 150.6; 8 / 2 heads, 16000, k = 60, not causal: 260, 242).
+bool two_ctas(const Geom &g) { return g.d == 64 || g.bq == 32; }
+
 template <class S>
 cudaError_t launch(int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
-    static_assert(kSmemBytes<S> <= 232448, "one CTA's shared memory");
+    static_assert((S::kTwo ? 2 : 1) * (kSmemBytes<S> + 1024) <= 228 * 1024, "shared memory of an SM");
     const cudaError_t e = cudaFuncSetAttribute(mask_tc_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<S>);
-    return e == cudaSuccess ? launch_kernel(mask_tc_kernel<S>, grid, kThreads, kSmemBytes<S>, st, 1, tq, tk, P) : e;
+    return e == cudaSuccess ? launch_kernel(mask_tc_kernel<S>, grid, S::kThreads, kSmemBytes<S>, st, 1, tq, tk, P) : e;
 }
 
-template <int kD, int kBlk>
+template <int kD, int kBlk, bool kTwo>
 cudaError_t launch_rows(const Geom &g, const Split &sp, int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
-    if (g.k_top > 32) return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, true, false, true>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, true, false>>(grid, st, tq, tk, P);
-    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, false, false, true>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, false, false>>(grid, st, tq, tk, P);
+    if (g.k_top > 32) return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, true, false, true, kTwo>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, true, false, false, kTwo>>(grid, st, tq, tk, P);
+    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, false, false, true, kTwo>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, false, false, false, kTwo>>(grid, st, tq, tk, P);
 }
 }  // namespace
 
 size_t mask_tc_score_memory_bytes(const Geom &g) {
     Split sp;
-    if (split_rows(g, 0, &sp) != STREAM_OK) return 0;
+    if (split_rows(g, 0, 1, &sp) != STREAM_OK) return 0;
     return (size_t)sp.grid * kR * (size_t)g.N_k * sizeof(unsigned long long);
 }
 
@@ -918,7 +931,8 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     P.first_qb = mk.n == 0 && score == nullptr ? whole_query_blocks(g) : 0;
     if (P.first_qb == g.n_qb) return launch_mask_whole(g, g.n_qb, mask, ws, st);
     Split sp;
-    rc = split_rows(g, P.first_qb, &sp);
+    const int ctas = mk.n == 0 && two_ctas(g) ? 2 : 1;
+    rc = split_rows(g, P.first_qb, ctas, &sp);
     if (rc != STREAM_OK) return rc;
     P.n_groups = (int)sp.n_groups;
     P.walked_heads = walked_heads(g);
@@ -930,7 +944,7 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     }
     // (more CTAs than groups where they have rows to write)
     const long long writers = P.first_qb > 0 ? whole_pieces(g, P.first_qb) / 4 : 0;
-    const int grid = writers > sp.grid ? (int)(writers < sm_count() ? writers : sm_count()) : sp.grid;
+    const int grid = writers > sp.grid ? (int)(writers < ctas * sm_count() ? writers : ctas * sm_count()) : sp.grid;
     P.mask = mask; P.score = score; P.ws = ws;
     // The largest k first: its nodes are the smallest, and where the numbers divide it meets all blocks that
     // the others would, in longer lists than theirs (8, 16, 32 at 32768 tokens: 2360 us, in rising order 2570).
@@ -950,8 +964,8 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     }
     if (mk.n >= 1 && score_memory == nullptr) { set_error("several k in one launch need the score memory"); return STREAM_ERR_WORKSPACE; }
     if (mk.n >= 1) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, true>>(grid, st, tq, tk, P);
-    else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64>(g, sp, grid, st, tq, tk, P) : launch_rows<128, 32>(g, sp, grid, st, tq, tk, P);
-    else e = g.bq == 64 ? launch_rows<64, 64>(g, sp, grid, st, tq, tk, P) : launch_rows<64, 32>(g, sp, grid, st, tq, tk, P);
+    else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64, false>(g, sp, grid, st, tq, tk, P) : launch_rows<128, 32, true>(g, sp, grid, st, tq, tk, P);
+    else e = g.bq == 64 ? launch_rows<64, 64, true>(g, sp, grid, st, tq, tk, P) : launch_rows<64, 32, true>(g, sp, grid, st, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tc launch");
     return STREAM_OK;
 }

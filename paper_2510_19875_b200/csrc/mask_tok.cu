@@ -139,7 +139,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         fence_async_smem();
     }
     for (int i = tid; i < kMaxNk / 32; i += kThreads) bitmap[i] = 0u;
-    if (warp == 1) tmem_alloc_512(smem_u32(&tl->tmem_base));  // all 512 columns (one CTA per SM)
+    if (warp == 1) tmem_alloc(smem_u32(&tl->tmem_base));  // all 512 columns (one CTA per SM)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

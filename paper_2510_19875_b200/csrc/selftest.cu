@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(64) probe_rates_kernel(const unsigned char *sr
     }
     tc::fence_async_smem();
     __syncthreads();
-    if (mode == 1 && warp == 1) tc::tmem_alloc_512(tc::smem_u32(&tmem_slot));
+    if (mode == 1 && warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_slot));
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(64) probe_rates_kernel(const unsigned char *sr
     }
     if (mode == 1 && warp == 1) {
         tc::tc_fence_after();
-        tc::tmem_dealloc_512(tmem_slot);
+        tc::tmem_dealloc(tmem_slot);
     }
 }
 

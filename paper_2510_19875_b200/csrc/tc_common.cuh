@@ -198,12 +198,14 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
     return r;
 }
 
-__device__ __forceinline__ void tmem_alloc_512(unsigned smem_dst) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(512) : "memory");
+template <int kColumns = 512>
+__device__ __forceinline__ void tmem_alloc(unsigned smem_dst) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(kColumns) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tmem_dealloc_512(unsigned tmem_base) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+template <int kColumns = 512>
+__device__ __forceinline__ void tmem_dealloc(unsigned tmem_base) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kColumns) : "memory");
 }
 
 // 32 lanes x 32 consecutive fp32 columns of TMEM: thread i gets lane (base lane + i). Issue only;
@@ -526,6 +528,7 @@ constexpr long long kL2KvBytes = 64ll << 20;  // K and V bytes that stay in the 
 
 // The end of a kernel, of all its threads; `owner`: the warp that has allocated TMEM. After an abort, copies and
 // MMAs may still be in flight: they have a bounded time to land before shared memory and TMEM are given back.
+template <int kColumns = 512>
 __device__ __forceinline__ void leave(const int *abort_flag, unsigned tmem_base, bool owner) {
     if (*(const volatile int *)abort_flag) {
         const long long t0 = clock64();
@@ -535,7 +538,7 @@ __device__ __forceinline__ void leave(const int *abort_flag, unsigned tmem_base,
     __syncthreads();
     if (owner) {
         tc_fence_after();
-        tmem_dealloc_512(tmem_base);
+        tmem_dealloc<kColumns>(tmem_base);
     }
 }
 
