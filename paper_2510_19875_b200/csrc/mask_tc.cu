@@ -30,7 +30,7 @@
 // busy 70 to 76 % of the clocks; beside them the way of a stage (a third of it transfer) and the
 // serial round of a row's level, list to ranked list, about 3500 clocks.
 //
-// Roles (608 threads; builds of two CTAs an SM have 384, one producer, two issuers and one epilogue group): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
+// Roles (608 threads; builds of two CTAs an SM have 320 or 384, one producer, two issuers and one epilogue group): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
 // 3, 13, 17 MMA issuers (warp 1 owns TMEM), warp 18 dispatcher (groups, first lists, Q tiles), warps 0,
 // 12, 16, 15 the controllers of rows 0..3, warps 4..7 and 8..11 the two epilogue groups (TMEM lane
 // quarter = warp % 4). All roles walk the same fixed unit order (level 1: stage-major, row-minor;
@@ -46,7 +46,6 @@ namespace {
 
 using namespace tc;
 
-constexpr int kR = 4;          // rows (query heads) per group
 constexpr int kStageKeys = 128;
 constexpr int kFinal = 1 << 16;  // (several k) added to the length of a row's last list
 
@@ -55,9 +54,10 @@ constexpr int kFinal = 1 << 16;  // (several k) added to the length of a row's l
 // are small enough).
 template <int kD_, int kBlk_, bool kWide_, bool kMulti_, bool kQbRows_ = false, bool kTwo_ = false>
 struct Shape {
+    static constexpr int kR = kTwo_ && kD_ == 128 && kBlk_ == 64 ? 2 : 4;  // rows (query heads, or query blocks) of a group, at most
     static constexpr int kD = kD_, kBlk = kBlk_;
     static constexpr bool kTwo = kTwo_;
-    static constexpr int kThreads = kTwo ? 384 : 608;
+    static constexpr int kThreads = kTwo ? 256 + 32 * kR : 608;
     static constexpr int kEpiGroups = kTwo ? 1 : 2;  // two: group g reduces the chains that land in slot g of their issuing warp; one: all
     static constexpr int kMmaWarps = kTwo ? 2 : 4;   // they take the stages in turn
     static constexpr int kProducers = kTwo ? 1 : 2;  // producer p fills the stage buffers b with b % kProducers == p
@@ -92,18 +92,18 @@ struct Tail {
     unsigned long long empty[S::kStages], tmem_full[S::kSlots], tmem_empty[S::kSlots];
     // Per row: its Q tile is there; the last products of a group with it are complete (one commit of
     // every issuing warp).
-    unsigned long long q_full[kR], q_free[kR];
+    unsigned long long q_full[S::kR], q_free[S::kR];
     // Lists 0..kR-1: the rows' lists of the later levels; list kR: the first level's, with the group
     // record. The scores of the two kinds are kept and reported apart, those of the first level twice
     // (by the parity of the record): the next record's first level may be scored before a row's
     // controller has looked at this one's last, but the one after that is only published when
     // the controllers have read the next record, and are done with this one.
-    unsigned long long jobs_ready[kR + 1], first_done[2][kR], scores_done[kR];
+    unsigned long long jobs_ready[S::kR + 1], first_done[2][S::kR], scores_done[S::kR];
     // jobs_ack[i]: every reader of list i has taken what it needs from n_jobs[i], its blocks and, for
     // i = kR, the group record; who publishes the list waits for it before it writes them again.
     // Without it a warp with nothing to do in a short list could still be about to read it when the
     // next one is written, or fall two phases behind jobs_ready[i].
-    unsigned long long jobs_ack[kR + 1];
+    unsigned long long jobs_ack[S::kR + 1];
     unsigned int tmem_base;
     int abort_flag;
     int grp_id, grp_b, grp_kvh, grp_qb, grp_h0, grp_R;
@@ -114,13 +114,13 @@ struct Tail {
     unsigned grp_on[2 * S::kNodes];  // bit i of [2 x], [2 x + 1]: the left, right candidate of node kNodes i + x is on the first list
     int grp_new_q;   // 0: another pass over the same rows (several k), the Q tiles are already there
     int grp_last;    // the last pass over these rows: the Q tiles are given back
-    int n_jobs[kR + 1];
-    int first_blk[S::kMaxJobs], jobs_blk[kR][S::kMaxRowJobs];
-    float first_part[2][kR][S::kMaxJobs][S::kParts], part[kR][S::kMaxRowJobs][S::kParts];
+    int n_jobs[S::kR + 1];
+    int first_blk[S::kMaxJobs], jobs_blk[S::kR][S::kMaxRowJobs];
+    float first_part[2][S::kR][S::kMaxJobs][S::kParts], part[S::kR][S::kMaxRowJobs][S::kParts];
     float no_part;   // (written before a list's first tile, not read)
-    alignas(16) unsigned keys[kR][S::kNodes == 1 ? 64 : 1];  // a row's candidates while it ranks them
-    int node_f[kR][32 * S::kNodes], node_l[kR][32 * S::kNodes];
-    float node_s[kR][32 * S::kNodes];
+    alignas(16) unsigned keys[S::kR][S::kNodes == 1 ? 64 : 1];  // a row's candidates while it ranks them
+    int node_f[S::kR][32 * S::kNodes], node_l[S::kR][32 * S::kNodes];
+    float node_s[S::kR][32 * S::kNodes];
 };
 template <class S>
 constexpr int kSmemBytes = S::kQBytes + S::kStages * S::kStageBytes + (int)sizeof(Tail<S>) + 1024;
@@ -181,7 +181,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
     unsigned grp_par = 0, jr_par = 0;  // jr_par: bit by bit for the rows
     unsigned long long fetched = 0;  // tiles this warp has asked TMA for
     for (;;) {
-        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 101)) return;
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[S::kR]), grp_par, tl, P.ws, 101)) return;
         grp_par ^= 1;
         if (tl->grp_id < 0) {
             if (elect_one()) atomicAdd(&P.ws->tiles_fetched, fetched);
@@ -192,7 +192,7 @@ __device__ void producer_role(const Params &P, const CUtensorMap *tk, Tail<S> *t
         for (int level = 0; S::kMulti ? level == 0 || open != 0 : level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
-                const int li = level == 0 ? kR : x;
+                const int li = level == 0 ? S::kR : x;
                 if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), (jr_par >> x) & 1u, tl, P.ws, 102)) return;
@@ -266,7 +266,7 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
     const unsigned q_lo = desc_lo_sw128(q_smem, 16);
     const unsigned a_lo0 = desc_lo_sw128(k_smem, 16);
     for (;;) {
-        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 201)) return;
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[S::kR]), grp_par, tl, P.ws, 201)) return;
         grp_par ^= 1;
         if (tl->grp_id < 0) return;
         const int R = tl->grp_R, levels = tl->grp_levels;
@@ -276,7 +276,7 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
         for (int level = 0; S::kMulti ? level == 0 || open != 0 : level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
-                const int li = level == 0 ? kR : x;
+                const int li = level == 0 ? S::kR : x;
                 if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), (jr_par >> x) & 1u, tl, P.ws, 203)) return;
@@ -323,7 +323,7 @@ __device__ void mma_role(const Params &P, Tail<S> *tl, unsigned q_smem, unsigned
 #pragma unroll
                                 for (int k4 = 0; k4 < 4; ++k4)
                                     tc_mma_bf16_split(d_tmem, a_lo + ((c * S::kStageHalf + k4 * 32) >> 4), kDescHi,
-                                                      b_lo + ((c * kR * S::kTile + k4 * 32) >> 4), kDescHi, idesc, (c | k4) != 0);
+                                                      b_lo + ((c * S::kR * S::kTile + k4 * 32) >> 4), kDescHi, idesc, (c | k4) != 0);
                                 if (c + 1 == S::kHalves) {
                                     tc_commit(smem_u32(&tl->tmem_full[slot]));
                                     if (two) tc_commit(smem_u32(&tl->tmem_full[slot + 1]));
@@ -373,7 +373,7 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
     const unsigned t_lane = tmem_base + ((unsigned)(wq * 32) << 16);
     const int whole_blocks = (int)(g.T / kBlk);
     for (;;) {
-        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 301)) return;
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[S::kR]), grp_par, tl, P.ws, 301)) return;
         const unsigned set = grp_par;
         grp_par ^= 1;
         if (tl->grp_id < 0) return;
@@ -441,7 +441,7 @@ __device__ void epilogue_role(const Params &P, Tail<S> *tl, unsigned tmem_base, 
         for (int level = 0; S::kMulti ? level == 0 || open != 0 : level < levels; ++level) {
             const int lists = level == 0 ? 1 : R;
             for (int x = 0; x < lists; ++x) {
-                const int li = level == 0 ? kR : x;
+                const int li = level == 0 ? S::kR : x;
                 if (S::kMulti && level > 0 && !((open >> x) & 1u)) continue;
                 if (level > 0) {
                     if (!mbar_wait_w(smem_u32(&tl->jobs_ready[x]), (jr_par >> x) & 1u, tl, P.ws, 302)) return;
@@ -520,14 +520,14 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
     constexpr int kNodes = S::kNodes;
     const unsigned lt = (1u << lane) - 1u;
     int splits_of = 0;  // lane i: of the group's pass i
-    unsigned ack_par = 1, q_par = (1u << kR) - 1u;  // (the first waits pass at once)
+    unsigned ack_par = 1, q_par = (1u << S::kR) - 1u;  // (the first waits pass at once)
     unsigned long long fetched = 0;  // Q tiles asked of TMA
     // (lane 0) the next group's number, if it has been fetched. The first one's is the CTA's own, the counter deals those behind.
     int next = (int)blockIdx.x;
     auto fetch = [&] { return (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u)); };
     for (;;) {
         // the previous list and record have been read by everybody
-        if (!mbar_wait_w(smem_u32(&tl->jobs_ack[kR]), ack_par, tl, P.ws, 402)) return;
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ack[S::kR]), ack_par, tl, P.ws, 402)) return;
         if (lane == 0 && next < 0) next = fetch();
         const int id = __shfl_sync(0xffffffffu, next, 0);
         const bool done = id >= P.n_groups || *(volatile int *)&tl->abort_flag;
@@ -571,7 +571,7 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
 #pragma unroll
             for (int x = 0; x < 2 * kNodes; ++x) ballots[x] = __ballot_sync(0xffffffffu, on[x]);
             int place = flags_before(ballots, lt);
-            if (pass > 0 && !mbar_wait_w(smem_u32(&tl->jobs_ack[kR]), ack_par, tl, P.ws, 409)) return;
+            if (pass > 0 && !mbar_wait_w(smem_u32(&tl->jobs_ack[S::kR]), ack_par, tl, P.ws, 409)) return;
             ack_par ^= 1;
 #pragma unroll
             for (int x = 0; x < 2 * kNodes; ++x)
@@ -579,7 +579,7 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
 #pragma unroll
             for (int x = 0; x < kNodes; ++x) { tl->grp_f[kNodes * lane + x] = nodes.f[x]; tl->grp_l[kNodes * lane + x] = nodes.l[x]; }
             if (lane == 0) {
-                tl->n_jobs[kR] = flags_all(ballots);
+                tl->n_jobs[S::kR] = flags_all(ballots);
                 tl->grp_id = done ? -1 : id; tl->grp_b = b; tl->grp_kvh = kvh; tl->grp_qb = qb; tl->grp_h0 = h0; tl->grp_R = R;
                 tl->grp_levels = levels - nodes.splits;
                 tl->grp_k = kq; tl->grp_pass = pass; tl->grp_nodes = nodes.n;
@@ -589,7 +589,7 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
                 tl->grp_last = pass + 1 == n_pass;
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[kR]));
+            if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ready[S::kR]));
             if (done) {
                 if (lane == 0) atomicAdd(&P.ws->tiles_fetched, fetched);
                 return;
@@ -602,7 +602,7 @@ __device__ void dispatcher_role(const Params &P, const CUtensorMap *tq, Tail<S> 
                     const unsigned bar = smem_u32(&tl->q_full[r]);
                     mbar_arrive_expect_tx(bar, (unsigned)(S::kHalves * S::kTile));
 #pragma unroll
-                    for (int c = 0; c < S::kHalves; ++c) tma_load_4d(q_smem + (c * kR + r) * S::kTile, tq, bar, c * 64, (S::kQbRows ? qb - (int)((P.row_back >> (2 * r)) & 3u) : qb) * S::kBlk, h0 + (S::kQbRows ? (int)((P.row_head >> (2 * r)) & 3u) : r), b);
+                    for (int c = 0; c < S::kHalves; ++c) tma_load_4d(q_smem + (c * S::kR + r) * S::kTile, tq, bar, c * 64, (S::kQbRows ? qb - (int)((P.row_back >> (2 * r)) & 3u) : qb) * S::kBlk, h0 + (S::kQbRows ? (int)((P.row_head >> (2 * r)) & 3u) : r), b);
                 }
                 __syncwarp();
             }
@@ -620,7 +620,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
     const unsigned lt = (1u << lane) - 1u;
     unsigned grp_par = 0, first_par = 0, sd_par = 0, ack_par = 1;  // first_par: bit by bit for the two sets
     // this CTA's score memory for the row (several k only)
-    unsigned long long *const cache = kMulti ? P.cache + ((size_t)blockIdx.x * kR + r) * g.N_k : nullptr;
+    unsigned long long *const cache = kMulti ? P.cache + ((size_t)blockIdx.x * S::kR + r) * g.N_k : nullptr;
     auto remembered = [&](int blk, unsigned tag, float &score) {
         const unsigned long long e = __ldcg(cache + blk);
         if ((unsigned)(e >> 32) != tag) return false;
@@ -630,7 +630,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
     auto tile_max = [](const float (&parts)[S::kParts]) { return S::kParts == 2 ? fmaxf(parts[0], parts[S::kParts - 1]) : parts[0]; };
     unsigned long long tiles_all = 0, rows_all = 0;
     for (;;) {
-        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[kR]), grp_par, tl, P.ws, 407)) return;
+        if (!mbar_wait_w(smem_u32(&tl->jobs_ready[S::kR]), grp_par, tl, P.ws, 407)) return;
         const unsigned set = grp_par;
         grp_par ^= 1;
         const int id = tl->grp_id, b = tl->grp_b, qb = S::kQbRows ? tl->grp_qb - (int)((P.row_back >> (2 * r)) & 3u) : tl->grp_qb, h = tl->grp_h0 + (S::kQbRows ? (int)((P.row_head >> (2 * r)) & 3u) : r), R = tl->grp_R, levels = tl->grp_levels;
@@ -642,7 +642,7 @@ __device__ void controller_role(const Params &P, Tail<S> *tl, int r, int lane) {
 #pragma unroll
         for (int x = 0; x < kNodes; ++x) { nf[x] = tl->grp_f[kNodes * lane + x]; nl[x] = tl->grp_l[kNodes * lane + x]; }
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ack[kR]));  // (the list itself is not needed)
+        if (lane == 0) mbar_arrive(smem_u32(&tl->jobs_ack[S::kR]));  // (the list itself is not needed)
         if (id < 0) {
             if (lane == 0) {
                 atomicAdd(&P.ws->tiles_scored, tiles_all);
@@ -793,8 +793,8 @@ mask_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             mbar_init(smem_u32(&tl->empty[i]), 1);
         }
         for (int i = 0; i < S::kSlots; ++i) { mbar_init(smem_u32(&tl->tmem_full[i]), 1); mbar_init(smem_u32(&tl->tmem_empty[i]), 4); }
-        for (int i = 0; i <= kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), S::kListReaders + (i == kR ? kR : 0)); }
-        for (int i = 0; i < kR; ++i) {
+        for (int i = 0; i <= S::kR; ++i) { mbar_init(smem_u32(&tl->jobs_ready[i]), 1); mbar_init(smem_u32(&tl->jobs_ack[i]), S::kListReaders + (i == S::kR ? S::kR : 0)); }
+        for (int i = 0; i < S::kR; ++i) {
             mbar_init(smem_u32(&tl->q_full[i]), 1); mbar_init(smem_u32(&tl->q_free[i]), S::kMmaWarps);
             mbar_init(smem_u32(&tl->first_done[0][i]), 4 * S::kEpiGroups); mbar_init(smem_u32(&tl->first_done[1][i]), 4 * S::kEpiGroups); mbar_init(smem_u32(&tl->scores_done[i]), 4 * S::kEpiGroups);
         }
@@ -855,38 +855,54 @@ bool mask_tc_auto(const Geom &g, int dtype) {
 }
 
 namespace {
-// CTAs of a launch, the groups they share and the rows of a group: four rows where there are enough
-// groups, since they share the key tiles of the first level and its chains of two rows, else fewer.
-// Two groups a CTA are enough up to k = 32 (7 query heads per kv head, 3419 tokens, k = 27, not causal:
-// four rows 61 us, two 83), three beyond, where a group is a long piece of work (4 heads per kv head,
-// 10502 tokens, d = 64, k = 50: four rows 182 us, two 126; 2713 tokens, d = 128, k = 45: 67 and 54). With
-// fewer than four heads per kv head the rows are neighbouring query blocks' (16 heads, each its
-// own keys, 8192 tokens, d = 64, k = 40, not causal: a row a group 229 us, four 156), unless k changes
-// from one to the next.
-struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
-stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, Split *s) {
-    const int n_sm = sm_count() * ctas_per_sm;
-    if (n_sm <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
-    s->n_chunks = (g.hpg + kR - 1) / kR;
-    s->head_rows = (g.hpg + s->n_chunks - 1) / s->n_chunks;  // (six heads as 3 + 3, not 4 + 2: 139 -> 135 us at 10007 tokens in blocks of 32, 115 -> 107 at 8221)
-    s->qb_rows = g.k_row == nullptr ? kR / g.hpg : 1;
-    if (s->qb_rows < 1) s->qb_rows = 1;
-    for (;;) {
-        s->n_chunks = (g.hpg + s->head_rows - 1) / s->head_rows;
-        s->n_groups = (long long)g.batch * g.G * ((g.n_qb - first_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
-        if (s->n_groups >= (g.k_top > 32 ? 3 : 2) * n_sm || s->head_rows * s->qb_rows == 1) break;
-        if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
-        else s->head_rows = (s->head_rows + 1) / 2;
-    }
-    s->grid = (int)(s->n_groups < n_sm ? s->n_groups : n_sm);
-    return STREAM_OK;
-}
-
 // Two CTAs an SM for the shapes whose Q and key tiles leave room for it. With lists of a few stages every role of a lone CTA waits for the
 // others most of the time; two groups fill each other's gaps (us, one and two: 12 / 2 heads, 10007 tokens in blocks of 32,
 // k = 8: 114.9, 94.1; 6 / 2 heads, 20000, k = 16: 166, 147.5; d = 64: 32 / 8 heads, 4000 tokens, k = 16: 76.0, 65.6; 16 heads,
 // 8192 tokens, k = 40, not causal: 157.2, 150.6; 8 / 2 heads, 16000, k = 60, not causal: 260, 242).
-bool two_ctas(const Geom &g) { return g.d == 64 || g.bq == 32; }
+bool small_tiles(const Geom &g) { return g.d == 64 || g.bq == 32; }
+// With d = 128 and blocks of 64 there is room for two CTAs of two rows and two stages each: better with up to eight blocks a list and no more than
+// eight groups a CTA (32 / 8 heads, 2500 tokens, k = 8: 45.1 -> 36.9; 28 / 4 heads, 1500, k = 5: 29.8 -> 26.7; 12 / 2 heads, 20000,
+// k = 6, not causal: 189 -> 180), worse where the tensor cores are the limit (28 / 4 heads, 6000 tokens, k = 12, not causal: 139 -> 144;
+// 32 / 8 heads, 60000, k = 10: 2139 -> 2200; 16384, k = 16: 486 -> 521).
+bool two_of_two_rows(const Geom &g) {
+    return !small_tiles(g) && g.k_top <= 8 && g.k_row == nullptr && (long long)g.batch * g.H * g.n_qb <= 2 * 8 * 2ll * sm_count();
+}
+
+// CTAs of a launch, the groups they share and the rows of a group. Rows share the key tiles of the first level and its chains of two;
+// fewer of them make more and shorter groups. Four rows (of several query blocks, unless k changes from one to the next, where a kv head
+// has fewer than four heads) are taken where every CTA has some groups of them, else two, else one.
+struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
+stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_rows, Split *s) {
+    const int n_cta = sm_count() * ctas_per_sm;
+    if (n_cta <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
+    s->n_chunks = (g.hpg + most_rows - 1) / most_rows;
+    s->head_rows = (g.hpg + s->n_chunks - 1) / s->n_chunks;  // (six heads as 3 + 3, not 4 + 2: 139 -> 135 us at 10007 tokens in blocks of 32, 115 -> 107 at 8221)
+    s->qb_rows = g.k_row == nullptr ? most_rows / g.hpg : 1;
+    if (s->qb_rows < 1) s->qb_rows = 1;
+    for (;;) {
+        const int rows = s->head_rows * s->qb_rows;
+        s->n_chunks = (g.hpg + s->head_rows - 1) / s->head_rows;
+        s->n_groups = (long long)g.batch * g.G * ((g.n_qb - first_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
+        // Groups that a CTA should have, in halves. One CTA an SM, us with four, two rows and one: 28 / 4 heads, 3000 tokens, k = 8 (2.1
+        // groups a CTA of four rows): 59.5, 50.0, 60.7; 3419, k = 27, not causal (2.9): 83, 74, 101; 8 / 2 heads, 20000, k = 24 (3.9):
+        // 210, 195; 8 / 2 heads, 13232, k = 59 (2.0): 186, 157, 188; but of several query blocks: 16 heads, 9000, k = 12 (3.5): 118, 124.
+        // Two rows and one: 8 / 2 heads, 8000, k = 16 (2.9 of two): 51, 68; 12 / 2 heads, 8000 (4.4): 69, 98; 16 heads, 2000, k = 12 (1.1):
+        // 24.5, 28.7; 32 / 8 heads, 1200, k = 8 (1.2): 22.5, 24.2. Two CTAs, rows of one or two nodes a lane apart: 12 / 2 heads, 5000 in blocks
+        // of 32, k = 8 (2.0 of three): 49.2, 47.2; 28 / 4 heads, 4600, k = 24, not causal (3.9): 114, 126; d = 64, two and one: 32 / 8 heads,
+        // 4000, k = 16 (2.5): 65.6, 54.7; 16 heads, 6000, k = 12 (2.2): 57, 51; 8 / 2 heads, 9000, k = 20 (1.6): 76, 68; two nodes: 28 / 4 heads,
+        // 1074 in blocks of 32, k = 33 (1.8): 26.7, 32.8; 4000, k = 50 (2.0 of four): 82.3, 81.3.
+        const bool wide = g.k_top > 32;
+        int halves;
+        if (small_tiles(g)) halves = rows > 2 ? (wide ? 4 : 6) : (wide ? 3 : 6);
+        else halves = rows > 2 ? (s->qb_rows > 1 ? 4 : 8) : 2;
+        if (2 * s->n_groups >= (long long)halves * n_cta || rows == 1) break;
+        if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
+        else s->head_rows = (s->head_rows + 1) / 2;
+    }
+    s->grid = (int)(s->n_groups < n_cta ? s->n_groups : n_cta);
+    return STREAM_OK;
+}
+constexpr int kMultiRows = Shape<128, 64, false, true>::kR;
 
 template <class S>
 cudaError_t launch(int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
@@ -904,8 +920,8 @@ cudaError_t launch_rows(const Geom &g, const Split &sp, int grid, cudaStream_t s
 
 size_t mask_tc_score_memory_bytes(const Geom &g) {
     Split sp;
-    if (split_rows(g, 0, 1, &sp) != STREAM_OK) return 0;
-    return (size_t)sp.grid * kR * (size_t)g.N_k * sizeof(unsigned long long);
+    if (split_rows(g, 0, 1, kMultiRows, &sp) != STREAM_OK) return 0;
+    return (size_t)sp.grid * kMultiRows * (size_t)g.N_k * sizeof(unsigned long long);
 }
 
 stream_status launch_mask_tc(const Geom &g, const void *q, const void *k, int32_t *mask, float *score,
@@ -931,8 +947,9 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     P.first_qb = mk.n == 0 && score == nullptr ? whole_query_blocks(g) : 0;
     if (P.first_qb == g.n_qb) return launch_mask_whole(g, g.n_qb, mask, ws, st);
     Split sp;
-    const int ctas = mk.n == 0 && two_ctas(g) ? 2 : 1;
-    rc = split_rows(g, P.first_qb, ctas, &sp);
+    const bool two_rows = mk.n == 0 && two_of_two_rows(g);
+    const int ctas = (mk.n == 0 && small_tiles(g)) || two_rows ? 2 : 1;
+    rc = split_rows(g, P.first_qb, ctas, two_rows ? 2 : 4, &sp);
     if (rc != STREAM_OK) return rc;
     P.n_groups = (int)sp.n_groups;
     P.walked_heads = walked_heads(g);
@@ -964,6 +981,7 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     }
     if (mk.n >= 1 && score_memory == nullptr) { set_error("several k in one launch need the score memory"); return STREAM_ERR_WORKSPACE; }
     if (mk.n >= 1) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, true>>(grid, st, tq, tk, P);
+    else if (two_rows) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, false, false, true>>(grid, st, tq, tk, P);
     else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64, false>(g, sp, grid, st, tq, tk, P) : launch_rows<128, 32, true>(g, sp, grid, st, tq, tk, P);
     else e = g.bq == 64 ? launch_rows<64, 64, true>(g, sp, grid, st, tq, tk, P) : launch_rows<64, 32, true>(g, sp, grid, st, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tc launch");
