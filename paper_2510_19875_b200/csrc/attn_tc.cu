@@ -238,7 +238,7 @@ __device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStre
     S.b = tl->m_item[S.ms.idx].b;
     S.kvh = tl->m_item[S.ms.idx].kvh;
     S.n = tl->m_count[S.ms.idx];
-    S.shared = tl->m_shared[S.ms.idx];
+    if (F::kShare) S.shared = tl->m_shared[S.ms.idx];
     S.e = 0;
     if (S.n > 0) S.cur = entry_at<F>(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
     return true;
@@ -473,7 +473,7 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         __syncwarp();
         if (lane == 0) {
             tl->m_count[mw.idx] = cnt;
-            tl->m_shared[mw.idx] = shared;
+            if (F::kShare) tl->m_shared[mw.idx] = shared;
             tl->m_item[mw.idx] = it;
             mbar_arrive(smem_u32(&tl->m_full[mw.idx]));
         }
@@ -519,7 +519,7 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
     const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
     for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
-        const int n_entries = tl->m_count[ms.idx], shared = tl->m_shared[ms.idx];  // the issuers need no more than the counts
+        const int n_entries = tl->m_count[ms.idx], shared = F::kShare ? tl->m_shared[ms.idx] : 0;  // the issuers need no more than the counts
         const unsigned q_lo = q_lo0 + qs.idx * (F::kOperand >> 4);
         if (n_entries > 0) {
             if (!wait_w(smem_u32(&tl->q_full[qs.idx]), qs.phase, tl, 201)) return;
@@ -563,7 +563,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
     const unsigned v_lo = desc_lo_sw128(v_smem, F::kPart), d_tmem = tmem_base + F::kOCol;
     for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
-        const int n_entries = tl->m_count[ms.idx], shared = tl->m_shared[ms.idx];
+        const int n_entries = tl->m_count[ms.idx], shared = F::kShare ? tl->m_shared[ms.idx] : 0;
         for (int i = 0; i < n_entries; ++i) {
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use % F::kPBufs;
             // (P is there: also, O is rescaled if it had to be)

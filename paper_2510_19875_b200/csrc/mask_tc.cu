@@ -890,10 +890,11 @@ stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_
         // 24.5, 28.7; 32 / 8 heads, 1200, k = 8 (1.2): 22.5, 24.2. Two CTAs, rows of one or two nodes a lane apart: 12 / 2 heads, 5000 in blocks
         // of 32, k = 8 (2.0 of three): 49.2, 47.2; 28 / 4 heads, 4600, k = 24, not causal (3.9): 114, 126; d = 64, two and one: 32 / 8 heads,
         // 4000, k = 16 (2.5): 65.6, 54.7; 16 heads, 6000, k = 12 (2.2): 57, 51; 8 / 2 heads, 9000, k = 20 (1.6): 76, 68; two nodes: 28 / 4 heads,
-        // 1074 in blocks of 32, k = 33 (1.8): 26.7, 32.8; 4000, k = 50 (2.0 of four): 82.3, 81.3.
+        // 1074 in blocks of 32, k = 33 (1.8): 26.7, 32.8; four and two: 4000, k = 50 (2.0): 82.3, 81.3; d = 64, not causal, with the attention,
+        // which begins earlier behind fewer and longer groups: 8 / 2 heads, 16000, k = 60 (1.7): 548, 557; 16 heads, 8192, k = 40 (1.7): 358, 360.
         const bool wide = g.k_top > 32;
         int halves;
-        if (small_tiles(g)) halves = rows > 2 ? (wide ? 4 : 6) : (wide ? 3 : 6);
+        if (small_tiles(g)) halves = rows > 2 ? (wide ? 2 : 6) : (wide ? 3 : 6);
         else halves = rows > 2 ? (s->qb_rows > 1 ? 4 : 8) : 2;
         if (2 * s->n_groups >= (long long)halves * n_cta || rows == 1) break;
         if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
