@@ -1,8 +1,8 @@
 // Tensor-core Stream mask kernel for sm_100a: bf16, d = 64 or 128, blocks of 32 or 64, k_top <= 64.
 // (Figures: d = 128, blocks of 64, unless they say otherwise.)
 //
-// One persistent CTA per SM works through "groups": up to four rows of one kv head, its query heads at
-// one query block or, where these are few, at some. Their Q tiles stay in shared memory for the whole
+// One persistent CTA per SM (two smaller ones where small_tiles or two_of_two_rows says so) works through "groups": up to four rows
+// of one kv head, its query heads at one query block or, where these are few, at some. Their Q tiles stay in shared memory for the whole
 // hierarchy (Algorithm 2).
 // Candidate key blocks are fetched by TMA (128-byte swizzle), 128 keys at a time, into a ring of
 // stages; one tcgen05.mma chain per (stage, row) computes the keys (128 x d) x Q_row^T (d x block)
@@ -26,9 +26,9 @@
 // products of this one. (One warp doing all of it, and ranking all four rows, kept the issuing
 // warps waiting for a group or a list for 17 % (T = 16384, k = 16) to 29 % (several k) of the time.)
 //
-// What bounds it: the chip's power limit (1500 MHz at T = 131072, 1590 at 16384, of 1965) with the tensor cores
-// busy 70 to 76 % of the clocks; beside them the way of a stage (a third of it transfer) and the
-// serial round of a row's level, list to ranked list, about 3500 clocks.
+// What bounds it: the chip's power limit (1500 to 1570 MHz at T = 131072, 1590 at 16384, of 1965) with the tensor cores
+// busy 70 to 88 % of the clocks; beside them the way of a stage (a third of it transfer) and the
+// serial round of a row's level, list to ranked list, about 3500 clocks, which is what short lists wait for.
 //
 // Roles (608 threads; builds of two CTAs an SM have 320 or 384, one producer, two issuers and one epilogue group): warps 2 and 14 TMA producers of key tiles (even and odd stage buffers), warps 1,
 // 3, 13, 17 MMA issuers (warp 1 owns TMEM), warp 18 dispatcher (groups, first lists, Q tiles), warps 0,

@@ -26,7 +26,8 @@
 // sixteen warps, eight tokens each. The levels are separated by CTA-wide barriers; inside a level the
 // roles meet on mbarriers, every wait bounded as in the other tensor-core kernels.
 // Bound: the levels' serial parts (32 / 8 heads, T = 4096, k = 16: products 19 000 clocks a group of 128
-// tokens, ranking, lists and barriers 21 000 before the last change to both; 225 us at first, 148 now).
+// tokens, ranking, lists and barriers 21 000 before both were changed; 225 us at first, 148 then, 109 since levels that cannot drop
+// anything are passed over and the long groups of all heads come first).
 #include <math_constants.h>
 
 #include "tc_common.cuh"
