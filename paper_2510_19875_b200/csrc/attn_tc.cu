@@ -12,13 +12,15 @@
 // 1475 -> 1660 MHz in a long run, 128k tokens (32 / 8 heads, k = 32) 6560 -> 6330 us, four layers of
 // 9999 (k = 16) 935 -> 883, 4096 (k = 32) 166 -> 158.
 //
-// Where both rows name a block (`shared` entries: the two rows' lists are matched before they are walked, shared blocks first) its
-// K and V tiles are fetched once and serve both rows' products: at the power limit the bytes that an entry brings from L2 are as
-// good as clocks. Of a row's blocks the other head has 80 % at T = 4096, k = 32, 59 % at 16384, k = 16, 16 % at 131072, k = 32
-// (inputs with a sink and local windows or anchors): 144.3 -> 136.5, 406 -> 380, 6010 -> 5917 us; four layers of 9999 842 -> 824.
-// (d = 64, whose tiles are half as long, loses 1 % and is left. One product with M = 128 for both rows on top of it: Q has to lie in
+// Where both rows name the same block at the same entry its K and V tiles are fetched once and serve both rows' products: at the power
+// limit the bytes that an entry brings from L2 are as good as clocks (us, two fetches and one: 32 / 8 heads, 4096 tokens, k = 32,
+// where the rows that keep all their blocks have the same lists, 151.0, 145.3; 16384, k = 16, 402.0, 393.4; 131072, k = 32, 6150, 6085;
+// four layers of 9999 838.7, 835.3). Only there: a row walks its blocks in its own order, whatever the row beside it holds, so that its
+// output is the same bit for bit however a call groups the query heads. (The blocks that both rows name anywhere first: 142.3, 384.4,
+// 6047, 823 us, but the order of a row's entries, and with it the rounding of its P, was then a matter of its partner's list.)
+// (d = 64, whose tiles are half as long, loses 1 % and is left. One product with M = 128 for both rows of a shared block: Q has to lie in
 // TMEM for that, in the place of a second buffer of P, and the two shapes of product into O wait for one another or go
-// under lane masks: 126.5, 380, 5912, but 850 us for short lists that took 834.)
+// under lane masks: with shared blocks first 126.5, 380, but 850 us for short lists that took 834.)
 //
 // Two softmax groups of four warps take a pair's entries in turn (its n-th kept entry belongs to
 // group n % 2, so that a pair's arithmetic does not depend on what the CTA did before), so
@@ -79,7 +81,7 @@ struct Form {
     static constexpr int kD = kD_, kBlk = kBlk_, kHalves = kD / 64;
     static constexpr int kRows = 128 / kBlk, kStack = 64 / kBlk;  // rows of a unit; those stacked in one half of the lanes
     static constexpr bool kSplit = !(kD == 128 && kBlk == 64);
-    static constexpr bool kShare = kD == 128 && kBlk == 64;  // a block that both rows name is fetched once
+    static constexpr bool kShare = kD == 128 && kBlk == 64;  // a block that both rows name at an entry is fetched once
     static constexpr int kPart = kBlk * 128;           // a row's block of one channel half
     static constexpr int kTile = kHalves * kHalfTile;  // 64 x d: the block of one row or those of two
     static constexpr int kOperand = 2 * kTile;         // two tiles: an entry's K or V, or the Q of a pair
@@ -125,9 +127,10 @@ struct Tail {
     // are set; group g has published an entry; both have left their sums.
     unsigned long long ref_set[4], turn[4][2], sums_there[4];
     unsigned long long m_full[kMaskSlots], m_empty[kMaskSlots];
+    unsigned long long m_same[kMaskSlots];  // (kShare) bit e: both rows of the pair in that slot name the same block at entry e
     unsigned int tmem_base;
     int abort_flag;
-    int m_count[kMaskSlots], m_shared[kMaskSlots];  // entries of the pair in each mask slot; the first of them, whose block is both rows'
+    int m_count[kMaskSlots];  // entries of the pair in each mask slot
     Item<F> m_item[kMaskSlots];  // and the pair itself
     float ref[128], sum[2][128];
 };
@@ -225,7 +228,8 @@ template <class F>
 struct LoadStream {
     int round, id;     // pair being walked
     int e;             // current entry (n = pair exhausted), -2 = pair not opened yet
-    int n = 0, shared = 0;  // entries of the pair; those whose block is both rows'
+    int n = 0;         // entries of the pair
+    unsigned long long same = 0;  // bit x: both rows name the same block at the entry x behind the current one
     Entry<F> cur;
     int b, kvh;
     Ring ring, ms;
@@ -238,7 +242,7 @@ __device__ __forceinline__ bool open_pair(const Params &P, Tail<F> *tl, LoadStre
     S.b = tl->m_item[S.ms.idx].b;
     S.kvh = tl->m_item[S.ms.idx].kvh;
     S.n = tl->m_count[S.ms.idx];
-    if (F::kShare) S.shared = tl->m_shared[S.ms.idx];
+    if (F::kShare) S.same = tl->m_same[S.ms.idx];
     S.e = 0;
     if (S.n > 0) S.cur = entry_at<F>(mask_rows(tl, P, S.ms.idx), P.row_stride, 0);
     return true;
@@ -254,6 +258,7 @@ __device__ __forceinline__ void close_pair(const Params &P, Tail<F> *tl, LoadStr
 }
 template <class F>
 __device__ __forceinline__ void next_entry(const Params &P, Tail<F> *tl, LoadStream<F> &S) {
+    S.same >>= 1;
     if (++S.e < S.n) S.cur = entry_at<F>(mask_rows(tl, P, S.ms.idx), P.row_stride, S.e);
 }
 
@@ -298,7 +303,7 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
         if (elect_one()) {
             // [half][row][keys][128 B]; a row without a block at an entry gets block 0, its logits are masked out
             const unsigned bar = smem_u32(&tl->k_full[S.ring.idx]), dst = k_smem + S.ring.idx * F::kOperand;
-            const bool both = F::kShare && S.e < S.shared;  // (in row 0's place)
+            const bool both = F::kShare && (S.same & 1u) != 0;  // (in row 0's place)
             mbar_arrive_expect_tx(bar, (unsigned)(both ? F::kTile : F::kOperand));
 #pragma unroll
             for (int c = 0; c < F::kHalves; ++c)
@@ -345,69 +350,6 @@ __device__ void k_producer_role(const Params &P, const CUtensorMap *tq, const CU
     }
 }
 
-// Is x among the ascending 32 kRegs values of a warp, value 32 r + i in register r of lane i?
-template <int kRegs>
-__device__ __forceinline__ bool among(const int (&v)[kRegs], int x) {
-    auto at = [&](int i) {
-        const int low = __shfl_sync(0xffffffffu, v[0], i & 31);
-        if (kRegs == 1) return low;
-        const int high = __shfl_sync(0xffffffffu, v[kRegs - 1], i & 31);  // (every lane takes part in both)
-        return i < 32 ? low : high;
-    };
-    int pos = 0;
-#pragma unroll
-    for (int step = 16 * kRegs; step > 0; step >>= 1) pos += at(pos + step - 1) < x ? step : 0;
-    return at(pos) == x;
-}
-
-// A pair's entries out of its rows' blocks, entry 32 x + lane in a[x], b[x] (negative: none): first those that both rows name, then the
-// rest of both side by side, -1 behind the shorter one. false: the rows are not ascending, as a mask build's are,
-// and nothing is written.
-template <int kRegs>
-__device__ __forceinline__ bool align_rows(const int (&a)[kRegs], const int (&b)[kRegs], int lane, int *to_a, int *to_b, int &count, int &shared) {
-    const unsigned lt = (1u << lane) - 1u;
-    int ka[kRegs], kb[kRegs];  // (none: behind all)
-    bool sorted = true;
-#pragma unroll
-    for (int x = 0; x < kRegs; ++x) { ka[x] = a[x] < 0 ? 0x7fffffff : a[x]; kb[x] = b[x] < 0 ? 0x7fffffff : b[x]; }
-#pragma unroll
-    for (int x = 0; x < kRegs; ++x) {
-        int na = __shfl_down_sync(0xffffffffu, ka[x], 1), nb = __shfl_down_sync(0xffffffffu, kb[x], 1);
-        if (kRegs > 1 && x + 1 < kRegs) {
-            const int ha = __shfl_sync(0xffffffffu, ka[kRegs - 1], 0), hb = __shfl_sync(0xffffffffu, kb[kRegs - 1], 0);
-            if (lane == 31) { na = ha; nb = hb; }
-        } else if (lane == 31) {
-            na = nb = 0x7fffffff;
-        }
-        sorted = sorted && (ka[x] < na || na == 0x7fffffff) && (kb[x] < nb || nb == 0x7fffffff);
-    }
-    // (the last clause: nothing follows an absent entry)
-    if (!__all_sync(0xffffffffu, sorted)) return false;
-    unsigned sa[kRegs], ua[kRegs], ub[kRegs];
-    int n_sa = 0, n_ua = 0, n_ub = 0;
-#pragma unroll
-    for (int x = 0; x < kRegs; ++x) {
-        const bool in_b = among(kb, ka[x]) && a[x] >= 0, in_a = among(ka, kb[x]) && b[x] >= 0;
-        sa[x] = __ballot_sync(0xffffffffu, in_b);
-        ua[x] = __ballot_sync(0xffffffffu, a[x] >= 0 && !in_b);
-        ub[x] = __ballot_sync(0xffffffffu, b[x] >= 0 && !in_a);
-        n_sa += __popc(sa[x]); n_ua += __popc(ua[x]); n_ub += __popc(ub[x]);
-    }
-    shared = n_sa;
-    count = n_sa + max(n_ua, n_ub);
-    int at_s = 0, at_a = n_sa, at_b = n_sa;
-#pragma unroll
-    for (int x = 0; x < kRegs; ++x) {
-        if ((sa[x] >> lane) & 1u) to_a[at_s + __popc(sa[x] & lt)] = to_b[at_s + __popc(sa[x] & lt)] = a[x];
-        if ((ua[x] >> lane) & 1u) to_a[at_a + __popc(ua[x] & lt)] = a[x];
-        if ((ub[x] >> lane) & 1u) to_b[at_b + __popc(ub[x] & lt)] = b[x];
-        at_s += __popc(sa[x]); at_a += __popc(ua[x]); at_b += __popc(ub[x]);
-    }
-    for (int i = at_a + lane; i < count; i += 32) to_a[i] = -1;
-    for (int i = at_b + lane; i < count; i += 32) to_b[i] = -1;
-    return true;
-}
-
 // The V tiles, and the pairs' mask rows up to two pairs ahead of everyone else: only the kept entries
 // of a pair (an entry is kept if either row has a block there) go to shared memory, in order, with
 // their number, so that the other roles index them instead of searching.
@@ -440,20 +382,9 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         }
         if (!probe_w(smem_u32(&tl->m_empty[mw.idx]), mw.phase ^ 1)) return false;
         int *dst = mask_rows(tl, P, mw.idx);
-        int cnt = 0, shared = 0;
-        bool done = false;
-        if constexpr (F::kShare) {
-            if (g.k_top <= 32) {
-                const int a[1] = {first[0]}, b[1] = {first[1]};
-                done = align_rows(a, b, lane, dst, dst + P.row_stride, cnt, shared);
-            } else if (g.k_top <= 64) {
-                int second[2];
-                fetch(lane + 32, second);
-                const int a[2] = {first[0], second[0]}, b[2] = {first[1], second[1]};
-                done = align_rows(a, b, lane, dst, dst + P.row_stride, cnt, shared);
-            }
-        }
-        for (int base = 0; base < g.k_top && !done; base += 32) {
+        int cnt = 0;
+        unsigned same[2] = {0u, 0u};
+        for (int base = 0; base < g.k_top; base += 32) {
             int blk[F::kRows];
             bool kept = false;
             if (base > 0) fetch(base + lane, blk);
@@ -463,17 +394,22 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
                 kept = kept || blk[r] >= 0;
             }
             const unsigned bal = __ballot_sync(0xffffffffu, kept);
+            const int pos = cnt + __popc(bal & ((1u << lane) - 1u));
             if (kept) {
-                const int pos = cnt + __popc(bal & ((1u << lane) - 1u));
 #pragma unroll
                 for (int r = 0; r < F::kRows; ++r) dst[r * P.row_stride + pos] = blk[r];
+            }
+            if (F::kShare && base < 64) {
+                const bool both = kept && blk[0] == blk[F::kRows - 1];
+#pragma unroll
+                for (int x = 0; x < 2; ++x) same[x] |= __reduce_or_sync(0xffffffffu, both && pos >> 5 == x ? 1u << (pos & 31) : 0u);
             }
             cnt += __popc(bal);
         }
         __syncwarp();
         if (lane == 0) {
             tl->m_count[mw.idx] = cnt;
-            if (F::kShare) tl->m_shared[mw.idx] = shared;
+            if (F::kShare) tl->m_same[mw.idx] = same[0] | (unsigned long long)same[1] << 32;
             tl->m_item[mw.idx] = it;
             mbar_arrive(smem_u32(&tl->m_full[mw.idx]));
         }
@@ -490,7 +426,7 @@ __device__ void v_producer_role(const Params &P, const CUtensorMap *tv, Tail<F> 
         if (!probe_w(smem_u32(&tl->v_empty[S.ring.idx]), S.ring.phase ^ 1)) return false;
         if (elect_one()) {  // [row][half][keys][128 B]
             const unsigned bar = smem_u32(&tl->v_full[S.ring.idx]), dst = v_smem + S.ring.idx * F::kOperand;
-            const bool both = F::kShare && S.e < S.shared;
+            const bool both = F::kShare && (S.same & 1u) != 0;
             mbar_arrive_expect_tx(bar, (unsigned)(both ? F::kTile : F::kOperand));
 #pragma unroll
             for (int r = 0; r < F::kRows; ++r)
@@ -519,18 +455,19 @@ __device__ void qk_role(const Params &P, Tail<F> *tl, unsigned q_smem, unsigned 
     const unsigned q_lo0 = desc_lo_sw128(q_smem, 16), k_lo = desc_lo_sw128(k_smem, 16);
     for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 207)) return;
-        const int n_entries = tl->m_count[ms.idx], shared = F::kShare ? tl->m_shared[ms.idx] : 0;  // the issuers need no more than the counts
+        const int n_entries = tl->m_count[ms.idx];  // the issuers need no more than the count and which entries are one tile
+        unsigned long long same = F::kShare ? tl->m_same[ms.idx] : 0ull;
         const unsigned q_lo = q_lo0 + qs.idx * (F::kOperand >> 4);
         if (n_entries > 0) {
             if (!wait_w(smem_u32(&tl->q_full[qs.idx]), qs.phase, tl, 201)) return;
             qs.advance(2);
         }
-        for (int i = 0; i < n_entries; ++i) {
+        for (int i = 0; i < n_entries; ++i, same >>= 1) {
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++;  // entry i of a pair belongs to group i % 2
             if (!wait_both_w(smem_u32(&tl->k_full[ks.idx]), ks.phase, 202, smem_u32(&tl->s_free[gi][use & 1u]), ((use >> 1) & 1u) ^ 1u, 203, tl)) return;
             tc_fence_after();
             const unsigned d_tmem = tmem_base + gi * 128 + (use & 1u) * 64;
-            const unsigned b_lo = k_lo + ks.idx * (F::kOperand >> 4), row_1 = F::kShare && i < shared ? 0u : (unsigned)kHalfTile >> 4;
+            const unsigned b_lo = k_lo + ks.idx * (F::kOperand >> 4), row_1 = F::kShare && (same & 1u) ? 0u : (unsigned)kHalfTile >> 4;
             if (elect_one()) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
@@ -563,8 +500,9 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
     const unsigned v_lo = desc_lo_sw128(v_smem, F::kPart), d_tmem = tmem_base + F::kOCol;
     for (int round = 0, id; (id = nth_item(round)) < P.n_items; ++round) {
         if (!wait_w(smem_u32(&tl->m_full[ms.idx]), ms.phase, tl, 208)) return;
-        const int n_entries = tl->m_count[ms.idx], shared = F::kShare ? tl->m_shared[ms.idx] : 0;
-        for (int i = 0; i < n_entries; ++i) {
+        const int n_entries = tl->m_count[ms.idx];
+        unsigned long long same = F::kShare ? tl->m_same[ms.idx] : 0ull;
+        for (int i = 0; i < n_entries; ++i, same >>= 1) {
             const unsigned gi = (unsigned)(i & 1), use = gi ? cnt[1]++ : cnt[0]++, pb = use % F::kPBufs;
             // (P is there: also, O is rescaled if it had to be)
             if (!wait_both_w(smem_u32(&tl->v_full[vs.idx]), vs.phase, 205, smem_u32(&tl->p_full[gi][pb]), (use / F::kPBufs) & 1u, 204, tl)) return;
@@ -573,7 +511,7 @@ __device__ void pv_role(const Params &P, Tail<F> *tl, unsigned v_smem, unsigned 
                 free_par ^= 1;
             }
             tc_fence_after();
-            const unsigned a_tmem = tmem_base + F::kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (F::kOperand >> 4), row_1 = F::kShare && i < shared ? 0u : (unsigned)F::kTile >> 4;
+            const unsigned a_tmem = tmem_base + F::kPCol + gi * 64 + pb * 32, b_lo = v_lo + vs.idx * (F::kOperand >> 4), row_1 = F::kShare && (same & 1u) ? 0u : (unsigned)F::kTile >> 4;
             if (elect_one()) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)  // row r of the pair: its P (or the parts of it), its V tile
