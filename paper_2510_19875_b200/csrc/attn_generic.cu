@@ -369,17 +369,19 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     // Four warps a CTA, so that several CTAs share an SM; eight when every row has an SM to itself
     // anyway. Fewer rows than half of the SMs: a row over two, four or eight CTAs, while each has a tile part for
     // every scheduler (28 rows, blocks of 64, k = 11, d = 64: 65.4 -> 34.8 us; 55 rows, blocks of 32, k = 9, d = 128:
-    // 38.9 -> 30.7). Not where a row has no more than eight tiles of 64 channels or fewer: a CTA alone begins while the kernel before it
-    // still runs, as no cluster does (us with the mask build, cluster and alone: 64 rows of blocks of 32, d = 64, k = 8: 43.0, 39.9;
-    // 40 rows: 31.8, 28.8; 72 rows, d = 32: 37.3, 34.8; 64 rows, k = 6: 45.0, 44.9, k = 10: 50.5, 51.3; 72 rows, d = 128, k = 8: 65.5,
-    // 69.7; 32 rows of blocks of 64, k = 6: 55.3, 69.6). The mask build gains from clusters at all of these but k = 4.
+    // 38.9 -> 30.7). Not where a row has little to share out, eight tiles of 32 queries and 64 channels or fewer: a CTA alone begins while
+    // the kernel before it still runs, as no cluster does (us with the mask build in a graph, cluster and alone: blocks of 32, k = 8: d = 64,
+    // 24 rows 32.9, 32.9, 72 rows 41.0, 40.5, d = 32 26.7, 25.5 and 32.8, 30.8, d = 16, 10 rows, 20.5, 18.6; blocks of 16, d = 16, k = 8, 24 rows
+    // 21.6, 18.5, but d = 32, 56 rows 27.4, 28.7; blocks of 64, whose rows are two warps' work a tile: k = 2, d = 32, 40 rows 36.9, 34.9, k = 3,
+    // d = 64, 24 rows 43.9, 47.2, k = 4 41.1, 50.4, 72 rows 59.5, 65.6, d = 16 36.9, 39.0; more tiles: 64 rows of blocks of 32, d = 64,
+    // k = 10, 50.5, 51.3; 72 rows, d = 128, k = 8, 65.5, 69.7).
     // T may have fewer blocks than k_top, and what counts are those that are there: a CTA of a cluster has two tile
     // parts at least, a group half of one (16 rows, T = 29, blocks of 48, k = 9, d = 16: 32 -> 10 us); with many
     // rows an idle group takes another CTA's shared memory (2500 rows, k = 1, d = 128, rows off 16 bytes: 397 -> 223).
     const int n_sm = sm_count_or_default(), n_sub = (g.bk + kKeys - 1) / kKeys, tiles = g.k_top * n_sub;
     const int there = (int)std::min((long long)g.k_top, (g.T + g.bk - 1) / g.bk) * n_sub;
     int splits = (rows <= n_sm ? 8 : 4) / m_warps, n_cta = 1;
-    const bool small = D <= 64 && there <= 8;
+    const bool small = D <= 64 && there * m_warps <= 8;
     while (!small && n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta && there >= 3 && there >= 2 * n_cta) n_cta *= 2;
     if (n_cta > 1) splits = std::min({splits, (tiles + n_cta - 1) / n_cta, 2 * ((there + n_cta - 1) / n_cta)});
     else if (rows > n_sm) splits = std::min(splits, rows > 4ll * n_sm ? there : 2 * there);
