@@ -872,7 +872,7 @@ bool two_of_two_rows(const Geom &g) {
 // fewer of them make more and shorter groups. Four rows (of several query blocks, unless k changes from one to the next, where a kv head
 // has fewer than four heads) are taken where every CTA has some groups of them, else two, else one.
 struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
-stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_rows, Split *s) {
+stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_rows, bool several_k, Split *s) {
     const int n_cta = sm_count() * ctas_per_sm;
     if (n_cta <= 0) { set_error("cannot read the SM count of the current device"); return STREAM_ERR_CUDA; }
     s->n_chunks = (g.hpg + most_rows - 1) / most_rows;
@@ -894,7 +894,11 @@ stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_
         // which begins earlier behind fewer and longer groups: 8 / 2 heads, 16000, k = 60 (1.7): 548, 557; 16 heads, 8192, k = 40 (1.7): 358, 360.
         const bool wide = g.k_top > 32;
         int halves;
-        if (small_tiles(g)) halves = rows > 2 ? (wide ? 2 : 6) : (wide ? 3 : 6);
+        // Several k: a group's passes make it long by themselves, and fewer rows share less. Groups of a build that is not causal, or of several query
+        // blocks, are nearly equally long (28 / 4 heads, 2992 tokens, k = 3, 7, 14, not causal (2.5): 115, 146; 24 / 8 heads, 4551, not causal (3.9): 164,
+        // 244; 2 heads, 40264 (2.1): two rows 1.3 times four; 8 / 2 heads, 10311, k = 5, 10, 21 (2.2): 201, 149; 5501 (2.3): 114, 97).
+        if (several_k) halves = rows > 2 ? (g.causal && s->qb_rows == 1 ? 5 : 3) : 2;
+        else if (small_tiles(g)) halves = rows > 2 ? (wide ? 2 : 6) : (wide ? 3 : 6);
         else halves = rows > 2 ? (s->qb_rows > 1 ? 4 : 8) : 2;
         if (2 * s->n_groups >= (long long)halves * n_cta || rows == 1) break;
         if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
@@ -921,7 +925,7 @@ cudaError_t launch_rows(const Geom &g, const Split &sp, int grid, cudaStream_t s
 
 size_t mask_tc_score_memory_bytes(const Geom &g) {
     Split sp;
-    if (split_rows(g, 0, 1, kMultiRows, &sp) != STREAM_OK) return 0;
+    if (split_rows(g, 0, 1, kMultiRows, true, &sp) != STREAM_OK) return 0;
     return (size_t)sp.grid * kMultiRows * (size_t)g.N_k * sizeof(unsigned long long);
 }
 
@@ -950,7 +954,7 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     Split sp;
     const bool two_rows = mk.n == 0 && two_of_two_rows(g);
     const int ctas = (mk.n == 0 && small_tiles(g)) || two_rows ? 2 : 1;
-    rc = split_rows(g, P.first_qb, ctas, two_rows ? 2 : 4, &sp);
+    rc = split_rows(g, P.first_qb, ctas, two_rows ? 2 : 4, mk.n >= 1, &sp);
     if (rc != STREAM_OK) return rc;
     P.n_groups = (int)sp.n_groups;
     P.walked_heads = walked_heads(g);
