@@ -1,7 +1,7 @@
 // Tensor-core Stream mask kernel for sm_100a: bf16, d = 64 or 128, blocks of 32 or 64, k_top <= 64.
 // (Figures: d = 128, blocks of 64, unless they say otherwise.)
 //
-// One persistent CTA per SM (two smaller ones where small_tiles or two_of_two_rows says so) works through "groups": up to four rows
+// One persistent CTA per SM (two smaller ones where two_of_four_rows or two_of_two_rows says so) works through "groups": up to four rows
 // of one kv head, its query heads at one query block or, where these are few, at some. Their Q tiles stay in shared memory for the whole
 // hierarchy (Algorithm 2).
 // Candidate key blocks are fetched by TMA (128-byte swizzle), 128 keys at a time, into a ring of
@@ -855,22 +855,26 @@ bool mask_tc_auto(const Geom &g, int dtype) {
 }
 
 namespace {
-// Two CTAs an SM for the shapes whose Q and key tiles leave room for it. With lists of a few stages every role of a lone CTA waits for the
-// others most of the time; two groups fill each other's gaps (us, one and two: 12 / 2 heads, 10007 tokens in blocks of 32,
-// k = 8: 114.9, 94.1; 6 / 2 heads, 20000, k = 16: 166, 147.5; d = 64: 32 / 8 heads, 4000 tokens, k = 16: 76.0, 65.6; 16 heads,
-// 8192 tokens, k = 40, not causal: 157.2, 150.6; 8 / 2 heads, 16000, k = 60, not causal: 260, 242).
-bool small_tiles(const Geom &g) { return g.d == 64 || g.bq == 32; }
+// Two CTAs an SM of up to four rows each, where Q and key tiles leave room for them. With lists of a few stages every role of a lone CTA waits
+// for the others most of the time; two groups fill each other's gaps (us, one and two: 12 / 2 heads, 10007 tokens in blocks of 32,
+// k = 8: 114.9, 94.1; d = 64: 32 / 8 heads, 4000 tokens, k = 16: 76.0, 65.6). Not for d = 128 in blocks of 32 with more than 32 blocks a list
+// but in long launches: two stages of 128 keys are too few there for one group to go on while the other waits (us, the better split
+// of one and of two, in brackets the rows an SM: 8 / 2 heads, 6835 tokens, k = 64 (8): 66, 84; 28 / 4 heads, 3973, k = 64 (12): 68, 75; 8 / 4 heads,
+// 11084, k = 51 (16): 139, 142; 24 / 8 heads, 4918, k = 34 (20): 125, 117; 5369, k = 38, not causal (27): 236, 202; 8 / 2 heads, 17789, k = 45 (30): 396, 398).
+bool two_of_four_rows(const Geom &g, int first_qb) {
+    return g.d == 64 || (g.bq == 32 && (g.k_top <= 32 || (long long)g.batch * g.H * (g.n_qb - first_qb) >= 18ll * sm_count()));
+}
 // With d = 128 and blocks of 64 there is room for two CTAs of two rows and two stages each: better with up to eight blocks a list and no more than
 // eight groups a CTA (32 / 8 heads, 2500 tokens, k = 8: 45.1 -> 36.9; 28 / 4 heads, 1500, k = 5: 29.8 -> 26.7; 12 / 2 heads, 20000,
 // k = 6, not causal: 189 -> 180), worse where the tensor cores are the limit (28 / 4 heads, 6000 tokens, k = 12, not causal: 139 -> 144;
 // 32 / 8 heads, 60000, k = 10: 2139 -> 2200; 16384, k = 16: 486 -> 521).
 bool two_of_two_rows(const Geom &g) {
-    return !small_tiles(g) && g.k_top <= 8 && g.k_row == nullptr && (long long)g.batch * g.H * g.n_qb <= 2 * 8 * 2ll * sm_count();
+    return g.d == 128 && g.bq == 64 && g.k_top <= 8 && g.k_row == nullptr && (long long)g.batch * g.H * g.n_qb <= 2 * 8 * 2ll * sm_count();
 }
 
 // CTAs of a launch, the groups they share and the rows of a group. Rows share the key tiles of the first level and its chains of two;
 // fewer of them make more and shorter groups. Four rows (of several query blocks, unless k changes from one to the next, where a kv head
-// has fewer than four heads) are taken where every CTA has some groups of them, else two, else one.
+// has fewer than four heads) are taken where there are rows for some groups of them a CTA, else two, else one.
 struct Split { int grid, head_rows, qb_rows, n_chunks; long long n_groups; };
 stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_rows, bool several_k, Split *s) {
     const int n_cta = sm_count() * ctas_per_sm;
@@ -883,24 +887,33 @@ stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_
         const int rows = s->head_rows * s->qb_rows;
         s->n_chunks = (g.hpg + s->head_rows - 1) / s->head_rows;
         s->n_groups = (long long)g.batch * g.G * ((g.n_qb - first_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
-        // Groups that a CTA should have, in halves. One CTA an SM, us with four, two rows and one: 28 / 4 heads, 3000 tokens, k = 8 (2.1
-        // groups a CTA of four rows): 59.5, 50.0, 60.7; 3419, k = 27, not causal (2.9): 83, 74, 101; 8 / 2 heads, 20000, k = 24 (3.9):
-        // 210, 195; 8 / 2 heads, 13232, k = 59 (2.0): 186, 157, 188; but of several query blocks: 16 heads, 9000, k = 12 (3.5): 118, 124.
-        // Two rows and one: 8 / 2 heads, 8000, k = 16 (2.9 of two): 51, 68; 12 / 2 heads, 8000 (4.4): 69, 98; 16 heads, 2000, k = 12 (1.1):
-        // 24.5, 28.7; 32 / 8 heads, 1200, k = 8 (1.2): 22.5, 24.2. Two CTAs, rows of one or two nodes a lane apart: 12 / 2 heads, 5000 in blocks
-        // of 32, k = 8 (2.0 of three): 49.2, 47.2; 28 / 4 heads, 4600, k = 24, not causal (3.9): 114, 126; d = 64, two and one: 32 / 8 heads,
-        // 4000, k = 16 (2.5): 65.6, 54.7; 16 heads, 6000, k = 12 (2.2): 57, 51; 8 / 2 heads, 9000, k = 20 (1.6): 76, 68; two nodes: 28 / 4 heads,
-        // 1074 in blocks of 32, k = 33 (1.8): 26.7, 32.8; four and two: 4000, k = 50 (2.0): 82.3, 81.3; d = 64, not causal, with the attention,
-        // which begins earlier behind fewer and longer groups: 8 / 2 heads, 16000, k = 60 (1.7): 548, 557; 16 heads, 8192, k = 40 (1.7): 358, 360.
+        // How many groups a CTA there should be rows for, in halves: from 545 drawn shapes (k = 2 to 64), each timed at every number of rows;
+        // over 220 others 2.4 % behind the best of these on average, with the attention behind it 1.3. Rows, not groups: three heads as 2 + 1 make more groups than they have work for (6 / 2
+        // heads, 4458 tokens, k = 24: two rows 44.2 us, one 34.8). Some of them, us with four (or three) rows, two and one, in brackets the
+        // groups of four a CTA. One CTA an SM: 28 / 4 heads, 3419 tokens, k = 27, not causal (2.9): 83, 74, 101; 8 / 2 heads, 20000, k = 24 (3.9):
+        // 210, 195; 8 / 2 heads, 13232, k = 59 (2.0): 186, 157, 188; of several query blocks: 16 heads, 9000, k = 12 (3.5): 118, 124, and with
+        // two nodes a lane: 1 head, 80291, k = 37 (2.0): 267, 235. Two CTAs, blocks of 64: 28 / 4 heads, 2500, k = 33, not causal (1.1): 73.6, 56.4, 43.0;
+        // 12 / 2 heads, 10922, k = 45 (1.7): 177, 156, 107; 2 heads, 73665, k = 16 (1.9): -, 168, 186. Blocks of 32, where a pair of rows is little
+        // more work than a row alone: 12 / 2 heads, 6000, k = 40 (2.0): 75.7, 69.7; 28 / 4 heads, 3000, k = 40, d = 128 (1.5): 61, 55, 70.
         const bool wide = g.k_top > 32;
         int halves;
-        // Several k: a group's passes make it long by themselves, and fewer rows share less. Groups of a build that is not causal, or of several query
-        // blocks, are nearly equally long (28 / 4 heads, 2992 tokens, k = 3, 7, 14, not causal (2.5): 115, 146; 24 / 8 heads, 4551, not causal (3.9): 164,
-        // 244; 2 heads, 40264 (2.1): two rows 1.3 times four; 8 / 2 heads, 10311, k = 5, 10, 21 (2.2): 201, 149; 5501 (2.3): 114, 97).
-        if (several_k) halves = rows > 2 ? (g.causal && s->qb_rows == 1 ? 5 : 3) : 2;
-        else if (small_tiles(g)) halves = rows > 2 ? (wide ? 2 : 6) : (wide ? 3 : 6);
-        else halves = rows > 2 ? (s->qb_rows > 1 ? 4 : 8) : 2;
-        if (2 * s->n_groups >= (long long)halves * n_cta || rows == 1) break;
+        bool full = false;
+        if (several_k) {
+            // A group's passes make it long by themselves, and fewer rows share less. Groups of a build that is not causal, or of several query blocks, are
+            // nearly equally long (28 / 4 heads, 2992 tokens, k = 3, 7, 14, not causal (2.5): 115, 146; 24 / 8 heads, 4551, not causal (3.9): 164,
+            // 244; 2 heads, 40264 (2.1): two rows 1.3 times four; 8 / 2 heads, 10311, k = 5, 10, 21 (2.2): 201, 149; 5501 (2.3): 114, 97).
+            halves = rows > 2 ? (g.causal && s->qb_rows == 1 ? 5 : 3) : 2;
+        } else if (ctas_per_sm == 2 && most_rows == 4) {
+            halves = rows > 2 ? 6 : (g.bq == 64 ? (wide ? 12 : 7) : (wide ? 3 : 2));
+            // Not causal, the groups are equally long: also where more than one round of them is five sixths full (16 heads, 8192 tokens, k = 40 (1.7):
+            // 153, 151, 154, with the attention behind them 350, -, 359; 8 / 2 heads, 16000, k = 60 (1.7): 246, 252; 16 heads, 5345, k = 37 (1.1): 113, 96, 94).
+            const long long rounds = (s->n_groups + n_cta - 1) / n_cta;
+            full = rows > 2 && !g.causal && rounds > 1 && 6 * s->n_groups >= 5 * rounds * n_cta;
+        } else {
+            halves = rows > 2 ? (s->qb_rows > 1 ? (wide ? 6 : 4) : (wide ? 7 : 8)) : 2;
+        }
+        const long long there = several_k ? s->n_groups : (long long)g.batch * g.H * (g.n_qb - first_qb) / rows;
+        if (full || 2 * there >= (long long)halves * n_cta || rows == 1) break;
         if (s->qb_rows > 1) s->qb_rows = (s->qb_rows + 1) / 2;
         else s->head_rows = (s->head_rows + 1) / 2;
     }
@@ -916,10 +929,9 @@ cudaError_t launch(int grid, cudaStream_t st, const CUtensorMap &tq, const CUten
     return e == cudaSuccess ? launch_kernel(mask_tc_kernel<S>, grid, S::kThreads, kSmemBytes<S>, st, 1, tq, tk, P) : e;
 }
 
-template <int kD, int kBlk, bool kTwo>
-cudaError_t launch_rows(const Geom &g, const Split &sp, int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
-    if (g.k_top > 32) return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, true, false, true, kTwo>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, true, false, false, kTwo>>(grid, st, tq, tk, P);
-    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, false, false, true, kTwo>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, false, false, false, kTwo>>(grid, st, tq, tk, P);
+template <int kD, int kBlk, bool kWide, bool kTwo>
+cudaError_t launch_rows(const Split &sp, int grid, cudaStream_t st, const CUtensorMap &tq, const CUtensorMap &tk, const Params &P) {
+    return sp.qb_rows > 1 ? launch<Shape<kD, kBlk, kWide, false, true, kTwo>>(grid, st, tq, tk, P) : launch<Shape<kD, kBlk, kWide, false, false, kTwo>>(grid, st, tq, tk, P);
 }
 }  // namespace
 
@@ -953,7 +965,7 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     if (P.first_qb == g.n_qb) return launch_mask_whole(g, g.n_qb, mask, ws, st);
     Split sp;
     const bool two_rows = mk.n == 0 && two_of_two_rows(g);
-    const int ctas = (mk.n == 0 && small_tiles(g)) || two_rows ? 2 : 1;
+    const int ctas = (mk.n == 0 && two_of_four_rows(g, P.first_qb)) || two_rows ? 2 : 1;
     rc = split_rows(g, P.first_qb, ctas, two_rows ? 2 : 4, mk.n >= 1, &sp);
     if (rc != STREAM_OK) return rc;
     P.n_groups = (int)sp.n_groups;
@@ -986,9 +998,12 @@ stream_status launch_mask_tc_multi(const Geom &g, const MultiK &mk, const void *
     }
     if (mk.n >= 1 && score_memory == nullptr) { set_error("several k in one launch need the score memory"); return STREAM_ERR_WORKSPACE; }
     if (mk.n >= 1) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, true>>(grid, st, tq, tk, P);
-    else if (two_rows) e = sp.qb_rows > 1 ? launch<Shape<128, 64, false, false, true, true>>(grid, st, tq, tk, P) : launch<Shape<128, 64, false, false, false, true>>(grid, st, tq, tk, P);
-    else if (g.d == 128) e = g.bq == 64 ? launch_rows<128, 64, false>(g, sp, grid, st, tq, tk, P) : launch_rows<128, 32, true>(g, sp, grid, st, tq, tk, P);
-    else e = g.bq == 64 ? launch_rows<64, 64, true>(g, sp, grid, st, tq, tk, P) : launch_rows<64, 32, true>(g, sp, grid, st, tq, tk, P);
+    else if (two_rows) e = launch_rows<128, 64, false, true>(sp, grid, st, tq, tk, P);
+    else if (g.d == 128 && g.bq == 64) e = g.k_top > 32 ? launch_rows<128, 64, true, false>(sp, grid, st, tq, tk, P) : launch_rows<128, 64, false, false>(sp, grid, st, tq, tk, P);
+    else if (g.d == 128 && g.k_top <= 32) e = launch_rows<128, 32, false, true>(sp, grid, st, tq, tk, P);
+    else if (g.d == 128) e = ctas == 2 ? launch_rows<128, 32, true, true>(sp, grid, st, tq, tk, P) : launch_rows<128, 32, true, false>(sp, grid, st, tq, tk, P);
+    else if (g.bq == 64) e = g.k_top > 32 ? launch_rows<64, 64, true, true>(sp, grid, st, tq, tk, P) : launch_rows<64, 64, false, true>(sp, grid, st, tq, tk, P);
+    else e = g.k_top > 32 ? launch_rows<64, 32, true, true>(sp, grid, st, tq, tk, P) : launch_rows<64, 32, false, true>(sp, grid, st, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tc launch");
     return STREAM_OK;
 }
