@@ -167,11 +167,6 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     unsigned q_par = 0;
     unsigned long long tiles_needed = 0, products = 0;  // per thread
 
-    // Warps without a part in the levels write the tokens' rows that belong to no group, beside the first one.
-    if (P.first_tb > 0 && (warp == 2 || warp >= 12)) {
-        write_whole_rows(g, P.first_tb * kTok, (int)blockIdx.x * 5 + (warp == 2 ? 0 : warp - 11), (int)gridDim.x * 5, lane, P.mask, P.ws);
-    }
-
     for (int id = (int)blockIdx.x;;) {  // (the first group is the CTA's own, the counter deals those behind)
         if (id >= P.n_items || *(volatile int *)&tl->abort_flag) break;
         // late token groups (most allowed blocks) of all the heads walked together first
@@ -208,13 +203,15 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int e_qlim = e_ok ? last_valid_block(g, (int)e_tq) : -1;
         const int key_end = e_ok ? (int)(g.causal ? e_tq + 1 : g.T) : 0;  // keys the token may look at: those before
         unsigned n_tiles = 0;  // tiles the token has needed so far (its own candidates, not the merged list)
+        // the next group's number is fetched beside this one's products, unless that could leave another CTA without work
+        const bool ahead = id + 2 * (int)gridDim.x < P.n_items;
 
         for (int level = 0;; ++level) {
             __syncthreads();  // the level's list is complete; the ranking of the level before is done
             const bool last = level + 1 == tl->n_levels;
             const int n_list = tl->n_list, n_st = (n_list + 1) >> 1;
 
-            if (warp == 13 && lane == 0 && level == 0) tl->item = (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
+            if (ahead && warp == 13 && lane == 0 && level == 0) tl->item = (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
             if (is_producer) {
                 for (int i = 0; i < n_st; ++i) {
                     const unsigned s = seq + (unsigned)i, buf = s & 3u;
@@ -495,8 +492,18 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
         if (*(volatile int *)&tl->abort_flag) break;
         if (warp == 0 && lane == 0) atomicAdd(&P.ws->rows, (unsigned long long)(tq_max - tok0 + 1));
+        if (!ahead) {
+            if (tid == 0) tl->item = P.n_items <= (int)gridDim.x ? P.n_items : (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
+            __syncthreads();
+        }
         id = tl->item;
         __syncthreads();
+    }
+    // The tokens' rows that belong to no group: by the CTAs without one, where a quarter of the launch has none, else by all behind their last.
+    if (P.first_tb > 0) {
+        const int spare = (int)gridDim.x - P.n_items, first = 4 * spare >= (int)gridDim.x ? P.n_items : 0, writer = (int)blockIdx.x - first;
+        constexpr int kWarps = kThreads / 32;
+        if (writer >= 0) write_whole_rows(g, P.first_tb * kTok, writer * kWarps + warp, ((int)gridDim.x - first) * kWarps, lane, P.mask, P.ws);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tiles_needed += __shfl_xor_sync(0xffffffffu, tiles_needed, o);
@@ -543,7 +550,8 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     auto kern = g.k_top <= 16 ? mask_tok_kernel<16> : mask_tok_kernel<32>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tok)");
-    const long long writers = P.first_tb > 0 ? (whole_pieces(g, P.first_tb * kTok) + 4) / 5 : 0, ctas = n_items > writers ? n_items : writers;
+    // (a CTA more for every four pieces of the rows kept whole)
+    const long long ctas = n_items + (P.first_tb > 0 ? (whole_pieces(g, P.first_tb * kTok) + 3) / 4 : 0);
     const int grid = (int)(ctas < n_sm ? ctas : n_sm);
     e = launch_kernel(kern, grid, kThreads, kSmemBytes, st, 1, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tok launch");
