@@ -83,6 +83,37 @@ def workload_config(spec, extra=None):
     return cfg
 
 
+def tiles_kept_whole(spec, block_q=0):
+    """Tiles of the rows that a causal build with one k and no scores asked for writes without products, because they have no more
+    allowed key blocks than k (``tiles_scored`` has them all the same): of the block kernel, or (block_q = 1) of the per-token
+    kernel, whose rows go in groups of 128 tokens. All of them where no row has more."""
+    bq = block_q or spec.block
+    n_qb, n_kb = -(-spec.T // bq), -(-spec.T // spec.block)
+    if n_kb == 1:
+        return 0  # (nothing to score)
+    n = n_qb if n_kb <= spec.k_top else spec.k_top * spec.block // bq
+    if bq == 1 and n < n_qb:
+        n -= n % 128
+    return spec.batch * spec.n_q_heads * sum((min((qb + 1) * bq, spec.T) - 1) // spec.block + 1 for qb in range(n))
+
+
+def attention_tiles_fetched(mask, n_kv_heads):
+    """K and V tiles that the tcgen05 attention with d = 128 and blocks of 64 copies into shared memory for these masks [B, H, n_qb, k]
+    as a build leaves them: two rows of a kv head's sequence (query block by query block, head by head, paired from the end) go
+    side by side, an entry brings a tile for either row, and one for both where the same block is the same entry's (of the first 64)."""
+    import torch
+
+    B, H, n_qb, k = mask.shape
+    rows = mask.view(B, n_kv_heads, H // n_kv_heads, n_qb, k).transpose(2, 3).reshape(B, n_kv_heads, -1, k)
+    if rows.shape[2] % 2:  # the first row is alone in its pair
+        rows = torch.cat([torch.full_like(rows[:, :, :1], -1), rows], 2)
+    pairs = rows.reshape(B, n_kv_heads, -1, 2, k)
+    a, b = pairs[..., 0, :], pairs[..., 1, :]
+    entries = ((a >= 0) | (b >= 0)).sum()
+    same = ((a >= 0) & (a == b))[..., :64].sum()
+    return 2 * int(2 * entries - same)
+
+
 class ClockSampler:
     """nvidia-smi clocks and throttle reasons, sampled every 50 ms while the timed region runs."""
 
@@ -348,6 +379,7 @@ def run_ours(args):
     attn_ms = statistics.mean(e[1].elapsed_time(e[2]) for e in ev)
     stats = S.stream_read_stats(ws, stream)
     kept = int((mask >= 0).sum().item())
+    fetched = attention_tiles_fetched(mask, spec.n_kv_heads) if spec.d == 128 and spec.block == 64 else 2 * kept
 
     # end to end through the host entry point: pinned host tensors in, mask + output back
     e2e = None
@@ -394,13 +426,17 @@ def run_ours(args):
     tile_bytes = spec.block * spec.d * esz
     peak, peak_kind = hbm_peak()
     tc = spec.dtype == "bf16" and spec.d == 128 and spec.block == 64 and args.kernels != "generic"
+    mask_tc = tc and spec.k_top <= (32 if args.kernels == "tensor" else 64)
+    # the tiles that were multiplied: without those of rows kept whole (all kernels write a mask of nothing but such rows)
+    whole = tiles_kept_whole(spec) if k_row is None and (mask_tc or spec.n_blocks <= spec.k_top) else 0
+    computed = S_tiles - whole
     # algorithmic bytes per launch: every scored / kept tile counted as one fetch, Q in, result out
     kernels = {
         "stream_build_mask": {
-            "kernel": "mask_tc_kernel" if tc and spec.k_top <= 32 else "mask_generic_kernel", "ms": mask_ms,
+            "kernel": "mask_whole_kernel" if computed == 0 else "mask_tc_kernel" if mask_tc else "mask_generic_kernel", "ms": mask_ms,
             "algorithmic_bytes": S_tiles * tile_bytes + units * spec.d * esz + spec.n_rows * spec.k_top * 4,
-            "tiles_scored": S_tiles, "value": units / (mask_ms * 1e-3), "unit": UNIT,
-            "tensor_tflops": S_tiles * 2.0 * spec.block * spec.block * spec.d / (mask_ms * 1e-3) / 1e12},
+            "tiles_scored": S_tiles, "tiles_computed": computed, "value": units / (mask_ms * 1e-3), "unit": UNIT,
+            "tensor_tflops": computed * 2.0 * spec.block * spec.block * spec.d / (mask_ms * 1e-3) / 1e12},
         "stream_sparse_attention": {
             "kernel": "attn_tc_kernel" if tc else "attn_generic_kernel", "ms": attn_ms,
             "algorithmic_bytes": kept * 2 * tile_bytes + 2 * units * spec.d * esz, "kept_blocks": kept,
@@ -453,9 +489,9 @@ def run_ours(args):
         cycles = dom["ms"] * 1e-3 * sm_mhz * 1e6  # per SM, at the sampled clock
         if dominant == "stream_build_mask":
             gathered = int(stats.tiles_fetched) * tile_bytes          # counted by the kernel
-            mma_cycles = S_tiles / 2 * 8 * unit_rates.mma_cycles_m128n64 / n_sm   # chains of two tiles, eight MMAs each
+            mma_cycles = computed / 2 * 8 * unit_rates.mma_cycles_m128n64 / n_sm   # chains of two tiles, eight MMAs each
         else:
-            gathered = kept * 2 * tile_bytes + units * spec.d * esz   # K and V tile per kept block, Q once
+            gathered = fetched * tile_bytes + units * spec.d * esz   # K and V tiles, Q once
             mma_cycles = None
         per_clk = gathered / n_sm / cycles
         roof["unit_rates"] = {
@@ -683,9 +719,9 @@ def run_per_token(args):
         "data": "synthetic",
         "config": workload_config(spec, {"block_q": 1, "kernels": args.kernels, "step": "per-token mask build only",
                                          "l2": "inputs larger than L2" if (q.numel() + k.numel()) * esz > 126e6 else "inputs fit L2"}),
-        "mask_build": {"kernel": "mask_tok_kernel" if on_tensor else "mask_generic_kernel", "ms": ms,
-                       "tiles_scored": int(st.tiles_scored), "tile_products": products,
-                       "useful_fraction_of_products": (int(st.tiles_scored) / 64.0) / products if products else None},
+        "mask_build": {"kernel": "mask_tok_kernel" if on_tensor else "mask_whole_kernel" if spec.n_blocks <= spec.k_top else "mask_generic_kernel",
+                       "ms": ms, "tiles_scored": int(st.tiles_scored), "tile_products": products,
+                       "useful_fraction_of_products": ((int(st.tiles_scored) - tiles_kept_whole(spec, 1)) / 64.0) / products if products else None},
         "roofline": {"bound": "tensor", "kernel": "mask_tok_kernel", "entry_point": "stream_build_mask", "achieved": achieved,
                      "peak": tpeak, "unit": "TFLOP/s", "frac": achieved / tpeak, "peak_kind": f"of {tpeak_kind}", "traffic": None,
                      "flops": "tile products the kernel computed (every fetched key tile x 128 tokens) x 2 x 64 x 64 x d",

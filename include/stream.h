@@ -76,19 +76,22 @@ typedef struct {
 
 /* Counters a mask build leaves in the first bytes of its workspace. */
 typedef struct {
-    uint64_t tiles_scored; /* (row, representative key block) tiles whose score was computed. (Where no scores are
-                              asked for, a row with no more allowed blocks than k needs none: it keeps
-                              them all. Its tiles are counted all the same.) */
+    uint64_t tiles_scored; /* (row, representative key block) tiles that the method scores. (A row with no more
+                              allowed blocks than k keeps them all whatever their scores: where these are
+                              not asked for it may be written without computing them. Its tiles
+                              are counted all the same.) */
     uint64_t rows;         /* rows finished */
     uint32_t error;        /* 0, or a code saying which bounded wait ran out (kernel returned early) */
     uint32_t error_info;
     uint64_t tile_products; /* 64 x 64 x d tile products the per-token tensor-core kernel computed (it
-                               multiplies every fetched key tile with 128 tokens at once, so this
-                               exceeds tiles_scored / 64); 0 from the other kernels, whose products
-                               are exactly the tiles scored */
+                               multiplies every fetched key tile with 128 tokens at once, so this exceeds
+                               what its tokens' scored tiles / 64 would be; none for groups of tokens
+                               that keep all they may); 0 from the other kernels, whose products are
+                               the tiles scored, but for rows written without them */
     uint64_t tiles_fetched; /* key and query tiles (block x d) the tensor-core block kernel copied into
                                shared memory: fewer than tiles_scored where a fetched key tile serves
-                               several rows; 0 from the kernels that do not count them */
+                               several rows, none for rows written without products; 0 from the
+                               kernels that do not count them */
 } stream_stats;
 
 /* Library version: major * 10000 + minor * 100 + patch. */
