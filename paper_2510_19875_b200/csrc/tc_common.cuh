@@ -622,8 +622,9 @@ inline bool tma_strides_ok(const Geom &g) {
 // One head after the other, the last one's long groups began when most CTAs were about to finish (us: 28 / 4 heads, 1500 tokens, k = 5:
 // 36.1 -> 29.2; 12 / 2 heads, 5000 tokens in blocks of 32, k = 8: 60.7 -> 55.3; three k at 5000 tokens, 28 / 4 heads: 179.6 -> 144.5,
 // at 12845, 12 / 2 heads: 288 -> 240; three layers of 11851, 8 / 2 heads, k = 21: 303 -> 271; per token, 32 / 8 heads, 4096 tokens,
-// k = 16: 119.5 -> 108.6. With 32 / 8 heads and 16000 tokens or more it makes no difference, but for three k at 16000: 879 -> 892. Half
-// or a quarter of the 32 MB gives the middle sizes' gain away: 271 -> 299).
+// k = 16: 119.5 -> 108.6. With 32 / 8 heads and 16000 tokens or more it makes no difference with one k. With
+// three it is the last groups' luck there: k = 5, 10, 20 at 14000 tokens 705 -> 672, 8, 16, 32 at 16000 875 -> 893, 4, 8, 16 at 21000 1183 -> 1136,
+// 8, 16, 32 at 32768 2122 -> 2136; 28 / 4 heads, 24000, 1205 -> 1195. Half or a quarter of the 32 MB gives the middle sizes' gain away: 271 -> 299, 164 -> 206).
 inline int walked_heads(const Geom &g) {
     const long long fit = (32ll << 20) / (g.T * g.d * 2), all = (long long)g.batch * g.G;
     return (int)(fit < 1 ? 1 : (fit > all ? all : fit));
