@@ -376,13 +376,17 @@ stream_status launch_qw(const Geom &g, const void *q, const void *k, const void 
     // d = 64, 24 rows 43.9, 47.2, k = 4 41.1, 50.4, 72 rows 59.5, 65.6, d = 16 36.9, 39.0; more tiles: 64 rows of blocks of 32, d = 64,
     // k = 10, 50.5, 51.3; 72 rows, d = 128, k = 8, 65.5, 69.7).
     // T may have fewer blocks than k_top, and what counts are those that are there: a CTA of a cluster has two tile
-    // parts at least, a group half of one (16 rows, T = 29, blocks of 48, k = 9, d = 16: 32 -> 10 us); with many
+    // parts at least, a group half of one (16 rows, T = 29, blocks of 48, k = 9, d = 16: 32 -> 10 us). With up to 64 channels they also decide on
+    // the next CTAs, unless each would have just one (us with the mask build, by k_top and by those there: k = 16 and 24, d = 64, three blocks of 64, 12 heads:
+    // 43.9, 24.6, six, 3 heads: 59.6, 26.7, four, one head: 23.5 with eight CTAs, 26.7 with four; d = 16, ten blocks of 32: 22.5, 20.5; d = 128
+    // gains as often as it loses: four blocks of 32 20.5, 24.6, three 23.4, 20.5); with many
     // rows an idle group takes another CTA's shared memory (2500 rows, k = 1, d = 128, rows off 16 bytes: 397 -> 223).
     const int n_sm = sm_count_or_default(), n_sub = (g.bk + kKeys - 1) / kKeys, tiles = g.k_top * n_sub;
     const int there = (int)std::min((long long)g.k_top, (g.T + g.bk - 1) / g.bk) * n_sub;
     int splits = (rows <= n_sm ? 8 : 4) / m_warps, n_cta = 1;
     const bool small = D <= 64 && there * m_warps <= 8;
-    while (!small && n_cta < 8 && rows * 2 * n_cta <= n_sm && tiles * m_warps >= 8 * n_cta && there >= 3 && there >= 2 * n_cta) n_cta *= 2;
+    auto worth = [&](int n) { return D > 64 ? tiles * m_warps >= 8 * n : there * m_warps >= 8 * n || (there < tiles && there == 2 * n); };
+    while (!small && n_cta < 8 && rows * 2 * n_cta <= n_sm && worth(n_cta) && there >= 3 && there >= 2 * n_cta) n_cta *= 2;
     if (n_cta > 1) splits = std::min({splits, (tiles + n_cta - 1) / n_cta, 2 * ((there + n_cta - 1) / n_cta)});
     else if (rows > n_sm) splits = std::min(splits, rows > 4ll * n_sm ? there : 2 * there);
     auto bytes = [&](int s, bool p_in_k) {
