@@ -888,12 +888,12 @@ stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_
         s->n_chunks = (g.hpg + s->head_rows - 1) / s->head_rows;
         s->n_groups = (long long)g.batch * g.G * ((g.n_qb - first_qb + s->qb_rows - 1) / s->qb_rows) * s->n_chunks;
         // How many groups a CTA there should be rows for, in halves: from 545 drawn shapes (k = 2 to 64), each timed at every number of rows;
-        // over 220 others 2.4 % behind the best of these on average, with the attention behind it 1.3. Rows, not groups: three heads as 2 + 1 make more groups than they have work for (6 / 2
+        // over 380 others 2.4 % behind the best of these on average, with the attention behind it 1.3. Rows, not groups: three heads as 2 + 1 make more groups than they have work for (6 / 2
         // heads, 4458 tokens, k = 24: two rows 44.2 us, one 34.8). Some of them, us with four (or three) rows, two and one, in brackets the
         // groups of four a CTA. One CTA an SM: 28 / 4 heads, 3419 tokens, k = 27, not causal (2.9): 83, 74, 101; 8 / 2 heads, 20000, k = 24 (3.9):
         // 210, 195; 8 / 2 heads, 13232, k = 59 (2.0): 186, 157, 188; of several query blocks: 16 heads, 9000, k = 12 (3.5): 118, 124, and with
         // two nodes a lane: 1 head, 80291, k = 37 (2.0): 267, 235. Two CTAs, blocks of 64: 28 / 4 heads, 2500, k = 33, not causal (1.1): 73.6, 56.4, 43.0;
-        // 12 / 2 heads, 10922, k = 45 (1.7): 177, 156, 107; 2 heads, 73665, k = 16 (1.9): -, 168, 186. Blocks of 32, where a pair of rows is little
+        // 12 / 2 heads, 10922, k = 45 (1.7): 177, 156, 107; 2 heads, 73665, k = 16 (1.9): -, 168, 186; 61140, k = 2, not causal (1.6), with the attention: -, 103, 129. Blocks of 32, where a pair of rows is little
         // more work than a row alone: 12 / 2 heads, 6000, k = 40 (2.0): 75.7, 69.7; 28 / 4 heads, 3000, k = 40, d = 128 (1.5): 61, 55, 70.
         const bool wide = g.k_top > 32;
         int halves;
@@ -904,11 +904,12 @@ stream_status split_rows(const Geom &g, int first_qb, int ctas_per_sm, int most_
             // 244; 2 heads, 40264 (2.1): two rows 1.3 times four; 8 / 2 heads, 10311, k = 5, 10, 21 (2.2): 201, 149; 5501 (2.3): 114, 97).
             halves = rows > 2 ? (g.causal && s->qb_rows == 1 ? 5 : 3) : 2;
         } else if (ctas_per_sm == 2 && most_rows == 4) {
-            halves = rows > 2 ? 6 : (g.bq == 64 ? (wide ? 12 : 7) : (wide ? 3 : 2));
-            // Not causal, the groups are equally long: also where more than one round of them is five sixths full (16 heads, 8192 tokens, k = 40 (1.7):
-            // 153, 151, 154, with the attention behind them 350, -, 359; 8 / 2 heads, 16000, k = 60 (1.7): 246, 252; 16 heads, 5345, k = 37 (1.1): 113, 96, 94).
+            halves = rows > 2 ? 6 : (g.bq == 64 ? (wide ? 8 : 6) : (wide ? 3 : 2));
+            // Not causal, the groups are equally long: with two nodes a lane also where more than one round of them is five sixths full (16 heads, 8192
+            // tokens, k = 40 (1.7): 153, 151, 154, with the attention behind them 350, -, 359; 8 / 2 heads, 16000, k = 60 (1.7): 246, 252; 16 heads, 5345,
+            // k = 37 (1.1): 113, 96, 94; but one node a lane: 6 / 2 heads, 17942, k = 5 (1.9): 90, 80).
             const long long rounds = (s->n_groups + n_cta - 1) / n_cta;
-            full = rows > 2 && !g.causal && rounds > 1 && 6 * s->n_groups >= 5 * rounds * n_cta;
+            full = wide && rows > 2 && !g.causal && rounds > 1 && 6 * s->n_groups >= 5 * rounds * n_cta;
         } else {
             halves = rows > 2 ? (s->qb_rows > 1 ? (wide ? 6 : 4) : (wide ? 7 : 8)) : 2;
         }
