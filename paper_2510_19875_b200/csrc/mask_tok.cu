@@ -550,8 +550,8 @@ stream_status launch_mask_tok(const Geom &g, const void *q, const void *k, int32
     auto kern = g.k_top <= 16 ? mask_tok_kernel<16> : mask_tok_kernel<32>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(mask_tok)");
-    // (a CTA more for every four pieces of the rows kept whole)
-    const long long ctas = n_items + (P.first_tb > 0 ? (whole_pieces(g, P.first_tb * kTok) + 3) / 4 : 0);
+    // (a CTA more for every piece of the rows kept whole)
+    const long long ctas = n_items + (P.first_tb > 0 ? whole_pieces(g, P.first_tb * kTok) : 0);
     const int grid = (int)(ctas < n_sm ? ctas : n_sm);
     e = launch_kernel(kern, grid, kThreads, kSmemBytes, st, 1, tq, tk, P);
     if (e != cudaSuccess) return cuda_fail(e, "mask_tok launch");
