@@ -203,7 +203,7 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const int e_qlim = e_ok ? last_valid_block(g, (int)e_tq) : -1;
         const int key_end = e_ok ? (int)(g.causal ? e_tq + 1 : g.T) : 0;  // keys the token may look at: those before
         unsigned n_tiles = 0;  // tiles the token has needed so far (its own candidates, not the merged list)
-        // the next group's number is fetched beside this one's products, unless that could leave another CTA without work
+        // the next group's number is fetched beside this one's first products or, where that could leave another CTA without work, its last
         const bool ahead = id + 2 * (int)gridDim.x < P.n_items;
 
         for (int level = 0;; ++level) {
@@ -211,7 +211,8 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const bool last = level + 1 == tl->n_levels;
             const int n_list = tl->n_list, n_st = (n_list + 1) >> 1;
 
-            if (ahead && warp == 13 && lane == 0 && level == 0) tl->item = (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
+            if (warp == 13 && lane == 0 && (ahead ? level == 0 : last))
+                tl->item = P.n_items <= (int)gridDim.x ? P.n_items : (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
             if (is_producer) {
                 for (int i = 0; i < n_st; ++i) {
                     const unsigned s = seq + (unsigned)i, buf = s & 3u;
@@ -492,10 +493,6 @@ mask_tok_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
         if (*(volatile int *)&tl->abort_flag) break;
         if (warp == 0 && lane == 0) atomicAdd(&P.ws->rows, (unsigned long long)(tq_max - tok0 + 1));
-        if (!ahead) {
-            if (tid == 0) tl->item = P.n_items <= (int)gridDim.x ? P.n_items : (int)(gridDim.x + atomicAdd(&P.ws->work_counter, 1u));
-            __syncthreads();
-        }
         id = tl->item;
         __syncthreads();
     }
